@@ -15,6 +15,7 @@
 #include "kernels_fused.cuh"
 #include "kernels_bwd.cuh"
 #include "kernels_gemm.cuh"
+#include "kernels_kk.cuh"
 #include "kernels_dense.cuh"
 #include "kernels_rtn.cuh"
 
@@ -230,6 +231,11 @@ struct KkWS {  // bf16 scratch, each [nbT * k * k]
 constexpr int NS_MAX_ITERS = 8;
 constexpr int NS_COLD_ITERS = 6;
 constexpr int NS_WARM_ITERS = 4;  // upper bound: converged blocks skip the later ones (see ns_inverse)
+// Fused kernel (ns_block_kernel): rounds at most, and the squared residual before an update that makes it the last one.
+// Warm: below 1e-2 before, hence below 1e-4 after it (the acceptance test of the elimination fall-back).  Cold starts are
+// paid once per run: they go on to 1e-3 (1e-6 after the update, the accuracy the products themselves carry).
+constexpr int NS_WARM_ROUNDS = 6, NS_COLD_ROUNDS = 10;
+constexpr double NS_GATE2 = 1e-4, NS_COLD_GATE2 = 1e-6;
 
 static bool kk_fast(int k) { return k == 64 || k == 128 || k == 256; }
 
@@ -291,6 +297,10 @@ __global__ void transpose_blocks_kernel(const float* __restrict__ in, float* __r
   }
 }
 
+__global__ void fill_f64_kernel(double* p, double v, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = v;
+}
+
 __global__ void zero_ns_kernel(double* rn, int n, int* flag) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) rn[i] = 0.0;
@@ -313,10 +323,9 @@ __global__ void colnorm_kernel(const float* __restrict__ X, int k, int nb, float
 
 static void launch_split(cudaStream_t st, const float* X, int k, long long n, uint16_t* hi, uint16_t* lo, uint16_t* thi,
                          uint16_t* tlo, const int* run_flag, const int32_t* status, const double* gate = nullptr,
-                         double gate_tol = 0.0, int parity_iters = 0, int parity_nb = 0) {
+                         double gate_tol = 0.0) {
   dim3 grid(k / 32, k / 32, (unsigned)(n / ((long long)k * k)));
-  CQ_LAUNCH(split_bf16_kernel, grid, dim3(32, 8), 0, st, X, k, hi, lo, thi, tlo, run_flag, status, gate, gate_tol, parity_iters,
-            parity_nb);
+  CQ_LAUNCH(split_bf16_kernel, grid, dim3(32, 8), 0, st, X, k, hi, lo, thi, tlo, run_flag, status, gate, gate_tol);
 }
 
 // Minv = inv(bf16(M)) by Newton-Schulz iteration X <- X + X (I - A X) on the tensor cores, from X0 = A^T
@@ -328,26 +337,42 @@ static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm,
                        int32_t* status, bool prepped = false, bool splits_kept = false) {
   const long long kk = (long long)nb * k * k;
   const int iters = warm ? NS_WARM_ITERS : NS_COLD_ITERS;
-  // A warm start runs up to NS_WARM_ITERS iterations, as many as the step size calls for: a block whose residual
-  // ||I - A X||_F was below 1e-2 before an update (below 1e-4 after it) skips the iterations that follow (their CTAs
-  // return at once).  Small steps take one or two iterations, a change of the transform by half its norm four.
-  constexpr double NS_GATE2 = 1e-4;  // squared: the same bound the acceptance test below puts on the residual before the last update
+  // A warm start runs as many rounds as the step size calls for: a block whose residual ||I - A X||_F was below 1e-2
+  // before an update (below 1e-4 after it) stops.  Small steps take one or two rounds, a change of the transform by
+  // half its norm four.
   int ti = kt_begin(3, st);
   if (!prepped) {  // otherwise step_prep_kernel has cleared rn / flag and written Ab
     CQ_LAUNCH(zero_ns_kernel, (NS_MAX_ITERS * nb + 127) / 128, 128, 0, st, w.rn, NS_MAX_ITERS * nb, w.flag);
     CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Mc, w.Ab, k, kk, 0, status);
   }
+  // Block sizes of the fused kernel: every round of a block runs in one launch, on row-major splits only.
+  w.mn = g_tb_enable.load(std::memory_order_relaxed) && tb_supported(k, 2);
+  if (w.mn) {
+    w.cur = 0;
+    // (splits_kept: the splits of X that the previous call left in set 0 are still there)
+    if (!warm) CQ_LAUNCH(ns_cold_start_kernel, dim3(k / 32, k / 32, nb), dim3(32, 8), 0, st, w.Ab, k, w.Xh[0], w.Xl[0], status);
+    else if (!splits_kept) launch_split(st, X, k, kk, w.Xh[0], w.Xl[0], nullptr, nullptr, nullptr, status);
+    NsParams np;
+    np.max_rounds = warm ? NS_WARM_ROUNDS : NS_COLD_ROUNDS;
+    np.gate2 = warm ? NS_GATE2 : NS_COLD_GATE2;
+    np.rn = w.rn;
+    np.status = status;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np) != CAFEQ_OK)
+      CQ_LAUNCH(fill_f64_kernel, 1, 128, 0, st, w.rn, 1.0, nb);  // (no tensor maps: everything goes to the elimination)
+    // a block that ran out of rounds is recomputed by elimination, and everything is split again then
+    launch_inverse(st, Mc, X, nullptr, nb, k, status, w.rn, 1e-4, w.flag, w.redo_total);
+    launch_split(st, X, k, kk, w.Xh[0], w.Xl[0], nullptr, nullptr, w.flag, status);
+    if (cnorm) {
+      dim3 grid((k + 127) / 128, nb);
+      CQ_LAUNCH(colnorm_kernel, grid, 128, 0, st, X, k, nb, cnorm);
+    }
+    kt_end(ti, st);
+    return;
+  }
   if (!warm) CQ_LAUNCH(transpose_blocks_kernel, grid_for(kk), 256, 0, st, Mc, X, k, kk);
   int cur = 0;
-  // Block sizes with the whole-block product kernel run the iteration on row-major arrays only (MN-major operands):
-  // no transposed split of X or R is written.
-  const bool mn = g_tb_enable.load(std::memory_order_relaxed) && tb_supported(k, 2);
-  w.mn = mn;
-  // (splits_kept: the splits of X that the previous call left in set 0 are still there)
-  if (!(warm && splits_kept)) {
-    if (mn) launch_split(st, X, k, kk, w.Xh[cur], w.Xl[cur], nullptr, nullptr, nullptr, status);
-    else launch_split(st, X, k, kk, w.Xh[cur], iters > 0 ? nullptr : w.Xl[cur], w.XTh[cur], w.XTl[cur], nullptr, status);
-  }
+  launch_split(st, X, k, kk, w.Xh[cur], iters > 0 ? nullptr : w.Xl[cur], w.XTh[cur], w.XTl[cur], nullptr, status);
   for (int it = 0; it < iters; ++it) {
     const double* gate = (warm && it > 0) ? w.rn + (size_t)(it - 1) * nb : nullptr;
     // R = I - A X needs X to full precision (the product cancels against I): two terms over the split of X.
@@ -355,22 +380,13 @@ static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm,
     // (the error it leaves is 2^-8 |R| relative, below 4e-5 for every accepted residual).
     const uint16_t* a1[2] = {w.Ab, w.Ab};
     const uint16_t* a2[1] = {w.Xh[cur]};
-    if (mn) {
-      const uint16_t* b1[2] = {w.Xh[cur], w.Xl[cur]};  // X stored [l][n]
-      launch_kk_tc(st, 2, a1, b1, nb, k, -1.f, 0.f, 1.f, nullptr, nullptr, w.RTh, nullptr, nullptr, nullptr, w.rn + (size_t)it * nb,
-                   nullptr, status, 1, gate, NS_GATE2, 0, 1);
-      const uint16_t* b2[1] = {w.RTh};                  // bf16(R), row-major here
-      launch_kk_tc(st, 1, a2, b2, nb, k, 1.f, 1.f, 0.f, X, X, w.Xh[cur ^ 1], w.Xl[cur ^ 1], nullptr, nullptr, nullptr, nullptr, status,
-                   1, gate, NS_GATE2, 0, 1);
-    } else {
-      const uint16_t* b1[2] = {w.XTh[cur], w.XTl[cur]};
-      launch_kk_tc(st, 2, a1, b1, nb, k, -1.f, 0.f, 1.f, nullptr, nullptr, nullptr, nullptr, w.RTh, nullptr, w.rn + (size_t)it * nb,
-                   nullptr, status, 1, gate, NS_GATE2);
-      const uint16_t* b2[1] = {w.RTh};
-      // (the row-major low half is only read after the last iteration, by the M^-1 path of the gradient)
-      launch_kk_tc(st, 1, a2, b2, nb, k, 1.f, 1.f, 0.f, X, X, w.Xh[cur ^ 1], (it == iters - 1) ? w.Xl[cur ^ 1] : nullptr,
-                   w.XTh[cur ^ 1], w.XTl[cur ^ 1], nullptr, nullptr, status, 1, gate, NS_GATE2);
-    }
+    const uint16_t* b1[2] = {w.XTh[cur], w.XTl[cur]};
+    launch_kk_tc(st, 2, a1, b1, nb, k, -1.f, 0.f, 1.f, nullptr, nullptr, nullptr, nullptr, w.RTh, nullptr, w.rn + (size_t)it * nb,
+                 nullptr, status, 1, gate, NS_GATE2);
+    const uint16_t* b2[1] = {w.RTh};
+    // (the row-major low half is only read after the last iteration, by the M^-1 path of the gradient)
+    launch_kk_tc(st, 1, a2, b2, nb, k, 1.f, 1.f, 0.f, X, X, w.Xh[cur ^ 1], (it == iters - 1) ? w.Xl[cur ^ 1] : nullptr,
+                 w.XTh[cur ^ 1], w.XTl[cur ^ 1], nullptr, nullptr, status, 1, gate, NS_GATE2);
     cur ^= 1;
   }
   w.cur = cur;
@@ -379,15 +395,8 @@ static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm,
   launch_inverse(st, Mc, X, nullptr, nb, k, status, w.rn + (size_t)(iters - 1) * nb, 1e-4, w.flag, w.redo_total);
   // final splits: written by the last iteration's epilogue, except for blocks that skipped it (and for everything
   // when the elimination recomputed a block)
-  if (mn) {
-    // every iteration writes both row-major splits, so a block that stopped early needs this only when its newest
-    // splits are in the other set
-    launch_split(st, X, k, kk, w.Xh[cur], w.Xl[cur], nullptr, nullptr, w.flag, status, (warm && iters > 1) ? w.rn : nullptr, NS_GATE2,
-                 iters, nb);
-  } else {
-    const double* last_gate = (warm && iters > 1) ? w.rn + (size_t)(iters - 2) * nb : nullptr;
-    launch_split(st, X, k, kk, w.Xh[cur], w.Xl[cur], w.XTh[cur], w.XTl[cur], w.flag, status, last_gate, NS_GATE2);
-  }
+  const double* last_gate = (warm && iters > 1) ? w.rn + (size_t)(iters - 2) * nb : nullptr;
+  launch_split(st, X, k, kk, w.Xh[cur], w.Xl[cur], w.XTh[cur], w.XTl[cur], w.flag, status, last_gate, NS_GATE2);
   if (cnorm) {
     dim3 grid((k + 127) / 128, nb);
     CQ_LAUNCH(colnorm_kernel, grid, 128, 0, st, X, k, nb, cnorm);
@@ -1743,11 +1752,16 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
   float* Mc = b.take<float>(kk);
   float* Minv = b.take<float>(kk);
   float* Minv_c = b.take<float>(kk);
+  KkWS kkw;
+  carve_kk(b, G1.nbT, G1.k, &kkw);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   if (M) {
     // the transformed pair U = W1 M (operator bf16(M)^T on the stored rows), V = M^-1 W2 (operator bf16(inv(bf16(M))))
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, M, Mc, kk, status);
-    launch_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, status);
+    // block sizes 128 / 256: elimination takes 5 ms at k = 256 (one CTA per block, k dependent steps); at k <= 64 it is
+    // short and stays
+    if (tb_supported(G1.k, 2)) ns_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, false, kkw, status);
+    else launch_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, status);
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, Minv, Minv_c, kk, status);
     launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
     launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);

@@ -1,0 +1,428 @@
+// Fused chains of k x k products on the tensor cores (k = 128 or 256): one CTA carries one operator block through a
+// whole chain, so that intermediate results stay in shared memory and no launch separates the products.
+#pragma once
+
+#include "kernels_gemm.cuh"
+
+namespace cafeq {
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+// all bulk stores of this thread are complete (visible in global memory)
+__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// ------------------------------------------------------------------------------------------------
+// Block inverse by Newton-Schulz: X <- X + X (I - A X), as many rounds as the block needs, in one launch.
+//   round: R = I - A X over X = hi + lo (two terms, 24-bit products against bf16 A), ||R||_F in the same epilogue,
+//          X += hi R (one term: the round corrects its own error), new hi / lo splits, fp32 X on the last round.
+// The last round is the one whose residual before the update is below the gate.
+//
+// What bounds it: one round at k = 256 moves 512 KB into the SM (A, hi, lo, hi again) at the 60 - 75 GB/s one SM takes
+// from L2, and spends 3 x 1.1 us per 64-column chunk of products; as two launches per round (residual, update) each
+// launch paid about 8 us of prologue, pipeline fill and drain on top, and the residual went to memory and back.
+// Measured (106 blocks of 256, a step that takes two rounds): 55 us; as separate launches 8 x 17.6 us (the later ones
+// gated off).  72 blocks of 128: 17.5 us against 8 x 7.1.  A cold start of 14 blocks of 256: 86 us against 12 x 18.
+// R stays in shared memory: written row-major in the 128-byte-swizzled layout of the operand boxes, which the second
+// product reads as its MN-major operand.  The updates are in place (a tile is read and written by the same warp after
+// every product of the round has read its operands).
+// Shared memory: NRING slots + the R area (K / 64 slots); the residual products stream through all slots, the update
+// products through the ring, the epilogue's tiles take over both afterwards.
+// ------------------------------------------------------------------------------------------------
+struct NsMaps {
+  CUtensorMap a;       // bf16 A, boxes of K rows x 64 (K-major operand)
+  CUtensorMap xh_mn, xl_mn;  // hi / lo of X, boxes of 64 x 64 (MN-major operand)
+  CUtensorMap xh_k;    // hi of X, boxes of K rows x 64 (K-major operand)
+  CUtensorMap xhl;     // hi and lo as two planes, boxes of 32 x 32 x 2, 64-byte swizzle
+  CUtensorMap x;       // fp32 X, boxes of 32 x 32, 128-byte swizzle
+};
+struct NsParams {
+  int max_rounds;
+  double gate2;        // squared residual below which a round is the last one
+  double* rn;          // [nb] squared residual before the last update
+  int32_t* status;
+};
+
+template <int K>
+struct NsCfg {
+  static constexpr int HALVES = K / 128;
+  static constexpr int KCH = K / 64;
+  static constexpr int SLOT = K * 128;
+  static constexpr int NRING = (K == 256) ? 3 : 10;
+  static constexpr int NSLOT = NRING + KCH;
+  static constexpr int EPI_WARPS = 16;
+  static constexpr int EPI_WARP_BYTES = 12288;  // two hi + lo tiles (in and out), one fp32 tile
+  static constexpr int NBAR = 2 * NSLOT + 3 + 2 * EPI_WARPS;
+  static constexpr int SMEM = 1024 + NSLOT * SLOT + 8 * NBAR + 8 * EPI_WARPS + 64;
+  static constexpr int TMEM_COLS = HALVES * K;
+  static constexpr int THREADS = 64 + 32 * EPI_WARPS;
+  static_assert(NSLOT * SLOT >= EPI_WARPS * EPI_WARP_BYTES, "epilogue tiles must fit");
+};
+
+template <int K>
+__global__ void __launch_bounds__(NsCfg<K>::THREADS, 1) ns_block_kernel(const __grid_constant__ NsMaps maps, const NsParams p) {
+  using C = NsCfg<K>;
+  if (p.status && *p.status) return;
+  const int b = blockIdx.x, row_b = b * K;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = (uint64_t*)(smem + C::NSLOT * C::SLOT);
+  const uint32_t bar_full = smem_u32(bars);
+  const uint32_t bar_empty = bar_full + 8 * C::NSLOT;
+  const uint32_t bar_acc = bar_empty + 8 * C::NSLOT;  // a product chain is complete
+  const uint32_t bar_r = bar_acc + 8;                 // R and the partial norms are in shared memory
+  const uint32_t bar_x = bar_r + 8;                   // the updated X is in global memory
+  const uint32_t bar_c0 = bar_x + 8;                  // two per epilogue warp
+  double* red = (double*)(bars + C::NBAR);            // [EPI_WARPS] partial squared norms
+  uint32_t* tmem_slot = (uint32_t*)(red + C::EPI_WARPS);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t sm_u = smem_u32(smem);
+  const uint32_t sR = sm_u + C::NRING * C::SLOT;
+
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&maps.a);
+    tma_prefetch_desc(&maps.xh_mn);
+    tma_prefetch_desc(&maps.xl_mn);
+    tma_prefetch_desc(&maps.xh_k);
+    for (int s = 0; s < C::NSLOT; ++s) {
+      mbar_init(bar_full + 8 * s, 1);
+      mbar_init(bar_empty + 8 * s, 1);
+    }
+    mbar_init(bar_acc, 1);
+    mbar_init(bar_r, C::EPI_WARPS);
+    mbar_init(bar_x, C::EPI_WARPS);
+    for (int s = 0; s < 2 * C::EPI_WARPS; ++s) mbar_init(bar_c0 + 8 * s, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"((uint32_t)C::TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  // every role takes the same decision from the same 16 partial sums
+  auto residual2 = [&]() {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < C::EPI_WARPS; ++w) s += ((volatile double*)red)[w];
+    return s;
+  };
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- TMA producer
+    if (lane == 0) {
+      uint32_t eph = 0xFFFFFFFFu;  // parity of the next wait on each slot's empty barrier (fresh barriers: 1 passes at once)
+      bool ok = true;
+      for (int it = 0; it < p.max_rounds && ok; ++it) {
+        if (it > 0) {
+          if (!mbar_wait(bar_x, (it - 1) & 1u, abort_flag, p.status)) break;
+          asm volatile("fence.proxy.async;" ::: "memory");
+        }
+        int s = 0;
+        for (int c = 0; c < C::KCH && ok; ++c)
+          for (int u = 0; u < 3; ++u) {
+            if (!mbar_wait(bar_empty + 8 * s, (eph >> s) & 1u, abort_flag, p.status)) { ok = false; break; }
+            eph ^= 1u << s;
+            mbar_expect_tx(bar_full + 8 * s, C::SLOT);
+            const uint32_t dst = sm_u + s * C::SLOT;
+            if (u == 0) {
+              tma_load_2d(dst, &maps.a, c * 64, row_b, bar_full + 8 * s);
+            } else {
+              const CUtensorMap* m = (u == 1) ? &maps.xh_mn : &maps.xl_mn;
+              for (int j = 0; j < K / 64; ++j) tma_load_2d(dst + j * 8192, m, j * 64, row_b + c * 64, bar_full + 8 * s);
+            }
+            if (++s == C::NSLOT) s = 0;
+          }
+        for (int c = 0; c < C::KCH && ok; ++c) {
+          const int sl = c % C::NRING;
+          if (!mbar_wait(bar_empty + 8 * sl, (eph >> sl) & 1u, abort_flag, p.status)) { ok = false; break; }
+          eph ^= 1u << sl;
+          mbar_expect_tx(bar_full + 8 * sl, C::SLOT);
+          tma_load_2d(sm_u + sl * C::SLOT, &maps.xh_k, c * 64, row_b, bar_full + 8 * sl);
+        }
+        if (!ok || !mbar_wait(bar_r, it & 1u, abort_flag, p.status)) break;
+        if (residual2() <= p.gate2) break;
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer (converged warp, one elected lane)
+    constexpr uint32_t idesc = umma_idesc_bf16(128, K, 0, 1);
+    uint32_t fph = 0;
+    bool ok = true;
+    for (int it = 0; it < p.max_rounds && ok; ++it) {
+      int s = 0;
+      auto next = [&](int q) { return q + 1 == C::NSLOT ? 0 : q + 1; };
+      for (int c = 0; c < C::KCH && ok; ++c) {
+        const int s0 = s, s1 = next(s0), s2 = next(s1);
+        s = next(s2);
+        ok = mbar_wait(bar_full + 8 * s0, (fph >> s0) & 1u, abort_flag, p.status) &&
+             mbar_wait(bar_full + 8 * s1, (fph >> s1) & 1u, abort_flag, p.status);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        fph ^= (1u << s0) | (1u << s1);
+        tc_fence_after();
+        const uint32_t alo = umma_desc_lo(sm_u + s0 * C::SLOT);
+        if (elect_one()) {
+          const uint32_t blo = umma_desc_lo(sm_u + s1 * C::SLOT, 8192);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int mh = 0; mh < C::HALVES; ++mh)
+              tc_mma_lo(tmem_base + mh * K, alo + mh * 1024 + kk * 2, blo + kk * 128, idesc, (c | kk) != 0 ? 1u : 0u);
+          tc_commit(bar_empty + 8 * s1);
+        }
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s2, (fph >> s2) & 1u, abort_flag, p.status));
+        if (!ok) break;
+        fph ^= 1u << s2;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t blo = umma_desc_lo(sm_u + s2 * C::SLOT, 8192);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int mh = 0; mh < C::HALVES; ++mh) tc_mma_lo(tmem_base + mh * K, alo + mh * 1024 + kk * 2, blo + kk * 128, idesc, 1u);
+          tc_commit(bar_empty + 8 * s0);
+          tc_commit(bar_empty + 8 * s2);
+          if (c == C::KCH - 1) tc_commit(bar_acc);
+        }
+        __syncwarp();
+      }
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar_r, it & 1u, abort_flag, p.status));
+      if (!ok) break;
+      tc_fence_after();
+      for (int c = 0; c < C::KCH && ok; ++c) {
+        const int sl = c % C::NRING;
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * sl, (fph >> sl) & 1u, abort_flag, p.status));
+        if (!ok) break;
+        fph ^= 1u << sl;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t alo = umma_desc_lo(sm_u + sl * C::SLOT), blo = umma_desc_lo(sR + c * C::SLOT, 8192);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int mh = 0; mh < C::HALVES; ++mh)
+              tc_mma_lo(tmem_base + mh * K, alo + mh * 1024 + kk * 2, blo + kk * 128, idesc, (c | kk) != 0 ? 1u : 0u);
+          tc_commit(bar_empty + 8 * sl);
+          if (c == C::KCH - 1) tc_commit(bar_acc);
+        }
+        __syncwarp();
+      }
+      if (!ok || it == p.max_rounds - 1 || residual2() <= p.gate2) break;
+      // the next round's first product overwrites the accumulators that the epilogue of this one reads
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_x, it & 1u, abort_flag, p.status));
+      tc_fence_after();
+    }
+  } else {
+    // ---------------------------------------------------------------- epilogues: 32 x 32 tiles
+    const int q = warp & 3, ew = warp - 2, part = ew >> 2;
+    constexpr int CPH = K / 32, NU = C::HALVES * CPH / 4;  // column tiles per accumulator, tiles per warp
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+    uint8_t* wbuf = smem + ew * C::EPI_WARP_BYTES;
+    const uint32_t tB = smem_u32(wbuf), tF = tB + 8192;
+    const uint32_t bc0 = bar_c0 + 16 * ew;
+    uint32_t accph = 0, c0ph = 0;
+    bool ok = true;
+    auto tile_of = [&](int i, int& mh, int& ch) { const int c2 = part + i * 4; mh = c2 / CPH; ch = c2 - mh * CPH; };
+    for (int it = 0; it < p.max_rounds && ok; ++it) {
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, accph, abort_flag, p.status));
+      accph ^= 1u;
+      if (!ok) break;
+      tc_fence_after();
+      float sq4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int i = 0; i < NU; ++i) {
+        int mh, ch;
+        tile_of(i, mh, ch);
+        const int l = mh * 128 + q * 32 + lane, col0 = ch * 32;
+        float v[32];
+        tc_ld32(taddr + mh * K + col0, v);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+          v[e] = ((col0 + e == l) ? 1.f : 0.f) - v[e];
+          sq4[e & 3] = fmaf(v[e], v[e], sq4[e & 3]);
+        }
+        // row l, columns col0 .. col0 + 31: four 16-byte pieces of one 128-byte swizzled row
+        const uint32_t rowp = sR + (l >> 6) * C::SLOT + (col0 >> 6) * 8192 + (l & 63) * 128;
+        const int c16 = (col0 & 63) >> 3;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          uint32_t h[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            h[j] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[8 * w + 2 * j])) |
+                   ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[8 * w + 2 * j + 1])) << 16);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowp + (((c16 + w) ^ (l & 7)) << 4)), "r"(h[0]), "r"(h[1]),
+                       "r"(h[2]), "r"(h[3])
+                       : "memory");
+        }
+      }
+      double sq = (double)((sq4[0] + sq4[1]) + (sq4[2] + sq4[3]));
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      if (lane == 0) red[ew] = sq;
+      fence_proxy_async_smem_tb();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_r);
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_r, it & 1u, abort_flag, p.status));
+      if (!ok) break;
+      const double r2 = residual2();
+      const bool last = (r2 <= p.gate2) || it == p.max_rounds - 1;
+      if (last && threadIdx.x == 64) p.rn[b] = r2;
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, accph, abort_flag, p.status));
+      accph ^= 1u;
+      if (!ok) break;
+      tc_fence_after();
+      // X += X R: old hi + lo tiles arrive one tile ahead, the new ones leave from the same buffer
+      if (lane == 0) {
+        int mh, ch;
+        tile_of(0, mh, ch);
+        mbar_expect_tx(bc0, 4096);
+        tma_load_3d(tB, &maps.xhl, ch * 32, row_b + mh * 128 + q * 32, 0, bc0);
+      }
+#pragma unroll 1
+      for (int i = 0; i < NU && ok; ++i) {
+        int mh, ch;
+        tile_of(i, mh, ch);
+        const int row0 = row_b + mh * 128 + q * 32, col0 = ch * 32;
+        const uint32_t buf = i & 1, tH = tB + buf * 4096, tL = tH + 2048;
+        float v[32];
+        tc_ld32(taddr + mh * K + col0, v);
+        ok = __all_sync(0xffffffffu, mbar_wait(bc0 + 8 * buf, (c0ph >> buf) & 1u, abort_flag, p.status));
+        if (!ok) break;
+        c0ph ^= 1u << buf;
+        const int sw2 = (lane >> 1) & 3;  // 64-byte rows, 16-byte pieces XOR-swizzled by (row / 2) mod 4
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint32_t off = lane * 64 + ((c ^ sw2) << 4);
+          uint32_t h[4], l[4];
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3]) : "r"(tH + off));
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(l[0]), "=r"(l[1]), "=r"(l[2]), "=r"(l[3]) : "r"(tL + off));
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            v[8 * c + 2 * j] += __uint_as_float(h[j] << 16) + __uint_as_float(l[j] << 16);
+            v[8 * c + 2 * j + 1] += __uint_as_float(h[j] & 0xFFFF0000u) + __uint_as_float(l[j] & 0xFFFF0000u);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float x0 = v[8 * c + 2 * j], x1 = v[8 * c + 2 * j + 1];
+            const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
+            h[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+            l[j] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x0 - __bfloat162float(h0))) |
+                   ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x1 - __bfloat162float(h1))) << 16);
+          }
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tH + off), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tL + off), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
+        }
+        // the stores of the previous tile have read their shared memory: its buffer takes the next old tile, and the
+        // fp32 tile can be overwritten
+        if (lane == 0) {
+          tma_store_wait_read();
+          if (i + 1 < NU) {
+            int mh2, ch2;
+            tile_of(i + 1, mh2, ch2);
+            const uint32_t bn = bc0 + 8 * (buf ^ 1u);
+            mbar_expect_tx(bn, 4096);
+            tma_load_3d(tB + (buf ^ 1u) * 4096, &maps.xhl, ch2 * 32, row_b + mh2 * 128 + q * 32, 0, bn);
+          }
+        }
+        __syncwarp();
+        if (last) {
+          const int sw = lane & 7;
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(tF + lane * 128 + ((c ^ sw) << 4)), "f"(v[4 * c]),
+                         "f"(v[4 * c + 1]), "f"(v[4 * c + 2]), "f"(v[4 * c + 3])
+                         : "memory");
+        }
+        fence_proxy_async_smem_tb();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_3d(&maps.xhl, tH, col0, row0, 0);
+          if (last) tma_store_2d(&maps.x, tF, col0, row0);
+          tma_store_commit();
+        }
+      }
+      if (lane == 0) tma_store_wait_all();
+      tc_fence_before();
+      __syncwarp();
+      if (!ok || last) break;
+      if (lane == 0) {
+        asm volatile("fence.proxy.async;" ::: "memory");
+        mbar_arrive(bar_x);
+      }
+      __syncwarp();
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+  }
+}
+
+template <int K>
+static int ns_block_launch_t(cudaStream_t st, const NsMaps& maps, int nb, const NsParams& p) {
+  using C = NsCfg<K>;
+  static std::atomic<unsigned long long> done{0};
+  if (!opt_in_smem(ns_block_kernel<K>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
+  ns_block_kernel<K><<<nb, C::THREADS, C::SMEM, st>>>(maps, p);
+  return CAFEQ_OK;
+}
+
+// hi and lo splits [nb * k, k] as the two planes of one 3-D view (lo must lie a multiple of 16 bytes after hi)
+static bool make_map_hl(CUtensorMap* m, const uint16_t* hi, const uint16_t* lo, long long rows, int k) {
+  EncodeTiledFn enc = get_encode_tiled();
+  if (!enc || lo <= hi || (((uintptr_t)lo - (uintptr_t)hi) & 15)) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)k, (cuuint64_t)rows, 2};
+  cuuint64_t strides[2] = {(cuuint64_t)k * 2, (cuuint64_t)((uintptr_t)lo - (uintptr_t)hi)};
+  cuuint32_t box[3] = {32, 32, 2};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t*>(hi), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// A, hi, lo: bf16 [nb * k, k]; X: fp32 [nb, k, k] (written, not read)
+static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uint16_t* lo, float* X, int nb, int k, const NsParams& p) {
+  NsMaps m;
+  const long long rows = (long long)nb * k;
+  if (!make_map_bf16(&m.a, A, k, rows, k, k) || !make_map_bf16(&m.xh_mn, hi, k, rows, k, 64) || !make_map_bf16(&m.xl_mn, lo, k, rows, k, 64) ||
+      !make_map_bf16(&m.xh_k, hi, k, rows, k, k) || !make_map_hl(&m.xhl, hi, lo, rows, k) ||
+      !make_map_2d(&m.x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, X, k, rows, k, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B))
+    return CAFEQ_ERR_UNSUPPORTED;
+  return k == 256 ? ns_block_launch_t<256>(st, m, nb, p) : ns_block_launch_t<128>(st, m, nb, p);
+}
+
+// hi = A^T, lo = 0: the cold start X0 = A^T of the iteration (A is bf16, so hi carries it exactly); 32 x 32 tiles
+__global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* __restrict__ A, int k, uint16_t* __restrict__ hi,
+                                                            uint16_t* __restrict__ lo, const int32_t* status) {
+  if (status && *status) return;
+  __shared__ uint16_t tile[32][34];
+  const size_t base = (size_t)blockIdx.z * k * k;
+  const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) tile[threadIdx.y + 8 * r][threadIdx.x] = A[base + (size_t)(i0 + threadIdx.y + 8 * r) * k + j0 + threadIdx.x];
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const size_t o = base + (size_t)(j0 + threadIdx.y + 8 * r) * k + i0 + threadIdx.x;
+    hi[o] = tile[threadIdx.x][threadIdx.y + 8 * r];
+    lo[o] = 0;
+  }
+}
+
+}  // namespace cafeq
