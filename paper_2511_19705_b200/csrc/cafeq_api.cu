@@ -404,30 +404,43 @@ static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm,
   kt_end(ti, st);
 }
 
-// G (op)= -X^T Gx X^T for every block, on the tensor cores with three-term bf16 splits; X = Minv with its
-// splits in w[w.cur]; Gx fp32 [nb,k,k] (dL/dMinv).  G += result when accumulate, else G = result.
-static void minv_path_tc(cudaStream_t st, const float* Gx, float* G, int nb, int k, bool accumulate, KkWS& w, int32_t* status) {
+// G -= X^T Gx X^T for every block, on the tensor cores with three-term bf16 splits; X = Minv with its splits in
+// w[w.cur]; Gx = dL/dMinv: fp32 [nb,k,k], or (scaled, fused kernel only) formed from X by the kernel itself.
+static int minv_path_tc(cudaStream_t st, const float* Gx, float* G, int nb, int k, KkWS& w, int32_t* status,
+                        const ChainParams* scaled = nullptr) {
   const long long kk = (long long)nb * k * k;
   const int c = w.cur;
   if (w.mn) {
-    // T1 = X^T Gx with both operands read from their row-major arrays: A_op[i][l] = X[l][i], B_op[j][l] = Gx[l][j]
-    launch_split(st, Gx, k, kk, w.Ph, w.Pl, nullptr, nullptr, nullptr, status);
-    const uint16_t* a1[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
-    const uint16_t* b1[3] = {w.Ph, w.Ph, w.Pl};
-    launch_kk_tc(st, 3, a1, b1, nb, k, 1.f, 0.f, 0.f, nullptr, nullptr, w.Qh, w.Ql, nullptr, nullptr, nullptr, nullptr, status, 1, nullptr,
-                 0.0, 1, 1);
-  } else {
-    launch_split(st, Gx, k, kk, nullptr, nullptr, w.Ph, w.Pl, nullptr, status);  // Gx^T splits
-    // T1 = X^T Gx : T1[i][j] = sum_l XT[i][l] * GxT[j][l]
-    const uint16_t* a1[3] = {w.XTh[c], w.XTl[c], w.XTh[c]};
-    const uint16_t* b1[3] = {w.Ph, w.Ph, w.Pl};
-    launch_kk_tc(st, 3, a1, b1, nb, k, 1.f, 0.f, 0.f, nullptr, nullptr, w.Qh, w.Ql, nullptr, nullptr, nullptr, nullptr, status);
+    ChainParams cp;
+    memset(&cp, 0, sizeof(cp));
+    if (scaled) cp = *scaled;
+    cp.G = Gx;
+    cp.status = status;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return kk_chain_launch(st, KK_MINV_PATH, w.Xh[c], w.Xl[c], G, nb, k, cp);
   }
+  launch_split(st, Gx, k, kk, nullptr, nullptr, w.Ph, w.Pl, nullptr, status);  // Gx^T splits
+  // T1 = X^T Gx : T1[i][j] = sum_l XT[i][l] * GxT[j][l]
+  const uint16_t* a1[3] = {w.XTh[c], w.XTl[c], w.XTh[c]};
+  const uint16_t* b1[3] = {w.Ph, w.Ph, w.Pl};
+  launch_kk_tc(st, 3, a1, b1, nb, k, 1.f, 0.f, 0.f, nullptr, nullptr, w.Qh, w.Ql, nullptr, nullptr, nullptr, nullptr, status);
   // G -= T1 X^T : [i][j] = sum_l T1[i][l] * X[j][l]
   const uint16_t* a2[3] = {w.Qh, w.Ql, w.Qh};
   const uint16_t* b2[3] = {w.Xh[c], w.Xh[c], w.Xl[c]};
-  launch_kk_tc(st, 3, a2, b2, nb, k, -1.f, accumulate ? 1.f : 0.f, 0.f, accumulate ? G : nullptr, G, nullptr, nullptr, nullptr,
-               nullptr, nullptr, nullptr, status);
+  return launch_kk_tc(st, 3, a2, b2, nb, k, -1.f, 1.f, 0.f, G, G, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status);
+}
+
+// Orthonormality penalty of nb blocks from the splits of the fp32 parameters (fused kernel, k = 128 / 256):
+// sq[b * sq_stride] += ||M_b M_b^T - I||_F^2 and, with want_out, out = (M M^T - I) M.
+static int penalty_tc(cudaStream_t st, const uint16_t* Mh, const uint16_t* Ml, float* out, bool want_out, double* sq, int sq_stride,
+                      int nb, int k, int32_t* status) {
+  ChainParams cp;
+  memset(&cp, 0, sizeof(cp));
+  cp.sq = sq; cp.sq_stride = sq_stride;
+  cp.want_out = want_out ? 1 : 0;
+  cp.status = status;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return kk_chain_launch(st, KK_PENALTY, Mh, Ml, out, nb, k, cp);
 }
 
 static void launch_absmax(cudaStream_t st, const float* U, long long ld, const Geo& G, float* a, float* usel, int* idx,
@@ -1098,7 +1111,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     CQ_LAUNCH(ste_scale_coef_kernel, (unsigned)((nrec * 32 + 255) / 256), 256, 0, st, s.m.D, (long long)G.d_in, s.m.Dbf, s.Dlo,
               (long long)G.d_in, G.d_out, G.ng, G.g, s.m.a, s.m.usel, 1, s.m.coef, status);
     launch_scatter(st, W, G, s.m.coef, s.m.idx, gradM, 0, status, 1);
-    minv_path_tc(st, s.gMinv, gradM, G.nbT, k, true, s.kk, status);
+    s.err = minv_path_tc(st, s.gMinv, gradM, G.nbT, k, s.kk, status);
     return;
   }
   if (need_l2) {
@@ -1125,6 +1138,16 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
   if (!want_grad) return;
   if (!ste) {
     launch_scatter(st, W, G, s.m.coef, s.m.idx, gradM, 0, status, fused ? 1 : 0);
+    if (tc && s.kk.mn) {
+      ChainParams cp;
+      memset(&cp, 0, sizeof(cp));
+      cp.n = 1;
+      cp.blk0[1] = G.nbT;
+      cp.A[0] = s.A; cp.Agrp[0] = in_r1 ? s.m.agrp : nullptr; cp.g[0] = G.g; cp.scale[0] = 2.f * kappa;
+      cp.X = s.Minv;
+      s.err = minv_path_tc(st, nullptr, gradM, G.nbT, k, s.kk, status, &cp);
+      return;
+    }
     CQ_LAUNCH(gminv_kernel, grid_for(kk), 256, 0, st, s.Minv, s.A, in_r1 ? s.m.agrp : nullptr, G.g, 2.f * kappa, k, kk, s.gMinv);
   } else {
     // gMinv = 2 * sum_free E Delta^T ; gDelta = 2 Minv^T o E (overwrites Delta) ; scale path through arg-max
@@ -1140,7 +1163,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
   }
   // gradM -= Minv^T gMinv Minv^T
   if (tc) {
-    minv_path_tc(st, s.gMinv, gradM, G.nbT, k, true, s.kk, status);
+    s.err = minv_path_tc(st, s.gMinv, gradM, G.nbT, k, s.kk, status);
   } else {
     launch_kk(st, s.Minv, 1, s.gMinv, 0, s.tmp, G.nbT, k, 1.f, GEMM_STORE, status);
     launch_kk(st, s.tmp, 0, s.Minv, 1, gradM, G.nbT, k, -1.f, GEMM_STORE | GEMM_ACCUM, status);
@@ -1455,6 +1478,11 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
   }
   // orthonormality penalty on the fp32 parameters: R = M M^T - I (not part of the straight-through PQE loss)
   if (ste) {
+  } else if (tc && p.kk.mn) {
+    KkWS& w = p.kk;
+    launch_split(st, M, k, kk, w.Ph, w.Pl, nullptr, nullptr, nullptr, status);
+    p.err = penalty_tc(st, w.Ph, w.Pl, p.RM, gradM && lambda != 0.f, p.acc + 1, 0, G1.nbT, k, status);
+    if (p.err) return;
   } else if (tc) {
     // R = M M^T - I (symmetric) with its bf16 splits, ||R||_F^2, and R M for the gradient
     KkWS& w = p.kk;
@@ -1541,7 +1569,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       launch_opgrad(st, w.V, G2.d_in, W2, 1, G2.ld, G2, p.gMinv, 0, 1.f, status);  // V side: operator Minv
     }
     if (tc) {
-      minv_path_tc(st, p.gMinv, gradM, G1.nbT, k, true, p.kk, status);
+      p.err = minv_path_tc(st, p.gMinv, gradM, G1.nbT, k, p.kk, status);
     } else {
       launch_kk(st, p.Minv, 1, p.gMinv, 0, p.RM, G1.nbT, k, 1.f, GEMM_STORE, status);
       launch_kk(st, p.RM, 0, p.Minv, 1, gradM, G1.nbT, k, -1.f, GEMM_STORE | GEMM_ACCUM, status);
@@ -1568,7 +1596,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     CQ_LAUNCH(axpy_norm_kernel, grid_for(kk), 256, 0, st, p.gMinv, p.T2, kk, p.acc, 3, (double)n1, 6, status);
   }
   if (tc) {
-    minv_path_tc(st, p.gMinv, gradM, G1.nbT, k, true, p.kk, status);
+    p.err = minv_path_tc(st, p.gMinv, gradM, G1.nbT, k, p.kk, status);
   } else {
     launch_kk(st, p.Minv, 1, p.gMinv, 0, p.RM, G1.nbT, k, 1.f, GEMM_STORE, status);
     launch_kk(st, p.RM, 0, p.Minv, 1, gradM, G1.nbT, k, -1.f, GEMM_STORE | GEMM_ACCUM, status);
@@ -1660,6 +1688,7 @@ extern "C" int cafeq_pair_loss_fwd_bwd(const cafeq_matrix_desc* d1, const void* 
   if (objective == 2) pair_grams((cudaStream_t)stream, W1, G1, W2, G2, p, status);
   pair_step((cudaStream_t)stream, d1, d2, G1, G2, W1, W2, M, P, lse_t, lambda_orth, want_pqe, losses, nullptr,
             want_grad ? gradM : nullptr, status, p, (flags & CAFEQ_FLAG_GENERIC) != 0, false, nullptr, ste, objective);
+  if (p.err) return p.err;
   return last_launch();
 }
 

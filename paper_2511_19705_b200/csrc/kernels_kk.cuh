@@ -425,4 +425,444 @@ __global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* __re
   }
 }
 
+// ------------------------------------------------------------------------------------------------
+// Two chained three-term products of one block with the intermediate kept in shared memory as hi / lo splits:
+//   KK_MINV_PATH:  grad -= (X^T G) X^T     X = M^-1 (hi / lo splits in memory), G = dL/dM^-1: either dense fp32, or for
+//                  Eq. 4 formed here, G[l][j] = scale X[l][j] A_j; the sixteen epilogue warps split it into the operand
+//                  layout while the tensor core works on the previous 64 rows of it
+//   KK_PENALTY:    R = M M^T - I with ||R||_F^2,  out = R M
+// What bounds it: one block's operands (1 MB at k = 256) enter one SM at 60 - 75 GB/s from L2, beside 13 us of products.
+// As separate launches (form G, split it, two products) the splits and the intermediate made the trip through memory
+// and every launch paid its own fill and drain.  Measured (106 blocks of 256): M^-1 path 36 us against 8.5 + 15 + 2 x 20;
+// 72 blocks of 128: 10.7 us against 4.4 + 2 x 9.5.
+// The intermediate T of k = 256 does not fit in shared memory as a whole (256 KB): its accumulators fill tensor memory,
+// each 128-row half is split into shared memory in turn and the second product of that half reuses its columns.
+// Shared memory: T area (4 slots; the split rows of G use it before T exists, two stages of hi + lo) + ring.
+// ------------------------------------------------------------------------------------------------
+enum { KK_MINV_PATH = 0, KK_PENALTY = 1 };
+constexpr int KK_MAX_PROBS = 8;
+
+struct ChainMaps {
+  CUtensorMap a1[2];  // hi / lo, first product: KK_MINV_PATH boxes of 64 x 64, KK_PENALTY boxes of K rows x 64
+  CUtensorMap b2[2];  // hi / lo, second product: KK_MINV_PATH boxes of K rows x 64, KK_PENALTY boxes of 64 x 64
+  CUtensorMap out;    // fp32, boxes of 32 x 32 (KK_MINV_PATH: read and written)
+};
+struct ChainParams {
+  // KK_MINV_PATH: blocks below blk0[n] belong to problems that scale X (blk0[p] <= b < blk0[p + 1]); the others are dense
+  int n;
+  int blk0[KK_MAX_PROBS + 1];
+  const float* A[KK_MAX_PROBS];     // per transformed index, or
+  const float* Agrp[KK_MAX_PROBS];  // per group of g transformed indices
+  int g[KK_MAX_PROBS];
+  float scale[KK_MAX_PROBS];
+  const float* X;                   // fp32 X
+  const float* G;                   // fp32 dense G
+  // KK_PENALTY
+  double* sq;                       // ||R_b||_F^2 is added to sq[b * sq_stride]
+  int sq_stride;
+  int want_out;                     // 0: only the norms
+  int32_t* status;
+};
+
+template <int K>
+struct ChainCfg {
+  static constexpr int HALVES = K / 128;
+  static constexpr int KCH = K / 64;
+  static constexpr int SLOT = K * 128;
+  static constexpr int NRING = (K == 256) ? 3 : 8;
+  static constexpr int NSLOT = NRING + 4;
+  static constexpr int EPI_WARPS = 16;
+  static constexpr int NBAR = 2 * NRING + 4 + 2 + 2 * EPI_WARPS;
+  static constexpr int SMEM = 1024 + NSLOT * SLOT + 8 * NBAR + 64;
+  static constexpr int TMEM_COLS = HALVES * K;
+  static constexpr int THREADS = 64 + 32 * EPI_WARPS;
+};
+
+// fp32 -> hi / lo of 8 consecutive values
+__device__ __forceinline__ void split8(const float* x, uint32_t* h, uint32_t* l) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const __nv_bfloat16 h0 = __float2bfloat16_rn(x[2 * j]), h1 = __float2bfloat16_rn(x[2 * j + 1]);
+    h[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+    l[j] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x[2 * j] - __bfloat162float(h0))) |
+           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x[2 * j + 1] - __bfloat162float(h1))) << 16);
+  }
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+
+template <int K, int MODE>
+__global__ void __launch_bounds__(ChainCfg<K>::THREADS, 1)
+kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainParams p) {
+  using C = ChainCfg<K>;
+  if (p.status && *p.status) return;
+  const int b = blockIdx.x, row_b = b * K;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = (uint64_t*)(smem + C::NSLOT * C::SLOT);
+  const uint32_t bar_full = smem_u32(bars);
+  const uint32_t bar_empty = bar_full + 8 * C::NRING;
+  const uint32_t bar_gfull = bar_empty + 8 * C::NRING;  // two stages of G
+  const uint32_t bar_gempty = bar_gfull + 16;
+  const uint32_t bar_acc = bar_gempty + 16;             // a product is complete
+  const uint32_t bar_t = bar_acc + 8;                   // a half of T is in shared memory
+  const uint32_t bar_c0 = bar_t + 8;                    // two per epilogue warp
+  uint32_t* tmem_slot = (uint32_t*)(bars + C::NBAR);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t sm_u = smem_u32(smem);
+  const uint32_t sT = sm_u, sRing = sm_u + 4 * C::SLOT;
+  const bool second = MODE == KK_MINV_PATH || p.want_out;
+
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&maps.a1[0]);
+    tma_prefetch_desc(&maps.a1[1]);
+    tma_prefetch_desc(&maps.b2[0]);
+    tma_prefetch_desc(&maps.b2[1]);
+    for (int s = 0; s < C::NRING; ++s) {
+      mbar_init(bar_full + 8 * s, 1);
+      mbar_init(bar_empty + 8 * s, 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(bar_gfull + 8 * s, C::EPI_WARPS);
+      mbar_init(bar_gempty + 8 * s, 1);
+    }
+    mbar_init(bar_acc, 1);
+    mbar_init(bar_t, C::EPI_WARPS);
+    for (int s = 0; s < 2 * C::EPI_WARPS; ++s) mbar_init(bar_c0 + 8 * s, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"((uint32_t)C::TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- TMA producer: hi and lo of every 64-entry chunk
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      const int rounds = second ? 1 + C::HALVES : 1;
+      for (int r = 0; r < rounds && ok; ++r) {
+        const bool kmajor = (MODE == KK_MINV_PATH) == (r > 0);  // boxes of K rows x 64 entries, or of 64 x 64
+        for (int c = 0; c < C::KCH && ok; ++c)
+          for (int u = 0; u < 2; ++u, ++it) {
+            const uint32_t s = it % C::NRING, ph = (it / C::NRING) & 1u;
+            if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, p.status)) { ok = false; break; }
+            mbar_expect_tx(bar_full + 8 * s, C::SLOT);
+            const CUtensorMap* m = r ? &maps.b2[u] : &maps.a1[u];
+            const uint32_t dst = sRing + s * C::SLOT;
+            if (kmajor) {
+              tma_load_2d(dst, m, c * 64, row_b, bar_full + 8 * s);
+            } else {
+              for (int j = 0; j < K / 64; ++j) tma_load_2d(dst + j * 8192, m, j * 64, row_b + c * 64, bar_full + 8 * s);
+            }
+          }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer (converged warp, one elected lane)
+    uint32_t it = 0;
+    bool ok = true;
+    auto wait_full = [&](uint32_t i) {
+      return __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * (i % C::NRING), (i / C::NRING) & 1u, abort_flag, p.status)) != 0;
+    };
+    // first product: k x k, three terms
+    for (int c = 0; c < C::KCH && ok; ++c, it += 2) {
+      const uint32_t sh = it % C::NRING, sl = (it + 1) % C::NRING;
+      if constexpr (MODE == KK_MINV_PATH) {
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_gfull + 8 * (c & 1), (c >> 1) & 1u, abort_flag, p.status)) && wait_full(it);
+        if (!ok) break;
+        tc_fence_after();
+        constexpr uint32_t idesc = umma_idesc_bf16(128, K, 1, 1);
+        const uint32_t gh = umma_desc_lo(sT + (c & 1) * 2 * C::SLOT, 8192), gl = gh + (C::SLOT >> 4);
+        if (elect_one()) {
+          const uint32_t xh = umma_desc_lo(sRing + sh * C::SLOT, 8192);
+#pragma unroll
+          for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+              for (int mh = 0; mh < C::HALVES; ++mh)
+                tc_mma_lo(tmem_base + mh * K, xh + mh * 1024 + kk * 128, (t ? gl : gh) + kk * 128, idesc, (c | t | kk) != 0 ? 1u : 0u);
+          tc_commit(bar_empty + 8 * sh);
+        }
+        __syncwarp();
+        ok = wait_full(it + 1);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t xl = umma_desc_lo(sRing + sl * C::SLOT, 8192);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int mh = 0; mh < C::HALVES; ++mh)
+              tc_mma_lo(tmem_base + mh * K, xl + mh * 1024 + kk * 128, gh + kk * 128, idesc, 1u);
+          tc_commit(bar_empty + 8 * sl);
+          tc_commit(bar_gempty + 8 * (c & 1));
+          if (c == C::KCH - 1) tc_commit(bar_acc);
+        }
+        __syncwarp();
+      } else {
+        ok = wait_full(it) && wait_full(it + 1);
+        if (!ok) break;
+        tc_fence_after();
+        constexpr uint32_t idesc = umma_idesc_bf16(128, K, 0, 0);
+        if (elect_one()) {
+          const uint32_t mhi = umma_desc_lo(sRing + sh * C::SLOT), mlo = umma_desc_lo(sRing + sl * C::SLOT);
+#pragma unroll
+          for (int t = 0; t < 3; ++t)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+              for (int mh = 0; mh < C::HALVES; ++mh)
+                tc_mma_lo(tmem_base + mh * K, (t == 1 ? mlo : mhi) + mh * 1024 + kk * 2, (t == 2 ? mlo : mhi) + kk * 2, idesc,
+                          (c | t | kk) != 0 ? 1u : 0u);
+          tc_commit(bar_empty + 8 * sh);
+          tc_commit(bar_empty + 8 * sl);
+          if (c == C::KCH - 1) tc_commit(bar_acc);
+        }
+        __syncwarp();
+      }
+    }
+    // second product: one 128-row half of T at a time
+    constexpr int BMN = (MODE == KK_MINV_PATH) ? 0 : 1;
+    constexpr uint32_t idesc2 = umma_idesc_bf16(128, K, 0, BMN);
+    constexpr uint32_t bstep = BMN ? 128 : 2, lbo = BMN ? 8192 : 16;
+    for (int h = 0; h < C::HALVES && ok && second; ++h) {
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_t, h & 1u, abort_flag, p.status));
+      tc_fence_after();
+      for (int c = 0; c < C::KCH && ok; ++c, it += 2) {
+        const uint32_t sh = it % C::NRING, sl = (it + 1) % C::NRING;
+        const uint32_t th = umma_desc_lo(sT + c * 16384), tl = th + (C::KCH * 16384 >> 4);
+        ok = wait_full(it);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t bh = umma_desc_lo(sRing + sh * C::SLOT, lbo);
+#pragma unroll
+          for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              tc_mma_lo(tmem_base + h * K, (t ? tl : th) + kk * 2, bh + kk * bstep, idesc2, (c | t | kk) != 0 ? 1u : 0u);
+          tc_commit(bar_empty + 8 * sh);
+        }
+        __syncwarp();
+        ok = wait_full(it + 1);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t bl = umma_desc_lo(sRing + sl * C::SLOT, lbo);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) tc_mma_lo(tmem_base + h * K, th + kk * 2, bl + kk * bstep, idesc2, 1u);
+          tc_commit(bar_empty + 8 * sl);
+          if (c == C::KCH - 1) tc_commit(bar_acc);
+        }
+        __syncwarp();
+      }
+    }
+  } else {
+    // ---------------------------------------------------------------- splitting of G, splitting of T, output
+    const int q = warp & 3, ew = warp - 2, part = ew >> 2;
+    const int et = threadIdx.x - 64;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+    bool ok = true;
+    if constexpr (MODE == KK_MINV_PATH) {
+      // a thread owns 8 consecutive columns (the same ones in every row it touches)
+      constexpr int CG = K / 8, NI = 64 * CG / (32 * C::EPI_WARPS);
+      const int cg = et % CG, r0 = et / CG;
+      constexpr int RSTEP = 32 * C::EPI_WARPS / CG;
+      int prob = -1;
+      for (int q2 = 0; q2 < p.n; ++q2)
+        if (b >= p.blk0[q2] && b < p.blk0[q2 + 1]) prob = q2;
+      float mul[8];
+      const float* src = (prob >= 0 ? p.X : p.G) + (size_t)b * K * K + cg * 8;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) mul[j] = 1.f;
+      if (prob >= 0) {
+        const int t0 = (b - p.blk0[prob]) * K + cg * 8;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          mul[j] = p.scale[prob] * (p.Agrp[prob] ? p.Agrp[prob][(t0 + j) / p.g[prob]] : p.A[prob][t0 + j]);
+      }
+      float4 nx[NI][2];
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const float4* s4 = reinterpret_cast<const float4*>(src + (size_t)(r0 + i * RSTEP) * K);
+        nx[i][0] = s4[0];
+        nx[i][1] = s4[1];
+      }
+#pragma unroll 1
+      for (int c = 0; c < C::KCH && ok; ++c) {
+        const uint32_t gb = sT + (c & 1) * 2 * C::SLOT;
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_gempty + 8 * (c & 1), ((c >> 1) & 1u) ^ 1u, abort_flag, p.status));
+        if (!ok) break;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          const int r = r0 + i * RSTEP;
+          const float x[8] = {nx[i][0].x * mul[0], nx[i][0].y * mul[1], nx[i][0].z * mul[2], nx[i][0].w * mul[3],
+                              nx[i][1].x * mul[4], nx[i][1].y * mul[5], nx[i][1].z * mul[6], nx[i][1].w * mul[7]};
+          uint32_t h[4], l[4];
+          split8(x, h, l);
+          const uint32_t o = gb + (cg >> 3) * 8192 + r * 128 + (((cg & 7) ^ (r & 7)) << 4);
+          sts128(o, h);
+          sts128(o + C::SLOT, l);
+        }
+        if (c + 1 < C::KCH) {
+#pragma unroll
+          for (int i = 0; i < NI; ++i) {
+            const float4* s4 = reinterpret_cast<const float4*>(src + (size_t)((c + 1) * 64 + r0 + i * RSTEP) * K);
+            nx[i][0] = s4[0];
+            nx[i][1] = s4[1];
+          }
+        }
+        fence_proxy_async_smem_tb();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_gfull + 8 * (c & 1));
+      }
+    }
+    constexpr int CPH = K / 32;
+    double sq = 0.0;
+    for (int h = 0; h < C::HALVES && ok; ++h) {
+      // h = 0: T is complete; later: the second product of the previous half has finished reading the T area
+      if (h == 0 || second) ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, h & 1u, abort_flag, p.status));
+      if (!ok) break;
+      tc_fence_after();
+      float sq4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int ch = part; ch < CPH; ch += 4) {
+        const int m = q * 32 + lane, col0 = ch * 32;
+        float v[32];
+        tc_ld32(taddr + h * K + col0, v);
+        if constexpr (MODE == KK_PENALTY) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            if (col0 + e == h * 128 + m) v[e] -= 1.f;
+            sq4[e & 3] = fmaf(v[e], v[e], sq4[e & 3]);
+          }
+        }
+        if (second) {
+          const uint32_t rowp = sT + (col0 >> 6) * 16384 + m * 128;
+          const int c16 = (col0 & 63) >> 3;
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            uint32_t hh[4], ll[4];
+            split8(v + 8 * w, hh, ll);
+            const uint32_t o = rowp + (((c16 + w) ^ (m & 7)) << 4);
+            sts128(o, hh);
+            sts128(o + C::KCH * 16384, ll);
+          }
+        }
+      }
+      if constexpr (MODE == KK_PENALTY) sq += (double)((sq4[0] + sq4[1]) + (sq4[2] + sq4[3]));
+      fence_proxy_async_smem_tb();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0 && second) mbar_arrive(bar_t);
+    }
+    if constexpr (MODE == KK_PENALTY) {
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      if (ok && lane == 0 && sq != 0.0) atomicAdd(p.sq + (long long)b * p.sq_stride, sq);
+    }
+    if (ok && second) ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, C::HALVES & 1u, abort_flag, p.status));
+    if (ok && second) {
+      tc_fence_after();
+      const uint32_t tB = sm_u + ew * 8192, bc0 = bar_c0 + 16 * ew;  // two fp32 tiles per warp (every slot is free now)
+      constexpr int NU = C::HALVES * CPH / 4;
+      auto tile_of = [&](int i, int& mh, int& ch) { const int c2 = part + i * 4; mh = c2 / CPH; ch = c2 - mh * CPH; };
+      const int sw = lane & 7;
+      if (MODE == KK_MINV_PATH && lane == 0) {
+        int mh, ch;
+        tile_of(0, mh, ch);
+        mbar_expect_tx(bc0, 4096);
+        tma_load_2d(tB, &maps.out, ch * 32, row_b + mh * 128 + q * 32, bc0);
+      }
+#pragma unroll 1
+      for (int i = 0; i < NU && ok; ++i) {
+        int mh, ch;
+        tile_of(i, mh, ch);
+        const uint32_t t = tB + (i & 1) * 4096;
+        float v[32];
+        tc_ld32(taddr + mh * K + ch * 32, v);
+        if constexpr (MODE == KK_MINV_PATH) {
+          ok = __all_sync(0xffffffffu, mbar_wait(bc0 + 8 * (i & 1), (i >> 1) & 1u, abort_flag, p.status));
+          if (!ok) break;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            float4 x;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
+                         : "r"(t + lane * 128 + ((c ^ sw) << 4)));
+            v[4 * c] = x.x - v[4 * c];
+            v[4 * c + 1] = x.y - v[4 * c + 1];
+            v[4 * c + 2] = x.z - v[4 * c + 2];
+            v[4 * c + 3] = x.w - v[4 * c + 3];
+          }
+        }
+        if (lane == 0) {
+          tma_store_wait_read();  // the previous tile's store has read the other buffer
+          if (MODE == KK_MINV_PATH && i + 1 < NU) {
+            int mh2, ch2;
+            tile_of(i + 1, mh2, ch2);
+            const uint32_t bn = bc0 + 8 * ((i + 1) & 1);
+            mbar_expect_tx(bn, 4096);
+            tma_load_2d(tB + ((i + 1) & 1) * 4096, &maps.out, ch2 * 32, row_b + mh2 * 128 + q * 32, bn);
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(t + lane * 128 + ((c ^ sw) << 4)), "f"(v[4 * c]),
+                       "f"(v[4 * c + 1]), "f"(v[4 * c + 2]), "f"(v[4 * c + 3])
+                       : "memory");
+        fence_proxy_async_smem_tb();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&maps.out, t, ch * 32, row_b + mh * 128 + q * 32);
+          tma_store_commit();
+        }
+      }
+      if (lane == 0) tma_store_wait_all();
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+  }
+}
+
+template <int K, int MODE>
+static int kk_chain_launch_t(cudaStream_t st, const ChainMaps& maps, int nb, const ChainParams& p) {
+  using C = ChainCfg<K>;
+  static std::atomic<unsigned long long> done{0};
+  if (!opt_in_smem(kk_chain_kernel<K, MODE>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
+  kk_chain_kernel<K, MODE><<<nb, C::THREADS, C::SMEM, st>>>(maps, p);
+  return CAFEQ_OK;
+}
+
+// hi, lo: splits of X (KK_MINV_PATH) or M (KK_PENALTY), bf16 [nb * k, k]; out fp32 [nb, k, k]
+static int kk_chain_launch(cudaStream_t st, int mode, const uint16_t* hi, const uint16_t* lo, float* out, int nb, int k,
+                           const ChainParams& p) {
+  ChainMaps m;
+  const long long rows = (long long)nb * k;
+  const int box1 = mode == KK_MINV_PATH ? 64 : k, box2 = mode == KK_MINV_PATH ? k : 64;
+  if (!make_map_bf16(&m.a1[0], hi, k, rows, k, box1) || !make_map_bf16(&m.a1[1], lo, k, rows, k, box1) ||
+      !make_map_bf16(&m.b2[0], hi, k, rows, k, box2) || !make_map_bf16(&m.b2[1], lo, k, rows, k, box2) ||
+      !make_map_2d(&m.out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, out, k, rows, k, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B))
+    return CAFEQ_ERR_UNSUPPORTED;
+  if (mode == KK_MINV_PATH) return k == 256 ? kk_chain_launch_t<256, KK_MINV_PATH>(st, m, nb, p) : kk_chain_launch_t<128, KK_MINV_PATH>(st, m, nb, p);
+  return k == 256 ? kk_chain_launch_t<256, KK_PENALTY>(st, m, nb, p) : kk_chain_launch_t<128, KK_PENALTY>(st, m, nb, p);
+}
+
 }  // namespace cafeq

@@ -117,36 +117,6 @@ __global__ void __launch_bounds__(256) layer_colnorm_kernel(const float* __restr
   }
 }
 
-// dL/dMinv of Eq. 4 for all single matrices: out[b][i][t] = scale_p * Minv[b][i][t] * A_t, A_t from the matrix's
-// group sums (input axis, one block per operator block) or from its per-row sums.
-struct LyGminvArgs {
-  int n, k;
-  int blk0[LY_MAX_PROBS + 1];
-  const float* A[LY_MAX_PROBS];
-  const float* Agrp[LY_MAX_PROBS];
-  int g[LY_MAX_PROBS];
-  float scale[LY_MAX_PROBS];
-};
-
-__global__ void __launch_bounds__(256) layer_gminv_kernel(const float* __restrict__ Minv, float* __restrict__ out, const LyGminvArgs a) {
-  const long long kk = (long long)a.k * a.k;
-  const long long total4 = (long long)a.blk0[a.n] * kk / 4;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total4; q += (long long)gridDim.x * blockDim.x) {
-    const long long e = q * 4;
-    const int b = (int)(e / kk);
-    int p = 0;
-    while (b >= a.blk0[p + 1]) ++p;
-    const int t = (int)(e % a.k);
-    const int bl = b - a.blk0[p];
-    float At[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) At[j] = a.Agrp[p] ? a.Agrp[p][(bl * a.k + t + j) / a.g[p]] : a.A[p][bl * a.k + t + j];
-    const float4 x = *reinterpret_cast<const float4*>(Minv + e);
-    const float sc = a.scale[p];
-    *reinterpret_cast<float4*>(out + e) = make_float4(sc * x.x * At[0], sc * x.y * At[1], sc * x.z * At[2], sc * x.w * At[3]);
-  }
-}
-
 // LogSumExp over the group maxima of both factors of every pair (blockIdx.y = pair): unnormalised routed
 // coefficients exp(t (a - max)) * sign(U at the arg-max) and Z = sum exp(t (a - max)); the maximum comes from the
 // transform passes (one word per matrix).
@@ -549,9 +519,8 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
   }
   bool any_lambda = false;
   for (int q = 0; q < L.n; ++q) any_lambda |= (L.p[q].pair && L.p[q].cfg.lambda_orth != 0.f);
-  // The pair blocks' penalty chain (splits of the parameters, R = M M^T - I, R M) does not depend on the inverse:
-  // it runs on a side stream beside the Newton-Schulz chain (both are chains of short, latency-bound launches that
-  // leave SMs idle) and joins before the transform pass, which reads bf16(M)^T.  Event record / wait pairs only, so
+  // The pair blocks' penalty (splits of the parameters, R = M M^T - I, R M) does not depend on the inverse: it runs on a
+  // side stream beside it (one CTA per block leaves SMs idle) and joins before the transform pass, which reads bf16(M)^T.  Event record / wait pairs only, so
   // the fork and the join are captured with the step when the caller's stream is being captured.
   LyAux* aux = (nbP > 0 && g_ly_dual.load(std::memory_order_relaxed) && w_mn_expected(k)) ? ly_aux() : nullptr;
   cudaStream_t so = st;
@@ -559,25 +528,16 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
     if (cudaEventRecord(aux->fork, st) != cudaSuccess || cudaStreamWaitEvent(aux->stream, aux->fork, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
     so = aux->stream;
   }
+  // (enqueued first: its CTAs run longer than the penalty's)
+  ns_inverse(st, L.Mc, L.Minv, nullptr, NB, k, true, w, status, true, true);
   if (nbP > 0) {
     // pair blocks: splits of the fp32 parameters (the transposed high halves are bf16(M)^T, the operator of the
-    // first factors' pass), R = M M^T - I with ||R_b||_F^2 per block, and R M for the penalty's gradient.
-    // On the side stream R's splits live in the transposed-split arrays, which the row-major refinement leaves unused
-    // (the Newton-Schulz chain writes its own residual into RTh meanwhile).
-    uint16_t* Rh = (aux ? w.XTh[0] : w.RTh) + offP;
-    uint16_t* Rl = (aux ? w.XTl[0] : w.RTl) + offP;
-    launch_split(so, L.Mf, k, (long long)nbP * kk1, w.Ph + offP, w.Pl + offP, w.Qh + offP, w.Ql + offP, nullptr, status);
-    const uint16_t* a1[3] = {w.Ph + offP, w.Pl + offP, w.Ph + offP};
-    const uint16_t* b1[3] = {w.Ph + offP, w.Ph + offP, w.Pl + offP};
-    launch_kk_tc(so, 3, a1, b1, nbP, k, 1.f, 0.f, -1.f, nullptr, nullptr, Rh, Rl, nullptr, nullptr, L.orth_sq, nullptr, status, 1);
-    if (any_lambda) {
-      const uint16_t* a2[3] = {Rh, Rl, Rh};
-      const uint16_t* b2[3] = {w.Qh + offP, w.Qh + offP, w.Ql + offP};
-      launch_kk_tc(so, 3, a2, b2, nbP, k, 1.f, 0.f, 0.f, nullptr, L.RM, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status);
-    }
+    // first factors' pass), then the penalty's norm and (M M^T - I) M in one launch
+    launch_split(so, L.Mf, k, (long long)nbP * kk1, w.Ph + offP, w.Pl + offP, w.Qh + offP, nullptr, nullptr, status);
+    const int rc = penalty_tc(so, w.Ph + offP, w.Pl + offP, L.RM, any_lambda, L.orth_sq, 1, nbP, k, status);
+    if (rc) return rc;
   }
   if (aux && cudaEventRecord(aux->join, aux->stream) != cudaSuccess) return CAFEQ_ERR_CUDA;
-  ns_inverse(st, L.Mc, L.Minv, nullptr, NB, k, true, w, status, true, true);
   if (aux && cudaStreamWaitEvent(st, aux->join, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
   // Eq. 4 weights of the single matrices (they own the first pair_blk0 blocks)
   if (L.pair_blk0 > 0) {
@@ -741,11 +701,10 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
         }
     }
   }
-  // dL/dMinv of Eq. 4 for the singles, then grad -= Minv^T (dL/dMinv) Minv^T over all blocks
-  if (L.pair_blk0 > 0) {
-    LyGminvArgs ga;
-    memset(&ga, 0, sizeof(ga));
-    ga.k = k;
+  // grad -= Minv^T (dL/dMinv) Minv^T over all blocks; the singles' dL/dMinv (Eq. 4) is formed from Minv by the kernel
+  {
+    ChainParams cp;
+    memset(&cp, 0, sizeof(cp));
     int ns = 0;
     for (int q = 0; q < L.n; ++q) {
       const LyProb& P = L.p[q];
@@ -754,18 +713,19 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
       const Geo& G = Mt.G;
       const bool in_r1 = (G.axis == CAFEQ_AXIS_IN && G.r == 1);
       if (G.axis == CAFEQ_AXIS_IN && !in_r1) CQ_LAUNCH(expand_agrp_kernel, (G.d_in + 127) / 128, 128, 0, st, Mt.agrp, G.d_in, G.g, k, G.r, Mt.A);
-      ga.blk0[ns] = P.blk0;
-      ga.A[ns] = Mt.A;
-      ga.Agrp[ns] = in_r1 ? Mt.agrp : nullptr;
-      ga.g[ns] = G.g;
-      ga.scale[ns] = 2.f * P.kappa;
+      cp.blk0[ns] = P.blk0;
+      cp.A[ns] = Mt.A;
+      cp.Agrp[ns] = in_r1 ? Mt.agrp : nullptr;
+      cp.g[ns] = G.g;
+      cp.scale[ns] = 2.f * P.kappa;
       ++ns;
     }
-    ga.blk0[ns] = L.pair_blk0;
-    ga.n = ns;
-    CQ_LAUNCH(layer_gminv_kernel, grid_for((long long)L.pair_blk0 * kk1 / 4), 256, 0, st, L.Minv, L.gMinv, ga);
+    cp.blk0[ns] = L.pair_blk0;
+    cp.n = ns;
+    cp.X = L.Minv;
+    const int rc = minv_path_tc(st, L.gMinv, L.grad, NB, k, w, status, &cp);
+    if (rc) return rc;
   }
-  minv_path_tc(st, L.gMinv, L.grad, NB, k, true, w, status);
   {
     LyFinishArgs f;
     memset(&f, 0, sizeof(f));
