@@ -70,7 +70,11 @@ struct BwCfg {
   static constexpr int S_TERM_BYTES = K * 64 * 2;  // S tile: K targets x 64 contraction entries, K-major, one 16-bit term
   static constexpr int S_BUF_BYTES = TERMS * S_TERM_BYTES;
   static constexpr int TMEM_COLS = HALVES * K;     // 128 or 512
-  static constexpr int SMEM = 1024 + NSTAGE * STAGE_BYTES + 2 * S_BUF_BYTES + 256;
+  // Records in flight per builder thread (8 bytes each, copied to shared memory ahead of their tile); the two-term form
+  // at K = 256 has no shared memory left for them and holds the next tile's record in registers.
+  static constexpr int RDEPTH = (K == 256 && !F16) ? 0 : 4;
+  static constexpr int REC_BYTES = RDEPTH * 256 * 8;
+  static constexpr int SMEM = 1024 + NSTAGE * STAGE_BYTES + 2 * S_BUF_BYTES + REC_BYTES + 256;
 };
 
 // instruction descriptor for fp16 operands (format field 0), fp32 accumulation
@@ -119,7 +123,8 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sStage = smem;
   uint8_t* sS = smem + C::NSTAGE * C::STAGE_BYTES;
-  uint64_t* bars = (uint64_t*)(sS + 2 * C::S_BUF_BYTES);
+  uint8_t* sRec = sS + 2 * C::S_BUF_BYTES;
+  uint64_t* bars = (uint64_t*)(sRec + C::REC_BYTES);
   // barrier slots: wfull[NSTAGE], wempty[NSTAGE], sfull[2], sempty[2], accf, acce
   const uint32_t bar_wfull = smem_u32(bars);
   const uint32_t bar_wempty = bar_wfull + 8 * C::NSTAGE;
@@ -255,59 +260,85 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
     // ---------------------------------------------------------------- operand builders (one record per thread and tile) and flush
     const int bt = threadIdx.x - 64;
     const int q = warp & 3, hw = (warp - 2) >> 2;
-    // The record of the NEXT tile is requested one tile ahead and only its raw words are kept: nothing may depend on
-    // them before the next iteration, or the thread would sit out the whole memory latency here, once per tile.
-    float rawC = 0.f;     // coefficient word
-    int rawI = 0;         // arg-max word
-    int rawBase = -1;     // input axis: column offset of this thread's group inside the block; output axis: first
-                          // column of the group minus the tile's first column; -1: no record for this thread
-    int rawKK = 0;        // input axis: contraction index (row inside the tile); output axis: target row
-    float rawScale = 1.f;
-    auto load_rec = [&](int sub, int tile) {
-      const BwParams& p = mp.p[sub];
-      const int major = tile / p.n_minor, t = tile - major * p.n_minor;
-      rawBase = -1;
-      rawC = 0.f;
-      rawI = 0;
+    // Position in the tile list, advanced without divisions: sub-problem, block, tile of the block.
+    struct Cursor { int gt, sub, major, t; };
+    auto advance = [&](Cursor& c) {
+      ++c.gt;
+      if (++c.t == mp.p[c.sub].n_minor) { c.t = 0; ++c.major; }
+      if (c.gt == mp.tile_end[c.sub] && c.gt < total_tiles) { ++c.sub; c.major = c.t = 0; }
+    };
+    // This thread's record of a tile: address (-1: none), and where its entry of S goes.
+    //   input axis: tile row bt & 63, group bt >> 6 of the block; column offset of that group inside the block
+    //   output axis: block row bt; first column of the row's group minus the tile's first column
+    auto rec_at = [&](const Cursor& c, int& colbase) -> long long {
+      const BwParams& p = mp.p[c.sub];
       if constexpr (FORM == BW_IN) {
         const int rl = bt & 63, qq = bt >> 6;
-        const int row = t * 64 + rl;
-        const int G0 = (major * K) / p.g;
+        const int row = c.t * 64 + rl;
+        const int G0 = (K >= p.g) ? c.major * p.NG : (c.major * K) / p.g;
         const int G = G0 + qq;
-        if (qq < p.NG && row < p.d_out && G < p.ng) {
-          const long long pi = p.gm ? (long long)G * p.d_out + row : (long long)row * p.ng + G;
-          rawC = __ldg(p.coef + pi);
-          rawI = __ldg(p.idx + pi);
-          rawBase = qq * p.g + (G0 * p.g - major * K) + (1 << 20);  // kept non-negative: the offset can be below zero
-          rawKK = rl;
-        }
+        colbase = G * p.g - c.major * K;
+        if (qq >= p.NG || row >= p.d_out || G >= p.ng) return -1;
+        return p.gm ? (long long)G * p.d_out + row : (long long)row * p.ng + G;
       } else {
-        if (bt < K) {
-          const int row = major * K + bt;
-          const int G = (t * 64) / p.g;
-          const long long pi = p.gm ? (long long)G * p.d_out + row : (long long)row * p.ng + G;
-          rawC = __ldg(p.coef + pi);
-          rawI = __ldg(p.idx + pi);
-          rawBase = G * p.g - t * 64 + (1 << 20);
-          rawKK = bt;
-        }
+        const int row = c.major * K + bt;
+        const int G = (p.g == 64) ? c.t : ((p.g == 128) ? c.t >> 1 : (c.t * 64) / p.g);
+        colbase = G * p.g - c.t * 64;
+        if (bt >= K) return -1;
+        return p.gm ? (long long)G * p.d_out + row : (long long)row * p.ng + G;
       }
-      if constexpr (F16) rawScale = bw_coef_scale(p.coefmax);
     };
-    // the record requested one iteration ago, decoded: coefficient, target row, contraction index (tg < 0: none)
-    auto take_rec = [&](float& cf, int& tg, int& kk) {
-      cf = 0.f;
-      tg = -1;
-      kk = 0;
-      if (rawBase >= 0) {
-        const int col = rawBase - (1 << 20) + rawI;
-        if constexpr (FORM == BW_IN) {
-          if (rawC != 0.f && (unsigned)col < (unsigned)K) { cf = rawC; tg = col; kk = rawKK; }
+    // What bounds the builders: fence.proxy.async waits for every load that the thread has in flight, so a record that is
+    // requested as a plain load ahead of the fence costs its whole memory latency once per tile (measured: 2100 cycles per
+    // tile in the builders against 1400 for the tile's weights from HBM; 700 now, and the whole backward of a 9B-shaped
+    // layer 133 -> 112 us, of a 27B-shaped one with groups of 64 371 -> 262 us).  Records are therefore copied to shared memory
+    // with cp.async, RDEPTH tiles ahead; a thread reads only what it copied itself, so no barrier is involved.  Without
+    // room for the ring the load is issued after the fence of the current tile and used before the fence of the next.
+    uint8_t* const my_rec = sRec + bt * 8;
+    Cursor ahead;
+    uint32_t pre = 0;          // tiles whose record has been requested
+    float rawC = 0.f;
+    int rawI = 0;
+    auto request = [&]() {
+      if (ahead.gt < t_end) {
+        int cb;
+        const long long pi = rec_at(ahead, cb);
+        const BwParams& p = mp.p[ahead.sub];
+        if constexpr (C::RDEPTH > 0) {
+          if (pi >= 0) {
+            uint8_t* dst = my_rec + (pre % C::RDEPTH) * 2048;
+            cp_async4(dst, p.coef + pi);
+            cp_async4(dst + 4, p.idx + pi);
+          }
         } else {
-          if (rawC != 0.f && (unsigned)col < 64u) { cf = rawC; tg = rawKK; kk = col; }
+          rawC = 0.f;
+          if (pi >= 0) { rawC = __ldg(p.coef + pi); rawI = __ldg(p.idx + pi); }
         }
+        advance(ahead);
       }
-      if constexpr (F16) cf *= rawScale;
+      if constexpr (C::RDEPTH > 0) cp_async_commit();
+      ++pre;
+    };
+    // record of the current tile, decoded: coefficient, target row, contraction index (tg < 0: none)
+    auto take_rec = [&](const Cursor& c, uint32_t tl, float scale, float& cf, int& tg, int& kk) {
+      tg = -1;
+      int cb, ix;
+      const long long pi = rec_at(c, cb);
+      if constexpr (C::RDEPTH > 0) {
+        cp_async_wait<C::RDEPTH - 1>();
+        asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=f"(cf), "=r"(ix) : "r"(smem_u32(my_rec) + (tl % C::RDEPTH) * 2048));
+      } else {
+        cf = rawC;
+        ix = rawI;
+      }
+      if (pi < 0 || cf == 0.f) return;
+      const int col = cb + ix;
+      if constexpr (FORM == BW_IN) {
+        if ((unsigned)col < (unsigned)K) { tg = col; kk = bt & 63; }
+      } else {
+        if ((unsigned)col < 64u) { tg = bt; kk = col; }
+      }
+      if constexpr (F16) cf *= scale;
     };
     // flush of one block: accumulators -> global memory, coalesced atomic adds straight from the registers
     // (accumulator row m = this thread's lane, 32 consecutive columns n per load)
@@ -339,23 +370,24 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
     };
 
     uint32_t prevA = BW_NONE, prevB = BW_NONE;  // offsets this thread wrote into S buffer 0 / 1
-    int sub = s_first;
-    int cur_sub = s_first, cur_major = (t_begin - (s_first ? mp.tile_end[s_first - 1] : 0)) / mp.p[s_first].n_minor;
-    uint32_t run = 0, tl = 0;
+    const int tile0 = t_begin - (s_first ? mp.tile_end[s_first - 1] : 0);
+    Cursor cur{t_begin, s_first, tile0 / mp.p[s_first].n_minor, tile0 % mp.p[s_first].n_minor};
+    ahead = cur;
+    int cur_sub = s_first, cur_major = cur.major;
+    uint32_t run = 0;
     bool ok = true;
-    load_rec(sub, t_begin - (sub ? mp.tile_end[sub - 1] : 0));
-    for (int gt = t_begin; gt < t_end && ok; ++gt, ++tl) {
-      while (gt >= mp.tile_end[sub]) ++sub;
-      const int tile = gt - (sub ? mp.tile_end[sub - 1] : 0);
-      const int major = tile / mp.p[sub].n_minor;
+    float scale = 1.f;
+    if constexpr (F16) scale = bw_coef_scale(mp.p[s_first].coefmax);
+    for (int i = 0; i < (C::RDEPTH > 0 ? C::RDEPTH : 1); ++i) request();
+    for (uint32_t tl = 0; cur.gt < t_end && ok; ++tl) {
+      const int sub = cur.sub, major = cur.major;
+      if constexpr (F16) {
+        if (sub != cur_sub) scale = bw_coef_scale(mp.p[sub].coefmax);
+      }
       float cf;
       int tg, kk;
-      take_rec(cf, tg, kk);
-      if (gt + 1 < t_end) {
-        int sn = sub;
-        while (gt + 1 >= mp.tile_end[sn]) ++sn;
-        load_rec(sn, gt + 1 - (sn ? mp.tile_end[sn - 1] : 0));
-      }
+      take_rec(cur, tl, scale, cf, tg, kk);
+      advance(cur);
       const uint32_t b = tl & 1u, sph = (tl >> 1) & 1u;
       if (major != cur_major || sub != cur_sub) {
         if (!flush(cur_sub, cur_major, run)) { ok = false; break; }
@@ -387,6 +419,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
       if (b) prevB = now; else prevA = now;
       fence_proxy_async_smem();
       mbar_arrive(bar_sfull + 8 * b);
+      request();
     }
     if (ok) flush(cur_sub, cur_major, run);
   }
