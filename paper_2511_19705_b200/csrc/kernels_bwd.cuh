@@ -295,7 +295,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
     // with cp.async, RDEPTH tiles ahead; a thread reads only what it copied itself, so no barrier is involved.  Without
     // room for the ring the load is issued after the fence of the current tile and used before the fence of the next.
     uint8_t* const my_rec = sRec + bt * 8;
-    Cursor ahead;
+    Cursor ahead{};
     uint32_t pre = 0;          // tiles whose record has been requested
     float rawC = 0.f;
     int rawI = 0;

@@ -6,8 +6,8 @@
 // X through a TMA ring; accumulators are double-buffered in tensor memory so the epilogue of tile t overlaps
 // the products of tile t+1.
 //
-// Warp roles (320 threads): warp 0 = TMA producer, warp 1 = MMA issuer (and tensor-memory owner),
-// warps 2..9 = epilogue (two warps per 32-lane quarter, each owning 128 accumulator columns).
+// Warp roles (576 threads): warp 0 = TMA producer, warp 1 = MMA issuer (and tensor-memory owner), warps 2..9 and 10..17 =
+// two epilogue sets, one per accumulator buffer (two warps per 32-lane quarter, each owning 128 accumulator columns).
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises CAFEQ_ERR_TIMEOUT in the status
 // word, all roles leave their loops, tensor memory is released and the kernel returns.
 #pragma once
@@ -27,6 +27,9 @@ namespace cafeq {
 
 enum { BD_IN = 0, BD_OUT = 1 };
 enum { EPI_ABSMAX = 1, EPI_DELTA = 2, EPI_CODES = 4, EPI_SQSUM = 8, EPI_SURR = 16, EPI_STORE = 32 };
+// compile-time kind of the epilogue: per-group records (ABSMAX, with or without SURR), records and residual, codes and
+// scales only, the transformed matrix itself, its sum of squares
+enum { BD_REC = 0, BD_DELTA = 1, BD_CODES = 2, BD_STORE = 3, BD_SQSUM = 4 };
 
 struct BdParams {
   int d_out, d_in;     // shape of X
@@ -70,7 +73,7 @@ struct BdMulti {
   BdParams p[BD_MAX_SUB];     // all share one status word
 };
 
-constexpr int BD_THREADS = 320;
+constexpr int BD_THREADS = 64 + 2 * 256;
 constexpr int BD_STAGE_BYTES = 16384;  // one TMA box: 64 columns x 128 rows of bf16
 constexpr int BD_STAGES_PER_TILE = 4;
 constexpr uint64_t BD_WAIT_NS = 2000000000ull;
@@ -207,29 +210,37 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// The same load without the wait, and a wait that names the destination registers so that no use of them can be
-// scheduled ahead of it: lets the load of the next 32 columns overlap the arithmetic on the current ones.
-__device__ __forceinline__ void tc_ld32_issue(uint32_t taddr, float* v) {
+// 16 columns
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
   uint32_t* r = reinterpret_cast<uint32_t*>(v);
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tc_ld_wait32(float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
-                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
-                 "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
-                 "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-               :
-               : "memory");
+
+// 32 bytes per lane: one whole sector (the lanes' rows are far apart in memory, so narrower stores are partial sectors).
+// Bases that are not 32-byte aligned take 16-byte pieces.
+__device__ __forceinline__ void store32(void* dst, const uint32_t* v, bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+  } else {
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    d[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    d[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
+}
+
+// max of m, |a| and |b|; a NaN stays
+__device__ __forceinline__ float max_abs2(float m, float a, float b) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(a), "f"(b));
+  return r;
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle, rows of 128 bytes, 8-row groups 1024 bytes apart.
@@ -271,13 +282,14 @@ struct BdCfg {
   static constexpr int KH = (K >= 128) ? K / 128 : 1;                 // OUT: 128-row halves of the block
   static constexpr int NC = 256 / KH;                                 // OUT: d_in columns per tile
   static constexpr int NCC = NC / 64;                                 // OUT: 64-column chunks per tile
-  static constexpr int NSTAGE = 6;                                    // even: the output-axis form consumes stages in pairs
+  // as many stages as fit (even: the output-axis form consumes stages in pairs)
+  static constexpr int NSTAGE = (T_BYTES > 65536) ? 6 : ((T_BYTES > 32768) ? 10 : 12);
   static constexpr int SMEM = 1024 + T_BYTES + NSTAGE * BD_STAGE_BYTES + 256;
 };
 
 // The body takes the CTA's index and the number of CTAs that share its tile list, so that one launch can run two
 // lists side by side (bd_pass_dual_kernel below).
-template <int FORM, int K, int G>
+template <int FORM, int K, int G, int MODE>
 __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& mp, const int cta, const int ncta) {
   using C = BdCfg<FORM, K, G>;
   static_assert(K == 64 || K == 128 || K == 256, "block size");
@@ -389,379 +401,448 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    // The whole warp runs the loop and one elected lane issues (operands in uniform registers, descriptors stepped by one
+    // 32-bit addition): beside the epilogue warps a single lane that builds 64-bit descriptors took 240 cycles per
+    // instruction against the 128 that a 128 x 256 x 16 product lasts.
+    {
       bool ok = true;
       uint32_t tfulls = 0;
       constexpr uint32_t idesc_in = umma_idesc_bf16(128, K, 0, 0);
       constexpr uint32_t idesc_out = umma_idesc_bf16(128, 128, 0, 1);
-      const uint32_t sT_u = smem_u32(sT), sSt_u = smem_u32(sStage);
-      uint32_t it = 0, tl = 0;
+      const uint32_t sSt_u = smem_u32(sStage);
+      const uint32_t tlo = umma_desc_lo(smem_u32(sT));
+      uint32_t st = 0, sph = 0, tl = 0;  // stage, its phase, tile
+      auto next = [&]() { if (++st == C::NSTAGE) { st = 0; sph ^= 1u; } };
+      auto wait_all = [&](uint32_t bar, uint32_t ph) { return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_flag, status)) != 0; };
       for (int sub = s_first; sub < mp.n && ok; ++sub) {
         const int base = sub ? mp.tile_end[sub - 1] : 0;
         if (base >= t_end) break;
         const int n_minor = mp.p[sub].n_minor;
         const int lo = (t_begin > base ? t_begin : base) - base;
         const int hi = (t_end < mp.tile_end[sub] ? t_end : mp.tile_end[sub]) - base;
-        int cur_major = -1;
+        int left = 0;  // tiles of this sub-problem left on the current operator block
         for (int tile = lo; tile < hi && ok; ++tile, ++tl) {
-          const int major = tile / n_minor;
-          const bool fresh = major != cur_major;  // first tile on a newly loaded operator block
+          const bool fresh = left == 0;  // first tile on a newly loaded operator block
+          if (fresh) left = n_minor - (tile == lo ? lo % n_minor : 0);
           const uint32_t tph = tfulls & 1u;
           if (fresh) {
             if constexpr (FORM == BD_OUT) {
-              for (int c = 0; c < K / 64 && ok; ++c) ok = mbar_wait(bar_tfull + 8 * c, tph, abort_flag, status);
+              for (int c = 0; c < K / 64 && ok; ++c) ok = wait_all(bar_tfull + 8 * c, tph);
               if (!ok) break;
             }
             ++tfulls;
-            cur_major = major;
           }
           const uint32_t buf = tl & 1u, aph = (tl >> 1) & 1u;
-          if (!mbar_wait(bar_acce + 8 * buf, aph ^ 1u, abort_flag, status)) { ok = false; break; }
+          ok = wait_all(bar_acce + 8 * buf, aph ^ 1u);
+          if (!ok) break;
           tc_fence_after();
           const uint32_t dbase = tmem_base + buf * 256u;
           if constexpr (FORM == BD_IN) {
-            for (int sidx = 0; sidx < BD_STAGES_PER_TILE; ++sidx, ++it) {
-              const uint32_t s = it % C::NSTAGE, ph = (it / C::NSTAGE) & 1u;
-              if (!mbar_wait(bar_full + 8 * s, ph, abort_flag, status)) { ok = false; break; }
-              // stage sidx multiplies the operator's chunk sidx
-              if (fresh && !mbar_wait(bar_tfull + 8 * sidx, tph, abort_flag, status)) { ok = false; break; }
-              tc_fence_after();
-              const uint32_t stage = sSt_u + s * BD_STAGE_BYTES;
-              const int bi = (sidx * 64) / K, ci = ((sidx * 64) % K) / 64;
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t ad = umma_desc_sw128(stage + kk * 32);
-                const uint64_t bd = umma_desc_sw128(sT_u + bi * K * K * 2 + ci * K * 128 + kk * 32);
-                tc_mma_bf16(dbase + bi * K, ad, bd, idesc_in, (ci | kk) != 0 ? 1u : 0u);
+            for (int sidx = 0; sidx < BD_STAGES_PER_TILE; ++sidx) {
+              ok = wait_all(bar_full + 8 * st, sph);
+              // stage sidx multiplies the operator's chunk sidx
+              if (ok && fresh) ok = wait_all(bar_tfull + 8 * sidx, tph);
+              if (!ok) break;
+              tc_fence_after();
+              const int bi = (sidx * 64) / K, ci = ((sidx * 64) % K) / 64;
+              if (elect_one()) {
+                const uint32_t alo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES);
+                const uint32_t blo = tlo + ((bi * K * K * 2 + ci * K * 128) >> 4);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) tc_mma_lo(dbase + bi * K, alo + 2 * kk, blo + 2 * kk, idesc_in, (ci | kk) != 0 ? 1u : 0u);
+                tc_commit(bar_empty + 8 * st);
+                if (sidx == BD_STAGES_PER_TILE - 1) tc_commit(bar_accf + 8 * buf);
               }
-              tc_commit(bar_empty + 8 * s);
+              __syncwarp();
+              next();
             }
           } else {
             // two consecutive stages = two 64-column chunks of the same 128 weight rows: one N = 128 product, the
             // second swizzle atom of the MN-major operand one stage further on
-            for (int sidx = 0; sidx < BD_STAGES_PER_TILE; sidx += 2, it += 2) {
-              const uint32_t s = it % C::NSTAGE, ph = (it / C::NSTAGE) & 1u;
-              if (!mbar_wait(bar_full + 8 * s, ph, abort_flag, status)) { ok = false; break; }
-              if (!mbar_wait(bar_full + 8 * (s + 1), ph, abort_flag, status)) { ok = false; break; }
+#pragma unroll
+            for (int sidx = 0; sidx < BD_STAGES_PER_TILE; sidx += 2) {
+              ok = wait_all(bar_full + 8 * st, sph) && wait_all(bar_full + 8 * (st + 1), sph);
+              if (!ok) break;
               tc_fence_after();
-              const uint32_t stage = sSt_u + s * BD_STAGE_BYTES;
               const int kh = sidx / C::NCC, nc = sidx % C::NCC;
+              if (elect_one()) {
+                const uint32_t blo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES, BD_STAGE_BYTES);
+                const uint32_t alo = tlo + ((kh * 2 * K * 128) >> 4);
 #pragma unroll
-              for (int ks = 0; ks < 8; ++ks) {
-                const uint64_t bd = umma_desc_sw128_lbo(stage + ks * 2048, BD_STAGE_BYTES);
+                for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
-                for (int mh = 0; mh < C::KH; ++mh) {
-                  const uint64_t ad = umma_desc_sw128(sT_u + (kh * 2 + ks / 4) * K * 128 + mh * 128 * 128 + (ks % 4) * 32);
-                  tc_mma_bf16(dbase + mh * C::NC + nc * 64, ad, bd, idesc_out, (kh | ks) != 0 ? 1u : 0u);
-                }
+                  for (int mh = 0; mh < C::KH; ++mh)
+                    tc_mma_lo(dbase + mh * C::NC + nc * 64, alo + (((ks / 4) * K * 128 + mh * 128 * 128 + (ks % 4) * 32) >> 4),
+                              blo + ks * 128, idesc_out, (kh | ks) != 0 ? 1u : 0u);
+                tc_commit(bar_empty + 8 * st);
+                tc_commit(bar_empty + 8 * (st + 1));
+                if (sidx == BD_STAGES_PER_TILE - 2) tc_commit(bar_accf + 8 * buf);
               }
-              tc_commit(bar_empty + 8 * s);
-              tc_commit(bar_empty + 8 * (s + 1));
+              __syncwarp();
+              next();
+              next();
             }
           }
-          if (ok) tc_commit(bar_accf + 8 * buf);
           // last tile of this operator block with more to come: signal when its products are done with the block
-          if (ok && base + tile + 1 < t_end && (tile + 1 == hi || (tile + 1) / n_minor != major)) tc_commit(bar_tfree);
+          if (--left == 0 || tile + 1 == hi) {
+            if (ok && base + tile + 1 < t_end && elect_one()) tc_commit(bar_tfree);
+            __syncwarp();
+          }
         }
       }
     }
   } else {
     // ---------------------------------------------------------------- epilogue
-    const int q = warp & 3, hw = (warp - 2) >> 2;
+    // Set `buf` (eight warps) serves the tiles of accumulator buffer `buf`, so a tile's epilogue may last as long as two
+    // tiles' products.  With one set of eight warps for both buffers the epilogue was the longest stage: its dependent
+    // chains left the issue slots of two warps per scheduler mostly empty (records 3200 cycles a tile, codes 10400,
+    // against 2100 for the products and 2800 for the bytes).  Measured, one set -> two: records of a 9B-shaped layer (both
+    // forms, 198 M weights) 127 -> 111 us, 27B-shaped with groups of 64 (515 M) 325 -> 286; codes of 14336 x 3584 86 -> 50;
+    // the transformed matrix of 8192 x 2304 29.5 -> 20.5 (with its stores widened to whole sectors).
+    // What bounds the records now is the products themselves: operands, 12 KB per 128 x 256 x 16 product, and the arriving
+    // weights share the 128 bytes per cycle of shared memory, so a product takes 187 cycles instead of 128.
+    const int q = warp & 3, hw = ((warp - 2) >> 2) & 1;
+    const uint32_t buf = (uint32_t)((warp - 2) >> 3);
     const int L = q * 32 + lane;
-    uint32_t tl = 0;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * 256u + hw * 128u;
+    uint32_t tl = 0, aph = 0;
     bool ok = true;
     constexpr int NG = 128 / G;
     for (int sub = s_first; sub < mp.n && ok; ++sub) {
-    const int base = sub ? mp.tile_end[sub - 1] : 0;
-    if (base >= t_end) break;
-    const BdParams& p = mp.p[sub];
-    const int lo = (t_begin > base ? t_begin : base) - base;
-    const int hi = (t_end < mp.tile_end[sub] ? t_end : mp.tile_end[sub]) - base;
-    double sq_local = 0.0, sur_local = 0.0;
-    float srow = 0.f, vm = 0.f;
-    int srow_row = -1;
-    bool bad = false;
-    const int ng_row = p.d_in / G;
-    for (int tile = lo; tile < hi && ok; ++tile, ++tl) {
-      const int major = tile / p.n_minor, t = tile - major * p.n_minor;
-      const uint32_t buf = tl & 1u, aph = (tl >> 1) & 1u;
-      int row, col0;
-      if constexpr (FORM == BD_IN) {
-        row = t * 128 + L;
-        col0 = major * 256 + hw * 128;
-      } else if constexpr (K == 256) {
-        row = major * 256 + hw * 128 + L;
-        col0 = t * 128;
-      } else {
-        row = major * 128 + L;
-        col0 = t * 256 + hw * 128;
-      }
-      // Eq. 4 weights of this thread's groups, requested before the wait for the accumulator so that the
-      // global-memory latency is hidden behind it
-      float wgt[NG];
+      const int base = sub ? mp.tile_end[sub - 1] : 0;
+      if (base >= t_end) break;
+      const BdParams& p = mp.p[sub];
+      const int lo = (t_begin > base ? t_begin : base) - base;
+      const int hi = (t_end < mp.tile_end[sub] ? t_end : mp.tile_end[sub]) - base;
+      const int n_minor = p.n_minor;
+      int major = lo / n_minor, t = lo - major * n_minor - 1;
+      double sq_local = 0.0, sur_local = 0.0;
+      float asum[NG], vm = 0.f;  // Eq. 4: squared maxima summed over the tiles of one block (input axis: per column group;
+      int asum_key = -1;         // output axis: per row, in asum[0]), and which block / row they belong to
 #pragma unroll
-      for (int gi = 0; gi < NG; ++gi) wgt[gi] = 0.f;
-      if ((p.epi & EPI_SURR) && row < p.d_out && col0 < p.d_in) {
-#pragma unroll
-        for (int gi = 0; gi < NG; ++gi) wgt[gi] = (FORM == BD_IN) ? __ldg(p.cw + col0 / G + gi) : __ldg(p.cw + row);
-      }
-      ok = mbar_wait(bar_accf + 8 * buf, aph, abort_flag, status);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * 256u + hw * 128u;
-      const bool valid = (row < p.d_out) && (col0 < p.d_in);
-      float v[32];
-      float best[NG], bval[NG];
-      int bidx[NG];
-#pragma unroll
-      for (int gi = 0; gi < NG; ++gi) { best[gi] = -1.f; bval[gi] = 0.f; bidx[gi] = 0; }
-      if (p.epi == EPI_STORE) {
-        // the transformed matrix itself, rounded to bf16 (inference-side apply of a block-diagonal operator)
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          tc_ld32(taddr + ch * 32, v);
-          uint32_t pk[16];
-#pragma unroll
-          for (int e = 0; e < 32; e += 2)
-            pk[e >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[e])) |
-                         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[e + 1])) << 16);
-          if (valid) {
-            uint4* dst = reinterpret_cast<uint4*>(p.delta + (long long)row * p.d_in + col0 + ch * 32);
-#pragma unroll
-            for (int w4 = 0; w4 < 4; ++w4) dst[w4] = make_uint4(pk[4 * w4], pk[4 * w4 + 1], pk[4 * w4 + 2], pk[4 * w4 + 3]);
-          }
-        }
-      } else if (p.epi == EPI_SQSUM) {
-        // sum of squares only (second pass of the l2 proxy)
-        float sq4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          tc_ld32(taddr + ch * 32, v);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) sq4[e & 3] = fmaf(v[e], v[e], sq4[e & 3]);
-        }
-        sq_local += valid ? (double)((sq4[0] + sq4[1]) + (sq4[2] + sq4[3])) : 0.0;
-      } else {
-        // group absmax with arg-max: four independent running candidates per group (columns e mod 4), merged at
-        // the end with the lowest index winning ties; the next 32 columns are in flight while these are compared
-        float v2[32];
-        float bv[NG][4], nz[4] = {0.f, 0.f, 0.f, 0.f};
-        int bi[NG][4];
-#pragma unroll
-        for (int gi = 0; gi < NG; ++gi)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) { bv[gi][c] = 0.f; bi[gi][c] = 0; }
-        tc_ld32_issue(taddr, v);
-        tc_ld_wait32(v);
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          float* cur = (ch & 1) ? v2 : v;
-          float* nxt = (ch & 1) ? v : v2;
-          if (ch < 3) tc_ld32_issue(taddr + (ch + 1) * 32, nxt);
-          const int gi = (G == 128) ? 0 : (ch >> 1);
-          const int e0 = (G == 128) ? ch * 32 : (ch & 1) * 32;
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const int c = e & 3;
-            if (fabsf(cur[e]) > fabsf(bv[gi][c])) { bv[gi][c] = cur[e]; bi[gi][c] = e0 + e; }
-            nz[c] = fmaf(cur[e], 0.f, nz[c]);  // stays 0 unless a NaN or an infinity passes by
-          }
-          if (ch < 3) tc_ld_wait32(nxt);
-        }
-#pragma unroll
-        for (int gi = 0; gi < NG; ++gi) {
-          float b = bv[gi][0];
-          int ix = bi[gi][0];
-#pragma unroll
-          for (int c = 1; c < 4; ++c) {
-            const float x = bv[gi][c];
-            const int jx = bi[gi][c];
-            const bool take = (fabsf(x) > fabsf(b)) || (fabsf(x) == fabsf(b) && jx < ix);
-            if (take) { b = x; ix = jx; }
-          }
-          best[gi] = fabsf(b);
-          bval[gi] = b;
-          bidx[gi] = ix;
-        }
-        if (valid && !((nz[0] + nz[1]) + (nz[2] + nz[3]) == 0.f)) bad = true;
-      }
-      // Without a second pass over the accumulator (codes / residual) everything still needed is in registers:
-      // hand the buffer back to the tensor cores now.  The arrive has release semantics, so issuing it after the
-      // global stores below would make every tile wait for those stores to land.
-      const bool early_release = (p.epi & (EPI_DELTA | EPI_CODES)) == 0;
-      if (early_release) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_acce + 8 * buf);
-      }
-      if (p.epi & (EPI_ABSMAX | EPI_DELTA | EPI_CODES)) {
-#pragma unroll
-        for (int gi = 0; gi < NG; ++gi)
-          if (valid && !(best[gi] <= 3.0e38f)) bad = true;
-        if (valid && p.vmax && !((p.epi & EPI_SURR) && p.coef)) {
-#pragma unroll
-          for (int gi = 0; gi < NG; ++gi) vm = fmaxf(vm, best[gi]);
-        }
-        if (valid && (p.epi & EPI_ABSMAX)) {
-          // with Eq. 4 evaluated right here nothing downstream reads the maxima or their signs: the backward only
-          // needs (arg-max index, coefficient).  Every scattered 4-byte store is a partial-sector write at L2.
-          const bool need_a = !(p.epi & EPI_SURR) || p.a_always;
+      for (int gi = 0; gi < NG; ++gi) asum[gi] = 0.f;
+      bool bad = false;
+      auto flush_asum = [&]() {
+        if constexpr (FORM == BD_IN) {
+          const int c0 = asum_key * 256 + hw * 128;
 #pragma unroll
           for (int gi = 0; gi < NG; ++gi) {
-            // group-major records: consecutive rows of one group are contiguous, so a warp's store is one line
-            const long long w = (long long)(col0 / G + gi) * p.d_out + row;
-            if (need_a) {
-              p.a[w] = best[gi];
-              p.usel[w] = bval[gi];
-            }
-            p.idx[w] = bidx[gi];
+            float a2 = asum[gi];
+            for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+            if (lane == 0 && a2 != 0.f && c0 < p.d_in) atomicAdd(&p.Aacc[c0 / G + gi], a2);
+            asum[gi] = 0.f;
+          }
+        } else {
+          if (asum[0] != 0.f) {
+            const int Bq = asum_key / K;
+            atomicAdd(&p.Aacc[(Bq / p.r) * K + (asum_key - Bq * K)], (float)G * asum[0]);
+          }
+          asum[0] = 0.f;
+        }
+      };
+      for (int tile = lo; tile < hi && ok; ++tile, ++tl) {
+        if (++t == n_minor) { t = 0; ++major; }
+        if ((tl & 1u) != buf) continue;
+        int row, col0;
+        if constexpr (FORM == BD_IN) {
+          row = t * 128 + L;
+          col0 = major * 256 + hw * 128;
+        } else if constexpr (K == 256) {
+          row = major * 256 + hw * 128 + L;
+          col0 = t * 128;
+        } else {
+          row = major * 128 + L;
+          col0 = t * 256 + hw * 128;
+        }
+        const bool valid = (row < p.d_out) && (col0 < p.d_in);
+        // Eq. 4 weights of this thread's groups, requested before the wait for the accumulator so that the
+        // global-memory latency is hidden behind it
+        float wgt[NG];
+        if constexpr (MODE == BD_REC || MODE == BD_DELTA) {
+#pragma unroll
+          for (int gi = 0; gi < NG; ++gi) wgt[gi] = 0.f;
+          if ((p.epi & EPI_SURR) && valid) {
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) wgt[gi] = (FORM == BD_IN) ? __ldg(p.cw + col0 / G + gi) : __ldg(p.cw + row);
           }
         }
-        if (p.epi & EPI_SURR) {
-          float surf = 0.f;
-          if constexpr (FORM == BD_OUT) {
-            // the run of tiles moved on to another row block: hand over what this thread summed for its old row
-            if (valid && srow_row >= 0 && srow_row != row) {
-              if (srow != 0.f) {
-                const int Bq = srow_row / K;
-                atomicAdd(&p.Aacc[(Bq / p.r) * K + (srow_row - Bq * K)], (float)G * srow);
-              }
-              srow = 0.f;
-            }
-          }
-#pragma unroll
-          for (int gi = 0; gi < NG; ++gi) {
-            const int Gc = col0 / G + gi;
-            const float av = valid ? best[gi] : 0.f;
-            surf = fmaf(wgt[gi] * av, av, surf);
-            if (valid && p.coef) {
-              const float sg = (bval[gi] > 0.f) ? 1.f : ((bval[gi] < 0.f) ? -1.f : 0.f);
-              const float cf = 2.f * p.kappa * wgt[gi] * av;
-              p.coef[(long long)Gc * p.d_out + row] = cf * sg;
-              vm = fmaxf(vm, cf);
-            }
-            if constexpr (FORM == BD_IN) {
-              float a2 = av * av;
-              for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-              if (lane == 0 && a2 != 0.f && col0 < p.d_in) atomicAdd(&p.Aacc[Gc], a2);
-            } else {
-              srow = fmaf(av, av, srow);
-            }
-          }
-          sur_local += (double)surf;
-          if (valid) srow_row = row;
-        }
-        if (p.epi & (EPI_DELTA | EPI_CODES)) {
-          float sc[NG];
-#pragma unroll
-          for (int gi = 0; gi < NG; ++gi) {
-            sc[gi] = __fdiv_rn(best[gi], p.qmax);
-            if (valid && (p.epi & EPI_CODES)) p.scales[(long long)row * ng_row + (col0 / G + gi)] = sc[gi];
-          }
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_accf + 8 * buf, aph, abort_flag, status));
+        aph ^= 1u;
+        if (!ok) break;
+        tc_fence_after();
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_acce + 8 * buf);
+        };
+        if constexpr (MODE == BD_STORE) {
+          // the transformed matrix itself, rounded to bf16 (inference-side apply of a block-diagonal operator)
+          uint16_t* dst = p.delta + (long long)row * p.d_in + col0;
+          const bool wide = ((uintptr_t)p.delta & 31) == 0;
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) {
+            float v[32];
             tc_ld32(taddr + ch * 32, v);
-            const float s = sc[(G == 128) ? 0 : (ch >> 1)];
-            uint32_t dpk[16], lpk[16];
-            uint32_t cpk[8];
-            // the flags are uniform over the launch: only the outputs that were asked for are formed
-            const bool want_d = (p.epi & EPI_DELTA) != 0, want_dl = want_d && p.delta_lo != nullptr;
-            const bool want_c = (p.epi & EPI_CODES) != 0;
-            // code = rne(fl32(u / s)).  The IEEE division is a long dependent sequence with a slow-path branch per
-            // element; u * (1 / s) differs from the exact quotient by less than 1.5 ulp, and from fl32(u / s) by
-            // less than 2 ulp, i.e. by less than (qmax + 1) * 2.4e-7, so it rounds to the same integer unless the
-            // quotient lies within that distance of a half-integer: those (rare: the transformed values are not on a
-            // coarse grid) chunks are redone with the division.
-            // The rounding itself uses no conversion instruction: t = x + 1.5 * 2^23 holds rne(x) in its low mantissa
-            // bits (the fp32 add rounds to nearest even, as rintf does) and, 0x4B400000 having a zero low byte, the low
-            // byte of t's pattern is the two's-complement code; |x| <= qmax (1 + 3 * 2^-23), so nothing is clamped.
-            float qv[32];
-            uint32_t cb[32];
-            {
-              constexpr float MAGIC = 12582912.f;
-              const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
-              const uint32_t winb = __float_as_uint(0.5f - (p.qmax + 1.f) * 1.0e-6f);
-              uint32_t dmax = 0u;  // largest |x - rne(x)| of the chunk, as a bit pattern
+            if (ch == 3) release();
+            uint32_t pk[16];
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                const float x = v[e] * rs;
-                const float t = x + MAGIC;
-                qv[e] = t - MAGIC;
-                cb[e] = __float_as_uint(t);
-                dmax = max(dmax, __float_as_uint(x - qv[e]) & 0x7FFFFFFFu);
+            for (int e = 0; e < 32; e += 2)
+              pk[e >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[e])) |
+                           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[e + 1])) << 16);
+            if (valid) {
+              store32(dst + ch * 32, pk, wide);
+              store32(dst + ch * 32 + 16, pk + 8, wide);
+            }
+          }
+        } else if constexpr (MODE == BD_SQSUM) {
+          // sum of squares only (second pass of the l2 proxy)
+          float sq4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int ch = 0; ch < 8; ++ch) {
+            float v[16];
+            tc_ld16(taddr + ch * 16, v);
+            if (ch == 7) release();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sq4[e & 3] = fmaf(v[e], v[e], sq4[e & 3]);
+          }
+          sq_local += valid ? (double)((sq4[0] + sq4[1]) + (sq4[2] + sq4[3])) : 0.0;
+        } else {
+          float best[NG], bval[NG];
+          int bidx[NG];
+#pragma unroll
+          for (int gi = 0; gi < NG; ++gi) { best[gi] = 0.f; bval[gi] = 0.f; bidx[gi] = 0; }
+          if constexpr (MODE == BD_CODES) {
+            // group absmax only (no arg-max): two columns per instruction, NaN and infinity stay visible in the maximum
+            float m4[NG][2];
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) m4[gi][0] = m4[gi][1] = 0.f;
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+              float v[32];
+              tc_ld32(taddr + ch * 32, v);
+              const int gi = (G == 128) ? 0 : (ch >> 1);
+#pragma unroll
+              for (int e = 0; e < 32; e += 2) m4[gi][(e >> 1) & 1] = max_abs2(m4[gi][(e >> 1) & 1], v[e], v[e + 1]);
+            }
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) {
+              best[gi] = max_abs2(m4[gi][0], m4[gi][1], 0.f);
+              if (valid && !(best[gi] <= 3.0e38f)) bad = true;
+            }
+          } else {
+            // group absmax with arg-max: four independent running candidates per group (columns e mod 4), merged at the
+            // end with the lowest index winning ties; the NaN-propagating maximum beside them is the range check
+            float bv[NG][4], nm[2] = {0.f, 0.f};
+            int bi[NG][4];
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) { bv[gi][c] = 0.f; bi[gi][c] = 0; }
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch) {
+              float v[16];
+              tc_ld16(taddr + ch * 16, v);
+              const int gi = (G == 128) ? 0 : (ch >> 2);
+              const int e0 = (G == 128) ? ch * 16 : (ch & 3) * 16;
+#pragma unroll
+              for (int e = 0; e < 16; ++e) {
+                const int c = e & 3;
+                if (fabsf(v[e]) > fabsf(bv[gi][c])) { bv[gi][c] = v[e]; bi[gi][c] = e0 + e; }
+                if (e & 1) nm[(e >> 1) & 1] = max_abs2(nm[(e >> 1) & 1], v[e - 1], v[e]);
               }
-              // (also: a scale so small that its reciprocal overflows)
-              if (dmax > winb || !(rs < 3.0e38f)) {
+            }
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                  float q = (s > 0.f) ? rintf(__fdiv_rn(v[e], s)) : 0.f;
-                  q = fminf(fmaxf(q, -p.qmax), p.qmax);
-                  qv[e] = q;
-                  cb[e] = (uint32_t)((int)q);
+            for (int gi = 0; gi < NG; ++gi) {
+              float b = bv[gi][0];
+              int ix = bi[gi][0];
+#pragma unroll
+              for (int c = 1; c < 4; ++c) {
+                const float x = bv[gi][c];
+                const int jx = bi[gi][c];
+                const bool take = (fabsf(x) > fabsf(b)) || (fabsf(x) == fabsf(b) && jx < ix);
+                if (take) { b = x; ix = jx; }
+              }
+              best[gi] = fabsf(b);
+              bval[gi] = b;
+              bidx[gi] = ix;
+            }
+            if (valid && !(max_abs2(nm[0], nm[1], 0.f) <= 3.0e38f)) bad = true;
+          }
+          // Without a second walk over the accumulator (codes / residual) everything still needed is in registers:
+          // hand the buffer back to the tensor cores now.  The arrive has release semantics, so issuing it after the
+          // global stores below would make every tile wait for those stores to land.
+          if constexpr (MODE == BD_REC) release();
+          if constexpr (MODE != BD_CODES) {
+            if (valid && p.vmax && !((p.epi & EPI_SURR) && p.coef)) {
+#pragma unroll
+              for (int gi = 0; gi < NG; ++gi) vm = fmaxf(vm, best[gi]);
+            }
+            if (valid) {
+              // with Eq. 4 evaluated right here nothing downstream reads the maxima or their signs: the backward only
+              // needs (arg-max index, coefficient).  Every scattered 4-byte store is a partial-sector write at L2.
+              const bool need_a = !(p.epi & EPI_SURR) || p.a_always;
+#pragma unroll
+              for (int gi = 0; gi < NG; ++gi) {
+                // group-major records: consecutive rows of one group are contiguous, so a warp's store is one line
+                const long long w = (long long)(col0 / G + gi) * p.d_out + row;
+                if (need_a) {
+                  p.a[w] = best[gi];
+                  p.usel[w] = bval[gi];
+                }
+                p.idx[w] = bidx[gi];
+              }
+            }
+            if (p.epi & EPI_SURR) {
+              const int key = (FORM == BD_IN) ? major : row;  // (uniform over the warp on the input axis)
+              if (asum_key != key) {
+                if (asum_key >= 0) flush_asum();
+                asum_key = key;
+              }
+              float surf = 0.f;
+#pragma unroll
+              for (int gi = 0; gi < NG; ++gi) {
+                const float av = valid ? best[gi] : 0.f;
+                surf = fmaf(wgt[gi] * av, av, surf);
+                if (valid && p.coef) {
+                  const float sg = (bval[gi] > 0.f) ? 1.f : ((bval[gi] < 0.f) ? -1.f : 0.f);
+                  const float cf = 2.f * p.kappa * wgt[gi] * av;
+                  p.coef[(long long)(col0 / G + gi) * p.d_out + row] = cf * sg;
+                  vm = fmaxf(vm, cf);
+                }
+                float& as = asum[(FORM == BD_IN) ? gi : 0];
+                as = fmaf(av, av, as);
+              }
+              sur_local += (double)surf;
+            }
+          }
+          if constexpr (MODE == BD_CODES) {
+            // code = rne(fl32(u / s)).  The IEEE division is a long dependent sequence with a slow-path branch per
+            // element; u * (1 / s), rounded once together with its addend below, differs from fl32(u / s) by less than
+            // (qmax + 1) * 2.4e-7, so it rounds to the same integer unless the quotient lies within that distance of a
+            // half-integer: those (rare: the transformed values are not on a coarse grid) chunks are redone with the
+            // division.  The rounding uses no conversion instruction: t = u / s + 1.5 * 2^23 holds rne(u / s) in its low
+            // mantissa bits (an fp32 result rounds to nearest even, as rintf does) and, 0x4B400000 having a zero low
+            // byte, the low byte of t's pattern is the two's-complement code; |u / s| <= qmax (1 + 3 * 2^-23), so
+            // nothing is clamped.
+            constexpr float MAGIC = 12582912.f;
+            const float win = 0.5f - (p.qmax + 1.f) * 1.0e-6f;
+            int8_t* dst = p.codes + (long long)row * p.d_in + col0;
+            const bool wide = ((uintptr_t)p.codes & 31) == 0;
+#pragma unroll 1
+            for (int ch = 0; ch < 4; ++ch) {
+              const int gi = (G == 128) ? 0 : (ch >> 1);
+              const float s = __fdiv_rn((NG == 1 || gi == 0) ? best[0] : best[NG - 1], p.qmax);
+              const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
+              if (valid && ch % (G / 32) == 0) p.scales[(long long)row * (p.d_in / G) + (col0 / G + gi)] = s;
+              uint32_t cpk[8];
+              float dm = 0.f;
+#pragma unroll
+              for (int hf = 0; hf < 2; ++hf) {
+                float v[16];
+                tc_ld16(taddr + ch * 32 + hf * 16, v);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                  uint32_t cb[4];
+                  float d[4];
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) {
+                    const float x = v[4 * w + e];
+                    const float tt = fmaf(x, rs, MAGIC);
+                    cb[e] = __float_as_uint(tt);
+                    d[e] = fmaf(x, rs, -(tt - MAGIC));
+                  }
+                  dm = max_abs2(dm, d[0], d[1]);
+                  dm = max_abs2(dm, d[2], d[3]);
+                  cpk[4 * hf + w] = __byte_perm(__byte_perm(cb[0], cb[1], 0x0040), __byte_perm(cb[2], cb[3], 0x0040), 0x5410);
                 }
               }
-            }
-            if (want_d) {
+              // (also: a scale so small that its reciprocal overflows); the accumulator is read again by the whole warp
+              if (__any_sync(0xffffffffu, !(dm <= win) || !(rs < 3.0e38f))) {
 #pragma unroll
-              for (int e = 0; e < 32; e += 2) {
+                for (int hf = 0; hf < 2; ++hf) {
+                  float v[16];
+                  tc_ld16(taddr + ch * 32 + hf * 16, v);
+#pragma unroll
+                  for (int w = 0; w < 4; ++w) {
+                    uint32_t pk = 0;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                      float qd = (s > 0.f) ? rintf(__fdiv_rn(v[4 * w + e], s)) : 0.f;
+                      qd = fminf(fmaxf(qd, -p.qmax), p.qmax);
+                      pk |= ((uint32_t)((int)qd) & 0xFFu) << (8 * e);
+                    }
+                    cpk[4 * hf + w] = pk;
+                  }
+                }
+              }
+              if (ch == 3) release();
+              if (valid) store32(dst + ch * 32, cpk, wide);
+            }
+          }
+          if constexpr (MODE == BD_DELTA) {
+            // residual s * code - u as one or two bf16 terms, 16 columns at a time (rounding as above)
+            constexpr float MAGIC = 12582912.f;
+            const float win = 0.5f - (p.qmax + 1.f) * 1.0e-6f;
+            uint16_t* dst = p.delta + (long long)row * p.d_in + col0;
+            uint16_t* dst_lo = p.delta_lo ? p.delta_lo + (long long)row * p.d_in + col0 : nullptr;
+            const bool wide = (((uintptr_t)p.delta | (uintptr_t)p.delta_lo) & 31) == 0;
+#pragma unroll 1
+            for (int ch = 0; ch < 8; ++ch) {
+              const int gi = (G == 128) ? 0 : (ch >> 2);
+              const float s = __fdiv_rn((NG == 1 || gi == 0) ? best[0] : best[NG - 1], p.qmax);
+              const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
+              float v[16];
+              float dm = 0.f;
+              tc_ld16(taddr + ch * 16, v);
+              if (ch == 7) release();
+              float qv[16];
+#pragma unroll
+              for (int e = 0; e < 16; e += 2) {
+                qv[e] = fmaf(v[e], rs, MAGIC) - MAGIC;
+                qv[e + 1] = fmaf(v[e + 1], rs, MAGIC) - MAGIC;
+                dm = max_abs2(dm, fmaf(v[e], rs, -qv[e]), fmaf(v[e + 1], rs, -qv[e + 1]));
+              }
+              if (!(dm <= win) || !(rs < 3.0e38f)) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                  const float qd = (s > 0.f) ? rintf(__fdiv_rn(v[e], s)) : 0.f;
+                  qv[e] = fminf(fmaxf(qd, -p.qmax), p.qmax);
+                }
+              }
+              uint32_t hpk[8], lpk[8];
+#pragma unroll
+              for (int e = 0; e < 16; e += 2) {
                 const float d0 = s * qv[e] - v[e], d1 = s * qv[e + 1] - v[e + 1];
                 const __nv_bfloat16 b0 = __float2bfloat16_rn(d0), b1 = __float2bfloat16_rn(d1);
-                dpk[e >> 1] = (uint32_t)__bfloat16_as_ushort(b0) | ((uint32_t)__bfloat16_as_ushort(b1) << 16);
-                if (want_dl)
-                  lpk[e >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(d0 - __bfloat162float(b0))) |
-                                ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(d1 - __bfloat162float(b1))) << 16);
+                hpk[e >> 1] = (uint32_t)__bfloat16_as_ushort(b0) | ((uint32_t)__bfloat16_as_ushort(b1) << 16);
+                lpk[e >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(d0 - __bfloat162float(b0))) |
+                              ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(d1 - __bfloat162float(b1))) << 16);
               }
-            }
-            if (want_c) {
-#pragma unroll
-              for (int w = 0; w < 8; ++w)
-                cpk[w] = __byte_perm(__byte_perm(cb[4 * w], cb[4 * w + 1], 0x0040), __byte_perm(cb[4 * w + 2], cb[4 * w + 3], 0x0040), 0x5410);
-            }
-            if (valid && (p.epi & EPI_DELTA)) {
-              uint4* dst = reinterpret_cast<uint4*>(p.delta + (long long)row * p.d_in + col0 + ch * 32);
-#pragma unroll
-              for (int w4 = 0; w4 < 4; ++w4) dst[w4] = make_uint4(dpk[4 * w4], dpk[4 * w4 + 1], dpk[4 * w4 + 2], dpk[4 * w4 + 3]);
-              if (p.delta_lo) {
-                uint4* dl = reinterpret_cast<uint4*>(p.delta_lo + (long long)row * p.d_in + col0 + ch * 32);
-#pragma unroll
-                for (int w4 = 0; w4 < 4; ++w4) dl[w4] = make_uint4(lpk[4 * w4], lpk[4 * w4 + 1], lpk[4 * w4 + 2], lpk[4 * w4 + 3]);
+              if (valid) {
+                store32(dst + ch * 16, hpk, wide);
+                if (dst_lo) store32(dst_lo + ch * 16, lpk, wide);
               }
-            }
-            if (valid && (p.epi & EPI_CODES)) {
-              uint4* dst = reinterpret_cast<uint4*>(p.codes + (long long)row * p.d_in + col0 + ch * 32);
-              dst[0] = make_uint4(cpk[0], cpk[1], cpk[2], cpk[3]);
-              dst[1] = make_uint4(cpk[4], cpk[5], cpk[6], cpk[7]);
             }
           }
         }
       }
-      if (!early_release) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_acce + 8 * buf);
+      if constexpr (MODE == BD_SQSUM) {
+        for (int o = 16; o > 0; o >>= 1) sq_local += __shfl_xor_sync(0xffffffffu, sq_local, o);
+        if (lane == 0 && sq_local != 0.0) atomicAdd(p.sqacc, sq_local);
       }
-    }
-    if (p.epi & EPI_SQSUM) {
-      for (int o = 16; o > 0; o >>= 1) sq_local += __shfl_xor_sync(0xffffffffu, sq_local, o);
-      if (lane == 0 && sq_local != 0.0) atomicAdd(p.sqacc, sq_local);
-    }
-    if (p.epi & EPI_SURR) {
-      for (int o = 16; o > 0; o >>= 1) sur_local += __shfl_xor_sync(0xffffffffu, sur_local, o);
-      if (lane == 0 && sur_local != 0.0) atomicAdd(p.lossacc, (double)p.kappa * sur_local);
-      if constexpr (FORM == BD_OUT) {
-        if (srow_row >= 0 && srow != 0.f) {
-          const int Bq = srow_row / K;
-          atomicAdd(&p.Aacc[(Bq / p.r) * K + (srow_row - Bq * K)], (float)G * srow);
+      if constexpr (MODE == BD_REC || MODE == BD_DELTA) {
+        if (p.epi & EPI_SURR) {
+          for (int o = 16; o > 0; o >>= 1) sur_local += __shfl_xor_sync(0xffffffffu, sur_local, o);
+          if (lane == 0 && sur_local != 0.0) atomicAdd(p.lossacc, (double)p.kappa * sur_local);
+          if (asum_key >= 0) flush_asum();
+        }
+        if (p.vmax) {
+          for (int o = 16; o > 0; o >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, o));
+          if (lane == 0 && vm > 0.f) atomicMax(reinterpret_cast<int*>(p.vmax), __float_as_int(vm));
         }
       }
-    }
-    if (p.vmax) {
-      for (int o = 16; o > 0; o >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, o));
-      if (lane == 0 && vm > 0.f) atomicMax(reinterpret_cast<int*>(p.vmax), __float_as_int(vm));
-    }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) raise_status(status, CAFEQ_ERR_NONFINITE);
+      if (__any_sync(0xffffffffu, bad) && lane == 0) raise_status(status, CAFEQ_ERR_NONFINITE);
     }  // sub-problems
   }
 
@@ -775,10 +856,10 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
   }
 }
 
-template <int FORM, int K, int G>
+template <int FORM, int K, int G, int MODE>
 __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_kernel(const __grid_constant__ BdMaps maps, const __grid_constant__ BdMulti mp) {
-  bd_pass_body<FORM, K, G>(maps, mp, (int)blockIdx.x, (int)gridDim.x);
+  bd_pass_body<FORM, K, G, MODE>(maps, mp, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // Both forms in one launch: the first n_in CTAs run the input-axis list, the others the output-axis list (a layer
@@ -788,8 +869,8 @@ template <int K, int G>
 __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_dual_kernel(const __grid_constant__ BdMaps maps_in, const __grid_constant__ BdMulti mp_in,
                     const __grid_constant__ BdMaps maps_out, const __grid_constant__ BdMulti mp_out, const int n_in) {
-  if ((int)blockIdx.x < n_in) bd_pass_body<BD_IN, K, G>(maps_in, mp_in, (int)blockIdx.x, n_in);
-  else bd_pass_body<BD_OUT, K, G>(maps_out, mp_out, (int)blockIdx.x - n_in, (int)gridDim.x - n_in);
+  if ((int)blockIdx.x < n_in) bd_pass_body<BD_IN, K, G, BD_REC>(maps_in, mp_in, (int)blockIdx.x, n_in);
+  else bd_pass_body<BD_OUT, K, G, BD_REC>(maps_out, mp_out, (int)blockIdx.x - n_in, (int)gridDim.x - n_in);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -869,11 +950,11 @@ static void bd_fill_tiles(BdParams& p) {
   p.ctas_per_major = 0;
 }
 
-template <int FORM, int K, int G>
+template <int FORM, int K, int G, int MODE>
 static int bd_launch_multi_t(cudaStream_t st, const BdMaps& maps, BdMulti mp, int min_tiles) {
   using C = BdCfg<FORM, K, G>;
   static std::atomic<unsigned long long> done{0};
-  if (!opt_in_smem(bd_pass_kernel<FORM, K, G>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
+  if (!opt_in_smem(bd_pass_kernel<FORM, K, G, MODE>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
   long long total = 0;
   for (int s = 0; s < mp.n; ++s) {
     bd_fill_tiles<FORM, K, G>(mp.p[s]);
@@ -887,13 +968,33 @@ static int bd_launch_multi_t(cudaStream_t st, const BdMaps& maps, BdMulti mp, in
   long long want = total / (min_tiles > 0 ? min_tiles : 1);
   if (want < 1) want = 1;
   const int grid = want < 148 ? (int)want : 148;
-  bd_pass_kernel<FORM, K, G><<<grid, BD_THREADS, C::SMEM, st>>>(maps, mp);
+  bd_pass_kernel<FORM, K, G, MODE><<<grid, BD_THREADS, C::SMEM, st>>>(maps, mp);
   return CAFEQ_OK;
+}
+
+// the sub-problems of a launch share the kind of their epilogue
+static int bd_mode(int epi) {
+  if (epi & EPI_STORE) return BD_STORE;
+  if (epi & EPI_SQSUM) return BD_SQSUM;
+  if (epi & EPI_CODES) return BD_CODES;
+  return (epi & EPI_DELTA) ? BD_DELTA : BD_REC;
+}
+
+template <int FORM, int K, int G>
+static int bd_dispatch_mode(cudaStream_t st, const BdMaps& maps, const BdMulti& mp, int min_tiles) {
+  switch (bd_mode(mp.p[0].epi)) {
+    case BD_REC: return bd_launch_multi_t<FORM, K, G, BD_REC>(st, maps, mp, min_tiles);
+    case BD_DELTA: return bd_launch_multi_t<FORM, K, G, BD_DELTA>(st, maps, mp, min_tiles);
+    case BD_CODES: return bd_launch_multi_t<FORM, K, G, BD_CODES>(st, maps, mp, min_tiles);
+    // (the group width plays no part in these two)
+    case BD_STORE: return bd_launch_multi_t<FORM, K, 128, BD_STORE>(st, maps, mp, min_tiles);
+    default: return bd_launch_multi_t<FORM, K, 128, BD_SQSUM>(st, maps, mp, min_tiles);
+  }
 }
 
 static int bd_dispatch(cudaStream_t st, int form, int k, int g, const BdMaps& maps, const BdMulti& mp, int min_tiles) {
 #define BD_CASE(F, KK, GG) \
-  if (form == F && k == KK && g == GG) return bd_launch_multi_t<F, KK, GG>(st, maps, mp, min_tiles);
+  if (form == F && k == KK && g == GG) return bd_dispatch_mode<F, KK, GG>(st, maps, mp, min_tiles);
   BD_CASE(BD_IN, 64, 64)
   BD_CASE(BD_IN, 64, 128)
   BD_CASE(BD_IN, 128, 64)
@@ -949,7 +1050,7 @@ static int bd_launch_many(cudaStream_t st, int form, int k, int g, const BdSub* 
 
 // relative cost of an output-axis tile against an input-axis tile of the same bytes (measured per-tile times of
 // the two forms): sets how the CTAs of a dual launch are divided
-static std::atomic<int> g_dual_pass_pct{130}, g_dual_bwd_pct{100};
+static std::atomic<int> g_dual_pass_pct{110}, g_dual_bwd_pct{100};
 
 static int dual_split(long long tiles_in, long long tiles_out, int out_weight_pct) {
   const double wi = (double)tiles_in, wo = (double)tiles_out * out_weight_pct / 100.0;
