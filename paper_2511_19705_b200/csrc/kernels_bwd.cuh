@@ -52,6 +52,7 @@ struct BwMaps {
 };
 struct BwMulti {
   int n;
+  int stream;  // as in BdMulti
   int tile_end[BW_MAX_SUB];
   BwParams p[BW_MAX_SUB];  // all share one status word
 };
@@ -173,6 +174,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
     if (lane == 0) {
       uint32_t it = 0;
       int sub = s_first;
+      const uint64_t pol = l2_evict_first_policy();
       for (int gt = t_begin; gt < t_end; ++gt, ++it) {
         while (gt >= mp.tile_end[sub]) ++sub;
         const int tile = gt - (sub ? mp.tile_end[sub - 1] : 0);
@@ -185,10 +187,14 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
         const uint32_t dst = smem_u32(sStage + s * C::STAGE_BYTES);
         if constexpr (FORM == BW_IN) {
           // 64 rows x K columns as K / 64 boxes of 64 x 64 (one swizzle atom of the MN-major operand each)
-          for (int n = 0; n < K / 64; ++n) tma_load_2d(dst + n * 8192, tmW, major * K + n * 64, t * 64, bar_wfull + 8 * s);
+          for (int n = 0; n < K / 64; ++n) {
+            if (mp.stream) tma_load_2d_hint(dst + n * 8192, tmW, major * K + n * 64, t * 64, bar_wfull + 8 * s, pol);
+            else tma_load_2d(dst + n * 8192, tmW, major * K + n * 64, t * 64, bar_wfull + 8 * s);
+          }
         } else {
           // K rows x 64 columns: one box, K-major operand
-          tma_load_2d(dst, tmW, t * 64, major * K, bar_wfull + 8 * s);
+          if (mp.stream) tma_load_2d_hint(dst, tmW, t * 64, major * K, bar_wfull + 8 * s, pol);
+          else tma_load_2d(dst, tmW, t * 64, major * K, bar_wfull + 8 * s);
         }
       }
     }
@@ -492,6 +498,7 @@ static int bw_launch_t(cudaStream_t st, const BwMaps& maps, BwMulti mp, int min_
     mp.tile_end[s] = (int)total;
   }
   for (int s = mp.n; s < BW_MAX_SUB; ++s) mp.tile_end[s] = (int)total;
+  mp.stream = l2_stream(128.0 * K * total);
   long long want = total / (min_tiles > 0 ? min_tiles : 1);
   if (want < majors) want = majors;
   if (want > total) want = total;
@@ -580,6 +587,7 @@ static int bw_launch_dual_t(cudaStream_t st, const BwMaps& mi, BwMulti pi, const
   }
   for (int s = po.n; s < BW_MAX_SUB; ++s) po.tile_end[s] = (int)to;
   // tiles of the two forms hold the same bytes (64 x K entries)
+  pi.stream = po.stream = l2_stream(128.0 * K * (ti + to));
   const int n_in = dual_split(ti, to, g_dual_bwd_pct.load(std::memory_order_relaxed));
   bd_bwd_dual_kernel<K, SWAP_IN, SWAP_OUT><<<148, BW_THREADS, C::SMEM, st>>>(mi, pi, mo, po, n_in);
   return CAFEQ_OK;

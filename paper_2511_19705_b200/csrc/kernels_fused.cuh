@@ -69,6 +69,7 @@ struct BdMaps {
 };
 struct BdMulti {
   int n;
+  int stream;                 // read the matrices with evict_first (l2_stream below)
   int tile_end[BD_MAX_SUB];
   BdParams p[BD_MAX_SUB];     // all share one status word
 };
@@ -151,6 +152,19 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
       "l"(map), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+
+// the same with an L2 policy: evict_first for data that is read once per step, so that it does not displace what is reused
+__device__ __forceinline__ uint64_t l2_evict_first_policy() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
+__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar, uint64_t pol) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(bar), "l"(pol)
       : "memory");
 }
 
@@ -356,6 +370,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
     if (lane == 0) {
       uint32_t it = 0, tloads = 0;
       bool ok = true;
+      const uint64_t pol = l2_evict_first_policy();
       for (int sub = s_first; sub < mp.n && ok; ++sub) {
         const int base = sub ? mp.tile_end[sub - 1] : 0;
         if (base >= t_end) break;
@@ -394,7 +409,8 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               x = t * C::NC + nc * 64;
               y = major * K + kh * 128;
             }
-            tma_load_2d(smem_u32(sStage + s * BD_STAGE_BYTES), tmX, x, y, bar_full + 8 * s);
+            if (mp.stream) tma_load_2d_hint(smem_u32(sStage + s * BD_STAGE_BYTES), tmX, x, y, bar_full + 8 * s, pol);
+            else tma_load_2d(smem_u32(sStage + s * BD_STAGE_BYTES), tmX, x, y, bar_full + 8 * s);
           }
         }
       }
@@ -922,6 +938,13 @@ static bool bd_supported(int form, int d_out, int d_in, long long ld, int k, int
   return true;
 }
 
+// Weights of a launch that take more than a quarter of L2 (126 MB) are read with evict_first, so that they displace one
+// another and not what the step comes back to (records, operators, k x k state).  Measured: layer step of a 2B-shaped pair
+// (85 MB) 148 -> 139 us, of a 42 MB pair 115 -> 107, of a 9B-shaped layer 410 -> 399; codes of 103 MB 72 -> 69; layers of
+// 6 to 20 MB the same either way.  Not for the inference side: activations usually come from the product before, through
+// L2 (38 MB read again and again: 23.6 us, with the hint 25.7).
+static int l2_stream(double bytes) { return bytes > 32.0 * (1 << 20) ? 1 : 0; }
+
 static std::atomic<int> g_bd_min_tiles{1};
 
 // opt the kernel into its dynamic shared memory once per device (the attribute is per device and per function)
@@ -962,6 +985,7 @@ static int bd_launch_multi_t(cudaStream_t st, const BdMaps& maps, BdMulti mp, in
     mp.tile_end[s] = (int)total;
   }
   for (int s = mp.n; s < BD_MAX_SUB; ++s) mp.tile_end[s] = (int)total;
+  mp.stream = (MODE == BD_REC || MODE == BD_CODES) ? l2_stream(65536.0 * total) : 0;
   // one persistent CTA per SM at most; when several problems overlap in streams, small matrices take fewer CTAs
   // (at least min_tiles tiles each): the fixed cost of a CTA is spread over more tiles and the SMs left over
   // run another problem's kernel
@@ -1078,6 +1102,7 @@ static int bd_launch_dual_t(cudaStream_t st, const BdMaps& mi, BdMulti pi, const
     po.tile_end[s] = (int)to;
   }
   for (int s = po.n; s < BD_MAX_SUB; ++s) po.tile_end[s] = (int)to;
+  pi.stream = po.stream = l2_stream(65536.0 * (ti + to));
   const int n_in = dual_split(ti, to, g_dual_pass_pct.load(std::memory_order_relaxed));
   bd_pass_dual_kernel<K, G><<<148, BD_THREADS, SMEM, st>>>(mi, pi, mo, po, n_in);
   return CAFEQ_OK;
