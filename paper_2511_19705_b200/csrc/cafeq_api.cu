@@ -8,6 +8,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "cafeq.h"
@@ -297,28 +298,10 @@ __global__ void transpose_blocks_kernel(const float* __restrict__ in, float* __r
   }
 }
 
-__global__ void fill_f64_kernel(double* p, double v, int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = v;
-}
-
 __global__ void zero_ns_kernel(double* rn, int n, int* flag) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) rn[i] = 0.0;
   if (i == 0) *flag = 0;
-}
-
-// c[b][t] = sum_i X[b][i][t]^2
-__global__ void colnorm_kernel(const float* __restrict__ X, int k, int nb, float* __restrict__ c) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int b = blockIdx.y;
-  if (t >= k || b >= nb) return;
-  const float* Xb = X + (size_t)b * k * k;
-  float s = 0.f;
-  for (int i = 0; i < k; ++i) {
-    const float v = Xb[(size_t)i * k + t];
-    s = fmaf(v, v, s);
-  }
-  c[(size_t)b * k + t] = s;
 }
 
 static void launch_split(cudaStream_t st, const float* X, int k, long long n, uint16_t* hi, uint16_t* lo, uint16_t* thi,
@@ -331,10 +314,10 @@ static void launch_split(cudaStream_t st, const float* X, int k, long long n, ui
 // Minv = inv(bf16(M)) by Newton-Schulz iteration X <- X + X (I - A X) on the tensor cores, from X0 = A^T
 // (cold: right for the near-orthogonal transforms the method starts from) or from the caller's previous
 // inverse (warm).  The last residual is checked on the device; if it is not small the Gauss-Jordan kernel
-// recomputes everything.  Leaves fp32 Minv in X, its bf16 splits in w.Xh/Xl/XTh/XTl[w.cur], and c = column
-// square norms of Minv (optional).
-static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm, int nb, int k, bool warm, KkWS& w,
-                       int32_t* status, bool prepped = false, bool splits_kept = false) {
+// recomputes the block.  Leaves fp32 Minv in X and its bf16 splits in w.Xh/Xl (and XTh/XTl unless w.mn) [w.cur].
+// eq4 (block sizes of the fused kernel): where the kernel puts the column norms / group weights, and what it ticks.
+static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k, bool warm, KkWS& w, int32_t* status,
+                      bool prepped = false, bool splits_kept = false, const NsParams* eq4 = nullptr) {
   const long long kk = (long long)nb * k * k;
   const int iters = warm ? NS_WARM_ITERS : NS_COLD_ITERS;
   // A warm start runs as many rounds as the step size calls for: a block whose residual ||I - A X||_F was below 1e-2
@@ -353,22 +336,17 @@ static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm,
     if (!warm) CQ_LAUNCH(ns_cold_start_kernel, dim3(k / 32, k / 32, nb), dim3(32, 8), 0, st, w.Ab, k, w.Xh[0], w.Xl[0], status);
     else if (!splits_kept) launch_split(st, X, k, kk, w.Xh[0], w.Xl[0], nullptr, nullptr, nullptr, status);
     NsParams np;
+    memset(&np, 0, sizeof(np));
+    if (eq4) np = *eq4;
     np.max_rounds = warm ? NS_WARM_ROUNDS : NS_COLD_ROUNDS;
     np.gate2 = warm ? NS_GATE2 : NS_COLD_GATE2;
-    np.rn = w.rn;
+    np.accept2 = NS_GATE2;
+    np.redo_count = w.redo_total;
     np.status = status;
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    if (ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np) != CAFEQ_OK)
-      CQ_LAUNCH(fill_f64_kernel, 1, 128, 0, st, w.rn, 1.0, nb);  // (no tensor maps: everything goes to the elimination)
-    // a block that ran out of rounds is recomputed by elimination, and everything is split again then
-    launch_inverse(st, Mc, X, nullptr, nb, k, status, w.rn, 1e-4, w.flag, w.redo_total);
-    launch_split(st, X, k, kk, w.Xh[0], w.Xl[0], nullptr, nullptr, w.flag, status);
-    if (cnorm) {
-      dim3 grid((k + 127) / 128, nb);
-      CQ_LAUNCH(colnorm_kernel, grid, 128, 0, st, X, k, nb, cnorm);
-    }
+    const int rc = ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np);
     kt_end(ti, st);
-    return;
+    return rc;
   }
   if (!warm) CQ_LAUNCH(transpose_blocks_kernel, grid_for(kk), 256, 0, st, Mc, X, k, kk);
   int cur = 0;
@@ -397,11 +375,8 @@ static void ns_inverse(cudaStream_t st, const float* Mc, float* X, float* cnorm,
   // when the elimination recomputed a block)
   const double* last_gate = (warm && iters > 1) ? w.rn + (size_t)(iters - 2) * nb : nullptr;
   launch_split(st, X, k, kk, w.Xh[cur], w.Xl[cur], w.XTh[cur], w.XTl[cur], w.flag, status, last_gate, NS_GATE2);
-  if (cnorm) {
-    dim3 grid((k + 127) / 128, nb);
-    CQ_LAUNCH(colnorm_kernel, grid, 128, 0, st, X, k, nb, cnorm);
-  }
   kt_end(ti, st);
+  return CAFEQ_OK;
 }
 
 // G -= X^T Gx X^T for every block, on the tensor cores with three-term bf16 splits; X = Minv with its splits in
@@ -470,6 +445,10 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
     }
     g_launches.fetch_sub(1, std::memory_order_relaxed);
   }
+  // Tiny matrices (a few CTAs whatever the split): one CTA per output strip, so that every sum has one order and a run
+  // repeats bit for bit.  An optimiser step that divides by the gradient's own size otherwise turns the order of the atomic
+  // additions into different bf16 operators.
+  const bool tiny = G.n <= 65536;
   const bool aligned = ((uintptr_t)W % 4 == 0) && (G.ld % 2 == 0);
   const int nG = (k >= G.g) ? k / G.g : 1;  // groups of one row inside one block (g | k or k | g on this path)
   if (kk_fast(k) && G.axis == CAFEQ_AXIS_IN && (k % G.g == 0 || G.g % k == 0) && nG <= 8 && ((uintptr_t)W % 16 == 0) &&
@@ -485,6 +464,7 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
     rp2 = ((rp2 + 31) / 32) * 32;
     if (rp2 < rows_per) rows_per = rp2;
     if (rows_per < 32) rows_per = 32;
+    if (tiny && G.d_out * nG <= SCB_SORTED) rows_per = G.d_out;
     const int splits = (G.d_out + rows_per - 1) / rows_per;
     dim3 grid(G.nbq, strips, splits);
     const size_t sh = (size_t)k * (strip + 1) * 4 + (size_t)SCB_MAXP * 6;
@@ -531,7 +511,7 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
   if (kk_fast(k) && G.g % 4 == 0 && G.g <= 128 && ((uintptr_t)W % 8 == 0) && (G.ld % 4 == 0) && G.axis == CAFEQ_AXIS_OUT) {
     const int strips = k / SC2_JS;
     int splits = (148 * 4 + G.nbq * strips - 1) / (G.nbq * strips);
-    if (splits < 1) splits = 1;
+    if (splits < 1 || tiny) splits = 1;
     int per = (G.ng + splits - 1) / splits;
     splits = (G.ng + per - 1) / per;
     dim3 grid(G.nbq, strips, splits);
@@ -970,7 +950,7 @@ static bool lean_single_ok(const Geo& G, const cafeq_opt_cfg* cfg, const void* W
 static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& G, const void* W, const float* M,
                         float* Minv_out, const void* offsets, int off_kind, int loss_kind, float kappa, bool want_exact,
                         float* losses, float* hist, float* gradM, int32_t* status, SingleWS& s, bool force_generic,
-                        bool warm = false, float* step_counter = nullptr, float* grad_offsets = nullptr) {
+                        bool warm = false, float* step_counter = nullptr, float* grad_offsets = nullptr, bool splits_kept = false) {
   const int k = G.k;
   const bool tc = kk_fast(k) && !force_generic;
   const long long kk = (long long)G.nbT * k * k;
@@ -996,9 +976,15 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     pa.step_counter = step_counter;
     pa.status = status;
     CQ_LAUNCH(step_prep_kernel, grid_for(kk), 256, 0, st, pa);
-    ns_inverse(st, s.Mc, s.Minv, nullptr, G.nbT, k, warm, s.kk, status, true);
-    dim3 cg(k / 32, G.nbT);
-    CQ_LAUNCH(colnorm_cw_kernel, cg, dim3(32, 8), 0, st, s.Minv, k, s.c, in_r1 ? s.m.cw : nullptr, G.g);
+    NsParams eq4;
+    memset(&eq4, 0, sizeof(eq4));
+    eq4.c = s.c;
+    eq4.n = 1;
+    eq4.blk0[1] = G.nbT;
+    eq4.cw[0] = in_r1 ? s.m.cw : nullptr;
+    eq4.g[0] = G.g;
+    if ((s.err = ns_inverse(st, s.Mc, s.Minv, G.nbT, k, warm, s.kk, status, true, splits_kept && tb_supported(k, 2), &eq4))) return;
+    if (!s.kk.mn) CQ_LAUNCH(colnorm_cw_kernel, dim3(k / 32, G.nbT), dim3(32, 8), 0, st, s.Minv, k, s.c, in_r1 ? s.m.cw : nullptr, G.g);
     if (!in_r1) {
       if (G.axis == CAFEQ_AXIS_IN) CQ_LAUNCH(cw_in_kernel, (G.ng + 127) / 128, 128, 0, st, s.c, G.d_in, G.g, k, G.r, s.m.cw);
       else CQ_LAUNCH(cw_out_kernel, (G.d_out + 127) / 128, 128, 0, st, s.c, G.d_out, G.g, k, G.r, s.m.cw);
@@ -1245,7 +1231,7 @@ extern "C" int cafeq_optimize_single(const cafeq_matrix_desc* d, const void* W, 
   for (int it = 0; it < cfg->steps; ++it) {
     bool eval = cfg->eval_every > 0 && (it % cfg->eval_every == 0);
     single_step(st, d, G, W, M, nullptr, nullptr, CAFEQ_OFFSETS_NONE, cfg->loss_kind, kappa, eval, nullptr,
-                loss_history + 2 * (size_t)it, grad, status, s, false, resume || it > 0, opt_state);
+                loss_history + 2 * (size_t)it, grad, status, s, false, resume || it > 0, opt_state, nullptr, it > 0);
     if (s.err) return s.err;
     if (cfg->optimizer == CAFEQ_OPT_GD) {
       CQ_LAUNCH(gd_update_kernel, grid_for(kk), 256, 0, st, M, grad, cfg->lr, kk, status);
@@ -1422,7 +1408,7 @@ static void cayley_update(cudaStream_t st, float* M, const float* grad, float* V
 static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_matrix_desc* d2, const Geo& G1, const Geo& G2,
                       const void* W1, const void* W2, const float* M, const float* P, float t, float lambda, bool want_pqe,
                       float* losses, float* hist, float* gradM, int32_t* status, PairWS& p, bool force_generic,
-                      bool warm = false, float* step_counter = nullptr, bool ste = false, int objective = 0) {
+                      bool warm = false, float* step_counter = nullptr, bool ste = false, int objective = 0, bool splits_kept = false) {
   const int k = G1.k;
   const bool tc = kk_fast(k) && !force_generic;
   const long long kk = (long long)G1.nbT * k * k;
@@ -1447,7 +1433,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     pa.step_counter = step_counter;
     pa.status = status;
     CQ_LAUNCH(step_prep_kernel, grid_for(kk), 256, 0, st, pa);
-    ns_inverse(st, p.Mc, p.Minv, nullptr, G1.nbT, k, warm, p.kk, status, true);
+    if ((p.err = ns_inverse(st, p.Mc, p.Minv, G1.nbT, k, warm, p.kk, status, true, splits_kept && tb_supported(k, 2)))) return;
   } else {
     CQ_LAUNCH(zero_f64_kernel, 1, 32, 0, st, p.acc, 8);
     CQ_LAUNCH(fill_f32_kernel, 1, 32, 0, st, p.amax, 0.f, 1);
@@ -1723,7 +1709,7 @@ extern "C" int cafeq_optimize_pair(const cafeq_matrix_desc* d1, const void* W1, 
   for (int it = 0; it < cfg->steps; ++it) {
     bool eval = ste || (any_pqe && (it % cfg->eval_every == 0));
     pair_step(st, d1, d2, G1, G2, W1, W2, M, P, cfg->lse_t, cfg->lambda_orth, eval, nullptr, loss_history + 2 * (size_t)it,
-              grad, status, p, false, resume || it > 0, opt_state, ste, objective);
+              grad, status, p, false, resume || it > 0, opt_state, ste, objective, it > 0);
     if (p.err) return p.err;
     if (cayley) {
       // momentum in the state's first-moment slot
@@ -1789,8 +1775,9 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, M, Mc, kk, status);
     // block sizes 128 / 256: elimination takes 5 ms at k = 256 (one CTA per block, k dependent steps); at k <= 64 it is
     // short and stays
-    if (tb_supported(G1.k, 2)) ns_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, false, kkw, status);
-    else launch_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, status);
+    if (tb_supported(G1.k, 2)) {
+      if ((rc = ns_inverse(st, Mc, Minv, G1.nbT, G1.k, false, kkw, status))) return rc;
+    } else launch_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, status);
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, Minv, Minv_c, kk, status);
     launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
     launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);

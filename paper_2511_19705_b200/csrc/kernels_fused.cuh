@@ -34,6 +34,7 @@ enum { BD_REC = 0, BD_DELTA = 1, BD_CODES = 2, BD_STORE = 3, BD_SQSUM = 4 };
 struct BdParams {
   int d_out, d_in;     // shape of X
   int r;               // matrix blocks per operator block
+  int t_mn;            // output axis: the operator blocks are stored transposed (T[j][i]; read as an MN-major operand)
   int n_major;         // IN: tile columns (256 d_in columns each); OUT: row blocks (k rows each)
   int n_minor;         // IN: row tiles of 128; OUT: column tiles of NC
   int ctas_per_major;
@@ -390,7 +391,13 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               for (int ci = 0; ci < K / 64; ++ci) {
                 const uint32_t bq = bar_tfull + 8 * (bi * (K / 64) + ci);  // at most four chunks: NBLK * K = 256 or NBLK = 1
                 mbar_expect_tx(bq, K * 128);
-                tma_load_2d(smem_u32(sT + bi * K * K * 2 + ci * K * 128), tmT, ci * 64, tb * K, bq);
+                const uint32_t dst = smem_u32(sT + bi * K * K * 2 + ci * K * 128);
+                if (FORM == BD_OUT && p.t_mn) {
+                  // 64 contraction rows x K columns as boxes of 64 x 64 (one swizzle atom each)
+                  for (int j = 0; j < K / 64; ++j) tma_load_2d(dst + j * 8192, tmT, j * 64, tb * K + ci * 64, bq);
+                } else {
+                  tma_load_2d(dst, tmT, ci * 64, tb * K, bq);
+                }
               }
             }
             cur_major = major;
@@ -424,7 +431,6 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
       bool ok = true;
       uint32_t tfulls = 0;
       constexpr uint32_t idesc_in = umma_idesc_bf16(128, K, 0, 0);
-      constexpr uint32_t idesc_out = umma_idesc_bf16(128, 128, 0, 1);
       const uint32_t sSt_u = smem_u32(sStage);
       const uint32_t tlo = umma_desc_lo(smem_u32(sT));
       uint32_t st = 0, sph = 0, tl = 0;  // stage, its phase, tile
@@ -434,6 +440,8 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
         const int base = sub ? mp.tile_end[sub - 1] : 0;
         if (base >= t_end) break;
         const int n_minor = mp.p[sub].n_minor;
+        const bool t_mn = FORM == BD_OUT && mp.p[sub].t_mn;
+        const uint32_t idesc_out = t_mn ? umma_idesc_bf16(128, 128, 1, 1) : umma_idesc_bf16(128, 128, 0, 1);
         const int lo = (t_begin > base ? t_begin : base) - base;
         const int hi = (t_end < mp.tile_end[sub] ? t_end : mp.tile_end[sub]) - base;
         int left = 0;  // tiles of this sub-problem left on the current operator block
@@ -484,12 +492,14 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               const int kh = sidx / C::NCC, nc = sidx % C::NCC;
               if (elect_one()) {
                 const uint32_t blo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES, BD_STAGE_BYTES);
-                const uint32_t alo = tlo + ((kh * 2 * K * 128) >> 4);
+                // K-major operator: steps of 32 bytes inside the swizzled rows; MN-major: steps of sixteen 128-byte rows
+                const uint32_t alo = (t_mn ? umma_desc_lo(smem_u32(sT), 8192) : tlo) + ((kh * 2 * K * 128) >> 4);
+                const uint32_t astep = t_mn ? 128 : 2;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
                   for (int mh = 0; mh < C::KH; ++mh)
-                    tc_mma_lo(dbase + mh * C::NC + nc * 64, alo + (((ks / 4) * K * 128 + mh * 128 * 128 + (ks % 4) * 32) >> 4),
+                    tc_mma_lo(dbase + mh * C::NC + nc * 64, alo + (((ks / 4) * K * 128 + mh * 128 * 128) >> 4) + (ks % 4) * astep,
                               blo + ks * 128, idesc_out, (kh | ks) != 0 ? 1u : 0u);
                 tc_commit(bar_empty + 8 * st);
                 tc_commit(bar_empty + 8 * (st + 1));
@@ -1039,7 +1049,7 @@ static int bd_launch(cudaStream_t st, int form, int k, int g, const void* X, lon
   BdMulti mp;
   memset(&mp, 0, sizeof(mp));
   if (!make_map_bf16(&maps.x[0], X, p.d_in, p.d_out, ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-  if (!make_map_bf16(&maps.t[0], Tb, k, (long long)nbT * k, k, k)) return CAFEQ_ERR_UNSUPPORTED;
+  if (!make_map_bf16(&maps.t[0], Tb, k, (long long)nbT * k, k, p.t_mn ? 64 : k)) return CAFEQ_ERR_UNSUPPORTED;
   for (int s = 1; s < BD_MAX_SUB; ++s) { maps.x[s] = maps.x[0]; maps.t[s] = maps.t[0]; }
   mp.n = 1;
   mp.p[0] = p;
@@ -1064,7 +1074,7 @@ static int bd_launch_many(cudaStream_t st, int form, int k, int g, const BdSub* 
   memset(&mp, 0, sizeof(mp));
   for (int s = 0; s < n; ++s) {
     if (!make_map_bf16(&maps.x[s], subs[s].X, subs[s].p.d_in, subs[s].p.d_out, subs[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&maps.t[s], subs[s].Tb, k, (long long)subs[s].nbT * k, k, k)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&maps.t[s], subs[s].Tb, k, (long long)subs[s].nbT * k, k, subs[s].p.t_mn ? 64 : k)) return CAFEQ_ERR_UNSUPPORTED;
     mp.p[s] = subs[s].p;
   }
   for (int s = n; s < BD_MAX_SUB; ++s) { maps.x[s] = maps.x[0]; maps.t[s] = maps.t[0]; }
@@ -1125,7 +1135,7 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
   for (int s = n_in; s < BD_MAX_SUB; ++s) { mi.x[s] = mi.x[0]; mi.t[s] = mi.t[0]; }
   for (int s = 0; s < n_out; ++s) {
     if (!make_map_bf16(&mo.x[s], out[s].X, out[s].p.d_in, out[s].p.d_out, out[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&mo.t[s], out[s].Tb, k, (long long)out[s].nbT * k, k, k)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&mo.t[s], out[s].Tb, k, (long long)out[s].nbT * k, k, out[s].p.t_mn ? 64 : k)) return CAFEQ_ERR_UNSUPPORTED;
     po.p[s] = out[s].p;
   }
   for (int s = n_out; s < BD_MAX_SUB; ++s) { mo.x[s] = mo.x[0]; mo.t[s] = mo.t[0]; }

@@ -177,19 +177,8 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
 // block inverse: Gauss-Jordan with partial pivoting, one CTA per k x k block, matrix kept in the output
 // buffer (global memory, L2 resident).  Also emits the column square norms c[t] = sum_i Minv[i][t]^2.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out,
-                                                             float* __restrict__ cnorm, int k, int32_t* status,
-                                                             const double* __restrict__ rn_check, double tol2, int* redo_flag,
-                                                             int* redo_count = nullptr) {
-  // rn_check: squared residual of an iterative inverse per block; the elimination only runs for blocks whose
-  // residual is above tol2 (or not finite) and then raises redo_flag for whoever depends on the result
-  if (status && *status) return;
-  if (rn_check) {
-    if (rn_check[blockIdx.x] <= tol2) return;
-    if (threadIdx.x == 0 && redo_flag) *redo_flag = 1;
-    if (threadIdx.x == 0 && redo_count) atomicAdd(redo_count, 1);  // blocks recomputed by elimination, over the run
-  }
-  extern __shared__ float sm[];  // prow[k], fcol[k], piv (int) [k], red
+// in place on A; every thread of the CTA takes part; sm: 3 k words of shared memory.  False: no usable pivot (reported).
+__device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* status) {
   float* prow = sm;
   float* fcol = sm + k;
   int* piv = (int*)(sm + 2 * k);
@@ -198,9 +187,6 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __rest
   __shared__ int s_r;
   __shared__ int s_bad;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const float* A0 = Min + (size_t)blockIdx.x * k * k;
-  float* A = Out + (size_t)blockIdx.x * k * k;
-  for (int e = tid; e < k * k; e += nt) A[e] = A0[e];
   if (tid == 0) s_bad = 0;
   __syncthreads();
   for (int p = 0; p < k; ++p) {
@@ -236,7 +222,7 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __rest
     __syncthreads();
     if (s_bad) {
       if (tid == 0) raise_status(status, CAFEQ_ERR_SINGULAR);
-      return;
+      return false;
     }
     const int r = s_r;
     // exchange rows p and r; keep the (new) pivot row in shared memory
@@ -274,6 +260,27 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __rest
     }
     __syncthreads();
   }
+  return true;
+}
+
+__global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out,
+                                                             float* __restrict__ cnorm, int k, int32_t* status,
+                                                             const double* __restrict__ rn_check, double tol2, int* redo_flag,
+                                                             int* redo_count = nullptr) {
+  // rn_check: squared residual of an iterative inverse per block; the elimination only runs for blocks whose
+  // residual is above tol2 (or not finite) and then raises redo_flag for whoever depends on the result
+  if (status && *status) return;
+  if (rn_check) {
+    if (rn_check[blockIdx.x] <= tol2) return;
+    if (threadIdx.x == 0 && redo_flag) *redo_flag = 1;
+    if (threadIdx.x == 0 && redo_count) atomicAdd(redo_count, 1);  // blocks recomputed by elimination, over the run
+  }
+  extern __shared__ float sm[];  // 3 k words
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const float* A0 = Min + (size_t)blockIdx.x * k * k;
+  float* A = Out + (size_t)blockIdx.x * k * k;
+  for (int e = tid; e < k * k; e += nt) A[e] = A0[e];
+  if (!gauss_jordan(A, k, sm, status)) return;
   if (cnorm) {
     for (int t = tid; t < k; t += nt) {
       float s = 0.f;
@@ -657,6 +664,7 @@ __global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t
 // The accumulators go through shared memory to a coalesced add into global memory.
 // K in {64, 128, 256}; rows_per_cta * NG <= SCB_MAXP; ld % 8 == 0 and W 16-byte aligned.
 constexpr int SCB_MAXP = 4096;
+constexpr int SCB_SORTED = 512;  // up to this many records a bucket is accumulated in row order
 
 template <int K, int STRIP>
 __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_t* __restrict__ W, long long ld, int d_out,
@@ -736,6 +744,19 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
   __syncthreads();
   // phase C: every thread walks its bucket
   const int b = tid / TPB, part = tid - b * TPB;
+  if (np <= SCB_SORTED) {  // few records: in row order (the placement above is in the order of its atomics)
+    if (part == 0) {
+      for (int i = start[b] + 1; i < start[b + 1]; ++i) {
+        const uint16_t o = rec_o[i];
+        const float c = rec_cf[i];
+        int j = i - 1;
+        for (; j >= start[b] && rec_o[j] > o; --j) { rec_o[j + 1] = rec_o[j]; rec_cf[j + 1] = rec_cf[j]; }
+        rec_o[j + 1] = o;
+        rec_cf[j + 1] = c;
+      }
+    }
+    __syncthreads();
+  }
   float acc[CPT];
 #pragma unroll
   for (int c = 0; c < CPT; ++c) acc[c] = 0.f;

@@ -19,7 +19,8 @@ __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bu
 // Block inverse by Newton-Schulz: X <- X + X (I - A X), as many rounds as the block needs, in one launch.
 //   round: R = I - A X over X = hi + lo (two terms, 24-bit products against bf16 A), ||R||_F in the same epilogue,
 //          X += hi R (one term: the round corrects its own error), new hi / lo splits, fp32 X on the last round.
-// The last round is the one whose residual before the update is below the gate.
+// The last round is the one whose residual before the update is below the gate; a block that never gets there is inverted by
+// elimination at the end.  The column square norms of the result (Eq. 4's weights) come out of the last update's epilogue.
 //
 // What bounds it: one round at k = 256 moves 512 KB into the SM (A, hi, lo, hi again) at the 60 - 75 GB/s one SM takes
 // from L2, and spends 3 x 1.1 us per 64-column chunk of products; as two launches per round (residual, update) each
@@ -39,10 +40,23 @@ struct NsMaps {
   CUtensorMap xhl;     // hi and lo as two planes, boxes of 32 x 32 x 2, 64-byte swizzle
   CUtensorMap x;       // fp32 X, boxes of 32 x 32, 128-byte swizzle
 };
+constexpr int KK_MAX_PROBS = 8;
 struct NsParams {
   int max_rounds;
   double gate2;        // squared residual below which a round is the last one
-  double* rn;          // [nb] squared residual before the last update
+  double accept2;      // a block whose last residual before an update is above this (squared) is inverted by elimination
+  const uint16_t* A;   // [nb, K, K]
+  uint16_t *hi, *lo;   // splits of X
+  float* X;
+  int* redo_count;     // optional: blocks inverted by elimination, added up
+  // Eq. 4's weights for the blocks of the first n problems (blk0[p] <= b < blk0[p + 1]):
+  float* c;            // column square norms c[b][t] = sum_i X[i][t]^2 (may be null)
+  int n;
+  int blk0[KK_MAX_PROBS + 1];
+  float* cw[KK_MAX_PROBS];  // sums of c over runs of g columns of the problem, added to cw (null: none)
+  int g[KK_MAX_PROBS];
+  int n_ticks;
+  float* tick[KK_MAX_PROBS];  // optimiser step counters, advanced by one
   int32_t* status;
 };
 
@@ -56,14 +70,15 @@ struct NsCfg {
   static constexpr int EPI_WARPS = 16;
   static constexpr int EPI_WARP_BYTES = 12288;  // two hi + lo tiles (in and out), one fp32 tile
   static constexpr int NBAR = 2 * NSLOT + 3 + 2 * EPI_WARPS;
-  static constexpr int SMEM = 1024 + NSLOT * SLOT + 8 * NBAR + 8 * EPI_WARPS + 64;
+  static constexpr int SMEM = 1024 + NSLOT * SLOT + 8 * NBAR + 8 * EPI_WARPS + 64 + 4 * K;
   static constexpr int TMEM_COLS = HALVES * K;
   static constexpr int THREADS = 64 + 32 * EPI_WARPS;
   static_assert(NSLOT * SLOT >= EPI_WARPS * EPI_WARP_BYTES, "epilogue tiles must fit");
 };
 
 template <int K>
-__global__ void __launch_bounds__(NsCfg<K>::THREADS, 1) ns_block_kernel(const __grid_constant__ NsMaps maps, const NsParams p) {
+__global__ void __launch_bounds__(NsCfg<K>::THREADS, 1)
+ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsParams p) {
   using C = NsCfg<K>;
   if (p.status && *p.status) return;
   const int b = blockIdx.x, row_b = b * K;
@@ -82,8 +97,17 @@ __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1) ns_block_kernel(const __
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t sm_u = smem_u32(smem);
   const uint32_t sR = sm_u + C::NRING * C::SLOT;
+  volatile int* not_converged = (volatile int*)(tmem_slot + 2);
+  float* cn = (float*)(tmem_slot + 16);  // [K] column square norms of the result
+  int prob = -1;
+  for (int q = 0; q < p.n; ++q)
+    if (b >= p.blk0[q] && b < p.blk0[q + 1]) prob = q;
+  const bool want_c = prob >= 0 && p.c;
+  for (int e = threadIdx.x; e < K; e += C::THREADS) cn[e] = 0.f;
+  if (b == 0 && threadIdx.x < p.n_ticks && p.tick[threadIdx.x]) *p.tick[threadIdx.x] += 1.f;
 
   if (threadIdx.x == 0) {
+    *not_converged = 0;
     tma_prefetch_desc(&maps.a);
     tma_prefetch_desc(&maps.xh_mn);
     tma_prefetch_desc(&maps.xl_mn);
@@ -279,7 +303,7 @@ __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1) ns_block_kernel(const __
       if (!ok) break;
       const double r2 = residual2();
       const bool last = (r2 <= p.gate2) || it == p.max_rounds - 1;
-      if (last && threadIdx.x == 64) p.rn[b] = r2;
+      if (last && threadIdx.x == 64 && !(r2 <= p.accept2)) *not_converged = 1;
       ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, accph, abort_flag, p.status));
       accph ^= 1u;
       if (!ok) break;
@@ -339,6 +363,21 @@ __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1) ns_block_kernel(const __
         }
         __syncwarp();
         if (last) {
+          if (want_c) {
+            // column sums of squares over the tile's 32 rows: a transposing reduction leaves column `lane` in each lane
+            float t2[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) t2[e] = v[e] * v[e];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+              for (int e = 0; e < o; ++e) {
+                const float keep = (lane & o) ? t2[e + o] : t2[e], send = (lane & o) ? t2[e] : t2[e + o];
+                t2[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+              }
+            }
+            atomicAdd(&cn[col0 + lane], t2[0]);
+          }
           const int sw = lane & 7;
 #pragma unroll
           for (int c = 0; c < 8; ++c)
@@ -373,6 +412,44 @@ __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1) ns_block_kernel(const __
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
   }
+  if (*abort_flag) return;
+  const size_t off = (size_t)b * K * K;
+  if (*not_converged) {
+    // a change of the transform that the rounds could not follow (or a singular block): elimination
+    if (threadIdx.x == 0 && p.redo_count) atomicAdd(p.redo_count, 1);
+    float* X = p.X + off;
+    asm volatile("fence.proxy.async;" ::: "memory");  // (the bulk stores to X are complete; this thread's view of it follows)
+    for (int e = threadIdx.x; e < K * K; e += C::THREADS) X[e] = __uint_as_float((uint32_t)p.A[off + e] << 16);
+    if (!gauss_jordan(X, K, reinterpret_cast<float*>(smem), p.status)) return;
+    for (int t = threadIdx.x; t < K; t += C::THREADS) {
+      float c = 0.f;
+      for (int i = 0; i < K; ++i) {
+        const float x = X[(size_t)i * K + t];
+        const __nv_bfloat16 h = __float2bfloat16_rn(x);
+        p.hi[off + (size_t)i * K + t] = __bfloat16_as_ushort(h);
+        p.lo[off + (size_t)i * K + t] = __bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(h)));
+        c = fmaf(x, x, c);
+      }
+      cn[t] = c;
+    }
+    __syncthreads();
+  }
+  if (want_c) {
+    float* cw = p.cw[prob];
+    for (int t = threadIdx.x; t < K; t += C::THREADS) {
+      float v = cn[t];
+      p.c[(size_t)b * K + t] = v;
+      if (cw) {
+        const int g = p.g[prob], col = (b - p.blk0[prob]) * K + t;
+        if (g % 32 == 0) {  // (whole warps: K is a multiple of 32)
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane == 0) atomicAdd(&cw[col / g], v);
+        } else {
+          atomicAdd(&cw[col / g], v);
+        }
+      }
+    }
+  }
 }
 
 template <int K>
@@ -397,8 +474,9 @@ static bool make_map_hl(CUtensorMap* m, const uint16_t* hi, const uint16_t* lo, 
 }
 
 // A, hi, lo: bf16 [nb * k, k]; X: fp32 [nb, k, k] (written, not read)
-static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uint16_t* lo, float* X, int nb, int k, const NsParams& p) {
+static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uint16_t* lo, float* X, int nb, int k, NsParams p) {
   NsMaps m;
+  p.A = A; p.hi = hi; p.lo = lo; p.X = X;
   const long long rows = (long long)nb * k;
   if (!make_map_bf16(&m.a, A, k, rows, k, k) || !make_map_bf16(&m.xh_mn, hi, k, rows, k, 64) || !make_map_bf16(&m.xl_mn, lo, k, rows, k, 64) ||
       !make_map_bf16(&m.xh_k, hi, k, rows, k, k) || !make_map_hl(&m.xhl, hi, lo, rows, k) ||
@@ -440,7 +518,6 @@ __global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* __re
 // Shared memory: T area (4 slots; the split rows of G use it before T exists, two stages of hi + lo) + ring.
 // ------------------------------------------------------------------------------------------------
 enum { KK_MINV_PATH = 0, KK_PENALTY = 1 };
-constexpr int KK_MAX_PROBS = 8;
 
 struct ChainMaps {
   CUtensorMap a1[2];  // hi / lo, first product: KK_MINV_PATH boxes of 64 x 64, KK_PENALTY boxes of K rows x 64

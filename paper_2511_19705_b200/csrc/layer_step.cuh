@@ -28,21 +28,31 @@ struct LyPrepArgs {
   int n, k;
   int blk0[LY_MAX_PROBS + 1];       // first operator block of problem p in the concatenated arrays
   const float* M[LY_MAX_PROBS];
-  float* step_counter[LY_MAX_PROBS];
   int pair_blk0;                    // first block of the pairs (they come last); total blocks when there is none
-  float* Mc;
-  uint16_t* Ab;
-  float* Mf;                        // fp32 parameters of the pair blocks, contiguous (orthonormality penalty)
+  uint16_t *Ab, *Pl;                // bf16(M), all blocks; M - bf16(M), pair blocks (orthonormality penalty)
   float* grad;                      // cleared: all blocks
   float* gMinv;                     // cleared: pair blocks
-  uint4* zone;                      // cleared: the per-step accumulators of every matrix and problem
+  uint4* zone;                      // cleared: the accumulators of one step
   long long zone_n16;
-  double* rn;
-  int rn_n;
-  int* flag;
   const int32_t* status;
 };
 
+// four parameters -> their bf16 roundings (and what is left, for the penalty's products)
+__device__ __forceinline__ void ly_put_operator(uint16_t* Ab, uint16_t* Pl, const float* m) {
+  uint32_t h[2], l[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const __nv_bfloat16 h0 = __float2bfloat16_rn(m[2 * j]), h1 = __float2bfloat16_rn(m[2 * j + 1]);
+    h[j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+    l[j] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(m[2 * j] - __bfloat162float(h0))) |
+           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(m[2 * j + 1] - __bfloat162float(h1))) << 16);
+  }
+  *reinterpret_cast<uint2*>(Ab) = make_uint2(h[0], h[1]);
+  if (Pl) *reinterpret_cast<uint2*>(Pl) = make_uint2(l[0], l[1]);
+}
+
+// Set-up of the first step of a call (the caller may have changed the parameters); the later ones are set up by the
+// parameter update of the step before.
 __global__ void __launch_bounds__(256) layer_prep_kernel(const LyPrepArgs a) {
   if (a.status && *a.status) return;
   const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -55,66 +65,12 @@ __global__ void __launch_bounds__(256) layer_prep_kernel(const LyPrepArgs a) {
     int p = 0;
     while (b >= a.blk0[p + 1]) ++p;
     const float4 m = *reinterpret_cast<const float4*>(a.M[p] + (e - (long long)a.blk0[p] * kk));
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(m.x), h1 = __float2bfloat16_rn(m.y);
-    const __nv_bfloat16 h2 = __float2bfloat16_rn(m.z), h3 = __float2bfloat16_rn(m.w);
-    *reinterpret_cast<float4*>(a.Mc + e) = make_float4(__bfloat162float(h0), __bfloat162float(h1), __bfloat162float(h2), __bfloat162float(h3));
-    *reinterpret_cast<uint2*>(a.Ab + e) = make_uint2((uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16),
-                                                     (uint32_t)__bfloat16_as_ushort(h2) | ((uint32_t)__bfloat16_as_ushort(h3) << 16));
+    const float mv[4] = {m.x, m.y, m.z, m.w};
+    ly_put_operator(a.Ab + e, e >= pair0 ? a.Pl + e : nullptr, mv);
     *reinterpret_cast<float4*>(a.grad + e) = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (e >= pair0) {
-      *reinterpret_cast<float4*>(a.Mf + (e - pair0)) = m;
-      *reinterpret_cast<float4*>(a.gMinv + e) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    if (e >= pair0) *reinterpret_cast<float4*>(a.gMinv + e) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   for (long long e = t0; e < a.zone_n16; e += stride) a.zone[e] = make_uint4(0u, 0u, 0u, 0u);
-  for (long long e = t0; e < a.rn_n; e += stride) a.rn[e] = 0.0;
-  if (t0 == 0) {
-    *a.flag = 0;
-    for (int p = 0; p < a.n; ++p)
-      if (a.step_counter[p]) *a.step_counter[p] += 1.f;
-  }
-}
-
-// Column square norms of the inverse for the single matrices' blocks (blockIdx.y = block, all singles in one launch):
-// c[b][t] = sum_i Minv[b][i][t]^2 and, for an input-axis matrix with one block per operator block, the group weights
-// of Eq. 4: cw[G] += sum_{t in G} c[t].
-struct LyColArgs {
-  int n, k;
-  int blk0[LY_MAX_PROBS + 1];   // block ranges of the singles (they come first)
-  float* cw[LY_MAX_PROBS];      // null: only c is written
-  int g[LY_MAX_PROBS];
-};
-
-__global__ void __launch_bounds__(256) layer_colnorm_kernel(const float* __restrict__ X, float* __restrict__ c, const LyColArgs a) {
-  __shared__ float part[8][33];
-  const int b = blockIdx.y, t = blockIdx.x * 32 + threadIdx.x, k = a.k;
-  int p = 0;
-  while (b >= a.blk0[p + 1]) ++p;
-  const float* Xb = X + (size_t)b * k * k;
-  float s = 0.f;
-  for (int i = threadIdx.y; i < k; i += 8) {
-    const float v = Xb[(size_t)i * k + t];
-    s = fmaf(v, v, s);
-  }
-  part[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0) {
-    float tot = 0.f;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) tot += part[q][threadIdx.x];
-    c[(size_t)b * k + t] = tot;
-    float* cw = a.cw[p];
-    if (cw) {
-      const int g = a.g[p];
-      const int col = (b - a.blk0[p]) * k + t;  // position along the transformed axis of that matrix
-      if (g >= 32) {
-        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        if (threadIdx.x == 0) atomicAdd(&cw[col / g], tot);
-      } else {
-        atomicAdd(&cw[col / g], tot);
-      }
-    }
-  }
 }
 
 // LogSumExp over the group maxima of both factors of every pair (blockIdx.y = pair): unnormalised routed
@@ -155,7 +111,10 @@ __global__ void __launch_bounds__(256) layer_lse_kernel(const LyLseArgs g) {
   }
 }
 
-// Losses, the orthonormality term of the gradient and the parameter update of every problem (blockIdx.y = problem).
+// Losses, the orthonormality term of the gradient and the parameter update of every problem (blockIdx.y = problem), and the
+// set-up of the next step: operators of the new parameters, gradients and the other set of accumulators cleared.
+// Bandwidth-bound (Adam: five arrays read, six written); as separate kernels the set-up read the parameters again and wrote
+// fp32 copies of them (9B-shaped layer: 31 + 22 us and a 34 us split beside the inverse).
 struct LyFinishArgs {
   int k;
   int blk0[LY_MAX_PROBS + 1];
@@ -169,8 +128,13 @@ struct LyFinishArgs {
   const float* amax[LY_MAX_PROBS];
   const double* orth_sq;             // per pair block: ||(M M^T - I)_b||_F^2, indexed from pair_blk0
   int pair_blk0;
-  const float* grad;
+  float* grad;
   const float* RM;                   // (M M^T - I) M, pair blocks, indexed from pair_blk0
+  int next;                          // 0: the last step of the call, nothing is set up
+  uint16_t *Ab, *Pl;
+  float* gMinv;
+  uint4* zone_next;
+  long long zone_n16;
   const int32_t* status;
 };
 
@@ -198,7 +162,7 @@ __global__ void __launch_bounds__(256) layer_finish_kernel(const LyFinishArgs f)
     f.hist[p][1] = nanf("");
   }
   float4* M4 = reinterpret_cast<float4*>(f.M[p]);
-  const float4* g4 = reinterpret_cast<const float4*>(f.grad + off);
+  float4* g4 = reinterpret_cast<float4*>(f.grad + off);
   const float4* RM4 = f.pair[p] ? reinterpret_cast<const float4*>(f.RM + (off - (long long)f.pair_blk0 * kk)) : nullptr;
   const float lr = f.lr[p];
   const long long n4 = n / 4;
@@ -240,6 +204,16 @@ __global__ void __launch_bounds__(256) layer_finish_kernel(const LyFinishArgs f)
       v4[i] = make_float4(vv[0], vv[1], vv[2], vv[3]);
     }
     M4[i] = make_float4(mv[0], mv[1], mv[2], mv[3]);
+    if (f.next) {
+      const long long e = off + 4 * i;
+      ly_put_operator(f.Ab + e, f.pair[p] ? f.Pl + e : nullptr, mv);
+      g4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (f.pair[p]) *reinterpret_cast<float4*>(f.gMinv + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  if (f.next) {
+    const long long t0 = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
+    for (long long e = t0; e < f.zone_n16; e += (long long)gridDim.x * gridDim.y * blockDim.x) f.zone_next[e] = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
@@ -310,8 +284,8 @@ struct LyMat {
   int bits;
   float *a, *usel, *coef;    // per (row, group) records, group-major
   int* idx;
-  float *cw, *agrp, *A;      // Eq. 4 weights and sums (cleared every step)
-  float* vmax;               // maximum coefficient / group maximum of the step (cleared every step)
+  float *cw, *agrp, *A;      // Eq. 4 weights and sums (accumulators: see LyPlan::zone)
+  float* vmax;               // maximum coefficient / group maximum of the step (accumulator)
   float *wmax, *winv;        // fp16 copy: max |w| and 2^-e (set by the prepare call)
   uint16_t* W16;
 };
@@ -323,7 +297,7 @@ struct LyProb {
   cafeq_opt_cfg cfg;
   float kappa;
   int blk0, nb;
-  double* acc;               // [8] cleared every step
+  double* acc;               // [8] accumulator
   float* amax;
 };
 
@@ -333,12 +307,15 @@ struct LyPlan {
   LyProb p[LY_MAX_PROBS];
   LyMat m[LY_MAX_MATS];
   // workspace
-  float *Minv, *Mc, *gMinv, *grad, *RM, *Mf, *c;
+  float *Minv, *gMinv, *grad, *RM, *c;
   KkWS kk;
   double* orth_sq;
   float* one;
+  // The accumulators of a step.  Two sets, used alternately: the update of a step reads its own and clears the other.
+  // The pointers above are those of set 0; ly_use_zone moves them.
   char* zone;
   size_t zone_bytes;
+  int zone_cur;
   size_t ws_used;
 };
 
@@ -416,11 +393,9 @@ static int ly_plan(const cafeq_layer_problem* probs, int n, void* ws, size_t ws_
   const size_t kk = (size_t)NB * L->k * L->k;
   const size_t kkP = (size_t)(NB - L->pair_blk0) * L->k * L->k;
   L->Minv = b.take<float>(kk);
-  L->Mc = b.take<float>(kk);
   L->gMinv = b.take<float>(kk);
   L->grad = b.take<float>(kk);
   L->RM = b.take<float>(kkP ? kkP : 1);
-  L->Mf = b.take<float>(kkP ? kkP : 1);
   L->c = b.take<float>((size_t)NB * L->k);
   carve_kk(b, NB, L->k, &L->kk);
   L->one = b.take<float>(64);
@@ -436,7 +411,7 @@ static int ly_plan(const cafeq_layer_problem* probs, int n, void* ws, size_t ws_
     Mt.wmax = b.take<float>(64);
     Mt.winv = Mt.wmax ? Mt.wmax + 1 : nullptr;
   }
-  // everything that is cleared at the start of every step, contiguous
+  // the accumulators, contiguous
   const size_t zone0 = b.used;
   for (int i = 0; i < nm; ++i) {
     LyMat& Mt = L->m[i];
@@ -452,9 +427,41 @@ static int ly_plan(const cafeq_layer_problem* probs, int n, void* ws, size_t ws_
   L->orth_sq = b.take<double>((size_t)(NB - L->pair_blk0) + 1);
   L->zone = ws ? (char*)ws + zone0 : nullptr;
   L->zone_bytes = b.used - zone0;
+  L->zone_cur = 0;
+  b.take<char>(L->zone_bytes);  // the second set
   L->ws_used = b.used;
   if (ws && b.overflow) return CAFEQ_ERR_WORKSPACE;
   return CAFEQ_OK;
+}
+
+// points the plan's accumulators at set z
+static void ly_use_zone(LyPlan& L, int z) {
+  const long long d = (long long)(z - L.zone_cur) * (long long)L.zone_bytes;
+  auto mv = [d](auto*& p) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(reinterpret_cast<char*>(p) + d); };
+  for (int i = 0; i < L.nm; ++i) {
+    LyMat& Mt = L.m[i];
+    mv(Mt.cw); mv(Mt.agrp); mv(Mt.A); mv(Mt.vmax);
+  }
+  for (int q = 0; q < L.n; ++q) { mv(L.p[q].acc); mv(L.p[q].amax); }
+  mv(L.orth_sq);
+  L.zone_cur = z;
+}
+
+// first step of a call, or the initial inverse: operators and cleared accumulators (set 0) from the current parameters
+static void ly_prep(cudaStream_t st, LyPlan& L, int32_t* status) {
+  LyPrepArgs a;
+  memset(&a, 0, sizeof(a));
+  a.n = L.n; a.k = L.k;
+  for (int q = 0; q < L.n; ++q) {
+    a.blk0[q] = L.p[q].blk0;
+    a.M[q] = L.p[q].M;
+  }
+  a.blk0[L.n] = L.NB;
+  a.pair_blk0 = L.pair_blk0;
+  a.Ab = L.kk.Ab; a.Pl = L.kk.Pl; a.grad = L.grad; a.gMinv = L.gMinv;
+  a.zone = reinterpret_cast<uint4*>(L.zone); a.zone_n16 = (long long)(L.zone_bytes / 16);
+  a.status = status;
+  CQ_LAUNCH(layer_prep_kernel, grid_for((long long)L.NB * L.k * L.k / 4), 256, 0, st, a);
 }
 
 // Side stream of the layer step with its fork / join events, one set per host thread and device (two threads that
@@ -493,30 +500,14 @@ static void ly_lists(const LyPlan& L, int axis, int transpose, int* out, int* cn
   }
 }
 
-// One optimisation step of every problem.  hist_row: which row of each loss history this step writes.
-static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
+// One optimisation step of every problem.  hist_row: which row of each loss history this step writes; last: no further step
+// follows in this call.
+static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t* status) {
   const int k = L.k, NB = L.NB;
-  const long long kk1 = (long long)k * k, kk = (long long)NB * kk1;
+  const long long kk1 = (long long)k * k;
   const int nbP = NB - L.pair_blk0;
   const long long offP = (long long)L.pair_blk0 * kk1;
   KkWS& w = L.kk;
-  {
-    LyPrepArgs a;
-    memset(&a, 0, sizeof(a));
-    a.n = L.n; a.k = k;
-    for (int q = 0; q < L.n; ++q) {
-      a.blk0[q] = L.p[q].blk0;
-      a.M[q] = L.p[q].M;
-      a.step_counter[q] = L.p[q].state;
-    }
-    a.blk0[L.n] = NB;
-    a.pair_blk0 = L.pair_blk0;
-    a.Mc = L.Mc; a.Ab = w.Ab; a.Mf = L.Mf; a.grad = L.grad; a.gMinv = L.gMinv;
-    a.zone = reinterpret_cast<uint4*>(L.zone); a.zone_n16 = (long long)(L.zone_bytes / 16);
-    a.rn = w.rn; a.rn_n = NS_MAX_ITERS * NB; a.flag = w.flag;
-    a.status = status;
-    CQ_LAUNCH(layer_prep_kernel, grid_for(kk / 4), 256, 0, st, a);
-  }
   bool any_lambda = false;
   for (int q = 0; q < L.n; ++q) any_lambda |= (L.p[q].pair && L.p[q].cfg.lambda_orth != 0.f);
   // The pair blocks' penalty (splits of the parameters, R = M M^T - I, R M) does not depend on the inverse: it runs on a
@@ -528,44 +519,41 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
     if (cudaEventRecord(aux->fork, st) != cudaSuccess || cudaStreamWaitEvent(aux->stream, aux->fork, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
     so = aux->stream;
   }
-  // (enqueued first: its CTAs run longer than the penalty's)
-  ns_inverse(st, L.Mc, L.Minv, nullptr, NB, k, true, w, status, true, true);
+  // (enqueued first: its CTAs run longer than the penalty's.)  The singles own the first pair_blk0 blocks: the column
+  // norms of their inverses are Eq. 4's weights.
+  {
+    NsParams eq4;
+    memset(&eq4, 0, sizeof(eq4));
+    eq4.c = L.c;
+    for (int q = 0; q < L.n; ++q) {
+      const LyProb& P = L.p[q];
+      eq4.tick[q] = P.state;
+      if (P.pair) continue;
+      const LyMat& Mt = L.m[P.m0];
+      eq4.blk0[eq4.n] = P.blk0;
+      eq4.cw[eq4.n] = (Mt.G.axis == CAFEQ_AXIS_IN && Mt.G.r == 1) ? Mt.cw : nullptr;
+      eq4.g[eq4.n] = Mt.G.g;
+      ++eq4.n;
+    }
+    eq4.blk0[eq4.n] = L.pair_blk0;
+    eq4.n_ticks = L.n;
+    const int rc = ns_inverse(st, nullptr, L.Minv, NB, k, true, w, status, true, true, &eq4);
+    if (rc) return rc;
+  }
   if (nbP > 0) {
-    // pair blocks: splits of the fp32 parameters (the transposed high halves are bf16(M)^T, the operator of the
-    // first factors' pass), then the penalty's norm and (M M^T - I) M in one launch
-    launch_split(so, L.Mf, k, (long long)nbP * kk1, w.Ph + offP, w.Pl + offP, w.Qh + offP, nullptr, nullptr, status);
-    const int rc = penalty_tc(so, w.Ph + offP, w.Pl + offP, L.RM, any_lambda, L.orth_sq, 1, nbP, k, status);
+    // the penalty's norm and (M M^T - I) M from the splits of the fp32 parameters
+    const int rc = penalty_tc(so, w.Ab + offP, w.Pl + offP, L.RM, any_lambda, L.orth_sq, 1, nbP, k, status);
     if (rc) return rc;
   }
   if (aux && cudaEventRecord(aux->join, aux->stream) != cudaSuccess) return CAFEQ_ERR_CUDA;
-  if (aux && cudaStreamWaitEvent(st, aux->join, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
-  // Eq. 4 weights of the single matrices (they own the first pair_blk0 blocks)
-  if (L.pair_blk0 > 0) {
-    LyColArgs ca;
-    memset(&ca, 0, sizeof(ca));
-    ca.k = k;
-    int ns = 0;
-    for (int q = 0; q < L.n; ++q) {
-      const LyProb& P = L.p[q];
-      if (P.pair) continue;
-      const Geo& G = L.m[P.m0].G;
-      ca.blk0[ns] = P.blk0;
-      ca.cw[ns] = (G.axis == CAFEQ_AXIS_IN && G.r == 1) ? L.m[P.m0].cw : nullptr;
-      ca.g[ns] = G.g;
-      ++ns;
-    }
-    ca.blk0[ns] = L.pair_blk0;
-    ca.n = ns;
-    CQ_LAUNCH(layer_colnorm_kernel, dim3(k / 32, L.pair_blk0), dim3(32, 8), 0, st, L.Minv, L.c, ca);
-    for (int q = 0; q < L.n; ++q) {
-      const LyProb& P = L.p[q];
-      if (P.pair) continue;
-      const LyMat& Mt = L.m[P.m0];
-      const Geo& G = Mt.G;
-      if (G.axis == CAFEQ_AXIS_IN && G.r == 1) continue;
-      if (G.axis == CAFEQ_AXIS_IN) CQ_LAUNCH(cw_in_kernel, (G.ng + 127) / 128, 128, 0, st, L.c + (size_t)P.blk0 * k, G.d_in, G.g, k, G.r, Mt.cw);
-      else CQ_LAUNCH(cw_out_kernel, (G.d_out + 127) / 128, 128, 0, st, L.c + (size_t)P.blk0 * k, G.d_out, G.g, k, G.r, Mt.cw);
-    }
+  for (int q = 0; q < L.n; ++q) {
+    const LyProb& P = L.p[q];
+    if (P.pair) continue;
+    const LyMat& Mt = L.m[P.m0];
+    const Geo& G = Mt.G;
+    if (G.axis == CAFEQ_AXIS_IN && G.r == 1) continue;
+    if (G.axis == CAFEQ_AXIS_IN) CQ_LAUNCH(cw_in_kernel, (G.ng + 127) / 128, 128, 0, st, L.c + (size_t)P.blk0 * k, G.d_in, G.g, k, G.r, Mt.cw);
+    else CQ_LAUNCH(cw_out_kernel, (G.d_out + 127) / 128, 128, 0, st, L.c + (size_t)P.blk0 * k, G.d_out, G.g, k, G.r, Mt.cw);
   }
   // transform passes: all matrices of a form in one launch, and both forms in the same launch when each has
   // enough tiles for its share of the CTAs
@@ -593,7 +581,9 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
         p.cw = Mt.cw; p.kappa = P.kappa; p.coef = Mt.coef; p.lossacc = P.acc;
         p.Aacc = (Mt.G.axis == CAFEQ_AXIS_IN) ? Mt.agrp : Mt.A;
       } else {
-        s.Tb = (Mt.side == 0) ? w.Qh + off : w.Xh[w.cur] + off;  // bf16(M)^T for U = W1 M, bf16(M^-1) for V = M^-1 W2
+        // U = W1 M: the operator is bf16(M)^T, read transposed; V = M^-1 W2: bf16(M^-1)
+        s.Tb = (Mt.side == 0) ? w.Ab + off : w.Xh[w.cur] + off;
+        p.t_mn = Mt.side == 0;
         p.epi = EPI_ABSMAX;
       }
       ntile[form] += (long long)Mt.G.n / 32768;  // tiles hold 32768 entries in both forms
@@ -726,6 +716,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
     const int rc = minv_path_tc(st, L.gMinv, L.grad, NB, k, w, status, &cp);
     if (rc) return rc;
   }
+  if (aux && cudaStreamWaitEvent(st, aux->join, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
   {
     LyFinishArgs f;
     memset(&f, 0, sizeof(f));
@@ -746,9 +737,13 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, int32_t* status) {
     f.blk0[L.n] = NB;
     f.orth_sq = L.orth_sq; f.pair_blk0 = L.pair_blk0;
     f.grad = L.grad; f.RM = L.RM;
+    f.next = last ? 0 : 1;
+    f.Ab = w.Ab; f.Pl = w.Pl; f.gMinv = L.gMinv;
+    f.zone_next = reinterpret_cast<uint4*>(L.zone + (L.zone_cur ^ 1) * L.zone_bytes); f.zone_n16 = (long long)(L.zone_bytes / 16);
     f.status = status;
     CQ_LAUNCH(layer_finish_kernel, dim3(grid_for(nmax / 4, 256, 148 * 4), L.n), 256, 0, st, f);
   }
+  ly_use_zone(L, L.zone_cur ^ 1);
   return CAFEQ_OK;
 }
 
@@ -780,24 +775,8 @@ extern "C" int cafeq_layer_prepare(const cafeq_layer_problem* probs, int n, int3
   CQ_LAUNCH(fill_f32_kernel, 1, 32, 0, st, L.one, 0.f, 16);  // (also clears the running count of elimination fall-backs)
   CQ_LAUNCH(set_f32_kernel, 1, 1, 0, st, L.one, 1.f);
   // inverse of the initial transforms from scratch; every step afterwards refines the previous step's inverse
-  const long long kk = (long long)L.NB * L.k * L.k;
-  {
-    LyPrepArgs a;
-    memset(&a, 0, sizeof(a));
-    a.n = L.n; a.k = L.k;
-    for (int q = 0; q < L.n; ++q) {
-      a.blk0[q] = L.p[q].blk0;
-      a.M[q] = L.p[q].M;
-    }
-    a.blk0[L.n] = L.NB;
-    a.pair_blk0 = L.pair_blk0;
-    a.Mc = L.Mc; a.Ab = L.kk.Ab; a.Mf = L.Mf; a.grad = L.grad; a.gMinv = L.gMinv;
-    a.zone = reinterpret_cast<uint4*>(L.zone); a.zone_n16 = (long long)(L.zone_bytes / 16);
-    a.rn = L.kk.rn; a.rn_n = NS_MAX_ITERS * L.NB; a.flag = L.kk.flag;
-    a.status = status;
-    CQ_LAUNCH(layer_prep_kernel, grid_for(kk / 4), 256, 0, st, a);
-  }
-  ns_inverse(st, L.Mc, L.Minv, nullptr, L.NB, L.k, false, L.kk, status, true);
+  ly_prep(st, L, status);
+  if ((rc = ns_inverse(st, nullptr, L.Minv, L.NB, L.k, false, L.kk, status, true))) return rc;
   return last_launch();
 }
 
@@ -809,8 +788,9 @@ extern "C" int cafeq_optimize_layer(const cafeq_layer_problem* probs, int n, int
   LyPlan L;
   if ((rc = ly_plan(probs, n, ws, ws_bytes, &L))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
+  if (steps > 0) ly_prep(st, L, status);
   for (int it = 0; it < steps; ++it)
-    if ((rc = ly_step(st, L, it, status))) return rc;
+    if ((rc = ly_step(st, L, it, it + 1 == steps, status))) return rc;
   return last_launch();
 }
 
