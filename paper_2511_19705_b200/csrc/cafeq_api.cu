@@ -425,6 +425,35 @@ static void launch_absmax(cudaStream_t st, const float* U, long long ld, const G
   CQ_LAUNCH(absmax_kernel, (unsigned)blocks, 256, 0, st, U, ld, G.d_out, G.ng, G.g, a, usel, idx, status);
 }
 
+// Group quantiser of an fp32 matrix U [rows, ng g] (pitch ld; Delta / Uhat share it): maxima, signed arg-max values, arg-max
+// positions, scales, residual, dequantised values, codes -- each optional except a / usel / idx.
+static void launch_group_quant(cudaStream_t st, const float* U, long long ld, int rows, int ng, int g, float qmax, const void* offsets,
+                               int off_kind, float* a, float* usel, int* idx, float* Delta, float* Uhat, int8_t* codes, float* scales,
+                               int32_t* status) {
+  const long long groups = (long long)rows * ng;
+  const bool vec = g % 4 == 0 && g <= 1024 && ld % 4 == 0 && !(((uintptr_t)U | (uintptr_t)Delta | (uintptr_t)Uhat) & 15) &&
+                   !((uintptr_t)codes & 3);
+  if (vec) {
+#define GQ(L, N)                                                                                                              \
+  CQ_LAUNCH((group_quant_kernel<L, N>), (unsigned)((groups * L + 255) / 256), 256, 0, st, U, ld, rows, ng, g, qmax, offsets, off_kind, \
+            a, usel, idx, Delta, Uhat, codes, scales, status)
+    // as many lanes as the group has float4s, up to a warp
+    if (g <= 32) GQ(8, 1);
+    else if (g <= 64) GQ(16, 1);
+    else if (g <= 128) GQ(32, 1);
+    else if (g <= 256) GQ(32, 2);
+    else if (g <= 512) GQ(32, 4);
+    else GQ(32, 8);
+#undef GQ
+    return;
+  }
+  CQ_LAUNCH(absmax_kernel, (unsigned)((groups * 32 + 255) / 256), 256, 0, st, U, ld, rows, ng, g, a, usel, idx, status);
+  if (Delta || Uhat || codes)
+    CQ_LAUNCH(quant_kernel, grid_for((long long)rows * ng * g), 256, 0, st, U, ld, rows, ng * g, g, a, qmax, offsets, off_kind, Delta, Uhat,
+              codes, status);
+  if (scales) CQ_LAUNCH(scales_kernel, grid_for(groups), 256, 0, st, a, scales, groups, qmax, status);
+}
+
 // gm: the (row, group) records are group-major (written by the fused pass) instead of row-major
 static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const float* coef, const int* idx, float* gT,
                            int transpose_out, const int32_t* status, int gm) {
@@ -686,13 +715,8 @@ static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits
   if (applied) {
   } else if (Tc) launch_apply(st, W, 1, G.ld, G, Tc, transposed, w.U, G.d_in, GEMM_STORE, nullptr, status);
   else CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G.n), 256, 0, st, (const uint16_t*)W, G.ld, G.d_out, G.d_in, w.U);
-  launch_absmax(st, w.U, G.d_in, G, w.a, w.usel, w.idx, status);
-  if (want_delta || Uhat || codes)
-    CQ_LAUNCH(quant_kernel, grid_for(G.n), 256, 0, st, w.U, G.d_in, G.d_out, G.d_in, G.g, w.a, qmax_of(bits), offsets, off_kind,
-              want_delta ? w.D : nullptr, Uhat, codes, status);
-  if (scales)
-    CQ_LAUNCH(scales_kernel, grid_for((long long)G.d_out * G.ng), 256, 0, st, w.a, scales, (long long)G.d_out * G.ng,
-              qmax_of(bits), status);
+  launch_group_quant(st, w.U, G.d_in, G.d_out, G.ng, G.g, qmax_of(bits), offsets, off_kind, w.a, w.usel, w.idx, want_delta ? w.D : nullptr,
+                     Uhat, codes, scales, status);
   return false;
 }
 

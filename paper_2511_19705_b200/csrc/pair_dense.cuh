@@ -225,14 +225,8 @@ namespace cafeq {
 // Group quantiser on an fp32 matrix T [rows, cols] (groups of g along the row): codes, scales, dequantised values
 static void quant_matrix(cudaStream_t st, const float* T, int rows, int cols, int g, int bits, int8_t* codes, float* scales,
                          float* That, DenseWS& w, int32_t* status) {
-  Geo G;
-  memset(&G, 0, sizeof(G));
-  G.d_out = rows; G.d_in = cols; G.g = g; G.ng = cols / g; G.ld = cols; G.n = (long long)rows * cols;
-  launch_absmax(st, T, cols, G, w.qa, w.qusel, w.qidx, status);
-  CQ_LAUNCH(quant_kernel, grid_for(G.n), 256, 0, st, T, (long long)cols, rows, cols, g, w.qa, qmax_of(bits), nullptr,
-            CAFEQ_OFFSETS_NONE, nullptr, That, codes, status);
-  if (scales)
-    CQ_LAUNCH(scales_kernel, grid_for((long long)rows * G.ng), 256, 0, st, w.qa, scales, (long long)rows * G.ng, qmax_of(bits), status);
+  launch_group_quant(st, T, cols, rows, cols / g, g, qmax_of(bits), nullptr, CAFEQ_OFFSETS_NONE, w.qa, w.qusel, w.qidx, nullptr, That,
+                     codes, scales, status);
 }
 
 // P = U_exp^T V^T for stored U [h, d1], V [d3, rh] (fp32): fp32 P [d1, d3] with its splits in w.Ph/Pl/PTh/PTl
