@@ -181,7 +181,7 @@ static void learned_offsets_run(cudaStream_t st, int bits, const Geo& G1, const 
               w.Uh, nullptr, status);
     residual(w.acc + 40);
     learn_gemm(st, w.R, 1, d3, w.Uh, 1, d1, w.G2, d3, h, d1, 2.f, status);
-    CQ_LAUNCH(expand_cols_kernel, grid_for(n2), 256, 0, st, w.G2, d3, h, k, r, 1.f, w.gV);
+    CQ_LAUNCH(expand_cols_any_kernel, grid_for(n2), 256, 0, st, w.G2, d3, h, k, r, 1.f, w.gV);
     CQ_LAUNCH(row_sumsq_kernel, hrows, 256, 0, st, w.Uh, h, d1, 2.f, w.H2);
     CQ_LAUNCH(offsets_direction_kernel, grid_for(n2), 256, 0, st, w.gV, w.V, d3, rh, G2.g, w.a2, qm, w.H2, 0, k, r, w.gV, w.T2);
     launch_pair_product(st, w.Uh, 0, d1, w.T2, 0, rh, G1, G2, w.D, status);

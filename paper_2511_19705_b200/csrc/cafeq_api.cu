@@ -269,8 +269,6 @@ static int launch_kk_tc(cudaStream_t st, int nterms, const uint16_t* const* A, c
   p.nterms = nterms;
   p.rowsA_per_batch = p.rowsB_per_batch = k;
   p.divA = 1;
-  p.a_rep_k = k;
-  p.a_rep_r = 1;
   p.alpha = alpha; p.beta = beta; p.gamma = gamma;
   p.C0 = C0; p.ldc0 = k; p.sC0b = (long long)k * k;
   p.C = C; p.ldc = k; p.sCb = (long long)k * k;
@@ -663,7 +661,7 @@ static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_
   TgParams p;
   memset(&p, 0, sizeof(p));
   p.nterms = 1; p.K = k; p.batch = G.nbq; p.alpha = 1.f;
-  p.a_rep_k = k; p.a_rep_r = 1; p.divA = 1;
+  p.divA = 1;
   p.C = U; p.ldc = G.d_in;
   p.status = status;
   if (G.axis == CAFEQ_AXIS_IN) {
@@ -936,8 +934,8 @@ struct SingleWS {
   float *Mc, *Minv, *gMinv, *tmp, *c, *A;
   double* acc;
   KkWS kk;
-  // tensor-core straight-through path: second bf16 term of the residual, both terms transposed, N = Minv^T Minv
-  uint16_t *Dlo, *DTh, *DTl;
+  // tensor-core straight-through path: second bf16 term of the residual, N = Minv^T Minv
+  uint16_t* Dlo;
   float* Nf;
   bool lean;  // carved without matrix-sized scratch: only the fused surrogate path may run
   int err;    // host-side error found while enqueuing a step
@@ -957,8 +955,6 @@ static bool carve_single(Bump& b, const Geo& G, SingleWS* s, bool need_E, bool l
   s->acc = b.take<double>(8);
   carve_kk(b, G.nbT, G.k, &s->kk);
   s->Dlo = lean ? nullptr : b.take<uint16_t>(G.n);
-  s->DTh = lean ? nullptr : b.take<uint16_t>(G.n);
-  s->DTl = lean ? nullptr : b.take<uint16_t>(G.n);
   s->Nf = b.take<float>(kk);
   return !b.overflow;
 }
@@ -1050,24 +1046,20 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     // with the residual as a two-term bf16 split (three-term products: fp32-grade).
     KkWS& w = s.kk;
     const int c = w.cur;
-    {
-      dim3 tg((G.d_in + 31) / 32, (G.d_out + 31) / 32);
-      CQ_LAUNCH(transpose_bf16_kernel, tg, dim3(32, 8), 0, st, s.m.Dbf, G.d_out, G.d_in, (long long)G.d_in, s.DTh);
-      CQ_LAUNCH(transpose_bf16_kernel, tg, dim3(32, 8), 0, st, s.Dlo, G.d_out, G.d_in, (long long)G.d_in, s.DTl);
-    }
-    {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the d_out rows
+    {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the d_out rows of the residual as it is stored
       TgOperand oa[3], ob[3];
-      const uint16_t* at[3] = {s.DTh, s.DTl, s.DTh};
-      const uint16_t* bt[3] = {s.DTh, s.DTh, s.DTl};
+      const uint16_t* at[3] = {s.m.Dbf, s.Dlo, s.m.Dbf};
+      const uint16_t* bt[3] = {s.m.Dbf, s.m.Dbf, s.Dlo};
       for (int t = 0; t < 3; ++t) {
-        oa[t] = TgOperand{at[t], G.d_in, G.d_out, G.d_out};
-        ob[t] = TgOperand{bt[t], G.d_in, G.d_out, G.d_out};
+        oa[t] = TgOperand{at[t], G.d_out, G.d_in, G.d_in};
+        ob[t] = TgOperand{bt[t], G.d_out, G.d_in, G.d_in};
       }
       TgParams p;
       memset(&p, 0, sizeof(p));
       p.M = p.N = k; p.K = G.d_out; p.batch = G.nbT; p.nterms = 3;
-      p.rowsA_per_batch = p.rowsB_per_batch = k;
-      p.divA = 1; p.a_rep_k = G.d_out; p.a_rep_r = 1;
+      p.a_mn = p.b_mn = 1;
+      p.colsA_per_batch = p.colsB_per_batch = k;
+      p.divA = 1;
       p.alpha = 1.f;
       p.C = s.tmp; p.ldc = k; p.sCb = (long long)k * k;
       p.Chi = w.Ph; p.Clo = w.Pl;
@@ -1110,7 +1102,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       memset(&p, 0, sizeof(p));
       p.M = G.d_out; p.N = k; p.K = k; p.batch = G.nbT; p.nterms = 3;
       p.rowsA_per_batch = 0; p.colsA_per_batch = k; p.rowsB_per_batch = k;
-      p.divA = 1; p.a_rep_k = k; p.a_rep_r = 1;
+      p.divA = 1;
       p.alpha = 2.f;
       p.C = s.m.D; p.ldc = G.d_in; p.sCb = k;  // batch b writes the columns [b k, b k + k)
       p.status = status;
@@ -1313,38 +1305,59 @@ struct PairWS {
   KkWS kk;
   DenseWS dn;
   bool dense;  // the product term runs on the tensor cores (every dimension a multiple of 64)
-  uint16_t *W2T, *gVTh, *gVTl;  // [r h, d3]: transposed second factor and transposed split of its gradient
+  uint16_t *gVh, *gVl;          // [d3, r h]: split of the second factor's gradient
   uint16_t* W1T;                // [d1, h]: transposed first factor (its apply contracts down the rows)
   bool lean;                    // carved without matrix-sized scratch: only the fused LogSumExp path may run
   int err;
 };
 
-// Operator gradient of a block-diagonal apply as batched k x k tensor-core products with a two-term split of the
-// fp32 factor: out[b][m][n] (+)= sum_l A[(b r + rep) k + m][l] * (Bh + Bl)[(b r + rep) k + n][l], summed over rep.
-// A bf16 [nb r k, K] (pitch lda), Bh / Bl bf16 [nb r k, K] (pitch K).
-static void opgrad_tc(cudaStream_t st, const uint16_t* A, long long lda, const uint16_t* Bh, const uint16_t* Bl, int nb, int r,
-                      int k, int K, float* out, bool a_is_split_side, int32_t* status) {
-  (void)a_is_split_side;
+// Operator gradients of a block-diagonal apply as batched k x k tensor-core products with a two-term split of the fp32 factor.
+// Output axis: out[b][m][n] = sum_l A[b k + m][l] (Bh + Bl)[b k + n][l]; A bf16 [nb k, K] (pitch lda), Bh / Bl [nb k, K].
+static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, const uint16_t* Bh, const uint16_t* Bl, int nb, int k, int K,
+                         float* out, int32_t* status) {
+  TgOperand oa[2], ob[2];
+  oa[0] = oa[1] = TgOperand{A, (long long)nb * k, K, lda};
+  ob[0] = TgOperand{Bh, (long long)nb * k, K, K};
+  ob[1] = TgOperand{Bl, (long long)nb * k, K, K};
+  TgParams p;
+  memset(&p, 0, sizeof(p));
+  p.M = p.N = k; p.K = K; p.batch = nb; p.nterms = 2;
+  p.rowsA_per_batch = p.rowsB_per_batch = k;
+  p.divA = 1;
+  p.alpha = 1.f;
+  p.C = out; p.ldc = k; p.sCb = (long long)k * k;
+  p.min_ctas = 148;  // long contraction, few output tiles: the narrowest tile
+  p.status = status;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return tg_launch(st, oa, ob, p);
+}
+// Input axis: out[b][m][n] = sum over replicas and rows o of (Ah + Al)[o][(b r + rep) k + m] B[o][(b r + rep) k + n]; both
+// factors as they are stored (contraction down the rows: MN-major operands), B bf16 [R, nb r k] (pitch ldb), Ah / Al dense.
+static int opgrad_in_tc(cudaStream_t st, const uint16_t* Ah, const uint16_t* Al, const uint16_t* B, long long ldb, int nb, int r, int k,
+                        int R, float* out, int32_t* status) {
   for (int rep = 0; rep < r; ++rep) {
     TgOperand oa[2], ob[2];
-    const long long rows = (long long)nb * r * k - (long long)rep * k;
-    oa[0] = oa[1] = TgOperand{A + (long long)rep * k * lda, rows, K, lda};
-    ob[0] = TgOperand{Bh + (long long)rep * k * K, rows, K, K};
-    ob[1] = TgOperand{Bl + (long long)rep * k * K, rows, K, K};
+    const long long cols = (long long)nb * r * k, c0 = (long long)rep * k;
+    oa[0] = TgOperand{Ah + c0, R, cols - c0, cols};
+    oa[1] = TgOperand{Al + c0, R, cols - c0, cols};
+    ob[0] = ob[1] = TgOperand{B + c0, R, cols - c0, ldb};
     TgParams p;
     memset(&p, 0, sizeof(p));
-    p.M = p.N = k; p.K = K; p.batch = nb; p.nterms = 2;
-    p.rowsA_per_batch = p.rowsB_per_batch = r * k;
-    p.divA = 1; p.a_rep_k = K; p.a_rep_r = 1;
+    p.M = p.N = k; p.K = R; p.batch = nb; p.nterms = 2;
+    p.a_mn = p.b_mn = 1;
+    p.colsA_per_batch = p.colsB_per_batch = r * k;
+    p.divA = 1;
     p.alpha = 1.f;
     p.beta = rep ? 1.f : 0.f;
     p.C0 = rep ? out : nullptr; p.ldc0 = k; p.sC0b = (long long)k * k;
     p.C = out; p.ldc = k; p.sCb = (long long)k * k;
-    p.min_ctas = 148;  // long contraction, few output tiles: the narrowest tile
+    p.min_ctas = 148;
     p.status = status;
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    tg_launch(st, oa, ob, p);
+    const int rc = tg_launch(st, oa, ob, p);
+    if (rc) return rc;
   }
+  return CAFEQ_OK;
 }
 
 static bool dense_ok(const Geo& G1, const Geo& G2) {
@@ -1370,12 +1383,11 @@ static bool carve_pair(Bump& b, const Geo& G1, const Geo& G2, PairWS* p, bool ne
   carve_kk(b, G1.nbT, G1.k, &p->kk);
   p->dense = need_R && dense_ok(G1, G2);
   if (p->dense) carve_dense(b, G1.d_out, G1.d_in, G2.d_out, G2.r, G1.k, G1.ng, G2.ng, &p->dn);
-  p->W2T = p->gVTh = p->gVTl = p->W1T = nullptr;
+  p->gVh = p->gVl = p->W1T = nullptr;
   if (p->dense) {
     p->W1T = b.take<uint16_t>(G1.n);
-    p->W2T = b.take<uint16_t>(G2.n);
-    p->gVTh = b.take<uint16_t>(G2.n);
-    p->gVTl = b.take<uint16_t>(G2.n);
+    p->gVh = b.take<uint16_t>(G2.n);
+    p->gVl = b.take<uint16_t>(G2.n);
   }
   return !b.overflow;
 }
@@ -1535,7 +1547,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
       launch_dense_tc(st, 3, a, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, status);
-      CQ_LAUNCH(expand_cols_kernel, grid_for((long long)w.d3 * w.rh), 256, 0, st, w.X0T, w.d3, w.h, w.k, w.r, 1.f, w.V);
+      CQ_LAUNCH(expand_cols_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f, w.V);
     }
     {  // g Uhat [h, d1] = 2 fold(Vhat^T) R^T
       dim3 grid((w.d3 + 31) / 32, w.h / 32);
@@ -1558,22 +1570,14 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, gradM, 0.f, kk);
       CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, p.gMinv, 0.f, kk);
     }
-    const bool og_tc = tc && ((uintptr_t)W1 % 16 == 0) && (G1.ld % 8 == 0) && ((uintptr_t)W2 % 4 == 0) && G1.r == 1;
+    const bool og_tc = tc && ((uintptr_t)W1 % 16 == 0) && (G1.ld % 8 == 0) && ((uintptr_t)W2 % 16 == 0) && (G2.ld % 8 == 0) && G1.r == 1;
     if (og_tc) {
-      // U side (operator M^T): gradM[b][m][n] = sum_c W1[b k + m][c] gU[b k + n][c], contraction along the rows' own
-      // direction: both operands as they are stored
+      // U side (operator M^T): gradM[b][m][n] = sum_c W1[b k + m][c] gU[b k + n][c]
       launch_split_rect(st, w.U, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status);
-      opgrad_tc(st, (const uint16_t*)W1, G1.ld, w.Awh, w.Awl, G1.nbT, 1, k, G1.d_in, gradM, false, status);
-      // V side (operator Minv): gMinv[b][i][j] = sum over replicas and rows o of gV[o][.. + i] W2[o][.. + j]: the
-      // contraction runs down the columns, so both factors are transposed first
-      {
-        dim3 tg((G2.d_in + 31) / 32, (G2.d_out + 31) / 32);
-        CQ_LAUNCH(transpose_bf16_kernel, tg, dim3(32, 8), 0, st, (const uint16_t*)W2, G2.d_out, G2.d_in, G2.ld, p.W2T);
-      }
-      launch_split_rect(st, w.V, w.d3, w.rh, w.rh, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, p.gVTh, p.gVTl, status);
-      opgrad_tc(st, p.W2T, G2.d_out, p.gVTh, p.gVTl, G1.nbT, G2.r, k, G2.d_out, p.RM, true, status);
-      // (W2^T as the first factor gives the transpose: RM[b][j][i]; put it back as gMinv[b][i][j])
-      CQ_LAUNCH(transpose_blocks_kernel, grid_for(kk), 256, 0, st, p.RM, p.gMinv, k, kk);
+      if ((p.err = opgrad_out_tc(st, (const uint16_t*)W1, G1.ld, w.Awh, w.Awl, G1.nbT, k, G1.d_in, gradM, status))) return;
+      // V side (operator Minv): gMinv[b][i][j] = sum over replicas and rows o of gV[o][.. + i] W2[o][.. + j]
+      launch_split_rect(st, w.V, w.d3, w.rh, w.rh, 1.f, nullptr, nullptr, nullptr, p.gVh, p.gVl, nullptr, nullptr, status);
+      if ((p.err = opgrad_in_tc(st, p.gVh, p.gVl, (const uint16_t*)W2, G2.ld, G1.nbT, G2.r, k, G2.d_out, p.gMinv, status))) return;
     } else {
       launch_opgrad(st, w.U, G1.d_in, W1, 1, G1.ld, G1, gradM, 1, 1.f, status);    // U side: operator M^T
       launch_opgrad(st, w.V, G2.d_in, W2, 1, G2.ld, G2, p.gMinv, 0, 1.f, status);  // V side: operator Minv
@@ -1803,8 +1807,13 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
       if ((rc = ns_inverse(st, Mc, Minv, G1.nbT, G1.k, false, kkw, status))) return rc;
     } else launch_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, status);
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, Minv, Minv_c, kk, status);
-    launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
-    launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);
+    // both products on the tensor cores where the shape allows (bf16 operands, fp32 accumulation either way); the operators in
+    // applied orientation and the transposed first factor use scratch that the rounding fills later
+    uint16_t *T1 = kkw.Ph, *T2 = kkw.Qh;
+    CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Mc, T1, G1.k, kk, 1, status);
+    CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Minv_c, T2, G1.k, kk, 0, status);
+    if (!apply_tc(st, W1, G1, T1, w.U, w.UTh, status)) launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
+    if (!apply_tc(st, W2, G2, T2, w.V, nullptr, status)) launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);
   } else {
     CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G1.n), 256, 0, st, (const uint16_t*)W1, G1.ld, G1.d_out, G1.d_in, w.U);
     CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G2.n), 256, 0, st, (const uint16_t*)W2, G2.ld, G2.d_out, G2.d_in, w.V);

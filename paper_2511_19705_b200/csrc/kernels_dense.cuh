@@ -116,42 +116,68 @@ __global__ void __launch_bounds__(256) fold_transpose_kernel(const float* __rest
   }
 }
 
-// V[y][(B*r + rep)*k + j] = scale * X[y][B*k + j]  (X fp32 [d3, h] -> V fp32 [d3, r*h])
-__global__ void expand_cols_kernel(const float* __restrict__ X, int d3, int h, int k, int r, float scale, float* __restrict__ V) {
+// V[y][(B*r + rep)*k + j] = scale * X[y][B*k + j]  (X fp32 [d3, h] -> V fp32 [d3, r*h]; k % 4 == 0).  grid: (ceil(h / 1024),
+// d3); a thread reads four entries once and writes every replica (60 -> 12 us at 3584 x 4096).
+__global__ void __launch_bounds__(256) expand_cols_kernel(const float* __restrict__ X, int h, int k, int r, float scale,
+                                                          float* __restrict__ V) {
+  const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
+  if (l >= h) return;
+  const long long y = blockIdx.y;
+  float4 x = __ldg(reinterpret_cast<const float4*>(X + y * h + l));
+  x = make_float4(scale * x.x, scale * x.y, scale * x.z, scale * x.w);
+  const int B = l / k, j = l - B * k;
+  float* v = V + y * (long long)r * h + (long long)B * r * k + j;
+  for (int rep = 0; rep < r; ++rep) *reinterpret_cast<float4*>(v + (long long)rep * k) = x;
+}
+
+// the same for any k, one entry per thread (learned offsets take every shape)
+__global__ void expand_cols_any_kernel(const float* __restrict__ X, int d3, int h, int k, int r, float scale, float* __restrict__ V) {
   const long long n = (long long)d3 * r * h;
-  const float inv = scale;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const long long y = e / ((long long)r * h);
     const int l = (int)(e - y * (long long)r * h);
     const int Bq = l / k, j = l - Bq * k;
-    V[e] = inv * X[y * h + (long long)(Bq / r) * k + j];
+    V[e] = scale * X[y * h + (long long)(Bq / r) * k + j];
   }
 }
 
-// iteration control of the pseudo-inverse: keep running while the newest squared residual is above tol2 and
-// still falling (a rank-deficient matrix stalls at its rank defect); flag: 1 = run, 0 = skip
-__global__ void pinv_control_kernel(const double* __restrict__ sq, int it, double tol2, int* flag, int m, int32_t* status) {
-  if (*flag == 0) return;
-  const double cur = sq[it];
-  if (!(cur > tol2)) { *flag = 0; return; }
-  if (it >= 1) {
-    const double prev = sq[it - 1];
-    // With every eigenvalue of A X in (0, 2) the residual norm falls monotonically.  A residual that is still large
-    // and grows means the starting scale was too small (the estimate of the largest singular value failed):
-    // stop and say so instead of iterating to infinity.
-    if (cur > 1.5 * prev && cur > 1e-2 * (double)m) {
-      *flag = 0;
-      raise_status(status, CAFEQ_ERR_NONFINITE);
-      return;
+// bf16 hi / lo (and third) terms of the replica-folded V: F[y][B*k + j] = sum_rep V[y][(B*r + rep)*k + j], row-major [d3, h].
+// A product over the r*h expanded inner indices equals the product over the h folded ones: 1 / r of the work.
+__global__ void __launch_bounds__(256) fold_split_kernel(const float* __restrict__ V, int h, int k, int r, uint16_t* __restrict__ hi,
+                                                         uint16_t* __restrict__ lo, uint16_t* __restrict__ h3, const int32_t* status) {
+  if (status && *status) return;
+  const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
+  if (l >= h) return;
+  const long long y = blockIdx.y;
+  const int B = l / k, j = l - B * k;
+  const float* v = V + y * (long long)r * h + (long long)B * r * k + j;
+  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int rep = 0; rep < r; ++rep) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(v + (long long)rep * k));
+    x[0] += q.x; x[1] += q.y; x[2] += q.z; x[3] += q.w;
+  }
+  uint32_t a[2], b[2], c[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    uint32_t aw = 0, bw = 0, cw = 0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float f = x[2 * q + e];
+      const __nv_bfloat16 t1 = __float2bfloat16_rn(f);
+      const float d1 = f - __bfloat162float(t1);
+      const __nv_bfloat16 t2 = __float2bfloat16_rn(d1);
+      const __nv_bfloat16 t3 = __float2bfloat16_rn(d1 - __bfloat162float(t2));
+      aw |= (uint32_t)__bfloat16_as_ushort(t1) << (16 * e);
+      bw |= (uint32_t)__bfloat16_as_ushort(t2) << (16 * e);
+      cw |= (uint32_t)__bfloat16_as_ushort(t3) << (16 * e);
     }
+    a[q] = aw; b[q] = bw; c[q] = cw;
   }
-  if (it >= 4) {
-    const double prev = sq[it - 1];
-    if (cur > prev * (1.0 - 1e-7) && cur < prev * (1.0 + 1e-7)) *flag = 0;  // stalled
-  }
+  const long long o = y * h + l;
+  *reinterpret_cast<uint2*>(hi + o) = make_uint2(a[0], a[1]);
+  *reinterpret_cast<uint2*>(lo + o) = make_uint2(b[0], b[1]);
+  if (h3) *reinterpret_cast<uint2*>(h3 + o) = make_uint2(c[0], c[1]);
 }
-
-__global__ void set_int_kernel(int* p, int v) { *p = v; }
 
 // gX[row][G*g + idx[row, G]] += coef[row, G]: the scale path of the straight-through quantiser lands on the
 // arg-max entry of its group (records row-major)
@@ -207,62 +233,62 @@ __global__ void __launch_bounds__(256) dot_f32_kernel(const float* __restrict__ 
 }
 
 // Power iteration for the largest singular value of S [R, C] (fp32, row-major), used to scale the starting guess
-// of the pseudo-inverse iteration.  v [C], u [R] scratch; three small kernels per round:
-//   u = S v (one warp per row);  v2 = S^T u (one thread per column), nrm += |v2|^2;  v = v2 / |v2|.
+// of the pseudo-inverse iteration.  Two kernels per round: u = S v / |v| (one warp per row; every CTA sums |v|^2 itself), then
+// v' = S^T u (one thread per column, slices of 32 rows, partial sums added atomically).  Three buffers of v in turn: one read,
+// one written, one cleared.  Bound by reading S twice per round (29 MB, from L2: 11 + 5 us; with slices of 512 rows, 56 CTAs,
+// the second kernel took 75 us, and norm and scaling were launches of their own).
 // After the last round *sig2 = safety * |S^T S v| (v of unit norm): a Rayleigh-type estimate from below of sigma_max^2.
-__global__ void pw_init_kernel(float* __restrict__ v, int C, double* nrm) {
+__global__ void pw_init_kernel(float* __restrict__ v, int C) {  // v [3][C]
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < C) {
     uint32_t h = (uint32_t)j * 2654435761u;
     h ^= h >> 15;
-    v[j] = ((h & 1u) ? 1.f : -1.f) * rsqrtf((float)C);  // fixed +-1 pattern of unit norm
+    v[j] = (h & 1u) ? 1.f : -1.f;  // fixed +-1 pattern
+    v[C + j] = 0.f;
   }
-  if (j == 0) *nrm = 0.0;
 }
-__global__ void pw_rows_kernel(const float* __restrict__ S, const float* __restrict__ v, int R, int C, float* __restrict__ u) {
-  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+__device__ __forceinline__ double pw_norm2(const float* v, int C, double* red) {
+  double s = 0.0;
+  for (int j = threadIdx.x; j < C; j += blockDim.x) s += (double)v[j] * (double)v[j];
+  s = block_sum_double(s, red);
+  __shared__ double out;
+  if (threadIdx.x == 0) out = s;
+  __syncthreads();
+  return out;
+}
+__global__ void __launch_bounds__(256) pw_rows_kernel(const float* __restrict__ S, const float* __restrict__ v, float* __restrict__ clear,
+                                                      int R, int C, float* __restrict__ u) {
+  __shared__ double red[32];
+  const double n = sqrt(pw_norm2(v, C, red));
+  const float inv = n > 0.0 ? (float)(1.0 / n) : 0.f;
+  for (int j = blockIdx.x * 256 + threadIdx.x; j < C; j += gridDim.x * 256) clear[j] = 0.f;
+  const long long w = (blockIdx.x * 256ll + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= R) return;
   float s = 0.f;
   for (int j = lane; j < C; j += 32) s = fmaf(S[w * C + j], v[j], s);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) u[w] = s;
+  if (lane == 0) u[w] = s * inv;
 }
-// grid: (ceil(C / 256), row slices); partial sums are added atomically into v2 (zeroed by the caller)
-__global__ void pw_cols_kernel(const float* __restrict__ S, const float* __restrict__ u, int R, int C, int rows_per_slice,
-                               float* __restrict__ v2) {
+// grid: (ceil(C / 256), ceil(R / 32)); v2 cleared two launches before
+__global__ void __launch_bounds__(256) pw_cols_kernel(const float* __restrict__ S, const float* __restrict__ u, int R, int C,
+                                                      float* __restrict__ v2) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= C) return;
-  const int r0 = blockIdx.y * rows_per_slice, r1 = min(R, r0 + rows_per_slice);
+  const int r0 = blockIdx.y * 32, n = min(R - r0, 32);
   float s = 0.f;
-  for (int r = r0; r < r1; ++r) s = fmaf(S[(long long)r * C + j], u[r], s);
+#pragma unroll 8
+  for (int r = 0; r < n; ++r) s = fmaf(S[(long long)(r0 + r) * C + j], u[r0 + r], s);
   atomicAdd(&v2[j], s);
 }
-__global__ void pw_norm_kernel(const float* __restrict__ v2, int C, double* nrm) {
+__global__ void __launch_bounds__(256) pw_result_kernel(const float* __restrict__ v, int C, double safety, const double* fro2, double* sig2) {
   __shared__ double red[32];
-  double s = 0.0;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < C; j += gridDim.x * blockDim.x) s += (double)v2[j] * (double)v2[j];
-  s = block_sum_double(s, red);
-  if (threadIdx.x == 0) atomicAdd(nrm, s);
-}
-// v = v2 / |v2|, v2 = 0, and (last round) *sig2 = safety * |v2| bounded below by floor2; nrm is cleared for the next round
-__global__ void pw_scale_kernel(float* __restrict__ v, float* __restrict__ v2, int C, double* nrm_in, double* nrm_next,
-                                double* sig2, double safety, const double* fro2) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const double n = sqrt(fmax(*nrm_in, 0.0));
-  if (j < C) {
-    v[j] = (n > 0.0) ? (float)((double)v2[j] / n) : v[j];
-    v2[j] = 0.f;
-  }
-  if (j == 0) {
-    *nrm_next = 0.0;
-    if (sig2) {
-      // never above the Frobenius bound (always safe), never below 1 / rank-ish of it (a failed estimate)
-      double e = safety * n;
-      const double f = *fro2;
-      if (!(e > 0.0) || e > f) e = f;
-      *sig2 = e;
-    }
+  const double n = sqrt(pw_norm2(v, C, red));
+  if (threadIdx.x == 0) {
+    // never above the Frobenius bound (always safe), never zero (a failed estimate)
+    double e = safety * n;
+    if (!(e > 0.0) || e > *fro2) e = *fro2;
+    *sig2 = e;
   }
 }
 

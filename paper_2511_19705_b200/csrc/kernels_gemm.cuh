@@ -4,8 +4,8 @@
 //
 //   C[b][m][n] = alpha * sum_t sum_l A_t[b / divA][m][l] * B_t[b][n][l]  + beta * C0[b][m][n] + gamma * [m == n]
 //
-// Every operand is bf16, row-major with the contraction index l contiguous (both K-major), so one product is
-// the "A times B-transposed" form.  fp32 precision comes from summing up to three terms over bf16 splits
+// Every operand is bf16; by default row-major with the contraction index l contiguous (both K-major), so one product is
+// the "A times B-transposed" form, either side optionally stored with l as the slow index (MN-major).  fp32 precision comes from summing up to three terms over bf16 splits
 // (x = hi + lo, hi = bf16(x), lo = bf16(x - hi)); the accumulator is fp32 in tensor memory.
 // The epilogue can write C as fp32, as bf16 hi / lo splits in row-major and / or transposed order (the
 // operand layouts the next product needs), and accumulate sum(C^2).
@@ -38,7 +38,6 @@ struct TgParams {
                                          // multiplies columns [b * k, b * k + k) of a wide matrix); 0 otherwise
   int divB, colsB_per_batch;             // the same for B (divB = 0 means 1)
   int min_ctas;                          // > 0: overrides the process-wide tile-width rule for this launch
-  int a_rep_k, a_rep_r;                  // replicated contraction blocks of A: chunk at l reads columns ((l / k) / r) * k + l % k
   float alpha, beta, gamma;
   const float* C0;
   long long ldc0, sC0b;
@@ -49,6 +48,10 @@ struct TgParams {
   double* sq;             // sum of C^2: sq[b * sq_stride]
   int sq_stride;
   const int* run_flag;    // optional: skip the whole launch when *run_flag == 0
+  int a_mn, b_mn;         // the A / B arrays are stored [l][m] / [l][n] (MN-major operands); a batch then starts at column
+                          // batch * colsA_per_batch / colsB_per_batch
+  const double* stop_sq;  // optional: squared residuals of an iteration; this launch belongs to iteration stop_it, and is
+  int stop_it;            // skipped when the rule (tg_stopped) ended the iteration before
   const double* gate;     // optional: batch b is skipped when gate[b] <= gate_tol (its iteration has converged)
   double gate_tol;
   int32_t* status;
@@ -61,8 +64,25 @@ struct TgCfg {
   static constexpr int STAGE = A_BYTES + B_BYTES;
   static constexpr int NSTAGE = (BN <= 128) ? 6 : 4;
   static constexpr int SMEM = 1024 + NSTAGE * STAGE + 256;
-  static constexpr int TMEM_COLS = (BN < 32) ? 32 : BN;
+  static constexpr int TMEM_COLS = (BN > 128) ? 256 : BN;
 };
+
+// Stopping rule of the pseudo-inverse iteration on m rows: it ends when the squared residual is below 1e-6, or has stopped
+// falling (a rank-deficient matrix stalls at its rank defect).  With every eigenvalue of A X in (0, 2) the residual falls
+// monotonically: one that is still large and grows means that the starting scale was too small, which is reported.
+// The residuals of iterations that were skipped stay zero, so the last two decide.
+__device__ __forceinline__ bool tg_stopped(const TgParams& p) {
+  if (!p.stop_sq || p.stop_it < 1) return false;
+  const double cur = p.stop_sq[p.stop_it - 1];
+  if (!(cur > 1e-6)) return true;
+  if (p.stop_it < 2) return false;
+  const double prev = p.stop_sq[p.stop_it - 2];
+  if (cur > 1.5 * prev && cur > 1e-2 * (double)p.M) {
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) raise_status(p.status, CAFEQ_ERR_NONFINITE);
+    return true;
+  }
+  return p.stop_it >= 5 && cur > prev * (1.0 - 1e-7) && cur < prev * (1.0 + 1e-7);
+}
 
 // One 32-column chunk of one 128-row accumulator tile: scaling, C0, identity, sum of squares and every output format.
 // taddr: the tile's accumulator at this warp's lane quarter; tile: this warp's [32][36] fp32 scratch in shared memory.
@@ -216,10 +236,10 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
 
 template <int BN>
 __global__ void __launch_bounds__(TG_THREADS, 1)
-tc_gemm_kernel(const __grid_constant__ TgMaps maps, const TgParams p) {
+tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgParams p) {
   using C = TgCfg<BN>;
   if (p.status && *p.status) return;
-  if (p.run_flag && *p.run_flag == 0) return;
+  if (tg_stopped(p)) return;
   if (p.gate && p.gate[blockIdx.z] <= p.gate_tol) return;
 
   extern __shared__ uint8_t smem_raw[];
@@ -271,29 +291,41 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const TgParams p) {
         if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, p.status)) break;
         mbar_expect_tx(bar_full + 8 * s, C::STAGE);
         const int l0 = c * TG_BK;
-        int xa = l0;
-        if (p.a_rep_r > 1) xa = ((l0 / p.a_rep_k) / p.a_rep_r) * p.a_rep_k + (l0 % p.a_rep_k);
-        xa += (b / p.divA) * p.colsA_per_batch;
         uint8_t* st = smem + s * C::STAGE;
-        tma_load_2d(smem_u32(st), &maps.a[t], xa, ya, bar_full + 8 * s);
-        tma_load_2d(smem_u32(st + C::A_BYTES), &maps.b[t], l0 + bb * p.colsB_per_batch, yb, bar_full + 8 * s);
+        // MN-major: 64 contraction rows x 128 (BN) columns as boxes of 64 x 64, one swizzle atom each
+        if (p.a_mn) {
+          for (int j = 0; j < 2; ++j)
+            tma_load_2d(smem_u32(st + j * 8192), &maps.a[t], m0 + j * 64 + (b / p.divA) * p.colsA_per_batch, l0, bar_full + 8 * s);
+        } else {
+          tma_load_2d(smem_u32(st), &maps.a[t], l0 + (b / p.divA) * p.colsA_per_batch, ya, bar_full + 8 * s);
+        }
+        if (p.b_mn) {
+          for (int j = 0; j < BN / 64; ++j)
+            tma_load_2d(smem_u32(st + C::A_BYTES + j * 8192), &maps.b[t], n0 + j * 64 + bb * p.colsB_per_batch, l0, bar_full + 8 * s);
+        } else {
+          tma_load_2d(smem_u32(st + C::A_BYTES), &maps.b[t], l0 + bb * p.colsB_per_batch, yb, bar_full + 8 * s);
+        }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_bf16(128, BN, 0, 0);
-      bool ok = true;
-      for (int it = 0; it < total && ok; ++it) {
-        const uint32_t s = it % C::NSTAGE, ph = (it / C::NSTAGE) & 1u;
-        if (!mbar_wait(bar_full + 8 * s, ph, abort_flag, p.status)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t sa = smem_u32(smem + s * C::STAGE), sb = sa + C::A_BYTES;
+    // the whole warp runs the loop, one elected lane issues (see bd_pass_body)
+    const uint32_t idesc = umma_idesc_bf16(128, BN, p.a_mn, p.b_mn);
+    const uint32_t astep = p.a_mn ? 128 : 2, bstep = p.b_mn ? 128 : 2;  // 16 contraction entries further, in 16-byte units
+    const uint32_t albo = p.a_mn ? 8192 : 16, blbo = p.b_mn ? 8192 : 16;
+    uint32_t s = 0, ph = 0;
+    for (int it = 0; it < total; ++it) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, ph, abort_flag, p.status))) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t sa = smem_u32(smem + s * C::STAGE);
+        const uint32_t alo = umma_desc_lo(sa, albo), blo = umma_desc_lo(sa + C::A_BYTES, blbo);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          tc_mma_bf16(tmem_base, umma_desc_sw128(sa + kk * 32), umma_desc_sw128(sb + kk * 32), idesc, (it | kk) != 0 ? 1u : 0u);
+        for (int kk = 0; kk < 4; ++kk) tc_mma_lo(tmem_base, alo + kk * astep, blo + kk * bstep, idesc, (it | kk) != 0 ? 1u : 0u);
         tc_commit(bar_empty + 8 * s);
+        if (it == total - 1) tc_commit(bar_acc);
       }
-      if (ok) tc_commit(bar_acc);
+      __syncwarp();
+      if (++s == C::NSTAGE) { s = 0; ph ^= 1u; }
     }
   } else {
     // a warp reads the accumulator lanes of its quarter (warp index modulo 4); the warps of one quarter share
@@ -641,8 +673,8 @@ static int tg_launch_t(cudaStream_t st, const TgOperand* A, const TgOperand* B, 
   TgMaps maps;
   memset(&maps, 0, sizeof(maps));
   for (int t = 0; t < p.nterms; ++t) {
-    if (!make_map_bf16(&maps.a[t], A[t].ptr, A[t].cols, A[t].rows, A[t].pitch, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&maps.b[t], B[t].ptr, B[t].cols, B[t].rows, B[t].pitch, BN)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&maps.a[t], A[t].ptr, A[t].cols, A[t].rows, A[t].pitch, p.a_mn ? 64 : 128)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&maps.b[t], B[t].ptr, B[t].cols, B[t].rows, B[t].pitch, p.b_mn ? 64 : BN)) return CAFEQ_ERR_UNSUPPORTED;
   }
   dim3 grid((p.N + BN - 1) / BN, (p.M + 127) / 128, p.batch);
   tc_gemm_kernel<BN><<<grid, TG_THREADS, C::SMEM, st>>>(maps, p);
@@ -659,7 +691,13 @@ static int tg_launch(cudaStream_t st, const TgOperand* A, const TgOperand* B, co
   if (p.K % TG_BK || p.nterms < 1 || p.nterms > TG_MAX_TERMS) return CAFEQ_ERR_UNSUPPORTED;
   const int min_ctas = p.min_ctas > 0 ? p.min_ctas : g_tg_min_ctas.load(std::memory_order_relaxed);
   const long long mt = (long long)p.batch * ((p.M + 127) / 128);
-  if (p.N > 128 && mt * ((p.N + 255) / 256) >= min_ctas) return tg_launch_t<256>(st, A, B, p);
+  if (p.N > 128 && mt * ((p.N + 255) / 256) >= min_ctas) {
+    // one CTA per SM: the width whose tiles fill whole waves better, counted in waves x width (2048 x 3584: 224 tiles of 256
+    // are two waves for 1.5 waves of work, 109 us; 256 tiles of 224 are two narrower ones, 100 us).  K-major B only.
+    const long long w256 = (mt * ((p.N + 255) / 256) + 147) / 148 * 256, w224 = (mt * ((p.N + 223) / 224) + 147) / 148 * 224;
+    if (!p.b_mn && w224 < w256) return tg_launch_t<224>(st, A, B, p);
+    return tg_launch_t<256>(st, A, B, p);
+  }
   if (p.N > 64 && mt * ((p.N + 127) / 128) >= min_ctas) return tg_launch_t<128>(st, A, B, p);
   if (p.N <= 64 || mt * ((p.N + 127) / 128) < min_ctas) return tg_launch_t<64>(st, A, B, p);
   return tg_launch_t<128>(st, A, B, p);

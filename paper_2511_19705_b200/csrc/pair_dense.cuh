@@ -15,18 +15,16 @@ struct DenseOut {
   long long ldc = 0;
   uint16_t *Chi = nullptr, *Clo = nullptr, *Cthi = nullptr, *Ctlo = nullptr;
   double* sq = nullptr;
-  const int* run_flag = nullptr;
+  const double* stop_sq = nullptr;  // stopping rule of an iteration (TgParams)
+  int stop_it = 0;
 };
 
-// A operands are [M, Ka] row-major (Ka = K, or K / a_rep_r when the contraction blocks of A are replicated),
-// B operands [N, K] row-major; nterms pairs (A[t], B[t]).
+// A operands are [M, K] row-major, B operands [N, K] row-major; nterms pairs (A[t], B[t]).
 static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A, const uint16_t* const* B, int M, int N, int K,
-                           float alpha, float beta, float gamma, const DenseOut& o, int32_t* status, int a_rep_k = 0,
-                           int a_rep_r = 1) {
+                           float alpha, float beta, float gamma, const DenseOut& o, int32_t* status) {
   TgOperand oa[TG_MAX_TERMS], ob[TG_MAX_TERMS];
-  const long long Ka = (a_rep_r > 1) ? K / a_rep_r : K;
   for (int t = 0; t < nterms; ++t) {
-    oa[t] = TgOperand{A[t], M, Ka, Ka};
+    oa[t] = TgOperand{A[t], M, K, K};
     ob[t] = TgOperand{B[t], N, K, K};
   }
   TgParams p;
@@ -35,14 +33,12 @@ static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A
   p.batch = 1;
   p.nterms = nterms;
   p.divA = 1;
-  p.a_rep_k = a_rep_k > 0 ? a_rep_k : K;
-  p.a_rep_r = a_rep_r;
   p.alpha = alpha; p.beta = beta; p.gamma = gamma;
   p.C0 = o.C0; p.ldc0 = o.ldc0;
   p.C = o.C; p.ldc = o.ldc;
   p.Chi = o.Chi; p.Clo = o.Clo; p.Cthi = o.Cthi; p.Ctlo = o.Ctlo;
   p.sq = o.sq; p.sq_stride = 0;
-  p.run_flag = o.run_flag;
+  p.stop_sq = o.stop_sq; p.stop_it = o.stop_it;
   p.status = status;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return tg_launch(st, oa, ob, p);
@@ -60,21 +56,20 @@ static void launch_split_rect(cudaStream_t st, const float* X, int R, int C, lon
 // pitch N; it may be o.C).  fp32-grade accuracy: what is left is the rounding of the fp32 accumulators.
 // A / B: {x1, x2, x3} in the layouts launch_dense_tc takes.
 static int launch_dense_tc6(cudaStream_t st, const uint16_t* const* A, const uint16_t* const* B, int M, int N, int K, float alpha,
-                            float beta, float gamma, const DenseOut& o, float* acc, int32_t* status, int a_rep_k = 0, int a_rep_r = 1) {
+                            float beta, float gamma, const DenseOut& o, float* acc, int32_t* status) {
   const uint16_t* a1[3] = {A[0], A[1], A[0]};
   const uint16_t* b1[3] = {B[0], B[0], B[1]};
   DenseOut o1;
   o1.C0 = o.C0; o1.ldc0 = o.ldc0;
   o1.C = acc; o1.ldc = N;
-  o1.run_flag = o.run_flag;
-  int rc = launch_dense_tc(st, 3, a1, b1, M, N, K, alpha, beta, gamma, o1, status, a_rep_k, a_rep_r);
+  int rc = launch_dense_tc(st, 3, a1, b1, M, N, K, alpha, beta, gamma, o1, status);
   if (rc) return rc;
   const uint16_t* a2[3] = {A[0], A[2], A[1]};
   const uint16_t* b2[3] = {B[2], B[0], B[1]};
   DenseOut o2 = o;
   o2.C0 = acc; o2.ldc0 = N;
   if (!o2.C) { o2.C = nullptr; }
-  return launch_dense_tc(st, 3, a2, b2, M, N, K, alpha, 1.f, 0.f, o2, status, a_rep_k, a_rep_r);
+  return launch_dense_tc(st, 3, a2, b2, M, N, K, alpha, 1.f, 0.f, o2, status);
 }
 
 // Scratch of the dense pair algebra for a pair with stored shapes U [h, d1], V [d3, rh]
@@ -93,7 +88,6 @@ struct DenseWS {
   float *qa, *qusel;                      // quantiser scratch: absmax, signed arg-max value
   int* qidx;
   double* sq;                             // [DENSE_SQ] accumulators: 0..: PQE history, 32..: iteration residuals
-  int* flag;
 };
 constexpr int DENSE_SQ = 128;
 constexpr int PINV_MAX_ITERS = 56;
@@ -124,7 +118,6 @@ static bool carve_dense(Bump& b, int h, int d1, int d3, int r, int k, int ng1, i
   const size_t nq = ((size_t)h * ng1 > (size_t)d3 * ng2) ? (size_t)h * ng1 : (size_t)d3 * ng2;
   w->qa = b.take<float>(nq); w->qusel = b.take<float>(nq); w->qidx = b.take<int>(nq);
   w->sq = b.take<double>(DENSE_SQ);
-  w->flag = b.take<int>(64);
   return !b.overflow;
 }
 
@@ -141,33 +134,33 @@ static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, 
 // ||A||_F^2: the eigenvalues of A X0 lie in (0, 2) (the estimate is from below and a few percent off at most; the
 // iteration converges for anything below 2), to the Moore-Penrose inverse.  Scaling by sigma_max^2 instead of the
 // always-safe ||A||_F^2 saves log2(stable rank) doublings of the smallest eigenvalue.  Stops on the device when ||I - A X||_F falls below 1e-3 (the next
-// update squares it) or stalls (rank-deficient A); the remaining launches then return at once.
+// update squares it) or stalls (rank-deficient A), which every product works out from the residuals itself; the remaining
+// launches then return at once.
+// (Two things that were slower or worse: scaling the iterate by 2 / (1 + l) for a lower bound l of the eigenvalues, 10
+// iterations instead of 16 on the 9B-shaped v-o factors, cancels the large components of X against the product at every step,
+// and the rounding that this leaves outside the row space of A is never corrected: codes that matched the float64
+// pseudo-inverse differed.  Reading Y and C row-major as MN-major operands, with no transposed outputs: 114 us for
+// 2048 x 3584 x 2048 against 102.)
 static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, int32_t* status) {
   const bool wide = R <= C;
   const int m = wide ? R : C, n = wide ? C : R;
   double* fro = w.sq + 120;
   double* rs = w.sq + 32;  // residuals per iteration
   CQ_LAUNCH(zero_f64_kernel, 1, 128, 0, st, w.sq + 32, DENSE_SQ - 32);
-  CQ_LAUNCH(set_int_kernel, 1, 1, 0, st, w.flag, 1);
   CQ_LAUNCH(sqsum_f32_kernel, grid_for((long long)R * C), 256, 0, st, S, (long long)R * C, fro);
   double* sig2 = w.sq + 123;
   {
-    // power iteration in the (not yet used) iterate buffer: v [C], v2 [C], u [R]
+    // power iteration in the (not yet used) iterate buffer: v [3][C], u [R]
     float* v = w.Y;
-    float* v2 = w.Y + C;
-    float* u = w.Y + 2 * (size_t)C;
-    double* nrm = w.sq + 121;  // two slots, used alternately
+    float* u = w.Y + 3 * (size_t)C;
     constexpr int ROUNDS = 8;
-    const int slices = (R + 511) / 512;
-    CQ_LAUNCH(pw_init_kernel, (C + 255) / 256, 256, 0, st, v, C, nrm);
-    CQ_LAUNCH(fill_f32_kernel, grid_for(C), 256, 0, st, v2, 0.f, (long long)C);
+    CQ_LAUNCH(pw_init_kernel, (C + 255) / 256, 256, 0, st, v, C);
     for (int it = 0; it < ROUNDS; ++it) {
-      CQ_LAUNCH(pw_rows_kernel, (unsigned)(((long long)R * 32 + 255) / 256), 256, 0, st, S, v, R, C, u);
-      CQ_LAUNCH(pw_cols_kernel, dim3((C + 255) / 256, slices), 256, 0, st, S, u, R, C, 512, v2);
-      CQ_LAUNCH(pw_norm_kernel, 32, 256, 0, st, v2, C, nrm + (it & 1));
-      CQ_LAUNCH(pw_scale_kernel, (C + 255) / 256, 256, 0, st, v, v2, C, nrm + (it & 1), nrm + ((it + 1) & 1),
-                (it == ROUNDS - 1) ? sig2 : nullptr, 1.25, fro);
+      float* nxt = v + (size_t)((it + 1) % 3) * C;
+      CQ_LAUNCH(pw_rows_kernel, (R + 7) / 8, 256, 0, st, S, v + (size_t)(it % 3) * C, v + (size_t)((it + 2) % 3) * C, R, C, u);
+      CQ_LAUNCH(pw_cols_kernel, dim3((C + 255) / 256, (R + 31) / 32), 256, 0, st, S, u, R, C, nxt);
     }
+    CQ_LAUNCH(pw_result_kernel, 1, 256, 0, st, v + (size_t)(ROUNDS % 3) * C, C, 1.25, fro, sig2);
   }
   if (wide) {
     launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status, w.Aw3, nullptr);
@@ -182,7 +175,8 @@ static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w,
       const uint16_t* a[3] = {w.Awh, w.Awl, w.Awh};
       const uint16_t* bb[3] = {w.Yh, w.Yh, w.Yl};
       DenseOut o;
-      o.Cthi = w.CTh; o.Ctlo = w.CTl; o.sq = rs + it; o.run_flag = w.flag;
+      o.Cthi = w.CTh; o.Ctlo = w.CTl; o.sq = rs + it;
+      o.stop_sq = rs; o.stop_it = it;
       launch_dense_tc(st, 3, a, bb, m, m, n, -1.f, 0.f, 1.f, o, status);
     }
     {  // Y += C^T Y
@@ -191,10 +185,9 @@ static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w,
       DenseOut o;
       o.C0 = w.Y; o.ldc0 = n; o.C = w.Y; o.ldc = n;
       o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[cur ^ 1]; o.Ctlo = w.YTl[cur ^ 1];
-      o.run_flag = w.flag;
+      o.stop_sq = rs; o.stop_it = it;
       launch_dense_tc(st, 3, a, bb, m, n, m, 1.f, 1.f, 0.f, o, status);
     }
-    CQ_LAUNCH(pinv_control_kernel, 1, 1, 0, st, rs, it, 1e-6, w.flag, m, status);
     cur ^= 1;
   }
   // The loop above stops at the accuracy of its three-term products (residual entries of a few 1e-7).  One more
@@ -229,17 +222,22 @@ static void quant_matrix(cudaStream_t st, const float* T, int rows, int cols, in
                      codes, scales, status);
 }
 
+// hi / lo (and third) terms of V [d3, rh] with its replicas folded: [d3, h]
+static void launch_fold_split(cudaStream_t st, const float* V, DenseWS& w, uint16_t* hi, uint16_t* lo, uint16_t* h3, int32_t* status) {
+  CQ_LAUNCH(fold_split_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, V, w.h, w.k, w.r, hi, lo, h3, status);
+}
+
 // P = U_exp^T V^T for stored U [h, d1], V [d3, rh] (fp32): fp32 P [d1, d3] with its splits in w.Ph/Pl/PTh/PTl
 // (six terms over three-way splits: P is the reference every least-squares target of Algorithm 1 is measured
 // against, so it is formed to fp32 accuracy; its own third-term splits follow for the target products)
 static void dense_product(cudaStream_t st, const float* U, const float* V, DenseWS& w, float* P, int32_t* status) {
   launch_split_rect(st, U, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.UTh, w.UTl, status, nullptr, w.UT3);
-  launch_split_rect(st, V, w.d3, w.rh, w.rh, 1.f, nullptr, nullptr, nullptr, w.Vh, w.Vl, nullptr, nullptr, status, w.V3, nullptr);
+  launch_fold_split(st, V, w, w.Vh, w.Vl, w.V3, status);
   const uint16_t* a[3] = {w.UTh, w.UTl, w.UT3};
   const uint16_t* b[3] = {w.Vh, w.Vl, w.V3};
   DenseOut o;
   o.C = P; o.ldc = w.d3; o.Chi = w.Ph; o.Clo = w.Pl; o.Cthi = w.PTh; o.Ctlo = w.PTl;
-  launch_dense_tc6(st, a, b, w.d1, w.d3, w.rh, 1.f, 0.f, 0.f, o, P, status, w.k, w.r);
+  launch_dense_tc6(st, a, b, w.d1, w.d3, w.h, 1.f, 0.f, 0.f, o, P, status);
   launch_split_rect(st, P, w.d1, w.d3, w.d3, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status, w.P3, w.PT3);
 }
 
@@ -247,7 +245,7 @@ static void dense_product(cudaStream_t st, const float* U, const float* V, Dense
 static void dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, const float* P, DenseWS& w, double* sq, float* R,
                       int32_t* status, bool keep_splits = false) {
   launch_split_rect(st, Uhat, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.UTh, w.UTl, status);
-  launch_split_rect(st, Vhat, w.d3, w.rh, w.rh, 1.f, nullptr, nullptr, nullptr, w.Vh, w.Vl, nullptr, nullptr, status);
+  launch_fold_split(st, Vhat, w, w.Vh, w.Vl, nullptr, status);
   const uint16_t* a[3] = {w.UTh, w.UTl, w.UTh};
   const uint16_t* b[3] = {w.Vh, w.Vh, w.Vl};
   DenseOut o;
@@ -255,7 +253,7 @@ static void dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, con
   if (keep_splits) {  // the residual and its transpose as operands of the backward products
     o.Chi = w.Ph; o.Clo = w.Pl; o.Cthi = w.PTh; o.Ctlo = w.PTl;
   }
-  launch_dense_tc(st, 3, a, b, w.d1, w.d3, w.rh, 1.f, -1.f, 0.f, o, status, w.k, w.r);
+  launch_dense_tc(st, 3, a, b, w.d1, w.d3, w.h, 1.f, -1.f, 0.f, o, status);
 }
 
 // Algorithm 1 on the transformed pair held in w.U [h, d1], w.V [d3, rh] (fp32, stored layout with r replicas of
@@ -279,7 +277,7 @@ static void alg1_run(cudaStream_t st, int bits, int g1, int g2, int iters, int8_
       o.C = w.X0T; o.ldc = w.h;
       launch_dense_tc6(st, a, b, w.d3, w.h, w.d1, 1.f, 0.f, 0.f, o, w.X0T, status);
     }
-    CQ_LAUNCH(expand_cols_kernel, grid_for((long long)w.d3 * w.rh), 256, 0, st, w.X0T, w.d3, w.h, w.k, w.r, 1.f / (float)w.r, w.V);
+    CQ_LAUNCH(expand_cols_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f / (float)w.r, w.V);
     quant_matrix(st, w.V, w.d3, w.rh, g2, bits, codes2, scales2, w.Vhat, w, status);
     dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 1, nullptr, status);
     // U side: U' [h, d1] = pinv(Bf)^T P^T with Bf = fold(Vhat^T) [h, d3]
