@@ -7,7 +7,9 @@ no CPU fallback: if the library has not been built, every call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+from types import SimpleNamespace
 
 import torch
 
@@ -60,6 +62,7 @@ class CafeqError(RuntimeError):
 
 
 _lib = None
+_fast = None
 
 
 def lib() -> ctypes.CDLL:
@@ -77,6 +80,37 @@ def lib() -> ctypes.CDLL:
         L.cafeq_debug_launch_count.restype = ctypes.c_longlong
         _lib = L
     return _lib
+
+
+def _hot():
+    """Typed prototypes of the calls that last as long on the host as on the device: plain integers as arguments, converted in
+    C (a decoding step spent 9 us wrapping each argument in a ctypes object and making the descriptor anew)."""
+    global _fast
+    if _fast is None:
+        p, i, z, ll = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_longlong
+        L = lib()
+        _fast = SimpleNamespace(
+            rtn=ctypes.CFUNCTYPE(i, p, p, p, p, p, p, z, p)(("cafeq_rtn", L)),
+            pack=ctypes.CFUNCTYPE(i, p, p, p, p)(("cafeq_pack", L)),
+            dequant=ctypes.CFUNCTYPE(i, p, p, p, p, ll, p)(("cafeq_dequant", L)),
+            apply=ctypes.CFUNCTYPE(i, p, p, p, p, p, p, z, p)(("cafeq_apply_transform", L)))
+    return _fast
+
+
+@functools.lru_cache(maxsize=256)
+def _plan(kind, d_out, d_in, bits, group, tblock, taxis, trole, replicas, ld):
+    """(address of a descriptor, scratch bytes, the descriptor) of one shape; read only, so threads share it."""
+    d = make_desc(d_out, d_in, bits, group, tblock, taxis, trole, replicas, ld)
+    n = ctypes.c_size_t(0)
+    if kind == "apply":
+        _check(lib().cafeq_apply_workspace_size(ctypes.byref(d), ctypes.byref(n)), "cafeq_apply_workspace_size")
+    elif kind == "rtn":
+        n.value = rtn_workspace_size(d, tblock > 0)
+    return ctypes.addressof(d), max(int(n.value), 256), d
+
+
+def _raw_stream() -> int:
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def status_string(code: int) -> str:
@@ -166,7 +200,7 @@ _ws_cache: dict = {}
 
 def workspace(nbytes: int, device="cuda") -> torch.Tensor:
     """A cached uint8 scratch tensor of at least nbytes (torch allocations are 512-byte aligned)."""
-    key = str(device)
+    key = device if isinstance(device, torch.device) else torch.device(device)
     t = _ws_cache.get(key)
     if t is None or t.numel() < nbytes:
         _ws_cache[key] = t = torch.empty(int(nbytes), dtype=torch.uint8, device=device)
@@ -192,13 +226,14 @@ def cafeq_rtn(W, T=None, *, bits, group, tblock=0, taxis=AXIS_IN, trole=APPLY_T,
     """Round-to-nearest codes (int8 [d_out,d_in]) and scales (fp32 [d_out, d_in/group]) of T o W."""
     W = _bits_tensor(W)
     d_out, d_in = W.shape
-    d = make_desc(d_out, d_in, bits, group, tblock if T is not None else 0, taxis, trole, replicas, W.stride(0))
+    desc, nbytes, _ = _plan("rtn", d_out, d_in, bits, group, tblock if T is not None else 0, taxis, trole, replicas, W.stride(0))
     g = group or d_in
-    codes = torch.empty((d_out, d_in), dtype=torch.int8, device=W.device)
-    scales = torch.empty((d_out, d_in // g), dtype=torch.float32, device=W.device)
-    ws = workspace(max(rtn_workspace_size(d, T is not None), 256), W.device)
-    rc = lib().cafeq_rtn(ctypes.byref(d), _p(W), _p(_f32(T, "T")), _p(codes), _p(scales), _p(ws),
-                         ctypes.c_size_t(ws.numel()), _stream())
+    dev = W.device
+    codes = torch.empty((d_out, d_in), dtype=torch.int8, device=dev)
+    scales = torch.empty((d_out, d_in // g), dtype=torch.float32, device=dev)
+    ws = workspace(nbytes, dev)
+    rc = _hot().rtn(desc, W.data_ptr(), None if T is None else _f32(T, "T").data_ptr(), codes.data_ptr(), scales.data_ptr(), ws.data_ptr(),
+                    ws.numel(), _raw_stream())
     _check(rc, "cafeq_rtn")
     return codes, scales
 
@@ -344,9 +379,9 @@ def cafeq_pack(codes, *, bits):
     if codes.dtype != torch.int8 or not codes.is_cuda or not codes.is_contiguous():
         raise ValueError("codes must be a contiguous CUDA int8 tensor")
     d_out, d_in = codes.shape
-    d = make_desc(d_out, d_in, bits, 0)
+    desc = _plan("", d_out, d_in, bits, 0, 0, AXIS_IN, APPLY_T, 1, d_in)[0]
     packed = torch.empty((d_out, d_in * bits // 8), dtype=torch.uint8, device=codes.device)
-    rc = lib().cafeq_pack(ctypes.byref(d), _p(codes), _p(packed), _stream())
+    rc = _hot().pack(desc, codes.data_ptr(), packed.data_ptr(), _raw_stream())
     _check(rc, "cafeq_pack")
     return packed
 
@@ -358,12 +393,12 @@ def cafeq_apply_transform(X, T, *, taxis=AXIS_IN, trole=APPLY_T, status=None):
         raise ValueError("X must be a CUDA bf16 matrix with unit column stride")
     d_out, d_in = X.shape
     k = T.shape[-1]
-    d = make_desc(d_out, d_in, 4, 128 if d_in % 128 == 0 else d_in, k, taxis, trole, 1, X.stride(0))
-    n = ctypes.c_size_t(0)
-    _check(lib().cafeq_apply_workspace_size(ctypes.byref(d), ctypes.byref(n)), "cafeq_apply_workspace_size")
-    ws = torch.empty(max(int(n.value), 256), dtype=torch.uint8, device=X.device)
-    Y = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=X.device)
-    rc = lib().cafeq_apply_transform(ctypes.byref(d), _p(X), _p(T), _p(Y), _p(status), _p(ws), ctypes.c_size_t(ws.numel()), _stream())
+    desc, nbytes, _ = _plan("apply", d_out, d_in, 4, 128 if d_in % 128 == 0 else d_in, k, taxis, trole, 1, X.stride(0))
+    dev = X.device
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+    Y = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=dev)
+    rc = _hot().apply(desc, X.data_ptr(), T.data_ptr(), Y.data_ptr(), None if status is None else status.data_ptr(), ws.data_ptr(), nbytes,
+                      _raw_stream())
     _check(rc, "cafeq_apply_transform")
     return Y
 
@@ -371,9 +406,9 @@ def cafeq_apply_transform(X, T, *, taxis=AXIS_IN, trole=APPLY_T, status=None):
 def cafeq_dequant(packed, scales, *, bits, group, d_in):
     """bf16 [d_out, d_in] = scales * codes from the bit stream of cafeq_pack."""
     d_out = packed.shape[0]
-    d = make_desc(d_out, d_in, bits, group)
+    desc = _plan("", d_out, d_in, bits, group, 0, AXIS_IN, APPLY_T, 1, d_in)[0]
     out = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=packed.device)
-    rc = lib().cafeq_dequant(ctypes.byref(d), _p(packed), _p(scales), _p(out), ctypes.c_longlong(d_in), _stream())
+    rc = _hot().dequant(desc, packed.data_ptr(), scales.data_ptr(), out.data_ptr(), d_in, _raw_stream())
     _check(rc, "cafeq_dequant")
     return out
 

@@ -238,6 +238,11 @@ constexpr int NS_WARM_ITERS = 4;  // upper bound: converged blocks skip the late
 constexpr int NS_WARM_ROUNDS = 6, NS_COLD_ROUNDS = 10;
 constexpr double NS_GATE2 = 1e-4, NS_COLD_GATE2 = 1e-6;
 
+static void launch_operator_bf16(cudaStream_t st, const float* T, uint16_t* out, int k, int nb, int transpose, int32_t* status,
+                                 int paired = 0) {
+  CQ_LAUNCH(operator_to_bf16_kernel, dim3(k / 32, k / 32, nb), 256, 0, st, T, out, k, transpose, paired, status);
+}
+
 static bool kk_fast(int k) { return k == 64 || k == 128 || k == 256; }
 
 static void carve_kk(Bump& b, int nbT, int k, KkWS* w) {
@@ -324,7 +329,7 @@ static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k,
   int ti = kt_begin(3, st);
   if (!prepped) {  // otherwise step_prep_kernel has cleared rn / flag and written Ab
     CQ_LAUNCH(zero_ns_kernel, (NS_MAX_ITERS * nb + 127) / 128, 128, 0, st, w.rn, NS_MAX_ITERS * nb, w.flag);
-    CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Mc, w.Ab, k, kk, 0, status);
+    launch_operator_bf16(st, Mc, w.Ab, k, nb, 0, status);
   }
   // Block sizes of the fused kernel: every round of a block runs in one launch, on row-major splits only.
   w.mn = g_tb_enable.load(std::memory_order_relaxed) && tb_supported(k, 2);
@@ -618,7 +623,8 @@ struct MatWS {
 // lean: the matrix goes through the fused tensor-core pass and nothing but the per-group records leaves it (Eq. 4 /
 // LogSumExp steps without the quantised loss): no matrix-sized scratch at all.
 static void carve_matrix(Bump& b, const Geo& G, MatWS* w, bool need_E, bool lean = false) {
-  w->Tb = b.take<uint16_t>((size_t)(G.nbT > 0 ? G.nbT : 1) * (G.k > 0 ? G.k : 1) * (G.k > 0 ? G.k : 1));
+  // (blocks of 32 may be widened to 64)
+  w->Tb = b.take<uint16_t>((size_t)(G.nbT > 0 ? G.nbT : 1) * (G.k > 0 ? G.k : 1) * (G.k > 0 ? G.k : 1) * (G.k == 32 ? 2 : 1) + (G.k == 32 ? 4096 : 0));
   w->Dbf = lean ? nullptr : b.take<uint16_t>(G.n);
   w->U = lean ? nullptr : b.take<float>(G.n);
   w->D = lean ? nullptr : b.take<float>(G.n);
@@ -636,27 +642,31 @@ static void carve_matrix(Bump& b, const Geo& G, MatWS* w, bool need_E, bool lean
 static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo& G, const float* Top, int transposed,
                        uint16_t* Tb, BdParams p, int32_t* status, const uint16_t* Tb_ready = nullptr) {
   const int form = (G.axis == CAFEQ_AXIS_IN) ? BD_IN : BD_OUT;
-  if (!bd_supported(form, G.d_out, G.d_in, ldx, G.k, G.g, X)) return false;
-  const long long kk = (long long)G.nbT * G.k * G.k;
+  // blocks of 32 go through as pairs on the diagonal of blocks of 64 (exact: the other products are with zeros)
+  const int two = (form == BD_IN && G.k == 32 && G.r == 1) ? 1 : 0;
+  const int k = two ? 64 : G.k, nbT = two ? G.nbT / 2 : G.nbT;
+  if (!bd_supported(form, G.d_out, G.d_in, ldx, k, G.g, X)) return false;
   if (Tb_ready && !transposed) Tb = const_cast<uint16_t*>(Tb_ready);  // bf16 operator already in applied orientation
-  else CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Top, Tb, G.k, kk, transposed, status);
+  else launch_operator_bf16(st, Top, Tb, G.k, G.nbT, transposed, status, two);
   p.d_out = G.d_out;
   p.d_in = G.d_in;
   p.r = G.r;
   p.status = status;
   int ti = kt_begin(5, st);
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  int rc = bd_launch(st, form, G.k, G.g, X, ldx, Tb, G.nbT, p);
+  int rc = bd_launch(st, form, k, G.g, X, ldx, Tb, nbT, p);
   kt_end(ti, st);
   return rc == CAFEQ_OK;
 }
+
+static bool tc_apply_ok(int k) { return k == 32 || kk_fast(k); }
 
 // U = T o W in fp32 as one-term batched products on the tensor cores (bf16 x bf16 products are exact, fp32
 // accumulation: the same arithmetic as the fused pass).  Tb: bf16 operator blocks in applied orientation
 // [nbT k, k].  Output axis: the contraction runs down the rows of W, so its transpose goes through WT first.
 static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_t* Tb, float* U, uint16_t* WT, int32_t* status) {
   const int k = G.k;
-  if (!kk_fast(k) || ((uintptr_t)W & 15) || (G.ld % 8) || (G.d_in % 4)) return false;
+  if (!tc_apply_ok(k) || ((uintptr_t)W & 15) || (G.ld % 8) || (G.d_in % 4)) return false;
   TgOperand oa[1], ob[1];
   TgParams p;
   memset(&p, 0, sizeof(p));
@@ -688,10 +698,11 @@ static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_
 
 // U = T o W, group absmax / arg-max, and (optionally) the quantiser outputs.  Returns true when the fused
 // tensor-core pass ran (then the residual is in w.Dbf as bf16 instead of w.D as fp32, and U is not stored).
+// T_rounded: scratch for the bf16 rounding of Tc where Tc is not rounded yet (the tensor-core paths round it themselves).
 static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits, const float* Tc, int transposed,
                           const MatWS& w, const void* offsets, int off_kind, bool want_delta, float* Uhat, int8_t* codes,
                           float* scales, int32_t* status, bool allow_fused, const BdParams* surr = nullptr,
-                          const uint16_t* Tb_ready = nullptr, uint16_t* WT_scratch = nullptr) {
+                          const uint16_t* Tb_ready = nullptr, uint16_t* WT_scratch = nullptr, float* T_rounded = nullptr) {
   if (Tc && allow_fused && off_kind == CAFEQ_OFFSETS_NONE && !Uhat) {
     BdParams p;
     memset(&p, 0, sizeof(p));
@@ -706,13 +717,17 @@ static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits
   bool applied = false;
   if (Tc && allow_fused) {  // (allow_fused is off when the caller asked for the shape-agnostic kernels)
     const uint16_t* Tb = (Tb_ready && !transposed) ? Tb_ready : w.Tb;
-    const long long kk = (long long)G.nbT * G.k * G.k;
-    if (Tb == w.Tb && kk_fast(G.k)) CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Tc, w.Tb, G.k, kk, transposed, status);
+    if (Tb == w.Tb && tc_apply_ok(G.k)) launch_operator_bf16(st, Tc, w.Tb, G.k, G.nbT, transposed, status);
     applied = apply_tc(st, W, G, Tb, w.U, WT_scratch, status);
   }
   if (applied) {
-  } else if (Tc) launch_apply(st, W, 1, G.ld, G, Tc, transposed, w.U, G.d_in, GEMM_STORE, nullptr, status);
-  else CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G.n), 256, 0, st, (const uint16_t*)W, G.ld, G.d_out, G.d_in, w.U);
+  } else if (Tc) {
+    if (T_rounded) {
+      const long long kk = (long long)G.nbT * G.k * G.k;
+      CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, Tc, T_rounded, kk, nullptr);
+    }
+    launch_apply(st, W, 1, G.ld, G, T_rounded ? T_rounded : Tc, transposed, w.U, G.d_in, GEMM_STORE, nullptr, status);
+  } else CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G.n), 256, 0, st, (const uint16_t*)W, G.ld, G.d_out, G.d_in, w.U);
   launch_group_quant(st, w.U, G.d_in, G.d_out, G.ng, G.g, qmax_of(bits), offsets, off_kind, w.a, w.usel, w.idx, want_delta ? w.D : nullptr,
                      Uhat, codes, scales, status);
   return false;
@@ -849,9 +864,8 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
   float* Tc = nullptr;
   rtn_scratch(G, has_T, W, codes, &b, &w, &Tc);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
-  if (has_T) CQ_LAUNCH(round_bf16_kernel, grid_for((long long)G.nbT * G.k * G.k), 256, 0, st, T, Tc, (long long)G.nbT * G.k * G.k, nullptr);
-  forward_quant(st, W, G, d->bits, Tc, d->trole == CAFEQ_APPLY_TT, w, nullptr, CAFEQ_OFFSETS_NONE, false, nullptr, codes,
-                scales, nullptr, true);
+  forward_quant(st, W, G, d->bits, has_T ? T : nullptr, d->trole == CAFEQ_APPLY_TT, w, nullptr, CAFEQ_OFFSETS_NONE, false, nullptr, codes,
+                scales, nullptr, true, nullptr, nullptr, nullptr, Tc);
   return last_launch();
 }
 
@@ -860,7 +874,7 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
 // ------------------------------------------------------------------------------------------------
 static size_t apply_scratch(const Geo& G, bool fused) {
   const size_t kk = (size_t)G.nbT * G.k * G.k;
-  return 1024 + kk * 6 + (fused ? 0 : (size_t)G.n * 4 + 256);
+  return 1024 + kk * 8 + (fused ? 0 : (size_t)G.n * 4 + 256);
 }
 static Geo apply_geo(Geo G) {
   // the store epilogue ignores the quantisation groups: any group width the pass is built for will do
@@ -876,7 +890,8 @@ extern "C" int cafeq_apply_workspace_size(const cafeq_matrix_desc* d, size_t* by
   const Geo Ga = apply_geo(G);
   // (X itself is not known here: 16-byte aligned rows are assumed; a call whose X does not qualify returns
   // CAFEQ_ERR_WORKSPACE)
-  const bool fused = bd_supported(G.axis == CAFEQ_AXIS_IN ? BD_IN : BD_OUT, Ga.d_out, Ga.d_in, Ga.ld, Ga.k, Ga.g, nullptr);
+  const bool two = G.axis == CAFEQ_AXIS_IN && G.k == 32 && G.r == 1;  // (see fused_pass)
+  const bool fused = bd_supported(G.axis == CAFEQ_AXIS_IN ? BD_IN : BD_OUT, Ga.d_out, Ga.d_in, Ga.ld, two ? 64 : Ga.k, Ga.g, nullptr);
   *bytes = apply_scratch(G, fused);
   return CAFEQ_OK;
 }
@@ -892,11 +907,16 @@ extern "C" int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, 
   const long long kk = (long long)G.nbT * G.k * G.k;
   Bump b(ws, ws_bytes);
   float* Tc = b.take<float>(kk);
-  uint16_t* Tb = b.take<uint16_t>(kk);
+  uint16_t* Tb = b.take<uint16_t>(G.k == 32 ? 2 * kk : kk);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   // the deployed operator is the bf16 rounding of the given one (what the tensor cores apply; the pass converts it
   // itself, the shape-agnostic kernels take the rounded fp32 copy)
   const int transposed = d->trole == CAFEQ_APPLY_TT;
+  if (G.axis == CAFEQ_AXIS_IN && G.d_out <= AS_MAX_ROWS && G.k % 32 == 0 && G.k <= 256 && ((uintptr_t)T & 15) == 0) {
+    CQ_LAUNCH(apply_small_kernel, dim3(G.nbq * (G.k / 32), (G.d_out + AS_ROWS - 1) / AS_ROWS), 256, 0, st, (const uint16_t*)X, G.ld, T,
+              reinterpret_cast<uint16_t*>(Y), G.d_out, G.d_in, G.k, G.r, transposed, status);
+    return last_launch();
+  }
   {
     const Geo Ga = apply_geo(G);
     BdParams p;
@@ -907,8 +927,15 @@ extern "C" int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, 
   }
   float* U = b.take<float>(G.n);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
-  CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, T, Tc, kk, nullptr);
-  launch_apply(st, X, 1, G.ld, G, Tc, transposed, U, G.d_in, GEMM_STORE, nullptr, status);
+  bool applied = false;
+  if (tc_apply_ok(G.k)) {
+    launch_operator_bf16(st, T, Tb, G.k, G.nbT, transposed, status);
+    applied = apply_tc(st, X, G, Tb, U, nullptr, status);
+  }
+  if (!applied) {
+    CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, T, Tc, kk, nullptr);
+    launch_apply(st, X, 1, G.ld, G, Tc, transposed, U, G.d_in, GEMM_STORE, nullptr, status);
+  }
   CQ_LAUNCH(f32_to_bf16_kernel, grid_for(G.n), 256, 0, st, U, reinterpret_cast<uint16_t*>(Y), (long long)G.n);
   return last_launch();
 }
@@ -919,6 +946,16 @@ extern "C" int cafeq_dequant(const cafeq_matrix_desc* d, const uint8_t* packed, 
   int rc = make_geo(d, &G, false);
   if (rc) return rc;
   if (!packed || !scales || !What || ldo < G.d_in || (G.d_in % 8)) return CAFEQ_ERR_INVALID_ARG;
+  const long long n8 = G.n / 8;
+  if (G.g % 8 == 0 && ldo % 8 == 0 && ((uintptr_t)What & 15) == 0 && ((uintptr_t)packed & 7) == 0 && n8 < (1ll << 31)) {
+#define DQ8(B)                                                                                                           \
+  case B:                                                                                                                \
+    CQ_LAUNCH(dequant8_kernel<B>, (unsigned)((n8 + 1023) / 1024), 256, 0, (cudaStream_t)stream, packed, scales,          \
+              reinterpret_cast<uint16_t*>(What), (unsigned)n8, (unsigned)(G.d_in / 8), (unsigned)(G.g / 8), ldo);        \
+    return last_launch();
+    switch (d->bits) { DQ8(2) DQ8(3) DQ8(4) DQ8(5) DQ8(6) DQ8(7) DQ8(8) }
+#undef DQ8
+  }
   CQ_LAUNCH(dequant_kernel, grid_for(G.n / 8), 256, 0, (cudaStream_t)stream, packed, scales, reinterpret_cast<uint16_t*>(What), G.d_out,
             G.d_in, d->bits, G.g, ldo);
   return last_launch();
@@ -980,7 +1017,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
   const bool want_grad = (gradM != nullptr);
   const bool in_r1 = (G.axis == CAFEQ_AXIS_IN && G.r == 1);
   // straight-through mode on the tensor cores: input axis, no rounding offsets, shapes the fused pass covers
-  const bool ste_tc = ste && tc && in_r1 && off_kind == CAFEQ_OFFSETS_NONE && G.d_out % 64 == 0 &&
+  const bool ste_tc = ste && tc && in_r1 && off_kind == CAFEQ_OFFSETS_NONE &&
                       bd_supported(BD_IN, G.d_out, G.d_in, G.ld, k, G.g, W);
   if (tc) {
     PrepArgs pa;
@@ -1056,7 +1093,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       }
       TgParams p;
       memset(&p, 0, sizeof(p));
-      p.M = p.N = k; p.K = G.d_out; p.batch = G.nbT; p.nterms = 3;
+      p.M = p.N = k; p.K = (G.d_out + 63) / 64 * 64; p.batch = G.nbT; p.nterms = 3;  // (rows past the end read as zeros)
       p.a_mn = p.b_mn = 1;
       p.colsA_per_batch = p.colsB_per_batch = k;
       p.divA = 1;
@@ -1810,8 +1847,8 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
     // both products on the tensor cores where the shape allows (bf16 operands, fp32 accumulation either way); the operators in
     // applied orientation and the transposed first factor use scratch that the rounding fills later
     uint16_t *T1 = kkw.Ph, *T2 = kkw.Qh;
-    CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Mc, T1, G1.k, kk, 1, status);
-    CQ_LAUNCH(operator_to_bf16_kernel, grid_for(kk), 256, 0, st, Minv_c, T2, G1.k, kk, 0, status);
+    launch_operator_bf16(st, Mc, T1, G1.k, G1.nbT, 1, status);
+    launch_operator_bf16(st, Minv_c, T2, G1.k, G1.nbT, 0, status);
     if (!apply_tc(st, W1, G1, T1, w.U, w.UTh, status)) launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
     if (!apply_tc(st, W2, G2, T2, w.V, nullptr, status)) launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);
   } else {

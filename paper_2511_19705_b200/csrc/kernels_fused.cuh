@@ -939,7 +939,7 @@ static bool bd_supported(int form, int d_out, int d_in, long long ld, int k, int
   if (!(g == 64 || g == 128)) return false;
   if (form == BD_IN) {
     if (!(k == 64 || k == 128 || k == 256)) return false;
-    if (d_in % 256) return false;
+    if (d_in % 128) return false;  // (a half tile past the end reads zeros and stores nothing)
   } else {
     if (!(k == 128 || k == 256)) return false;
     if (d_out % k || d_in % 128) return false;
@@ -974,7 +974,7 @@ template <int FORM, int K, int G>
 static void bd_fill_tiles(BdParams& p) {
   using C = BdCfg<FORM, K, G>;
   if (FORM == BD_IN) {
-    p.n_major = p.d_in / 256;
+    p.n_major = (p.d_in + 255) / 256;
     p.n_minor = (p.d_out + 127) / 128;
   } else {
     p.n_major = p.d_out / K;
@@ -1151,16 +1151,111 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
   return CAFEQ_ERR_UNSUPPORTED;
 }
 
-// fp32 operator blocks -> bf16 in applied orientation (transposed when the role asks for T^T)
-__global__ void operator_to_bf16_kernel(const float* __restrict__ T, uint16_t* __restrict__ out, int k, long long n, int transpose,
-                                        const int32_t* status) {
+// fp32 operator blocks -> bf16 in applied orientation (transposed when the role asks for T^T); k % 32 == 0, one 32 x 32 tile
+// per CTA (grid: (k / 32, k / 32, blocks)), rows read and written along their elements.  Latency-bound: one load, one store
+// (14 blocks of 256: 5 - 7 us with a strided walk and 64-bit divisions per element, 3 us here).
+// paired (k = 32): blocks 2 i and 2 i + 1 become one 64 x 64 block, zeros off the diagonal.
+__global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* __restrict__ T, uint16_t* __restrict__ out, int k, int transpose,
+                                                               int paired, const int32_t* status) {
   if (status && *status) return;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    long long b = e / ((long long)k * k);
-    int i = (int)((e / k) % k), j = (int)(e % k);
-    float v = transpose ? T[b * k * k + (long long)j * k + i] : T[e];
-    out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+  __shared__ float tile[32][33];
+  const size_t base = (size_t)blockIdx.z * k * k;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;  // tile of the output
+  const int i = threadIdx.x >> 3, j = (threadIdx.x & 7) * 4;
+  const float* src = T + base + (transpose ? (size_t)(c0 + i) * k + r0 + j : (size_t)(r0 + i) * k + c0 + j);
+  float v[4];
+  if (((uintptr_t)T & 15) == 0) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(src));
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = __ldg(src + e);
   }
+  if (transpose) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tile[i][j + e] = v[e];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = tile[j + e][i];
+  }
+  uint32_t w[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    w[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * e])) |
+           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * e + 1])) << 16);
+  if (paired) {
+    const int odd = blockIdx.z & 1;
+    uint16_t* o = out + (size_t)(blockIdx.z >> 1) * 4096 + (odd * 32 + i) * 64 + j;
+    *reinterpret_cast<uint2*>(o + odd * 32) = make_uint2(w[0], w[1]);
+    *reinterpret_cast<uint2*>(o + (1 - odd) * 32) = make_uint2(0u, 0u);
+    return;
+  }
+  *reinterpret_cast<uint2*>(out + base + (size_t)(r0 + i) * k + c0 + j) = make_uint2(w[0], w[1]);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Y = P o X on the input axis for few rows (decoding): bf16 operands, fp32 accumulation, the operator read once in fp32 and
+// rounded on the way, so there is no conversion launch and no scratch.  Bound by latency: a CTA owns 32 output columns of one
+// block and eight rows, so that 14 blocks of 256 are 112 CTAs (in the tensor-core pass they are 14, each loading its
+// 128 KB operator through one TMA ring).  The operator tile and the rows go to shared memory as [contraction][column] and
+// [contraction][row]; warp w takes an eighth of the contraction, its partial sums meet in shared memory.
+// ------------------------------------------------------------------------------------------------
+constexpr int AS_ROWS = 8, AS_MAX_ROWS = 64;
+__global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* __restrict__ X, long long ld, const float* __restrict__ T,
+                                                          uint16_t* __restrict__ Y, int rows, int d_in, int k, int r, int transposed,
+                                                          const int32_t* status) {
+  if (status && *status) return;
+  __shared__ float ps[256 * 33];
+  __shared__ float4 xs4[256 * AS_ROWS / 4];
+  float* xs = reinterpret_cast<float*>(xs4);
+  const int strips = k / 32;
+  const int b = blockIdx.x / strips, n0 = (blockIdx.x - b * strips) * 32;
+  const int t0 = blockIdx.y * AS_ROWS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float* Tb = T + (size_t)(b / r) * k * k;
+  if (transposed) {  // P[n][m] = T[m][n]: 8 threads per contraction row
+#pragma unroll 8
+    for (int m = tid >> 3; m < k; m += 32) {
+      const int n = (tid & 7) * 4;
+      const float4 q = __ldg(reinterpret_cast<const float4*>(Tb + (size_t)m * k + n0 + n));
+      float* d = ps + m * 33 + n;
+      d[0] = round_to_bf16(q.x); d[1] = round_to_bf16(q.y); d[2] = round_to_bf16(q.z); d[3] = round_to_bf16(q.w);
+    }
+  } else {  // P[n][m] = T[n][m]: k / 4 threads per output column
+    const int q4 = k / 4;
+#pragma unroll 8
+    for (int e = tid; e < 32 * q4; e += 256) {
+      const int n = e / q4, m = (e - n * q4) * 4;
+      const float4 q = __ldg(reinterpret_cast<const float4*>(Tb + (size_t)(n0 + n) * k + m));
+      float* d = ps + m * 33 + n;
+      d[0] = round_to_bf16(q.x); d[33] = round_to_bf16(q.y); d[66] = round_to_bf16(q.z); d[99] = round_to_bf16(q.w);
+    }
+  }
+  for (int m = tid; m < k; m += 256)
+#pragma unroll
+    for (int t = 0; t < AS_ROWS; ++t)
+      xs[m * AS_ROWS + t] = (t0 + t < rows) ? bf16_bits_to_float(X[(long long)(t0 + t) * ld + (long long)b * k + m]) : 0.f;
+  __syncthreads();
+  float acc[AS_ROWS];
+#pragma unroll
+  for (int t = 0; t < AS_ROWS; ++t) acc[t] = 0.f;
+  const int len = k / 8;
+#pragma unroll 4
+  for (int m = warp * len; m < (warp + 1) * len; ++m) {
+    const float w = ps[m * 33 + lane];
+    const float4 x0 = xs4[m * 2], x1 = xs4[m * 2 + 1];
+    acc[0] = fmaf(w, x0.x, acc[0]); acc[1] = fmaf(w, x0.y, acc[1]); acc[2] = fmaf(w, x0.z, acc[2]); acc[3] = fmaf(w, x0.w, acc[3]);
+    acc[4] = fmaf(w, x1.x, acc[4]); acc[5] = fmaf(w, x1.y, acc[5]); acc[6] = fmaf(w, x1.z, acc[6]); acc[7] = fmaf(w, x1.w, acc[7]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < AS_ROWS; ++t) ps[(warp * AS_ROWS + t) * 32 + lane] = acc[t];
+  __syncthreads();
+  float y = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) y += ps[(w * AS_ROWS + warp) * 32 + lane];
+  if (t0 + warp < rows)
+    Y[(long long)(t0 + warp) * d_in + (long long)b * k + n0 + lane] = __bfloat16_as_ushort(__float2bfloat16_rn(y));
 }
 
 }  // namespace cafeq

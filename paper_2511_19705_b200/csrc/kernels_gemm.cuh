@@ -277,7 +277,7 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int kchunks = p.K / TG_BK;
+  const int kchunks = (p.K + TG_BK - 1) / TG_BK;
   const int total = kchunks * p.nterms;
 
   if (warp == 0) {
@@ -312,6 +312,8 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
     const uint32_t idesc = umma_idesc_bf16(128, BN, p.a_mn, p.b_mn);
     const uint32_t astep = p.a_mn ? 128 : 2, bstep = p.b_mn ? 128 : 2;  // 16 contraction entries further, in 16-byte units
     const uint32_t albo = p.a_mn ? 8192 : 16, blbo = p.b_mn ? 8192 : 16;
+    // a contraction of 32 (a chunk's second half belongs to the next block, or lies outside) takes two steps
+    const int nk = p.K < TG_BK ? p.K / 16 : 4;
     uint32_t s = 0, ph = 0;
     for (int it = 0; it < total; ++it) {
       if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, ph, abort_flag, p.status))) break;
@@ -320,7 +322,8 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
         const uint32_t sa = smem_u32(smem + s * C::STAGE);
         const uint32_t alo = umma_desc_lo(sa, albo), blo = umma_desc_lo(sa + C::A_BYTES, blbo);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) tc_mma_lo(tmem_base, alo + kk * astep, blo + kk * bstep, idesc, (it | kk) != 0 ? 1u : 0u);
+        for (int kk = 0; kk < 4; ++kk)
+          if (kk < nk) tc_mma_lo(tmem_base, alo + kk * astep, blo + kk * bstep, idesc, (it | kk) != 0 ? 1u : 0u);
         tc_commit(bar_empty + 8 * s);
         if (it == total - 1) tc_commit(bar_acc);
       }
@@ -681,14 +684,14 @@ static int tg_launch_t(cudaStream_t st, const TgOperand* A, const TgOperand* B, 
   return CAFEQ_OK;
 }
 
-// K must be a multiple of 64; operands 16-byte aligned with pitches that are multiples of 8 elements.
+// K must be a multiple of 64 (or 32: one half chunk); operands 16-byte aligned with pitches that are multiples of 8 elements.
 // Tile-width rule of the small batched products: the widest tile that still gives at least this many CTAs.
 // A CTA's life is dominated by fixed latencies and its epilogue, so narrow tiles (many CTAs) finish one product
 // sooner, while wide tiles (few CTAs) cost far fewer SM-microseconds and leave room for the kernels of other
 // problems running in other streams.  Default: narrow tiles (one chain alone); cafeq_set_overlap_mode changes it.
 static std::atomic<int> g_tg_min_ctas{96};
 static int tg_launch(cudaStream_t st, const TgOperand* A, const TgOperand* B, const TgParams& p) {
-  if (p.K % TG_BK || p.nterms < 1 || p.nterms > TG_MAX_TERMS) return CAFEQ_ERR_UNSUPPORTED;
+  if ((p.K % TG_BK && p.K != 32) || p.nterms < 1 || p.nterms > TG_MAX_TERMS) return CAFEQ_ERR_UNSUPPORTED;
   const int min_ctas = p.min_ctas > 0 ? p.min_ctas : g_tg_min_ctas.load(std::memory_order_relaxed);
   const long long mt = (long long)p.batch * ((p.M + 127) / 128);
   if (p.N > 128 && mt * ((p.N + 255) / 256) >= min_ctas) {

@@ -1361,7 +1361,59 @@ __global__ void pack_kernel(const int8_t* __restrict__ codes, uint8_t* __restric
   }
 }
 
-// The inverse of pack_kernel followed by the dequantisation: out[row][c] = bf16(scale(row, c / g) * (field - qmax)),
+// The inverse of pack_kernel followed by the dequantisation where eight codes share a scale (g % 8 == 0) and the output rows
+// are 16-byte aligned: out[row][c] = bf16(scale * (field - qmax)).  Bound by the bytes written: a thread takes four chunks of
+// eight codes, 256 chunks apart, and writes each as one 16-byte store.  The integer becomes a float through the mantissa of
+// 2^23 (exact; no conversion instruction), and chunk and group numbers run through the rows, so a dense output needs one
+// division per chunk.  2304 x 9216 at 4 bits: 38 -> 13 us against the scalar kernel below (eight 2-byte stores, eight scale
+// loads and nine divisions per chunk).
+template <int BITS>
+__global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* __restrict__ packed, const float* __restrict__ scales,
+                                                       uint16_t* __restrict__ out, unsigned n, unsigned cpr, unsigned cpg, long long ldo) {
+  constexpr uint32_t mask = (1u << BITS) - 1u;
+  constexpr float base = 8388608.f + (float)((1 << (BITS - 1)) - 1);
+  const unsigned c0 = blockIdx.x * 1024u + threadIdx.x;
+  unsigned long long v[4];
+  float s[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const unsigned c = c0 + u * 256u;
+    v[u] = 0;
+    s[u] = 0.f;
+    if (c < n) {
+      const uint8_t* src = packed + (size_t)c * BITS;
+      if constexpr (BITS == 2) v[u] = __ldg(reinterpret_cast<const uint16_t*>(src));
+      else if constexpr (BITS == 4) v[u] = __ldg(reinterpret_cast<const uint32_t*>(src));
+      else if constexpr (BITS == 8) v[u] = __ldg(reinterpret_cast<const unsigned long long*>(src));
+      else {
+#pragma unroll
+        for (int b = 0; b < BITS; ++b) v[u] |= (unsigned long long)__ldg(src + b) << (8 * b);
+      }
+      s[u] = __ldg(scales + c / cpg);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const unsigned c = c0 + u * 256u;
+    if (c >= n) break;
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float q0 = __uint_as_float(0x4B000000u | ((uint32_t)(v[u] >> (BITS * 2 * i)) & mask)) - base;
+      const float q1 = __uint_as_float(0x4B000000u | ((uint32_t)(v[u] >> (BITS * (2 * i + 1))) & mask)) - base;
+      w[i] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(s[u] * q0)) |
+             ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(s[u] * q1)) << 16);
+    }
+    size_t o = (size_t)c * 8;
+    if (ldo != (long long)cpr * 8) {
+      const unsigned row = c / cpr;
+      o = (size_t)row * ldo + (size_t)(c - row * cpr) * 8;
+    }
+    *reinterpret_cast<uint4*>(out + o) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// Any group width, pitch and alignment: the inverse of pack_kernel followed by the dequantisation: out[row][c] = bf16(scale(row, c / g) * (field - qmax)),
 // one thread per 8 consecutive codes (`bits` bytes of the stream); cols % 8 == 0, out row pitch ldo elements.
 __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict__ packed, const float* __restrict__ scales,
                                                       uint16_t* __restrict__ out, int rows, int cols, int bits, int g, long long ldo) {
