@@ -16,6 +16,7 @@
 #include "kernels_fused.cuh"
 #include "kernels_bwd.cuh"
 #include "kernels_gemm.cuh"
+#include "kernels_small.cuh"
 #include "kernels_kk.cuh"
 #include "kernels_dense.cuh"
 #include "kernels_rtn.cuh"
@@ -209,11 +210,14 @@ static void launch_kk(cudaStream_t st, const float* A, int tA, const float* B, i
 }
 
 static void launch_inverse(cudaStream_t st, const float* Mc, float* Minv, float* cnorm, int nb, int k, int32_t* status,
-                           const double* rn_check = nullptr, double tol2 = 0.0, int* redo_flag = nullptr, int* redo_count = nullptr) {
-  int threads = k * k >= 1024 ? 1024 : ((k * k + 31) / 32) * 32;
-  size_t sh = (size_t)3 * k * sizeof(float);
-  int ti = rn_check ? -1 : kt_begin(3, st);
-  CQ_LAUNCH(block_inverse_kernel, nb, threads, sh, st, Mc, Minv, cnorm, k, status, rn_check, tol2, redo_flag, redo_count);
+                           uint16_t* hi = nullptr, uint16_t* lo = nullptr, uint16_t* thi = nullptr, uint16_t* tlo = nullptr) {
+  int ti = kt_begin(3, st);
+  if (k == 32) CQ_LAUNCH(small_inverse_kernel<32>, nb, 256, 0, st, Mc, Minv, cnorm, hi, lo, thi, tlo, status);
+  else if (k == 64) CQ_LAUNCH(small_inverse_kernel<64>, nb, 256, 0, st, Mc, Minv, cnorm, hi, lo, thi, tlo, status);
+  else {  // (no splits)
+    const int threads = k * k >= 1024 ? 1024 : ((k * k + 31) / 32) * 32;
+    CQ_LAUNCH(block_inverse_kernel, nb, threads, (size_t)3 * k * sizeof(float), st, Mc, Minv, cnorm, k, status);
+  }
   kt_end(ti, st);
 }
 
@@ -230,8 +234,6 @@ struct KkWS {  // bf16 scratch, each [nbT * k * k]
                // transposed splits XTh / XTl are not maintained
 };
 constexpr int NS_MAX_ITERS = 8;
-constexpr int NS_COLD_ITERS = 6;
-constexpr int NS_WARM_ITERS = 4;  // upper bound: converged blocks skip the later ones (see ns_inverse)
 // Fused kernel (ns_block_kernel): rounds at most, and the squared residual before an update that makes it the last one.
 // Warm: below 1e-2 before, hence below 1e-4 after it (the acceptance test of the elimination fall-back).  Cold starts are
 // paid once per run: they go on to 1e-3 (1e-6 after the update, the accuracy the products themselves carry).
@@ -260,8 +262,7 @@ static void carve_kk(Bump& b, int nbT, int k, KkWS* w) {
 // C[b] = alpha * sum_t A_t[b] B_t[b]^T + beta * C0[b] + gamma * I for nb blocks of k x k; operands bf16 [nb*k, k]
 static int launch_kk_tc(cudaStream_t st, int nterms, const uint16_t* const* A, const uint16_t* const* B, int nb, int k,
                         float alpha, float beta, float gamma, const float* C0, float* C, uint16_t* Chi, uint16_t* Clo,
-                        uint16_t* Cthi, uint16_t* Ctlo, double* sq, const int* run_flag, int32_t* status, int sq_stride = 1,
-                        const double* gate = nullptr, double gate_tol = 0.0, int a_mn = 0, int b_mn = 0) {
+                        uint16_t* Cthi, uint16_t* Ctlo, double* sq, int32_t* status, int sq_stride = 1, int a_mn = 0, int b_mn = 0) {
   TgOperand oa[TG_MAX_TERMS], ob[TG_MAX_TERMS];
   for (int t = 0; t < nterms; ++t) {
     oa[t] = TgOperand{A[t], (long long)nb * k, k, k};
@@ -279,26 +280,14 @@ static int launch_kk_tc(cudaStream_t st, int nterms, const uint16_t* const* A, c
   p.C = C; p.ldc = k; p.sCb = (long long)k * k;
   p.Chi = Chi; p.Clo = Clo; p.Cthi = Cthi; p.Ctlo = Ctlo;
   p.sq = sq; p.sq_stride = sq_stride;
-  p.run_flag = run_flag;
-  p.gate = gate;
-  p.gate_tol = gate_tol;
   p.status = status;
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  if (g_tb_enable.load(std::memory_order_relaxed) && tb_supported(k, nterms)) {
+  if (tb_supported(k, nterms)) {
     const int rc = tb_launch(st, nterms, A, B, a_mn, b_mn, (long long)nb * k, (long long)nb * k, k, p);
     if (rc != CAFEQ_ERR_UNSUPPORTED) return rc;
   }
   if (a_mn || b_mn) return CAFEQ_ERR_UNSUPPORTED;  // the tiled kernel takes K-major operands only
   return tg_launch(st, oa, ob, p);
-}
-
-__global__ void transpose_blocks_kernel(const float* __restrict__ in, float* __restrict__ out, int k, long long n) {
-  const long long kk = (long long)k * k;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const long long b = e / kk, r = e - b * kk;
-    const int i = (int)(r / k), j = (int)(r - (long long)i * k);
-    out[e] = in[b * kk + (long long)j * k + i];
-  }
 }
 
 __global__ void zero_ns_kernel(double* rn, int n, int* flag) {
@@ -308,104 +297,64 @@ __global__ void zero_ns_kernel(double* rn, int n, int* flag) {
 }
 
 static void launch_split(cudaStream_t st, const float* X, int k, long long n, uint16_t* hi, uint16_t* lo, uint16_t* thi,
-                         uint16_t* tlo, const int* run_flag, const int32_t* status, const double* gate = nullptr,
-                         double gate_tol = 0.0) {
+                         uint16_t* tlo, const int32_t* status) {
   dim3 grid(k / 32, k / 32, (unsigned)(n / ((long long)k * k)));
-  CQ_LAUNCH(split_bf16_kernel, grid, dim3(32, 8), 0, st, X, k, hi, lo, thi, tlo, run_flag, status, gate, gate_tol);
+  CQ_LAUNCH(split_bf16_kernel, grid, dim3(32, 8), 0, st, X, k, hi, lo, thi, tlo, status);
 }
 
-// Minv = inv(bf16(M)) by Newton-Schulz iteration X <- X + X (I - A X) on the tensor cores, from X0 = A^T
-// (cold: right for the near-orthogonal transforms the method starts from) or from the caller's previous
-// inverse (warm).  The last residual is checked on the device; if it is not small the Gauss-Jordan kernel
-// recomputes the block.  Leaves fp32 Minv in X and its bf16 splits in w.Xh/Xl (and XTh/XTl unless w.mn) [w.cur].
-// eq4 (block sizes of the fused kernel): where the kernel puts the column norms / group weights, and what it ticks.
+// Minv = inv(bf16(M)).  k = 128, 256: Newton-Schulz iteration X <- X + X (I - A X) on the tensor cores, every round of a block
+// in one launch, from X0 = A^T (cold: right for the near-orthogonal transforms the method starts from) or from the caller's
+// previous inverse (warm); a warm start runs as many rounds as the step size calls for (a block whose residual ||I - A X||_F
+// was below 1e-2 before an update, 1e-4 after it, stops); a residual that does not become small falls back to elimination.
+// k = 32, 64: elimination, which takes less than one round's launches there.  Leaves fp32 Minv in X and its bf16 splits in
+// w.Xh / Xl (and XTh / XTl unless w.mn) [w.cur].
+// eq4 (k = 128, 256): where the kernel puts the column norms / group weights, and what it ticks.
 static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k, bool warm, KkWS& w, int32_t* status,
                       bool prepped = false, bool splits_kept = false, const NsParams* eq4 = nullptr) {
-  const long long kk = (long long)nb * k * k;
-  const int iters = warm ? NS_WARM_ITERS : NS_COLD_ITERS;
-  // A warm start runs as many rounds as the step size calls for: a block whose residual ||I - A X||_F was below 1e-2
-  // before an update (below 1e-4 after it) stops.  Small steps take one or two rounds, a change of the transform by
-  // half its norm four.
+  w.cur = 0;
+  w.mn = tb_supported(k, 2);
+  if (!w.mn) {
+    launch_inverse(st, Mc, X, nullptr, nb, k, status, w.Xh[0], w.Xl[0], w.XTh[0], w.XTl[0]);
+    return CAFEQ_OK;
+  }
   int ti = kt_begin(3, st);
   if (!prepped) {  // otherwise step_prep_kernel has cleared rn / flag and written Ab
     CQ_LAUNCH(zero_ns_kernel, (NS_MAX_ITERS * nb + 127) / 128, 128, 0, st, w.rn, NS_MAX_ITERS * nb, w.flag);
     launch_operator_bf16(st, Mc, w.Ab, k, nb, 0, status);
   }
-  // Block sizes of the fused kernel: every round of a block runs in one launch, on row-major splits only.
-  w.mn = g_tb_enable.load(std::memory_order_relaxed) && tb_supported(k, 2);
-  if (w.mn) {
-    w.cur = 0;
-    // (splits_kept: the splits of X that the previous call left in set 0 are still there)
-    if (!warm) CQ_LAUNCH(ns_cold_start_kernel, dim3(k / 32, k / 32, nb), dim3(32, 8), 0, st, w.Ab, k, w.Xh[0], w.Xl[0], status);
-    else if (!splits_kept) launch_split(st, X, k, kk, w.Xh[0], w.Xl[0], nullptr, nullptr, nullptr, status);
-    NsParams np;
-    memset(&np, 0, sizeof(np));
-    if (eq4) np = *eq4;
-    np.max_rounds = warm ? NS_WARM_ROUNDS : NS_COLD_ROUNDS;
-    np.gate2 = warm ? NS_GATE2 : NS_COLD_GATE2;
-    np.accept2 = NS_GATE2;
-    np.redo_count = w.redo_total;
-    np.status = status;
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    const int rc = ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np);
-    kt_end(ti, st);
-    return rc;
-  }
-  if (!warm) CQ_LAUNCH(transpose_blocks_kernel, grid_for(kk), 256, 0, st, Mc, X, k, kk);
-  int cur = 0;
-  launch_split(st, X, k, kk, w.Xh[cur], iters > 0 ? nullptr : w.Xl[cur], w.XTh[cur], w.XTl[cur], nullptr, status);
-  for (int it = 0; it < iters; ++it) {
-    const double* gate = (warm && it > 0) ? w.rn + (size_t)(it - 1) * nb : nullptr;
-    // R = I - A X needs X to full precision (the product cancels against I): two terms over the split of X.
-    // X += X R: the correction is small and the iteration corrects its own errors, so one bf16 term is enough
-    // (the error it leaves is 2^-8 |R| relative, below 4e-5 for every accepted residual).
-    const uint16_t* a1[2] = {w.Ab, w.Ab};
-    const uint16_t* a2[1] = {w.Xh[cur]};
-    const uint16_t* b1[2] = {w.XTh[cur], w.XTl[cur]};
-    launch_kk_tc(st, 2, a1, b1, nb, k, -1.f, 0.f, 1.f, nullptr, nullptr, nullptr, nullptr, w.RTh, nullptr, w.rn + (size_t)it * nb,
-                 nullptr, status, 1, gate, NS_GATE2);
-    const uint16_t* b2[1] = {w.RTh};
-    // (the row-major low half is only read after the last iteration, by the M^-1 path of the gradient)
-    launch_kk_tc(st, 1, a2, b2, nb, k, 1.f, 1.f, 0.f, X, X, w.Xh[cur ^ 1], (it == iters - 1) ? w.Xl[cur ^ 1] : nullptr,
-                 w.XTh[cur ^ 1], w.XTl[cur ^ 1], nullptr, nullptr, status, 1, gate, NS_GATE2);
-    cur ^= 1;
-  }
-  w.cur = cur;
-  // accept when ||I - A X||_F before the last update was below 1e-2 (the update squares it: <= 1e-4 after); a block
-  // that skipped the last iteration has a zero there and was accepted by the gate
-  launch_inverse(st, Mc, X, nullptr, nb, k, status, w.rn + (size_t)(iters - 1) * nb, 1e-4, w.flag, w.redo_total);
-  // final splits: written by the last iteration's epilogue, except for blocks that skipped it (and for everything
-  // when the elimination recomputed a block)
-  const double* last_gate = (warm && iters > 1) ? w.rn + (size_t)(iters - 2) * nb : nullptr;
-  launch_split(st, X, k, kk, w.Xh[cur], w.Xl[cur], w.XTh[cur], w.XTl[cur], w.flag, status, last_gate, NS_GATE2);
+  // (splits_kept: the splits of X that the previous call left in set 0 are still there)
+  if (!warm) CQ_LAUNCH(ns_cold_start_kernel, dim3(k / 32, k / 32, nb), dim3(32, 8), 0, st, w.Ab, k, w.Xh[0], w.Xl[0], status);
+  else if (!splits_kept) launch_split(st, X, k, (long long)nb * k * k, w.Xh[0], w.Xl[0], nullptr, nullptr, status);
+  NsParams np;
+  memset(&np, 0, sizeof(np));
+  if (eq4) np = *eq4;
+  np.max_rounds = warm ? NS_WARM_ROUNDS : NS_COLD_ROUNDS;
+  np.gate2 = warm ? NS_GATE2 : NS_COLD_GATE2;
+  np.accept2 = NS_GATE2;
+  np.redo_count = w.redo_total;
+  np.status = status;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  const int rc = ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np);
   kt_end(ti, st);
-  return CAFEQ_OK;
+  return rc;
 }
 
-// G -= X^T Gx X^T for every block, on the tensor cores with three-term bf16 splits; X = Minv with its splits in
-// w[w.cur]; Gx = dL/dMinv: fp32 [nb,k,k], or (scaled, fused kernel only) formed from X by the kernel itself.
-static int minv_path_tc(cudaStream_t st, const float* Gx, float* G, int nb, int k, KkWS& w, int32_t* status,
+// G -= X^T Gx X^T for every block; X = Minv.  k = 128, 256: on the tensor cores from its splits in w[w.cur], three-term
+// products; 32, 64: in fp32.  Gx = dL/dMinv: fp32 [nb, k, k], or (scaled) formed from X by the kernel itself.
+static int minv_path_tc(cudaStream_t st, const float* X, const float* Gx, float* G, int nb, int k, KkWS& w, int32_t* status,
                         const ChainParams* scaled = nullptr) {
-  const long long kk = (long long)nb * k * k;
-  const int c = w.cur;
+  ChainParams cp;
+  memset(&cp, 0, sizeof(cp));
+  if (scaled) cp = *scaled;
   if (w.mn) {
-    ChainParams cp;
-    memset(&cp, 0, sizeof(cp));
-    if (scaled) cp = *scaled;
     cp.G = Gx;
     cp.status = status;
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return kk_chain_launch(st, KK_MINV_PATH, w.Xh[c], w.Xl[c], G, nb, k, cp);
+    return kk_chain_launch(st, KK_MINV_PATH, w.Xh[w.cur], w.Xl[w.cur], G, nb, k, cp);
   }
-  launch_split(st, Gx, k, kk, nullptr, nullptr, w.Ph, w.Pl, nullptr, status);  // Gx^T splits
-  // T1 = X^T Gx : T1[i][j] = sum_l XT[i][l] * GxT[j][l]
-  const uint16_t* a1[3] = {w.XTh[c], w.XTl[c], w.XTh[c]};
-  const uint16_t* b1[3] = {w.Ph, w.Ph, w.Pl};
-  launch_kk_tc(st, 3, a1, b1, nb, k, 1.f, 0.f, 0.f, nullptr, nullptr, w.Qh, w.Ql, nullptr, nullptr, nullptr, nullptr, status);
-  // G -= T1 X^T : [i][j] = sum_l T1[i][l] * X[j][l]
-  const uint16_t* a2[3] = {w.Qh, w.Ql, w.Qh};
-  const uint16_t* b2[3] = {w.Xh[c], w.Xh[c], w.Xl[c]};
-  return launch_kk_tc(st, 3, a2, b2, nb, k, -1.f, 1.f, 0.f, G, G, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status);
+  if (k == 32) CQ_LAUNCH(small_chain_kernel<32>, nb, 64, 0, st, X, Gx, cp.A[0], cp.Agrp[0], cp.g[0], cp.scale[0], G, status);
+  else CQ_LAUNCH(small_chain_kernel<64>, nb, 256, 0, st, X, Gx, cp.A[0], cp.Agrp[0], cp.g[0], cp.scale[0], G, status);
+  return CAFEQ_OK;
 }
 
 // Orthonormality penalty of nb blocks from the splits of the fp32 parameters (fused kernel, k = 128 / 256):
@@ -430,26 +379,36 @@ static void launch_absmax(cudaStream_t st, const float* U, long long ld, const G
 
 // Group quantiser of an fp32 matrix U [rows, ng g] (pitch ld; Delta / Uhat share it): maxima, signed arg-max values, arg-max
 // positions, scales, residual, dequantised values, codes -- each optional except a / usel / idx.
+template <typename SRC>
+static bool launch_group_quant_vec(cudaStream_t st, const SRC* U, long long ld, int rows, int ng, int g, float qmax, const void* offsets,
+                                   int off_kind, float* a, float* usel, int* idx, float* Delta, float* Uhat, int8_t* codes, float* scales,
+                                   int32_t* status) {
+  const long long groups = (long long)rows * ng;
+  if (g % 4 || g > 16384 || ld % 4 || ((uintptr_t)U & (4 * sizeof(SRC) - 1)) || (((uintptr_t)Delta | (uintptr_t)Uhat) & 15) ||
+      ((uintptr_t)codes & 3))
+    return false;
+#define GQ(L, N)                                                                                                              \
+  CQ_LAUNCH((group_quant_kernel<L, N, SRC>), (unsigned)((groups * L + 255) / 256), 256, 0, st, U, ld, rows, ng, g, qmax, offsets, off_kind, \
+            a, usel, idx, Delta, Uhat, codes, scales, status)
+  // as many lanes as the group has vectors of four, up to a warp; above eight vectors a lane, the whole CTA
+  if (g <= 32) GQ(8, 1);
+  else if (g <= 64) GQ(16, 1);
+  else if (g <= 128) GQ(32, 1);
+  else if (g <= 256) GQ(32, 2);
+  else if (g <= 512) GQ(32, 4);
+  else if (g <= 1024) GQ(32, 8);
+  else if (g <= 2048) GQ(256, 2);
+  else if (g <= 4096) GQ(256, 4);
+  else if (g <= 8192) GQ(256, 8);
+  else GQ(256, 16);
+#undef GQ
+  return true;
+}
 static void launch_group_quant(cudaStream_t st, const float* U, long long ld, int rows, int ng, int g, float qmax, const void* offsets,
                                int off_kind, float* a, float* usel, int* idx, float* Delta, float* Uhat, int8_t* codes, float* scales,
                                int32_t* status) {
   const long long groups = (long long)rows * ng;
-  const bool vec = g % 4 == 0 && g <= 1024 && ld % 4 == 0 && !(((uintptr_t)U | (uintptr_t)Delta | (uintptr_t)Uhat) & 15) &&
-                   !((uintptr_t)codes & 3);
-  if (vec) {
-#define GQ(L, N)                                                                                                              \
-  CQ_LAUNCH((group_quant_kernel<L, N>), (unsigned)((groups * L + 255) / 256), 256, 0, st, U, ld, rows, ng, g, qmax, offsets, off_kind, \
-            a, usel, idx, Delta, Uhat, codes, scales, status)
-    // as many lanes as the group has float4s, up to a warp
-    if (g <= 32) GQ(8, 1);
-    else if (g <= 64) GQ(16, 1);
-    else if (g <= 128) GQ(32, 1);
-    else if (g <= 256) GQ(32, 2);
-    else if (g <= 512) GQ(32, 4);
-    else GQ(32, 8);
-#undef GQ
-    return;
-  }
+  if (launch_group_quant_vec<float>(st, U, ld, rows, ng, g, qmax, offsets, off_kind, a, usel, idx, Delta, Uhat, codes, scales, status)) return;
   CQ_LAUNCH(absmax_kernel, (unsigned)((groups * 32 + 255) / 256), 256, 0, st, U, ld, rows, ng, g, a, usel, idx, status);
   if (Delta || Uhat || codes)
     CQ_LAUNCH(quant_kernel, grid_for((long long)rows * ng * g), 256, 0, st, U, ld, rows, ng * g, g, a, qmax, offsets, off_kind, Delta, Uhat,
@@ -646,7 +605,7 @@ static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo&
   const int two = (form == BD_IN && G.k == 32 && G.r == 1) ? 1 : 0;
   const int k = two ? 64 : G.k, nbT = two ? G.nbT / 2 : G.nbT;
   if (!bd_supported(form, G.d_out, G.d_in, ldx, k, G.g, X)) return false;
-  if (Tb_ready && !transposed) Tb = const_cast<uint16_t*>(Tb_ready);  // bf16 operator already in applied orientation
+  if (Tb_ready && !transposed && !two) Tb = const_cast<uint16_t*>(Tb_ready);  // bf16 operator already in applied orientation
   else launch_operator_bf16(st, Top, Tb, G.k, G.nbT, transposed, status, two);
   p.d_out = G.d_out;
   p.d_in = G.d_in;
@@ -663,8 +622,8 @@ static bool tc_apply_ok(int k) { return k == 32 || kk_fast(k); }
 
 // U = T o W in fp32 as one-term batched products on the tensor cores (bf16 x bf16 products are exact, fp32
 // accumulation: the same arithmetic as the fused pass).  Tb: bf16 operator blocks in applied orientation
-// [nbT k, k].  Output axis: the contraction runs down the rows of W, so its transpose goes through WT first.
-static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_t* Tb, float* U, uint16_t* WT, int32_t* status) {
+// [nbT k, k].
+static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_t* Tb, float* U, int32_t* status) {
   const int k = G.k;
   if (!tc_apply_ok(k) || ((uintptr_t)W & 15) || (G.ld % 8) || (G.d_in % 4)) return false;
   TgOperand oa[1], ob[1];
@@ -681,15 +640,13 @@ static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_
     p.rowsA_per_batch = 0; p.colsA_per_batch = k;
     p.rowsB_per_batch = k; p.divB = G.r;
     p.sCb = k;
-  } else {
-    if (!WT || (G.d_out % 8)) return false;
-    dim3 tg((G.d_in + 31) / 32, (G.d_out + 31) / 32);
-    CQ_LAUNCH(transpose_bf16_kernel, tg, dim3(32, 8), 0, st, (const uint16_t*)W, G.d_out, G.d_in, G.ld, WT);
+  } else {  // the contraction runs down the rows of W as they are stored
     oa[0] = TgOperand{Tb, (long long)G.nbT * k, k, k};
-    ob[0] = TgOperand{WT, G.d_in, G.d_out, G.d_out};
+    ob[0] = TgOperand{W, G.d_out, G.d_in, G.ld};
     p.M = k; p.N = G.d_in;
+    p.b_mn = 1;
     p.rowsA_per_batch = k; p.divA = G.r;
-    p.rowsB_per_batch = 0; p.colsB_per_batch = k;
+    p.rowsB_per_batch = k;
     p.sCb = (long long)k * G.d_in;
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -702,7 +659,7 @@ static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_
 static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits, const float* Tc, int transposed,
                           const MatWS& w, const void* offsets, int off_kind, bool want_delta, float* Uhat, int8_t* codes,
                           float* scales, int32_t* status, bool allow_fused, const BdParams* surr = nullptr,
-                          const uint16_t* Tb_ready = nullptr, uint16_t* WT_scratch = nullptr, float* T_rounded = nullptr) {
+                          const uint16_t* Tb_ready = nullptr, float* T_rounded = nullptr) {
   if (Tc && allow_fused && off_kind == CAFEQ_OFFSETS_NONE && !Uhat) {
     BdParams p;
     memset(&p, 0, sizeof(p));
@@ -718,7 +675,7 @@ static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits
   if (Tc && allow_fused) {  // (allow_fused is off when the caller asked for the shape-agnostic kernels)
     const uint16_t* Tb = (Tb_ready && !transposed) ? Tb_ready : w.Tb;
     if (Tb == w.Tb && tc_apply_ok(G.k)) launch_operator_bf16(st, Tc, w.Tb, G.k, G.nbT, transposed, status);
-    applied = apply_tc(st, W, G, Tb, w.U, WT_scratch, status);
+    applied = apply_tc(st, W, G, Tb, w.U, status);
   }
   if (applied) {
   } else if (Tc) {
@@ -857,6 +814,9 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (rtn_stream_launch(st, W, G.ld, G.d_out, G.d_in, G.g, qmax_of(d->bits), codes, scales)) return last_launch();
     g_launches.fetch_sub(1, std::memory_order_relaxed);
+    if (launch_group_quant_vec<uint16_t>(st, (const uint16_t*)W, G.ld, G.d_out, G.ng, G.g, qmax_of(d->bits), nullptr, CAFEQ_OFFSETS_NONE,
+                                         nullptr, nullptr, nullptr, nullptr, nullptr, codes, scales, nullptr))
+      return last_launch();
   }
   if ((rc = check_ws(ws, ws_bytes))) return rc;
   Bump b(ws, ws_bytes);
@@ -865,7 +825,7 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
   rtn_scratch(G, has_T, W, codes, &b, &w, &Tc);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   forward_quant(st, W, G, d->bits, has_T ? T : nullptr, d->trole == CAFEQ_APPLY_TT, w, nullptr, CAFEQ_OFFSETS_NONE, false, nullptr, codes,
-                scales, nullptr, true, nullptr, nullptr, nullptr, Tc);
+                scales, nullptr, true, nullptr, nullptr, Tc);
   return last_launch();
 }
 
@@ -930,7 +890,7 @@ extern "C" int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, 
   bool applied = false;
   if (tc_apply_ok(G.k)) {
     launch_operator_bf16(st, T, Tb, G.k, G.nbT, transposed, status);
-    applied = apply_tc(st, X, G, Tb, U, nullptr, status);
+    applied = apply_tc(st, X, G, Tb, U, status);
   }
   if (!applied) {
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, T, Tc, kk, nullptr);
@@ -1009,7 +969,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
                         float* losses, float* hist, float* gradM, int32_t* status, SingleWS& s, bool force_generic,
                         bool warm = false, float* step_counter = nullptr, float* grad_offsets = nullptr, bool splits_kept = false) {
   const int k = G.k;
-  const bool tc = kk_fast(k) && !force_generic;
+  const bool tc = (k == 32 || kk_fast(k)) && !force_generic;
   const long long kk = (long long)G.nbT * k * k;
   const float qm = qmax_of(d->bits);
   const bool ste = (loss_kind == CAFEQ_LOSS_L2_STE);
@@ -1109,12 +1069,11 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       if (w.mn) {  // both operands are X read transposed from its row-major splits
         const uint16_t* a1[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
         const uint16_t* b1[3] = {w.Xh[c], w.Xh[c], w.Xl[c]};
-        launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, nullptr, status, 1,
-                     nullptr, 0.0, 1, 1);
+        launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status, 1, 1, 1);
       } else {
         const uint16_t* a1[3] = {w.XTh[c], w.XTl[c], w.XTh[c]};
         const uint16_t* b1[3] = {w.XTh[c], w.XTh[c], w.XTl[c]};
-        launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, nullptr, status);
+        launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status);
       }
     }
     CQ_LAUNCH(dot_f32_kernel, grid_for(kk), 256, 0, st, s.Nf, s.tmp, kk, s.acc + 1);
@@ -1124,7 +1083,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     {  // dL/dMinv = 2 Minv Gram (Gram is symmetric: its rows serve as the contraction-major second operand)
       const uint16_t* a2[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
       const uint16_t* b2[3] = {w.Ph, w.Ph, w.Pl};
-      launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+      launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr,
                    status);
     }
     {  // gDelta[o, B k + j] = 2 sum_l N_B[j][l] Delta[o, B k + l]  -> s.m.D (fp32 [d_out, d_in])
@@ -1150,7 +1109,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     CQ_LAUNCH(ste_scale_coef_kernel, (unsigned)((nrec * 32 + 255) / 256), 256, 0, st, s.m.D, (long long)G.d_in, s.m.Dbf, s.Dlo,
               (long long)G.d_in, G.d_out, G.ng, G.g, s.m.a, s.m.usel, 1, s.m.coef, status);
     launch_scatter(st, W, G, s.m.coef, s.m.idx, gradM, 0, status, 1);
-    s.err = minv_path_tc(st, s.gMinv, gradM, G.nbT, k, s.kk, status);
+    s.err = minv_path_tc(st, s.Minv, s.gMinv, gradM, G.nbT, k, s.kk, status);
     return;
   }
   if (need_l2) {
@@ -1177,14 +1136,14 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
   if (!want_grad) return;
   if (!ste) {
     launch_scatter(st, W, G, s.m.coef, s.m.idx, gradM, 0, status, fused ? 1 : 0);
-    if (tc && s.kk.mn) {
+    if (tc) {
       ChainParams cp;
       memset(&cp, 0, sizeof(cp));
       cp.n = 1;
       cp.blk0[1] = G.nbT;
       cp.A[0] = s.A; cp.Agrp[0] = in_r1 ? s.m.agrp : nullptr; cp.g[0] = G.g; cp.scale[0] = 2.f * kappa;
       cp.X = s.Minv;
-      s.err = minv_path_tc(st, nullptr, gradM, G.nbT, k, s.kk, status, &cp);
+      s.err = minv_path_tc(st, s.Minv, nullptr, gradM, G.nbT, k, s.kk, status, &cp);
       return;
     }
     CQ_LAUNCH(gminv_kernel, grid_for(kk), 256, 0, st, s.Minv, s.A, in_r1 ? s.m.agrp : nullptr, G.g, 2.f * kappa, k, kk, s.gMinv);
@@ -1202,7 +1161,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
   }
   // gradM -= Minv^T gMinv Minv^T
   if (tc) {
-    s.err = minv_path_tc(st, s.gMinv, gradM, G.nbT, k, s.kk, status);
+    s.err = minv_path_tc(st, s.Minv, s.gMinv, gradM, G.nbT, k, s.kk, status);
   } else {
     launch_kk(st, s.Minv, 1, s.gMinv, 0, s.tmp, G.nbT, k, 1.f, GEMM_STORE, status);
     launch_kk(st, s.tmp, 0, s.Minv, 1, gradM, G.nbT, k, -1.f, GEMM_STORE | GEMM_ACCUM, status);
@@ -1343,7 +1302,6 @@ struct PairWS {
   DenseWS dn;
   bool dense;  // the product term runs on the tensor cores (every dimension a multiple of 64)
   uint16_t *gVh, *gVl;          // [d3, r h]: split of the second factor's gradient
-  uint16_t* W1T;                // [d1, h]: transposed first factor (its apply contracts down the rows)
   bool lean;                    // carved without matrix-sized scratch: only the fused LogSumExp path may run
   int err;
 };
@@ -1420,9 +1378,8 @@ static bool carve_pair(Bump& b, const Geo& G1, const Geo& G2, PairWS* p, bool ne
   carve_kk(b, G1.nbT, G1.k, &p->kk);
   p->dense = need_R && dense_ok(G1, G2);
   if (p->dense) carve_dense(b, G1.d_out, G1.d_in, G2.d_out, G2.r, G1.k, G1.ng, G2.ng, &p->dn);
-  p->gVh = p->gVl = p->W1T = nullptr;
+  p->gVh = p->gVl = nullptr;
   if (p->dense) {
-    p->W1T = b.take<uint16_t>(G1.n);
     p->gVh = b.take<uint16_t>(G2.n);
     p->gVl = b.take<uint16_t>(G2.n);
   }
@@ -1517,7 +1474,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
   CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, p.Minv, p.Minv_c, kk, status);
   // U = M_c^T o W1 (axis OUT), V = Minv_c o W2 (axis IN); Uhat kept in the E buffers when PQE is wanted
   const bool f1 = forward_quant(st, W1, G1, d1->bits, p.Mc, 1, p.m1, nullptr, CAFEQ_OFFSETS_NONE, false, want_pqe ? p.m1.E : nullptr, nullptr,
-                nullptr, status, !force_generic, nullptr, nullptr, p.W1T);
+                nullptr, status, !force_generic);
   const bool f2 = forward_quant(st, W2, G2, d2->bits, p.Minv_c, 0, p.m2, nullptr, CAFEQ_OFFSETS_NONE, false, want_pqe ? p.m2.E : nullptr,
                 nullptr, nullptr, status, !force_generic, nullptr, tc ? p.kk.Xh[p.kk.cur] : nullptr);  // Xh = bf16(Minv)
   const long long n1 = (long long)G1.d_out * G1.ng, n2 = (long long)G2.d_out * G2.ng;
@@ -1539,21 +1496,21 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
   if (ste) {
   } else if (tc && p.kk.mn) {
     KkWS& w = p.kk;
-    launch_split(st, M, k, kk, w.Ph, w.Pl, nullptr, nullptr, nullptr, status);
+    launch_split(st, M, k, kk, w.Ph, w.Pl, nullptr, nullptr, status);
     p.err = penalty_tc(st, w.Ph, w.Pl, p.RM, gradM && lambda != 0.f, p.acc + 1, 0, G1.nbT, k, status);
     if (p.err) return;
   } else if (tc) {
     // R = M M^T - I (symmetric) with its bf16 splits, ||R||_F^2, and R M for the gradient
     KkWS& w = p.kk;
-    launch_split(st, M, k, kk, w.Ph, w.Pl, w.Qh, w.Ql, nullptr, status);
+    launch_split(st, M, k, kk, w.Ph, w.Pl, w.Qh, w.Ql, status);
     const uint16_t* a1[3] = {w.Ph, w.Pl, w.Ph};
     const uint16_t* b1[3] = {w.Ph, w.Ph, w.Pl};
-    launch_kk_tc(st, 3, a1, b1, G1.nbT, k, 1.f, 0.f, -1.f, nullptr, nullptr, w.RTh, w.RTl, nullptr, nullptr, p.acc + 1, nullptr,
+    launch_kk_tc(st, 3, a1, b1, G1.nbT, k, 1.f, 0.f, -1.f, nullptr, nullptr, w.RTh, w.RTl, nullptr, nullptr, p.acc + 1,
                  status, 0);
     if (gradM && lambda != 0.f) {
       const uint16_t* a2[3] = {w.RTh, w.RTl, w.RTh};
       const uint16_t* b2[3] = {w.Qh, w.Qh, w.Ql};
-      launch_kk_tc(st, 3, a2, b2, G1.nbT, k, 1.f, 0.f, 0.f, nullptr, p.RM, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+      launch_kk_tc(st, 3, a2, b2, G1.nbT, k, 1.f, 0.f, 0.f, nullptr, p.RM, nullptr, nullptr, nullptr, nullptr, nullptr,
                    status);
     }
   } else {
@@ -1620,7 +1577,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       launch_opgrad(st, w.V, G2.d_in, W2, 1, G2.ld, G2, p.gMinv, 0, 1.f, status);  // V side: operator Minv
     }
     if (tc) {
-      p.err = minv_path_tc(st, p.gMinv, gradM, G1.nbT, k, p.kk, status);
+      p.err = minv_path_tc(st, p.Minv, p.gMinv, gradM, G1.nbT, k, p.kk, status);
     } else {
       launch_kk(st, p.Minv, 1, p.gMinv, 0, p.RM, G1.nbT, k, 1.f, GEMM_STORE, status);
       launch_kk(st, p.RM, 0, p.Minv, 1, gradM, G1.nbT, k, -1.f, GEMM_STORE | GEMM_ACCUM, status);
@@ -1647,7 +1604,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     CQ_LAUNCH(axpy_norm_kernel, grid_for(kk), 256, 0, st, p.gMinv, p.T2, kk, p.acc, 3, (double)n1, 6, status);
   }
   if (tc) {
-    p.err = minv_path_tc(st, p.gMinv, gradM, G1.nbT, k, p.kk, status);
+    p.err = minv_path_tc(st, p.Minv, p.gMinv, gradM, G1.nbT, k, p.kk, status);
   } else {
     launch_kk(st, p.Minv, 1, p.gMinv, 0, p.RM, G1.nbT, k, 1.f, GEMM_STORE, status);
     launch_kk(st, p.RM, 0, p.Minv, 1, gradM, G1.nbT, k, -1.f, GEMM_STORE | GEMM_ACCUM, status);
@@ -1849,8 +1806,8 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
     uint16_t *T1 = kkw.Ph, *T2 = kkw.Qh;
     launch_operator_bf16(st, Mc, T1, G1.k, G1.nbT, 1, status);
     launch_operator_bf16(st, Minv_c, T2, G1.k, G1.nbT, 0, status);
-    if (!apply_tc(st, W1, G1, T1, w.U, w.UTh, status)) launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
-    if (!apply_tc(st, W2, G2, T2, w.V, nullptr, status)) launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);
+    if (!apply_tc(st, W1, G1, T1, w.U, status)) launch_apply(st, W1, 1, G1.ld, G1, Mc, 1, w.U, G1.d_in, GEMM_STORE, nullptr, status);
+    if (!apply_tc(st, W2, G2, T2, w.V, status)) launch_apply(st, W2, 1, G2.ld, G2, Minv_c, 0, w.V, G2.d_in, GEMM_STORE, nullptr, status);
   } else {
     CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G1.n), 256, 0, st, (const uint16_t*)W1, G1.ld, G1.d_out, G1.d_in, w.U);
     CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G2.n), 256, 0, st, (const uint16_t*)W2, G2.ld, G2.d_out, G2.d_in, w.V);

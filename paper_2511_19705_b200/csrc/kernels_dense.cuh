@@ -72,25 +72,6 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
   }
 }
 
-// bf16 [R, C] (pitch ld) -> bf16 transposed [C, R]
-__global__ void __launch_bounds__(256) transpose_bf16_kernel(const uint16_t* __restrict__ X, int R, int C, long long ld,
-                                                             uint16_t* __restrict__ T) {
-  __shared__ uint16_t tile[32][34];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = r0 + ty + 8 * q, c = c0 + tx;
-    tile[ty + 8 * q][tx] = (r < R && c < C) ? X[(long long)r * ld + c] : (uint16_t)0;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int c = c0 + ty + 8 * q, r = r0 + tx;
-    if (r < R && c < C) T[(long long)c * R + r] = tile[tx][ty + 8 * q];
-  }
-}
-
 // Bf[B*k + j][y] = sum_rep V[y][(B*r + rep)*k + j]: fold the r replicas of every block of the inner dimension
 // and transpose (V fp32 [d3, r*h] -> Bf fp32 [h, d3]).  grid: ceil(d3/32), h/32 (k % 32 == 0); block 32 x 8.
 __global__ void __launch_bounds__(256) fold_transpose_kernel(const float* __restrict__ V, int d3, int h, int k, int r,

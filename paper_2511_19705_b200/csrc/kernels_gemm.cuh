@@ -47,13 +47,10 @@ struct TgParams {
   uint16_t *Cthi, *Ctlo;  // bf16 splits, transposed [batch][N][M] (ld = M)
   double* sq;             // sum of C^2: sq[b * sq_stride]
   int sq_stride;
-  const int* run_flag;    // optional: skip the whole launch when *run_flag == 0
   int a_mn, b_mn;         // the A / B arrays are stored [l][m] / [l][n] (MN-major operands); a batch then starts at column
-                          // batch * colsA_per_batch / colsB_per_batch
+                          // batch * colsA_per_batch / colsB_per_batch (B: its contraction at row batch * rowsB_per_batch)
   const double* stop_sq;  // optional: squared residuals of an iteration; this launch belongs to iteration stop_it, and is
   int stop_it;            // skipped when the rule (tg_stopped) ended the iteration before
-  const double* gate;     // optional: batch b is skipped when gate[b] <= gate_tol (its iteration has converged)
-  double gate_tol;
   int32_t* status;
 };
 
@@ -240,7 +237,6 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
   using C = TgCfg<BN>;
   if (p.status && *p.status) return;
   if (tg_stopped(p)) return;
-  if (p.gate && p.gate[blockIdx.z] <= p.gate_tol) return;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -282,29 +278,32 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
 
   if (warp == 0) {
     if (lane == 0) {
-      const int ya = (b / p.divA) * p.rowsA_per_batch + m0;
-      const int bb = p.divB > 1 ? b / p.divB : b;
-      const int yb = bb * p.rowsB_per_batch + n0;
+      const int ba = b / p.divA, bb = p.divB > 1 ? b / p.divB : b;
+      // K-major: box at (contraction, row); MN-major: 64 contraction rows x 128 (BN) columns as boxes of 64 x 64, one swizzle
+      // atom each, at (column, contraction)
+      const int a_mn = p.a_mn, b_mn = p.b_mn;
+      const int xa = ba * p.colsA_per_batch + (a_mn ? m0 : 0), ya = ba * p.rowsA_per_batch + (a_mn ? 0 : m0);
+      const int xb = bb * p.colsB_per_batch + (b_mn ? n0 : 0), yb = bb * p.rowsB_per_batch + (b_mn ? 0 : n0);
+      uint32_t s = 0, ph = 1;
+      int t = 0, c = 0;
       for (int it = 0; it < total; ++it) {
-        const int t = it / kchunks, c = it - t * kchunks;
-        const uint32_t s = it % C::NSTAGE, ph = (it / C::NSTAGE) & 1u;
-        if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, p.status)) break;
+        if (!mbar_wait(bar_empty + 8 * s, ph, abort_flag, p.status)) break;
         mbar_expect_tx(bar_full + 8 * s, C::STAGE);
         const int l0 = c * TG_BK;
-        uint8_t* st = smem + s * C::STAGE;
-        // MN-major: 64 contraction rows x 128 (BN) columns as boxes of 64 x 64, one swizzle atom each
-        if (p.a_mn) {
-          for (int j = 0; j < 2; ++j)
-            tma_load_2d(smem_u32(st + j * 8192), &maps.a[t], m0 + j * 64 + (b / p.divA) * p.colsA_per_batch, l0, bar_full + 8 * s);
+        const uint32_t st = smem_u32(smem) + s * C::STAGE;
+        if (a_mn) {
+          for (int j = 0; j < 2; ++j) tma_load_2d(st + j * 8192, &maps.a[t], xa + j * 64, ya + l0, bar_full + 8 * s);
         } else {
-          tma_load_2d(smem_u32(st), &maps.a[t], l0 + (b / p.divA) * p.colsA_per_batch, ya, bar_full + 8 * s);
+          tma_load_2d(st, &maps.a[t], xa + l0, ya, bar_full + 8 * s);
         }
-        if (p.b_mn) {
+        if (b_mn) {
           for (int j = 0; j < BN / 64; ++j)
-            tma_load_2d(smem_u32(st + C::A_BYTES + j * 8192), &maps.b[t], n0 + j * 64 + bb * p.colsB_per_batch, l0, bar_full + 8 * s);
+            tma_load_2d(st + C::A_BYTES + j * 8192, &maps.b[t], xb + j * 64, yb + l0, bar_full + 8 * s);
         } else {
-          tma_load_2d(smem_u32(st + C::A_BYTES), &maps.b[t], l0 + bb * p.colsB_per_batch, yb, bar_full + 8 * s);
+          tma_load_2d(st + C::A_BYTES, &maps.b[t], xb + l0, yb, bar_full + 8 * s);
         }
+        if (++c == kchunks) { c = 0; ++t; }
+        if (++s == C::NSTAGE) { s = 0; ph ^= 1u; }
       }
     }
   } else if (warp == 1) {
@@ -425,9 +424,7 @@ tc_block_kernel(const __grid_constant__ TbMaps maps, const TbTerms tt, const TgP
   using C = TbCfg<K>;
   static_assert(K == 128 || K == 256, "block size");
   if (p.status && *p.status) return;
-  if (p.run_flag && *p.run_flag == 0) return;
   const int b = blockIdx.x;
-  if (p.gate && p.gate[b] <= p.gate_tol) return;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -724,7 +721,6 @@ static bool make_map_2d(CUtensorMap* m, CUtensorMapDataType dt, int esize, const
 // a_mn / b_mn: the A / B arrays hold the operand transposed ([l][m] / [l][n]).  p filled as for tg_launch with
 // M = N = K = k, contiguous k x k blocks in C0 / C / Chi / Clo, no transposed outputs.  Distinct pointers among the
 // terms are found here.
-static std::atomic<int> g_tb_enable{1};
 template <int K>
 static int tb_launch_t(cudaStream_t st, const TbMaps& maps, const TbTerms& tt, const TgParams& p) {
   using C = TbCfg<K>;
@@ -786,15 +782,8 @@ static int tb_launch(cudaStream_t st, int nterms, const uint16_t* const* A, cons
 // (grid: k/32, k/32, nb; block 32 x 8), transposed outputs staged through shared memory.  k % 32 == 0.
 __global__ void __launch_bounds__(256) split_bf16_kernel(const float* __restrict__ X, int k, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
-                                                         uint16_t* __restrict__ tlo, const int* run_flag, const int32_t* status,
-                                                         const double* gate = nullptr, double gate_tol = 0.0) {
-  // runs for every block by default; with run_flag and / or gate: only when *run_flag != 0, or for the blocks
-  // with gate[block] <= gate_tol
+                                                         uint16_t* __restrict__ tlo, const int32_t* status) {
   if (status && *status) return;
-  if (run_flag || gate) {
-    const bool run = (run_flag && *run_flag != 0) || (gate && gate[blockIdx.z] <= gate_tol);
-    if (!run) return;
-  }
   __shared__ uint32_t tile[32][33];
   const size_t base = (size_t)blockIdx.z * k * k;
   const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;

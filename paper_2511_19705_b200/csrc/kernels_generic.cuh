@@ -264,17 +264,8 @@ __device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* s
 }
 
 __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out,
-                                                             float* __restrict__ cnorm, int k, int32_t* status,
-                                                             const double* __restrict__ rn_check, double tol2, int* redo_flag,
-                                                             int* redo_count = nullptr) {
-  // rn_check: squared residual of an iterative inverse per block; the elimination only runs for blocks whose
-  // residual is above tol2 (or not finite) and then raises redo_flag for whoever depends on the result
+                                                             float* __restrict__ cnorm, int k, int32_t* status) {
   if (status && *status) return;
-  if (rn_check) {
-    if (rn_check[blockIdx.x] <= tol2) return;
-    if (threadIdx.x == 0 && redo_flag) *redo_flag = 1;
-    if (threadIdx.x == 0 && redo_count) atomicAdd(redo_count, 1);  // blocks recomputed by elimination, over the run
-  }
   extern __shared__ float sm[];  // 3 k words
   const int tid = threadIdx.x, nt = blockDim.x;
   const float* A0 = Min + (size_t)blockIdx.x * k * k;
@@ -377,10 +368,12 @@ __global__ void quant_kernel(const float* __restrict__ U, long long ld, int rows
 // transform pass: u * (1 / s) + 1.5 * 2^23 rounds to nearest even, the exact division decides where the quotient lies
 // within its error of a half-integer.  Memory-bound: 4 bytes in, up to 9 out per element.  Measured, 3584 x 4096 to codes and
 // dequantised values: 28 + 85 + 3 us as three kernels, 33 us in one.
-// Needs g % 4 == 0, g <= 4 LPG NV, 16-byte aligned rows; the old kernels take every other shape.
+// SRC: fp32, or the bf16 weights themselves where nothing is applied to them (no fp32 copy first).  Groups of more than 1024
+// values (one scale per row, say) take the whole CTA: 7680 rows of 2528 to codes 120 us as three kernels, 40 us here.
+// Needs g % 4 == 0, g <= 4 LPG NV, rows aligned to four values; the old kernels take every other shape.
 // ------------------------------------------------------------------------------------------------
-template <int LPG, int NV>
-__global__ void __launch_bounds__(256) group_quant_kernel(const float* __restrict__ U, long long ld, int rows, int ng, int g, float qmax,
+template <int LPG, int NV, typename SRC>
+__global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict__ U, long long ld, int rows, int ng, int g, float qmax,
                                                           const void* __restrict__ offsets, int off_kind, float* __restrict__ a,
                                                           float* __restrict__ usel, int* __restrict__ idx, float* __restrict__ Delta,
                                                           float* __restrict__ Uhat, int8_t* __restrict__ codes,
@@ -393,7 +386,7 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const float* __restric
   const bool live = w < total;
   const long long wc = live ? w : total - 1;
   const int row = (int)(wc / ng), G = (int)(wc - (long long)row * ng);
-  const float* p = U + row * ld + (long long)G * g;
+  const SRC* p = U + row * ld + (long long)G * g;
   float v[NV][4];
   float best = 0.f, sel = 0.f;
   int bi = 0;
@@ -402,7 +395,15 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const float* __restric
   for (int i = 0; i < NV; ++i) {
     const int e = (l + i * LPG) * 4;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (e < g) q = __ldg(reinterpret_cast<const float4*>(p + e));
+    if constexpr (sizeof(SRC) == 4) {
+      if (e < g) q = __ldg(reinterpret_cast<const float4*>(p + e));
+    } else {
+      if (e < g) {
+        const uint2 h = __ldg(reinterpret_cast<const uint2*>(p + e));
+        q = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xFFFF0000u), __uint_as_float(h.y << 16),
+                        __uint_as_float(h.y & 0xFFFF0000u));
+      }
+    }
     v[i][0] = q.x; v[i][1] = q.y; v[i][2] = q.z; v[i][3] = q.w;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -410,17 +411,27 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const float* __restric
       if (fabsf(v[i][j]) > best) { best = fabsf(v[i][j]); bi = e + j; sel = v[i][j]; }
     }
   }
-  for (int o = LPG / 2; o > 0; o >>= 1) {
+  for (int o = (LPG < 32 ? LPG : 32) / 2; o > 0; o >>= 1) {
     const float ob = __shfl_xor_sync(0xffffffffu, best, o), os = __shfl_xor_sync(0xffffffffu, sel, o);
     const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
     if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; sel = os; }
+  }
+  if constexpr (LPG == 256) {
+    __shared__ float wb[8], ws[8];
+    __shared__ int wi[8];
+    if ((threadIdx.x & 31) == 0) { wb[threadIdx.x >> 5] = best; ws[threadIdx.x >> 5] = sel; wi[threadIdx.x >> 5] = bi; }
+    __syncthreads();
+    best = wb[0]; sel = ws[0]; bi = wi[0];
+#pragma unroll
+    for (int q = 1; q < 8; ++q)
+      if (wb[q] > best || (wb[q] == best && wi[q] < bi)) { best = wb[q]; bi = wi[q]; sel = ws[q]; }
   }
   if (bad && live) raise_status(status, CAFEQ_ERR_NONFINITE);
   if (!live) return;
   const float sc = __fdiv_rn(best, qmax);
   if (l == 0) {
     if (a) a[w] = best;
-    if (usel) usel[w] = (best > 0.f) ? sel : p[0];
+    if (usel) usel[w] = (best > 0.f) ? sel : v[0][0];  // (lane 0 holds the group's first value)
     if (idx) idx[w] = (best > 0.f) ? bi : 0;
     if (scales) scales[w] = sc;
   }
@@ -1047,7 +1058,7 @@ __global__ void __launch_bounds__(256) colnorm_cw_kernel(const float* __restrict
     if (c) c[(size_t)b * k + t] = tot;
     if (cw) {
       const int col = b * k + t;  // position along the transformed axis
-      if (g >= 32) {
+      if (g % 32 == 0) {  // the 32 columns lie in one group
         for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
         if (threadIdx.x == 0) atomicAdd(&cw[col / g], tot);
       } else {

@@ -487,7 +487,7 @@ static LyAux* ly_aux() {
   return &slots[dev];
 }
 // block sizes whose inverse refinement runs on row-major arrays (the transposed split arrays are then free)
-static bool w_mn_expected(int k) { return g_tb_enable.load(std::memory_order_relaxed) && tb_supported(k, 2); }
+static bool w_mn_expected(int k) { return tb_supported(k, 2); }
 
 static void ly_lists(const LyPlan& L, int axis, int transpose, int* out, int* cnt) {
   // matrices whose backward shares (axis, output orientation): singles store gradT plainly, a pair's first factor
@@ -713,7 +713,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     cp.blk0[ns] = L.pair_blk0;
     cp.n = ns;
     cp.X = L.Minv;
-    const int rc = minv_path_tc(st, L.gMinv, L.grad, NB, k, w, status, &cp);
+    const int rc = minv_path_tc(st, L.Minv, L.gMinv, L.grad, NB, k, w, status, &cp);
     if (rc) return rc;
   }
   if (aux && cudaStreamWaitEvent(st, aux->join, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;

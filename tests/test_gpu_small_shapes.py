@@ -78,3 +78,39 @@ def test_ste_edges(cq, k, group, shape):
     f = orc.single_forward(w64(Wb), M, 4, group, "in")
     assert abs(out["losses"][1].item() - f["L2"]) <= 1e-4 * f["L2"]
     assert rel_err(out["gradM"].cpu().numpy(), orc.single_grad_ste(w64(Wb), f, 4, group, "in")) <= 1e-4  # as at whole tiles
+
+
+# groups as wide as the row: the widest a warp holds, the first a CTA takes, its variants' edges, and beyond (the separate kernels)
+@pytest.mark.parametrize("d_out,d_in", [(3, 1024), (3, 1032), (2, 2048), (2, 4104), (2, 8192), (1, 16384), (1, 16392)])
+def test_rtn_whole_rows(cq, d_out, d_in):
+    Wb = syn.weight_student_t(d_out, d_in, 7, 2, 10.0)
+    Q = orc.quant_sym(w64(Wb), 4, 0)
+    for T in (None, f32_dev(syn.identity_blocks(d_in, 1))):  # bf16 source; fp32 source (the identity is exact)
+        codes, scales = cq.cafeq_rtn(to_dev(Wb), T, bits=4, group=0, tblock=0 if T is None else 1)
+        assert np.array_equal(codes.cpu().numpy().astype(np.int32), Q["q"]) and np.array_equal(scales.cpu().numpy(), Q["s"])
+
+
+# elimination in registers: pivoting across both halves of the rows, exact permutations, the singular block
+@pytest.mark.parametrize("k", [32, 64])
+def test_small_inverse(cq, k):
+    rng = np.random.default_rng(k)
+    nb = 6
+    M = rng.standard_normal((nb, k, k))
+    M[0] = np.eye(k)[::-1]                                   # every pivot off the diagonal
+    M[1] = np.eye(k)[rng.permutation(k)] * np.where(rng.random(k) < 0.5, -1.0, 1.0)
+    M[2] = syn.perturbed_blocks(1, k, 3, 0.1)[0]
+    M[3, 0, 0] = 0.0
+    M = orc.round_bf16(M.astype(np.float32)).astype(np.float64)
+    W = torch.zeros((64, nb * k), dtype=torch.bfloat16, device="cuda")
+    for flags in (cq.FLAG_NO_GRAD, cq.FLAG_NO_GRAD | cq.FLAG_GENERIC):
+        out = cq.cafeq_proxy_loss_fwd_bwd(W, f32_dev(M), bits=4, group=0, flags=flags, want_minv=True)
+        assert int(out["status"].item()) == 0
+        X = out["Minv"].cpu().numpy().astype(np.float64)
+        for b in range(nb):
+            ref = np.linalg.inv(M[b])
+            # backward error of elimination: k 2^-24 times the condition number (growth under partial pivoting is small)
+            assert np.linalg.norm(X[b] - ref, 2) <= 4 * k * 2.0 ** -24 * np.linalg.cond(M[b]) * np.linalg.norm(ref, 2)
+        assert np.array_equal(X[:2], np.linalg.inv(M[:2]))
+    M[4, :, 5] = 0.0
+    out = cq.cafeq_proxy_loss_fwd_bwd(W, f32_dev(M), bits=4, group=0, flags=cq.FLAG_NO_GRAD)
+    assert int(out["status"].item()) == 5                   # singular block
