@@ -1355,6 +1355,23 @@ static int opgrad_in_tc(cudaStream_t st, const uint16_t* Ah, const uint16_t* Al,
   return CAFEQ_OK;
 }
 
+// straight-through gradient of one factor as operand splits (ste_grad_split_kernel); gX has one column per r replicas
+static bool ste_split_ok(int g) { return g % 4 == 0 && g <= 1024; }
+static void launch_ste_split(cudaStream_t st, const MatWS& m, const float* gX, long long ldg, const Geo& G, int k, int r, float qmax,
+                             uint16_t* hi, uint16_t* lo, int32_t* status) {
+  const long long groups = (long long)G.d_out * G.ng;
+#define SGS(L, N)                                                                                                              \
+  CQ_LAUNCH((ste_grad_split_kernel<L, N>), (unsigned)((groups * L + 255) / 256), 256, 0, st, m.U, gX, ldg, G.d_out, G.ng, G.g, k, r, \
+            m.a, m.usel, m.idx, qmax, hi, lo, status)
+  if (G.g <= 32) SGS(8, 1);
+  else if (G.g <= 64) SGS(16, 1);
+  else if (G.g <= 128) SGS(32, 1);
+  else if (G.g <= 256) SGS(32, 2);
+  else if (G.g <= 512) SGS(32, 4);
+  else SGS(32, 8);
+#undef SGS
+}
+
 static bool dense_ok(const Geo& G1, const Geo& G2) {
   return G1.d_out % 64 == 0 && G1.d_in % 64 == 0 && G2.d_out % 64 == 0 && G2.d_in % 64 == 0 && G1.k % 32 == 0;
 }
@@ -1534,45 +1551,43 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     // its transpose are in p.dn.Ph/Pl/PTh/PTl; the quantiser passes gradients through except for its scale,
     // whose dependence on the group's arg-max entry is kept.
     DenseWS& w = p.dn;
-    {  // g Vhat' [d3, h] = 2 R^T Uhat^T, then one copy per replica of every inner block
-      launch_split_rect(st, p.m1.E, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status);
+    {  // g Vhat' [d3, h] = 2 R^T Uhat^T (one column for the replicas of an inner column)
       const uint16_t* a[3] = {w.PTh, w.PTl, w.PTh};
       const uint16_t* b[3] = {w.Awh, w.Awh, w.Awl};
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
       launch_dense_tc(st, 3, a, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, status);
-      CQ_LAUNCH(expand_cols_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f, w.V);
     }
-    {  // g Uhat [h, d1] = 2 fold(Vhat^T) R^T
-      dim3 grid((w.d3 + 31) / 32, w.h / 32);
-      CQ_LAUNCH(fold_transpose_kernel, grid, dim3(32, 8), 0, st, p.m2.E, w.d3, w.h, w.k, w.r, w.Bf);
-      launch_split_rect(st, w.Bf, w.h, w.d3, w.d3, 1.f, nullptr, nullptr, nullptr, w.Yh, w.Yl, nullptr, nullptr, status);
-      const uint16_t* a[3] = {w.Yh, w.Yl, w.Yh};
+    {  // g Uhat [h, d1] = 2 fold(Vhat^T) R^T (the folded splits are read as they are stored: an MN-major operand costs the
+      // product 10 %, 14 us, where folding, transposing and splitting again took 60)
+      const uint16_t* a[3] = {w.Vh, w.Vl, w.Vh};
       const uint16_t* b[3] = {w.Ph, w.Ph, w.Pl};
       DenseOut o;
       o.C = w.U; o.ldc = w.d1;
-      launch_dense_tc(st, 3, a, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, status);
+      launch_dense_tc(st, 3, a, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, status, 1);
     }
-    const long long n1w = (long long)G1.d_out * G1.ng, n2w = (long long)G2.d_out * G2.ng;
-    CQ_LAUNCH(ste_scale_path_kernel, (unsigned)((n1w * 32 + 255) / 256), 256, 0, st, p.m1.U, w.U, G1.d_in, G1.d_out, G1.ng, G1.g,
-              p.m1.a, p.m1.usel, qmax_of(d1->bits), nullptr, CAFEQ_OFFSETS_NONE, G1.d_in, p.m1.coef, status);
-    CQ_LAUNCH(add_argmax_kernel, grid_for(n1w), 256, 0, st, w.U, G1.d_in, G1.d_out, G1.ng, G1.g, p.m1.coef, p.m1.idx, status);
-    CQ_LAUNCH(ste_scale_path_kernel, (unsigned)((n2w * 32 + 255) / 256), 256, 0, st, p.m2.U, w.V, G2.d_in, G2.d_out, G2.ng, G2.g,
-              p.m2.a, p.m2.usel, qmax_of(d2->bits), nullptr, CAFEQ_OFFSETS_NONE, G2.d_in, p.m2.coef, status);
-    CQ_LAUNCH(add_argmax_kernel, grid_for(n2w), 256, 0, st, w.V, G2.d_in, G2.d_out, G2.ng, G2.g, p.m2.coef, p.m2.idx, status);
     if (!tc) {
       CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, gradM, 0.f, kk);
       CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, p.gMinv, 0.f, kk);
     }
-    const bool og_tc = tc && ((uintptr_t)W1 % 16 == 0) && (G1.ld % 8 == 0) && ((uintptr_t)W2 % 16 == 0) && (G2.ld % 8 == 0) && G1.r == 1;
+    const bool og_tc = tc && ((uintptr_t)W1 % 16 == 0) && (G1.ld % 8 == 0) && ((uintptr_t)W2 % 16 == 0) && (G2.ld % 8 == 0) && G1.r == 1 &&
+                       ste_split_ok(G1.g) && ste_split_ok(G2.g);
     if (og_tc) {
       // U side (operator M^T): gradM[b][m][n] = sum_c W1[b k + m][c] gU[b k + n][c]
-      launch_split_rect(st, w.U, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status);
+      launch_ste_split(st, p.m1, w.U, w.d1, G1, k, 1, qmax_of(d1->bits), w.Awh, w.Awl, status);
       if ((p.err = opgrad_out_tc(st, (const uint16_t*)W1, G1.ld, w.Awh, w.Awl, G1.nbT, k, G1.d_in, gradM, status))) return;
       // V side (operator Minv): gMinv[b][i][j] = sum over replicas and rows o of gV[o][.. + i] W2[o][.. + j]
-      launch_split_rect(st, w.V, w.d3, w.rh, w.rh, 1.f, nullptr, nullptr, nullptr, p.gVh, p.gVl, nullptr, nullptr, status);
+      launch_ste_split(st, p.m2, w.X0T, w.h, G2, k, G2.r, qmax_of(d2->bits), p.gVh, p.gVl, status);
       if ((p.err = opgrad_in_tc(st, p.gVh, p.gVl, (const uint16_t*)W2, G2.ld, G1.nbT, G2.r, k, G2.d_out, p.gMinv, status))) return;
     } else {
+      CQ_LAUNCH(expand_cols_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f, w.V);
+      const long long n1w = (long long)G1.d_out * G1.ng, n2w = (long long)G2.d_out * G2.ng;
+      CQ_LAUNCH(ste_scale_path_kernel, (unsigned)((n1w * 32 + 255) / 256), 256, 0, st, p.m1.U, w.U, G1.d_in, G1.d_out, G1.ng, G1.g,
+                p.m1.a, p.m1.usel, qmax_of(d1->bits), nullptr, CAFEQ_OFFSETS_NONE, G1.d_in, p.m1.coef, status);
+      CQ_LAUNCH(add_argmax_kernel, grid_for(n1w), 256, 0, st, w.U, G1.d_in, G1.d_out, G1.ng, G1.g, p.m1.coef, p.m1.idx, status);
+      CQ_LAUNCH(ste_scale_path_kernel, (unsigned)((n2w * 32 + 255) / 256), 256, 0, st, p.m2.U, w.V, G2.d_in, G2.d_out, G2.ng, G2.g,
+                p.m2.a, p.m2.usel, qmax_of(d2->bits), nullptr, CAFEQ_OFFSETS_NONE, G2.d_in, p.m2.coef, status);
+      CQ_LAUNCH(add_argmax_kernel, grid_for(n2w), 256, 0, st, w.V, G2.d_in, G2.d_out, G2.ng, G2.g, p.m2.coef, p.m2.idx, status);
       launch_opgrad(st, w.U, G1.d_in, W1, 1, G1.ld, G1, gradM, 1, 1.f, status);    // U side: operator M^T
       launch_opgrad(st, w.V, G2.d_in, W2, 1, G2.ld, G2, p.gMinv, 0, 1.f, status);  // V side: operator Minv
     }

@@ -15,7 +15,9 @@ namespace cafeq {
 // (row-major) and YT (transposed, holding hi + lo: used only as a starting guess).  h3 / t3: optional third term
 // bf16(x - hi - lo) in row-major / transposed order (hi + lo + third carries 24 significand bits: products over the
 // three-way split reach fp32 accuracy).
-// One 32 x 32 tile per CTA (grid: ceil(C/32), ceil(R/32); block 32 x 8).
+// One 64 x 64 tile per CTA (grid: C / 64, R / 64; every caller's sizes are multiples of 64).  Memory-bound: two values per
+// thread and access, so that every row of a tile is a 128-byte line in both orders (one value each, 32 x 32 tiles: 22 us for
+// the two row-major terms of 3584 x 2048, 9 us here).
 __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict__ X, int R, int C, long long ld, float scale,
                                                          const double* __restrict__ inv_scale, float* __restrict__ Y,
                                                          float* __restrict__ YT, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
@@ -23,51 +25,56 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
                                                          uint16_t* __restrict__ t3 = nullptr) {
   if (status && *status) return;
-  __shared__ uint32_t tile[32][33];
-  __shared__ uint16_t tile3[32][34];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
+  __shared__ uint32_t tile[64][65];
+  __shared__ uint16_t tile3[64][66];
+  const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   float sc = scale;
   if (inv_scale) sc = (float)((double)scale / fmax(*inv_scale, 1e-300));
+  const bool trans = thi || tlo || YT;
+  float2 x2[8];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = r0 + ty + 8 * q, c = c0 + tx;
-    uint32_t packed = 0;
-    if (r < R && c < C) {
-      const float x = sc * X[(long long)r * ld + c];
-      const __nv_bfloat16 h = __float2bfloat16_rn(x);
-      const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
-      const uint16_t hb = __bfloat16_as_ushort(h), lb = __bfloat16_as_ushort(l);
-      if (Y) Y[(long long)r * C + c] = x;
-      if (hi) hi[(long long)r * C + c] = hb;
-      if (lo) lo[(long long)r * C + c] = lb;
-      packed = (uint32_t)hb | ((uint32_t)lb << 16);
+  for (int q = 0; q < 8; ++q) x2[q] = __ldg(reinterpret_cast<const float2*>(X + (long long)(r0 + ty + 8 * q) * ld + c0 + 2 * tx));
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = ty + 8 * q;
+    const long long o = (long long)(r0 + i) * C + c0 + 2 * tx;
+    const float x[2] = {sc * x2[q].x, sc * x2[q].y};
+    uint32_t hw = 0, lw = 0, w3 = 0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(x[e]);
+      const float d = x[e] - __bfloat162float(h);
+      const __nv_bfloat16 l = __float2bfloat16_rn(d);
+      const uint32_t hb = __bfloat16_as_ushort(h), lb = __bfloat16_as_ushort(l);
+      hw |= hb << (16 * e);
+      lw |= lb << (16 * e);
+      if (trans) tile[i][2 * tx + e] = hb | (lb << 16);
       if (h3 || t3) {
-        const uint16_t b3 = __bfloat16_as_ushort(__float2bfloat16_rn((x - __bfloat162float(h)) - __bfloat162float(l)));
-        if (h3) h3[(long long)r * C + c] = b3;
-        tile3[ty + 8 * q][tx] = b3;
+        const uint32_t b3 = __bfloat16_as_ushort(__float2bfloat16_rn(d - __bfloat162float(l)));
+        w3 |= b3 << (16 * e);
+        tile3[i][2 * tx + e] = (uint16_t)b3;
       }
     }
-    tile[ty + 8 * q][tx] = packed;
+    if (Y) *reinterpret_cast<float2*>(Y + o) = make_float2(x[0], x[1]);
+    if (hi) *reinterpret_cast<uint32_t*>(hi + o) = hw;
+    if (lo) *reinterpret_cast<uint32_t*>(lo + o) = lw;
+    if (h3) *reinterpret_cast<uint32_t*>(h3 + o) = w3;
   }
+  if (!trans && !t3) return;
   __syncthreads();
-  if (t3) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + ty + 8 * q, r = r0 + tx;
-      if (r < R && c < C) t3[(long long)c * R + r] = tile3[tx][ty + 8 * q];
-    }
-  }
-  if (thi || tlo || YT) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = c0 + ty + 8 * q, r = r0 + tx;
-      if (r < R && c < C) {
-        const uint32_t v = tile[tx][ty + 8 * q];
-        if (thi) thi[(long long)c * R + r] = (uint16_t)(v & 0xFFFFu);
-        if (tlo) tlo[(long long)c * R + r] = (uint16_t)(v >> 16);
-        if (YT) YT[(long long)c * R + r] = __uint_as_float(v << 16) + __uint_as_float(v & 0xFFFF0000u);
-      }
+  for (int q = 0; q < 8; ++q) {
+    const int j = ty + 8 * q;
+    const long long o = (long long)(c0 + j) * R + r0 + 2 * tx;
+    if (t3) *reinterpret_cast<uint32_t*>(t3 + o) = (uint32_t)tile3[2 * tx][j] | ((uint32_t)tile3[2 * tx + 1][j] << 16);
+    if (trans) {
+      const uint32_t v0 = tile[2 * tx][j], v1 = tile[2 * tx + 1][j];
+      if (thi) *reinterpret_cast<uint32_t*>(thi + o) = (v0 & 0xFFFFu) | (v1 << 16);
+      if (tlo) *reinterpret_cast<uint32_t*>(tlo + o) = (v0 >> 16) | (v1 & 0xFFFF0000u);
+      if (YT)
+        *reinterpret_cast<float2*>(YT + o) = make_float2(__uint_as_float(v0 << 16) + __uint_as_float(v0 & 0xFFFF0000u),
+                                                         __uint_as_float(v1 << 16) + __uint_as_float(v1 & 0xFFFF0000u));
     }
   }
 }
@@ -170,6 +177,86 @@ __global__ void add_argmax_kernel(float* __restrict__ gX, long long ld, int rows
     const long long row = w / ng;
     const int G = (int)(w - row * ng);
     gX[row * ld + (long long)G * g + idx[w]] += coef[w];
+  }
+}
+
+// Gradient with respect to the quantiser's input, ready as an operand: gX (d loss / d Uhat, fp32, pitch ldg) passes through,
+// the scale's part sign(U at arg-max) / qmax * sum_e gX_e (q_e - U_e / s) is added at the group's arg-max entry, and the sum is
+// written as a bf16 hi / lo split.  U dense [rows, ng g]; r > 1: gX holds one column for the r replicas of each inner column
+// (block b of k columns reads block b / r).  Memory-bound, 8 bytes read and 4 written per value: LPG lanes own a group and keep
+// it in registers.  3584 x 4096 + 2048 x 3584: expansion, scale path with two divisions per value, arg-max addition and split
+// 190 us as seven launches, 60 us here as two.
+template <int LPG, int NV>
+__global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* __restrict__ U, const float* __restrict__ gX, long long ldg, int rows,
+                                                             int ng, int g, int k, int r, const float* __restrict__ a,
+                                                             const float* __restrict__ usel, const int* __restrict__ idx, float qmax,
+                                                             uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, const int32_t* status) {
+  if (status && *status) return;
+  const int l = threadIdx.x % LPG;
+  const long long total = (long long)rows * ng;
+  const long long w = (blockIdx.x * 256ll + threadIdx.x) / LPG;
+  const bool live = w < total;
+  const long long wc = live ? w : total - 1;
+  const int row = (int)(wc / ng), G = (int)(wc - (long long)row * ng);
+  const long long u0 = (long long)row * ng * g + (long long)G * g;
+  const float* gr = gX + (long long)row * ldg;
+  float4 u4[NV], d4[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int e = (l + i * LPG) * 4;
+    u4[i] = d4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e < g) {
+      u4[i] = __ldg(reinterpret_cast<const float4*>(U + u0 + e));
+      int col = G * g + e;
+      if (r > 1) {
+        const int b = col / k;
+        col = (b / r) * k + (col - b * k);
+      }
+      d4[i] = __ldg(reinterpret_cast<const float4*>(gr + col));
+    }
+  }
+  const float av = a[wc], us = usel[wc];
+  const int am = idx[wc];
+  const float s = __fdiv_rn(av, qmax);
+  const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
+  const bool fast = rs < 3.0e38f;
+  const float win = 0.5f - (qmax + 1.f) * 1.0e-6f;
+  constexpr float MAGIC = 12582912.f;
+  float sum = 0.f;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const float u[4] = {u4[i].x, u4[i].y, u4[i].z, u4[i].w}, dv[4] = {d4[i].x, d4[i].y, d4[i].z, d4[i].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      // U / s with one correction step; the quotient's rounding as in the quantiser (exact division next to a half-integer)
+      const float x0 = u[j] * rs;
+      float x = fmaf(fmaf(-s, x0, u[j]), rs, x0);
+      float q = (x + MAGIC) - MAGIC;
+      if (!(fabsf(x - q) <= win) || !fast) {
+        x = (s > 0.f) ? __fdiv_rn(u[j], s) : 0.f;
+        q = fminf(fmaxf(rintf(x), -qmax), qmax);
+      }
+      sum = fmaf(dv[j], q - x, sum);
+    }
+  }
+  for (int o = LPG / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (!live) return;
+  const float cf = sum * ((us > 0.f) ? 1.f : ((us < 0.f) ? -1.f : 0.f)) / qmax;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int e = (l + i * LPG) * 4;
+    if (e >= g) break;
+    const float dv[4] = {d4[i].x, d4[i].y, d4[i].z, d4[i].w};
+    uint32_t hw[2] = {0u, 0u}, lw[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float x = dv[j] + ((e + j == am) ? cf : 0.f);
+      const __nv_bfloat16 h = __float2bfloat16_rn(x);
+      hw[j >> 1] |= (uint32_t)__bfloat16_as_ushort(h) << (16 * (j & 1));
+      lw[j >> 1] |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(h))) << (16 * (j & 1));
+    }
+    *reinterpret_cast<uint2*>(hi + u0 + e) = make_uint2(hw[0], hw[1]);
+    *reinterpret_cast<uint2*>(lo + u0 + e) = make_uint2(lw[0], lw[1]);
   }
 }
 

@@ -19,12 +19,12 @@ struct DenseOut {
   int stop_it = 0;
 };
 
-// A operands are [M, K] row-major, B operands [N, K] row-major; nterms pairs (A[t], B[t]).
+// A operands are [M, K] row-major (a_mn: [K, M]), B operands [N, K] row-major; nterms pairs (A[t], B[t]).
 static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A, const uint16_t* const* B, int M, int N, int K,
-                           float alpha, float beta, float gamma, const DenseOut& o, int32_t* status) {
+                           float alpha, float beta, float gamma, const DenseOut& o, int32_t* status, int a_mn = 0) {
   TgOperand oa[TG_MAX_TERMS], ob[TG_MAX_TERMS];
   for (int t = 0; t < nterms; ++t) {
-    oa[t] = TgOperand{A[t], M, K, K};
+    oa[t] = a_mn ? TgOperand{A[t], K, M, M} : TgOperand{A[t], M, K, K};
     ob[t] = TgOperand{B[t], N, K, K};
   }
   TgParams p;
@@ -38,6 +38,7 @@ static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A
   p.C = o.C; p.ldc = o.ldc;
   p.Chi = o.Chi; p.Clo = o.Clo; p.Cthi = o.Cthi; p.Ctlo = o.Ctlo;
   p.sq = o.sq; p.sq_stride = 0;
+  p.a_mn = a_mn;
   p.stop_sq = o.stop_sq; p.stop_it = o.stop_it;
   p.status = status;
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -47,8 +48,7 @@ static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A
 static void launch_split_rect(cudaStream_t st, const float* X, int R, int C, long long ld, float scale, const double* inv_scale,
                               float* Y, float* YT, uint16_t* hi, uint16_t* lo, uint16_t* thi, uint16_t* tlo, const int32_t* status,
                               uint16_t* h3 = nullptr, uint16_t* t3 = nullptr) {
-  dim3 grid((C + 31) / 32, (R + 31) / 32);
-  CQ_LAUNCH(split_rect_kernel, grid, dim3(32, 8), 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3);
+  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3);
 }
 
 // The same product with both operands split three ways (x = x1 + x2 + x3, 24 significand bits): the six terms down to
@@ -241,10 +241,12 @@ static void dense_product(cudaStream_t st, const float* U, const float* V, Dense
   launch_split_rect(st, P, w.d1, w.d3, w.d3, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status, w.P3, w.PT3);
 }
 
-// *sq += || Uhat_exp^T Vhat^T - P ||_F^2 ; optionally stores the residual R [d1, d3]
+// *sq += || Uhat_exp^T Vhat^T - P ||_F^2 ; optionally stores the residual R [d1, d3].  keep_splits: leaves the residual and its
+// transpose in w.Ph / Pl / PTh / PTl and Uhat, as stored, in w.Awh / Awl (Vhat, replicas folded, is in w.Vh / Vl either way)
 static void dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, const float* P, DenseWS& w, double* sq, float* R,
                       int32_t* status, bool keep_splits = false) {
-  launch_split_rect(st, Uhat, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.UTh, w.UTl, status);
+  launch_split_rect(st, Uhat, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, keep_splits ? w.Awh : nullptr,
+                    keep_splits ? w.Awl : nullptr, w.UTh, w.UTl, status);
   launch_fold_split(st, Vhat, w, w.Vh, w.Vl, nullptr, status);
   const uint16_t* a[3] = {w.UTh, w.UTl, w.UTh};
   const uint16_t* b[3] = {w.Vh, w.Vh, w.Vl};
