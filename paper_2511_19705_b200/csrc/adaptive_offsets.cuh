@@ -17,6 +17,7 @@ constexpr float LEARN_LAMBDA = 0.5f;  // final weight of the push towards {0, 1}
 // rho = x - floor(x), x = fl(u / s) (the quantiser's own fp32 quotient)
 __global__ void offsets_init_kernel(const float* __restrict__ U, int rows, int cols, int g, const float* __restrict__ a, float qmax,
                                     float* __restrict__ rho) {
+  pdl_enter();
   const int ng = cols / g;
   const long long n = (long long)rows * cols;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -29,6 +30,7 @@ __global__ void offsets_init_kernel(const float* __restrict__ U, int rows, int c
 
 // Bf[B k + j][y] = sum_rep V[y][(B r + rep) k + j]   (V [d3, r h] -> Bf [h, d3]); any k
 __global__ void fold_t_any_kernel(const float* __restrict__ V, int d3, int h, int k, int r, float* __restrict__ Bf) {
+  pdl_enter();
   const long long n = (long long)h * d3;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const int l = (int)(e / d3), y = (int)(e - (long long)l * d3);
@@ -41,6 +43,7 @@ __global__ void fold_t_any_kernel(const float* __restrict__ V, int d3, int h, in
 
 // out[row] = scale * sum_c X[row][c]^2, one warp per row
 __global__ void row_sumsq_kernel(const float* __restrict__ X, int rows, int cols, float scale, float* __restrict__ out) {
+  pdl_enter();
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= rows) return;
@@ -60,6 +63,7 @@ __global__ void row_sumsq_kernel(const float* __restrict__ X, int rows, int cols
 __global__ void offsets_direction_kernel(const float* gX /* may be d_rho */, const float* __restrict__ U, int rows, int cols, int g,
                                          const float* __restrict__ a, float qmax, const float* __restrict__ H, int hrow, int k,
                                          int r, float* d_rho, float* __restrict__ d_val) {
+  pdl_enter();
   const int ng = cols / g;
   const long long n = (long long)rows * cols;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -82,6 +86,7 @@ __global__ void offsets_direction_kernel(const float* gX /* may be d_rho */, con
 // rho <- clip(rho - alpha d, 0, 1) with the exact line-search step alpha = <R, D> / <D, D> (0 when D = 0)
 __global__ void offsets_step_kernel(float* __restrict__ rho, const float* __restrict__ d_rho, long long n, const double* __restrict__ rd,
                                     const double* __restrict__ dd) {
+  pdl_enter();
   const float alpha = (*dd > 0.0) ? (float)(*rd / *dd) : 0.f;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
     rho[e] = fminf(fmaxf(rho[e] - alpha * d_rho[e], 0.f), 1.f);
@@ -89,6 +94,7 @@ __global__ void offsets_step_kernel(float* __restrict__ rho, const float* __rest
 
 // rho <- clip(rho + lam (2 rho - 1), 0, 1)
 __global__ void offsets_push_kernel(float* __restrict__ rho, long long n, float lam) {
+  pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const float rv = rho[e];
     rho[e] = fminf(fmaxf(rv + lam * (2.f * rv - 1.f), 0.f), 1.f);
@@ -96,6 +102,7 @@ __global__ void offsets_push_kernel(float* __restrict__ rho, long long n, float 
 }
 
 __global__ void harden_kernel(float* __restrict__ rho, long long n) {
+  pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
     rho[e] = (rho[e] >= 0.5f) ? 1.f : 0.f;
 }

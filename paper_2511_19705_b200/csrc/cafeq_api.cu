@@ -26,11 +26,12 @@ namespace cafeq {
 // Process-wide count of kernel launches made by this library (read by benchmarks through
 // cafeq_debug_launch_count; it has no effect on any result).
 static std::atomic<long long> g_launches{0};
-#define CQ_LAUNCH(kernel, grid, block, smem, st, ...)       \
-  do {                                                      \
-    g_launches.fetch_add(1, std::memory_order_relaxed);     \
-    kernel<<<grid, block, smem, st>>>(__VA_ARGS__);         \
+#define CQ_LAUNCH_IF(overlap, kernel, grid, block, smem, st, ...)       \
+  do {                                                                  \
+    g_launches.fetch_add(1, std::memory_order_relaxed);                 \
+    launch_pdl_if(overlap, kernel, grid, block, smem, st, __VA_ARGS__); \
   } while (0)
+#define CQ_LAUNCH(kernel, grid, block, smem, st, ...) CQ_LAUNCH_IF(true, kernel, grid, block, smem, st, __VA_ARGS__)
 
 // Optional per-launch timing of selected kernels with CUDA events on the launching stream (benchmarks
 // only; off unless cafeq_debug_timer_begin was called).  Kinds: 1 transform pass (shape-agnostic kernels),
@@ -291,6 +292,7 @@ static int launch_kk_tc(cudaStream_t st, int nterms, const uint16_t* const* A, c
 }
 
 __global__ void zero_ns_kernel(double* rn, int n, int* flag) {
+  pdl_enter();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) rn[i] = 0.0;
   if (i == 0) *flag = 0;
@@ -310,7 +312,7 @@ static void launch_split(cudaStream_t st, const float* X, int k, long long n, ui
 // w.Xh / Xl (and XTh / XTl unless w.mn) [w.cur].
 // eq4 (k = 128, 256): where the kernel puts the column norms / group weights, and what it ticks.
 static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k, bool warm, KkWS& w, int32_t* status,
-                      bool prepped = false, bool splits_kept = false, const NsParams* eq4 = nullptr) {
+                      bool prepped = false, bool splits_kept = false, const NsParams* eq4 = nullptr, bool overlap = true) {
   w.cur = 0;
   w.mn = tb_supported(k, 2);
   if (!w.mn) {
@@ -334,7 +336,7 @@ static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k,
   np.redo_count = w.redo_total;
   np.status = status;
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  const int rc = ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np);
+  const int rc = ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np, overlap);
   kt_end(ti, st);
   return rc;
 }
@@ -342,7 +344,7 @@ static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k,
 // G -= X^T Gx X^T for every block; X = Minv.  k = 128, 256: on the tensor cores from its splits in w[w.cur], three-term
 // products; 32, 64: in fp32.  Gx = dL/dMinv: fp32 [nb, k, k], or (scaled) formed from X by the kernel itself.
 static int minv_path_tc(cudaStream_t st, const float* X, const float* Gx, float* G, int nb, int k, KkWS& w, int32_t* status,
-                        const ChainParams* scaled = nullptr) {
+                        const ChainParams* scaled = nullptr, bool overlap = true) {
   ChainParams cp;
   memset(&cp, 0, sizeof(cp));
   if (scaled) cp = *scaled;
@@ -350,7 +352,7 @@ static int minv_path_tc(cudaStream_t st, const float* X, const float* Gx, float*
     cp.G = Gx;
     cp.status = status;
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return kk_chain_launch(st, KK_MINV_PATH, w.Xh[w.cur], w.Xl[w.cur], G, nb, k, cp);
+    return kk_chain_launch(st, KK_MINV_PATH, w.Xh[w.cur], w.Xl[w.cur], G, nb, k, cp, overlap);
   }
   if (k == 32) CQ_LAUNCH(small_chain_kernel<32>, nb, 64, 0, st, X, Gx, cp.A[0], cp.Agrp[0], cp.g[0], cp.scale[0], G, status);
   else CQ_LAUNCH(small_chain_kernel<64>, nb, 256, 0, st, X, Gx, cp.A[0], cp.Agrp[0], cp.g[0], cp.scale[0], G, status);
@@ -360,14 +362,14 @@ static int minv_path_tc(cudaStream_t st, const float* X, const float* Gx, float*
 // Orthonormality penalty of nb blocks from the splits of the fp32 parameters (fused kernel, k = 128 / 256):
 // sq[b * sq_stride] += ||M_b M_b^T - I||_F^2 and, with want_out, out = (M M^T - I) M.
 static int penalty_tc(cudaStream_t st, const uint16_t* Mh, const uint16_t* Ml, float* out, bool want_out, double* sq, int sq_stride,
-                      int nb, int k, int32_t* status) {
+                      int nb, int k, int32_t* status, bool overlap = true) {
   ChainParams cp;
   memset(&cp, 0, sizeof(cp));
   cp.sq = sq; cp.sq_stride = sq_stride;
   cp.want_out = want_out ? 1 : 0;
   cp.status = status;
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  return kk_chain_launch(st, KK_PENALTY, Mh, Ml, out, nb, k, cp);
+  return kk_chain_launch(st, KK_PENALTY, Mh, Ml, out, nb, k, cp, overlap);
 }
 
 static void launch_absmax(cudaStream_t st, const float* U, long long ld, const Geo& G, float* a, float* usel, int* idx,
@@ -546,6 +548,7 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
 }
 
 __global__ void bf16_to_f32_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols, float* __restrict__ U) {
+  pdl_enter();
   const long long n = (long long)rows * cols;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     int row = (int)(e / cols), col = (int)(e - (long long)row * cols);
@@ -555,6 +558,7 @@ __global__ void bf16_to_f32_kernel(const uint16_t* __restrict__ W, long long ld,
 
 __global__ void resid_sq_kernel(float* __restrict__ R, const float* __restrict__ P, long long n, double* acc,
                                 const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ double red[32];
   double local = 0.0;
@@ -567,7 +571,8 @@ __global__ void resid_sq_kernel(float* __restrict__ R, const float* __restrict__
   if (threadIdx.x == 0) atomicAdd(acc, s);
 }
 
-__global__ void store_sqrt_kernel(const double* acc, float* out) { *out = (float)sqrt(*acc); }
+__global__ void store_sqrt_kernel(const double* acc, float* out) {
+  pdl_enter(); *out = (float)sqrt(*acc); }
 
 // ------------------------------------------------------------------------------------------------
 // per-matrix scratch

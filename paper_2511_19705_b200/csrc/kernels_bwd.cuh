@@ -431,6 +431,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
   }
 
   // ---------------------------------------------------------------- teardown
+  pdl_release();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -442,6 +443,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
 
 template <int FORM, int K, int SWAP, int F16>
 __global__ void __launch_bounds__(BW_THREADS, 1) bd_bwd_kernel(const __grid_constant__ BwMaps maps, const __grid_constant__ BwMulti mp) {
+  pdl_wait();
   bd_bwd_body<FORM, K, SWAP, F16>(maps, mp, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -451,6 +453,7 @@ template <int K, int SWAP_IN, int SWAP_OUT>
 __global__ void __launch_bounds__(BW_THREADS, 1)
 bd_bwd_dual_kernel(const __grid_constant__ BwMaps maps_in, const __grid_constant__ BwMulti mp_in,
                    const __grid_constant__ BwMaps maps_out, const __grid_constant__ BwMulti mp_out, const int n_in) {
+  pdl_wait();
   if ((int)blockIdx.x < n_in) bd_bwd_body<BW_IN, K, SWAP_IN, 1>(maps_in, mp_in, (int)blockIdx.x, n_in);
   else bd_bwd_body<BW_OUT, K, SWAP_OUT, 1>(maps_out, mp_out, (int)blockIdx.x - n_in, (int)gridDim.x - n_in);
 }
@@ -503,7 +506,7 @@ static int bw_launch_t(cudaStream_t st, const BwMaps& maps, BwMulti mp, int min_
   if (want < majors) want = majors;
   if (want > total) want = total;
   const int grid = want < 148 ? (int)want : 148;
-  bd_bwd_kernel<FORM, K, SWAP, F16><<<grid, BW_THREADS, C::SMEM, st>>>(maps, mp);
+  launch_pdl(bd_bwd_kernel<FORM, K, SWAP, F16>, grid, BW_THREADS, C::SMEM, st, maps, mp);
   return CAFEQ_OK;
 }
 
@@ -567,7 +570,7 @@ static int bw_launch_many(cudaStream_t st, int axis_in, int k, int transpose_out
 }
 
 template <int K, int SWAP_IN, int SWAP_OUT>
-static int bw_launch_dual_t(cudaStream_t st, const BwMaps& mi, BwMulti pi, const BwMaps& mo, BwMulti po) {
+static int bw_launch_dual_t(cudaStream_t st, const BwMaps& mi, BwMulti pi, const BwMaps& mo, BwMulti po, bool overlap) {
   using C = BwCfg<K, 1>;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(bd_bwd_dual_kernel<K, SWAP_IN, SWAP_OUT>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
@@ -589,13 +592,13 @@ static int bw_launch_dual_t(cudaStream_t st, const BwMaps& mi, BwMulti pi, const
   // tiles of the two forms hold the same bytes (64 x K entries)
   pi.stream = po.stream = l2_stream(128.0 * K * (ti + to));
   const int n_in = dual_split(ti, to, g_dual_bwd_pct.load(std::memory_order_relaxed));
-  bd_bwd_dual_kernel<K, SWAP_IN, SWAP_OUT><<<148, BW_THREADS, C::SMEM, st>>>(mi, pi, mo, po, n_in);
+  launch_pdl_if(overlap, bd_bwd_dual_kernel<K, SWAP_IN, SWAP_OUT>, 148, BW_THREADS, C::SMEM, st, mi, pi, mo, po, n_in);
   return CAFEQ_OK;
 }
 
 // fp16 single-term form only; each list holds at least 148 * 6 tiles (the caller checks with bw_dual_ok)
 static bool bw_dual_ok(int k) { return k == 128 || k == 256; }
-static int bw_launch_dual(cudaStream_t st, int k, int tr_in, const BwSub* in, int n_in, int tr_out, const BwSub* out, int n_out) {
+static int bw_launch_dual(cudaStream_t st, int k, int tr_in, const BwSub* in, int n_in, int tr_out, const BwSub* out, int n_out, bool overlap) {
   if (n_in < 1 || n_in > BW_MAX_SUB || n_out < 1 || n_out > BW_MAX_SUB || !bw_dual_ok(k)) return CAFEQ_ERR_INVALID_ARG;
   BwMaps mi, mo;
   BwMulti pi, po;
@@ -617,7 +620,7 @@ static int bw_launch_dual(cudaStream_t st, int k, int tr_in, const BwSub* in, in
   po.n = n_out;
   const int si = tr_in ? 0 : 1, so = tr_out ? 0 : 1;
 #define BW_DUAL(KK, SI, SO) \
-  if (k == KK && si == SI && so == SO) return bw_launch_dual_t<KK, SI, SO>(st, mi, pi, mo, po);
+  if (k == KK && si == SI && so == SO) return bw_launch_dual_t<KK, SI, SO>(st, mi, pi, mo, po, overlap);
   BW_DUAL(128, 0, 0)
   BW_DUAL(128, 0, 1)
   BW_DUAL(128, 1, 0)

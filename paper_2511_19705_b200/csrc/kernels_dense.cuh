@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
                                                          uint16_t* __restrict__ thi, uint16_t* __restrict__ tlo,
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
                                                          uint16_t* __restrict__ t3 = nullptr) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ uint32_t tile[64][65];
   __shared__ uint16_t tile3[64][66];
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
 // and transpose (V fp32 [d3, r*h] -> Bf fp32 [h, d3]).  grid: ceil(d3/32), h/32 (k % 32 == 0); block 32 x 8.
 __global__ void __launch_bounds__(256) fold_transpose_kernel(const float* __restrict__ V, int d3, int h, int k, int r,
                                                              float* __restrict__ Bf) {
+  pdl_enter();
   __shared__ float tile[32][33];
   const int y0 = blockIdx.x * 32, l0 = blockIdx.y * 32;  // l0 inside one block of k
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -108,6 +110,7 @@ __global__ void __launch_bounds__(256) fold_transpose_kernel(const float* __rest
 // d3); a thread reads four entries once and writes every replica (60 -> 12 us at 3584 x 4096).
 __global__ void __launch_bounds__(256) expand_cols_kernel(const float* __restrict__ X, int h, int k, int r, float scale,
                                                           float* __restrict__ V) {
+  pdl_enter();
   const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
   if (l >= h) return;
   const long long y = blockIdx.y;
@@ -120,6 +123,7 @@ __global__ void __launch_bounds__(256) expand_cols_kernel(const float* __restric
 
 // the same for any k, one entry per thread (learned offsets take every shape)
 __global__ void expand_cols_any_kernel(const float* __restrict__ X, int d3, int h, int k, int r, float scale, float* __restrict__ V) {
+  pdl_enter();
   const long long n = (long long)d3 * r * h;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const long long y = e / ((long long)r * h);
@@ -133,6 +137,7 @@ __global__ void expand_cols_any_kernel(const float* __restrict__ X, int d3, int 
 // A product over the r*h expanded inner indices equals the product over the h folded ones: 1 / r of the work.
 __global__ void __launch_bounds__(256) fold_split_kernel(const float* __restrict__ V, int h, int k, int r, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ h3, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
   if (l >= h) return;
@@ -171,6 +176,7 @@ __global__ void __launch_bounds__(256) fold_split_kernel(const float* __restrict
 // arg-max entry of its group (records row-major)
 __global__ void add_argmax_kernel(float* __restrict__ gX, long long ld, int rows, int ng, int g, const float* __restrict__ coef,
                                   const int* __restrict__ idx, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const long long n = (long long)rows * ng;
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < n; w += (long long)gridDim.x * blockDim.x) {
@@ -191,6 +197,7 @@ __global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* __rest
                                                              int ng, int g, int k, int r, const float* __restrict__ a,
                                                              const float* __restrict__ usel, const int* __restrict__ idx, float qmax,
                                                              uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const int l = threadIdx.x % LPG;
   const long long total = (long long)rows * ng;
@@ -268,6 +275,7 @@ __global__ void ste_scale_coef_kernel(const float* __restrict__ gD, long long ld
                                       const uint16_t* __restrict__ Dl, long long ldd, int rows, int ng, int g,
                                       const float* __restrict__ a, const float* __restrict__ usel, int gm,
                                       float* __restrict__ coef, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -292,6 +300,7 @@ __global__ void ste_scale_coef_kernel(const float* __restrict__ gD, long long ld
 // acc += sum x[i] y[i]  (fp32 products summed in double; one atomic per block)
 __global__ void __launch_bounds__(256) dot_f32_kernel(const float* __restrict__ x, const float* __restrict__ y, long long n,
                                                       double* acc) {
+  pdl_enter();
   __shared__ double red[32];
   double s = 0.0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -306,7 +315,8 @@ __global__ void __launch_bounds__(256) dot_f32_kernel(const float* __restrict__ 
 // one written, one cleared.  Bound by reading S twice per round (29 MB, from L2: 11 + 5 us; with slices of 512 rows, 56 CTAs,
 // the second kernel took 75 us, and norm and scaling were launches of their own).
 // After the last round *sig2 = safety * |S^T S v| (v of unit norm): a Rayleigh-type estimate from below of sigma_max^2.
-__global__ void pw_init_kernel(float* __restrict__ v, int C) {  // v [3][C]
+__global__ void pw_init_kernel(float* __restrict__ v, int C) {
+  pdl_enter();  // v [3][C]
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < C) {
     uint32_t h = (uint32_t)j * 2654435761u;
@@ -326,6 +336,7 @@ __device__ __forceinline__ double pw_norm2(const float* v, int C, double* red) {
 }
 __global__ void __launch_bounds__(256) pw_rows_kernel(const float* __restrict__ S, const float* __restrict__ v, float* __restrict__ clear,
                                                       int R, int C, float* __restrict__ u) {
+  pdl_enter();
   __shared__ double red[32];
   const double n = sqrt(pw_norm2(v, C, red));
   const float inv = n > 0.0 ? (float)(1.0 / n) : 0.f;
@@ -341,6 +352,7 @@ __global__ void __launch_bounds__(256) pw_rows_kernel(const float* __restrict__ 
 // grid: (ceil(C / 256), ceil(R / 32)); v2 cleared two launches before
 __global__ void __launch_bounds__(256) pw_cols_kernel(const float* __restrict__ S, const float* __restrict__ u, int R, int C,
                                                       float* __restrict__ v2) {
+  pdl_enter();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= C) return;
   const int r0 = blockIdx.y * 32, n = min(R - r0, 32);
@@ -350,6 +362,7 @@ __global__ void __launch_bounds__(256) pw_cols_kernel(const float* __restrict__ 
   atomicAdd(&v2[j], s);
 }
 __global__ void __launch_bounds__(256) pw_result_kernel(const float* __restrict__ v, int C, double safety, const double* fro2, double* sig2) {
+  pdl_enter();
   __shared__ double red[32];
   const double n = sqrt(pw_norm2(v, C, red));
   if (threadIdx.x == 0) {
@@ -361,6 +374,7 @@ __global__ void __launch_bounds__(256) pw_result_kernel(const float* __restrict_
 }
 
 __global__ void sqrt_hist_kernel(const double* __restrict__ sq, float* __restrict__ out, int n) {
+  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (float)sqrt(fmax(sq[i], 0.0));
 }

@@ -873,6 +873,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
   }
 
   // ---------------------------------------------------------------- teardown
+  pdl_release();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -885,6 +886,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
 template <int FORM, int K, int G, int MODE>
 __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_kernel(const __grid_constant__ BdMaps maps, const __grid_constant__ BdMulti mp) {
+  pdl_wait();
   bd_pass_body<FORM, K, G, MODE>(maps, mp, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -895,6 +897,7 @@ template <int K, int G>
 __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_dual_kernel(const __grid_constant__ BdMaps maps_in, const __grid_constant__ BdMulti mp_in,
                     const __grid_constant__ BdMaps maps_out, const __grid_constant__ BdMulti mp_out, const int n_in) {
+  pdl_wait();
   if ((int)blockIdx.x < n_in) bd_pass_body<BD_IN, K, G, BD_REC>(maps_in, mp_in, (int)blockIdx.x, n_in);
   else bd_pass_body<BD_OUT, K, G, BD_REC>(maps_out, mp_out, (int)blockIdx.x - n_in, (int)gridDim.x - n_in);
 }
@@ -1002,7 +1005,7 @@ static int bd_launch_multi_t(cudaStream_t st, const BdMaps& maps, BdMulti mp, in
   long long want = total / (min_tiles > 0 ? min_tiles : 1);
   if (want < 1) want = 1;
   const int grid = want < 148 ? (int)want : 148;
-  bd_pass_kernel<FORM, K, G, MODE><<<grid, BD_THREADS, C::SMEM, st>>>(maps, mp);
+  launch_pdl(bd_pass_kernel<FORM, K, G, MODE>, grid, BD_THREADS, C::SMEM, st, maps, mp);
   return CAFEQ_OK;
 }
 
@@ -1095,7 +1098,7 @@ static int dual_split(long long tiles_in, long long tiles_out, int out_weight_pc
 }
 
 template <int K, int G>
-static int bd_launch_dual_t(cudaStream_t st, const BdMaps& mi, BdMulti pi, const BdMaps& mo, BdMulti po) {
+static int bd_launch_dual_t(cudaStream_t st, const BdMaps& mi, BdMulti pi, const BdMaps& mo, BdMulti po, bool overlap) {
   constexpr int SMEM = BdCfg<BD_IN, K, G>::SMEM > BdCfg<BD_OUT, K, G>::SMEM ? BdCfg<BD_IN, K, G>::SMEM : BdCfg<BD_OUT, K, G>::SMEM;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(bd_pass_dual_kernel<K, G>, SMEM, done)) return CAFEQ_ERR_CUDA;
@@ -1114,14 +1117,14 @@ static int bd_launch_dual_t(cudaStream_t st, const BdMaps& mi, BdMulti pi, const
   for (int s = po.n; s < BD_MAX_SUB; ++s) po.tile_end[s] = (int)to;
   pi.stream = po.stream = l2_stream(65536.0 * (ti + to));
   const int n_in = dual_split(ti, to, g_dual_pass_pct.load(std::memory_order_relaxed));
-  bd_pass_dual_kernel<K, G><<<148, BD_THREADS, SMEM, st>>>(mi, pi, mo, po, n_in);
+  launch_pdl_if(overlap, bd_pass_dual_kernel<K, G>, 148, BD_THREADS, SMEM, st, mi, pi, mo, po, n_in);
   return CAFEQ_OK;
 }
 
 // Input-axis and output-axis matrices of one block size and group size in ONE persistent launch (both lists
 // non-empty, each at least 148 tiles so that every CTA has work; otherwise the caller launches them separately).
 static bool bd_dual_ok(int k, int g) { return (k == 128 || k == 256) && (g == 64 || g == 128); }
-static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_in, const BdSub* out, int n_out) {
+static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_in, const BdSub* out, int n_out, bool overlap) {
   if (n_in < 1 || n_in > BD_MAX_SUB || n_out < 1 || n_out > BD_MAX_SUB || !bd_dual_ok(k, g)) return CAFEQ_ERR_INVALID_ARG;
   BdMaps mi, mo;
   BdMulti pi, po;
@@ -1142,7 +1145,7 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
   pi.n = n_in;
   po.n = n_out;
 #define BD_DUAL(KK, GG) \
-  if (k == KK && g == GG) return bd_launch_dual_t<KK, GG>(st, mi, pi, mo, po);
+  if (k == KK && g == GG) return bd_launch_dual_t<KK, GG>(st, mi, pi, mo, po, overlap);
   BD_DUAL(128, 64)
   BD_DUAL(128, 128)
   BD_DUAL(256, 64)
@@ -1157,6 +1160,7 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
 // paired (k = 32): blocks 2 i and 2 i + 1 become one 64 x 64 block, zeros off the diagonal.
 __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* __restrict__ T, uint16_t* __restrict__ out, int k, int transpose,
                                                                int paired, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ float tile[32][33];
   const size_t base = (size_t)blockIdx.z * k * k;
@@ -1204,6 +1208,7 @@ constexpr int AS_ROWS = 8, AS_MAX_ROWS = 64;
 __global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* __restrict__ X, long long ld, const float* __restrict__ T,
                                                           uint16_t* __restrict__ Y, int rows, int d_in, int k, int r, int transposed,
                                                           const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ float ps[256 * 33];
   __shared__ float4 xs4[256 * AS_ROWS / 4];

@@ -234,6 +234,7 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
 template <int BN>
 __global__ void __launch_bounds__(TG_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgParams p) {
+  pdl_enter();
   using C = TgCfg<BN>;
   if (p.status && *p.status) return;
   if (tg_stopped(p)) return;
@@ -421,6 +422,7 @@ __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.b
 template <int K>
 __global__ void __launch_bounds__(TG_THREADS, 1)
 tc_block_kernel(const __grid_constant__ TbMaps maps, const TbTerms tt, const TgParams p) {
+  pdl_enter();
   using C = TbCfg<K>;
   static_assert(K == 128 || K == 256, "block size");
   if (p.status && *p.status) return;
@@ -677,7 +679,7 @@ static int tg_launch_t(cudaStream_t st, const TgOperand* A, const TgOperand* B, 
     if (!make_map_bf16(&maps.b[t], B[t].ptr, B[t].cols, B[t].rows, B[t].pitch, p.b_mn ? 64 : BN)) return CAFEQ_ERR_UNSUPPORTED;
   }
   dim3 grid((p.N + BN - 1) / BN, (p.M + 127) / 128, p.batch);
-  tc_gemm_kernel<BN><<<grid, TG_THREADS, C::SMEM, st>>>(maps, p);
+  launch_pdl(tc_gemm_kernel<BN>, grid, TG_THREADS, C::SMEM, st, maps, p);
   return CAFEQ_OK;
 }
 
@@ -726,7 +728,7 @@ static int tb_launch_t(cudaStream_t st, const TbMaps& maps, const TbTerms& tt, c
   using C = TbCfg<K>;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(tc_block_kernel<K>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
-  tc_block_kernel<K><<<p.batch, TG_THREADS, C::SMEM, st>>>(maps, tt, p);
+  launch_pdl(tc_block_kernel<K>, p.batch, TG_THREADS, C::SMEM, st, maps, tt, p);
   return CAFEQ_OK;
 }
 static bool tb_supported(int k, int nterms) { return (k == 128 || k == 256) && nterms >= 1 && nterms <= TG_MAX_TERMS; }
@@ -783,6 +785,7 @@ static int tb_launch(cudaStream_t st, int nterms, const uint16_t* const* A, cons
 __global__ void __launch_bounds__(256) split_bf16_kernel(const float* __restrict__ X, int k, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
                                                          uint16_t* __restrict__ tlo, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ uint32_t tile[32][33];
   const size_t base = (size_t)blockIdx.z * k * k;

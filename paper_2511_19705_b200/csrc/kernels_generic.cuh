@@ -8,6 +8,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "cafeq.h"
 
 namespace cafeq {
@@ -15,6 +17,36 @@ namespace cafeq {
 // ------------------------------------------------------------------------------------------------
 // small helpers
 // ------------------------------------------------------------------------------------------------
+// Every kernel is launched with programmatic stream serialisation: its CTAs may become resident while the kernel before it in
+// the stream drains, and wait here until that kernel is complete and its writes are visible; then the next kernel may do the
+// same.  Nothing in global memory is read or written before the wait.  (Between two kernels of a step lay 1.6 - 2.6 us.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter() {
+  pdl_wait();
+  pdl_release();
+}
+
+// overlap = false: an ordinary launch, after the kernel before it (the wait then returns at once)
+template <typename... P, typename... A>
+static inline void launch_pdl_if(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+static inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  launch_pdl_if(true, kernel, grid, block, smem, st, std::forward<A>(args)...);
+}
+
 __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) { return __uint_as_float(((uint32_t)b) << 16); }
 
 __device__ __forceinline__ float round_to_bf16(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
@@ -41,11 +73,13 @@ __device__ __forceinline__ double block_sum_double(double v, double* sh) {
 // fill / copy / round
 // ------------------------------------------------------------------------------------------------
 __global__ void fill_f32_kernel(float* p, float v, long long n) {
+  pdl_enter();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     p[i] = v;
 }
 
 __global__ void zero_f64_kernel(double* p, int n) {
+  pdl_enter();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = 0.0;
 }
@@ -53,12 +87,14 @@ __global__ void zero_f64_kernel(double* p, int n) {
 // out = float(bf16(in)): the operand actually fed to the transform products.
 __global__ void round_bf16_kernel(const float* __restrict__ in, float* __restrict__ out, long long n,
                                   const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = round_to_bf16(in[i]);
 }
 
 __global__ void copy_f32_kernel(const float* __restrict__ in, float* __restrict__ out, long long n) {
+  pdl_enter();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = in[i];
 }
@@ -88,6 +124,7 @@ struct GemmArgs {
 
 template <bool ABF, bool BBF>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
+  pdl_enter();
   if (g.status && *g.status) return;
   constexpr int BM = 64, BN = 64, BK = 16;
   __shared__ float As[BK][BM + 4];
@@ -265,6 +302,7 @@ __device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* s
 
 __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out,
                                                              float* __restrict__ cnorm, int k, int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   extern __shared__ float sm[];  // 3 k words
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -289,6 +327,7 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __rest
 // ------------------------------------------------------------------------------------------------
 __global__ void absmax_kernel(const float* __restrict__ U, long long ld, int rows, int ng, int g,
                               float* __restrict__ a, float* __restrict__ usel, int* __restrict__ idx, int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -322,6 +361,7 @@ __global__ void absmax_kernel(const float* __restrict__ U, long long ld, int row
 
 __global__ void scales_kernel(const float* __restrict__ a, float* __restrict__ s, long long n, float qmax,
                               const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     s[i] = __fdiv_rn(a[i], qmax);
@@ -343,6 +383,7 @@ __global__ void quant_kernel(const float* __restrict__ U, long long ld, int rows
                              const float* __restrict__ a, float qmax, const void* __restrict__ offsets, int off_kind,
                              float* __restrict__ Delta, float* __restrict__ Uhat, int8_t* __restrict__ codes,
                              const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const int ng = cols / g;
   const long long n = (long long)rows * cols;
@@ -378,6 +419,7 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict_
                                                           float* __restrict__ usel, int* __restrict__ idx, float* __restrict__ Delta,
                                                           float* __restrict__ Uhat, int8_t* __restrict__ codes,
                                                           float* __restrict__ scales, int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const int cols = ng * g;
   const int l = threadIdx.x % LPG;
@@ -479,6 +521,7 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict_
 // ------------------------------------------------------------------------------------------------
 // axis IN:  cw[Gc] = sum_{t in group Gc} c[t'],  t' = (B / r) * k + (t mod k), B = t / k
 __global__ void cw_in_kernel(const float* __restrict__ c, int d_in, int g, int k, int r, float* __restrict__ cw) {
+  pdl_enter();
   int Gc = blockIdx.x * blockDim.x + threadIdx.x;
   if (Gc >= d_in / g) return;
   float s = 0.f;
@@ -492,6 +535,7 @@ __global__ void cw_in_kernel(const float* __restrict__ c, int d_in, int g, int k
 
 // axis OUT: cw[row] = g * c[t'(row)]
 __global__ void cw_out_kernel(const float* __restrict__ c, int d_out, int g, int k, int r, float* __restrict__ cw) {
+  pdl_enter();
   int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= d_out) return;
   int B = row / k;
@@ -506,6 +550,7 @@ __global__ void surrogate_rows_kernel(const float* __restrict__ a, const float* 
                                       const float* __restrict__ cw, float kappa, int k, int r, float* __restrict__ coef,
                                       float* __restrict__ Agrp, float* __restrict__ A, double* __restrict__ acc,
                                       const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ double red[32];
   int row = blockIdx.x * blockDim.x + threadIdx.x;
@@ -537,6 +582,7 @@ __global__ void surrogate_rows_kernel(const float* __restrict__ a, const float* 
 
 // axis IN: A[t'] += Agrp[group of t]
 __global__ void expand_agrp_kernel(const float* __restrict__ Agrp, int d_in, int g, int k, int r, float* __restrict__ A) {
+  pdl_enter();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= d_in) return;
   int B = t / k;
@@ -546,6 +592,7 @@ __global__ void expand_agrp_kernel(const float* __restrict__ Agrp, int d_in, int
 // gMinv[b][i][t] = scale * Minv[b][i][t] * A[b][t]
 __global__ void scale_cols_kernel(const float* __restrict__ Minv, const float* __restrict__ A, float scale, int k,
                                   long long n, float* __restrict__ out) {
+  pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     long long b = e / ((long long)k * k);
     int t = (int)(e % k);
@@ -561,6 +608,7 @@ __global__ void ste_scale_path_kernel(const float* __restrict__ U, const float* 
                                       int ng, int g, const float* __restrict__ a, const float* __restrict__ usel, float qmax,
                                       const void* __restrict__ offsets, int off_kind, int cols, float* __restrict__ coef,
                                       const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -592,6 +640,7 @@ __global__ void ste_scale_path_kernel(const float* __restrict__ U, const float* 
 __global__ void grad_offsets_kernel(const float* __restrict__ U, const float* __restrict__ gUhat, long long ld, int rows, int cols,
                                     int g, const float* __restrict__ a, float qmax, float* __restrict__ out,
                                     const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const int ng = cols / g;
   const long long n = (long long)rows * cols;
@@ -617,6 +666,7 @@ __global__ void __launch_bounds__(256) scatter_in_kernel(const uint16_t* __restr
                                                          int g, int k, int r, const float* __restrict__ coef,
                                                          const int* __restrict__ idx, float* __restrict__ gradT,
                                                          int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
+  pdl_enter();
   if (status && *status) return;
   extern __shared__ float acc[];  // [k][SCATTER_JS]
   const int B = blockIdx.x, js = blockIdx.y * SCATTER_JS;
@@ -650,6 +700,7 @@ __global__ void __launch_bounds__(256) scatter_out_kernel(const uint16_t* __rest
                                                           int g, int k, int r, const float* __restrict__ coef,
                                                           const int* __restrict__ idx, float* __restrict__ gradT,
                                                           int transpose_out, int groups_per_cta, const int32_t* status, int gm) {
+  pdl_enter();
   if (status && *status) return;
   extern __shared__ float acc[];  // [k][SCATTER_JS]
   const int B = blockIdx.x, js = blockIdx.y * SCATTER_JS;
@@ -698,6 +749,7 @@ __global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t
                                                                   int d_in, int g, int k, int r, const float* __restrict__ coef,
                                                                   const int* __restrict__ idx, float* __restrict__ gradT,
                                                                   int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
+  pdl_enter();
   if (status && *status) return;
   extern __shared__ float acc[];  // [k][64]
   const int B = blockIdx.x, js = blockIdx.y * SC2_JS;
@@ -774,6 +826,7 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
                                                                    int d_in, int g, int r, int NG, const float* __restrict__ coef,
                                                                    const int* __restrict__ idx, float* __restrict__ gradT,
                                                                    int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
+  pdl_enter();
   if (status && *status) return;
   constexpr int TPB = 256 / K;      // threads per bucket
   constexpr int CPT = STRIP / TPB;  // strip columns per thread
@@ -929,6 +982,7 @@ __global__ void __launch_bounds__(256) scatter_out_strip_kernel(const uint16_t* 
                                                                 int d_in, int g, int r, const float* __restrict__ coef,
                                                                 const int* __restrict__ idx, float* __restrict__ gradT,
                                                                 int transpose_out, int groups_per_cta, const int32_t* status, int gm) {
+  pdl_enter();
   if (status && *status) return;
   constexpr int RW = K / 8;  // rows of the block per warp
   extern __shared__ __align__(16) uint16_t tiles[];  // two tiles [64][g + 4]
@@ -1015,6 +1069,7 @@ struct PrepArgs {
 };
 
 __global__ void step_prep_kernel(PrepArgs a) {
+  pdl_enter();
   if (a.status && *a.status) return;
   const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   for (long long e = t0; e < a.kk; e += stride) {
@@ -1041,6 +1096,7 @@ __global__ void step_prep_kernel(PrepArgs a) {
 // of the concatenated blocks, r = 1)
 __global__ void __launch_bounds__(256) colnorm_cw_kernel(const float* __restrict__ X, int k, float* __restrict__ c,
                                                          float* __restrict__ cw, int g) {
+  pdl_enter();
   __shared__ float part[8][33];
   const int b = blockIdx.y, t = blockIdx.x * 32 + threadIdx.x;
   const float* Xb = X + (size_t)b * k * k;
@@ -1071,6 +1127,7 @@ __global__ void __launch_bounds__(256) colnorm_cw_kernel(const float* __restrict
 // dL/dMinv of Eq. 4: out[b][i][t] = scale * Minv[b][i][t] * A_t; input axis with r = 1 reads A_t = Agrp[(b k + t) / g]
 __global__ void gminv_kernel(const float* __restrict__ Minv, const float* __restrict__ A, const float* __restrict__ Agrp,
                              int g, float scale, int k, long long n, float* __restrict__ out) {
+  pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const long long b = e / ((long long)k * k);
     const int t = (int)(e % k);
@@ -1084,6 +1141,7 @@ __global__ void gminv_kernel(const float* __restrict__ Minv, const float* __rest
 // ------------------------------------------------------------------------------------------------
 __global__ void gd_update_kernel(float* __restrict__ M, const float* __restrict__ g, float lr, long long n,
                                  const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     M[i] = M[i] - lr * g[i];
@@ -1091,12 +1149,14 @@ __global__ void gd_update_kernel(float* __restrict__ M, const float* __restrict_
 
 // state = {step, m[n], v[n]}; the step counter is advanced by adam_tick_kernel before the update.
 __global__ void adam_tick_kernel(float* state, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   state[0] += 1.f;
 }
 
 __global__ void adam_update_kernel(float* __restrict__ M, const float* __restrict__ g, float* __restrict__ state, float lr,
                                    float b1, float b2, float eps, long long n, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const float step = state[0];
   const float c1 = 1.f - powf(b1, step), c2 = 1.f - powf(b2, step);
@@ -1117,6 +1177,7 @@ __global__ void adam_update_kernel(float* __restrict__ M, const float* __restric
 // ------------------------------------------------------------------------------------------------
 __global__ void sqsum_bf16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols, double* acc,
                                   const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ double red[32];
   double local = 0.0;
@@ -1155,6 +1216,7 @@ __global__ void sqsum_bf16_kernel(const uint16_t* __restrict__ W, long long ld, 
 // ------------------------------------------------------------------------------------------------
 __global__ void max_f32_kernel(const float* __restrict__ a, long long n, float* __restrict__ out_max,
                                const int32_t* status) {
+  pdl_enter();
   // a >= 0, so an integer atomicMax on the bit pattern orders correctly
   if (status && *status) return;
   float m = 0.f;
@@ -1166,6 +1228,7 @@ __global__ void max_f32_kernel(const float* __restrict__ a, long long n, float* 
 
 __global__ void sumexp_kernel(const float* __restrict__ a, long long n, const float* __restrict__ amax, float t,
                               double* __restrict__ acc, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ double red[32];
   const float mx = *amax;
@@ -1180,6 +1243,7 @@ __global__ void sumexp_kernel(const float* __restrict__ a, long long n, const fl
 __global__ void lse_coef_kernel(const float* __restrict__ a, const float* __restrict__ usel, long long n,
                                 const float* __restrict__ amax, float t, const double* __restrict__ Z,
                                 float* __restrict__ coef, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const float mx = *amax;
   const float zinv = (float)(1.0 / *Z);
@@ -1193,6 +1257,7 @@ __global__ void lse_coef_kernel(const float* __restrict__ a, const float* __rest
 // two-array forms of the three LogSumExp kernels (the group maxima of U and of V in one launch each)
 __global__ void max2_f32_kernel(const float* __restrict__ a1, long long n1, const float* __restrict__ a2, long long n2,
                                 float* __restrict__ out_max, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   float m = 0.f;
   const long long n = n1 + n2;
@@ -1204,6 +1269,7 @@ __global__ void max2_f32_kernel(const float* __restrict__ a1, long long n1, cons
 
 __global__ void sumexp2_kernel(const float* __restrict__ a1, long long n1, const float* __restrict__ a2, long long n2,
                                const float* __restrict__ amax, float t, double* __restrict__ acc, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ double red[32];
   const float mx = *amax;
@@ -1218,6 +1284,7 @@ __global__ void sumexp2_kernel(const float* __restrict__ a1, long long n1, const
 __global__ void lse_coef2_kernel(const float* __restrict__ a1, const float* __restrict__ u1, float* __restrict__ c1, long long n1,
                                  const float* __restrict__ a2, const float* __restrict__ u2, float* __restrict__ c2, long long n2,
                                  const float* __restrict__ amax, float t, const double* __restrict__ Z, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const float mx = *amax;
   const float zinv = (float)(1.0 / *Z);
@@ -1235,6 +1302,7 @@ __global__ void lse_coef2_kernel(const float* __restrict__ a1, const float* __re
 
 // R = M M^T - I in place on a [nb,k,k] buffer that already holds M M^T
 __global__ void sub_identity_kernel(float* __restrict__ R, int k, long long n) {
+  pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     long long q = e % ((long long)k * k);
     if (q / k == q % k) R[e] -= 1.f;
@@ -1242,6 +1310,7 @@ __global__ void sub_identity_kernel(float* __restrict__ R, int k, long long n) {
 }
 
 __global__ void sqsum_f32_kernel(const float* __restrict__ x, long long n, double* acc) {
+  pdl_enter();
   __shared__ double red[32];
   double local = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -1254,6 +1323,7 @@ __global__ void sqsum_f32_kernel(const float* __restrict__ x, long long n, doubl
 // (the un-squared norm has no gradient at R = 0 and below the fp32 noise floor its direction is noise)
 __global__ void orth_grad_kernel(float* __restrict__ gradM, const float* __restrict__ RM, const double* __restrict__ r2,
                                  float lambda, float sqrt_h, long long n) {
+  pdl_enter();
   const double nrm = sqrt(*r2);
   if (nrm < 1e-5 * (double)sqrt_h) return;
   const float f = (float)(2.0 * lambda / (nrm * sqrt_h));
@@ -1266,6 +1336,7 @@ __global__ void orth_grad_kernel(float* __restrict__ gradM, const float* __restr
 // ------------------------------------------------------------------------------------------------
 // single: acc = {surrogate, L2, ||W||^2}
 __global__ void finalize_single_kernel(const double* acc, float* losses, float* hist /*[2] or NULL*/, int want_exact) {
+  pdl_enter();
   if (losses) {
     losses[0] = (float)acc[0];
     losses[1] = want_exact ? (float)acc[1] : 0.f;
@@ -1283,6 +1354,7 @@ __global__ void finalize_single_kernel(const double* acc, float* losses, float* 
 __global__ void sumsq_coef2_kernel(const float* __restrict__ a1, const float* __restrict__ u1, float* __restrict__ c1, long long n1,
                                    const float* __restrict__ a2, const float* __restrict__ u2, float* __restrict__ c2, long long n2,
                                    const double* __restrict__ acc, int weighted, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const float w1 = (weighted ? (float)sqrt(acc[6]) : 1.f) * 2.f / (float)n1;
   const float w2 = (weighted ? (float)sqrt(acc[5]) : 1.f) * 2.f / (float)n2;
@@ -1300,6 +1372,7 @@ __global__ void sumsq_coef2_kernel(const float* __restrict__ a1, const float* __
 // dst += (acc[num] / count) / sqrt(acc[den]) * src   (the dense terms of the weighted form: mean(a^2) d||X||_F)
 __global__ void axpy_norm_kernel(float* __restrict__ dst, const float* __restrict__ src, long long n, const double* __restrict__ acc,
                                  int num, double count, int den, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   const double d = sqrt(acc[den]);
   const float f = d > 0.0 ? (float)(acc[num] / count / d) : 0.f;
@@ -1309,6 +1382,7 @@ __global__ void axpy_norm_kernel(float* __restrict__ dst, const float* __restric
 
 // out = T - T^T per block (the skew part that drives a Cayley step)
 __global__ void skew_blocks_kernel(const float* __restrict__ T, float* __restrict__ out, int k, long long n) {
+  pdl_enter();
   const long long kk = (long long)k * k;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const long long b = e / kk, q = e - b * kk;
@@ -1320,11 +1394,13 @@ __global__ void skew_blocks_kernel(const float* __restrict__ T, float* __restric
 // out = x + alpha * y  /  x = beta * x + y
 __global__ void lincomb_kernel(float* __restrict__ out, const float* __restrict__ x, float alpha, const float* __restrict__ y,
                                long long n, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = fmaf(alpha, y[i], x[i]);
 }
 __global__ void momentum_kernel(float* __restrict__ v, float beta, const float* __restrict__ g, long long n, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     v[i] = fmaf(beta, v[i], g[i]);
@@ -1335,6 +1411,7 @@ __global__ void momentum_kernel(float* __restrict__ v, float beta, const float* 
 __global__ void finalize_pair_kernel(const double* acc, const float* amax, float t, float lambda, float sqrt_h,
                                      float* losses, float* hist, int want_pqe, int objective = 0, double n1 = 1.0,
                                      double n2 = 1.0) {
+  pdl_enter();
   float lse = *amax + (float)(log(acc[0]) / (double)t);
   if (objective == 1) lse = (float)(acc[3] / n1 + acc[4] / n2);
   if (objective == 2) lse = (float)(sqrt(acc[6]) * acc[3] / n1 + sqrt(acc[5]) * acc[4] / n2);
@@ -1357,6 +1434,7 @@ __global__ void finalize_pair_kernel(const double* acc, const float* amax, float
 // pack: u = q + qmax, little-endian bit stream per row; one thread per output 32-bit word group
 // ------------------------------------------------------------------------------------------------
 __global__ void pack_kernel(const int8_t* __restrict__ codes, uint8_t* __restrict__ packed, int rows, int cols, int bits) {
+  pdl_enter();
   // one thread packs 8 consecutive codes into `bits` bytes
   const long long chunks_per_row = cols / 8;
   const long long n = (long long)rows * chunks_per_row;
@@ -1381,6 +1459,7 @@ __global__ void pack_kernel(const int8_t* __restrict__ codes, uint8_t* __restric
 template <int BITS>
 __global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* __restrict__ packed, const float* __restrict__ scales,
                                                        uint16_t* __restrict__ out, unsigned n, unsigned cpr, unsigned cpg, long long ldo) {
+  pdl_enter();
   constexpr uint32_t mask = (1u << BITS) - 1u;
   constexpr float base = 8388608.f + (float)((1 << (BITS - 1)) - 1);
   const unsigned c0 = blockIdx.x * 1024u + threadIdx.x;
@@ -1428,6 +1507,7 @@ __global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* __restrict
 // one thread per 8 consecutive codes (`bits` bytes of the stream); cols % 8 == 0, out row pitch ldo elements.
 __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict__ packed, const float* __restrict__ scales,
                                                       uint16_t* __restrict__ out, int rows, int cols, int bits, int g, long long ldo) {
+  pdl_enter();
   const long long chunks_per_row = cols / 8;
   const long long n = (long long)rows * chunks_per_row;
   const int qmax = (1 << (bits - 1)) - 1;
@@ -1450,6 +1530,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict_
 }
 
 __global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* __restrict__ in, uint16_t* __restrict__ out, long long n) {
+  pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
     out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(in[e]));
 }
@@ -1459,6 +1540,7 @@ __global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* __restric
 template <int BITS>
 __global__ void __launch_bounds__(256) pack32_kernel(const int8_t* __restrict__ codes, uint32_t* __restrict__ packed, int rows,
                                                      int cols) {
+  pdl_enter();
   const long long chunks_per_row = cols / 32;
   const long long n = (long long)rows * chunks_per_row;
   constexpr int qmax = (1 << (BITS - 1)) - 1;

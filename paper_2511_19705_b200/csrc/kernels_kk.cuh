@@ -79,6 +79,7 @@ struct NsCfg {
 template <int K>
 __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1)
 ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsParams p) {
+  pdl_wait();  // (releases at its end: a layer's penalty chain shares the SMs with it, which waiting CTAs of the pass would take)
   using C = NsCfg<K>;
   if (p.status && *p.status) return;
   const int b = blockIdx.x, row_b = b * K;
@@ -434,6 +435,7 @@ ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     }
     __syncthreads();
   }
+  pdl_release();
   if (want_c) {
     float* cw = p.cw[prob];
     for (int t = threadIdx.x; t < K; t += C::THREADS) {
@@ -453,11 +455,11 @@ ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
 }
 
 template <int K>
-static int ns_block_launch_t(cudaStream_t st, const NsMaps& maps, int nb, const NsParams& p) {
+static int ns_block_launch_t(cudaStream_t st, const NsMaps& maps, int nb, const NsParams& p, bool overlap) {
   using C = NsCfg<K>;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(ns_block_kernel<K>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
-  ns_block_kernel<K><<<nb, C::THREADS, C::SMEM, st>>>(maps, p);
+  launch_pdl_if(overlap, ns_block_kernel<K>, nb, C::THREADS, C::SMEM, st, maps, p);
   return CAFEQ_OK;
 }
 
@@ -474,7 +476,7 @@ static bool make_map_hl(CUtensorMap* m, const uint16_t* hi, const uint16_t* lo, 
 }
 
 // A, hi, lo: bf16 [nb * k, k]; X: fp32 [nb, k, k] (written, not read)
-static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uint16_t* lo, float* X, int nb, int k, NsParams p) {
+static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uint16_t* lo, float* X, int nb, int k, NsParams p, bool overlap) {
   NsMaps m;
   p.A = A; p.hi = hi; p.lo = lo; p.X = X;
   const long long rows = (long long)nb * k;
@@ -482,12 +484,13 @@ static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uin
       !make_map_bf16(&m.xh_k, hi, k, rows, k, k) || !make_map_hl(&m.xhl, hi, lo, rows, k) ||
       !make_map_2d(&m.x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, X, k, rows, k, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B))
     return CAFEQ_ERR_UNSUPPORTED;
-  return k == 256 ? ns_block_launch_t<256>(st, m, nb, p) : ns_block_launch_t<128>(st, m, nb, p);
+  return k == 256 ? ns_block_launch_t<256>(st, m, nb, p, overlap) : ns_block_launch_t<128>(st, m, nb, p, overlap);
 }
 
 // hi = A^T, lo = 0: the cold start X0 = A^T of the iteration (A is bf16, so hi carries it exactly); 32 x 32 tiles
 __global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* __restrict__ A, int k, uint16_t* __restrict__ hi,
                                                             uint16_t* __restrict__ lo, const int32_t* status) {
+  pdl_enter();
   if (status && *status) return;
   __shared__ uint16_t tile[32][34];
   const size_t base = (size_t)blockIdx.z * k * k;
@@ -572,6 +575,7 @@ __device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* v) {
 template <int K, int MODE>
 __global__ void __launch_bounds__(ChainCfg<K>::THREADS, 1)
 kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainParams p) {
+  pdl_enter();
   using C = ChainCfg<K>;
   if (p.status && *p.status) return;
   const int b = blockIdx.x, row_b = b * K;
@@ -920,17 +924,17 @@ kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ 
 }
 
 template <int K, int MODE>
-static int kk_chain_launch_t(cudaStream_t st, const ChainMaps& maps, int nb, const ChainParams& p) {
+static int kk_chain_launch_t(cudaStream_t st, const ChainMaps& maps, int nb, const ChainParams& p, bool overlap) {
   using C = ChainCfg<K>;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(kk_chain_kernel<K, MODE>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
-  kk_chain_kernel<K, MODE><<<nb, C::THREADS, C::SMEM, st>>>(maps, p);
+  launch_pdl_if(overlap, kk_chain_kernel<K, MODE>, nb, C::THREADS, C::SMEM, st, maps, p);
   return CAFEQ_OK;
 }
 
 // hi, lo: splits of X (KK_MINV_PATH) or M (KK_PENALTY), bf16 [nb * k, k]; out fp32 [nb, k, k]
 static int kk_chain_launch(cudaStream_t st, int mode, const uint16_t* hi, const uint16_t* lo, float* out, int nb, int k,
-                           const ChainParams& p) {
+                           const ChainParams& p, bool overlap = true) {
   ChainMaps m;
   const long long rows = (long long)nb * k;
   const int box1 = mode == KK_MINV_PATH ? 64 : k, box2 = mode == KK_MINV_PATH ? k : 64;
@@ -938,8 +942,8 @@ static int kk_chain_launch(cudaStream_t st, int mode, const uint16_t* hi, const 
       !make_map_bf16(&m.b2[0], hi, k, rows, k, box2) || !make_map_bf16(&m.b2[1], lo, k, rows, k, box2) ||
       !make_map_2d(&m.out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, out, k, rows, k, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B))
     return CAFEQ_ERR_UNSUPPORTED;
-  if (mode == KK_MINV_PATH) return k == 256 ? kk_chain_launch_t<256, KK_MINV_PATH>(st, m, nb, p) : kk_chain_launch_t<128, KK_MINV_PATH>(st, m, nb, p);
-  return k == 256 ? kk_chain_launch_t<256, KK_PENALTY>(st, m, nb, p) : kk_chain_launch_t<128, KK_PENALTY>(st, m, nb, p);
+  if (mode == KK_MINV_PATH) return k == 256 ? kk_chain_launch_t<256, KK_MINV_PATH>(st, m, nb, p, overlap) : kk_chain_launch_t<128, KK_MINV_PATH>(st, m, nb, p, overlap);
+  return k == 256 ? kk_chain_launch_t<256, KK_PENALTY>(st, m, nb, p, overlap) : kk_chain_launch_t<128, KK_PENALTY>(st, m, nb, p, overlap);
 }
 
 }  // namespace cafeq

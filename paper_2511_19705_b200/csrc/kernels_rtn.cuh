@@ -21,6 +21,7 @@ namespace cafeq {
 template <int LG>
 __global__ void __launch_bounds__(256) rtn_stream_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols,
                                                          float qmax, int8_t* __restrict__ codes, float* __restrict__ scales) {
+  pdl_enter();
   constexpr int UPG = 4 * LG;               // 16-byte chunks per group
   const int cpr = cols / 8;                 // chunks per row; a multiple of UPG
   const long long nch = (long long)rows * cpr;
@@ -117,10 +118,10 @@ static bool rtn_stream_launch(cudaStream_t st, const void* W, long long ld, int 
   if (blocks < 1) blocks = 1;
   const uint16_t* w = (const uint16_t*)W;
   switch (g) {
-    case 32: rtn_stream_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(w, ld, rows, cols, qmax, codes, scales); break;
-    case 64: rtn_stream_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(w, ld, rows, cols, qmax, codes, scales); break;
-    case 128: rtn_stream_kernel<4><<<(unsigned)blocks, 256, 0, st>>>(w, ld, rows, cols, qmax, codes, scales); break;
-    default: rtn_stream_kernel<8><<<(unsigned)blocks, 256, 0, st>>>(w, ld, rows, cols, qmax, codes, scales); break;
+    case 32: launch_pdl(rtn_stream_kernel<1>, (unsigned)blocks, 256, 0, st, w, ld, rows, cols, qmax, codes, scales); break;
+    case 64: launch_pdl(rtn_stream_kernel<2>, (unsigned)blocks, 256, 0, st, w, ld, rows, cols, qmax, codes, scales); break;
+    case 128: launch_pdl(rtn_stream_kernel<4>, (unsigned)blocks, 256, 0, st, w, ld, rows, cols, qmax, codes, scales); break;
+    default: launch_pdl(rtn_stream_kernel<8>, (unsigned)blocks, 256, 0, st, w, ld, rows, cols, qmax, codes, scales); break;
   }
   return true;
 }

@@ -54,6 +54,7 @@ __device__ __forceinline__ void ly_put_operator(uint16_t* Ab, uint16_t* Pl, cons
 // Set-up of the first step of a call (the caller may have changed the parameters); the later ones are set up by the
 // parameter update of the step before.
 __global__ void __launch_bounds__(256) layer_prep_kernel(const LyPrepArgs a) {
+  pdl_enter();
   if (a.status && *a.status) return;
   const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long kk = (long long)a.k * a.k;
@@ -89,6 +90,7 @@ struct LyLseArgs {
 };
 
 __global__ void __launch_bounds__(256) layer_lse_kernel(const LyLseArgs g) {
+  pdl_enter();
   if (g.status && *g.status) return;
   __shared__ double red[32];
   const int p = blockIdx.y;
@@ -139,6 +141,7 @@ struct LyFinishArgs {
 };
 
 __global__ void __launch_bounds__(256) layer_finish_kernel(const LyFinishArgs f) {
+  pdl_enter();
   if (f.status && *f.status) return;
   const int p = blockIdx.y;
   const long long kk = (long long)f.k * f.k;
@@ -220,6 +223,7 @@ __global__ void __launch_bounds__(256) layer_finish_kernel(const LyFinishArgs f)
 // max |w| of a bf16 matrix (bit pattern of a non-negative float, atomic integer maximum)
 __global__ void __launch_bounds__(256) absmax_bf16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols,
                                                           float* __restrict__ out) {
+  pdl_enter();
   float m = 0.f;
   const int cpr = cols / 8;
   const long long nch = (long long)rows * cpr;
@@ -244,6 +248,7 @@ __global__ void __launch_bounds__(256) absmax_bf16_kernel(const uint16_t* __rest
 __global__ void __launch_bounds__(256) bf16_to_scaled_f16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols,
                                                                  const float* __restrict__ wmax, uint16_t* __restrict__ out,
                                                                  float* __restrict__ inv_scale) {
+  pdl_enter();
   const float m = *wmax;
   int e = 0;
   if (m > 0.f) {
@@ -272,7 +277,8 @@ __global__ void __launch_bounds__(256) bf16_to_scaled_f16_kernel(const uint16_t*
   }
 }
 
-__global__ void set_f32_kernel(float* p, float v) { *p = v; }
+__global__ void set_f32_kernel(float* p, float v) {
+  pdl_enter(); *p = v; }
 
 // ------------------------------------------------------------------------------------------------
 // host side
@@ -514,6 +520,10 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
   // side stream beside it (one CTA per block leaves SMs idle) and joins before the transform pass, which reads bf16(M)^T.  Event record / wait pairs only, so
   // the fork and the join are captured with the step when the caller's stream is being captured.
   LyAux* aux = (nbP > 0 && g_ly_dual.load(std::memory_order_relaxed) && w_mn_expected(k)) ? ly_aux() : nullptr;
+  // Inverse and penalty take one CTA per block.  Where they do not fit side by side, a programmatic launch hurts: CTAs that
+  // wait for the kernel before them take SMs from the penalty, and the pass then starts late on those (9B-shaped, 106 + 64
+  // blocks: 372 us a step with ordinary launches, 392 without; 2B-shaped, all resident: 122 and 117).
+  const bool overlap = NB + nbP <= 148;
   cudaStream_t so = st;
   if (aux) {
     if (cudaEventRecord(aux->fork, st) != cudaSuccess || cudaStreamWaitEvent(aux->stream, aux->fork, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
@@ -537,12 +547,12 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     }
     eq4.blk0[eq4.n] = L.pair_blk0;
     eq4.n_ticks = L.n;
-    const int rc = ns_inverse(st, nullptr, L.Minv, NB, k, true, w, status, true, true, &eq4);
+    const int rc = ns_inverse(st, nullptr, L.Minv, NB, k, true, w, status, true, true, &eq4, overlap);
     if (rc) return rc;
   }
   if (nbP > 0) {
     // the penalty's norm and (M M^T - I) M from the splits of the fp32 parameters
-    const int rc = penalty_tc(so, w.Ab + offP, w.Pl + offP, L.RM, any_lambda, L.orth_sq, 1, nbP, k, status);
+    const int rc = penalty_tc(so, w.Ab + offP, w.Pl + offP, L.RM, any_lambda, L.orth_sq, 1, nbP, k, status, overlap);
     if (rc) return rc;
   }
   if (aux && cudaEventRecord(aux->join, aux->stream) != cudaSuccess) return CAFEQ_ERR_CUDA;
@@ -593,7 +603,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     if (dual) {
       int ti = kt_begin(5, st);
       g_launches.fetch_add(1, std::memory_order_relaxed);
-      int rc = bd_launch_dual(st, k, L.g, subs[0], ns[0], subs[1], ns[1]);
+      int rc = bd_launch_dual(st, k, L.g, subs[0], ns[0], subs[1], ns[1], overlap);
       kt_end(ti, st);
       if (rc) return rc;
     } else {
@@ -628,7 +638,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
       ++np;
     }
     g.status = status;
-    if (np) CQ_LAUNCH(layer_lse_kernel, dim3(grid_for(nmax, 256, 148 * 4), np), 256, 0, st, g);
+    if (np) CQ_LAUNCH_IF(overlap, layer_lse_kernel, dim3(grid_for(nmax, 256, 148 * 4), np), 256, 0, st, g);
   }
   // sparse backward, fp16 single-term form: all matrices of one (axis, orientation) in one launch; when the layer has
   // exactly one input-axis and one output-axis group, both in the same launch
@@ -676,7 +686,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     if (dual) {
       int ti = kt_begin(2, st);
       g_launches.fetch_add(1, std::memory_order_relaxed);
-      int rc = bw_launch_dual(st, k, ci & 1, subs[ci], cnt[ci], co & 1, subs[co], cnt[co]);
+      int rc = bw_launch_dual(st, k, ci & 1, subs[ci], cnt[ci], co & 1, subs[co], cnt[co], overlap);
       kt_end(ti, st);
       if (rc) return rc;
     } else {
@@ -713,7 +723,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     cp.blk0[ns] = L.pair_blk0;
     cp.n = ns;
     cp.X = L.Minv;
-    const int rc = minv_path_tc(st, L.Minv, L.gMinv, L.grad, NB, k, w, status, &cp);
+    const int rc = minv_path_tc(st, L.Minv, L.gMinv, L.grad, NB, k, w, status, &cp, overlap);
     if (rc) return rc;
   }
   if (aux && cudaStreamWaitEvent(st, aux->join, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
@@ -741,7 +751,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     f.Ab = w.Ab; f.Pl = w.Pl; f.gMinv = L.gMinv;
     f.zone_next = reinterpret_cast<uint4*>(L.zone + (L.zone_cur ^ 1) * L.zone_bytes); f.zone_n16 = (long long)(L.zone_bytes / 16);
     f.status = status;
-    CQ_LAUNCH(layer_finish_kernel, dim3(grid_for(nmax / 4, 256, 148 * 4), L.n), 256, 0, st, f);
+    CQ_LAUNCH_IF(overlap, layer_finish_kernel, dim3(grid_for(nmax / 4, 256, 148 * 4), L.n), 256, 0, st, f);
   }
   ly_use_zone(L, L.zone_cur ^ 1);
   return CAFEQ_OK;

@@ -114,3 +114,11 @@ def test_small_inverse(cq, k):
     M[4, :, 5] = 0.0
     out = cq.cafeq_proxy_loss_fwd_bwd(W, f32_dev(M), bits=4, group=0, flags=cq.FLAG_NO_GRAD)
     assert int(out["status"].item()) == 5                   # singular block
+
+
+# group widths of every variant of the fused gradient split (one lane's vector to a warp's eight), with and without replicas
+@pytest.mark.parametrize("k,r,h,d1,d3,g1,g2", [(64, 1, 128, 256, 192, 32, 32), (64, 2, 256, 256, 128, 256, 512), (64, 4, 256, 1024, 64, 1024, 1024),
+                                               (64, 1, 128, 192, 128, 96, 128)])
+def test_pair_ste_group_widths(cq, k, r, h, d1, d3, g1, g2):
+    import test_gpu_pqe_ste as pqe
+    pqe.test_pqe_ste_gradient_matches_oracle(cq, k, r, h, d1, d3, g1, g2, 4, False)
