@@ -134,6 +134,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // and waits again (expected: success).  result[0] = 1 when the first wait gave up, result[1] = 1 when the second
 // succeeded.  Nothing here can block: both waits are bounded and the only arrival is the thread's own.
 __global__ void wait_probe_kernel(uint64_t limit_ns, int32_t* status, int* result) {
+  pdl_enter();
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {

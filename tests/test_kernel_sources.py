@@ -1,0 +1,52 @@
+"""Rules that every kernel of the library keeps because all of them are launched with programmatic stream serialisation,
+checked on the sources (what they prevent is a race: it shows on a device now and then or never)."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_19705_b200", "csrc")
+
+
+def _strip(text):
+    text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
+    return re.sub(r"//[^\n]*", " ", text)
+
+
+def _close(text, i, pair):
+    depth = 0
+    for j in range(i, len(text)):
+        depth += (text[j] == pair[0]) - (text[j] == pair[1])
+        if depth == 0:
+            return j
+    raise ValueError("unbalanced source")
+
+
+def _functions(marker):
+    """(file, name, body) of every function defined after `marker`."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        text = _strip(open(path).read())
+        for m in re.finditer(marker, text):
+            head = re.compile(r"(\w+)\s*\(").search(text, m.end())
+            while head.group(1) in ("__launch_bounds__", "__align__"):
+                head = re.compile(r"(\w+)\s*\(").search(text, _close(text, head.end() - 1, "()") + 1)
+            end = _close(text, head.end() - 1, "()")
+            if text[end + 1:].lstrip()[:1] != "{":
+                continue  # a declaration
+            body = text.index("{", end)
+            out.append((os.path.basename(path), head.group(1), text[body + 1:_close(text, body, "{}")].strip()))
+    return out
+
+
+KERNELS = _functions(r"__global__")
+
+
+def test_kernels_are_found():
+    assert len(KERNELS) > 60 and {"ns_block_kernel", "bd_pass_kernel", "wait_probe_kernel"} <= {n for _, n, _ in KERNELS}
+
+
+@pytest.mark.parametrize("file,name,body", KERNELS, ids=[f"{f}-{n}" for f, n, _ in KERNELS])
+def test_kernel_waits_for_its_predecessor_first(file, name, body):
+    assert re.match(r"pdl_(enter|wait)\(\);", body), f"{name} does not begin with the wait for the kernel before it"
