@@ -559,7 +559,7 @@ __global__ void bf16_to_f32_kernel(const uint16_t* __restrict__ W, long long ld,
 __global__ void resid_sq_kernel(float* __restrict__ R, const float* __restrict__ P, long long n, double* acc,
                                 const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ double red[32];
   double local = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {

@@ -112,7 +112,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
   using C = BwCfg<K, F16>;
   static_assert(K == 128 || K == 256, "block size");
   int32_t* const status = mp.p[0].status;
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   const int total_tiles = mp.tile_end[mp.n - 1];
   const int t_begin = (int)(((long long)cta * total_tiles) / ncta);
   const int t_end = (int)(((long long)(cta + 1) * total_tiles) / ncta);

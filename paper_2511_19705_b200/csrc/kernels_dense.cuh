@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
                                                          uint16_t* __restrict__ t3 = nullptr) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ uint32_t tile[64][65];
   __shared__ uint16_t tile3[64][66];
   const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* __rest
                                                              const float* __restrict__ usel, const int* __restrict__ idx, float qmax,
                                                              uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   const int l = threadIdx.x % LPG;
   const long long total = (long long)rows * ng;
   const long long w = (blockIdx.x * 256ll + threadIdx.x) / LPG;
@@ -276,7 +276,7 @@ __global__ void ste_scale_coef_kernel(const float* __restrict__ gD, long long ld
                                       const float* __restrict__ a, const float* __restrict__ usel, int gm,
                                       float* __restrict__ coef, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= (long long)rows * ng) return;

@@ -312,7 +312,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
   static_assert(FORM == BD_IN || K >= 128, "output-axis form needs k >= 128");
   static_assert(G == 64 || G == 128, "group size");
   int32_t* const status = mp.p[0].status;
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
 
   // persistent CTA: a contiguous run of tiles in (sub-problem, major, minor) order; the operator block is reloaded
   // when the run crosses into the next major or the next sub-problem
@@ -1162,7 +1162,7 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
 __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* __restrict__ T, uint16_t* __restrict__ out, int k, int transpose,
                                                                int paired, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ float tile[32][33];
   const size_t base = (size_t)blockIdx.z * k * k;
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;  // tile of the output
@@ -1210,7 +1210,7 @@ __global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* __rest
                                                           uint16_t* __restrict__ Y, int rows, int d_in, int k, int r, int transposed,
                                                           const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ float ps[256 * 33];
   __shared__ float4 xs4[256 * AS_ROWS / 4];
   float* xs = reinterpret_cast<float*>(xs4);

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgParams p) {
   pdl_enter();
   using C = TgCfg<BN>;
-  if (p.status && *p.status) return;
+  if (cta_stopped(p.status)) return;
   if (tg_stopped(p)) return;
 
   extern __shared__ uint8_t smem_raw[];
@@ -425,7 +425,7 @@ tc_block_kernel(const __grid_constant__ TbMaps maps, const TbTerms tt, const TgP
   pdl_enter();
   using C = TbCfg<K>;
   static_assert(K == 128 || K == 256, "block size");
-  if (p.status && *p.status) return;
+  if (cta_stopped(p.status)) return;
   const int b = blockIdx.x;
 
   extern __shared__ uint8_t smem_raw[];
@@ -786,7 +786,7 @@ __global__ void __launch_bounds__(256) split_bf16_kernel(const float* __restrict
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
                                                          uint16_t* __restrict__ tlo, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ uint32_t tile[32][33];
   const size_t base = (size_t)blockIdx.z * k * k;
   const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;

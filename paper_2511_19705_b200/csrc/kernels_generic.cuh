@@ -54,6 +54,12 @@ __device__ __forceinline__ float round_to_bf16(float x) { return __bfloat162floa
 __device__ __forceinline__ void raise_status(int32_t* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
+// Whether an earlier failure lets this CTA skip its work: one answer for all its threads.  Another CTA of the same launch, or a
+// kernel on a side stream, may raise the word at any time; threads that each looked for themselves could disagree, and the
+// ones that went on would wait at barriers (or on tensor memory) for the ones that had left.
+__device__ __forceinline__ bool cta_stopped(const int32_t* status) {
+  return __syncthreads_or(status && *(const volatile int32_t*)status) != 0;
+}
 
 __device__ __forceinline__ double block_sum_double(double v, double* sh) {
   // sh: at least 32 doubles of shared memory
@@ -125,7 +131,7 @@ struct GemmArgs {
 template <bool ABF, bool BBF>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
   pdl_enter();
-  if (g.status && *g.status) return;
+  if (cta_stopped(g.status)) return;
   constexpr int BM = 64, BN = 64, BK = 16;
   __shared__ float As[BK][BM + 4];
   __shared__ float Bs[BK][BN + 4];
@@ -303,7 +309,7 @@ __device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* s
 __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out,
                                                              float* __restrict__ cnorm, int k, int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   extern __shared__ float sm[];  // 3 k words
   const int tid = threadIdx.x, nt = blockDim.x;
   const float* A0 = Min + (size_t)blockIdx.x * k * k;
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __rest
 __global__ void absmax_kernel(const float* __restrict__ U, long long ld, int rows, int ng, int g,
                               float* __restrict__ a, float* __restrict__ usel, int* __restrict__ idx, int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)rows * ng;
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict_
                                                           float* __restrict__ Uhat, int8_t* __restrict__ codes,
                                                           float* __restrict__ scales, int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   const int cols = ng * g;
   const int l = threadIdx.x % LPG;
   const long long total = (long long)rows * ng;
@@ -551,7 +557,7 @@ __global__ void surrogate_rows_kernel(const float* __restrict__ a, const float* 
                                       float* __restrict__ Agrp, float* __restrict__ A, double* __restrict__ acc,
                                       const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ double red[32];
   int row = blockIdx.x * blockDim.x + threadIdx.x;
   double local = 0.0;
@@ -609,7 +615,7 @@ __global__ void ste_scale_path_kernel(const float* __restrict__ U, const float* 
                                       const void* __restrict__ offsets, int off_kind, int cols, float* __restrict__ coef,
                                       const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= (long long)rows * ng) return;
@@ -667,7 +673,7 @@ __global__ void __launch_bounds__(256) scatter_in_kernel(const uint16_t* __restr
                                                          const int* __restrict__ idx, float* __restrict__ gradT,
                                                          int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   extern __shared__ float acc[];  // [k][SCATTER_JS]
   const int B = blockIdx.x, js = blockIdx.y * SCATTER_JS;
   const int r0 = blockIdx.z * rows_per_cta, r1 = min(d_out, r0 + rows_per_cta);
@@ -701,7 +707,7 @@ __global__ void __launch_bounds__(256) scatter_out_kernel(const uint16_t* __rest
                                                           const int* __restrict__ idx, float* __restrict__ gradT,
                                                           int transpose_out, int groups_per_cta, const int32_t* status, int gm) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   extern __shared__ float acc[];  // [k][SCATTER_JS]
   const int B = blockIdx.x, js = blockIdx.y * SCATTER_JS;
   const int ng = d_in / g;
@@ -750,7 +756,7 @@ __global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t
                                                                   const int* __restrict__ idx, float* __restrict__ gradT,
                                                                   int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   extern __shared__ float acc[];  // [k][64]
   const int B = blockIdx.x, js = blockIdx.y * SC2_JS;
   const int r0 = blockIdx.z * rows_per_cta, r1 = min(d_out, r0 + rows_per_cta);
@@ -827,7 +833,7 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
                                                                    const int* __restrict__ idx, float* __restrict__ gradT,
                                                                    int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   constexpr int TPB = 256 / K;      // threads per bucket
   constexpr int CPT = STRIP / TPB;  // strip columns per thread
   constexpr int SP = STRIP + 1;     // padded row of the staging buffer
@@ -983,7 +989,7 @@ __global__ void __launch_bounds__(256) scatter_out_strip_kernel(const uint16_t* 
                                                                 const int* __restrict__ idx, float* __restrict__ gradT,
                                                                 int transpose_out, int groups_per_cta, const int32_t* status, int gm) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   constexpr int RW = K / 8;  // rows of the block per warp
   extern __shared__ __align__(16) uint16_t tiles[];  // two tiles [64][g + 4]
   __shared__ float s_cf[2][K];
@@ -1178,7 +1184,7 @@ __global__ void adam_update_kernel(float* __restrict__ M, const float* __restric
 __global__ void sqsum_bf16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols, double* acc,
                                   const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ double red[32];
   double local = 0.0;
   if ((cols % 8) == 0 && (ld % 8) == 0 && ((uintptr_t)W % 16) == 0) {
@@ -1218,7 +1224,7 @@ __global__ void max_f32_kernel(const float* __restrict__ a, long long n, float* 
                                const int32_t* status) {
   pdl_enter();
   // a >= 0, so an integer atomicMax on the bit pattern orders correctly
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   float m = 0.f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     m = fmaxf(m, a[i]);
@@ -1229,7 +1235,7 @@ __global__ void max_f32_kernel(const float* __restrict__ a, long long n, float* 
 __global__ void sumexp_kernel(const float* __restrict__ a, long long n, const float* __restrict__ amax, float t,
                               double* __restrict__ acc, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ double red[32];
   const float mx = *amax;
   double local = 0.0;
@@ -1258,7 +1264,7 @@ __global__ void lse_coef_kernel(const float* __restrict__ a, const float* __rest
 __global__ void max2_f32_kernel(const float* __restrict__ a1, long long n1, const float* __restrict__ a2, long long n2,
                                 float* __restrict__ out_max, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   float m = 0.f;
   const long long n = n1 + n2;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -1270,7 +1276,7 @@ __global__ void max2_f32_kernel(const float* __restrict__ a1, long long n1, cons
 __global__ void sumexp2_kernel(const float* __restrict__ a1, long long n1, const float* __restrict__ a2, long long n2,
                                const float* __restrict__ amax, float t, double* __restrict__ acc, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ double red[32];
   const float mx = *amax;
   double local = 0.0;

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1)
 ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsParams p) {
   pdl_wait();  // (releases at its end: a layer's penalty chain shares the SMs with it, which waiting CTAs of the pass would take)
   using C = NsCfg<K>;
-  if (p.status && *p.status) return;
+  if (cta_stopped(p.status)) return;
   const int b = blockIdx.x, row_b = b * K;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -491,7 +491,7 @@ static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uin
 __global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* __restrict__ A, int k, uint16_t* __restrict__ hi,
                                                             uint16_t* __restrict__ lo, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   __shared__ uint16_t tile[32][34];
   const size_t base = (size_t)blockIdx.z * k * k;
   const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(ChainCfg<K>::THREADS, 1)
 kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainParams p) {
   pdl_enter();
   using C = ChainCfg<K>;
-  if (p.status && *p.status) return;
+  if (cta_stopped(p.status)) return;
   const int b = blockIdx.x, row_b = b * K;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);

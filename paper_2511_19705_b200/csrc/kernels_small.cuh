@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(256) small_inverse_kernel(const float* __restr
                                                             uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
                                                             uint16_t* __restrict__ tlo, int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   constexpr int R = K / 32, CW = K / 8;
   __shared__ float tile[K][K + 1];
   __shared__ float fcol[2][K];
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(K * K / 16) small_chain_kernel(const float* __
                                                                  const float* __restrict__ A, const float* __restrict__ Agrp, int g,
                                                                  float scale, float* __restrict__ G, const int32_t* status) {
   pdl_enter();
-  if (status && *status) return;
+  if (cta_stopped(status)) return;
   constexpr int N = K * K / 16, T = K / 4;
   __shared__ float4 xs4[K][T + 1], gs4[K][T + 1];
   const int tid = threadIdx.x, ti = tid / T, tj = tid % T;

@@ -91,7 +91,7 @@ struct LyLseArgs {
 
 __global__ void __launch_bounds__(256) layer_lse_kernel(const LyLseArgs g) {
   pdl_enter();
-  if (g.status && *g.status) return;
+  if (cta_stopped(g.status)) return;
   __shared__ double red[32];
   const int p = blockIdx.y;
   const float mx = fmaxf(*g.vmax[p][0], *g.vmax[p][1]);

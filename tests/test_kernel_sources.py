@@ -50,3 +50,15 @@ def test_kernels_are_found():
 @pytest.mark.parametrize("file,name,body", KERNELS, ids=[f"{f}-{n}" for f, n, _ in KERNELS])
 def test_kernel_waits_for_its_predecessor_first(file, name, body):
     assert re.match(r"pdl_(enter|wait)\(\);", body), f"{name} does not begin with the wait for the kernel before it"
+
+
+# functions that meet at a barrier or exchange values between lanes, directly or in what they call
+COLLECTIVE = re.compile(r"__syncthreads|__syncwarp|_sync\(|mbar_|block_sum_double|gauss_jordan|pw_norm2")
+
+
+@pytest.mark.parametrize("file,name,body", [f for f in KERNELS + _functions(r"__device__ __forceinline__ void(?= bd_)") if COLLECTIVE.search(f[2])],
+                         ids=lambda v: v if isinstance(v, str) and len(v) < 40 else "")
+def test_a_block_stops_as_a_whole(file, name, body):
+    """The status word may be raised while a block starts.  Threads that looked at it one by one could disagree, and those
+    that went on would wait at barriers for the ones that left."""
+    assert not re.search(r"if \([^;{]*\*\s*(\w+\.)?status\)", body), f"{name}: every thread reads the status word for itself"
