@@ -15,7 +15,7 @@ namespace cafeq {
 constexpr float LEARN_LAMBDA = 0.5f;  // final weight of the push towards {0, 1}
 
 // rho = x - floor(x), x = fl(u / s) (the quantiser's own fp32 quotient)
-__global__ void offsets_init_kernel(const float* __restrict__ U, int rows, int cols, int g, const float* __restrict__ a, float qmax,
+__global__ void offsets_init_kernel(const float* U, int rows, int cols, int g, const float* a, float qmax,
                                     float* __restrict__ rho) {
   pdl_enter();
   const int ng = cols / g;
@@ -29,7 +29,7 @@ __global__ void offsets_init_kernel(const float* __restrict__ U, int rows, int c
 }
 
 // Bf[B k + j][y] = sum_rep V[y][(B r + rep) k + j]   (V [d3, r h] -> Bf [h, d3]); any k
-__global__ void fold_t_any_kernel(const float* __restrict__ V, int d3, int h, int k, int r, float* __restrict__ Bf) {
+__global__ void fold_t_any_kernel(const float* V, int d3, int h, int k, int r, float* __restrict__ Bf) {
   pdl_enter();
   const long long n = (long long)h * d3;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -42,7 +42,7 @@ __global__ void fold_t_any_kernel(const float* __restrict__ V, int d3, int h, in
 }
 
 // out[row] = scale * sum_c X[row][c]^2, one warp per row
-__global__ void row_sumsq_kernel(const float* __restrict__ X, int rows, int cols, float scale, float* __restrict__ out) {
+__global__ void row_sumsq_kernel(const float* X, int rows, int cols, float scale, float* __restrict__ out) {
   pdl_enter();
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -60,8 +60,8 @@ __global__ void row_sumsq_kernel(const float* __restrict__ X, int rows, int cols
 // the entries that have an offset (not the group's arg-max, scale > 0, curvature > 0), zero elsewhere.  H is indexed
 // by the row (hrow = 1) or by the column folded over the replicas (hrow = 0: column l of [., r h] uses
 // H[(l / (r k)) k + l mod k]).
-__global__ void offsets_direction_kernel(const float* gX /* may be d_rho */, const float* __restrict__ U, int rows, int cols, int g,
-                                         const float* __restrict__ a, float qmax, const float* __restrict__ H, int hrow, int k,
+__global__ void offsets_direction_kernel(const float* gX /* may be d_rho */, const float* U, int rows, int cols, int g,
+                                         const float* a, float qmax, const float* H, int hrow, int k,
                                          int r, float* d_rho, float* __restrict__ d_val) {
   pdl_enter();
   const int ng = cols / g;
@@ -84,8 +84,8 @@ __global__ void offsets_direction_kernel(const float* gX /* may be d_rho */, con
 }
 
 // rho <- clip(rho - alpha d, 0, 1) with the exact line-search step alpha = <R, D> / <D, D> (0 when D = 0)
-__global__ void offsets_step_kernel(float* __restrict__ rho, const float* __restrict__ d_rho, long long n, const double* __restrict__ rd,
-                                    const double* __restrict__ dd) {
+__global__ void offsets_step_kernel(float* __restrict__ rho, const float* d_rho, long long n, const double* rd,
+                                    const double* dd) {
   pdl_enter();
   const float alpha = (*dd > 0.0) ? (float)(*rd / *dd) : 0.f;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)

@@ -547,7 +547,7 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
   kt_end(ti, st);
 }
 
-__global__ void bf16_to_f32_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols, float* __restrict__ U) {
+__global__ void bf16_to_f32_kernel(const uint16_t* W, long long ld, int rows, int cols, float* __restrict__ U) {
   pdl_enter();
   const long long n = (long long)rows * cols;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -556,7 +556,7 @@ __global__ void bf16_to_f32_kernel(const uint16_t* __restrict__ W, long long ld,
   }
 }
 
-__global__ void resid_sq_kernel(float* __restrict__ R, const float* __restrict__ P, long long n, double* acc,
+__global__ void resid_sq_kernel(float* __restrict__ R, const float* P, long long n, double* acc,
                                 const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;

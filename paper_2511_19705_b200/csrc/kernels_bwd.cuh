@@ -86,7 +86,7 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N, int a_mn_maj
 
 // power of two that brings max |coef| just below 2^14 (fp16 holds up to 65504); 1 when there is nothing to scale
 __device__ __forceinline__ float bw_coef_scale(const float* coefmax) {
-  const float m = coefmax ? __ldg(coefmax) : 0.f;
+  const float m = coefmax ? ld_plain(coefmax) : 0.f;
   if (!(m > 0.f) || !(m < 3.0e38f)) return 1.f;
   int e;
   frexpf(m, &e);  // m = f * 2^e, f in [0.5, 1)
@@ -318,7 +318,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
           }
         } else {
           rawC = 0.f;
-          if (pi >= 0) { rawC = __ldg(p.coef + pi); rawI = __ldg(p.idx + pi); }
+          if (pi >= 0) { rawC = ld_plain(p.coef + pi); rawI = ld_plain(p.idx + pi); }
         }
         advance(ahead);
       }
@@ -355,7 +355,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
       if (!okw) return false;
       tc_fence_after();
       float mul = 1.f;
-      if constexpr (F16) mul = (p.w_inv_scale ? __ldg(p.w_inv_scale) : 1.f) / bw_coef_scale(p.coefmax);
+      if constexpr (F16) mul = (p.w_inv_scale ? ld_plain(p.w_inv_scale) : 1.f) / bw_coef_scale(p.coefmax);
       if (p.out_div) mul = (float)((double)mul / *p.out_div);
       float* out = p.gradT + (size_t)(major / p.r) * K * K;
       constexpr int CH = (K == 256) ? 8 : 2;  // 32-column chunks per thread

@@ -18,8 +18,8 @@ namespace cafeq {
 // One 64 x 64 tile per CTA (grid: C / 64, R / 64; every caller's sizes are multiples of 64).  Memory-bound: two values per
 // thread and access, so that every row of a tile is a 128-byte line in both orders (one value each, 32 x 32 tiles: 22 us for
 // the two row-major terms of 3584 x 2048, 9 us here).
-__global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict__ X, int R, int C, long long ld, float scale,
-                                                         const double* __restrict__ inv_scale, float* __restrict__ Y,
+__global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, int C, long long ld, float scale,
+                                                         const double* inv_scale, float* __restrict__ Y,
                                                          float* __restrict__ YT, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
                                                          uint16_t* __restrict__ thi, uint16_t* __restrict__ tlo,
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
   const bool trans = thi || tlo || YT;
   float2 x2[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) x2[q] = __ldg(reinterpret_cast<const float2*>(X + (long long)(r0 + ty + 8 * q) * ld + c0 + 2 * tx));
+  for (int q = 0; q < 8; ++q) x2[q] = ld_plain(reinterpret_cast<const float2*>(X + (long long)(r0 + ty + 8 * q) * ld + c0 + 2 * tx));
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int i = ty + 8 * q;
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* __restrict
 
 // Bf[B*k + j][y] = sum_rep V[y][(B*r + rep)*k + j]: fold the r replicas of every block of the inner dimension
 // and transpose (V fp32 [d3, r*h] -> Bf fp32 [h, d3]).  grid: ceil(d3/32), h/32 (k % 32 == 0); block 32 x 8.
-__global__ void __launch_bounds__(256) fold_transpose_kernel(const float* __restrict__ V, int d3, int h, int k, int r,
+__global__ void __launch_bounds__(256) fold_transpose_kernel(const float* V, int d3, int h, int k, int r,
                                                              float* __restrict__ Bf) {
   pdl_enter();
   __shared__ float tile[32][33];
@@ -108,13 +108,13 @@ __global__ void __launch_bounds__(256) fold_transpose_kernel(const float* __rest
 
 // V[y][(B*r + rep)*k + j] = scale * X[y][B*k + j]  (X fp32 [d3, h] -> V fp32 [d3, r*h]; k % 4 == 0).  grid: (ceil(h / 1024),
 // d3); a thread reads four entries once and writes every replica (60 -> 12 us at 3584 x 4096).
-__global__ void __launch_bounds__(256) expand_cols_kernel(const float* __restrict__ X, int h, int k, int r, float scale,
+__global__ void __launch_bounds__(256) expand_cols_kernel(const float* X, int h, int k, int r, float scale,
                                                           float* __restrict__ V) {
   pdl_enter();
   const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
   if (l >= h) return;
   const long long y = blockIdx.y;
-  float4 x = __ldg(reinterpret_cast<const float4*>(X + y * h + l));
+  float4 x = ld_plain(reinterpret_cast<const float4*>(X + y * h + l));
   x = make_float4(scale * x.x, scale * x.y, scale * x.z, scale * x.w);
   const int B = l / k, j = l - B * k;
   float* v = V + y * (long long)r * h + (long long)B * r * k + j;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(256) expand_cols_kernel(const float* __restric
 }
 
 // the same for any k, one entry per thread (learned offsets take every shape)
-__global__ void expand_cols_any_kernel(const float* __restrict__ X, int d3, int h, int k, int r, float scale, float* __restrict__ V) {
+__global__ void expand_cols_any_kernel(const float* X, int d3, int h, int k, int r, float scale, float* __restrict__ V) {
   pdl_enter();
   const long long n = (long long)d3 * r * h;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -135,7 +135,7 @@ __global__ void expand_cols_any_kernel(const float* __restrict__ X, int d3, int 
 
 // bf16 hi / lo (and third) terms of the replica-folded V: F[y][B*k + j] = sum_rep V[y][(B*r + rep)*k + j], row-major [d3, h].
 // A product over the r*h expanded inner indices equals the product over the h folded ones: 1 / r of the work.
-__global__ void __launch_bounds__(256) fold_split_kernel(const float* __restrict__ V, int h, int k, int r, uint16_t* __restrict__ hi,
+__global__ void __launch_bounds__(256) fold_split_kernel(const float* V, int h, int k, int r, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ h3, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256) fold_split_kernel(const float* __restrict
   const float* v = V + y * (long long)r * h + (long long)B * r * k + j;
   float x[4] = {0.f, 0.f, 0.f, 0.f};
   for (int rep = 0; rep < r; ++rep) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(v + (long long)rep * k));
+    const float4 q = ld_plain(reinterpret_cast<const float4*>(v + (long long)rep * k));
     x[0] += q.x; x[1] += q.y; x[2] += q.z; x[3] += q.w;
   }
   uint32_t a[2], b[2], c[2];
@@ -174,8 +174,8 @@ __global__ void __launch_bounds__(256) fold_split_kernel(const float* __restrict
 
 // gX[row][G*g + idx[row, G]] += coef[row, G]: the scale path of the straight-through quantiser lands on the
 // arg-max entry of its group (records row-major)
-__global__ void add_argmax_kernel(float* __restrict__ gX, long long ld, int rows, int ng, int g, const float* __restrict__ coef,
-                                  const int* __restrict__ idx, const int32_t* status) {
+__global__ void add_argmax_kernel(float* __restrict__ gX, long long ld, int rows, int ng, int g, const float* coef,
+                                  const int* idx, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
   const long long n = (long long)rows * ng;
@@ -193,9 +193,9 @@ __global__ void add_argmax_kernel(float* __restrict__ gX, long long ld, int rows
 // it in registers.  3584 x 4096 + 2048 x 3584: expansion, scale path with two divisions per value, arg-max addition and split
 // 190 us as seven launches, 60 us here as two.
 template <int LPG, int NV>
-__global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* __restrict__ U, const float* __restrict__ gX, long long ldg, int rows,
-                                                             int ng, int g, int k, int r, const float* __restrict__ a,
-                                                             const float* __restrict__ usel, const int* __restrict__ idx, float qmax,
+__global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* U, const float* gX, long long ldg, int rows,
+                                                             int ng, int g, int k, int r, const float* a,
+                                                             const float* usel, const int* idx, float qmax,
                                                              uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -213,13 +213,13 @@ __global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* __rest
     const int e = (l + i * LPG) * 4;
     u4[i] = d4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (e < g) {
-      u4[i] = __ldg(reinterpret_cast<const float4*>(U + u0 + e));
+      u4[i] = ld_plain(reinterpret_cast<const float4*>(U + u0 + e));
       int col = G * g + e;
       if (r > 1) {
         const int b = col / k;
         col = (b / r) * k + (col - b * k);
       }
-      d4[i] = __ldg(reinterpret_cast<const float4*>(gr + col));
+      d4[i] = ld_plain(reinterpret_cast<const float4*>(gr + col));
     }
   }
   const float av = a[wc], us = usel[wc];
@@ -271,9 +271,9 @@ __global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* __rest
 // derivative of Uhat with respect to the scale is q - U / s = Delta / s, and s = a / qmax, so the coefficient routed
 // to the group's arg-max entry is sign(U at arg-max) / qmax * sum_e gDelta_e Delta_e / s = sign * sum_e gDelta_e Delta_e / a.
 // Delta comes as a two-term bf16 split (row pitch ldd); records are group-major when gm is set.  One warp per record.
-__global__ void ste_scale_coef_kernel(const float* __restrict__ gD, long long ldg, const uint16_t* __restrict__ Dh,
-                                      const uint16_t* __restrict__ Dl, long long ldd, int rows, int ng, int g,
-                                      const float* __restrict__ a, const float* __restrict__ usel, int gm,
+__global__ void ste_scale_coef_kernel(const float* gD, long long ldg, const uint16_t* Dh,
+                                      const uint16_t* Dl, long long ldd, int rows, int ng, int g,
+                                      const float* a, const float* usel, int gm,
                                       float* __restrict__ coef, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -298,7 +298,7 @@ __global__ void ste_scale_coef_kernel(const float* __restrict__ gD, long long ld
 }
 
 // acc += sum x[i] y[i]  (fp32 products summed in double; one atomic per block)
-__global__ void __launch_bounds__(256) dot_f32_kernel(const float* __restrict__ x, const float* __restrict__ y, long long n,
+__global__ void __launch_bounds__(256) dot_f32_kernel(const float* x, const float* y, long long n,
                                                       double* acc) {
   pdl_enter();
   __shared__ double red[32];
@@ -334,7 +334,7 @@ __device__ __forceinline__ double pw_norm2(const float* v, int C, double* red) {
   __syncthreads();
   return out;
 }
-__global__ void __launch_bounds__(256) pw_rows_kernel(const float* __restrict__ S, const float* __restrict__ v, float* __restrict__ clear,
+__global__ void __launch_bounds__(256) pw_rows_kernel(const float* S, const float* v, float* __restrict__ clear,
                                                       int R, int C, float* __restrict__ u) {
   pdl_enter();
   __shared__ double red[32];
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(256) pw_rows_kernel(const float* __restrict__ 
   if (lane == 0) u[w] = s * inv;
 }
 // grid: (ceil(C / 256), ceil(R / 32)); v2 cleared two launches before
-__global__ void __launch_bounds__(256) pw_cols_kernel(const float* __restrict__ S, const float* __restrict__ u, int R, int C,
+__global__ void __launch_bounds__(256) pw_cols_kernel(const float* S, const float* u, int R, int C,
                                                       float* __restrict__ v2) {
   pdl_enter();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(256) pw_cols_kernel(const float* __restrict__ 
   for (int r = 0; r < n; ++r) s = fmaf(S[(long long)(r0 + r) * C + j], u[r0 + r], s);
   atomicAdd(&v2[j], s);
 }
-__global__ void __launch_bounds__(256) pw_result_kernel(const float* __restrict__ v, int C, double safety, const double* fro2, double* sig2) {
+__global__ void __launch_bounds__(256) pw_result_kernel(const float* v, int C, double safety, const double* fro2, double* sig2) {
   pdl_enter();
   __shared__ double red[32];
   const double n = sqrt(pw_norm2(v, C, red));
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) pw_result_kernel(const float* __restrict_
   }
 }
 
-__global__ void sqrt_hist_kernel(const double* __restrict__ sq, float* __restrict__ out, int n) {
+__global__ void sqrt_hist_kernel(const double* sq, float* __restrict__ out, int n) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (float)sqrt(fmax(sq[i], 0.0));

@@ -591,7 +591,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
           for (int gi = 0; gi < NG; ++gi) wgt[gi] = 0.f;
           if ((p.epi & EPI_SURR) && valid) {
 #pragma unroll
-            for (int gi = 0; gi < NG; ++gi) wgt[gi] = (FORM == BD_IN) ? __ldg(p.cw + col0 / G + gi) : __ldg(p.cw + row);
+            for (int gi = 0; gi < NG; ++gi) wgt[gi] = (FORM == BD_IN) ? ld_plain(p.cw + col0 / G + gi) : ld_plain(p.cw + row);
           }
         }
         ok = __all_sync(0xffffffffu, mbar_wait(bar_accf + 8 * buf, aph, abort_flag, status));
@@ -1159,7 +1159,7 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
 // per CTA (grid: (k / 32, k / 32, blocks)), rows read and written along their elements.  Latency-bound: one load, one store
 // (14 blocks of 256: 5 - 7 us with a strided walk and 64-bit divisions per element, 3 us here).
 // paired (k = 32): blocks 2 i and 2 i + 1 become one 64 x 64 block, zeros off the diagonal.
-__global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* __restrict__ T, uint16_t* __restrict__ out, int k, int transpose,
+__global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* T, uint16_t* __restrict__ out, int k, int transpose,
                                                                int paired, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -1170,11 +1170,11 @@ __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* __re
   const float* src = T + base + (transpose ? (size_t)(c0 + i) * k + r0 + j : (size_t)(r0 + i) * k + c0 + j);
   float v[4];
   if (((uintptr_t)T & 15) == 0) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(src));
+    const float4 q = ld_plain(reinterpret_cast<const float4*>(src));
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
   } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) v[e] = __ldg(src + e);
+    for (int e = 0; e < 4; ++e) v[e] = ld_plain(src + e);
   }
   if (transpose) {
 #pragma unroll
@@ -1206,7 +1206,7 @@ __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* __re
 // [contraction][row]; warp w takes an eighth of the contraction, its partial sums meet in shared memory.
 // ------------------------------------------------------------------------------------------------
 constexpr int AS_ROWS = 8, AS_MAX_ROWS = 64;
-__global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* __restrict__ X, long long ld, const float* __restrict__ T,
+__global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* X, long long ld, const float* T,
                                                           uint16_t* __restrict__ Y, int rows, int d_in, int k, int r, int transposed,
                                                           const int32_t* status) {
   pdl_enter();
@@ -1223,7 +1223,7 @@ __global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* __rest
 #pragma unroll 8
     for (int m = tid >> 3; m < k; m += 32) {
       const int n = (tid & 7) * 4;
-      const float4 q = __ldg(reinterpret_cast<const float4*>(Tb + (size_t)m * k + n0 + n));
+      const float4 q = ld_plain(reinterpret_cast<const float4*>(Tb + (size_t)m * k + n0 + n));
       float* d = ps + m * 33 + n;
       d[0] = round_to_bf16(q.x); d[1] = round_to_bf16(q.y); d[2] = round_to_bf16(q.z); d[3] = round_to_bf16(q.w);
     }
@@ -1232,7 +1232,7 @@ __global__ void __launch_bounds__(256) apply_small_kernel(const uint16_t* __rest
 #pragma unroll 8
     for (int e = tid; e < 32 * q4; e += 256) {
       const int n = e / q4, m = (e - n * q4) * 4;
-      const float4 q = __ldg(reinterpret_cast<const float4*>(Tb + (size_t)(n0 + n) * k + m));
+      const float4 q = ld_plain(reinterpret_cast<const float4*>(Tb + (size_t)(n0 + n) * k + m));
       float* d = ps + m * 33 + n;
       d[0] = round_to_bf16(q.x); d[33] = round_to_bf16(q.y); d[66] = round_to_bf16(q.z); d[99] = round_to_bf16(q.w);
     }

@@ -109,14 +109,14 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
       float4 cv[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        cv[i] = __ldg(reinterpret_cast<const float4*>(p.C0 + c0b + (long long)(rbase + i * 4 + r4) * p.ldc0 + nb0 + c4));
+        cv[i] = ld_plain(reinterpret_cast<const float4*>(p.C0 + c0b + (long long)(rbase + i * 4 + r4) * p.ldc0 + nb0 + c4));
 #pragma unroll
       for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + (i * 4 + r4) * 36 + c4) = cv[i];
     } else {
 #pragma unroll 1
       for (int r = 0; r < 32; ++r) {
         float x = 0.f;
-        if (rbase + r < p.M && ncol < p.N) x = __ldg(p.C0 + c0b + (long long)(rbase + r) * p.ldc0 + ncol);
+        if (rbase + r < p.M && ncol < p.N) x = ld_plain(p.C0 + c0b + (long long)(rbase + r) * p.ldc0 + ncol);
         tile[r * 36 + lane] = x;
       }
     }
@@ -782,7 +782,7 @@ static int tb_launch(cudaStream_t st, int nterms, const uint16_t* const* A, cons
 
 // fp32 blocks [nb][k][k] -> bf16 hi / lo splits in row-major and transposed order; one 32 x 32 tile per CTA
 // (grid: k/32, k/32, nb; block 32 x 8), transposed outputs staged through shared memory.  k % 32 == 0.
-__global__ void __launch_bounds__(256) split_bf16_kernel(const float* __restrict__ X, int k, uint16_t* __restrict__ hi,
+__global__ void __launch_bounds__(256) split_bf16_kernel(const float* X, int k, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
                                                          uint16_t* __restrict__ tlo, const int32_t* status) {
   pdl_enter();

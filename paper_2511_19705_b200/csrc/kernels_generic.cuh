@@ -27,6 +27,12 @@ __device__ __forceinline__ void pdl_enter() {
   pdl_release();
 }
 
+// A kernel's lifetime begins before the kernel that writes its inputs has ended, so no input is constant over it: inputs are read
+// with ordinary loads, which stay behind the wait, and `const` pointers carry no __restrict__ (with it the compiler may take the
+// read-only path, which promises that the data does not change and which nothing orders after the wait).  Outputs carry it.
+template <typename T>
+__device__ __forceinline__ T ld_plain(const T* p) { return *p; }
+
 // overlap = false: an ordinary launch, after the kernel before it (the wait then returns at once)
 template <typename... P, typename... A>
 static inline void launch_pdl_if(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
@@ -91,7 +97,7 @@ __global__ void zero_f64_kernel(double* p, int n) {
 }
 
 // out = float(bf16(in)): the operand actually fed to the transform products.
-__global__ void round_bf16_kernel(const float* __restrict__ in, float* __restrict__ out, long long n,
+__global__ void round_bf16_kernel(const float* in, float* __restrict__ out, long long n,
                                   const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -99,7 +105,7 @@ __global__ void round_bf16_kernel(const float* __restrict__ in, float* __restric
     out[i] = round_to_bf16(in[i]);
 }
 
-__global__ void copy_f32_kernel(const float* __restrict__ in, float* __restrict__ out, long long n) {
+__global__ void copy_f32_kernel(const float* in, float* __restrict__ out, long long n) {
   pdl_enter();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = in[i];
@@ -306,7 +312,7 @@ __device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* s
   return true;
 }
 
-__global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out,
+__global__ void __launch_bounds__(1024) block_inverse_kernel(const float* Min, float* __restrict__ Out,
                                                              float* __restrict__ cnorm, int k, int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* __rest
 // ------------------------------------------------------------------------------------------------
 // group absmax with arg-max (lowest index on ties): one warp per (row, group)
 // ------------------------------------------------------------------------------------------------
-__global__ void absmax_kernel(const float* __restrict__ U, long long ld, int rows, int ng, int g,
+__global__ void absmax_kernel(const float* U, long long ld, int rows, int ng, int g,
                               float* __restrict__ a, float* __restrict__ usel, int* __restrict__ idx, int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -365,7 +371,7 @@ __global__ void absmax_kernel(const float* __restrict__ U, long long ld, int row
   }
 }
 
-__global__ void scales_kernel(const float* __restrict__ a, float* __restrict__ s, long long n, float qmax,
+__global__ void scales_kernel(const float* a, float* __restrict__ s, long long n, float qmax,
                               const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -385,8 +391,8 @@ __device__ __forceinline__ float quantise_one(float u, float s, float a, float q
   return fminf(fmaxf(q, -qmax), qmax);
 }
 
-__global__ void quant_kernel(const float* __restrict__ U, long long ld, int rows, int cols, int g,
-                             const float* __restrict__ a, float qmax, const void* __restrict__ offsets, int off_kind,
+__global__ void quant_kernel(const float* U, long long ld, int rows, int cols, int g,
+                             const float* a, float qmax, const void* offsets, int off_kind,
                              float* __restrict__ Delta, float* __restrict__ Uhat, int8_t* __restrict__ codes,
                              const int32_t* status) {
   pdl_enter();
@@ -420,8 +426,8 @@ __global__ void quant_kernel(const float* __restrict__ U, long long ld, int rows
 // Needs g % 4 == 0, g <= 4 LPG NV, rows aligned to four values; the old kernels take every other shape.
 // ------------------------------------------------------------------------------------------------
 template <int LPG, int NV, typename SRC>
-__global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict__ U, long long ld, int rows, int ng, int g, float qmax,
-                                                          const void* __restrict__ offsets, int off_kind, float* __restrict__ a,
+__global__ void __launch_bounds__(256) group_quant_kernel(const SRC* U, long long ld, int rows, int ng, int g, float qmax,
+                                                          const void* offsets, int off_kind, float* __restrict__ a,
                                                           float* __restrict__ usel, int* __restrict__ idx, float* __restrict__ Delta,
                                                           float* __restrict__ Uhat, int8_t* __restrict__ codes,
                                                           float* __restrict__ scales, int32_t* status) {
@@ -444,10 +450,10 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict_
     const int e = (l + i * LPG) * 4;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (sizeof(SRC) == 4) {
-      if (e < g) q = __ldg(reinterpret_cast<const float4*>(p + e));
+      if (e < g) q = ld_plain(reinterpret_cast<const float4*>(p + e));
     } else {
       if (e < g) {
-        const uint2 h = __ldg(reinterpret_cast<const uint2*>(p + e));
+        const uint2 h = ld_plain(reinterpret_cast<const uint2*>(p + e));
         q = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xFFFF0000u), __uint_as_float(h.y << 16),
                         __uint_as_float(h.y & 0xFFFF0000u));
       }
@@ -526,7 +532,7 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const SRC* __restrict_
 // surrogate (Eq. 4 per entry): weights cw, loss, arg-max coefficients, A_t
 // ------------------------------------------------------------------------------------------------
 // axis IN:  cw[Gc] = sum_{t in group Gc} c[t'],  t' = (B / r) * k + (t mod k), B = t / k
-__global__ void cw_in_kernel(const float* __restrict__ c, int d_in, int g, int k, int r, float* __restrict__ cw) {
+__global__ void cw_in_kernel(const float* c, int d_in, int g, int k, int r, float* __restrict__ cw) {
   pdl_enter();
   int Gc = blockIdx.x * blockDim.x + threadIdx.x;
   if (Gc >= d_in / g) return;
@@ -540,7 +546,7 @@ __global__ void cw_in_kernel(const float* __restrict__ c, int d_in, int g, int k
 }
 
 // axis OUT: cw[row] = g * c[t'(row)]
-__global__ void cw_out_kernel(const float* __restrict__ c, int d_out, int g, int k, int r, float* __restrict__ cw) {
+__global__ void cw_out_kernel(const float* c, int d_out, int g, int k, int r, float* __restrict__ cw) {
   pdl_enter();
   int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= d_out) return;
@@ -551,9 +557,9 @@ __global__ void cw_out_kernel(const float* __restrict__ c, int d_out, int g, int
 // one thread per row: loss partial sum and arg-max coefficients  coef = scale * cw * a * sign(U[e*]).
 // A_t accumulation: axis IN  Agrp[Gc] += a^2 (per column group, expanded later);
 //                   axis OUT A[t'(row)] += g * sum_G a^2.
-__global__ void surrogate_rows_kernel(const float* __restrict__ a, const float* __restrict__ usel, int rows, int ng,
+__global__ void surrogate_rows_kernel(const float* a, const float* usel, int rows, int ng,
                                       int g, int axis,
-                                      const float* __restrict__ cw, float kappa, int k, int r, float* __restrict__ coef,
+                                      const float* cw, float kappa, int k, int r, float* __restrict__ coef,
                                       float* __restrict__ Agrp, float* __restrict__ A, double* __restrict__ acc,
                                       const int32_t* status) {
   pdl_enter();
@@ -587,7 +593,7 @@ __global__ void surrogate_rows_kernel(const float* __restrict__ a, const float* 
 }
 
 // axis IN: A[t'] += Agrp[group of t]
-__global__ void expand_agrp_kernel(const float* __restrict__ Agrp, int d_in, int g, int k, int r, float* __restrict__ A) {
+__global__ void expand_agrp_kernel(const float* Agrp, int d_in, int g, int k, int r, float* __restrict__ A) {
   pdl_enter();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= d_in) return;
@@ -596,7 +602,7 @@ __global__ void expand_agrp_kernel(const float* __restrict__ Agrp, int d_in, int
 }
 
 // gMinv[b][i][t] = scale * Minv[b][i][t] * A[b][t]
-__global__ void scale_cols_kernel(const float* __restrict__ Minv, const float* __restrict__ A, float scale, int k,
+__global__ void scale_cols_kernel(const float* Minv, const float* A, float scale, int k,
                                   long long n, float* __restrict__ out) {
   pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -610,9 +616,9 @@ __global__ void scale_cols_kernel(const float* __restrict__ Minv, const float* _
 // straight-through scale path: coef[row, G] = sign(U[e*]) / qmax * sum_{e in G} gDelta_e (q_e - U_e / s_G)
 // (+ optionally, for the pair PQE loss, the direct term stays in gU and is handled by a dense product)
 // ------------------------------------------------------------------------------------------------
-__global__ void ste_scale_path_kernel(const float* __restrict__ U, const float* __restrict__ gD, long long ld, int rows,
-                                      int ng, int g, const float* __restrict__ a, const float* __restrict__ usel, float qmax,
-                                      const void* __restrict__ offsets, int off_kind, int cols, float* __restrict__ coef,
+__global__ void ste_scale_path_kernel(const float* U, const float* gD, long long ld, int rows,
+                                      int ng, int g, const float* a, const float* usel, float qmax,
+                                      const void* offsets, int off_kind, int cols, float* __restrict__ coef,
                                       const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -643,8 +649,8 @@ __global__ void ste_scale_path_kernel(const float* __restrict__ U, const float* 
 
 // d loss / d rho for soft rounding offsets: Uhat = s (floor(U/s) + rho) with the scale kept, so d Uhat / d rho = s and
 // the gradient is s * gUhat; entries attaining their group's absmax are coded +-qmax whatever rho and get 0.
-__global__ void grad_offsets_kernel(const float* __restrict__ U, const float* __restrict__ gUhat, long long ld, int rows, int cols,
-                                    int g, const float* __restrict__ a, float qmax, float* __restrict__ out,
+__global__ void grad_offsets_kernel(const float* U, const float* gUhat, long long ld, int rows, int cols,
+                                    int g, const float* a, float qmax, float* __restrict__ out,
                                     const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -668,9 +674,9 @@ __global__ void grad_offsets_kernel(const float* __restrict__ U, const float* __
 // ------------------------------------------------------------------------------------------------
 constexpr int SCATTER_JS = 32;
 
-__global__ void __launch_bounds__(256) scatter_in_kernel(const uint16_t* __restrict__ W, long long ld, int d_out, int d_in,
-                                                         int g, int k, int r, const float* __restrict__ coef,
-                                                         const int* __restrict__ idx, float* __restrict__ gradT,
+__global__ void __launch_bounds__(256) scatter_in_kernel(const uint16_t* W, long long ld, int d_out, int d_in,
+                                                         int g, int k, int r, const float* coef,
+                                                         const int* idx, float* __restrict__ gradT,
                                                          int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -702,9 +708,9 @@ __global__ void __launch_bounds__(256) scatter_in_kernel(const uint16_t* __restr
   }
 }
 
-__global__ void __launch_bounds__(256) scatter_out_kernel(const uint16_t* __restrict__ W, long long ld, int d_out, int d_in,
-                                                          int g, int k, int r, const float* __restrict__ coef,
-                                                          const int* __restrict__ idx, float* __restrict__ gradT,
+__global__ void __launch_bounds__(256) scatter_out_kernel(const uint16_t* W, long long ld, int d_out, int d_in,
+                                                          int g, int k, int r, const float* coef,
+                                                          const int* idx, float* __restrict__ gradT,
                                                           int transpose_out, int groups_per_cta, const int32_t* status, int gm) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -751,9 +757,9 @@ constexpr int SC2_MAXG = 4;  // groups of one row that can fall into one block (
 // inside the accumulator the even columns sit in the first half of a row and the odd ones in the second, so both
 // atomics of a warp are bank-conflict free.  NG = groups of one row that fall into one block.
 template <int NG>
-__global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t* __restrict__ W, long long ld, int d_out,
-                                                                  int d_in, int g, int k, int r, const float* __restrict__ coef,
-                                                                  const int* __restrict__ idx, float* __restrict__ gradT,
+__global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t* W, long long ld, int d_out,
+                                                                  int d_in, int g, int k, int r, const float* coef,
+                                                                  const int* idx, float* __restrict__ gradT,
                                                                   int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -779,8 +785,8 @@ __global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t
 #pragma unroll
       for (int q = 0; q < NG; ++q) {
         const long long pq = gm ? (long long)(G0 + q) * d_out + oo : (long long)oo * ng + G0 + q;
-        const int ix = __ldg(idx + pq);
-        const float c = __ldg(coef + pq);
+        const int ix = ld_plain(idx + pq);
+        const float c = ld_plain(coef + pq);
         const int col = q * g + ix + off;
         const bool in = ok && (unsigned)col < (unsigned)k;
         cf[q] = in ? c : 0.f;
@@ -793,7 +799,7 @@ __global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int row = base + c8 + u;
-        w[u] = (row < r1) ? __ldg(Wp + row * ldw) : 0u;
+        w[u] = (row < r1) ? ld_plain(Wp + row * ldw) : 0u;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -828,9 +834,9 @@ constexpr int SCB_MAXP = 4096;
 constexpr int SCB_SORTED = 512;  // up to this many records a bucket is accumulated in row order
 
 template <int K, int STRIP>
-__global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_t* __restrict__ W, long long ld, int d_out,
-                                                                   int d_in, int g, int r, int NG, const float* __restrict__ coef,
-                                                                   const int* __restrict__ idx, float* __restrict__ gradT,
+__global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_t* W, long long ld, int d_out,
+                                                                   int d_in, int g, int r, int NG, const float* coef,
+                                                                   const int* idx, float* __restrict__ gradT,
                                                                    int transpose_out, int rows_per_cta, const int32_t* status, int gm) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -864,8 +870,8 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
     if (e < np) {
       const int row = e / NG, q = e - row * NG;
       const long long p = gm ? (long long)(G0 + q) * d_out + r0 + row : (long long)(r0 + row) * ng + G0 + q;
-      const float c = __ldg(coef + p);
-      const int col = q * g + __ldg(idx + p) + off;
+      const float c = ld_plain(coef + p);
+      const int col = q * g + ld_plain(idx + p) + off;
       if ((unsigned)col < (unsigned)K && c != 0.f) {
         bk[u] = (short)col;
         cfv[u] = c;
@@ -932,7 +938,7 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
     cf = rec_cf[p];
     const uint4* src = reinterpret_cast<const uint4*>(Wb + (long long)rec_o[p] * ld);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) w[v] = __ldg(src + v);
+    for (int v = 0; v < NV; ++v) w[v] = ld_plain(src + v);
   };
   auto accumulate = [&](const uint4* w, float cf) {
 #pragma unroll
@@ -984,9 +990,9 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 template <int K>
-__global__ void __launch_bounds__(256) scatter_out_strip_kernel(const uint16_t* __restrict__ W, long long ld, int d_out,
-                                                                int d_in, int g, int r, const float* __restrict__ coef,
-                                                                const int* __restrict__ idx, float* __restrict__ gradT,
+__global__ void __launch_bounds__(256) scatter_out_strip_kernel(const uint16_t* W, long long ld, int d_out,
+                                                                int d_in, int g, int r, const float* coef,
+                                                                const int* idx, float* __restrict__ gradT,
                                                                 int transpose_out, int groups_per_cta, const int32_t* status, int gm) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -1100,7 +1106,7 @@ __global__ void step_prep_kernel(PrepArgs a) {
 // c[b][t] = sum_i X[b][i][t]^2 for 32 columns t per CTA (grid: k/32, nb; block 32 x 8), and optionally the
 // input-axis group weights cw[Gc] += sum_{t in Gc} c[t] (cw cleared by the caller; groups are runs of g columns
 // of the concatenated blocks, r = 1)
-__global__ void __launch_bounds__(256) colnorm_cw_kernel(const float* __restrict__ X, int k, float* __restrict__ c,
+__global__ void __launch_bounds__(256) colnorm_cw_kernel(const float* X, int k, float* __restrict__ c,
                                                          float* __restrict__ cw, int g) {
   pdl_enter();
   __shared__ float part[8][33];
@@ -1131,7 +1137,7 @@ __global__ void __launch_bounds__(256) colnorm_cw_kernel(const float* __restrict
 }
 
 // dL/dMinv of Eq. 4: out[b][i][t] = scale * Minv[b][i][t] * A_t; input axis with r = 1 reads A_t = Agrp[(b k + t) / g]
-__global__ void gminv_kernel(const float* __restrict__ Minv, const float* __restrict__ A, const float* __restrict__ Agrp,
+__global__ void gminv_kernel(const float* Minv, const float* A, const float* Agrp,
                              int g, float scale, int k, long long n, float* __restrict__ out) {
   pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -1145,7 +1151,7 @@ __global__ void gminv_kernel(const float* __restrict__ Minv, const float* __rest
 // ------------------------------------------------------------------------------------------------
 // optimiser updates and bookkeeping
 // ------------------------------------------------------------------------------------------------
-__global__ void gd_update_kernel(float* __restrict__ M, const float* __restrict__ g, float lr, long long n,
+__global__ void gd_update_kernel(float* __restrict__ M, const float* g, float lr, long long n,
                                  const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -1160,7 +1166,7 @@ __global__ void adam_tick_kernel(float* state, const int32_t* status) {
   state[0] += 1.f;
 }
 
-__global__ void adam_update_kernel(float* __restrict__ M, const float* __restrict__ g, float* __restrict__ state, float lr,
+__global__ void adam_update_kernel(float* __restrict__ M, const float* g, float* __restrict__ state, float lr,
                                    float b1, float b2, float eps, long long n, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -1181,7 +1187,7 @@ __global__ void adam_update_kernel(float* __restrict__ M, const float* __restric
 // ------------------------------------------------------------------------------------------------
 // reductions: sum of squares of bf16 / fp32 arrays
 // ------------------------------------------------------------------------------------------------
-__global__ void sqsum_bf16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols, double* acc,
+__global__ void sqsum_bf16_kernel(const uint16_t* W, long long ld, int rows, int cols, double* acc,
                                   const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -1194,7 +1200,7 @@ __global__ void sqsum_bf16_kernel(const uint16_t* __restrict__ W, long long ld, 
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nch; c += (long long)gridDim.x * blockDim.x) {
       const long long row = c / cpr;
       const int cc = (int)(c - row * cpr);
-      const uint4 q = __ldg(reinterpret_cast<const uint4*>(W + row * ld) + cc);
+      const uint4 q = ld_plain(reinterpret_cast<const uint4*>(W + row * ld) + cc);
       const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
       float s = 0.f;
 #pragma unroll
@@ -1220,7 +1226,7 @@ __global__ void sqsum_bf16_kernel(const uint16_t* __restrict__ W, long long ld, 
 // ------------------------------------------------------------------------------------------------
 // pair: LogSumExp over group maxima (two passes), orthonormality penalty
 // ------------------------------------------------------------------------------------------------
-__global__ void max_f32_kernel(const float* __restrict__ a, long long n, float* __restrict__ out_max,
+__global__ void max_f32_kernel(const float* a, long long n, float* __restrict__ out_max,
                                const int32_t* status) {
   pdl_enter();
   // a >= 0, so an integer atomicMax on the bit pattern orders correctly
@@ -1232,7 +1238,7 @@ __global__ void max_f32_kernel(const float* __restrict__ a, long long n, float* 
   if ((threadIdx.x & 31) == 0) atomicMax((int*)out_max, __float_as_int(m));
 }
 
-__global__ void sumexp_kernel(const float* __restrict__ a, long long n, const float* __restrict__ amax, float t,
+__global__ void sumexp_kernel(const float* a, long long n, const float* amax, float t,
                               double* __restrict__ acc, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -1246,8 +1252,8 @@ __global__ void sumexp_kernel(const float* __restrict__ a, long long n, const fl
 }
 
 // coef[w] = exp(t (a - max)) / Z * sign(U[arg-max])
-__global__ void lse_coef_kernel(const float* __restrict__ a, const float* __restrict__ usel, long long n,
-                                const float* __restrict__ amax, float t, const double* __restrict__ Z,
+__global__ void lse_coef_kernel(const float* a, const float* usel, long long n,
+                                const float* amax, float t, const double* Z,
                                 float* __restrict__ coef, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -1261,7 +1267,7 @@ __global__ void lse_coef_kernel(const float* __restrict__ a, const float* __rest
 }
 
 // two-array forms of the three LogSumExp kernels (the group maxima of U and of V in one launch each)
-__global__ void max2_f32_kernel(const float* __restrict__ a1, long long n1, const float* __restrict__ a2, long long n2,
+__global__ void max2_f32_kernel(const float* a1, long long n1, const float* a2, long long n2,
                                 float* __restrict__ out_max, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
@@ -1273,8 +1279,8 @@ __global__ void max2_f32_kernel(const float* __restrict__ a1, long long n1, cons
   if ((threadIdx.x & 31) == 0) atomicMax((int*)out_max, __float_as_int(m));
 }
 
-__global__ void sumexp2_kernel(const float* __restrict__ a1, long long n1, const float* __restrict__ a2, long long n2,
-                               const float* __restrict__ amax, float t, double* __restrict__ acc, const int32_t* status) {
+__global__ void sumexp2_kernel(const float* a1, long long n1, const float* a2, long long n2,
+                               const float* amax, float t, double* __restrict__ acc, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
   __shared__ double red[32];
@@ -1287,9 +1293,9 @@ __global__ void sumexp2_kernel(const float* __restrict__ a1, long long n1, const
   if (threadIdx.x == 0) atomicAdd(acc, s);
 }
 
-__global__ void lse_coef2_kernel(const float* __restrict__ a1, const float* __restrict__ u1, float* __restrict__ c1, long long n1,
-                                 const float* __restrict__ a2, const float* __restrict__ u2, float* __restrict__ c2, long long n2,
-                                 const float* __restrict__ amax, float t, const double* __restrict__ Z, const int32_t* status) {
+__global__ void lse_coef2_kernel(const float* a1, const float* u1, float* __restrict__ c1, long long n1,
+                                 const float* a2, const float* u2, float* __restrict__ c2, long long n2,
+                                 const float* amax, float t, const double* Z, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
   const float mx = *amax;
@@ -1315,7 +1321,7 @@ __global__ void sub_identity_kernel(float* __restrict__ R, int k, long long n) {
   }
 }
 
-__global__ void sqsum_f32_kernel(const float* __restrict__ x, long long n, double* acc) {
+__global__ void sqsum_f32_kernel(const float* x, long long n, double* acc) {
   pdl_enter();
   __shared__ double red[32];
   double local = 0.0;
@@ -1327,7 +1333,7 @@ __global__ void sqsum_f32_kernel(const float* __restrict__ x, long long n, doubl
 
 // gradM += lambda * 2 (R M) / (||R||_F sqrt(h));  RM holds R M;  nothing when ||R||_F / sqrt(h) < 1e-5
 // (the un-squared norm has no gradient at R = 0 and below the fp32 noise floor its direction is noise)
-__global__ void orth_grad_kernel(float* __restrict__ gradM, const float* __restrict__ RM, const double* __restrict__ r2,
+__global__ void orth_grad_kernel(float* __restrict__ gradM, const float* RM, const double* r2,
                                  float lambda, float sqrt_h, long long n) {
   pdl_enter();
   const double nrm = sqrt(*r2);
@@ -1357,9 +1363,9 @@ __global__ void finalize_single_kernel(const double* acc, float* losses, float* 
 
 // Appendix D.1's sums of squares over the group maxima: coef = w * 2 a sign(U at the arg-max) / count, with
 // w = the other factor's Frobenius norm in the weighted form (acc[5] = ||U||_F^2, acc[6] = ||V||_F^2), else 1
-__global__ void sumsq_coef2_kernel(const float* __restrict__ a1, const float* __restrict__ u1, float* __restrict__ c1, long long n1,
-                                   const float* __restrict__ a2, const float* __restrict__ u2, float* __restrict__ c2, long long n2,
-                                   const double* __restrict__ acc, int weighted, const int32_t* status) {
+__global__ void sumsq_coef2_kernel(const float* a1, const float* u1, float* __restrict__ c1, long long n1,
+                                   const float* a2, const float* u2, float* __restrict__ c2, long long n2,
+                                   const double* acc, int weighted, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
   const float w1 = (weighted ? (float)sqrt(acc[6]) : 1.f) * 2.f / (float)n1;
@@ -1376,7 +1382,7 @@ __global__ void sumsq_coef2_kernel(const float* __restrict__ a1, const float* __
 }
 
 // dst += (acc[num] / count) / sqrt(acc[den]) * src   (the dense terms of the weighted form: mean(a^2) d||X||_F)
-__global__ void axpy_norm_kernel(float* __restrict__ dst, const float* __restrict__ src, long long n, const double* __restrict__ acc,
+__global__ void axpy_norm_kernel(float* __restrict__ dst, const float* src, long long n, const double* acc,
                                  int num, double count, int den, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
@@ -1387,7 +1393,7 @@ __global__ void axpy_norm_kernel(float* __restrict__ dst, const float* __restric
 }
 
 // out = T - T^T per block (the skew part that drives a Cayley step)
-__global__ void skew_blocks_kernel(const float* __restrict__ T, float* __restrict__ out, int k, long long n) {
+__global__ void skew_blocks_kernel(const float* T, float* __restrict__ out, int k, long long n) {
   pdl_enter();
   const long long kk = (long long)k * k;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -1398,14 +1404,14 @@ __global__ void skew_blocks_kernel(const float* __restrict__ T, float* __restric
 }
 
 // out = x + alpha * y  /  x = beta * x + y
-__global__ void lincomb_kernel(float* __restrict__ out, const float* __restrict__ x, float alpha, const float* __restrict__ y,
+__global__ void lincomb_kernel(float* __restrict__ out, const float* x, float alpha, const float* y,
                                long long n, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = fmaf(alpha, y[i], x[i]);
 }
-__global__ void momentum_kernel(float* __restrict__ v, float beta, const float* __restrict__ g, long long n, const int32_t* status) {
+__global__ void momentum_kernel(float* __restrict__ v, float beta, const float* g, long long n, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -1439,7 +1445,7 @@ __global__ void finalize_pair_kernel(const double* acc, const float* amax, float
 // ------------------------------------------------------------------------------------------------
 // pack: u = q + qmax, little-endian bit stream per row; one thread per output 32-bit word group
 // ------------------------------------------------------------------------------------------------
-__global__ void pack_kernel(const int8_t* __restrict__ codes, uint8_t* __restrict__ packed, int rows, int cols, int bits) {
+__global__ void pack_kernel(const int8_t* codes, uint8_t* __restrict__ packed, int rows, int cols, int bits) {
   pdl_enter();
   // one thread packs 8 consecutive codes into `bits` bytes
   const long long chunks_per_row = cols / 8;
@@ -1463,7 +1469,7 @@ __global__ void pack_kernel(const int8_t* __restrict__ codes, uint8_t* __restric
 // division per chunk.  2304 x 9216 at 4 bits: 38 -> 13 us against the scalar kernel below (eight 2-byte stores, eight scale
 // loads and nine divisions per chunk).
 template <int BITS>
-__global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* __restrict__ packed, const float* __restrict__ scales,
+__global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* packed, const float* scales,
                                                        uint16_t* __restrict__ out, unsigned n, unsigned cpr, unsigned cpg, long long ldo) {
   pdl_enter();
   constexpr uint32_t mask = (1u << BITS) - 1u;
@@ -1478,14 +1484,14 @@ __global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* __restrict
     s[u] = 0.f;
     if (c < n) {
       const uint8_t* src = packed + (size_t)c * BITS;
-      if constexpr (BITS == 2) v[u] = __ldg(reinterpret_cast<const uint16_t*>(src));
-      else if constexpr (BITS == 4) v[u] = __ldg(reinterpret_cast<const uint32_t*>(src));
-      else if constexpr (BITS == 8) v[u] = __ldg(reinterpret_cast<const unsigned long long*>(src));
+      if constexpr (BITS == 2) v[u] = ld_plain(reinterpret_cast<const uint16_t*>(src));
+      else if constexpr (BITS == 4) v[u] = ld_plain(reinterpret_cast<const uint32_t*>(src));
+      else if constexpr (BITS == 8) v[u] = ld_plain(reinterpret_cast<const unsigned long long*>(src));
       else {
 #pragma unroll
-        for (int b = 0; b < BITS; ++b) v[u] |= (unsigned long long)__ldg(src + b) << (8 * b);
+        for (int b = 0; b < BITS; ++b) v[u] |= (unsigned long long)ld_plain(src + b) << (8 * b);
       }
-      s[u] = __ldg(scales + c / cpg);
+      s[u] = ld_plain(scales + c / cpg);
     }
   }
 #pragma unroll
@@ -1511,7 +1517,7 @@ __global__ void __launch_bounds__(256) dequant8_kernel(const uint8_t* __restrict
 
 // Any group width, pitch and alignment: the inverse of pack_kernel followed by the dequantisation: out[row][c] = bf16(scale(row, c / g) * (field - qmax)),
 // one thread per 8 consecutive codes (`bits` bytes of the stream); cols % 8 == 0, out row pitch ldo elements.
-__global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict__ packed, const float* __restrict__ scales,
+__global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* packed, const float* scales,
                                                       uint16_t* __restrict__ out, int rows, int cols, int bits, int g, long long ldo) {
   pdl_enter();
   const long long chunks_per_row = cols / 8;
@@ -1528,14 +1534,14 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict_
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int col = (int)ch * 8 + i;
-      const float s = __ldg(scales + row * ng + col / g);
+      const float s = ld_plain(scales + row * ng + col / g);
       const int q = (int)((v >> (bits * i)) & mask) - qmax;
       dst[i] = __bfloat16_as_ushort(__float2bfloat16_rn(s * (float)q));
     }
   }
 }
 
-__global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* __restrict__ in, uint16_t* __restrict__ out, long long n) {
+__global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* in, uint16_t* __restrict__ out, long long n) {
   pdl_enter();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
     out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(in[e]));
@@ -1544,7 +1550,7 @@ __global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* __restric
 // The same stream, 32 codes per thread: 32 b-bit fields are exactly b 32-bit words, so a thread reads two 16-byte
 // vectors of codes and writes whole words (cols % 32 == 0, codes 16-byte aligned, packed 4-byte aligned).
 template <int BITS>
-__global__ void __launch_bounds__(256) pack32_kernel(const int8_t* __restrict__ codes, uint32_t* __restrict__ packed, int rows,
+__global__ void __launch_bounds__(256) pack32_kernel(const int8_t* codes, uint32_t* __restrict__ packed, int rows,
                                                      int cols) {
   pdl_enter();
   const long long chunks_per_row = cols / 32;
@@ -1553,7 +1559,7 @@ __global__ void __launch_bounds__(256) pack32_kernel(const int8_t* __restrict__ 
   constexpr uint32_t mask = (1u << BITS) - 1u;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
     const uint4* src = reinterpret_cast<const uint4*>(codes) + 2 * c;  // rows are contiguous: chunk c starts at 32 c
-    const uint4 q0 = __ldg(src), q1 = __ldg(src + 1);
+    const uint4 q0 = ld_plain(src), q1 = ld_plain(src + 1);
     const uint32_t w8[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
     uint32_t out[BITS];
 #pragma unroll

@@ -488,7 +488,7 @@ static int ns_block_launch(cudaStream_t st, const uint16_t* A, uint16_t* hi, uin
 }
 
 // hi = A^T, lo = 0: the cold start X0 = A^T of the iteration (A is bf16, so hi carries it exactly); 32 x 32 tiles
-__global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* __restrict__ A, int k, uint16_t* __restrict__ hi,
+__global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* A, int k, uint16_t* __restrict__ hi,
                                                             uint16_t* __restrict__ lo, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;

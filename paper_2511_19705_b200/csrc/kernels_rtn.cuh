@@ -19,7 +19,7 @@ namespace cafeq {
 // division and reciprocal are paid once per 32 weights.  Within a warp's 2 KB span lane l works on group l / LG and
 // its u-th chunk is the group's chunk u * LG + l % LG: a load instruction of the warp covers whole 64-byte pieces.
 template <int LG>
-__global__ void __launch_bounds__(256) rtn_stream_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols,
+__global__ void __launch_bounds__(256) rtn_stream_kernel(const uint16_t* W, long long ld, int rows, int cols,
                                                          float qmax, int8_t* __restrict__ codes, float* __restrict__ scales) {
   pdl_enter();
   constexpr int UPG = 4 * LG;               // 16-byte chunks per group

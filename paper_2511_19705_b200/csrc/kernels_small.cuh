@@ -19,7 +19,7 @@ namespace cafeq {
 // plays row p, and the permutation is applied when the result is written.  Optional: column norms (sum_i Out[i][t]^2), bf16
 // hi / lo splits, row-major and transposed.
 template <int K>
-__global__ void __launch_bounds__(256) small_inverse_kernel(const float* __restrict__ Min, float* __restrict__ Out, float* __restrict__ cnorm,
+__global__ void __launch_bounds__(256) small_inverse_kernel(const float* Min, float* __restrict__ Out, float* __restrict__ cnorm,
                                                             uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
                                                             uint16_t* __restrict__ tlo, int32_t* status) {
   pdl_enter();
@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(256) small_inverse_kernel(const float* __restr
 // operands in shared memory, 4 x 4 outputs per thread from 16-byte reads (the pitch of K + 4 spreads eight rows over the
 // banks); the intermediate product takes the place of Gx.
 template <int K>
-__global__ void __launch_bounds__(K * K / 16) small_chain_kernel(const float* __restrict__ X, const float* __restrict__ Gx,
-                                                                 const float* __restrict__ A, const float* __restrict__ Agrp, int g,
+__global__ void __launch_bounds__(K * K / 16) small_chain_kernel(const float* X, const float* Gx,
+                                                                 const float* A, const float* Agrp, int g,
                                                                  float scale, float* __restrict__ G, const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(256) layer_finish_kernel(const LyFinishArgs f)
 }
 
 // max |w| of a bf16 matrix (bit pattern of a non-negative float, atomic integer maximum)
-__global__ void __launch_bounds__(256) absmax_bf16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols,
+__global__ void __launch_bounds__(256) absmax_bf16_kernel(const uint16_t* W, long long ld, int rows, int cols,
                                                           float* __restrict__ out) {
   pdl_enter();
   float m = 0.f;
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) absmax_bf16_kernel(const uint16_t* __rest
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nch; c += (long long)gridDim.x * blockDim.x) {
     const long long row = c / cpr;
     const int cc = (int)(c - row * cpr);
-    const uint4 q = __ldg(reinterpret_cast<const uint4*>(W + row * ld) + cc);
+    const uint4 q = ld_plain(reinterpret_cast<const uint4*>(W + row * ld) + cc);
     const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(256) absmax_bf16_kernel(const uint16_t* __rest
 // fp16 copy of a bf16 matrix, scaled by the power of two that brings max |w| just below 2^14:  out = fp16(w * 2^e),
 // *inv_scale = 2^-e.  bf16 carries 8 significand bits, fp16 11, so every entry down to 2^-38 of the largest is copied
 // exactly; smaller ones round to the fp16 subnormal grid (absolute error below 2^-39 of the largest entry).
-__global__ void __launch_bounds__(256) bf16_to_scaled_f16_kernel(const uint16_t* __restrict__ W, long long ld, int rows, int cols,
-                                                                 const float* __restrict__ wmax, uint16_t* __restrict__ out,
+__global__ void __launch_bounds__(256) bf16_to_scaled_f16_kernel(const uint16_t* W, long long ld, int rows, int cols,
+                                                                 const float* wmax, uint16_t* __restrict__ out,
                                                                  float* __restrict__ inv_scale) {
   pdl_enter();
   const float m = *wmax;
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(256) bf16_to_scaled_f16_kernel(const uint16_t*
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nch; c += (long long)gridDim.x * blockDim.x) {
     const long long row = c / cpr;
     const int cc = (int)(c - row * cpr);
-    const uint4 q = __ldg(reinterpret_cast<const uint4*>(W + row * ld) + cc);
+    const uint4 q = ld_plain(reinterpret_cast<const uint4*>(W + row * ld) + cc);
     const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
     uint32_t o4[4];
 #pragma unroll

@@ -62,3 +62,11 @@ def test_a_block_stops_as_a_whole(file, name, body):
     """The status word may be raised while a block starts.  Threads that looked at it one by one could disagree, and those
     that went on would wait at barriers for the ones that left."""
     assert not re.search(r"if \([^;{]*\*\s*(\w+\.)?status\)", body), f"{name}: every thread reads the status word for itself"
+
+
+@pytest.mark.parametrize("path", sorted(glob.glob(os.path.join(CSRC, "*.cu*"))), ids=os.path.basename)
+def test_inputs_are_read_with_ordinary_loads(path):
+    """An overlapped kernel's inputs change during its lifetime: no read-only loads, and no promise that allows them."""
+    text = _strip(open(path).read())
+    assert not re.search(r"__ldg\b|ld\.global\.nc", text)
+    assert not re.search(r"\bconst\s+\w+\s*\*\s*__restrict__", text)
