@@ -112,7 +112,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
   using C = BwCfg<K, F16>;
   static_assert(K == 128 || K == 256, "block size");
   int32_t* const status = mp.p[0].status;
-  if (cta_stopped(status)) return;
+  const bool raised = status_raised(status);  // (awaited at the end of the set-up)
   const int total_tiles = mp.tile_end[mp.n - 1];
   const int t_begin = (int)(((long long)cta * total_tiles) / ncta);
   const int t_end = (int)(((long long)(cta + 1) * total_tiles) / ncta);
@@ -165,9 +165,13 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  const bool stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (stopped) {
+    if (warp == 1) tmem_free(tmem_base, C::TMEM_COLS);
+    return;
+  }
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer: one weight tile per stage
@@ -437,7 +441,7 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+    tmem_free(tmem_base, C::TMEM_COLS);
   }
 }
 

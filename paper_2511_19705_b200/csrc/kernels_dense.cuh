@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(256) ste_grad_split_kernel(const float* U, con
                                                              const float* usel, const int* idx, float qmax,
                                                              uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, const int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  if (warp_stopped(status)) return;
   const int l = threadIdx.x % LPG;
   const long long total = (long long)rows * ng;
   const long long w = (blockIdx.x * 256ll + threadIdx.x) / LPG;
@@ -276,22 +276,32 @@ __global__ void ste_scale_coef_kernel(const float* gD, long long ldg, const uint
                                       const float* a, const float* usel, int gm,
                                       float* __restrict__ coef, const int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  if (warp_stopped(status)) return;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= (long long)rows * ng) return;
   // consecutive warps take consecutive groups of one row (the rows of gD and Delta are read contiguously)
   const int row = (int)(w / ng), G = (int)(w - (long long)row * ng);
+  const long long pi = gm ? (long long)G * rows + row : w;
+  const float av = a[pi], u = usel[pi];
+  const long long c0 = (long long)G * g;
   float sum = 0.f;
-  for (int e = lane; e < g; e += 32) {
-    const long long col = (long long)G * g + e;
-    const float d = bf16_bits_to_float(Dh[row * ldd + col]) + bf16_bits_to_float(Dl[row * ldd + col]);
-    sum = fmaf(gD[row * ldg + col], d, sum);
+  for (int e0 = lane; e0 < g; e0 += 128) {  // (four values requested before the first is used: 33 -> 28 us at 4096 x 3584)
+    float x[4], d[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int e = e0 + 32 * j;
+      x[j] = d[j] = 0.f;
+      if (e < g) {
+        x[j] = gD[row * ldg + c0 + e];
+        d[j] = bf16_bits_to_float(Dh[row * ldd + c0 + e]) + bf16_bits_to_float(Dl[row * ldd + c0 + e]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sum = fmaf(x[j], d[j], sum);
   }
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) {
-    const long long pi = gm ? (long long)G * rows + row : w;
-    const float av = a[pi], u = usel[pi];
     const float sgn = (u > 0.f) ? 1.f : ((u < 0.f) ? -1.f : 0.f);
     coef[pi] = (av > 0.f) ? sgn * sum / av : 0.f;
   }

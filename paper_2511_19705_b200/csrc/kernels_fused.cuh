@@ -177,6 +177,11 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// one converged warp releases the tensor memory that it allocated
+__device__ __forceinline__ void tmem_free(uint32_t base, uint32_t cols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
+}
+
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -312,7 +317,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
   static_assert(FORM == BD_IN || K >= 128, "output-axis form needs k >= 128");
   static_assert(G == 64 || G == 128, "group size");
   int32_t* const status = mp.p[0].status;
-  if (cta_stopped(status)) return;
+  const bool raised = status_raised(status);  // (awaited at the end of the set-up)
 
   // persistent CTA: a contiguous run of tiles in (sub-problem, major, minor) order; the operator block is reloaded
   // when the run crosses into the next major or the next sub-problem
@@ -363,9 +368,13 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  const bool stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (stopped) {
+    if (warp == 1) tmem_free(tmem_base, 512u);
+    return;
+  }
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
@@ -880,7 +889,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    tmem_free(tmem_base, 512u);
   }
 }
 

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgParams p) {
   pdl_enter();
   using C = TgCfg<BN>;
-  if (cta_stopped(p.status)) return;
+  const bool raised = status_raised(p.status);  // (awaited at the end of the set-up)
   if (tg_stopped(p)) return;
 
   extern __shared__ uint8_t smem_raw[];
@@ -271,9 +271,13 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  const bool stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (stopped) {
+    if (warp == 1) tmem_free(tmem_base, C::TMEM_COLS);
+    return;
+  }
   const int kchunks = (p.K + TG_BK - 1) / TG_BK;
   const int total = kchunks * p.nterms;
 
@@ -356,7 +360,7 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+    tmem_free(tmem_base, C::TMEM_COLS);
   }
 }
 
@@ -425,7 +429,7 @@ tc_block_kernel(const __grid_constant__ TbMaps maps, const TbTerms tt, const TgP
   pdl_enter();
   using C = TbCfg<K>;
   static_assert(K == 128 || K == 256, "block size");
-  if (cta_stopped(p.status)) return;
+  const bool raised = status_raised(p.status);  // (awaited at the end of the set-up)
   const int b = blockIdx.x;
 
   extern __shared__ uint8_t smem_raw[];
@@ -471,9 +475,13 @@ tc_block_kernel(const __grid_constant__ TbMaps maps, const TbTerms tt, const TgP
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  const bool stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (stopped) {
+    if (warp == 1) tmem_free(tmem_base, C::TMEM_COLS);
+    return;
+  }
 
   if (warp == 0) {
     if (lane == 0) {
@@ -657,7 +665,7 @@ tc_block_kernel(const __grid_constant__ TbMaps maps, const TbTerms tt, const TgP
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+    tmem_free(tmem_base, C::TMEM_COLS);
   }
 }
 
@@ -791,10 +799,13 @@ __global__ void __launch_bounds__(256) split_bf16_kernel(const float* X, int k, 
   const size_t base = (size_t)blockIdx.z * k * k;
   const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
+  float x4[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) x4[r] = X[base + (size_t)(i0 + ty + 8 * r) * k + j0 + tx];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int i = i0 + ty + 8 * r, j = j0 + tx;
-    const float x = X[base + (size_t)i * k + j];
+    const float x = x4[r];
     const __nv_bfloat16 h = __float2bfloat16_rn(x);
     const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
     const uint16_t hb = __bfloat16_as_ushort(h), lb = __bfloat16_as_ushort(l);

@@ -63,9 +63,10 @@ __device__ __forceinline__ void raise_status(int32_t* status, int code) {
 // Whether an earlier failure lets this CTA skip its work: one answer for all its threads.  Another CTA of the same launch, or a
 // kernel on a side stream, may raise the word at any time; threads that each looked for themselves could disagree, and the
 // ones that went on would wait at barriers (or on tensor memory) for the ones that had left.
-__device__ __forceinline__ bool cta_stopped(const int32_t* status) {
-  return __syncthreads_or(status && *(const volatile int32_t*)status) != 0;
-}
+__device__ __forceinline__ bool status_raised(const int32_t* status) { return status && *status; }
+__device__ __forceinline__ bool cta_stopped(const int32_t* status) { return __syncthreads_or(status_raised(status)) != 0; }
+// the same for kernels whose threads meet inside a warp only
+__device__ __forceinline__ bool warp_stopped(const int32_t* status) { return __any_sync(0xffffffffu, status_raised(status)) != 0; }
 
 __device__ __forceinline__ double block_sum_double(double v, double* sh) {
   // sh: at least 32 doubles of shared memory
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(1024) block_inverse_kernel(const float* Min, f
 __global__ void absmax_kernel(const float* U, long long ld, int rows, int ng, int g,
                               float* __restrict__ a, float* __restrict__ usel, int* __restrict__ idx, int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  if (warp_stopped(status)) return;
   long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)rows * ng;
@@ -432,7 +433,7 @@ __global__ void __launch_bounds__(256) group_quant_kernel(const SRC* U, long lon
                                                           float* __restrict__ Uhat, int8_t* __restrict__ codes,
                                                           float* __restrict__ scales, int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  if (LPG > 32 ? cta_stopped(status) : warp_stopped(status)) return;
   const int cols = ng * g;
   const int l = threadIdx.x % LPG;
   const long long total = (long long)rows * ng;
@@ -621,7 +622,7 @@ __global__ void ste_scale_path_kernel(const float* U, const float* gD, long long
                                       const void* offsets, int off_kind, int cols, float* __restrict__ coef,
                                       const int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  if (warp_stopped(status)) return;
   long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= (long long)rows * ng) return;
@@ -1230,7 +1231,7 @@ __global__ void max_f32_kernel(const float* a, long long n, float* __restrict__ 
                                const int32_t* status) {
   pdl_enter();
   // a >= 0, so an integer atomicMax on the bit pattern orders correctly
-  if (cta_stopped(status)) return;
+  if (warp_stopped(status)) return;
   float m = 0.f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     m = fmaxf(m, a[i]);
@@ -1270,7 +1271,7 @@ __global__ void lse_coef_kernel(const float* a, const float* usel, long long n,
 __global__ void max2_f32_kernel(const float* a1, long long n1, const float* a2, long long n2,
                                 float* __restrict__ out_max, const int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  if (warp_stopped(status)) return;
   float m = 0.f;
   const long long n = n1 + n2;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(NsCfg<K>::THREADS, 1)
 ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsParams p) {
   pdl_wait();  // (releases at its end: a layer's penalty chain shares the SMs with it, which waiting CTAs of the pass would take)
   using C = NsCfg<K>;
-  if (cta_stopped(p.status)) return;
+  const bool raised = status_raised(p.status);  // (awaited at the end of the set-up)
   const int b = blockIdx.x, row_b = b * K;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -105,7 +105,6 @@ ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     if (b >= p.blk0[q] && b < p.blk0[q + 1]) prob = q;
   const bool want_c = prob >= 0 && p.c;
   for (int e = threadIdx.x; e < K; e += C::THREADS) cn[e] = 0.f;
-  if (b == 0 && threadIdx.x < p.n_ticks && p.tick[threadIdx.x]) *p.tick[threadIdx.x] += 1.f;
 
   if (threadIdx.x == 0) {
     *not_converged = 0;
@@ -131,9 +130,14 @@ ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  const bool stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (stopped) {
+    if (warp == 1) tmem_free(tmem_base, C::TMEM_COLS);
+    return;
+  }
+  if (b == 0 && threadIdx.x < p.n_ticks && p.tick[threadIdx.x]) *p.tick[threadIdx.x] += 1.f;
 
   // every role takes the same decision from the same 16 partial sums
   auto residual2 = [&]() {
@@ -411,7 +415,7 @@ ns_block_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+    tmem_free(tmem_base, C::TMEM_COLS);
   }
   if (*abort_flag) return;
   const size_t off = (size_t)b * K * K;
@@ -495,8 +499,11 @@ __global__ void __launch_bounds__(256) ns_cold_start_kernel(const uint16_t* A, i
   __shared__ uint16_t tile[32][34];
   const size_t base = (size_t)blockIdx.z * k * k;
   const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+  uint16_t v[4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) tile[threadIdx.y + 8 * r][threadIdx.x] = A[base + (size_t)(i0 + threadIdx.y + 8 * r) * k + j0 + threadIdx.x];
+  for (int r = 0; r < 4; ++r) v[r] = A[base + (size_t)(i0 + threadIdx.y + 8 * r) * k + j0 + threadIdx.x];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) tile[threadIdx.y + 8 * r][threadIdx.x] = v[r];
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -577,7 +584,7 @@ __global__ void __launch_bounds__(ChainCfg<K>::THREADS, 1)
 kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainParams p) {
   pdl_enter();
   using C = ChainCfg<K>;
-  if (cta_stopped(p.status)) return;
+  const bool raised = status_raised(p.status);  // (awaited at the end of the set-up)
   const int b = blockIdx.x, row_b = b * K;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -622,9 +629,13 @@ kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  const bool stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (stopped) {
+    if (warp == 1) tmem_free(tmem_base, C::TMEM_COLS);
+    return;
+  }
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer: hi and lo of every 64-entry chunk
@@ -919,7 +930,7 @@ kk_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant__ 
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)C::TMEM_COLS) : "memory");
+    tmem_free(tmem_base, C::TMEM_COLS);
   }
 }
 
