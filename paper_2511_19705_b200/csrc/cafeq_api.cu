@@ -1585,7 +1585,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       launch_ste_split(st, p.m2, w.X0T, w.h, G2, k, G2.r, qmax_of(d2->bits), p.gVh, p.gVl, status);
       if ((p.err = opgrad_in_tc(st, p.gVh, p.gVl, (const uint16_t*)W2, G2.ld, G1.nbT, G2.r, k, G2.d_out, p.gMinv, status))) return;
     } else {
-      CQ_LAUNCH(expand_cols_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f, w.V);
+      CQ_LAUNCH(expand_cols_kernel, dim3(w.d3, (w.h + 1023) / 1024), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f, w.V);
       const long long n1w = (long long)G1.d_out * G1.ng, n2w = (long long)G2.d_out * G2.ng;
       CQ_LAUNCH(ste_scale_path_kernel, (unsigned)((n1w * 32 + 255) / 256), 256, 0, st, p.m1.U, w.U, G1.d_in, G1.d_out, G1.ng, G1.g,
                 p.m1.a, p.m1.usel, qmax_of(d1->bits), nullptr, CAFEQ_OFFSETS_NONE, G1.d_in, p.m1.coef, status);

@@ -106,14 +106,15 @@ __global__ void __launch_bounds__(256) fold_transpose_kernel(const float* V, int
   }
 }
 
-// V[y][(B*r + rep)*k + j] = scale * X[y][B*k + j]  (X fp32 [d3, h] -> V fp32 [d3, r*h]; k % 4 == 0).  grid: (ceil(h / 1024),
-// d3); a thread reads four entries once and writes every replica (60 -> 12 us at 3584 x 4096).
+// V[y][(B*r + rep)*k + j] = scale * X[y][B*k + j]  (X fp32 [d3, h] -> V fp32 [d3, r*h]; k % 4 == 0).  grid: (d3,
+// ceil(h / 1024)) -- d3 may exceed what the second dimension of a grid holds; a thread reads four entries once and writes every
+// replica (60 -> 12 us at 3584 x 4096).
 __global__ void __launch_bounds__(256) expand_cols_kernel(const float* X, int h, int k, int r, float scale,
                                                           float* __restrict__ V) {
   pdl_enter();
-  const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
+  const int l = (blockIdx.y * 256 + threadIdx.x) * 4;
   if (l >= h) return;
-  const long long y = blockIdx.y;
+  const long long y = blockIdx.x;
   float4 x = ld_plain(reinterpret_cast<const float4*>(X + y * h + l));
   x = make_float4(scale * x.x, scale * x.y, scale * x.z, scale * x.w);
   const int B = l / k, j = l - B * k;
@@ -134,14 +135,15 @@ __global__ void expand_cols_any_kernel(const float* X, int d3, int h, int k, int
 }
 
 // bf16 hi / lo (and third) terms of the replica-folded V: F[y][B*k + j] = sum_rep V[y][(B*r + rep)*k + j], row-major [d3, h].
-// A product over the r*h expanded inner indices equals the product over the h folded ones: 1 / r of the work.
+// A product over the r*h expanded inner indices equals the product over the h folded ones: 1 / r of the work.  grid: (d3,
+// ceil(h / 1024)).
 __global__ void __launch_bounds__(256) fold_split_kernel(const float* V, int h, int k, int r, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ lo, uint16_t* __restrict__ h3, const int32_t* status) {
   pdl_enter();
   if (status && *status) return;
-  const int l = (blockIdx.x * 256 + threadIdx.x) * 4;
+  const int l = (blockIdx.y * 256 + threadIdx.x) * 4;
   if (l >= h) return;
-  const long long y = blockIdx.y;
+  const long long y = blockIdx.x;
   const int B = l / k, j = l - B * k;
   const float* v = V + y * (long long)r * h + (long long)B * r * k + j;
   float x[4] = {0.f, 0.f, 0.f, 0.f};

@@ -224,7 +224,7 @@ static void quant_matrix(cudaStream_t st, const float* T, int rows, int cols, in
 
 // hi / lo (and third) terms of V [d3, rh] with its replicas folded: [d3, h]
 static void launch_fold_split(cudaStream_t st, const float* V, DenseWS& w, uint16_t* hi, uint16_t* lo, uint16_t* h3, int32_t* status) {
-  CQ_LAUNCH(fold_split_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, V, w.h, w.k, w.r, hi, lo, h3, status);
+  CQ_LAUNCH(fold_split_kernel, dim3(w.d3, (w.h + 1023) / 1024), 256, 0, st, V, w.h, w.k, w.r, hi, lo, h3, status);
 }
 
 // P = U_exp^T V^T for stored U [h, d1], V [d3, rh] (fp32): fp32 P [d1, d3] with its splits in w.Ph/Pl/PTh/PTl
@@ -279,7 +279,7 @@ static void alg1_run(cudaStream_t st, int bits, int g1, int g2, int iters, int8_
       o.C = w.X0T; o.ldc = w.h;
       launch_dense_tc6(st, a, b, w.d3, w.h, w.d1, 1.f, 0.f, 0.f, o, w.X0T, status);
     }
-    CQ_LAUNCH(expand_cols_kernel, dim3((w.h + 1023) / 1024, w.d3), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f / (float)w.r, w.V);
+    CQ_LAUNCH(expand_cols_kernel, dim3(w.d3, (w.h + 1023) / 1024), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f / (float)w.r, w.V);
     quant_matrix(st, w.V, w.d3, w.rh, g2, bits, codes2, scales2, w.Vhat, w, status);
     dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 1, nullptr, status);
     // U side: U' [h, d1] = pinv(Bf)^T P^T with Bf = fold(Vhat^T) [h, d3]
