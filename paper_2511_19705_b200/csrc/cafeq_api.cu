@@ -243,7 +243,7 @@ constexpr double NS_GATE2 = 1e-4, NS_COLD_GATE2 = 1e-6;
 
 static void launch_operator_bf16(cudaStream_t st, const float* T, uint16_t* out, int k, int nb, int transpose, int32_t* status,
                                  int paired = 0) {
-  CQ_LAUNCH(operator_to_bf16_kernel, dim3(k / 32, k / 32, nb), 256, 0, st, T, out, k, transpose, paired, status);
+  CQ_LAUNCH(operator_to_bf16_kernel, dim3(nb, k / 32, k / 32), 256, 0, st, T, out, k, transpose, paired, status);
 }
 
 static bool kk_fast(int k) { return k == 64 || k == 128 || k == 256; }

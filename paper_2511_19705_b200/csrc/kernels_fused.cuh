@@ -1165,7 +1165,8 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
 }
 
 // fp32 operator blocks -> bf16 in applied orientation (transposed when the role asks for T^T); k % 32 == 0, one 32 x 32 tile
-// per CTA (grid: (k / 32, k / 32, blocks)), rows read and written along their elements.  Latency-bound: one load, one store
+// per CTA (grid: (blocks, k / 32, k / 32): only the first dimension holds any number of blocks), rows read and written along
+// their elements.  Latency-bound: one load, one store
 // (14 blocks of 256: 5 - 7 us with a strided walk and 64-bit divisions per element, 3 us here).
 // paired (k = 32): blocks 2 i and 2 i + 1 become one 64 x 64 block, zeros off the diagonal.
 __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* T, uint16_t* __restrict__ out, int k, int transpose,
@@ -1173,8 +1174,8 @@ __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* T, u
   pdl_enter();
   if (cta_stopped(status)) return;
   __shared__ float tile[32][33];
-  const size_t base = (size_t)blockIdx.z * k * k;
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;  // tile of the output
+  const size_t base = (size_t)blockIdx.x * k * k;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.z * 32;  // tile of the output
   const int i = threadIdx.x >> 3, j = (threadIdx.x & 7) * 4;
   const float* src = T + base + (transpose ? (size_t)(c0 + i) * k + r0 + j : (size_t)(r0 + i) * k + c0 + j);
   float v[4];
@@ -1198,8 +1199,8 @@ __global__ void __launch_bounds__(256) operator_to_bf16_kernel(const float* T, u
     w[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * e])) |
            ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * e + 1])) << 16);
   if (paired) {
-    const int odd = blockIdx.z & 1;
-    uint16_t* o = out + (size_t)(blockIdx.z >> 1) * 4096 + (odd * 32 + i) * 64 + j;
+    const int odd = blockIdx.x & 1;
+    uint16_t* o = out + (size_t)(blockIdx.x >> 1) * 4096 + (odd * 32 + i) * 64 + j;
     *reinterpret_cast<uint2*>(o + odd * 32) = make_uint2(w[0], w[1]);
     *reinterpret_cast<uint2*>(o + (1 - odd) * 32) = make_uint2(0u, 0u);
     return;

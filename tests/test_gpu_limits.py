@@ -44,3 +44,12 @@ def test_second_factor_of_more_rows_than_a_grid_has_slices(cq):
     Minv = torch.from_numpy(orc.round_bf16(orc.block_inverse(Mc.cpu().numpy()[None]))).cuda().double()[0]
     target = (Mc.T @ W1.double()).T @ (W2.double() @ Minv.T).T
     assert abs(float((U.T @ V.T - target).norm()) / float(r["pqe"][2]) - 1) <= 1e-3
+
+
+def test_more_operator_blocks_than_a_grid_has_slices(cq):
+    """65 600 blocks of 64: row and operators repeat every 64 blocks, and so must the codes and scales."""
+    W = to_dev(syn.weight_student_t(1, 4096, 3))
+    T = f32_dev(syn.perturbed_blocks(64, 64, 5, 0.1))
+    codes, scales = cq.cafeq_rtn(W.repeat(1, 1025), T.repeat(1025, 1, 1), bits=4, group=128, tblock=64)
+    c0, s0 = cq.cafeq_rtn(W, T, bits=4, group=128, tblock=64)
+    assert torch.equal(codes.view(1025, -1), c0.repeat(1025, 1)) and torch.equal(scales.view(1025, -1), s0.repeat(1025, 1))
