@@ -99,7 +99,8 @@ def _hot():
 
 @functools.lru_cache(maxsize=256)
 def _plan(kind, d_out, d_in, bits, group, tblock, taxis, trole, replicas, ld):
-    """(address of a descriptor, scratch bytes, the descriptor) of one shape; read only, so threads share it."""
+    """(address of a descriptor, scratch bytes, the descriptor) of one shape; read only, so threads share it.  A caller holds
+    the descriptor until its C call has returned: another thread's shapes may push the entry out of the cache at any time."""
     d = make_desc(d_out, d_in, bits, group, tblock, taxis, trole, replicas, ld)
     n = ctypes.c_size_t(0)
     if kind == "apply":
@@ -226,7 +227,7 @@ def cafeq_rtn(W, T=None, *, bits, group, tblock=0, taxis=AXIS_IN, trole=APPLY_T,
     """Round-to-nearest codes (int8 [d_out,d_in]) and scales (fp32 [d_out, d_in/group]) of T o W."""
     W = _bits_tensor(W)
     d_out, d_in = W.shape
-    desc, nbytes, _ = _plan("rtn", d_out, d_in, bits, group, tblock if T is not None else 0, taxis, trole, replicas, W.stride(0))
+    desc, nbytes, held = _plan("rtn", d_out, d_in, bits, group, tblock if T is not None else 0, taxis, trole, replicas, W.stride(0))
     g = group or d_in
     dev = W.device
     codes = torch.empty((d_out, d_in), dtype=torch.int8, device=dev)
@@ -379,7 +380,7 @@ def cafeq_pack(codes, *, bits):
     if codes.dtype != torch.int8 or not codes.is_cuda or not codes.is_contiguous():
         raise ValueError("codes must be a contiguous CUDA int8 tensor")
     d_out, d_in = codes.shape
-    desc = _plan("", d_out, d_in, bits, 0, 0, AXIS_IN, APPLY_T, 1, d_in)[0]
+    desc, _, held = _plan("", d_out, d_in, bits, 0, 0, AXIS_IN, APPLY_T, 1, d_in)  # (held: until the call has read it)
     packed = torch.empty((d_out, d_in * bits // 8), dtype=torch.uint8, device=codes.device)
     rc = _hot().pack(desc, codes.data_ptr(), packed.data_ptr(), _raw_stream())
     _check(rc, "cafeq_pack")
@@ -393,7 +394,7 @@ def cafeq_apply_transform(X, T, *, taxis=AXIS_IN, trole=APPLY_T, status=None):
         raise ValueError("X must be a CUDA bf16 matrix with unit column stride")
     d_out, d_in = X.shape
     k = T.shape[-1]
-    desc, nbytes, _ = _plan("apply", d_out, d_in, 4, 128 if d_in % 128 == 0 else d_in, k, taxis, trole, 1, X.stride(0))
+    desc, nbytes, held = _plan("apply", d_out, d_in, 4, 128 if d_in % 128 == 0 else d_in, k, taxis, trole, 1, X.stride(0))
     dev = X.device
     ws = torch.empty(nbytes, dtype=torch.uint8, device=dev)
     Y = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=dev)
@@ -406,7 +407,7 @@ def cafeq_apply_transform(X, T, *, taxis=AXIS_IN, trole=APPLY_T, status=None):
 def cafeq_dequant(packed, scales, *, bits, group, d_in):
     """bf16 [d_out, d_in] = scales * codes from the bit stream of cafeq_pack."""
     d_out = packed.shape[0]
-    desc = _plan("", d_out, d_in, bits, group, 0, AXIS_IN, APPLY_T, 1, d_in)[0]
+    desc, _, held = _plan("", d_out, d_in, bits, group, 0, AXIS_IN, APPLY_T, 1, d_in)
     out = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=packed.device)
     rc = _hot().dequant(desc, packed.data_ptr(), scales.data_ptr(), out.data_ptr(), d_in, _raw_stream())
     _check(rc, "cafeq_dequant")
