@@ -166,6 +166,11 @@ def _p(t):
     return ctypes.c_void_p(int(t))
 
 
+def _addr(t):
+    """The same as a plain integer, for the typed calls."""
+    return None if t is None else (t.data_ptr() if isinstance(t, torch.Tensor) else int(t))
+
+
 def _stream():
     return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
@@ -398,7 +403,7 @@ def cafeq_apply_transform(X, T, *, taxis=AXIS_IN, trole=APPLY_T, status=None):
     dev = X.device
     ws = torch.empty(nbytes, dtype=torch.uint8, device=dev)
     Y = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=dev)
-    rc = _hot().apply(desc, X.data_ptr(), T.data_ptr(), Y.data_ptr(), None if status is None else status.data_ptr(), ws.data_ptr(), nbytes,
+    rc = _hot().apply(desc, X.data_ptr(), T.data_ptr(), Y.data_ptr(), _addr(status), ws.data_ptr(), nbytes,
                       _raw_stream())
     _check(rc, "cafeq_apply_transform")
     return Y
@@ -409,7 +414,7 @@ def cafeq_dequant(packed, scales, *, bits, group, d_in):
     d_out = packed.shape[0]
     desc, _, held = _plan("", d_out, d_in, bits, group, 0, AXIS_IN, APPLY_T, 1, d_in)
     out = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=packed.device)
-    rc = _hot().dequant(desc, packed.data_ptr(), scales.data_ptr(), out.data_ptr(), d_in, _raw_stream())
+    rc = _hot().dequant(desc, packed.data_ptr(), _addr(scales), out.data_ptr(), d_in, _raw_stream())
     _check(rc, "cafeq_dequant")
     return out
 

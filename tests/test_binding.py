@@ -55,3 +55,25 @@ def test_descriptor_outlives_the_call(cq, monkeypatch):
     cq.cafeq_pack(_Codes(), bits=4)
     cq.cafeq_dequant(torch.zeros((4, 32), dtype=torch.uint8), torch.zeros((4, 1)), bits=4, group=64, d_in=64)
     assert [n for n, _ in calls.args] == ["pack", "dequant"]
+
+
+def test_addresses_in_place_of_tensors(cq, monkeypatch):
+    """Arrays whose shape the binding does not need may be given as device addresses, or left out."""
+    calls = _Calls(cq)
+    monkeypatch.setattr(cq, "_hot", lambda: calls)
+    packed = torch.zeros((4, 32), dtype=torch.uint8)
+    cq.cafeq_dequant(packed, 8192, bits=4, group=64, d_in=64)
+    assert calls.args[-1][1][:2] == (packed.data_ptr(), 8192)
+    cq.cafeq_dequant(packed, None, bits=4, group=64, d_in=64)  # (refused by the C call)
+    assert calls.args[-1][1][1] in (None, 0)
+
+    class X(_Codes):
+        dtype = torch.bfloat16
+
+        def stride(self, i):
+            return (64, 1)[i]
+
+    T = torch.zeros((1, 64, 64))
+    for status, given in ((None, (None, 0)), (12288, (12288,)), (torch.zeros(1, dtype=torch.int32), None)):
+        cq.cafeq_apply_transform(X(), T, status=status)
+        assert calls.args[-1][1][3] in (given or (status.data_ptr(),))
