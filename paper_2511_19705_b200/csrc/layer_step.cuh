@@ -15,6 +15,8 @@
 // This file is included by cafeq_api.cu after the per-problem paths, whose helpers it reuses.
 #pragma once
 
+#include "side_branch.cuh"
+
 namespace cafeq {
 
 constexpr int LY_MAX_PROBS = 8;
@@ -516,17 +518,17 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
   KkWS& w = L.kk;
   bool any_lambda = false;
   for (int q = 0; q < L.n; ++q) any_lambda |= (L.p[q].pair && L.p[q].cfg.lambda_orth != 0.f);
-  // The pair blocks' penalty (splits of the parameters, R = M M^T - I, R M) does not depend on the inverse: it runs on a
-  // side stream beside it (one CTA per block leaves SMs idle) and joins before the transform pass, which reads bf16(M)^T.  Event record / wait pairs only, so
-  // the fork and the join are captured with the step when the caller's stream is being captured.
+  // The pair blocks' penalty (R = M M^T - I, its norm, R M) does not depend on the inverse: it runs on a side stream beside it
+  // (one CTA per block leaves SMs idle).  Only the parameter update reads its results: it joins there, or on any earlier way out.
   LyAux* aux = (nbP > 0 && g_ly_dual.load(std::memory_order_relaxed) && w_mn_expected(k)) ? ly_aux() : nullptr;
   // Inverse and penalty take one CTA per block.  Where they do not fit side by side, a programmatic launch hurts: CTAs that
   // wait for the kernel before them take SMs from the penalty, and the pass then starts late on those (9B-shaped, 106 + 64
-  // blocks: 372 us a step with ordinary launches, 392 without; 2B-shaped, all resident: 122 and 117).
+  // blocks: 372 us a step with ordinary launches, 392 with programmatic ones; 2B-shaped, all resident: 122 and 117).
   const bool overlap = NB + nbP <= 148;
   cudaStream_t so = st;
+  SideBranch branch;
   if (aux) {
-    if (cudaEventRecord(aux->fork, st) != cudaSuccess || cudaStreamWaitEvent(aux->stream, aux->fork, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
+    if (!branch.fork(st, aux->stream, aux->fork, aux->join)) return CAFEQ_ERR_CUDA;
     so = aux->stream;
   }
   // (enqueued first: its CTAs run longer than the penalty's.)  The singles own the first pair_blk0 blocks: the column
@@ -555,7 +557,6 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     const int rc = penalty_tc(so, w.Ab + offP, w.Pl + offP, L.RM, any_lambda, L.orth_sq, 1, nbP, k, status, overlap);
     if (rc) return rc;
   }
-  if (aux && cudaEventRecord(aux->join, aux->stream) != cudaSuccess) return CAFEQ_ERR_CUDA;
   for (int q = 0; q < L.n; ++q) {
     const LyProb& P = L.p[q];
     if (P.pair) continue;
@@ -726,7 +727,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
     const int rc = minv_path_tc(st, L.Minv, L.gMinv, L.grad, NB, k, w, status, &cp, overlap);
     if (rc) return rc;
   }
-  if (aux && cudaStreamWaitEvent(st, aux->join, 0) != cudaSuccess) return CAFEQ_ERR_CUDA;
+  if (!branch.join()) return CAFEQ_ERR_CUDA;
   {
     LyFinishArgs f;
     memset(&f, 0, sizeof(f));

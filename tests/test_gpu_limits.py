@@ -53,3 +53,37 @@ def test_more_operator_blocks_than_a_grid_has_slices(cq):
     codes, scales = cq.cafeq_rtn(W.repeat(1, 1025), T.repeat(1025, 1, 1), bits=4, group=128, tblock=64)
     c0, s0 = cq.cafeq_rtn(W, T, bits=4, group=128, tblock=64)
     assert torch.equal(codes.view(1025, -1), c0.repeat(1025, 1)) and torch.equal(scales.view(1025, -1), s0.repeat(1025, 1))
+
+
+def test_captured_step_of_a_small_layer(cq):
+    """Few enough blocks that every kernel of the step is launched programmatically, with the penalty on its side stream: a graph's
+    replays are the steps made one by one."""
+    def layer():
+        mk = lambda *a: to_dev(syn.weight_student_t(*a, 2, 10.0))  # noqa: E731
+        k = 128
+        singles = [dict(W=mk(384, 512, 1), M=f32_dev(syn.perturbed_blocks(4, k, 5, 0.02)), bits=4, group=128,
+                        cfg=cq.make_cfg(optimizer=cq.OPT_ADAM, lr=1e-4))]
+        pairs = [dict(W1=mk(256, 1024, 3), W2=mk(640, 512, 4), M=f32_dev(syn.perturbed_blocks(2, k, 6, 0.02)), bits=4, group1=128, group2=128,
+                      replicas=2, cfg=cq.make_cfg(loss_kind=cq.LOSS_LSE, optimizer=cq.OPT_ADAM, lr=1e-4, lambda_orth=0.1))]
+        lay = cq.LayerOptimizer(singles, pairs, 3)
+        lay.prepare()
+        return lay
+
+    a, b = layer(), layer()
+    for _ in range(4):
+        a.step(3)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        b.step(3)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            b.step(3)
+        for _ in range(3):
+            g.replay()
+    torch.cuda.synchronize()
+    assert int(a.status.item()) == 0 == int(b.status.item())
+    for x, y, hx, hy, sx, sy in zip(a.M, b.M, a.hist, b.hist, a.state, b.state):
+        assert float(sx[0]) == 12.0 == float(sy[0])
+        # (the order of atomic additions differs from run to run: 1e-5 of the change that twelve steps of 1e-4 make)
+        assert rel_err(x.cpu().numpy(), y.cpu().numpy()) <= 1e-5 and rel_err(hx[:, 0].cpu().numpy(), hy[:, 0].cpu().numpy()) <= 1e-5
