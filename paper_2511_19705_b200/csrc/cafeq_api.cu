@@ -438,10 +438,6 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
     }
     g_launches.fetch_sub(1, std::memory_order_relaxed);
   }
-  // Tiny matrices (a few CTAs whatever the split): one CTA per output strip, so that every sum has one order and a run
-  // repeats bit for bit.  An optimiser step that divides by the gradient's own size otherwise turns the order of the atomic
-  // additions into different bf16 operators.
-  const bool tiny = G.n <= 65536;
   const bool aligned = ((uintptr_t)W % 4 == 0) && (G.ld % 2 == 0);
   const int nG = (k >= G.g) ? k / G.g : 1;  // groups of one row inside one block (g | k or k | g on this path)
   if (kk_fast(k) && G.axis == CAFEQ_AXIS_IN && (k % G.g == 0 || G.g % k == 0) && nG <= 8 && ((uintptr_t)W % 16 == 0) &&
@@ -457,7 +453,6 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
     rp2 = ((rp2 + 31) / 32) * 32;
     if (rp2 < rows_per) rows_per = rp2;
     if (rows_per < 32) rows_per = 32;
-    if (tiny && G.d_out * nG <= SCB_SORTED) rows_per = G.d_out;
     const int splits = (G.d_out + rows_per - 1) / rows_per;
     dim3 grid(G.nbq, strips, splits);
     const size_t sh = (size_t)k * (strip + 1) * 4 + (size_t)SCB_MAXP * 6;
@@ -504,7 +499,7 @@ static void launch_scatter(cudaStream_t st, const void* W, const Geo& G, const f
   if (kk_fast(k) && G.g % 4 == 0 && G.g <= 128 && ((uintptr_t)W % 8 == 0) && (G.ld % 4 == 0) && G.axis == CAFEQ_AXIS_OUT) {
     const int strips = k / SC2_JS;
     int splits = (148 * 4 + G.nbq * strips - 1) / (G.nbq * strips);
-    if (splits < 1 || tiny) splits = 1;
+    if (splits < 1) splits = 1;
     int per = (G.ng + splits - 1) / splits;
     splits = (G.ng + per - 1) / per;
     dim3 grid(G.nbq, strips, splits);

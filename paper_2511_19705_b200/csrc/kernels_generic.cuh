@@ -832,7 +832,6 @@ __global__ void __launch_bounds__(256, 3) scatter_in_strip_kernel(const uint16_t
 // The accumulators go through shared memory to a coalesced add into global memory.
 // K in {64, 128, 256}; rows_per_cta * NG <= SCB_MAXP; ld % 8 == 0 and W 16-byte aligned.
 constexpr int SCB_MAXP = 4096;
-constexpr int SCB_SORTED = 512;  // up to this many records a bucket is accumulated in row order
 
 template <int K, int STRIP>
 __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_t* W, long long ld, int d_out,
@@ -913,19 +912,6 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
   __syncthreads();
   // phase C: every thread walks its bucket
   const int b = tid / TPB, part = tid - b * TPB;
-  if (np <= SCB_SORTED) {  // few records: in row order (the placement above is in the order of its atomics)
-    if (part == 0) {
-      for (int i = start[b] + 1; i < start[b + 1]; ++i) {
-        const uint16_t o = rec_o[i];
-        const float c = rec_cf[i];
-        int j = i - 1;
-        for (; j >= start[b] && rec_o[j] > o; --j) { rec_o[j + 1] = rec_o[j]; rec_cf[j + 1] = rec_cf[j]; }
-        rec_o[j + 1] = o;
-        rec_cf[j + 1] = c;
-      }
-    }
-    __syncthreads();
-  }
   float acc[CPT];
 #pragma unroll
   for (int c = 0; c < CPT; ++c) acc[c] = 0.f;

@@ -87,3 +87,17 @@ def test_captured_step_of_a_small_layer(cq):
         assert float(sx[0]) == 12.0 == float(sy[0])
         # (the order of atomic additions differs from run to run: 1e-5 of the change that twelve steps of 1e-4 make)
         assert rel_err(x.cpu().numpy(), y.cpu().numpy()) <= 1e-5 and rel_err(hx[:, 0].cpu().numpy(), hy[:, 0].cpu().numpy()) <= 1e-5
+
+
+@pytest.mark.parametrize("d_out,d_in,k,group", [(512, 128, 64, 64), (256, 256, 64, 16), (64, 128, 64, 128), (300, 192, 64, 64), (4096, 256, 64, 64)])
+def test_gradient_with_every_maximum_in_one_column(cq, d_out, d_in, k, group):
+    """One outlier channel holds the maximum of every row's group: all records of a block go to one row of its gradient."""
+    Wb = syn.weight_student_t(d_out, d_in, 3)
+    W64 = w64(Wb)
+    W64[:, 70] *= 40.0
+    W = torch.from_numpy(W64).cuda().bfloat16()
+    M = syn.perturbed_blocks(d_in // k, k, 5, 0.02)
+    a = cq.cafeq_proxy_loss_fwd_bwd(W, f32_dev(M), bits=4, group=group)
+    W64 = W.double().cpu().numpy()
+    f = orc.single_forward(W64, M, 4, group, "in")
+    assert rel_err(a["gradM"].cpu().numpy(), orc.single_grad_surrogate(W64, f, group, "in")) <= 1e-4
