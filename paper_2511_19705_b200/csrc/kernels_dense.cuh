@@ -34,8 +34,16 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, 
   if (inv_scale) sc = (float)((double)scale / fmax(*inv_scale, 1e-300));
   const bool trans = thi || tlo || YT;
   float2 x2[8];
+  if (((uintptr_t)X & 7) == 0 && (ld & 1) == 0) {
 #pragma unroll
-  for (int q = 0; q < 8; ++q) x2[q] = ld_plain(reinterpret_cast<const float2*>(X + (long long)(r0 + ty + 8 * q) * ld + c0 + 2 * tx));
+    for (int q = 0; q < 8; ++q) x2[q] = ld_plain(reinterpret_cast<const float2*>(X + (long long)(r0 + ty + 8 * q) * ld + c0 + 2 * tx));
+  } else {  // (the caller's product may be any float array)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float* x = X + (long long)(r0 + ty + 8 * q) * ld + c0 + 2 * tx;
+      x2[q] = make_float2(x[0], x[1]);
+    }
+  }
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int i = ty + 8 * q;

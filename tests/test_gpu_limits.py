@@ -101,3 +101,21 @@ def test_gradient_with_every_maximum_in_one_column(cq, d_out, d_in, k, group):
     W64 = W.double().cpu().numpy()
     f = orc.single_forward(W64, M, 4, group, "in")
     assert rel_err(a["gradM"].cpu().numpy(), orc.single_grad_surrogate(W64, f, group, "in")) <= 1e-4
+
+
+@pytest.mark.parametrize("h,d1,d3,k,r", [(64, 64, 128, 64, 1), (128, 192, 64, 32, 2)])
+def test_product_at_any_float_address(cq, h, d1, d3, k, r):
+    """The product is any float array: one that starts 4 bytes off a 16-byte boundary holds the same, and serves as the target."""
+    W1, W2 = to_dev(syn.weight_student_t(h, d1, 3)), to_dev(syn.weight_student_t(d3, r * h, 4))
+    d1_, d2_ = cq._pair_descs(W1, W2, k, 4, 64, 64, r)
+    ws = torch.empty(cq.workspace_size(d1_, d2_), dtype=torch.uint8, device="cuda")
+    buf = torch.full((d1 * d3 + 2,), 9.0, device="cuda")
+    off = buf[1:-1].view(d1, d3)
+    assert off.data_ptr() % 8 == 4
+    rc = cq.lib().cafeq_pair_product(ctypes.byref(d1_), cq._p(W1), ctypes.byref(d2_), cq._p(W2), cq._p(off), cq._p(ws),
+                                     ctypes.c_size_t(ws.numel()), cq._stream())
+    P = cq.cafeq_pair_product(W1, W2, k=k, replicas=r)
+    assert rc == 0 and torch.equal(off, P) and float(buf[0]) == 9.0 == float(buf[-1])
+    M = f32_dev(syn.perturbed_blocks(h // k, k, 5, 0.02))
+    a, b = (cq.cafeq_pair_loss_fwd_bwd(W1, W2, M, bits=4, group1=64, group2=64, replicas=r, P=x, loss_kind=cq.LOSS_PQE_STE) for x in (off, P))
+    assert rel_err(a["gradM"].cpu().numpy(), b["gradM"].cpu().numpy()) <= 1e-5 and abs(float(a["losses"][3] / b["losses"][3]) - 1) <= 1e-5
