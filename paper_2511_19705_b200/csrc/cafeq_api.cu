@@ -770,6 +770,10 @@ static int check_ws(void* ws, size_t ws_bytes) {
   return CAFEQ_OK;
 }
 
+// The fused gradient chain reads and writes the gradient through a tensor map, which wants 16-byte alignment: a gradient array that
+// starts elsewhere is filled from one in the workspace (the size queries count it).
+static bool grad_off_16(const float* gradM) { return ((uintptr_t)gradM & 15) != 0; }
+
 static int last_launch() { return cudaGetLastError() == cudaSuccess ? CAFEQ_OK : CAFEQ_ERR_CUDA; }
 
 // ------------------------------------------------------------------------------------------------
@@ -1191,6 +1195,8 @@ extern "C" int cafeq_proxy_loss_fwd_bwd(const cafeq_matrix_desc* d, const void* 
   cudaStream_t st = (cudaStream_t)stream;
   Bump b(ws, ws_bytes);
   SingleWS s;
+  const long long kk = (long long)G.nbT * G.k * G.k;
+  const bool off_grad = want_grad && grad_off_16(gradM);
   // Eq. 4 alone on a shape the tensor-core pass covers leaves nothing matrix-sized in scratch (the lean size of
   // cafeq_workspace_size with a CAFEQ_LOSS_SURROGATE configuration is enough); everything else takes the full carving
   bool lean = false;
@@ -1204,15 +1210,19 @@ extern "C" int cafeq_proxy_loss_fwd_bwd(const cafeq_matrix_desc* d, const void* 
       Bump probe(nullptr, 0);
       SingleWS tmp;
       carve_single(probe, G, &tmp, true, false);
+      if (off_grad) probe.take<float>(kk);
       if (probe.used <= ws_bytes) lean = false;
     }
   }
   if (!carve_single(b, G, &s, true, lean)) return CAFEQ_ERR_WORKSPACE;
+  float* grad = off_grad ? b.take<float>(kk) : gradM;
+  if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   const bool warm = (flags & CAFEQ_FLAG_WARM_MINV) && Minv;
-  if (warm) CQ_LAUNCH(copy_f32_kernel, grid_for((long long)G.nbT * G.k * G.k), 256, 0, st, Minv, s.Minv, (long long)G.nbT * G.k * G.k);
+  if (warm) CQ_LAUNCH(copy_f32_kernel, grid_for(kk), 256, 0, st, Minv, s.Minv, kk);
   single_step(st, d, G, W, M, Minv, offsets, offsets_kind, loss_kind, kappa, (flags & CAFEQ_FLAG_EXACT_LOSS) != 0, losses,
-              nullptr, want_grad ? gradM : nullptr, status, s, (flags & CAFEQ_FLAG_GENERIC) != 0, warm, nullptr, grad_offsets);
+              nullptr, want_grad ? grad : nullptr, status, s, (flags & CAFEQ_FLAG_GENERIC) != 0, warm, nullptr, grad_offsets);
   if (s.err) return s.err;
+  if (off_grad) CQ_LAUNCH(copy_f32_kernel, grid_for(kk), 256, 0, st, grad, gradM, kk);
   return last_launch();
 }
 
@@ -1708,10 +1718,15 @@ extern "C" int cafeq_pair_loss_fwd_bwd(const cafeq_matrix_desc* d1, const void* 
   Bump b(ws, ws_bytes);
   PairWS p;
   if (!carve_pair(b, G1, G2, &p, want_pqe)) return CAFEQ_ERR_WORKSPACE;
+  const long long kk = (long long)G1.nbT * G1.k * G1.k;
+  const bool off_grad = want_grad && grad_off_16(gradM);
+  float* grad = off_grad ? b.take<float>(kk) : gradM;
+  if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   if (objective == 2) pair_grams((cudaStream_t)stream, W1, G1, W2, G2, p, status);
   pair_step((cudaStream_t)stream, d1, d2, G1, G2, W1, W2, M, P, lse_t, lambda_orth, want_pqe, losses, nullptr,
-            want_grad ? gradM : nullptr, status, p, (flags & CAFEQ_FLAG_GENERIC) != 0, false, nullptr, ste, objective);
+            want_grad ? grad : nullptr, status, p, (flags & CAFEQ_FLAG_GENERIC) != 0, false, nullptr, ste, objective);
   if (p.err) return p.err;
+  if (off_grad) CQ_LAUNCH(copy_f32_kernel, grid_for(kk), 256, 0, (cudaStream_t)stream, grad, gradM, kk);
   return last_launch();
 }
 

@@ -119,3 +119,37 @@ def test_product_at_any_float_address(cq, h, d1, d3, k, r):
     M = f32_dev(syn.perturbed_blocks(h // k, k, 5, 0.02))
     a, b = (cq.cafeq_pair_loss_fwd_bwd(W1, W2, M, bits=4, group1=64, group2=64, replicas=r, P=x, loss_kind=cq.LOSS_PQE_STE) for x in (off, P))
     assert rel_err(a["gradM"].cpu().numpy(), b["gradM"].cpu().numpy()) <= 1e-5 and abs(float(a["losses"][3] / b["losses"][3]) - 1) <= 1e-5
+
+
+def _call_proxy(cq, W, M, grad, k, group=128):
+    d = cq.make_desc(W.shape[0], W.shape[1], 4, group, k, cq.AXIS_IN, cq.APPLY_T, 1, W.stride(0))
+    losses, status = torch.zeros(4, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(cq.workspace_size(d), dtype=torch.uint8, device="cuda")
+    rc = cq.lib().cafeq_proxy_loss_fwd_bwd(ctypes.byref(d), cq._p(W), cq._p(M), None, None, 0, cq.LOSS_SURROGATE, ctypes.c_float(0), 0,
+                                           cq._p(losses), cq._p(grad), None, cq._p(status), cq._p(ws), ctypes.c_size_t(ws.numel()), cq._stream())
+    assert rc == 0 and int(status.item()) == 0
+    return losses
+
+
+@pytest.mark.parametrize("k", [32, 64, 128, 256])
+def test_gradient_at_any_float_address(cq, k):
+    """The gradient's array is any float array: one that starts 4 bytes off a 16-byte boundary holds the same."""
+    W = to_dev(syn.weight_student_t(192, 512, 3))
+    M = f32_dev(syn.perturbed_blocks(512 // k, k, 5, 0.05))
+    aligned, buf = torch.empty_like(M), torch.full((M.numel() + 2,), 9.0, device="cuda")
+    off = buf[1:-1]
+    assert off.data_ptr() % 16 == 4
+    _call_proxy(cq, W, M, aligned, k)
+    _call_proxy(cq, W, M, off, k)
+    assert rel_err(off.cpu().numpy(), aligned.flatten().cpu().numpy()) <= 1e-5 and float(buf[0]) == 9.0 == float(buf[-1])
+    # the same for a pair
+    W1 = to_dev(syn.weight_student_t(512, 256, 4))
+    d1, d2 = cq._pair_descs(W1, W, k, 4, 128, 128, 1)
+    ws = torch.empty(cq.workspace_size(d1, d2), dtype=torch.uint8, device="cuda")
+    for g in (aligned, off):
+        losses, status = torch.zeros(4, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        rc = cq.lib().cafeq_pair_loss_fwd_bwd(ctypes.byref(d1), cq._p(W1), ctypes.byref(d2), cq._p(W), cq._p(M), None, cq.LOSS_LSE,
+                                              ctypes.c_float(5.0), ctypes.c_float(0.1), 0, cq._p(losses), cq._p(g), cq._p(status),
+                                              cq._p(ws), ctypes.c_size_t(ws.numel()), cq._stream())
+        assert rc == 0 and int(status.item()) == 0
+    assert rel_err(off.cpu().numpy(), aligned.flatten().cpu().numpy()) <= 1e-5 and float(buf[0]) == 9.0 == float(buf[-1])
