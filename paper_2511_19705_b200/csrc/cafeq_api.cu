@@ -774,6 +774,22 @@ static int check_ws(void* ws, size_t ws_bytes) {
 // starts elsewhere is filled from one in the workspace (the size queries count it).
 static bool grad_off_16(const float* gradM) { return ((uintptr_t)gradM & 15) != 0; }
 
+// Where an optimiser state keeps the inverse of the last step's transform.  The kernels move it 16 bytes at a time: one that starts
+// elsewhere is copied to the workspace's own array (`ws_inv`) for the call and back.
+struct StoredInverse {
+  float *slot, *inv;
+  long long kk;
+  cudaStream_t st;
+  bool copied() const { return slot && inv != slot; }
+  StoredInverse(float* opt_state, float* ws_inv, long long n, bool resume, cudaStream_t stream)
+      : slot(opt_state ? opt_state + CAFEQ_OPT_STATE_HEADER + 2 * n : nullptr), inv(slot && !((uintptr_t)slot & 15) ? slot : ws_inv), kk(n), st(stream) {
+    if (copied() && resume) CQ_LAUNCH(copy_f32_kernel, grid_for(kk), 256, 0, st, slot, inv, kk);
+  }
+  void keep(int steps) const {
+    if (copied() && steps > 0) CQ_LAUNCH(copy_f32_kernel, grid_for(kk), 256, 0, st, inv, slot, kk);
+  }
+};
+
 static int last_launch() { return cudaGetLastError() == cudaSuccess ? CAFEQ_OK : CAFEQ_ERR_CUDA; }
 
 // ------------------------------------------------------------------------------------------------
@@ -1249,7 +1265,8 @@ extern "C" int cafeq_optimize_single(const cafeq_matrix_desc* d, const void* W, 
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   // the inverse of the last step's transform lives in the optimiser state, so a resumed run refines it
   const bool resume = cfg->resume && opt_state;
-  if (opt_state) s.Minv = opt_state + CAFEQ_OPT_STATE_HEADER + 2 * kk;
+  const StoredInverse stored(opt_state, s.Minv, kk, resume, st);
+  s.Minv = stored.inv;
   for (int it = 0; it < cfg->steps; ++it) {
     bool eval = cfg->eval_every > 0 && (it % cfg->eval_every == 0);
     single_step(st, d, G, W, M, nullptr, nullptr, CAFEQ_OFFSETS_NONE, cfg->loss_kind, kappa, eval, nullptr,
@@ -1262,6 +1279,7 @@ extern "C" int cafeq_optimize_single(const cafeq_matrix_desc* d, const void* W, 
                                                        status);
     }
   }
+  stored.keep(cfg->steps);
   return last_launch();
 }
 
@@ -1756,7 +1774,8 @@ extern "C" int cafeq_optimize_pair(const cafeq_matrix_desc* d1, const void* W1, 
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   // the inverse of the last step's transform lives in the optimiser state, so a resumed run refines it
   const bool resume = cfg->resume && opt_state;
-  if (opt_state) p.Minv = opt_state + CAFEQ_OPT_STATE_HEADER + 2 * kk;
+  const StoredInverse stored(opt_state, p.Minv, kk, resume, st);
+  p.Minv = stored.inv;
   if (objective == 2) pair_grams(st, W1, G1, W2, G2, p, status);
   for (int it = 0; it < cfg->steps; ++it) {
     bool eval = ste || (any_pqe && (it % cfg->eval_every == 0));
@@ -1773,6 +1792,7 @@ extern "C" int cafeq_optimize_pair(const cafeq_matrix_desc* d1, const void* W1, 
                                                        status);
     }
   }
+  stored.keep(cfg->steps);
   return last_launch();
 }
 

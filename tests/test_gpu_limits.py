@@ -153,3 +153,29 @@ def test_gradient_at_any_float_address(cq, k):
                                               cq._p(ws), ctypes.c_size_t(ws.numel()), cq._stream())
         assert rc == 0 and int(status.item()) == 0
     assert rel_err(off.cpu().numpy(), aligned.flatten().cpu().numpy()) <= 1e-5 and float(buf[0]) == 9.0 == float(buf[-1])
+
+
+@pytest.mark.parametrize("k", [32, 64, 128, 256])
+@pytest.mark.parametrize("pair", [False, True])
+def test_optimiser_state_at_any_float_address(cq, k, pair):
+    """The per-problem runs take a state that starts 4 bytes off a 16-byte boundary, and resume from it."""
+    W = to_dev(syn.weight_student_t(192, 512, 3))
+    W1 = to_dev(syn.weight_student_t(512, 256, 4))
+    M0 = f32_dev(syn.perturbed_blocks(512 // k, k, 5, 0.02))
+    n = cq.OPT_STATE_HEADER + 3 * M0.numel()
+    got = []
+    for shift in (0, 1):
+        buf = torch.zeros(n + 4, device="cuda")
+        state, M = buf[shift:shift + n], M0.clone()
+        assert state.data_ptr() % 16 == 4 * shift
+        for resume in (0, 1):
+            cfg = cq.make_cfg(loss_kind=cq.LOSS_LSE if pair else cq.LOSS_SURROGATE, optimizer=cq.OPT_ADAM, lr=1e-4, beta1=0.9, steps=3, resume=resume)
+            if pair:
+                h, st, _ = cq.cafeq_optimize_pair(W1, W, M, cfg, bits=4, group1=128, group2=128, opt_state=state)
+            else:
+                h, st, _ = cq.cafeq_optimize_single(W, M, cfg, bits=4, group=128, opt_state=state)
+            assert int(st.item()) == 0
+        assert float(buf[:shift].abs().sum()) == 0.0 == float(buf[shift + n:].abs().sum()) and float(state[0]) == 6.0
+        got.append((M, state[cq.OPT_STATE_HEADER + 2 * M0.numel():].clone(), h[:, 0]))
+    for a, b in zip(*got):  # parameters, the stored inverse, losses
+        assert rel_err(a.cpu().numpy(), b.cpu().numpy()) <= 1e-5
