@@ -601,7 +601,7 @@ static void carve_matrix(Bump& b, const Geo& G, MatWS* w, bool need_E, bool lean
 static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo& G, const float* Top, int transposed,
                        uint16_t* Tb, BdParams p, int32_t* status, const uint16_t* Tb_ready = nullptr) {
   const int form = (G.axis == CAFEQ_AXIS_IN) ? BD_IN : BD_OUT;
-  // blocks of 32 go through as pairs on the diagonal of blocks of 64 (exact: the other products are with zeros)
+  // blocks of 32 go through as pairs on the diagonal of blocks of 64
   const int two = (form == BD_IN && G.k == 32 && G.r == 1) ? 1 : 0;
   const int k = two ? 64 : G.k, nbT = two ? G.nbT / 2 : G.nbT;
   if (!bd_supported(form, G.d_out, G.d_in, ldx, k, G.g, X)) return false;
@@ -610,6 +610,7 @@ static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo&
   p.d_out = G.d_out;
   p.d_in = G.d_in;
   p.r = G.r;
+  p.pairs = two;
   p.status = status;
   int ti = kt_begin(5, st);
   g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -35,6 +35,7 @@ struct BdParams {
   int d_out, d_in;     // shape of X
   int r;               // matrix blocks per operator block
   int t_mn;            // output axis: the operator blocks are stored transposed (T[j][i]; read as an MN-major operand)
+  int pairs;           // input axis, K = 64: blocks of 32, two on the diagonal of each operator block
   int n_major;         // IN: tile columns (256 d_in columns each); OUT: row blocks (k rows each)
   int n_minor;         // IN: row tiles of 128; OUT: column tiles of NC
   int ctas_per_major;
@@ -451,6 +452,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
         if (base >= t_end) break;
         const int n_minor = mp.p[sub].n_minor;
         const bool t_mn = FORM == BD_OUT && mp.p[sub].t_mn;
+        const bool pairs = FORM == BD_IN && K == 64 && mp.p[sub].pairs;
         const uint32_t idesc_out = t_mn ? umma_idesc_bf16(128, 128, 1, 1) : umma_idesc_bf16(128, 128, 0, 1);
         const int lo = (t_begin > base ? t_begin : base) - base;
         const int hi = (t_end < mp.tile_end[sub] ? t_end : mp.tile_end[sub]) - base;
@@ -483,8 +485,16 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               if (elect_one()) {
                 const uint32_t alo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES);
                 const uint32_t blo = tlo + ((bi * K * K * 2 + ci * K * 128) >> 4);
+                if (K == 64 && pairs) {
+                  // Each 32 columns meet their own block only, the diagonal quarter of the operator tile (rows 32 half ..).  The
+                  // whole tile would add products with zeros: exact, but an infinity or NaN times zero is NaN.
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) tc_mma_lo(dbase + bi * K, alo + 2 * kk, blo + 2 * kk, idesc_in, (ci | kk) != 0 ? 1u : 0u);
+                  for (int kk = 0; kk < 4; ++kk)
+                    tc_mma_lo(dbase + bi * K + (kk >> 1) * 32, alo + 2 * kk, blo + (kk >> 1) * 256 + 2 * kk, umma_idesc_bf16(128, 32, 0, 0), kk & 1);
+                } else {
+#pragma unroll
+                  for (int kk = 0; kk < 4; ++kk) tc_mma_lo(dbase + bi * K, alo + 2 * kk, blo + 2 * kk, idesc_in, (ci | kk) != 0 ? 1u : 0u);
+                }
                 tc_commit(bar_empty + 8 * st);
                 if (sidx == BD_STAGES_PER_TILE - 1) tc_commit(bar_accf + 8 * buf);
               }

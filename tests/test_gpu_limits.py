@@ -179,3 +179,18 @@ def test_optimiser_state_at_any_float_address(cq, k, pair):
         got.append((M, state[cq.OPT_STATE_HEADER + 2 * M0.numel():].clone(), h[:, 0]))
     for a, b in zip(*got):  # parameters, the stored inverse, losses
         assert rel_err(a.cpu().numpy(), b.cpu().numpy()) <= 1e-5
+
+
+@pytest.mark.parametrize("rows", [5, 130])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+@pytest.mark.parametrize("k", [32, 64, 128])
+def test_non_finite_activation_stays_in_its_block(cq, k, value, rows):
+    X = to_dev(syn.weight_student_t(rows, 512, 3))
+    T = f32_dev(syn.perturbed_blocks(512 // k, k, 5, 0.1))
+    clean = cq.cafeq_apply_transform(X, T)
+    X[3, 70] = value
+    out = cq.cafeq_apply_transform(X, T)
+    b = 70 // k
+    hit = torch.zeros_like(out, dtype=torch.bool)
+    hit[3, b * k:(b + 1) * k] = True
+    assert not torch.isfinite(out[hit]).any() and torch.equal(out[~hit], clean[~hit])
