@@ -582,8 +582,7 @@ struct MatWS {
 // lean: the matrix goes through the fused tensor-core pass and nothing but the per-group records leaves it (Eq. 4 /
 // LogSumExp steps without the quantised loss): no matrix-sized scratch at all.
 static void carve_matrix(Bump& b, const Geo& G, MatWS* w, bool need_E, bool lean = false) {
-  // (blocks of 32 may be widened to 64)
-  w->Tb = b.take<uint16_t>((size_t)(G.nbT > 0 ? G.nbT : 1) * (G.k > 0 ? G.k : 1) * (G.k > 0 ? G.k : 1) * (G.k == 32 ? 2 : 1) + (G.k == 32 ? 4096 : 0));
+  w->Tb = b.take<uint16_t>((size_t)(G.nbT > 0 ? G.nbT : 1) * (G.k > 0 ? G.k : 1) * (G.k > 0 ? G.k : 1));
   w->Dbf = lean ? nullptr : b.take<uint16_t>(G.n);
   w->U = lean ? nullptr : b.take<float>(G.n);
   w->D = lean ? nullptr : b.take<float>(G.n);
@@ -599,12 +598,14 @@ static void carve_matrix(Bump& b, const Geo& G, MatWS* w, bool need_E, bool lean
 
 // One fused tensor-core pass (see kernels_fused.cuh); returns false when the shape is not covered.
 static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo& G, const float* Top, int transposed,
-                       uint16_t* Tb, BdParams p, int32_t* status, const uint16_t* Tb_ready = nullptr) {
+                       uint16_t* Tb, BdParams p, int32_t* status, const uint16_t* Tb_ready = nullptr, void* pair_scratch = nullptr) {
   const int form = (G.axis == CAFEQ_AXIS_IN) ? BD_IN : BD_OUT;
-  // blocks of 32 go through as pairs on the diagonal of blocks of 64
-  const int two = (form == BD_IN && G.k == 32 && G.r == 1) ? 1 : 0;
+  // blocks of 32 go through as pairs on the diagonal of blocks of 64, which take twice the room: 4 bytes per operator entry that
+  // the pass leaves alone (pair_scratch; null: not in pairs)
+  const int two = (form == BD_IN && G.k == 32 && G.r == 1 && pair_scratch) ? 1 : 0;
   const int k = two ? 64 : G.k, nbT = two ? G.nbT / 2 : G.nbT;
   if (!bd_supported(form, G.d_out, G.d_in, ldx, k, G.g, X)) return false;
+  if (two) Tb = (uint16_t*)pair_scratch;
   if (Tb_ready && !transposed && !two) Tb = const_cast<uint16_t*>(Tb_ready);  // bf16 operator already in applied orientation
   else launch_operator_bf16(st, Top, Tb, G.k, G.nbT, transposed, status, two);
   p.d_out = G.d_out;
@@ -618,6 +619,9 @@ static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo&
   kt_end(ti, st);
   return rc == CAFEQ_OK;
 }
+
+// The pass stores no U, so the array for it can hold paired operators: 64 d_in bf16 against d_out d_in fp32.
+static void* pair_scratch(const MatWS& w, const Geo& G) { return G.d_out >= 32 ? w.U : nullptr; }
 
 static bool tc_apply_ok(int k) { return k == 32 || kk_fast(k); }
 
@@ -669,7 +673,7 @@ static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits
     p.qmax = qmax_of(bits);
     p.a = w.a; p.usel = w.usel; p.idx = w.idx;
     p.delta = w.Dbf; p.codes = codes; p.scales = scales;
-    if (fused_pass(st, W, G.ld, G, Tc, transposed, w.Tb, p, status, Tb_ready)) return true;
+    if (fused_pass(st, W, G.ld, G, Tc, transposed, w.Tb, p, status, Tb_ready, pair_scratch(w, G))) return true;
   }
   if (!w.U) return false;  // lean workspace: there is no scratch for the shape-agnostic kernels (callers check first)
   bool applied = false;
@@ -855,7 +859,7 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
 // ------------------------------------------------------------------------------------------------
 static size_t apply_scratch(const Geo& G, bool fused) {
   const size_t kk = (size_t)G.nbT * G.k * G.k;
-  return 1024 + kk * 8 + (fused ? 0 : (size_t)G.n * 4 + 256);
+  return 1024 + kk * 6 + (fused ? 0 : (size_t)G.n * 4 + 256);
 }
 static Geo apply_geo(Geo G) {
   // the store epilogue ignores the quantisation groups: any group width the pass is built for will do
@@ -888,7 +892,7 @@ extern "C" int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, 
   const long long kk = (long long)G.nbT * G.k * G.k;
   Bump b(ws, ws_bytes);
   float* Tc = b.take<float>(kk);
-  uint16_t* Tb = b.take<uint16_t>(G.k == 32 ? 2 * kk : kk);
+  uint16_t* Tb = b.take<uint16_t>(kk);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
   // the deployed operator is the bf16 rounding of the given one (what the tensor cores apply; the pass converts it
   // itself, the shape-agnostic kernels take the rounded fp32 copy)
@@ -904,7 +908,7 @@ extern "C" int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, 
     memset(&p, 0, sizeof(p));
     p.epi = EPI_STORE;
     p.delta = reinterpret_cast<uint16_t*>(Y);
-    if (fused_pass(st, X, G.ld, Ga, T, transposed, Tb, p, status, nullptr)) return last_launch();
+    if (fused_pass(st, X, G.ld, Ga, T, transposed, Tb, p, status, nullptr, Tc)) return last_launch();
   }
   float* U = b.take<float>(G.n);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
@@ -1141,7 +1145,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       memset(&bp, 0, sizeof(bp));
       bp.epi = EPI_SQSUM;
       bp.sqacc = s.acc + 1;
-      done = fused_pass(st, s.m.Dbf, G.d_in, G, s.Minv, 0, s.m.Tb, bp, status);
+      done = fused_pass(st, s.m.Dbf, G.d_in, G, s.Minv, 0, s.m.Tb, bp, status, nullptr, pair_scratch(s.m, G));
     }
     if (!done)
       launch_apply(st, s.m.D, 0, G.d_in, G, s.Minv, 0, s.m.E, G.d_in, (ste ? GEMM_STORE : 0) | GEMM_SQSUM, s.acc + 1, status);

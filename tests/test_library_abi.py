@@ -72,3 +72,21 @@ def test_missing_library_fails_loudly(cq, monkeypatch):
     monkeypatch.setattr(m, "LIB_PATH", os.path.join(ROOT, "does_not_exist.so"))
     with pytest.raises(RuntimeError):
         m.lib()
+
+
+def test_scratch_of_blocks_of_32_is_that_of_any_block(cq):
+    """cafeq_rtn's scratch beside the matrix-sized buffers is its operator, once in fp32 and once in bf16, whatever the block size:
+    paired blocks need no room of their own (the built-in buffer of cafeq_rtn_noalloc holds what it always held)."""
+    for d_out, d_in, axis in ((1, 512, cq.AXIS_IN), (64, 4096, cq.AXIS_IN), (500, 384, cq.AXIS_IN), (1024, 512, cq.AXIS_OUT)):
+        for group in (0, 64, 128):
+            n = {k: cq.rtn_workspace_size(cq.make_desc(d_out, d_in, 4, group, k, axis), True) for k in (16, 32)}
+            dim = d_in if axis == cq.AXIS_IN else d_out
+            assert n[32] - n[16] == 6 * dim * 16, (d_out, d_in, axis, group)
+
+
+def test_apply_scratch_is_two_forms_of_the_operator(cq):
+    for k in (32, 64, 256):
+        d = cq.make_desc(300, 512, 4, 128, k)
+        n = ctypes.c_size_t(0)
+        assert cq.lib().cafeq_apply_workspace_size(ctypes.byref(d), ctypes.byref(n)) == 0
+        assert n.value <= 1024 + 6 * 512 * k + (300 * 512 * 4 + 256 if k == 32 else 0)
