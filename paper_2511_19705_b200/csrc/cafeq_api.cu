@@ -798,6 +798,14 @@ struct StoredInverse {
 static int last_launch() { return cudaGetLastError() == cudaSuccess ? CAFEQ_OK : CAFEQ_ERR_CUDA; }
 
 // ------------------------------------------------------------------------------------------------
+// Shapes whose scratch is sized for the tensor-core pass alone, so that weights which the pass cannot take (rows off 16-byte
+// boundaries) are refused for lack of scratch.  A last half tile of 128 columns goes through the pass too, but its scratch stays
+// that of the shape-agnostic kernels: such weights are taken at any address.
+static bool sized_for_pass(const Geo& G, const void* W) {
+  const bool in = G.axis == CAFEQ_AXIS_IN;
+  return kk_fast(G.k) && bd_supported(in ? BD_IN : BD_OUT, G.d_out, G.d_in, G.ld, G.k, G.g, W) && (!in || G.d_in % 256 == 0);
+}
+
 // What cafeq_rtn needs from its workspace: nothing when the streaming kernel covers the call (no transform, group 32 /
 // 64 / 128 / 256, aligned rows), the per-group records and the rounded operator when the fused tensor-core pass
 // covers it, matrix-sized fp32 buffers otherwise.  W / codes may be null (a size query): aligned pointers are assumed.
@@ -809,8 +817,7 @@ static size_t rtn_scratch(const Geo& G, bool has_T, const void* W, const int8_t*
   if (!has_T && (G.g == 32 || G.g == 64 || G.g == 128 || G.g == 256) && !((uintptr_t)W & 15) && !(G.ld % 8) &&
       !((uintptr_t)codes & 7))
     return 0;
-  const bool lean = has_T && kk_fast(G.k) &&
-                    bd_supported(G.axis == CAFEQ_AXIS_IN ? BD_IN : BD_OUT, G.d_out, G.d_in, G.ld, G.k, G.g, W);
+  const bool lean = has_T && sized_for_pass(G, W);
   carve_matrix(b, G, &m, false, lean);
   float* t = has_T ? b.take<float>((size_t)G.nbT * G.k * G.k) : nullptr;
   if (Tc) *Tc = t;
@@ -875,9 +882,7 @@ extern "C" int cafeq_apply_workspace_size(const cafeq_matrix_desc* d, size_t* by
   const Geo Ga = apply_geo(G);
   // (X itself is not known here: 16-byte aligned rows are assumed; a call whose X does not qualify returns
   // CAFEQ_ERR_WORKSPACE)
-  const bool two = G.axis == CAFEQ_AXIS_IN && G.k == 32 && G.r == 1;  // (see fused_pass)
-  const bool fused = bd_supported(G.axis == CAFEQ_AXIS_IN ? BD_IN : BD_OUT, Ga.d_out, Ga.d_in, Ga.ld, two ? 64 : Ga.k, Ga.g, nullptr);
-  *bytes = apply_scratch(G, fused);
+  *bytes = apply_scratch(G, sized_for_pass(Ga, nullptr));
   return CAFEQ_OK;
 }
 
@@ -986,7 +991,7 @@ static bool carve_single(Bump& b, const Geo& G, SingleWS* s, bool need_E, bool l
 // call whose weights turn out not to qualify returns CAFEQ_ERR_WORKSPACE.)
 static bool lean_single_ok(const Geo& G, const cafeq_opt_cfg* cfg, const void* W) {
   if (!cfg || cfg->loss_kind != CAFEQ_LOSS_SURROGATE || cfg->eval_every != 0) return false;
-  return kk_fast(G.k) && bd_supported(G.axis == CAFEQ_AXIS_IN ? BD_IN : BD_OUT, G.d_out, G.d_in, G.ld, G.k, G.g, W);
+  return sized_for_pass(G, W);
 }
 // Enqueue one forward(+backward) for a single matrix; gradM may be null.  hist is an optional [2] slot.
 static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& G, const void* W, const float* M,
@@ -1439,8 +1444,7 @@ static bool carve_pair(Bump& b, const Geo& G1, const Geo& G2, PairWS* p, bool ne
 static bool lean_pair_ok(const Geo& G1, const Geo& G2, const cafeq_opt_cfg* cfg, const void* W1, const void* W2) {
   if (!cfg || cfg->eval_every != 0) return false;
   if (cfg->loss_kind != CAFEQ_LOSS_LSE && cfg->loss_kind != CAFEQ_LOSS_SUMSQ && cfg->loss_kind != CAFEQ_LOSS_SUMSQ_WEIGHTED) return false;
-  return kk_fast(G1.k) && bd_supported(BD_OUT, G1.d_out, G1.d_in, G1.ld, G1.k, G1.g, W1) &&
-         bd_supported(BD_IN, G2.d_out, G2.d_in, G2.ld, G2.k, G2.g, W2);
+  return sized_for_pass(G1, W1) && sized_for_pass(G2, W2);
 }
 
 // Block Grams of a pair's weights (constants of a run): G1[b][i][j] = sum_x W1[b k + i, x] W1[b k + j, x] and

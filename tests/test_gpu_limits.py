@@ -194,3 +194,24 @@ def test_non_finite_activation_stays_in_its_block(cq, k, value, rows):
     hit = torch.zeros_like(out, dtype=torch.bool)
     hit[3, b * k:(b + 1) * k] = True
     assert not torch.isfinite(out[hit]).any() and torch.equal(out[~hit], clean[~hit])
+
+
+@pytest.mark.parametrize("k", [32, 64, 128])
+@pytest.mark.parametrize("shift", [1, 2])
+def test_weights_and_activations_at_any_address(cq, monkeypatch, k, shift):
+    """384 columns of a wider array: the workspace that a call's own size query gives is enough wherever they start."""
+    monkeypatch.setattr(cq, "workspace", lambda n, device="cuda": torch.empty(int(n), dtype=torch.uint8, device=device))  # (not a larger one)
+    wide = torch.zeros((300, 392), dtype=torch.bfloat16, device="cuda")
+    off = wide[:, shift:shift + 384]
+    off.copy_(to_dev(syn.weight_student_t(300, 384, 3, 2, 10.0)))
+    W = off.contiguous()
+    T = f32_dev(syn.perturbed_blocks(384 // k, k, 5, 0.1))
+    a, b = cq.cafeq_apply_transform(off, T), cq.cafeq_apply_transform(W, T)
+    assert rel_err(a.float().cpu().numpy(), b.float().cpu().numpy()) <= 1e-3  # (sums in another order, then bf16)
+    for group in (64, 128):
+        (c1, s1), (c2, s2) = (cq.cafeq_rtn(x, T, bits=4, group=group, tblock=k) for x in (off, W))
+        assert float((c1 != c2).float().mean()) <= 1e-4 and rel_err(s1.cpu().numpy(), s2.cpu().numpy()) <= 1e-6
+    M1, M2 = T.clone(), T.clone()
+    cfg = cq.make_cfg(steps=2, lr=1e-3)
+    (h1, st1, _), (h2, st2, _) = (cq.cafeq_optimize_single(x, m, cfg, bits=4, group=128) for x, m in ((off, M1), (W, M2)))
+    assert int(st1.item()) == 0 == int(st2.item()) and rel_err(h1[:, 0].cpu().numpy(), h2[:, 0].cpu().numpy()) <= 1e-5
