@@ -384,8 +384,7 @@ static int ly_plan(const cafeq_layer_problem* probs, int n, void* ws, size_t ws_
       Mt.bits = side ? in.d2.bits : in.d1.bits;
       // every matrix goes through the tensor-core pass and the tensor-core backward with one block and group size
       if (Mt.G.k != L->k || Mt.G.g != L->g || !(L->k == 128 || L->k == 256)) return CAFEQ_ERR_UNSUPPORTED;
-      const int form = Mt.G.axis == CAFEQ_AXIS_IN ? BD_IN : BD_OUT;
-      if (!bd_supported(form, Mt.G.d_out, Mt.G.d_in, Mt.G.ld, Mt.G.k, Mt.G.g, Mt.W)) return CAFEQ_ERR_UNSUPPORTED;
+      if (!sized_for_pass(Mt.G, Mt.W)) return CAFEQ_ERR_UNSUPPORTED;  // (no half tiles)
       if (!bw_supported(Mt.G.axis == CAFEQ_AXIS_IN, Mt.G.d_out, Mt.G.d_in, Mt.G.ld, Mt.G.k, Mt.G.g, Mt.W)) return CAFEQ_ERR_UNSUPPORTED;
       if (Mt.G.d_in % 8) return CAFEQ_ERR_UNSUPPORTED;
       if (side) P.m1 = nm;

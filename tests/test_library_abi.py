@@ -90,3 +90,14 @@ def test_apply_scratch_is_two_forms_of_the_operator(cq):
         n = ctypes.c_size_t(0)
         assert cq.lib().cafeq_apply_workspace_size(ctypes.byref(d), ctypes.byref(n)) == 0
         assert n.value <= 1024 + 6 * 512 * k + (300 * 512 * 4 + 256 if k == 32 else 0)
+
+
+def test_layer_calls_take_the_widths_that_they_state(cq):
+    """d_in a multiple of 256 on the input axis; other widths belong to the per-problem calls."""
+    for d_in, rc in ((512, 0), (384, 2)):
+        p = cq.LayerProblem()
+        p.struct_size, p.pair = ctypes.sizeof(cq.LayerProblem), 0
+        p.d1 = p.d2 = cq.make_desc(256, d_in, 4, 128, 128)
+        p.W1, p.M, p.loss_history, p.cfg = 4096, 4096, 4096, cq.make_cfg()
+        n = ctypes.c_size_t(0)
+        assert cq.lib().cafeq_layer_workspace_size(ctypes.byref(p), 1, ctypes.byref(n)) == rc
