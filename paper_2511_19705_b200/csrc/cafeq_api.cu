@@ -846,9 +846,6 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (rtn_stream_launch(st, W, G.ld, G.d_out, G.d_in, G.g, qmax_of(d->bits), codes, scales)) return last_launch();
     g_launches.fetch_sub(1, std::memory_order_relaxed);
-    if (launch_group_quant_vec<uint16_t>(st, (const uint16_t*)W, G.ld, G.d_out, G.ng, G.g, qmax_of(d->bits), nullptr, CAFEQ_OFFSETS_NONE,
-                                         nullptr, nullptr, nullptr, nullptr, nullptr, codes, scales, nullptr))
-      return last_launch();
   }
   if ((rc = check_ws(ws, ws_bytes))) return rc;
   Bump b(ws, ws_bytes);
@@ -856,6 +853,10 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
   float* Tc = nullptr;
   rtn_scratch(G, has_T, W, codes, &b, &w, &Tc);
   if (b.overflow) return CAFEQ_ERR_WORKSPACE;
+  // (other groups without a transform: one kernel from the weights themselves where rows and widths allow, the workspace unused)
+  if (!has_T && launch_group_quant_vec<uint16_t>(st, (const uint16_t*)W, G.ld, G.d_out, G.ng, G.g, qmax_of(d->bits), nullptr,
+                                                 CAFEQ_OFFSETS_NONE, nullptr, nullptr, nullptr, nullptr, nullptr, codes, scales, nullptr))
+    return last_launch();
   forward_quant(st, W, G, d->bits, has_T ? T : nullptr, d->trole == CAFEQ_APPLY_TT, w, nullptr, CAFEQ_OFFSETS_NONE, false, nullptr, codes,
                 scales, nullptr, true, nullptr, nullptr, Tc);
   return last_launch();

@@ -101,3 +101,16 @@ def test_layer_calls_take_the_widths_that_they_state(cq):
         p.W1, p.M, p.loss_history, p.cfg = 4096, 4096, 4096, cq.make_cfg()
         n = ctypes.c_size_t(0)
         assert cq.lib().cafeq_layer_workspace_size(ctypes.byref(p), 1, ctypes.byref(n)) == rc
+
+
+def test_rounding_without_a_transform_asks_for_its_workspace(cq):
+    """Groups of 32 / 64 / 128 / 256 need none; every other width is refused without the one that the size query states."""
+    p = ctypes.c_void_p(4096)  # (never read: the check comes first)
+    for group in (512, 16, 0):
+        d = cq.make_desc(8, 512, 4, group)
+        need = cq.rtn_workspace_size(d, False)
+        assert need > 0
+        for ws, n in ((None, 0), (p, need - 256), (ctypes.c_void_p(4100), need)):
+            assert cq.lib().cafeq_rtn(ctypes.byref(d), p, None, p, p, ws, ctypes.c_size_t(n), None) == 3
+    for group in (32, 64, 128, 256):
+        assert cq.rtn_workspace_size(cq.make_desc(8, 512, 4, group), False) == 0
