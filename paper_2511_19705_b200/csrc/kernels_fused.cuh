@@ -671,10 +671,27 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
 #pragma unroll
               for (int e = 0; e < 32; e += 2) m4[gi][(e >> 1) & 1] = max_abs2(m4[gi][(e >> 1) & 1], v[e], v[e + 1]);
             }
+            bool nan = false;
 #pragma unroll
             for (int gi = 0; gi < NG; ++gi) {
               best[gi] = max_abs2(m4[gi][0], m4[gi][1], 0.f);
               if (valid && !(best[gi] <= 3.0e38f)) bad = true;
+              nan = nan || best[gi] != best[gi];
+            }
+            // A group with a NaN keeps the maximum of its numbers (a non-finite weight spoils its own block only; the NaN itself
+            // is coded -qmax): one more walk, by the whole warp, where any lane has met one.
+            if (__any_sync(0xffffffffu, nan)) {
+#pragma unroll
+              for (int gi = 0; gi < NG; ++gi) {
+                best[gi] = 0.f;
+#pragma unroll 1
+                for (int ch = 0; ch < G / 16; ++ch) {
+                  float v[16];
+                  tc_ld16(taddr + gi * G + ch * 16, v);
+#pragma unroll
+                  for (int e = 0; e < 16; ++e) best[gi] = fmaxf(best[gi], fabsf(v[e]));
+                }
+              }
             }
           } else {
             // group absmax with arg-max: four independent running candidates per group (columns e mod 4), merged at the

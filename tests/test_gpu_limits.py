@@ -215,3 +215,33 @@ def test_weights_and_activations_at_any_address(cq, monkeypatch, k, shift):
     cfg = cq.make_cfg(steps=2, lr=1e-3)
     (h1, st1, _), (h2, st2, _) = (cq.cafeq_optimize_single(x, m, cfg, bits=4, group=128) for x, m in ((off, M1), (W, M2)))
     assert int(st1.item()) == 0 == int(st2.item()) and rel_err(h1[:, 0].cpu().numpy(), h2[:, 0].cpu().numpy()) <= 1e-5
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("k,group", [(64, 128), (64, 64), (128, 64), (256, 128)])
+def test_rounding_beside_a_non_finite_block(cq, k, group, bad):
+    """A non-finite weight spoils its block of its row.  A group that also covers another block takes its maximum over the values
+    that are numbers; the codes of those are the ones of that maximum, and what is not a number is coded -qmax."""
+    W = to_dev(syn.weight_student_t(130, 512, 3))
+    T = f32_dev(syn.perturbed_blocks(512 // k, k, 5, 0.1))
+    c0, s0 = cq.cafeq_rtn(W, T, bits=4, group=group, tblock=k)
+    U = cq.cafeq_apply_transform(W, T).float()
+    W[3, 70] = bad
+    c1, s1 = cq.cafeq_rtn(W, T, bits=4, group=group, tblock=k)
+    b, rows = 70 // k, [r for r in range(130) if r != 3]
+    assert torch.equal(c1[rows], c0[rows]) and torch.equal(s1[rows], s0[rows])
+    touched = {c // group for c in range(b * k, (b + 1) * k)}
+    for G in range(512 // group):
+        g = slice(G * group, (G + 1) * group)
+        if G not in touched:
+            assert torch.equal(c1[3, g], c0[3, g]) and s1[3, G] == s0[3, G]
+        elif bad != bad and group > k:  # half of the group is numbers
+            keep = torch.tensor([c for c in range(G * group, (G + 1) * group) if c // k != b], device="cuda")
+            lost = torch.tensor([c for c in range(G * group, (G + 1) * group) if c // k == b], device="cuda")
+            m = float(U[3, keep].abs().max())
+            assert abs(float(s1[3, G]) * 7 / m - 1) <= 2.0 ** -7
+            assert (c1[3, keep].abs().max() == 7) and (c1[3, lost] == -7).all()
+        elif bad != bad:  # nothing left: no maximum, codes 0
+            assert float(s1[3, G]) == 0.0 and not c1[3, g].any()
+        else:
+            assert not torch.isfinite(s1[3, G])
