@@ -85,8 +85,9 @@ def test_captured_step_of_a_small_layer(cq):
     assert int(a.status.item()) == 0 == int(b.status.item())
     for x, y, hx, hy, sx, sy in zip(a.M, b.M, a.hist, b.hist, a.state, b.state):
         assert float(sx[0]) == 12.0 == float(sy[0])
-        # (the order of atomic additions differs from run to run: 1e-5 of the change that twelve steps of 1e-4 make)
-        assert rel_err(x.cpu().numpy(), y.cpu().numpy()) <= 1e-5 and rel_err(hx[:, 0].cpu().numpy(), hy[:, 0].cpu().numpy()) <= 1e-5
+        # An entry whose gradient drowns in the order of the atomic additions moves by up to 1e-4 a step either way: at most 2.4e-3
+        # of entries of about 0.09 after twelve.  One in a thousand of them would make a difference of 0.027 * 1e-3 ** 0.5 = 8e-4.
+        assert rel_err(x.cpu().numpy(), y.cpu().numpy()) <= 1e-3 and rel_err(hx[:, 0].cpu().numpy(), hy[:, 0].cpu().numpy()) <= 1e-4
 
 
 @pytest.mark.parametrize("d_out,d_in,k,group", [(512, 128, 64, 64), (256, 256, 64, 16), (64, 128, 64, 128), (300, 192, 64, 64), (4096, 256, 64, 64)])
