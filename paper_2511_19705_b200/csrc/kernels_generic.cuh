@@ -237,6 +237,7 @@ __device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* s
   __shared__ int s_r;
   __shared__ int s_bad;
   const int tid = threadIdx.x, nt = blockDim.x;
+  const bool vec = k % 4 == 0 && ((uintptr_t)A & 15) == 0;
   if (tid == 0) s_bad = 0;
   __syncthreads();
   for (int p = 0; p < k; ++p) {
@@ -286,6 +287,34 @@ __device__ __noinline__ bool gauss_jordan(float* A, int k, float* sm, int32_t* s
     // column p after the exchange (factors); row p itself handled separately
     for (int i = tid; i < k; i += nt) fcol[i] = (i == p) ? 0.f : A[(size_t)i * k + p];
     __syncthreads();
+    if (vec) {
+      // four values per access and four accesses in flight per thread: one SM's loads from L2 are latency (a 256 x 256 block by
+      // 576 threads, one value at a time: 32 us a step, 13 us here)
+      float4* A4 = reinterpret_cast<float4*>(A);
+      const int k4 = k / 4, n4 = k * k4;
+      for (int e0 = tid; e0 < n4; e0 += 4 * nt) {
+        float4 c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (e0 + u * nt < n4) c[u] = A4[e0 + u * nt];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int e = e0 + u * nt;
+          if (e >= n4) break;
+          const int i = e / k4, j = (e - i * k4) * 4;
+          float x[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
+          const float f = -fcol[i];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float sp = (j + q == p) ? d : prow[j + q] * d;
+            x[q] = (i == p) ? sp : fmaf(f, sp, (j + q == p) ? 0.f : x[q]);
+          }
+          A4[e] = make_float4(x[0], x[1], x[2], x[3]);
+        }
+      }
+      __syncthreads();
+      continue;
+    }
     for (int e = tid; e < k * k; e += nt) {
       int i = e / k, j = e - i * k;
       float sp = (j == p) ? d : prow[j] * d;

@@ -246,3 +246,21 @@ def test_rounding_beside_a_non_finite_block(cq, k, group, bad):
             assert float(s1[3, G]) == 0.0 and not c1[3, g].any()
         else:
             assert not torch.isfinite(s1[3, G])
+
+
+@pytest.mark.parametrize("k,nb", [(128, 3), (256, 2), (256, 150), (48, 2), (100, 2), (50, 2), (512, 1)])
+def test_elimination_of_any_block(cq, k, nb):
+    """Blocks far from orthogonal: the iteration's fall-back inside its own kernel (128, 256) and the kernel of the other sizes, four
+    values at a time or (50) one."""
+    rng = np.random.default_rng(k)
+    M = rng.standard_normal((min(nb, 3), k, k)).astype(np.float32)
+    M = np.tile(orc.round_bf16(M).astype(np.float32), (-(-nb // len(M)), 1, 1))[:nb]
+    W = torch.zeros((32, nb * k), dtype=torch.bfloat16, device="cuda")
+    out = cq.cafeq_proxy_loss_fwd_bwd(W, f32_dev(M), bits=4, group=0, flags=cq.FLAG_NO_GRAD, want_minv=True)
+    assert int(out["status"].item()) == 0
+    X = out["Minv"].cpu().numpy().astype(np.float64)
+    for b in range(min(nb, 3)):
+        ref = np.linalg.inv(M[b].astype(np.float64))
+        # backward error of elimination: k 2^-24 times the condition number (growth under partial pivoting is small)
+        assert np.linalg.norm(X[b] - ref, 2) <= 4 * k * 2.0 ** -24 * np.linalg.cond(M[b].astype(np.float64)) * np.linalg.norm(ref, 2)
+        assert all(np.array_equal(X[c], X[b]) for c in range(b, nb, min(nb, 3)))
