@@ -903,8 +903,16 @@ extern "C" int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, 
   // the deployed operator is the bf16 rounding of the given one (what the tensor cores apply; the pass converts it
   // itself, the shape-agnostic kernels take the rounded fp32 copy)
   const int transposed = d->trole == CAFEQ_APPLY_TT;
-  if (G.axis == CAFEQ_AXIS_IN && G.d_out <= AS_MAX_ROWS && G.k % 32 == 0 && G.k <= 256 && ((uintptr_t)T & 15) == 0) {
-    CQ_LAUNCH(apply_small_kernel, dim3(G.nbq * (G.k / 32), (G.d_out + AS_ROWS - 1) / AS_ROWS), 256, 0, st, (const uint16_t*)X, G.ld, T,
+  const long long row_groups = (G.d_out + AS_ROWS - 1) / AS_ROWS, ctas = row_groups * G.nbq * (G.k / 32);
+  // Few rows: every group of eight reads the operators again, so the small kernel loses against one pass over them when groups and
+  // width multiply.  Its time follows CTAs x (k + 32): 250 000 is 13 us, what the call with the pass takes on the host (two kernels
+  // and a tensor map; the small kernel's 10).  Measured, small against pass, device time in us: k = 256, d_in = 8192, 24 rows
+  // 12.4 / 10.1, 64 rows 26.6 / 10.3; k = 128, 14336, 24 rows 11.6 / 9.3, 64 rows 25.8 / 9.5; k = 64, 14336, 48 rows 12.7 / 8.8,
+  // 64 rows 16.1 / 8.7; k = 32, 14336, 64 rows 12.2 / 8.1.  (On the device alone they meet at 108 000, 8 us.)  One group is faster at
+  // every width (k = 256, 14336: 10.4 / 11.9), and what the pass does not take has only slower kernels beside this one.
+  const bool few = row_groups == 1 || ctas * (G.k + 32) <= 250000 || !tc_apply_ok(G.k) || ((uintptr_t)X & 15) || G.ld % 8;
+  if (G.axis == CAFEQ_AXIS_IN && few && G.d_out <= AS_MAX_ROWS && G.k % 32 == 0 && G.k <= 256 && ((uintptr_t)T & 15) == 0) {
+    CQ_LAUNCH(apply_small_kernel, dim3(G.nbq * (G.k / 32), (unsigned)row_groups), 256, 0, st, (const uint16_t*)X, G.ld, T,
               reinterpret_cast<uint16_t*>(Y), G.d_out, G.d_in, G.k, G.r, transposed, status);
     return last_launch();
   }

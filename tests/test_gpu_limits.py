@@ -264,3 +264,18 @@ def test_elimination_of_any_block(cq, k, nb):
         # backward error of elimination: k 2^-24 times the condition number (growth under partial pivoting is small)
         assert np.linalg.norm(X[b] - ref, 2) <= 4 * k * 2.0 ** -24 * np.linalg.cond(M[b].astype(np.float64)) * np.linalg.norm(ref, 2)
         assert all(np.array_equal(X[c], X[b]) for c in range(b, nb, min(nb, 3)))
+
+
+@pytest.mark.parametrize("k,d_in", [(32, 14336), (64, 14336), (128, 8192), (256, 3584), (256, 8192), (96, 9600)])
+@pytest.mark.parametrize("rows", [8, 9, 24, 32, 64])
+def test_apply_few_rows_of_any_width(cq, k, d_in, rows):
+    """Both sides of the line between the kernel for few rows and the pass over the operators."""
+    g = torch.Generator(device="cuda").manual_seed(k + rows)
+    X = torch.randn((rows, d_in), device="cuda", generator=g).bfloat16()
+    T = torch.randn((d_in // k, k, k), device="cuda", generator=g) * k ** -0.5
+    Y = cq.cafeq_apply_transform(X, T).double()
+    Tc, Xb = T.bfloat16().double(), X.double().view(rows, d_in // k, k)
+    ref = torch.einsum("bij,obj->obi", Tc, Xb).reshape(rows, d_in)
+    mag = torch.einsum("bij,obj->obi", Tc.abs(), Xb.abs()).reshape(rows, d_in)
+    # half a bf16 step of the result plus the error of k fp32 additions (2^-24 each, on the sum of magnitudes)
+    assert ((Y - ref).abs() <= 2.0 ** -8 * ref.abs() + 2.0 ** -24 * k * mag).all()
