@@ -1359,8 +1359,8 @@ static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, cons
                          float* out, int32_t* status) {
   TgOperand oa[2], ob[2];
   oa[0] = oa[1] = TgOperand{A, (long long)nb * k, K, lda};
-  ob[0] = TgOperand{Bh, (long long)nb * k, K, K};
-  ob[1] = TgOperand{Bl, (long long)nb * k, K, K};
+  ob[0] = TgOperand{Bl, (long long)nb * k, K, K};
+  ob[1] = TgOperand{Bh, (long long)nb * k, K, K};
   TgParams p;
   memset(&p, 0, sizeof(p));
   p.M = p.N = k; p.K = K; p.batch = nb; p.nterms = 2;
@@ -1380,8 +1380,8 @@ static int opgrad_in_tc(cudaStream_t st, const uint16_t* Ah, const uint16_t* Al,
   for (int rep = 0; rep < r; ++rep) {
     TgOperand oa[2], ob[2];
     const long long cols = (long long)nb * r * k, c0 = (long long)rep * k;
-    oa[0] = TgOperand{Ah + c0, R, cols - c0, cols};
-    oa[1] = TgOperand{Al + c0, R, cols - c0, cols};
+    oa[0] = TgOperand{Al + c0, R, cols - c0, cols};
+    oa[1] = TgOperand{Ah + c0, R, cols - c0, cols};
     ob[0] = ob[1] = TgOperand{B + c0, R, cols - c0, ldb};
     TgParams p;
     memset(&p, 0, sizeof(p));
@@ -1598,16 +1598,16 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     // whose dependence on the group's arg-max entry is kept.
     DenseWS& w = p.dn;
     {  // g Vhat' [d3, h] = 2 R^T Uhat^T (one column for the replicas of an inner column)
-      const uint16_t* a[3] = {w.PTh, w.PTl, w.PTh};
-      const uint16_t* b[3] = {w.Awh, w.Awh, w.Awl};
+      const uint16_t* a[3] = {w.PTl, w.PTh, w.PTh};  // (small terms first, here and below: see launch_dense_tc6)
+      const uint16_t* b[3] = {w.Awh, w.Awl, w.Awh};
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
       launch_dense_tc(st, 3, a, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, status);
     }
     {  // g Uhat [h, d1] = 2 fold(Vhat^T) R^T (the folded splits are read as they are stored: an MN-major operand costs the
       // product 10 %, 14 us, where folding, transposing and splitting again took 60)
-      const uint16_t* a[3] = {w.Vh, w.Vl, w.Vh};
-      const uint16_t* b[3] = {w.Ph, w.Ph, w.Pl};
+      const uint16_t* a[3] = {w.Vl, w.Vh, w.Vh};
+      const uint16_t* b[3] = {w.Ph, w.Pl, w.Ph};
       DenseOut o;
       o.C = w.U; o.ldc = w.d1;
       launch_dense_tc(st, 3, a, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, status, 1);

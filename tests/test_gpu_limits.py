@@ -279,3 +279,18 @@ def test_apply_few_rows_of_any_width(cq, k, d_in, rows):
     mag = torch.einsum("bij,obj->obi", Tc.abs(), Xb.abs()).reshape(rows, d_in)
     # half a bf16 step of the result plus the error of k fp32 additions (2^-24 each, on the sum of magnitudes)
     assert ((Y - ref).abs() <= 2.0 ** -8 * ref.abs() + 2.0 ** -24 * k * mag).all()
+
+
+@pytest.mark.parametrize("k,r,h", [(32, 2, 128), (32, 4, 64), (96, 2, 192), (64, 2, 128), (128, 3, 128)])
+def test_replicas_with_any_block_size(cq, k, r, h):
+    """The replicas of a factor's blocks are summed before the product: its error is that of fp32 sums for every block size.  h / 16 <= 12
+    additions to an accumulator, 2^-24 of a sum that is half of its final size on average: 3.6e-7; the second terms of the sums, added
+    first, cost next to nothing."""
+    W1, W2 = to_dev(syn.weight_student_t(h, 192, 3)), to_dev(syn.weight_student_t(128, r * h, 4))
+    P = cq.cafeq_pair_product(W1, W2, k=k, replicas=r)
+    P64 = orc.pair_product(W1.double().cpu().numpy(), W2.double().cpu().numpy(), k, r)
+    assert rel_err(P.cpu().numpy(), P64) <= 3.6e-7
+    M = syn.perturbed_blocks(h // k, k, 5, 0.02)
+    out = cq.cafeq_pair_loss_fwd_bwd(W1, W2, f32_dev(M), bits=4, group1=64, group2=64, replicas=r, P=P, flags=cq.FLAG_EXACT_LOSS)
+    f = orc.pair_forward(W1.double().cpu().numpy(), W2.double().cpu().numpy(), M, 4, 64, 64, r, 5.0, 0.0, True)
+    assert abs(float(out["losses"][3]) / f["pqe"] ** 2 - 1) <= 1e-3
