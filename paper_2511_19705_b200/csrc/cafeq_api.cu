@@ -1102,18 +1102,19 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       p.min_ctas = 148;  // a long contraction: as many CTAs as the tile shapes give
       p.status = status;
       g_launches.fetch_add(1, std::memory_order_relaxed);
-      tg_launch(st, oa, ob, p);
+      if ((s.err = tg_launch(st, oa, ob, p))) return;
     }
     {  // N = Minv^T Minv (fp32 in s.Nf, splits in w.Qh / w.Ql)
       if (w.mn) {  // both operands are X read transposed from its row-major splits
         const uint16_t* a1[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
         const uint16_t* b1[3] = {w.Xh[c], w.Xh[c], w.Xl[c]};
-        launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status, 1, 1, 1);
+        s.err = launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status, 1, 1, 1);
       } else {
         const uint16_t* a1[3] = {w.XTh[c], w.XTl[c], w.XTh[c]};
         const uint16_t* b1[3] = {w.XTh[c], w.XTh[c], w.XTl[c]};
-        launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status);
+        s.err = launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status);
       }
+      if (s.err) return;
     }
     CQ_LAUNCH(dot_f32_kernel, grid_for(kk), 256, 0, st, s.Nf, s.tmp, kk, s.acc + 1);
     CQ_LAUNCH(sqsum_bf16_kernel, grid_for(G.n), 256, 0, st, (const uint16_t*)W, G.ld, G.d_out, G.d_in, s.acc + 2, status);
@@ -1122,8 +1123,8 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     {  // dL/dMinv = 2 Minv Gram (Gram is symmetric: its rows serve as the contraction-major second operand)
       const uint16_t* a2[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
       const uint16_t* b2[3] = {w.Ph, w.Ph, w.Pl};
-      launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr,
-                   status);
+      if ((s.err = launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr,
+                   status))) return;
     }
     {  // gDelta[o, B k + j] = 2 sum_l N_B[j][l] Delta[o, B k + l]  -> s.m.D (fp32 [d_out, d_in])
       TgOperand oa[3], ob[3];
@@ -1142,7 +1143,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       p.C = s.m.D; p.ldc = G.d_in; p.sCb = k;  // batch b writes the columns [b k, b k + k)
       p.status = status;
       g_launches.fetch_add(1, std::memory_order_relaxed);
-      tg_launch(st, oa, ob, p);
+      if ((s.err = tg_launch(st, oa, ob, p))) return;
     }
     const long long nrec = (long long)G.d_out * G.ng;
     CQ_LAUNCH(ste_scale_coef_kernel, (unsigned)((nrec * 32 + 255) / 256), 256, 0, st, s.m.D, (long long)G.d_in, s.m.Dbf, s.Dlo,
@@ -1568,13 +1569,13 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     launch_split(st, M, k, kk, w.Ph, w.Pl, w.Qh, w.Ql, status);
     const uint16_t* a1[3] = {w.Ph, w.Pl, w.Ph};
     const uint16_t* b1[3] = {w.Ph, w.Ph, w.Pl};
-    launch_kk_tc(st, 3, a1, b1, G1.nbT, k, 1.f, 0.f, -1.f, nullptr, nullptr, w.RTh, w.RTl, nullptr, nullptr, p.acc + 1,
-                 status, 0);
+    if ((p.err = launch_kk_tc(st, 3, a1, b1, G1.nbT, k, 1.f, 0.f, -1.f, nullptr, nullptr, w.RTh, w.RTl, nullptr, nullptr, p.acc + 1,
+                 status, 0))) return;
     if (gradM && lambda != 0.f) {
       const uint16_t* a2[3] = {w.RTh, w.RTl, w.RTh};
       const uint16_t* b2[3] = {w.Qh, w.Qh, w.Ql};
-      launch_kk_tc(st, 3, a2, b2, G1.nbT, k, 1.f, 0.f, 0.f, nullptr, p.RM, nullptr, nullptr, nullptr, nullptr, nullptr,
-                   status);
+      if ((p.err = launch_kk_tc(st, 3, a2, b2, G1.nbT, k, 1.f, 0.f, 0.f, nullptr, p.RM, nullptr, nullptr, nullptr, nullptr, nullptr,
+                   status))) return;
     }
   } else {
     launch_kk(st, M, 0, M, 1, p.tmp, G1.nbT, k, 1.f, GEMM_STORE, status);
@@ -1583,7 +1584,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
   }
   if (want_pqe && p.dense) {
     // Eq. 5 on the tensor cores: || Uhat_exp^T Vhat^T - P ||_F^2 with three-term bf16 splits of the dequantised values
-    dense_pqe(st, p.m1.E, p.m2.E, P, p.dn, p.acc + 2, nullptr, status, ste);
+    if ((p.err = dense_pqe(st, p.m1.E, p.m2.E, P, p.dn, p.acc + 2, nullptr, status, ste))) return;
   } else if (want_pqe) {
     launch_pair_product(st, p.m1.E, 0, G1.d_in, p.m2.E, 0, G2.d_in, G1, G2, p.R, status);
     CQ_LAUNCH(resid_sq_kernel, grid_for((long long)G1.d_in * G2.d_out), 256, 0, st, p.R, P, (long long)G1.d_in * G2.d_out, p.acc + 2,
@@ -1602,7 +1603,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       const uint16_t* b[3] = {w.Awh, w.Awl, w.Awh};
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
-      launch_dense_tc(st, 3, a, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, status);
+      if ((p.err = launch_dense_tc(st, 3, a, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, status))) return;
     }
     {  // g Uhat [h, d1] = 2 fold(Vhat^T) R^T (the folded splits are read as they are stored: an MN-major operand costs the
       // product 10 %, 14 us, where folding, transposing and splitting again took 60)
@@ -1610,7 +1611,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       const uint16_t* b[3] = {w.Ph, w.Pl, w.Ph};
       DenseOut o;
       o.C = w.U; o.ldc = w.d1;
-      launch_dense_tc(st, 3, a, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, status, 1);
+      if ((p.err = launch_dense_tc(st, 3, a, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, status, 1))) return;
     }
     if (!tc) {
       CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, gradM, 0.f, kk);
@@ -1725,7 +1726,7 @@ extern "C" int cafeq_pair_product(const cafeq_matrix_desc* d1, const void* W1, c
     if (carve_dense(b, G1.d_out, G1.d_in, G2.d_out, G2.r, G1.k, G1.ng, G2.ng, &w)) {
       CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G1.n), 256, 0, st, (const uint16_t*)W1, G1.ld, G1.d_out, G1.d_in, w.U);
       CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G2.n), 256, 0, st, (const uint16_t*)W2, G2.ld, G2.d_out, G2.d_in, w.V);
-      dense_product(st, w.U, w.V, w, P, nullptr);
+      if ((rc = dense_product(st, w.U, w.V, w, P, nullptr))) return rc;
       return last_launch();
     }
   }
@@ -1880,7 +1881,7 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
     CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G1.n), 256, 0, st, (const uint16_t*)W1, G1.ld, G1.d_out, G1.d_in, w.U);
     CQ_LAUNCH(bf16_to_f32_kernel, grid_for(G2.n), 256, 0, st, (const uint16_t*)W2, G2.ld, G2.d_out, G2.d_in, w.V);
   }
-  alg1_run(st, d1->bits, G1.g, G2.g, iters, codes1, scales1, codes2, scales2, pqe_history, w, status);
+  if ((rc = alg1_run(st, d1->bits, G1.g, G2.g, iters, codes1, scales1, codes2, scales2, pqe_history, w, status))) return rc;
   return last_launch();
 }
 

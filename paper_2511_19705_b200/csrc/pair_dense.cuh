@@ -71,7 +71,6 @@ static int launch_dense_tc6(cudaStream_t st, const uint16_t* const* A, const uin
   const uint16_t* b2[3] = {B[2], B[0], B[1]};
   DenseOut o2 = o;
   o2.C0 = acc; o2.ldc0 = N;
-  if (!o2.C) { o2.C = nullptr; }
   return launch_dense_tc(st, 3, a2, b2, M, N, K, alpha, 1.f, 0.f, o2, status);
 }
 
@@ -144,7 +143,7 @@ static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, 
 // and the rounding that this leaves outside the row space of A is never corrected: codes that matched the float64
 // pseudo-inverse differed.  Reading Y and C row-major as MN-major operands, with no transposed outputs: 114 us for
 // 2048 x 3584 x 2048 against 102.)
-static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, int32_t* status) {
+static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, int32_t* status) {
   const bool wide = R <= C;
   const int m = wide ? R : C, n = wide ? C : R;
   double* fro = w.sq + 120;
@@ -172,7 +171,7 @@ static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w,
     launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Awh, w.Awl, status, nullptr, w.Aw3);
     launch_split_rect(st, S, R, C, C, 1.f, sig2, nullptr, w.Y, w.YTh[0], w.YTl[0], w.Yh, w.Yl, status);
   }
-  int cur = 0;
+  int cur = 0, rc;
   for (int it = 0; it < PINV_MAX_ITERS; ++it) {
     {  // C = I - A X, kept transposed
       const uint16_t* a[3] = {w.Awh, w.Awl, w.Awh};
@@ -180,7 +179,7 @@ static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w,
       DenseOut o;
       o.Cthi = w.CTh; o.Ctlo = w.CTl; o.sq = rs + it;
       o.stop_sq = rs; o.stop_it = it;
-      launch_dense_tc(st, 3, a, bb, m, m, n, -1.f, 0.f, 1.f, o, status);
+      if ((rc = launch_dense_tc(st, 3, a, bb, m, m, n, -1.f, 0.f, 1.f, o, status))) return rc;
     }
     {  // Y += C^T Y
       const uint16_t* a[3] = {w.CTh, w.CTl, w.CTh};
@@ -189,7 +188,7 @@ static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w,
       o.C0 = w.Y; o.ldc0 = n; o.C = w.Y; o.ldc = n;
       o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[cur ^ 1]; o.Ctlo = w.YTl[cur ^ 1];
       o.stop_sq = rs; o.stop_it = it;
-      launch_dense_tc(st, 3, a, bb, m, n, m, 1.f, 1.f, 0.f, o, status);
+      if ((rc = launch_dense_tc(st, 3, a, bb, m, n, m, 1.f, 1.f, 0.f, o, status))) return rc;
     }
     cur ^= 1;
   }
@@ -203,15 +202,16 @@ static void pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w,
     const uint16_t* bb[3] = {w.Yh, w.Yl, w.Y3};
     DenseOut o;
     o.Cthi = w.CTh; o.Ctlo = w.CTl;
-    launch_dense_tc6(st, a, bb, m, m, n, -1.f, 0.f, 1.f, o, w.Cf, status);
+    if ((rc = launch_dense_tc6(st, a, bb, m, m, n, -1.f, 0.f, 1.f, o, w.Cf, status))) return rc;
     const uint16_t* a2[3] = {w.CTh, w.CTl, w.CTh};
     const uint16_t* b2[3] = {w.YTh[0], w.YTh[0], w.YTl[0]};
     DenseOut o2;
     o2.C0 = w.Y; o2.ldc0 = n; o2.C = w.Y; o2.ldc = n;
-    launch_dense_tc(st, 3, a2, b2, m, n, m, 1.f, 1.f, 0.f, o2, status);
+    if ((rc = launch_dense_tc(st, 3, a2, b2, m, n, m, 1.f, 1.f, 0.f, o2, status))) return rc;
   }
   if (wide) launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, w.Oh, w.Ol, nullptr, nullptr, status, w.O3, nullptr);
   else launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Oh, w.Ol, status, nullptr, w.O3);
+  return CAFEQ_OK;
 }
 
 }  // namespace cafeq
@@ -233,20 +233,22 @@ static void launch_fold_split(cudaStream_t st, const float* V, DenseWS& w, uint1
 // P = U_exp^T V^T for stored U [h, d1], V [d3, rh] (fp32): fp32 P [d1, d3] with its splits in w.Ph/Pl/PTh/PTl
 // (six terms over three-way splits: P is the reference every least-squares target of Algorithm 1 is measured
 // against, so it is formed to fp32 accuracy; its own third-term splits follow for the target products)
-static void dense_product(cudaStream_t st, const float* U, const float* V, DenseWS& w, float* P, int32_t* status) {
+static int dense_product(cudaStream_t st, const float* U, const float* V, DenseWS& w, float* P, int32_t* status) {
   launch_split_rect(st, U, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.UTh, w.UTl, status, nullptr, w.UT3);
   launch_fold_split(st, V, w, w.Vh, w.Vl, w.V3, status);
   const uint16_t* a[3] = {w.UTh, w.UTl, w.UT3};
   const uint16_t* b[3] = {w.Vh, w.Vl, w.V3};
   DenseOut o;
   o.C = P; o.ldc = w.d3; o.Chi = w.Ph; o.Clo = w.Pl; o.Cthi = w.PTh; o.Ctlo = w.PTl;
-  launch_dense_tc6(st, a, b, w.d1, w.d3, w.h, 1.f, 0.f, 0.f, o, P, status);
+  const int rc = launch_dense_tc6(st, a, b, w.d1, w.d3, w.h, 1.f, 0.f, 0.f, o, P, status);
+  if (rc) return rc;
   launch_split_rect(st, P, w.d1, w.d3, w.d3, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status, w.P3, w.PT3);
+  return CAFEQ_OK;
 }
 
 // *sq += || Uhat_exp^T Vhat^T - P ||_F^2 ; optionally stores the residual R [d1, d3].  keep_splits: leaves the residual and its
 // transpose in w.Ph / Pl / PTh / PTl and Uhat, as stored, in w.Awh / Awl (Vhat, replicas folded, is in w.Vh / Vl either way)
-static void dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, const float* P, DenseWS& w, double* sq, float* R,
+static int dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, const float* P, DenseWS& w, double* sq, float* R,
                       int32_t* status, bool keep_splits = false) {
   launch_split_rect(st, Uhat, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, keep_splits ? w.Awh : nullptr,
                     keep_splits ? w.Awl : nullptr, w.UTh, w.UTl, status);
@@ -258,50 +260,52 @@ static void dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, con
   if (keep_splits) {  // the residual and its transpose as operands of the backward products
     o.Chi = w.Ph; o.Clo = w.Pl; o.Cthi = w.PTh; o.Ctlo = w.PTl;
   }
-  launch_dense_tc(st, 3, a, b, w.d1, w.d3, w.h, 1.f, -1.f, 0.f, o, status);
+  return launch_dense_tc(st, 3, a, b, w.d1, w.d3, w.h, 1.f, -1.f, 0.f, o, status);
 }
 
 // Algorithm 1 on the transformed pair held in w.U [h, d1], w.V [d3, rh] (fp32, stored layout with r replicas of
 // every inner block on the V side).  With E the replica expansion, the V update is Q((pinv((E Uhat)^T) P)^T) =
 // Q(expand(pinv(Uhat^T) P) / r) (Uhat^T of full column rank) and the U update is Q((P pinv(fold(Vhat^T)))^T),
 // which is the printed algorithm when r = 1.  pqe_hist: fp32 [2 iters + 1].
-static void alg1_run(cudaStream_t st, int bits, int g1, int g2, int iters, int8_t* codes1, float* scales1, int8_t* codes2,
+static int alg1_run(cudaStream_t st, int bits, int g1, int g2, int iters, int8_t* codes1, float* scales1, int8_t* codes2,
                      float* scales2, float* pqe_hist, DenseWS& w, int32_t* status) {
+  int rc;
   CQ_LAUNCH(zero_f64_kernel, 1, 128, 0, st, w.sq, DENSE_SQ);
-  dense_product(st, w.U, w.V, w, w.P, status);
+  if ((rc = dense_product(st, w.U, w.V, w, w.P, status))) return rc;
   quant_matrix(st, w.U, w.h, w.d1, g1, bits, codes1, scales1, w.Uhat, w, status);
   quant_matrix(st, w.V, w.d3, w.rh, g2, bits, codes2, scales2, w.Vhat, w, status);
-  dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 0, nullptr, status);
+  if ((rc = dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 0, nullptr, status))) return rc;
   for (int it = 0; it < iters; ++it) {
     // V side: X0^T [d3, h] = P^T pinv(Uhat^T)^T, then expand the replicas
-    pinv_rows(st, w.Uhat, w.h, w.d1, w, status);
+    if ((rc = pinv_rows(st, w.Uhat, w.h, w.d1, w, status))) return rc;
     {
       const uint16_t* a[3] = {w.PTh, w.PTl, w.PT3};
       const uint16_t* b[3] = {w.Oh, w.Ol, w.O3};
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
-      launch_dense_tc6(st, a, b, w.d3, w.h, w.d1, 1.f, 0.f, 0.f, o, w.X0T, status);
+      if ((rc = launch_dense_tc6(st, a, b, w.d3, w.h, w.d1, 1.f, 0.f, 0.f, o, w.X0T, status))) return rc;
     }
     CQ_LAUNCH(expand_cols_kernel, dim3(w.d3, (w.h + 1023) / 1024), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f / (float)w.r, w.V);
     quant_matrix(st, w.V, w.d3, w.rh, g2, bits, codes2, scales2, w.Vhat, w, status);
-    dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 1, nullptr, status);
+    if ((rc = dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 1, nullptr, status))) return rc;
     // U side: U' [h, d1] = pinv(Bf)^T P^T with Bf = fold(Vhat^T) [h, d3]
     {
       dim3 grid((w.d3 + 31) / 32, w.h / 32);
       CQ_LAUNCH(fold_transpose_kernel, grid, dim3(32, 8), 0, st, w.Vhat, w.d3, w.h, w.k, w.r, w.Bf);
     }
-    pinv_rows(st, w.Bf, w.h, w.d3, w, status);
+    if ((rc = pinv_rows(st, w.Bf, w.h, w.d3, w, status))) return rc;
     {
       const uint16_t* a[3] = {w.Oh, w.Ol, w.O3};
       const uint16_t* b[3] = {w.Ph, w.Pl, w.P3};
       DenseOut o;
       o.C = w.U; o.ldc = w.d1;
-      launch_dense_tc6(st, a, b, w.h, w.d1, w.d3, 1.f, 0.f, 0.f, o, w.U, status);
+      if ((rc = launch_dense_tc6(st, a, b, w.h, w.d1, w.d3, 1.f, 0.f, 0.f, o, w.U, status))) return rc;
     }
     quant_matrix(st, w.U, w.h, w.d1, g1, bits, codes1, scales1, w.Uhat, w, status);
-    dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 2, nullptr, status);
+    if ((rc = dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 2, nullptr, status))) return rc;
   }
   CQ_LAUNCH(sqrt_hist_kernel, 1, 128, 0, st, w.sq, pqe_hist, 2 * iters + 1);
+  return CAFEQ_OK;
 }
 
 }  // namespace cafeq

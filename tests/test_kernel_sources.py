@@ -70,3 +70,15 @@ def test_inputs_are_read_with_ordinary_loads(path):
     text = _strip(open(path).read())
     assert not re.search(r"__ldg\b|ld\.global\.nc", text)
     assert not re.search(r"\bconst\s+\w+\s*\*\s*__restrict__", text)
+
+
+RETURNING = (r"launch_dense_tc6?|launch_kk_tc|tg_launch|tb_launch|bd_launch\w*|bw_launch\w*|ns_block_launch|kk_chain_launch|ns_inverse|"
+             r"minv_path_tc|penalty_tc|opgrad_\w+_tc|pinv_rows|dense_product|dense_pqe|alg1_run")
+
+
+@pytest.mark.parametrize("path", sorted(glob.glob(os.path.join(CSRC, "*.cu*"))), ids=os.path.basename)
+def test_no_launch_result_is_dropped(path):
+    """A launch that could not be made (an operand that a tensor map does not take) must end the call, not leave stale results."""
+    dropped = re.findall(r"[;{})]\s*((?:%s)\s*\([^;{}]*;)" % RETURNING, _strip(open(path).read()))
+    assert not dropped, dropped
+    assert not re.search(r"static void (%s)\(" % RETURNING, _strip(open(path).read()))
