@@ -226,18 +226,16 @@ static void launch_inverse(cudaStream_t st, const float* Mc, float* Minv, float*
 // k x k algebra on the tensor cores: split-precision products and the Newton-Schulz inverse
 // ------------------------------------------------------------------------------------------------
 struct KkWS {  // bf16 scratch, each [nbT * k * k]
-  uint16_t *Ab, *Xh[2], *Xl[2], *XTh[2], *XTl[2], *RTh, *RTl, *Ph, *Pl, *Qh, *Ql;
-  double* rn;  // [NS_MAX_ITERS][nbT] squared residual norms
-  int* flag;   // 1 => Newton-Schulz did not converge, the Gauss-Jordan kernel takes over
-  int* redo_total;  // optional running count of blocks recomputed by elimination (never cleared by a step)
-  int cur;     // which of the ping-pong split sets holds the current inverse (host bookkeeping)
-  bool mn;     // the inverse was refined on row-major arrays only (whole-block products with MN-major operands): the
-               // transposed splits XTh / XTl are not maintained
+  uint16_t *Ab;              // bf16(M)
+  uint16_t *Xh, *Xl;         // splits of the inverse, and transposed:
+  uint16_t *XTh, *XTl;       // (blocks of 32 and 64 only)
+  uint16_t *RTh, *RTl, *Ph, *Pl, *Qh, *Ql;
+  int* redo_total;           // optional running count of blocks recomputed by elimination (never cleared by a step)
+  bool mn;                   // the inverse was refined on row-major arrays only (blocks of 128 and 256): XTh / XTl are not maintained
 };
-constexpr int NS_MAX_ITERS = 8;
 // Fused kernel (ns_block_kernel): rounds at most, and the squared residual before an update that makes it the last one.
 // Warm: below 1e-2 before, hence below 1e-4 after it (the acceptance test of the elimination fall-back).  Cold starts are
-// paid once per run: they go on to 1e-3 (1e-6 after the update, the accuracy the products themselves carry).
+// paid once per run: they go on to 1e-3 (1e-6 after the update, and up to 4e-6 from the update's single term).
 constexpr int NS_WARM_ROUNDS = 6, NS_COLD_ROUNDS = 10;
 constexpr double NS_GATE2 = 1e-4, NS_COLD_GATE2 = 1e-6;
 
@@ -248,16 +246,13 @@ static void launch_operator_bf16(cudaStream_t st, const float* T, uint16_t* out,
 
 static bool kk_fast(int k) { return k == 64 || k == 128 || k == 256; }
 
-static void carve_kk(Bump& b, int nbT, int k, KkWS* w) {
+// layer: what the layer step uses of it
+static void carve_kk(Bump& b, int nbT, int k, KkWS* w, bool layer = false) {
   const size_t kk = (size_t)nbT * k * k;
-  uint16_t** all[] = {&w->Ab, &w->Xh[0], &w->Xh[1], &w->Xl[0], &w->Xl[1], &w->XTh[0], &w->XTh[1], &w->XTl[0], &w->XTl[1],
-                      &w->RTh, &w->RTl, &w->Ph, &w->Pl, &w->Qh, &w->Ql};
-  for (auto pp : all) *pp = b.take<uint16_t>(kk);
-  w->rn = b.take<double>((size_t)NS_MAX_ITERS * nbT);
-  w->flag = b.take<int>(64);
-  w->redo_total = nullptr;
-  w->cur = 0;
-  w->mn = false;
+  memset(w, 0, sizeof(*w));
+  for (uint16_t** p : {&w->Ab, &w->Xh, &w->Xl, &w->Pl}) *p = b.take<uint16_t>(kk);
+  if (layer) return;
+  for (uint16_t** p : {&w->XTh, &w->XTl, &w->RTh, &w->RTl, &w->Ph, &w->Qh, &w->Ql}) *p = b.take<uint16_t>(kk);
 }
 
 // C[b] = alpha * sum_t A_t[b] B_t[b]^T + beta * C0[b] + gamma * I for nb blocks of k x k; operands bf16 [nb*k, k]
@@ -291,13 +286,6 @@ static int launch_kk_tc(cudaStream_t st, int nterms, const uint16_t* const* A, c
   return tg_launch(st, oa, ob, p);
 }
 
-__global__ void zero_ns_kernel(double* rn, int n, int* flag) {
-  pdl_enter();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) rn[i] = 0.0;
-  if (i == 0) *flag = 0;
-}
-
 static void launch_split(cudaStream_t st, const float* X, int k, long long n, uint16_t* hi, uint16_t* lo, uint16_t* thi,
                          uint16_t* tlo, const int32_t* status) {
   dim3 grid(k / 32, k / 32, (unsigned)(n / ((long long)k * k)));
@@ -309,24 +297,20 @@ static void launch_split(cudaStream_t st, const float* X, int k, long long n, ui
 // previous inverse (warm); a warm start runs as many rounds as the step size calls for (a block whose residual ||I - A X||_F
 // was below 1e-2 before an update, 1e-4 after it, stops); a residual that does not become small falls back to elimination.
 // k = 32, 64: elimination, which takes less than one round's launches there.  Leaves fp32 Minv in X and its bf16 splits in
-// w.Xh / Xl (and XTh / XTl unless w.mn) [w.cur].
+// w.Xh / Xl (and XTh / XTl unless w.mn).
 // eq4 (k = 128, 256): where the kernel puts the column norms / group weights, and what it ticks.
 static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k, bool warm, KkWS& w, int32_t* status,
                       bool prepped = false, bool splits_kept = false, const NsParams* eq4 = nullptr, bool overlap = true) {
-  w.cur = 0;
   w.mn = tb_supported(k, 2);
   if (!w.mn) {
-    launch_inverse(st, Mc, X, nullptr, nb, k, status, w.Xh[0], w.Xl[0], w.XTh[0], w.XTl[0]);
+    launch_inverse(st, Mc, X, nullptr, nb, k, status, w.Xh, w.Xl, w.XTh, w.XTl);
     return CAFEQ_OK;
   }
   int ti = kt_begin(3, st);
-  if (!prepped) {  // otherwise step_prep_kernel has cleared rn / flag and written Ab
-    CQ_LAUNCH(zero_ns_kernel, (NS_MAX_ITERS * nb + 127) / 128, 128, 0, st, w.rn, NS_MAX_ITERS * nb, w.flag);
-    launch_operator_bf16(st, Mc, w.Ab, k, nb, 0, status);
-  }
-  // (splits_kept: the splits of X that the previous call left in set 0 are still there)
-  if (!warm) CQ_LAUNCH(ns_cold_start_kernel, dim3(k / 32, k / 32, nb), dim3(32, 8), 0, st, w.Ab, k, w.Xh[0], w.Xl[0], status);
-  else if (!splits_kept) launch_split(st, X, k, (long long)nb * k * k, w.Xh[0], w.Xl[0], nullptr, nullptr, status);
+  if (!prepped) launch_operator_bf16(st, Mc, w.Ab, k, nb, 0, status);  // (otherwise the step's set-up has written it)
+  // (splits_kept: the splits of X that the previous call left are still there)
+  if (!warm) CQ_LAUNCH(ns_cold_start_kernel, dim3(k / 32, k / 32, nb), dim3(32, 8), 0, st, w.Ab, k, w.Xh, w.Xl, status);
+  else if (!splits_kept) launch_split(st, X, k, (long long)nb * k * k, w.Xh, w.Xl, nullptr, nullptr, status);
   NsParams np;
   memset(&np, 0, sizeof(np));
   if (eq4) np = *eq4;
@@ -336,12 +320,12 @@ static int ns_inverse(cudaStream_t st, const float* Mc, float* X, int nb, int k,
   np.redo_count = w.redo_total;
   np.status = status;
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  const int rc = ns_block_launch(st, w.Ab, w.Xh[0], w.Xl[0], X, nb, k, np, overlap);
+  const int rc = ns_block_launch(st, w.Ab, w.Xh, w.Xl, X, nb, k, np, overlap);
   kt_end(ti, st);
   return rc;
 }
 
-// G -= X^T Gx X^T for every block; X = Minv.  k = 128, 256: on the tensor cores from its splits in w[w.cur], three-term
+// G -= X^T Gx X^T for every block; X = Minv.  k = 128, 256: on the tensor cores from its splits in w, three-term
 // products; 32, 64: in fp32.  Gx = dL/dMinv: fp32 [nb, k, k], or (scaled) formed from X by the kernel itself.
 static int minv_path_tc(cudaStream_t st, const float* X, const float* Gx, float* G, int nb, int k, KkWS& w, int32_t* status,
                         const ChainParams* scaled = nullptr, bool overlap = true) {
@@ -352,7 +336,7 @@ static int minv_path_tc(cudaStream_t st, const float* X, const float* Gx, float*
     cp.G = Gx;
     cp.status = status;
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return kk_chain_launch(st, KK_MINV_PATH, w.Xh[w.cur], w.Xl[w.cur], G, nb, k, cp, overlap);
+    return kk_chain_launch(st, KK_MINV_PATH, w.Xh, w.Xl, G, nb, k, cp, overlap);
   }
   if (k == 32) CQ_LAUNCH(small_chain_kernel<32>, nb, 64, 0, st, X, Gx, cp.A[0], cp.Agrp[0], cp.g[0], cp.scale[0], G, status);
   else CQ_LAUNCH(small_chain_kernel<64>, nb, 256, 0, st, X, Gx, cp.A[0], cp.Agrp[0], cp.g[0], cp.scale[0], G, status);
@@ -1026,9 +1010,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     pa.zero_f[1] = s.m.agrp; pa.zero_fn[1] = G.ng;
     if (in_r1) { pa.zero_f[2] = s.m.cw; pa.zero_fn[2] = G.ng; }
     if (want_grad) { pa.zero_f[3] = gradM; pa.zero_fn[3] = kk; }
-    pa.zero_d[0] = s.acc; pa.zero_dn[0] = 8;
-    pa.zero_d[1] = s.kk.rn; pa.zero_dn[1] = NS_MAX_ITERS * G.nbT;
-    pa.flag = s.kk.flag;
+    pa.zero_d = s.acc; pa.zero_dn = 8;
     pa.step_counter = step_counter;
     pa.status = status;
     CQ_LAUNCH(step_prep_kernel, grid_for(kk), 256, 0, st, pa);
@@ -1081,7 +1063,6 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     // apply), and the scale path needs sum_e gDelta_e Delta_e per group.  Every product runs on the tensor cores
     // with the residual as a two-term bf16 split (three-term products: fp32-grade).
     KkWS& w = s.kk;
-    const int c = w.cur;
     {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the d_out rows of the residual as it is stored
       TgOperand oa[3], ob[3];
       const uint16_t* at[3] = {s.m.Dbf, s.Dlo, s.m.Dbf};
@@ -1106,12 +1087,12 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     }
     {  // N = Minv^T Minv (fp32 in s.Nf, splits in w.Qh / w.Ql)
       if (w.mn) {  // both operands are X read transposed from its row-major splits
-        const uint16_t* a1[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
-        const uint16_t* b1[3] = {w.Xh[c], w.Xh[c], w.Xl[c]};
+        const uint16_t* a1[3] = {w.Xh, w.Xl, w.Xh};
+        const uint16_t* b1[3] = {w.Xh, w.Xh, w.Xl};
         s.err = launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status, 1, 1, 1);
       } else {
-        const uint16_t* a1[3] = {w.XTh[c], w.XTl[c], w.XTh[c]};
-        const uint16_t* b1[3] = {w.XTh[c], w.XTh[c], w.XTl[c]};
+        const uint16_t* a1[3] = {w.XTh, w.XTl, w.XTh};
+        const uint16_t* b1[3] = {w.XTh, w.XTh, w.XTl};
         s.err = launch_kk_tc(st, 3, a1, b1, G.nbT, k, 1.f, 0.f, 0.f, nullptr, s.Nf, w.Qh, w.Ql, nullptr, nullptr, nullptr, status);
       }
       if (s.err) return;
@@ -1121,7 +1102,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     CQ_LAUNCH(finalize_single_kernel, 1, 1, 0, st, s.acc, losses, hist, 1);
     if (!want_grad) return;
     {  // dL/dMinv = 2 Minv Gram (Gram is symmetric: its rows serve as the contraction-major second operand)
-      const uint16_t* a2[3] = {w.Xh[c], w.Xl[c], w.Xh[c]};
+      const uint16_t* a2[3] = {w.Xh, w.Xl, w.Xh};
       const uint16_t* b2[3] = {w.Ph, w.Ph, w.Pl};
       if ((s.err = launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr,
                    status))) return;
@@ -1521,9 +1502,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
       pa.zero_f[1] = gradM; pa.zero_fn[1] = kk;
       pa.zero_f[2] = p.gMinv; pa.zero_fn[2] = kk;
     }
-    pa.zero_d[0] = p.acc; pa.zero_dn[0] = 8;
-    pa.zero_d[1] = p.kk.rn; pa.zero_dn[1] = NS_MAX_ITERS * G1.nbT;
-    pa.flag = p.kk.flag;
+    pa.zero_d = p.acc; pa.zero_dn = 8;
     pa.step_counter = step_counter;
     pa.status = status;
     CQ_LAUNCH(step_prep_kernel, grid_for(kk), 256, 0, st, pa);
@@ -1540,7 +1519,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
   const bool f1 = forward_quant(st, W1, G1, d1->bits, p.Mc, 1, p.m1, nullptr, CAFEQ_OFFSETS_NONE, false, want_pqe ? p.m1.E : nullptr, nullptr,
                 nullptr, status, !force_generic);
   const bool f2 = forward_quant(st, W2, G2, d2->bits, p.Minv_c, 0, p.m2, nullptr, CAFEQ_OFFSETS_NONE, false, want_pqe ? p.m2.E : nullptr,
-                nullptr, nullptr, status, !force_generic, nullptr, tc ? p.kk.Xh[p.kk.cur] : nullptr);  // Xh = bf16(Minv)
+                nullptr, nullptr, status, !force_generic, nullptr, tc ? p.kk.Xh : nullptr);  // Xh = bf16(Minv)
   const long long n1 = (long long)G1.d_out * G1.ng, n2 = (long long)G2.d_out * G2.ng;
   CQ_LAUNCH(max2_f32_kernel, grid_for(n1 + n2), 256, 0, st, p.m1.a, n1, p.m2.a, n2, p.amax, status);
   CQ_LAUNCH(sumexp2_kernel, grid_for(n1 + n2), 256, 0, st, p.m1.a, n1, p.m2.a, n2, p.amax, t, p.acc + 0, status);
@@ -1871,7 +1850,7 @@ extern "C" int cafeq_adaptive_round(const cafeq_matrix_desc* d1, const void* W1,
     } else launch_inverse(st, Mc, Minv, nullptr, G1.nbT, G1.k, status);
     CQ_LAUNCH(round_bf16_kernel, grid_for(kk), 256, 0, st, Minv, Minv_c, kk, status);
     // both products on the tensor cores where the shape allows (bf16 operands, fp32 accumulation either way); the operators in
-    // applied orientation and the transposed first factor use scratch that the rounding fills later
+    // applied orientation use scratch that nothing else needs here
     uint16_t *T1 = kkw.Ph, *T2 = kkw.Qh;
     launch_operator_bf16(st, Mc, T1, G1.k, G1.nbT, 1, status);
     launch_operator_bf16(st, Minv_c, T2, G1.k, G1.nbT, 0, status);

@@ -38,7 +38,6 @@ struct BdParams {
   int pairs;           // input axis, K = 64: blocks of 32, two on the diagonal of each operator block
   int n_major;         // IN: tile columns (256 d_in columns each); OUT: row blocks (k rows each)
   int n_minor;         // IN: row tiles of 128; OUT: column tiles of NC
-  int ctas_per_major;
   int epi;
   float qmax;
   // per (row, group) records are stored GROUP-MAJOR: index = group * d_out + row
@@ -1020,7 +1019,6 @@ static void bd_fill_tiles(BdParams& p) {
     p.n_major = p.d_out / K;
     p.n_minor = (p.d_in + C::NC - 1) / C::NC;
   }
-  p.ctas_per_major = 0;
 }
 
 template <int FORM, int K, int G, int MODE>

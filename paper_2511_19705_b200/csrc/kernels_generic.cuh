@@ -1089,9 +1089,8 @@ struct PrepArgs {
   long long kk;
   float* zero_f[4];      // fp32 arrays to clear
   long long zero_fn[4];
-  double* zero_d[2];     // double arrays to clear
-  int zero_dn[2];
-  int* flag;             // cleared
+  double* zero_d;        // double array to clear
+  int zero_dn;
   float* step_counter;   // += 1 (optimiser state), may be null
   const int32_t* status;
 };
@@ -1109,14 +1108,9 @@ __global__ void step_prep_kernel(PrepArgs a) {
   for (int q = 0; q < 4; ++q)
     if (a.zero_f[q])
       for (long long e = t0; e < a.zero_fn[q]; e += stride) a.zero_f[q][e] = 0.f;
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-    if (a.zero_d[q])
-      for (long long e = t0; e < a.zero_dn[q]; e += stride) a.zero_d[q][e] = 0.0;
-  if (t0 == 0) {
-    if (a.flag) *a.flag = 0;
-    if (a.step_counter) *a.step_counter += 1.f;
-  }
+  if (a.zero_d)
+    for (long long e = t0; e < a.zero_dn; e += stride) a.zero_d[e] = 0.0;
+  if (t0 == 0 && a.step_counter) *a.step_counter += 1.f;
 }
 
 // c[b][t] = sum_i X[b][i][t]^2 for 32 columns t per CTA (grid: k/32, nb; block 32 x 8), and optionally the

@@ -404,7 +404,7 @@ static int ly_plan(const cafeq_layer_problem* probs, int n, void* ws, size_t ws_
   L->grad = b.take<float>(kk);
   L->RM = b.take<float>(kkP ? kkP : 1);
   L->c = b.take<float>((size_t)NB * L->k);
-  carve_kk(b, NB, L->k, &L->kk);
+  carve_kk(b, NB, L->k, &L->kk, true);
   L->one = b.take<float>(64);
   L->kk.redo_total = reinterpret_cast<int*>(L->one ? L->one + 8 : nullptr);
   for (int i = 0; i < nm; ++i) {
@@ -493,9 +493,6 @@ static LyAux* ly_aux() {
   }
   return &slots[dev];
 }
-// block sizes whose inverse refinement runs on row-major arrays (the transposed split arrays are then free)
-static bool w_mn_expected(int k) { return tb_supported(k, 2); }
-
 static void ly_lists(const LyPlan& L, int axis, int transpose, int* out, int* cnt) {
   // matrices whose backward shares (axis, output orientation): singles store gradT plainly, a pair's first factor
   // (operator M^T) stores it transposed, its second factor feeds dL/dMinv plainly
@@ -519,7 +516,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
   for (int q = 0; q < L.n; ++q) any_lambda |= (L.p[q].pair && L.p[q].cfg.lambda_orth != 0.f);
   // The pair blocks' penalty (R = M M^T - I, its norm, R M) does not depend on the inverse: it runs on a side stream beside it
   // (one CTA per block leaves SMs idle).  Only the parameter update reads its results: it joins there, or on any earlier way out.
-  LyAux* aux = (nbP > 0 && g_ly_dual.load(std::memory_order_relaxed) && w_mn_expected(k)) ? ly_aux() : nullptr;
+  LyAux* aux = (nbP > 0 && g_ly_dual.load(std::memory_order_relaxed)) ? ly_aux() : nullptr;
   // Inverse and penalty take one CTA per block.  Where they do not fit side by side, a programmatic launch hurts: CTAs that
   // wait for the kernel before them take SMs from the penalty, and the pass then starts late on those (9B-shaped, 106 + 64
   // blocks: 372 us a step with ordinary launches, 392 with programmatic ones; 2B-shaped, all resident: 122 and 117).
@@ -592,7 +589,7 @@ static int ly_step(cudaStream_t st, LyPlan& L, int hist_row, bool last, int32_t*
         p.Aacc = (Mt.G.axis == CAFEQ_AXIS_IN) ? Mt.agrp : Mt.A;
       } else {
         // U = W1 M: the operator is bf16(M)^T, read transposed; V = M^-1 W2: bf16(M^-1)
-        s.Tb = (Mt.side == 0) ? w.Ab + off : w.Xh[w.cur] + off;
+        s.Tb = (Mt.side == 0) ? w.Ab + off : w.Xh + off;
         p.t_mn = Mt.side == 0;
         p.epi = EPI_ABSMAX;
       }
