@@ -113,7 +113,7 @@ typedef struct {
  * bf16 buffers: about 30 bytes per weight).
  * cfg given: the size cafeq_optimize_single / cafeq_optimize_pair need for exactly that configuration.  For the
  * paper's objectives (CAFEQ_LOSS_SURROGATE / CAFEQ_LOSS_LSE) with eval_every = 0, block size 64 / 128 / 256 and a
- * shape the tensor-core pass covers, nothing matrix-sized is needed: the per-(row, group) records (16 bytes per
+ * shape the tensor-core pass covers without a half tile (d_in a multiple of 256 on the input axis), nothing matrix-sized is needed: the per-(row, group) records (16 bytes per
  * group) and the k x k scratch.  The size assumes 16-byte aligned weight rows; a call whose weights do not qualify
  * then returns CAFEQ_ERR_WORKSPACE. */
 int cafeq_workspace_size(const cafeq_matrix_desc* d1, const cafeq_matrix_desc* d2, const cafeq_opt_cfg* cfg,
@@ -129,7 +129,7 @@ int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float* T, int8_t*
 /* Scratch bytes cafeq_rtn takes from its workspace for this descriptor (host out), with (has_transform != 0) or
  * without an operator, for 16-byte aligned W and 8-byte aligned codes: 0 without a transform when the group is
  * 32 / 64 / 128 / 256 (one streaming kernel, ws may then be NULL); the per-group records when the tensor-core pass
- * covers the transformed call; matrix-sized buffers otherwise.  Never more than cafeq_workspace_size(d, NULL, NULL). */
+ * covers the transformed call without a half tile (as above); matrix-sized buffers otherwise.  Never more than cafeq_workspace_size(d, NULL, NULL). */
 int cafeq_rtn_workspace_size(const cafeq_matrix_desc* d, int has_transform, size_t* bytes);
 
 /* cafeq_rtn for callers that cannot allocate device memory and therefore have no workspace to hand
@@ -156,7 +156,8 @@ int cafeq_rtn_noalloc(const cafeq_matrix_desc* d, const void* W, const float* T,
  *   M       [nb,k,k] fp32 transform parameters; the transform applied is bf16(M).
  *   Minv    optional out [nb,k,k]: inverse of bf16(M) as computed on the device; with
  *           CAFEQ_FLAG_WARM_MINV also an input, a nearby inverse that Newton-Schulz steps refine (block sizes
- *           64/128/256; the result is checked on the device and recomputed by elimination if it did not converge).
+ *           128/256; the result is checked on the device and recomputed by elimination if it did not converge.  The
+ *           other sizes are eliminated from scratch either way).
  *   offsets optional rounding offsets [d_out,d_in] (row stride d_in): uint8 {0,1} or fp32 in [0,1]
  *           (offsets_kind); code = clamp(floor(u/s) + offset) instead of round-to-nearest.
  *   losses  out fp32[4]: {surrogate (Eq. 4), ||M^-1 Q(MW) - W||_F^2 (Eq. 3), ||W||_F^2, 0};
@@ -179,8 +180,8 @@ int cafeq_proxy_loss_fwd_bwd(const cafeq_matrix_desc* d, const void* W, const fl
 /* `cfg->steps` optimisation steps on a single matrix (Section 4.1: gradient descent on Eq. 4 from the
  * caller's initial M; Adam selectable).  M is updated in place (fp32 master parameters).
  * opt_state: fp32 [CAFEQ_OPT_STATE_HEADER + 3*nb*k*k] = {step count, 3 reserved floats, Adam first moments, Adam
- * second moments, inverse of the last step's transform}, 16-byte aligned (so that each array is: the kernels move
- * them 16 bytes at a time); required for Adam, optional for gradient descent.  Carrying it over between calls with
+ * second moments, inverse of the last step's transform}, best 16-byte aligned (the inverse of one that is not is copied to the
+ * workspace and back in every call); required for Adam, optional for gradient descent.  Carrying it over between calls with
  * cfg->resume = 1 resumes a run; the caller zeroes it before the first call.  loss_history: out fp32 [steps, 2] =
  * {surrogate, quantised loss or NaN when not evaluated at that step}. */
 int cafeq_optimize_single(const cafeq_matrix_desc* d, const void* W, float* M, float* opt_state,
@@ -256,10 +257,12 @@ int cafeq_pack(const cafeq_matrix_desc* d, const int8_t* codes, uint8_t* packed,
  *     Y[o, B k + i] = sum_j P[B][i][j] X[o, B k + j],   P = T (d->trole = CAFEQ_APPLY_T) or T^T (CAFEQ_APPLY_TT),
  * (CAFEQ_AXIS_OUT: the operator acts on the row index instead), with the operator rounded to bf16, fp32
  * accumulation, and Y written as bf16 [d_out, d_in], dense (row pitch d_in).  T: fp32 [d_in / k, k, k] on the device.
- * d->group and d->bits are not used.  Shapes the tensor-core pass covers (k in {64, 128, 256}, d_in a multiple of
- * 256, 16-byte aligned rows) run in one kernel; all others on the shape-agnostic kernels with an fp32 copy of Y in
- * the workspace.  Workspace: cafeq_apply_workspace_size bytes (sized for 16-byte aligned rows; CAFEQ_ERR_WORKSPACE
- * otherwise).  Device status word as elsewhere (may be NULL). */
+ * d->group and d->bits are not used.  On the input axis, few rows (up to 64, fewer when the matrix is wide; k a multiple of 32 up
+ * to 256) run in one small kernel; shapes the tensor-core pass covers (k in {32, 64, 128, 256}, d_in a multiple of 128; on the
+ * output axis k in {128, 256}; 16-byte aligned rows) in that pass; all others with an fp32 copy of Y in the workspace.
+ * Workspace: cafeq_apply_workspace_size bytes.  For k in {64, 128, 256} and d_in a multiple of 256 (output axis: 128) it is sized
+ * for 16-byte aligned rows, and a larger X whose rows are not gets CAFEQ_ERR_WORKSPACE.  Device status word as elsewhere (may be
+ * NULL). */
 int cafeq_apply_workspace_size(const cafeq_matrix_desc* d, size_t* bytes);
 int cafeq_apply_transform(const cafeq_matrix_desc* d, const void* X, const float* T, void* Y, int32_t* status, void* ws,
                           size_t ws_bytes, void* stream);
