@@ -604,9 +604,6 @@ static bool fused_pass(cudaStream_t st, const void* X, long long ldx, const Geo&
   return rc == CAFEQ_OK;
 }
 
-// The pass stores no U, so the array for it can hold paired operators: 64 d_in bf16 against d_out d_in fp32.
-static void* pair_scratch(const MatWS& w, const Geo& G) { return G.d_out >= 32 ? w.U : nullptr; }
-
 static bool tc_apply_ok(int k) { return k == 32 || kk_fast(k); }
 
 // U = T o W in fp32 as one-term batched products on the tensor cores (bf16 x bf16 products are exact, fp32
@@ -645,10 +642,11 @@ static bool apply_tc(cudaStream_t st, const void* W, const Geo& G, const uint16_
 // U = T o W, group absmax / arg-max, and (optionally) the quantiser outputs.  Returns true when the fused
 // tensor-core pass ran (then the residual is in w.Dbf as bf16 instead of w.D as fp32, and U is not stored).
 // T_rounded: scratch for the bf16 rounding of Tc where Tc is not rounded yet (the tensor-core paths round it themselves).
+// pair_scratch: see fused_pass.
 static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits, const float* Tc, int transposed,
                           const MatWS& w, const void* offsets, int off_kind, bool want_delta, float* Uhat, int8_t* codes,
                           float* scales, int32_t* status, bool allow_fused, const BdParams* surr = nullptr,
-                          const uint16_t* Tb_ready = nullptr, float* T_rounded = nullptr) {
+                          const uint16_t* Tb_ready = nullptr, float* T_rounded = nullptr, void* pair_scratch = nullptr) {
   if (Tc && allow_fused && off_kind == CAFEQ_OFFSETS_NONE && !Uhat) {
     BdParams p;
     memset(&p, 0, sizeof(p));
@@ -657,7 +655,7 @@ static bool forward_quant(cudaStream_t st, const void* W, const Geo& G, int bits
     p.qmax = qmax_of(bits);
     p.a = w.a; p.usel = w.usel; p.idx = w.idx;
     p.delta = w.Dbf; p.codes = codes; p.scales = scales;
-    if (fused_pass(st, W, G.ld, G, Tc, transposed, w.Tb, p, status, Tb_ready, pair_scratch(w, G))) return true;
+    if (fused_pass(st, W, G.ld, G, Tc, transposed, w.Tb, p, status, Tb_ready, pair_scratch)) return true;
   }
   if (!w.U) return false;  // lean workspace: there is no scratch for the shape-agnostic kernels (callers check first)
   bool applied = false;
@@ -842,7 +840,7 @@ extern "C" int cafeq_rtn(const cafeq_matrix_desc* d, const void* W, const float*
                                                  CAFEQ_OFFSETS_NONE, nullptr, nullptr, nullptr, nullptr, nullptr, codes, scales, nullptr))
     return last_launch();
   forward_quant(st, W, G, d->bits, has_T ? T : nullptr, d->trole == CAFEQ_APPLY_TT, w, nullptr, CAFEQ_OFFSETS_NONE, false, nullptr, codes,
-                scales, nullptr, true, nullptr, nullptr, Tc);
+                scales, nullptr, true, nullptr, nullptr, Tc, Tc);
   return last_launch();
 }
 
@@ -1056,7 +1054,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     return;
   }
   const bool fused = forward_quant(st, W, G, d->bits, s.Mc, 0, s.m, offsets, off_kind, need_l2, nullptr, nullptr, nullptr,
-                                   status, (!ste || ste_tc) && !force_generic, &sp, tc ? s.kk.Ab : nullptr);
+                                   status, (!ste || ste_tc) && !force_generic, &sp, tc ? s.kk.Ab : nullptr, nullptr, s.tmp);
   if (ste_tc && fused) {
     // Nothing below needs E = Minv o Delta itself.  With Gram_B = sum_o Delta[o, B]^T Delta[o, B] (k x k per block) and
     // N = Minv^T Minv:  L2 = <N, Gram>,  dL/dMinv = 2 Minv Gram,  gDelta = 2 N o Delta (one more block-diagonal
@@ -1141,7 +1139,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       memset(&bp, 0, sizeof(bp));
       bp.epi = EPI_SQSUM;
       bp.sqacc = s.acc + 1;
-      done = fused_pass(st, s.m.Dbf, G.d_in, G, s.Minv, 0, s.m.Tb, bp, status, nullptr, pair_scratch(s.m, G));
+      done = fused_pass(st, s.m.Dbf, G.d_in, G, s.Minv, 0, s.m.Tb, bp, status, nullptr, s.tmp);
     }
     if (!done)
       launch_apply(st, s.m.D, 0, G.d_in, G, s.Minv, 0, s.m.E, G.d_in, (ste ? GEMM_STORE : 0) | GEMM_SQSUM, s.acc + 1, status);
@@ -1519,7 +1517,7 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
   const bool f1 = forward_quant(st, W1, G1, d1->bits, p.Mc, 1, p.m1, nullptr, CAFEQ_OFFSETS_NONE, false, want_pqe ? p.m1.E : nullptr, nullptr,
                 nullptr, status, !force_generic);
   const bool f2 = forward_quant(st, W2, G2, d2->bits, p.Minv_c, 0, p.m2, nullptr, CAFEQ_OFFSETS_NONE, false, want_pqe ? p.m2.E : nullptr,
-                nullptr, nullptr, status, !force_generic, nullptr, tc ? p.kk.Xh : nullptr);  // Xh = bf16(Minv)
+                nullptr, nullptr, status, !force_generic, nullptr, tc ? p.kk.Xh : nullptr, nullptr, p.tmp);  // Xh = bf16(Minv)
   const long long n1 = (long long)G1.d_out * G1.ng, n2 = (long long)G2.d_out * G2.ng;
   CQ_LAUNCH(max2_f32_kernel, grid_for(n1 + n2), 256, 0, st, p.m1.a, n1, p.m2.a, n2, p.amax, status);
   CQ_LAUNCH(sumexp2_kernel, grid_for(n1 + n2), 256, 0, st, p.m1.a, n1, p.m2.a, n2, p.amax, t, p.acc + 0, status);
