@@ -64,9 +64,9 @@ __device__ __forceinline__ void raise_status(int32_t* status, int code) {
 // kernel on a side stream, may raise the word at any time; threads that each looked for themselves could disagree, and the
 // ones that went on would wait at barriers (or on tensor memory) for the ones that had left.
 __device__ __forceinline__ bool status_raised(const int32_t* status) { return status && *status; }
-__device__ __forceinline__ bool cta_stopped(const int32_t* status) { return __syncthreads_or(status_raised(status)) != 0; }
+__device__ __forceinline__ bool cta_stopped(const int32_t* status) { return status && __syncthreads_or(*status) != 0; }
 // the same for kernels whose threads meet inside a warp only
-__device__ __forceinline__ bool warp_stopped(const int32_t* status) { return __any_sync(0xffffffffu, status_raised(status)) != 0; }
+__device__ __forceinline__ bool warp_stopped(const int32_t* status) { return status && __any_sync(0xffffffffu, *status) != 0; }
 
 __device__ __forceinline__ double block_sum_double(double v, double* sh) {
   // sh: at least 32 doubles of shared memory
@@ -720,14 +720,30 @@ __global__ void __launch_bounds__(256) scatter_in_kernel(const uint16_t* W, long
   const int j = js + lane;
   // groups that intersect this block: columns [B*k, B*k + k)
   const int G0 = (B * k) / g, G1 = (B * k + k - 1) / g;
-  for (int o = r0 + warp; o < r1; o += nw) {
-    float w = (j < k) ? bf16_bits_to_float(W[o * ld + (long long)B * k + j]) : 0.f;
+  for (int o0 = r0 + warp; o0 < r1; o0 += 4 * nw) {
+    float w[4];  // (four rows' loads before their atomic additions)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int o = o0 + u * nw;
+      w[u] = (o < r1 && j < k) ? bf16_bits_to_float(W[o * ld + (long long)B * k + j]) : 0.f;
+    }
     for (int G = G0; G <= G1; ++G) {
-      long long p = gm ? (long long)G * d_out + o : (long long)o * ng + G;
-      int col = G * g + idx[p];          // arg-max column of the group
-      if (col < B * k || col >= B * k + k) continue;  // group larger than the block: arg-max in another block
-      float cf = coef[p];
-      if (j < k && cf != 0.f) atomicAdd(&acc[(col - B * k) * SCATTER_JS + lane], cf * w);
+      int col[4];
+      float cf[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int o = o0 + u * nw;
+        col[u] = -1;
+        cf[u] = 0.f;
+        if (o < r1) {
+          const long long p = gm ? (long long)G * d_out + o : (long long)o * ng + G;
+          col[u] = G * g + idx[p] - B * k;  // arg-max column of the group (of a larger group: perhaps in another block)
+          cf[u] = coef[p];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if ((unsigned)col[u] < (unsigned)k && j < k && cf[u] != 0.f) atomicAdd(&acc[col[u] * SCATTER_JS + lane], cf[u] * w[u]);
     }
   }
   __syncthreads();
@@ -899,14 +915,15 @@ __global__ void __launch_bounds__(256, 2) scatter_in_bucket_kernel(const uint16_
     if (e < np) {
       const int row = e / NG, q = e - row * NG;
       const long long p = gm ? (long long)(G0 + q) * d_out + r0 + row : (long long)(r0 + row) * ng + G0 + q;
-      const float c = ld_plain(coef + p);
+      cfv[u] = ld_plain(coef + p);
       const int col = q * g + ld_plain(idx + p) + off;
-      if ((unsigned)col < (unsigned)K && c != 0.f) {
-        bk[u] = (short)col;
-        cfv[u] = c;
-        atomicAdd(&cnt[col], 1);
-      }
+      if ((unsigned)col < (unsigned)K) bk[u] = (short)col;
     }
+  }
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) {  // (after every load: they may not be moved past an atomic addition)
+    if (cfv[u] == 0.f) bk[u] = -1;
+    if (bk[u] >= 0) atomicAdd(&cnt[bk[u]], 1);
   }
   __syncthreads();
   // exclusive scan of cnt -> start (K <= 256: one entry per thread)
@@ -1541,20 +1558,28 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* packed, con
     unsigned long long v = 0;
     for (int b = 0; b < bits; ++b) v |= (unsigned long long)src[b] << (8 * b);
     uint16_t* dst = out + row * ldo + ch * 8;
+    float s[8];  // (every load before the first store, which may not be moved past one)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] = ld_plain(scales + row * ng + ((int)ch * 8 + i) / g);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int col = (int)ch * 8 + i;
-      const float s = ld_plain(scales + row * ng + col / g);
       const int q = (int)((v >> (bits * i)) & mask) - qmax;
-      dst[i] = __bfloat16_as_ushort(__float2bfloat16_rn(s * (float)q));
+      dst[i] = __bfloat16_as_ushort(__float2bfloat16_rn(s[i] * (float)q));
     }
   }
 }
 
 __global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* in, uint16_t* __restrict__ out, long long n) {
   pdl_enter();
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-    out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(in[e]));
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; e0 < n; e0 += 4 * stride) {
+    float x[4];  // (four loads before the first store)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = (e0 + u * stride < n) ? in[e0 + u * stride] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (e0 + u * stride < n) out[e0 + u * stride] = __bfloat16_as_ushort(__float2bfloat16_rn(x[u]));
+  }
 }
 
 // The same stream, 32 codes per thread: 32 b-bit fields are exactly b 32-bit words, so a thread reads two 16-byte
