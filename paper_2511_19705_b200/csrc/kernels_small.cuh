@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(256) small_inverse_kernel(const float* Min, fl
                                                             uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, uint16_t* __restrict__ thi,
                                                             uint16_t* __restrict__ tlo, int32_t* status) {
   pdl_enter();
-  if (cta_stopped(status)) return;
+  const bool raised = status_raised(status);  // (awaited with the block's loads)
   constexpr int R = K / 32, CW = K / 8;
   __shared__ float tile[K][K + 1];
   __shared__ float fcol[2][K];
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) small_inverse_kernel(const float* Min, fl
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t base = (size_t)blockIdx.x * K * K;
   for (int e = tid; e < K * K; e += 256) tile[e / K][e % K] = Min[base + e];
-  __syncthreads();
+  if (__syncthreads_or(raised)) return;
   float a[R][CW];
 #pragma unroll
   for (int q = 0; q < R; ++q)
