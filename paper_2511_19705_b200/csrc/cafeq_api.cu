@@ -1576,19 +1576,19 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     // whose dependence on the group's arg-max entry is kept.
     DenseWS& w = p.dn;
     {  // g Vhat' [d3, h] = 2 R^T Uhat^T (one column for the replicas of an inner column)
-      const uint16_t* a[3] = {w.PTl, w.PTh, w.PTh};  // (small terms first, here and below: see launch_dense_tc6)
-      const uint16_t* b[3] = {w.Awh, w.Awl, w.Awh};
+      const uint16_t* a[2] = {w.PTh, w.PTl};
+      const uint16_t* b[2] = {w.Awh, w.Awl};
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
-      if ((p.err = launch_dense_tc(st, 3, a, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, status))) return;
+      if ((p.err = launch_dense_tc(st, 2, a, 2, b, w.d3, w.h, w.d1, 2.f, 0.f, 0.f, o, nullptr, status))) return;
     }
     {  // g Uhat [h, d1] = 2 fold(Vhat^T) R^T (the folded splits are read as they are stored: an MN-major operand costs the
       // product 10 %, 14 us, where folding, transposing and splitting again took 60)
-      const uint16_t* a[3] = {w.Vl, w.Vh, w.Vh};
-      const uint16_t* b[3] = {w.Ph, w.Pl, w.Ph};
+      const uint16_t* a[2] = {w.Vh, w.Vl};
+      const uint16_t* b[2] = {w.Ph, w.Pl};
       DenseOut o;
       o.C = w.U; o.ldc = w.d1;
-      if ((p.err = launch_dense_tc(st, 3, a, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, status, 1))) return;
+      if ((p.err = launch_dense_tc(st, 2, a, 2, b, w.h, w.d1, w.d3, 2.f, 0.f, 0.f, o, nullptr, status, 1))) return;
     }
     if (!tc) {
       CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, gradM, 0.f, kk);

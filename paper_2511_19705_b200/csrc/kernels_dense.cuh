@@ -23,8 +23,9 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, 
                                                          float* __restrict__ YT, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
                                                          uint16_t* __restrict__ thi, uint16_t* __restrict__ tlo,
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
-                                                         uint16_t* __restrict__ t3 = nullptr) {
+                                                         uint16_t* __restrict__ t3 = nullptr, const double* only_bad = nullptr) {
   pdl_enter();
+  if (only_bad && *only_bad <= 0.25) return;  // (a restart that is not needed)
   if (cta_stopped(status)) return;
   __shared__ uint32_t tile[64][65];
   __shared__ uint16_t tile3[64][66];
@@ -329,67 +330,54 @@ __global__ void __launch_bounds__(256) dot_f32_kernel(const float* x, const floa
   if (threadIdx.x == 0 && s != 0.0) atomicAdd(acc, s);
 }
 
-// Power iteration for the largest singular value of S [R, C] (fp32, row-major), used to scale the starting guess
-// of the pseudo-inverse iteration.  Two kernels per round: u = S v / |v| (one warp per row; every CTA sums |v|^2 itself), then
-// v' = S^T u (one thread per column, slices of 32 rows, partial sums added atomically).  Three buffers of v in turn: one read,
-// one written, one cleared.  Bound by reading S twice per round (29 MB, from L2: 11 + 5 us; with slices of 512 rows, 56 CTAs,
-// the second kernel took 75 us, and norm and scaling were launches of their own).
-// After the last round *sig2 = safety * |S^T S v| (v of unit norm): a Rayleigh-type estimate from below of sigma_max^2.
-__global__ void pw_init_kernel(float* __restrict__ v, int C) {
-  pdl_enter();  // v [3][C]
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < C) {
-    uint32_t h = (uint32_t)j * 2654435761u;
-    h ^= h >> 15;
-    v[j] = (h & 1u) ? 1.f : -1.f;  // fixed +-1 pattern
-    v[C + j] = 0.f;
+// Start of the Gram iteration: G = A A^T (fp32 [m, m], tiles of 256 on and above the diagonal) -> B0 = G / c with c = 1.0001 ||G||_F,
+// so that its eigenvalues lie in [0, 1], and Y1 = (2 mu I - mu^2 B0) / c, both as fp32 (same tiles; B in place of G) and as bf16
+// splits of the whole symmetric matrix.  *c_out = c.  One 64 x 64 tile per CTA (grid: m / 64, m / 64); memory-bound.
+__global__ void __launch_bounds__(256) gram_start_kernel(float* G, int m, const double* fro2, float mu, float* __restrict__ Y,
+                                                         uint16_t* __restrict__ Bh, uint16_t* __restrict__ Bl,
+                                                         uint16_t* __restrict__ Yh, uint16_t* __restrict__ Yl,
+                                                         double* __restrict__ c_out, const int32_t* status) {
+  pdl_enter();
+  if (cta_stopped(status)) return;
+  if ((blockIdx.x >> 2) < (blockIdx.y >> 2)) return;
+  __shared__ uint32_t tb[64][65], ty[64][65];
+  const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
+  const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const double c = 1.0001 * sqrt(*fro2);
+  const float inv = c > 0.0 ? (float)(1.0 / c) : 0.f;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *c_out = c;
+  auto split = [](float x) -> uint32_t {
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    return (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(h))) << 16);
+  };
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = w + 8 * q, row = r0 + i, col = c0 + 2 * tx;
+    const long long o = (long long)row * m + col;
+    const float2 g = ld_plain(reinterpret_cast<const float2*>(G + o));
+    const float2 b = make_float2(g.x * inv, g.y * inv);
+    const float2 y = make_float2(((row == col ? 2.f * mu : 0.f) - mu * mu * b.x) * inv, ((row == col + 1 ? 2.f * mu : 0.f) - mu * mu * b.y) * inv);
+    *reinterpret_cast<float2*>(G + o) = b;
+    *reinterpret_cast<float2*>(Y + o) = y;
+    const uint32_t b0 = split(b.x), b1 = split(b.y), y0 = split(y.x), y1 = split(y.y);
+    *reinterpret_cast<uint32_t*>(Bh + o) = (b0 & 0xFFFFu) | (b1 << 16);
+    *reinterpret_cast<uint32_t*>(Bl + o) = (b0 >> 16) | (b1 & 0xFFFF0000u);
+    *reinterpret_cast<uint32_t*>(Yh + o) = (y0 & 0xFFFFu) | (y1 << 16);
+    *reinterpret_cast<uint32_t*>(Yl + o) = (y0 >> 16) | (y1 & 0xFFFF0000u);
+    tb[i][2 * tx] = b0; tb[i][2 * tx + 1] = b1;
+    ty[i][2 * tx] = y0; ty[i][2 * tx + 1] = y1;
   }
-}
-__device__ __forceinline__ double pw_norm2(const float* v, int C, double* red) {
-  double s = 0.0;
-  for (int j = threadIdx.x; j < C; j += blockDim.x) s += (double)v[j] * (double)v[j];
-  s = block_sum_double(s, red);
-  __shared__ double out;
-  if (threadIdx.x == 0) out = s;
+  if ((blockIdx.x >> 2) == (blockIdx.y >> 2)) return;  // (diagonal tiles are stored whole)
   __syncthreads();
-  return out;
-}
-__global__ void __launch_bounds__(256) pw_rows_kernel(const float* S, const float* v, float* __restrict__ clear,
-                                                      int R, int C, float* __restrict__ u) {
-  pdl_enter();
-  __shared__ double red[32];
-  const double n = sqrt(pw_norm2(v, C, red));
-  const float inv = n > 0.0 ? (float)(1.0 / n) : 0.f;
-  for (int j = blockIdx.x * 256 + threadIdx.x; j < C; j += gridDim.x * 256) clear[j] = 0.f;
-  const long long w = (blockIdx.x * 256ll + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= R) return;
-  float s = 0.f;
-  for (int j = lane; j < C; j += 32) s = fmaf(S[w * C + j], v[j], s);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) u[w] = s * inv;
-}
-// grid: (ceil(C / 256), ceil(R / 32)); v2 cleared two launches before
-__global__ void __launch_bounds__(256) pw_cols_kernel(const float* S, const float* u, int R, int C,
-                                                      float* __restrict__ v2) {
-  pdl_enter();
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= C) return;
-  const int r0 = blockIdx.y * 32, n = min(R - r0, 32);
-  float s = 0.f;
-#pragma unroll 8
-  for (int r = 0; r < n; ++r) s = fmaf(S[(long long)(r0 + r) * C + j], u[r0 + r], s);
-  atomicAdd(&v2[j], s);
-}
-__global__ void __launch_bounds__(256) pw_result_kernel(const float* v, int C, double safety, const double* fro2, double* sig2) {
-  pdl_enter();
-  __shared__ double red[32];
-  const double n = sqrt(pw_norm2(v, C, red));
-  if (threadIdx.x == 0) {
-    // never above the Frobenius bound (always safe), never zero (a failed estimate)
-    double e = safety * n;
-    if (!(e > 0.0) || e > *fro2) e = *fro2;
-    *sig2 = e;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int j = w + 8 * q;
+    const long long o = (long long)(c0 + j) * m + r0 + 2 * tx;
+    const uint32_t b0 = tb[2 * tx][j], b1 = tb[2 * tx + 1][j], y0 = ty[2 * tx][j], y1 = ty[2 * tx + 1][j];
+    *reinterpret_cast<uint32_t*>(Bh + o) = (b0 & 0xFFFFu) | (b1 << 16);
+    *reinterpret_cast<uint32_t*>(Bl + o) = (b0 >> 16) | (b1 & 0xFFFF0000u);
+    *reinterpret_cast<uint32_t*>(Yh + o) = (y0 & 0xFFFFu) | (y1 << 16);
+    *reinterpret_cast<uint32_t*>(Yl + o) = (y0 >> 16) | (y1 & 0xFFFF0000u);
   }
 }
 

@@ -51,6 +51,7 @@ struct TgParams {
                           // batch * colsA_per_batch / colsB_per_batch (B: its contraction at row batch * rowsB_per_batch)
   const double* stop_sq;  // optional: squared residuals of an iteration; this launch belongs to iteration stop_it, and is
   int stop_it;            // skipped when the rule (tg_stopped) ended the iteration before
+  int stop_guard;         // 1: iteration 0 checks its start; 2: this is its update, skipped when the start is bad
   int32_t* status;
 };
 
@@ -68,23 +69,35 @@ struct TgCfg {
 // falling (a rank-deficient matrix stalls at its rank defect).  With every eigenvalue of A X in (0, 2) the residual falls
 // monotonically: one that is still large and grows means that the starting scale was too small, which is reported.
 // The residuals of iterations that were skipped stay zero, so the last two decide.
-__device__ __forceinline__ bool tg_stopped(const TgParams& p) {
-  if (!p.stop_sq || p.stop_it < 1) return false;
-  const double cur = p.stop_sq[p.stop_it - 1];
+// With stop_guard, iteration 0 checks a start that is only good when its squared residual is at most 1/4; otherwise the iteration
+// has been restarted, and what came before iteration 1 does not count.  Iteration 0 itself then updates nothing.
+__device__ __forceinline__ bool tg_bad_start(const volatile double* stop_sq) { return !(stop_sq[0] <= 0.25); }
+__device__ __forceinline__ bool tg_stopped(const TgParams& p, int it) {
+  const volatile double* sq = p.stop_sq;  // (one launch may run several iterations: never from a cached line)
+  if (!sq) return false;
+  if (p.stop_guard) {
+    if (it == 0) return p.stop_guard == 2 && tg_bad_start(sq);
+    if (tg_bad_start(sq)) { ++sq; --it; }
+  }
+  if (it < 1) return false;
+  const double cur = sq[it - 1];
   if (!(cur > 1e-6)) return true;
-  if (p.stop_it < 2) return false;
-  const double prev = p.stop_sq[p.stop_it - 2];
+  if (it < 2) return false;
+  const double prev = sq[it - 2];
   if (cur > 1.5 * prev && cur > 1e-2 * (double)p.M) {
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) raise_status(p.status, CAFEQ_ERR_NONFINITE);
     return true;
   }
-  return p.stop_it >= 5 && cur > prev * (1.0 - 1e-7) && cur < prev * (1.0 + 1e-7);
+  return it >= 5 && cur > prev * (1.0 - 1e-7) && cur < prev * (1.0 + 1e-7);
 }
+__device__ __forceinline__ bool tg_stopped(const TgParams& p) { return tg_stopped(p, p.stop_it); }
 
 // One 32-column chunk of one 128-row accumulator tile: scaling, C0, identity, sum of squares and every output format.
 // taddr: the tile's accumulator at this warp's lane quarter; tile: this warp's [32][36] fp32 scratch in shared memory.
+// taddr2: a second accumulator that is added to the first (0: none).  Cthi / Ctlo as in p, or none for this tile.
 __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b, const int m0, const int n0, const int ch,
-                                                  const uint32_t taddr, float* tile, const int q, const int lane, double& sq) {
+                                                  const uint32_t taddr, const uint32_t taddr2, uint16_t* Cthi, uint16_t* Ctlo,
+                                                  float* tile, const int q, const int lane, double& sq) {
   const int row = m0 + q * 32 + lane;
   const bool rv = row < p.M;
   const long long cb = (long long)b * p.sCb, c0b = (long long)b * p.sC0b;
@@ -94,9 +107,18 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
   const int rbase = m0 + q * 32;
   const int r4 = lane >> 3, c4 = (lane & 7) * 4;
   const int nb0 = n0 + ch * 32;
-  if (nb0 >= p.N) return;
+  if (nb0 >= p.N || rbase >= p.M) return;
   float v[32];
   tc_ld32(taddr + ch * 32, v);
+  if (taddr2) {
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      float w[16];
+      tc_ld16(taddr2 + ch * 32 + hf * 16, w);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[hf * 16 + e] += w[e];
+    }
+  }
   const bool inner = (nb0 + 32 <= p.N) && (m0 + 128 <= p.M);  // no edge in this chunk
   // Vector path (no edge, every pitch a multiple of 4 elements, aligned bases): a lane moves 16 bytes per
   // shared-memory access (pitch 36 floats: conflict-free by quarter warps) and a warp instruction covers
@@ -147,7 +169,7 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
       if (e < nv) sqf = fmaf(v[e], v[e], sqf);
     sq += (double)sqf;
   }
-  if (p.C || p.Chi || (p.Cthi && !(inner && (p.M & 1) == 0))) {
+  if (p.C || p.Chi || (Cthi && !(inner && (p.M & 1) == 0))) {
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       *reinterpret_cast<float4*>(tile + lane * 36 + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
@@ -192,10 +214,10 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
         }
       }
     }
-    if (p.Cthi && !(inner && (p.M & 1) == 0) && rv) {
+    if (Cthi && !(inner && (p.M & 1) == 0) && rv) {
       // transposed outputs on an edge: this lane's row, one column at a time (read back from its tile row)
-      uint16_t* cth = p.Cthi + sb_mn + (long long)nb0 * p.M + row;
-      uint16_t* ctl = p.Ctlo ? p.Ctlo + sb_mn + (long long)nb0 * p.M + row : nullptr;
+      uint16_t* cth = Cthi + sb_mn + (long long)nb0 * p.M + row;
+      uint16_t* ctl = Ctlo ? Ctlo + sb_mn + (long long)nb0 * p.M + row : nullptr;
 #pragma unroll 1
       for (int e = 0; e < 32; ++e) {
         if (nb0 + e < p.N) {
@@ -208,7 +230,7 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
     }
     __syncwarp();
   }
-  if (p.Cthi && inner && (p.M & 1) == 0) {
+  if (Cthi && inner && (p.M & 1) == 0) {
     // transposed outputs: consecutive lanes are consecutive rows = consecutive addresses.  Neighbouring
     // lanes trade one value so that every lane stores a 32-bit pair of rows: even lanes write column e,
     // odd lanes column e + 1.
@@ -225,8 +247,8 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
       const uint32_t other = __shfl_xor_sync(0xffffffffu, odd ? p0 : p1, 1);  // the neighbour row's, same column
       const uint32_t lo_row = odd ? other : mine, hi_row = odd ? mine : other;  // rows (2j, 2j + 1)
       const long long o = sb_mn + (long long)(nb0 + e + odd) * p.M + rowpair;
-      *reinterpret_cast<uint32_t*>(p.Cthi + o) = (lo_row & 0xFFFFu) | (hi_row << 16);
-      if (p.Ctlo) *reinterpret_cast<uint32_t*>(p.Ctlo + o) = (lo_row >> 16) | (hi_row & 0xFFFF0000u);
+      *reinterpret_cast<uint32_t*>(Cthi + o) = (lo_row & 0xFFFFu) | (hi_row << 16);
+      if (Ctlo) *reinterpret_cast<uint32_t*>(Ctlo + o) = (lo_row >> 16) | (hi_row & 0xFFFF0000u);
     }
   }
 }
@@ -347,7 +369,7 @@ tc_gemm_kernel(const __grid_constant__ TgMaps maps, const __grid_constant__ TgPa
       double sq = 0.0;
       float* tile = reinterpret_cast<float*>(smem + (warp - 2) * 4608);  // [32][36] per warp (stage buffers are free now)
 #pragma unroll 1
-      for (int ch = part; ch < BN / 32; ch += TG_EPI_PARTS) tg_epilogue_chunk(p, b, m0, n0, ch, taddr, tile, q, lane, sq);
+      for (int ch = part; ch < BN / 32; ch += TG_EPI_PARTS) tg_epilogue_chunk(p, b, m0, n0, ch, taddr, 0u, p.Cthi, p.Ctlo, tile, q, lane, sq);
       if (p.sq) {
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         if (lane == 0 && sq != 0.0) atomicAdd(p.sq + (long long)b * p.sq_stride, sq);

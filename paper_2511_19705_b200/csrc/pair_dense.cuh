@@ -4,6 +4,7 @@
 #pragma once
 
 #include "kernels_dense.cuh"
+#include "kernels_gemm2.cuh"
 
 namespace cafeq {
 
@@ -16,22 +17,14 @@ struct DenseOut {
   uint16_t *Chi = nullptr, *Clo = nullptr, *Cthi = nullptr, *Ctlo = nullptr;
   double* sq = nullptr;
   const double* stop_sq = nullptr;  // stopping rule of an iteration (TgParams)
-  int stop_it = 0;
+  int stop_it = 0, stop_guard = 0;
 };
 
-// A operands are [M, K] row-major (a_mn: [K, M]), B operands [N, K] row-major; nterms pairs (A[t], B[t]).
-static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A, const uint16_t* const* B, int M, int N, int K,
-                           float alpha, float beta, float gamma, const DenseOut& o, int32_t* status, int a_mn = 0) {
-  TgOperand oa[TG_MAX_TERMS], ob[TG_MAX_TERMS];
-  for (int t = 0; t < nterms; ++t) {
-    oa[t] = a_mn ? TgOperand{A[t], K, M, M} : TgOperand{A[t], M, K, K};
-    ob[t] = TgOperand{B[t], N, K, K};
-  }
+static TgParams dense_params(int M, int N, int K, float alpha, float beta, float gamma, const DenseOut& o, int32_t* status, int a_mn) {
   TgParams p;
   memset(&p, 0, sizeof(p));
   p.M = M; p.N = N; p.K = K;
   p.batch = 1;
-  p.nterms = nterms;
   p.divA = 1;
   p.alpha = alpha; p.beta = beta; p.gamma = gamma;
   p.C0 = o.C0; p.ldc0 = o.ldc0;
@@ -39,39 +32,80 @@ static int launch_dense_tc(cudaStream_t st, int nterms, const uint16_t* const* A
   p.Chi = o.Chi; p.Clo = o.Clo; p.Cthi = o.Cthi; p.Ctlo = o.Ctlo;
   p.sq = o.sq; p.sq_stride = 0;
   p.a_mn = a_mn;
-  p.stop_sq = o.stop_sq; p.stop_it = o.stop_it;
+  p.stop_sq = o.stop_sq; p.stop_it = o.stop_it; p.stop_guard = o.stop_guard;
   p.status = status;
+  return p;
+}
+
+// One launch of up to three terms on the tiled kernel, in the order given.
+static int tg_launch_dense(cudaStream_t st, int nterms, const uint16_t* const* A, const uint16_t* const* B, int M, int N, int K,
+                              float alpha, float beta, float gamma, const DenseOut& o, int32_t* status, int a_mn) {
+  TgOperand oa[TG_MAX_TERMS], ob[TG_MAX_TERMS];
+  for (int t = 0; t < nterms; ++t) {
+    oa[t] = a_mn ? TgOperand{A[t], K, M, M} : TgOperand{A[t], M, K, K};
+    ob[t] = TgOperand{B[t], N, K, K};
+  }
+  TgParams p = dense_params(M, N, K, alpha, beta, gamma, o, status, a_mn);
+  p.nterms = nterms;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return tg_launch(st, oa, ob, p);
 }
 
-static void launch_split_rect(cudaStream_t st, const float* X, int R, int C, long long ld, float scale, const double* inv_scale,
-                              float* Y, float* YT, uint16_t* hi, uint16_t* lo, uint16_t* thi, uint16_t* tlo, const int32_t* status,
-                              uint16_t* h3 = nullptr, uint16_t* t3 = nullptr) {
-  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3);
-}
-
-// The same product with both operands split three ways (x = x1 + x2 + x3, 24 significand bits): the six terms down to
-// 2^-24 relative, as two launches of three terms that accumulate through the fp32 output `acc` (row-major [M, N],
-// pitch N; it may be o.C).  fp32-grade accuracy: what is left is the rounding of the fp32 accumulators.
-// A / B: {x1, x2, x3} in the layouts launch_dense_tc takes.
-static int launch_dense_tc6(cudaStream_t st, const uint16_t* const* A, const uint16_t* const* B, int M, int N, int K, float alpha,
-                            float beta, float gamma, const DenseOut& o, float* acc, int32_t* status) {
+// C = alpha * A B^T + beta * C0 + gamma * I with A [M, K] (a_mn: [K, M]) and B [N, K] given as sums of na and nb bf16 arrays
+// ({hi, lo}: 16 significand bits, {hi, lo, third}: 24): the terms A_i B_j with i + j < max(na, nb).  With two arrays each these
+// are three terms (fp32-grade to about 2^-17 per entry), with three each six, down to 2^-24: what is left is the rounding of the
+// fp32 accumulators.  acc: fp32 [M, N] for the first half of more than three terms on the tiled kernel (it may be o.C).
+//
+// Large products run on CTA pairs.  The line lies where tiles of 256 rows fill the chip worse than the tiled kernel's 128-row
+// ones by more than the latter lose to their operand traffic.
+static int launch_dense_tc(cudaStream_t st, int na, const uint16_t* const* A, int nb, const uint16_t* const* B, int M, int N, int K,
+                        float alpha, float beta, float gamma, const DenseOut& o, float* acc, int32_t* status, int a_mn = 0) {
+  const int order = na > nb ? na : nb;
+  double cost;
+  const int bn = t2_width(M, N, 0, &cost);
+  if (K % TG_BK == 0 && t2_wanted(M, N, cost)) {
+    T2Maps maps;
+    T2Params tp;
+    memset(&maps, 0, sizeof(maps));
+    memset(&tp, 0, sizeof(tp));
+    bool ok = true;
+    for (int i = 0; i < na; ++i)
+      ok = ok && make_map_bf16(&maps.a[0][i], A[i], a_mn ? M : K, a_mn ? K : M, a_mn ? M : K, a_mn ? 64 : 128);
+    for (int j = 0; j < nb; ++j) ok = ok && make_map_bf16(&maps.b[j], B[j], K, N, K, bn / 2);
+    if (ok) {
+      tp.p[0] = dense_params(M, N, K, alpha, beta, gamma, o, status, a_mn);
+      tp.nprob = 1;
+      tp.sh = t2_shape(M, N, bn, na, nb, order);
+      g_launches.fetch_add(1, std::memory_order_relaxed);
+      return t2_launch(st, maps, tp);
+    }
+  }
   // The small terms first: every addition to an accumulator is rounded at the accumulator's size, so small terms that follow the
   // large ones cost as much accuracy as those.  Product of bf16 weights with two replicas folded (their sums have a second term),
   // 2048 x 3584 x 3584, against float64: 2.0e-6, large terms first 6.0e-6.
   const uint16_t* a1[3] = {A[1], A[0], A[0]};
   const uint16_t* b1[3] = {B[0], B[1], B[0]};
+  if (order == 2) return tg_launch_dense(st, 3, a1, b1, M, N, K, alpha, beta, gamma, o, status, a_mn);
   DenseOut o1;
   o1.C0 = o.C0; o1.ldc0 = o.ldc0;
   o1.C = acc; o1.ldc = N;
-  int rc = launch_dense_tc(st, 3, a1, b1, M, N, K, alpha, beta, gamma, o1, status);
+  int rc = tg_launch_dense(st, 3, a1, b1, M, N, K, alpha, beta, gamma, o1, status, a_mn);
   if (rc) return rc;
-  const uint16_t* a2[3] = {A[0], A[2], A[1]};
-  const uint16_t* b2[3] = {B[2], B[0], B[1]};
+  const uint16_t* a2[3];
+  const uint16_t* b2[3];
+  int n2 = 0;
+  if (nb > 2) { a2[n2] = A[0]; b2[n2++] = B[2]; }
+  if (na > 2) { a2[n2] = A[2]; b2[n2++] = B[0]; }
+  a2[n2] = A[1]; b2[n2++] = B[1];
   DenseOut o2 = o;
   o2.C0 = acc; o2.ldc0 = N;
-  return launch_dense_tc(st, 3, a2, b2, M, N, K, alpha, 1.f, 0.f, o2, status);
+  return tg_launch_dense(st, n2, a2, b2, M, N, K, alpha, 1.f, 0.f, o2, status, a_mn);
+}
+
+static void launch_split_rect(cudaStream_t st, const float* X, int R, int C, long long ld, float scale, const double* inv_scale,
+                              float* Y, float* YT, uint16_t* hi, uint16_t* lo, uint16_t* thi, uint16_t* tlo, const int32_t* status,
+                              uint16_t* h3 = nullptr, uint16_t* t3 = nullptr, const double* only_bad = nullptr) {
+  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3, only_bad);
 }
 
 // Scratch of the dense pair algebra for a pair with stored shapes U [h, d1], V [d3, rh]
@@ -92,7 +126,7 @@ struct DenseWS {
   double* sq;                             // [DENSE_SQ] accumulators: 0..: PQE history, 32..: iteration residuals
 };
 constexpr int DENSE_SQ = 128;
-constexpr int PINV_MAX_ITERS = 56;
+constexpr int PINV_MAX_ITERS = 60;
 
 static bool carve_dense(Bump& b, int h, int d1, int d3, int r, int k, int ng1, int ng2, DenseWS* w) {
   const size_t rh = (size_t)r * h, D = (size_t)(d1 > d3 ? d1 : d3);
@@ -130,67 +164,161 @@ static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, 
   return b.used + 4096;
 }
 
-// out (hi / lo, shape [R, C] of S) = pinv(S^T) = pinv(S)^T by the Newton-Schulz iteration X <- X + X (I - A X) on
-// the wide orientation A of S ([m, n], m <= n), carried as Y = X^T so that every product has both operands
-// contraction-major.  Start X0 = A^T / c with c = 1.25 x a power-iteration estimate of sigma_max(A)^2, capped by
-// ||A||_F^2: the eigenvalues of A X0 lie in (0, 2) (the estimate is from below and a few percent off at most; the
-// iteration converges for anything below 2), to the Moore-Penrose inverse.  Scaling by sigma_max^2 instead of the
-// always-safe ||A||_F^2 saves log2(stable rank) doublings of the smallest eigenvalue.  Stops on the device when ||I - A X||_F falls below 1e-3 (the next
-// update squares it) or stalls (rank-deficient A), which every product works out from the residuals itself; the remaining
-// launches then return at once.
-// (Two things that were slower or worse: scaling the iterate by 2 / (1 + l) for a lower bound l of the eigenvalues, 10
-// iterations instead of 16 on the 9B-shaped v-o factors, cancels the large components of X against the product at every step,
-// and the rounding that this leaves outside the row space of A is never corrected: codes that matched the float64
-// pseudo-inverse differed.  Reading Y and C row-major as MN-major operands, with no transposed outputs: 114 us for
-// 2048 x 3584 x 2048 against 102.)
+// Approximate G^-1 = (A A^T)^-1 for the splits of A in w.Aw* ([m, n], m <= n), left as bf16 splits in w.CTh / w.CTl; w.sq + 123: c.
+// Y <- 2 mu Y - mu^2 Y B and B <- 2 mu B - mu^2 B B from B = G / c (c a little above ||G||_F), Y = I / c: B = G Y c throughout, and
+// with mu = 2 / (1 + l) for the smallest eigenvalue l of B the eigenvalues of B go to 1, l growing fourfold a step at first.
+// Both are polynomials in G, so one launch does both products on their upper tiles: 36 + 36 pairs at m = 2048, one wave, 45 us; a
+// step of the rectangular iteration takes 160.  l starts at 2^-14: smaller eigenvalues grow as far as that and are finished by the
+// rectangular iteration.  (Nothing here need be accurate: whatever Y is, A^T Y lies in the row space of A, and its error is what the
+// rectangular iteration corrects.)
+constexpr int GRAM_STEPS = 9;
+static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2, int32_t* status) {
+  T2Maps maps;
+  T2Params tp;
+  int rc;
+  const uint16_t* aw[2] = {w.Awh, w.Awl};
+  memset(&maps, 0, sizeof(maps));
+  memset(&tp, 0, sizeof(tp));
+  for (int i = 0; i < 2; ++i)
+    if (!make_map_bf16(&maps.a[0][i], aw[i], n, m, n, 128) || !make_map_bf16(&maps.b[i], aw[i], n, m, n, 128)) return CAFEQ_ERR_UNSUPPORTED;
+  DenseOut g;
+  g.C = w.Y; g.ldc = m; g.sq = fro2;
+  tp.p[0] = dense_params(m, m, n, 1.f, 0.f, 0.f, g, status, 0);
+  tp.nprob = 1;
+  tp.sh = t2_shape(m, m, 256, 2, 2, 2);
+  tp.sh.sym = 1;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  if ((rc = t2_launch(st, maps, tp))) return rc;
+  uint16_t* Bs[2][2] = {{w.Yh, w.Yl}, {w.YTh[0], w.YTl[0]}};
+  uint16_t* Ys[2][2] = {{w.YTh[1], w.YTl[1]}, {w.CTh, w.CTl}};
+  static_assert(GRAM_STEPS % 2 == 1, "the result is left in the second pair of buffers");
+  double l = 1.0 / 16384.0;
+  for (int j = 0; j < GRAM_STEPS; ++j) {
+    const float mu = (float)(2.0 / (1.0 + l));
+    l = 4.0 * l / ((1.0 + l) * (1.0 + l));
+    if (j == 0)
+      CQ_LAUNCH(gram_start_kernel, dim3(m / 64, m / 64), 256, 0, st, w.Y, m, fro2, mu, w.Cf, Bs[0][0], Bs[0][1], Ys[1][0], Ys[1][1],
+                w.sq + 123, status);
+    const int b = j & 1;
+    tp.nprob = 0;
+    auto add = [&](uint16_t* (*S)[2], float* X) {
+      DenseOut o;
+      o.C0 = X; o.ldc0 = m; o.C = X; o.ldc = m;
+      o.Chi = S[b ^ 1][0]; o.Clo = S[b ^ 1][1];
+      tp.p[tp.nprob] = dense_params(m, m, m, -mu * mu, 2.f * mu, 0.f, o, status, 0);
+      for (int i = 0; i < 2; ++i)
+        if (!make_map_bf16(&maps.a[tp.nprob][i], S[b][i], m, m, m, 128)) return false;
+      ++tp.nprob;
+      return true;
+    };
+    if (j + 1 < GRAM_STEPS && !add(Bs, w.Y)) return CAFEQ_ERR_UNSUPPORTED;
+    if (j > 0 && !add(Ys, w.Cf)) return CAFEQ_ERR_UNSUPPORTED;
+    for (int i = 0; i < 2; ++i)
+      if (!make_map_bf16(&maps.b[i], Bs[b][i], m, m, m, 128)) return CAFEQ_ERR_UNSUPPORTED;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if ((rc = t2_launch(st, maps, tp))) return rc;
+  }
+  return CAFEQ_OK;
+}
+
+// out (hi / lo, shape [R, C] of S) = pinv(S^T) = pinv(S)^T on the wide orientation A of S ([m, n], m <= n), carried as Y = X^T so
+// that every product has both operands contraction-major.
+//   1. X0 = A^T G^-1 with the approximate inverse of the Gram matrix (gram_inverse), as five terms over A split three ways: the
+//      iteration below never corrects what lies outside the row space of A, so X0 must not leave it.
+//   2. Newton-Schulz X <- X + X (I - A X), until ||I - A X||_F falls below 1e-3 (the next update squares it) or stalls, which every
+//      product works out from the residuals itself.  Two updates for the 9B-shaped v-o factors (kappa^2 some thousands) instead of
+//      the sixteen from X0 = A^T / c.
+//   3. One step with the residual over three-way splits.
+// When A X0 is not within 1/2 of I (rank-deficient or very badly conditioned A) the iteration restarts from X0 = A^T / c, c a
+// little above ||A A^T||_F: the eigenvalues of A X0 then lie in [0, 1], and it converges to the Moore-Penrose inverse (stalling at
+// the rank defect).  From there on it is one launch.
+// Error against a float64 pseudo-inverse (512 x 768, kappa^2 4000, emulated products): 1.3e-7; from X0 = A^T / c 7e-6.
 static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, int32_t* status) {
   const bool wide = R <= C;
   const int m = wide ? R : C, n = wide ? C : R;
-  double* fro = w.sq + 120;
+  double* fro2 = w.sq + 120;
+  double* c = w.sq + 123;
   double* rs = w.sq + 32;  // residuals per iteration
+  int rc;
   CQ_LAUNCH(zero_f64_kernel, 1, 128, 0, st, w.sq + 32, DENSE_SQ - 32);
-  CQ_LAUNCH(sqsum_f32_kernel, grid_for((long long)R * C), 256, 0, st, S, (long long)R * C, fro);
-  double* sig2 = w.sq + 123;
+  if (wide) launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status, w.Aw3, nullptr);
+  else launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Awh, w.Awl, status, nullptr, w.Aw3);
+  if ((rc = gram_inverse(st, m, n, w, fro2, status))) return rc;
+  {  // Y = G^-1 A (the rows of A, the contraction, are read as they are stored)
+    const uint16_t* g[2] = {w.CTh, w.CTl};
+    const uint16_t* a[3] = {w.Awh, w.Awl, w.Aw3};
+    const int bn = t2_width(m, n, 1, nullptr);
+    T2Maps maps;
+    T2Params tp;
+    memset(&maps, 0, sizeof(maps));
+    memset(&tp, 0, sizeof(tp));
+    bool ok = true;
+    for (int i = 0; i < 2; ++i) ok = ok && make_map_bf16(&maps.a[0][i], g[i], m, m, m, 128);
+    for (int i = 0; i < 3; ++i) ok = ok && make_map_bf16(&maps.b[i], a[i], n, m, n, 64);
+    if (!ok) return CAFEQ_ERR_UNSUPPORTED;
+    DenseOut o;
+    o.C = w.Y; o.ldc = n;
+    o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[0]; o.Ctlo = w.YTl[0];
+    tp.p[0] = dense_params(m, n, m, 1.f, 0.f, 0.f, o, status, 0);
+    tp.p[0].b_mn = 1;
+    tp.nprob = 1;
+    tp.sh = t2_shape(m, n, bn, 2, 3, 3);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if ((rc = t2_launch(st, maps, tp))) return rc;
+  }
+  const uint16_t* aw[2] = {w.Awh, w.Awl};
+  const uint16_t* ct[2] = {w.CTh, w.CTl};
+  const uint16_t* y[2] = {w.Yh, w.Yl};
+  auto residual = [&](DenseOut& o) { o.Cthi = w.CTh; o.Ctlo = w.CTl; o.sq = rs; o.stop_sq = rs; o.stop_guard = 1; };  // C = I - A X, kept transposed
+  auto update = [&](DenseOut& o, int cur) {                                                      // Y += C^T Y
+    o.C0 = w.Y; o.ldc0 = n; o.C = w.Y; o.ldc = n;
+    o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[cur ^ 1]; o.Ctlo = w.YTl[cur ^ 1];
+    o.stop_sq = rs; o.stop_guard = 1;
+  };
+  constexpr int LAUNCHED = 3;
+  for (int it = 0; it < LAUNCHED; ++it) {
+    const int cur = it & 1;
+    DenseOut o;
+    residual(o);
+    o.sq = rs + it; o.stop_it = it;
+    if ((rc = launch_dense_tc(st, 2, aw, 2, y, m, m, n, -1.f, 0.f, 1.f, o, nullptr, status))) return rc;
+    const uint16_t* yt[2] = {w.YTh[cur], w.YTl[cur]};
+    DenseOut u;
+    update(u, cur);
+    u.stop_it = it;
+    if (it == 0) u.stop_guard = 2;
+    if ((rc = launch_dense_tc(st, 2, ct, 2, yt, m, n, m, 1.f, 1.f, 0.f, u, nullptr, status))) return rc;
+    if (it == 0) {  // the restart: what update 0 would have written
+      if (wide) launch_split_rect(st, S, R, C, C, 1.f, c, w.Y, nullptr, w.Yh, w.Yl, w.YTh[1], w.YTl[1], status, nullptr, nullptr, rs);
+      else launch_split_rect(st, S, R, C, C, 1.f, c, nullptr, w.Y, w.YTh[1], w.YTl[1], w.Yh, w.Yl, status, nullptr, nullptr, rs);
+    }
+  }
   {
-    // power iteration in the (not yet used) iterate buffer: v [3][C], u [R]
-    float* v = w.Y;
-    float* u = w.Y + 3 * (size_t)C;
-    constexpr int ROUNDS = 8;
-    CQ_LAUNCH(pw_init_kernel, (C + 255) / 256, 256, 0, st, v, C);
-    for (int it = 0; it < ROUNDS; ++it) {
-      float* nxt = v + (size_t)((it + 1) % 3) * C;
-      CQ_LAUNCH(pw_rows_kernel, (R + 7) / 8, 256, 0, st, S, v + (size_t)(it % 3) * C, v + (size_t)((it + 2) % 3) * C, R, C, u);
-      CQ_LAUNCH(pw_cols_kernel, dim3((C + 255) / 256, (R + 31) / 32), 256, 0, st, S, u, R, C, nxt);
+    T2LoopMaps maps;
+    T2LoopParams lp;
+    memset(&maps, 0, sizeof(maps));
+    memset(&lp, 0, sizeof(lp));
+    const int bm = t2_width(m, m, 0, nullptr), bn = t2_width(m, n, 0, nullptr);
+    bool ok = true;
+    for (int i = 0; i < 2; ++i) {
+      ok = ok && make_map_bf16(&maps.a[0][i], aw[i], n, m, n, 128) && make_map_bf16(&maps.b[0][i], y[i], n, m, n, bm / 2);
+      ok = ok && make_map_bf16(&maps.a[1][i], ct[i], m, m, m, 128);
+      for (int cur = 0; cur < 2; ++cur) ok = ok && make_map_bf16(&maps.b[1 + cur][i], i ? w.YTl[cur] : w.YTh[cur], m, n, m, bn / 2);
     }
-    CQ_LAUNCH(pw_result_kernel, 1, 256, 0, st, v + (size_t)(ROUNDS % 3) * C, C, 1.25, fro, sig2);
-  }
-  if (wide) {
-    launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status, w.Aw3, nullptr);
-    launch_split_rect(st, S, R, C, C, 1.f, sig2, w.Y, nullptr, w.Yh, w.Yl, w.YTh[0], w.YTl[0], status);
-  } else {
-    launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Awh, w.Awl, status, nullptr, w.Aw3);
-    launch_split_rect(st, S, R, C, C, 1.f, sig2, nullptr, w.Y, w.YTh[0], w.YTl[0], w.Yh, w.Yl, status);
-  }
-  int cur = 0, rc;
-  for (int it = 0; it < PINV_MAX_ITERS; ++it) {
-    {  // C = I - A X, kept transposed
-      const uint16_t* a[3] = {w.Awh, w.Awl, w.Awh};
-      const uint16_t* bb[3] = {w.Yh, w.Yh, w.Yl};
-      DenseOut o;
-      o.Cthi = w.CTh; o.Ctlo = w.CTl; o.sq = rs + it;
-      o.stop_sq = rs; o.stop_it = it;
-      if ((rc = launch_dense_tc(st, 3, a, bb, m, m, n, -1.f, 0.f, 1.f, o, status))) return rc;
+    if (!ok) return CAFEQ_ERR_UNSUPPORTED;
+    for (int cur = 0; cur < 2; ++cur) {
+      DenseOut o, u;
+      residual(o);
+      update(u, cur);
+      lp.p[0][cur] = dense_params(m, m, n, -1.f, 0.f, 1.f, o, status, 0);
+      lp.p[1][cur] = dense_params(m, n, m, 1.f, 1.f, 0.f, u, status, 0);
     }
-    {  // Y += C^T Y
-      const uint16_t* a[3] = {w.CTh, w.CTl, w.CTh};
-      const uint16_t* bb[3] = {w.YTh[cur], w.YTh[cur], w.YTl[cur]};
-      DenseOut o;
-      o.C0 = w.Y; o.ldc0 = n; o.C = w.Y; o.ldc = n;
-      o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[cur ^ 1]; o.Ctlo = w.YTl[cur ^ 1];
-      o.stop_sq = rs; o.stop_it = it;
-      if ((rc = launch_dense_tc(st, 3, a, bb, m, n, m, 1.f, 1.f, 0.f, o, status))) return rc;
-    }
-    cur ^= 1;
+    lp.sh[0] = t2_shape(m, m, bm, 2, 2, 2);
+    lp.sh[1] = t2_shape(m, n, bn, 2, 2, 2);
+    lp.it0 = LAUNCHED; lp.it1 = PINV_MAX_ITERS;
+    lp.arrived = reinterpret_cast<uint32_t*>(w.sq + 124);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if ((rc = pinv_loop_launch(st, maps, lp))) return rc;
   }
   // The loop above stops at the accuracy of its three-term products (residual entries of a few 1e-7).  One more
   // step with the residual evaluated over three-way splits (fp32-grade) squares what is left: the quantised targets
@@ -202,12 +330,12 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     const uint16_t* bb[3] = {w.Yh, w.Yl, w.Y3};
     DenseOut o;
     o.Cthi = w.CTh; o.Ctlo = w.CTl;
-    if ((rc = launch_dense_tc6(st, a, bb, m, m, n, -1.f, 0.f, 1.f, o, w.Cf, status))) return rc;
-    const uint16_t* a2[3] = {w.CTh, w.CTl, w.CTh};
-    const uint16_t* b2[3] = {w.YTh[0], w.YTh[0], w.YTl[0]};
+    if ((rc = launch_dense_tc(st, 3, a, 3, bb, m, m, n, -1.f, 0.f, 1.f, o, w.Cf, status))) return rc;
+    const uint16_t* a2[2] = {w.CTh, w.CTl};
+    const uint16_t* b2[2] = {w.YTh[0], w.YTl[0]};
     DenseOut o2;
     o2.C0 = w.Y; o2.ldc0 = n; o2.C = w.Y; o2.ldc = n;
-    if ((rc = launch_dense_tc(st, 3, a2, b2, m, n, m, 1.f, 1.f, 0.f, o2, status))) return rc;
+    if ((rc = launch_dense_tc(st, 2, a2, 2, b2, m, n, m, 1.f, 1.f, 0.f, o2, nullptr, status))) return rc;
   }
   if (wide) launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, w.Oh, w.Ol, nullptr, nullptr, status, w.O3, nullptr);
   else launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Oh, w.Ol, status, nullptr, w.O3);
@@ -240,7 +368,7 @@ static int dense_product(cudaStream_t st, const float* U, const float* V, DenseW
   const uint16_t* b[3] = {w.Vh, w.Vl, w.V3};
   DenseOut o;
   o.C = P; o.ldc = w.d3; o.Chi = w.Ph; o.Clo = w.Pl; o.Cthi = w.PTh; o.Ctlo = w.PTl;
-  const int rc = launch_dense_tc6(st, a, b, w.d1, w.d3, w.h, 1.f, 0.f, 0.f, o, P, status);
+  const int rc = launch_dense_tc(st, 3, a, 3, b, w.d1, w.d3, w.h, 1.f, 0.f, 0.f, o, P, status);
   if (rc) return rc;
   launch_split_rect(st, P, w.d1, w.d3, w.d3, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, status, w.P3, w.PT3);
   return CAFEQ_OK;
@@ -253,14 +381,14 @@ static int dense_pqe(cudaStream_t st, const float* Uhat, const float* Vhat, cons
   launch_split_rect(st, Uhat, w.h, w.d1, w.d1, 1.f, nullptr, nullptr, nullptr, keep_splits ? w.Awh : nullptr,
                     keep_splits ? w.Awl : nullptr, w.UTh, w.UTl, status);
   launch_fold_split(st, Vhat, w, w.Vh, w.Vl, nullptr, status);
-  const uint16_t* a[3] = {w.UTl, w.UTh, w.UTh};  // (the small terms first, as in P)
-  const uint16_t* b[3] = {w.Vh, w.Vl, w.Vh};
+  const uint16_t* a[2] = {w.UTh, w.UTl};
+  const uint16_t* b[2] = {w.Vh, w.Vl};
   DenseOut o;
   o.C0 = P; o.ldc0 = w.d3; o.C = R; o.ldc = w.d3; o.sq = sq;
   if (keep_splits) {  // the residual and its transpose as operands of the backward products
     o.Chi = w.Ph; o.Clo = w.Pl; o.Cthi = w.PTh; o.Ctlo = w.PTl;
   }
-  return launch_dense_tc(st, 3, a, b, w.d1, w.d3, w.h, 1.f, -1.f, 0.f, o, status);
+  return launch_dense_tc(st, 2, a, 2, b, w.d1, w.d3, w.h, 1.f, -1.f, 0.f, o, nullptr, status);
 }
 
 // Algorithm 1 on the transformed pair held in w.U [h, d1], w.V [d3, rh] (fp32, stored layout with r replicas of
@@ -283,7 +411,7 @@ static int alg1_run(cudaStream_t st, int bits, int g1, int g2, int iters, int8_t
       const uint16_t* b[3] = {w.Oh, w.Ol, w.O3};
       DenseOut o;
       o.C = w.X0T; o.ldc = w.h;
-      if ((rc = launch_dense_tc6(st, a, b, w.d3, w.h, w.d1, 1.f, 0.f, 0.f, o, w.X0T, status))) return rc;
+      if ((rc = launch_dense_tc(st, 3, a, 3, b, w.d3, w.h, w.d1, 1.f, 0.f, 0.f, o, w.X0T, status))) return rc;
     }
     CQ_LAUNCH(expand_cols_kernel, dim3(w.d3, (w.h + 1023) / 1024), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f / (float)w.r, w.V);
     quant_matrix(st, w.V, w.d3, w.rh, g2, bits, codes2, scales2, w.Vhat, w, status);
@@ -299,7 +427,7 @@ static int alg1_run(cudaStream_t st, int bits, int g1, int g2, int iters, int8_t
       const uint16_t* b[3] = {w.Ph, w.Pl, w.P3};
       DenseOut o;
       o.C = w.U; o.ldc = w.d1;
-      if ((rc = launch_dense_tc6(st, a, b, w.h, w.d1, w.d3, 1.f, 0.f, 0.f, o, w.U, status))) return rc;
+      if ((rc = launch_dense_tc(st, 3, a, 3, b, w.h, w.d1, w.d3, 1.f, 0.f, 0.f, o, w.U, status))) return rc;
     }
     quant_matrix(st, w.U, w.h, w.d1, g1, bits, codes1, scales1, w.Uhat, w, status);
     if ((rc = dense_pqe(st, w.Uhat, w.Vhat, w.P, w, w.sq + 2 * it + 2, nullptr, status))) return rc;

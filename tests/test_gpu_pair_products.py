@@ -1,0 +1,89 @@
+"""Dense products on CTA pairs (tiles of 256 rows, up to 256 columns, chosen by size) and the pseudo-inverse built from them, at
+sizes where tiles end inside the matrix, against float64."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _weights(h, d1, d3, r, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    W1 = torch.randn((h, d1), generator=g, device="cuda") / d1 ** 0.5
+    W2 = torch.randn((d3, r * h), generator=g, device="cuda") / (r * h) ** 0.5
+    W1[:, :: max(1, d1 // 3)] *= 15.0
+    return W1.bfloat16(), W2.bfloat16()
+
+
+def _fold(X, h, k, r):
+    return X.reshape(X.shape[0], h // k, r, k).sum(2).reshape(X.shape[0], h)
+
+
+# one tile; edges inside a tile in both directions; a single row tile; several waves of 74 pairs; replicas
+@pytest.mark.parametrize("h,d1,d3,k,r", [(64, 256, 256, 64, 1), (192, 832, 1088, 64, 1), (256, 2368, 192, 128, 2), (320, 4544, 4160, 64, 1),
+                                         (1024, 2048, 2304, 256, 2)])
+def test_product_against_float64(h, d1, d3, k, r):
+    import paper_2511_19705_b200 as cq
+    W1, W2 = _weights(h, d1, d3, r, 3)
+    P = cq.cafeq_pair_product(W1, W2, k=k, replicas=r).reshape(d1, d3).double()
+    ref = W1.double().t() @ _fold(W2.double(), h, k, r).t()
+    # fp32 accumulation of h terms: rounding steps of 2^-24 at the accumulator's size add like a walk, sqrt(h) of them at most
+    assert ((P - ref).norm() / ref.norm()).item() <= 2.0 ** -24 * h ** 0.5 * 2
+
+
+def _quant(T, g, bits):
+    qm = 2 ** (bits - 1) - 1
+    x = T.float().reshape(T.shape[0], -1, g)
+    a = x.abs().amax(-1, keepdim=True)
+    s = a / torch.full_like(a, qm)
+    q = torch.round(x / torch.where(s > 0, s, torch.ones_like(s))).clamp(-qm, qm)
+    return q, s, (q * s).reshape(T.shape).double()
+
+
+# full rank; one row tile of 64; the inner dimension above the outer ones (tall factor); repeated rows and a zero row (the start
+# from the Gram matrix is not usable and the iteration restarts)
+@pytest.mark.parametrize("h,d1,d3,k,case", [(512, 832, 768, 128, "full"), (64, 192, 256, 64, "full"), (640, 384, 448, 64, "tall"),
+                                            (512, 768, 896, 128, "repeated"), (256, 512, 448, 64, "zero")])
+def test_first_half_step_against_float64(h, d1, d3, k, case):
+    import paper_2511_19705_b200 as cq
+    bits, g = 4, 64
+    W1, W2 = _weights(h, d1, d3, 1, 5)
+    if case == "repeated":
+        W1[:3] = W1[k:k + 3]
+    if case == "zero":
+        W1[7] = 0
+    M = torch.eye(k, device="cuda").repeat(h // k, 1, 1)
+    o = cq.cafeq_adaptive_round(W1, W2, M, iters=1, bits=bits, group1=g, group2=g)
+    assert int(o["status"].item()) in ((0, 6) if case == "tall" else (0,))  # (tall: the second half-step is rank-deficient)
+    U, V = W1.double(), W2.double()
+    _, _, Uh = _quant(U, g, bits)
+    pinv = torch.linalg.pinv(Uh.t(), rtol=1e-10)
+    q, s, _ = _quant((pinv @ (U.t() @ V.t())).t(), g, bits)
+    s2 = o["scales2"].double().reshape(s.shape[:2])
+    # targets carry the condition of Uhat (tens) times 2^-24 sqrt(terms); a code may turn at a rounding tie of that width
+    assert ((s2 - s[..., 0]).norm() / s.norm()).item() <= 3e-5
+    assert (o["codes2"].double().reshape(q.shape) != q).double().mean().item() <= 1e-4
+
+
+def test_same_codes_under_capture():
+    import paper_2511_19705_b200 as cq
+    h, d1, d3, k = 256, 512, 448, 64
+    W1, W2 = _weights(h, d1, d3, 1, 9)
+    M = torch.eye(k, device="cuda").repeat(h // k, 1, 1)
+
+    def call():
+        return cq.cafeq_adaptive_round(W1, W2, M, iters=1, bits=4, group1=64, group2=64)
+
+    want = call()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        call()
+    torch.cuda.current_stream().wait_stream(s)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = call()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(got["codes1"], want["codes1"]) and torch.equal(got["codes2"], want["codes2"])
+    del graph
