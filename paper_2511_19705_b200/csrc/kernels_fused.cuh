@@ -6,6 +6,7 @@
 // X through a TMA ring; accumulators are double-buffered in tensor memory so the epilogue of tile t overlaps
 // the products of tile t+1.
 //
+// Blocks of 256 run on pairs of CTAs (cta_group::2, BdCfg below): the leader issues products of 256 rows for both.
 // Warp roles (576 threads): warp 0 = TMA producer, warp 1 = MMA issuer (and tensor-memory owner), warps 2..9 and 10..17 =
 // two epilogue sets, one per accumulator buffer (two warps per 32-lane quarter, each owning 128 accumulator columns).
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises CAFEQ_ERR_TIMEOUT in the status
@@ -21,7 +22,7 @@
 #include <stdint.h>
 
 #include "cafeq.h"
-#include "kernels_generic.cuh"
+#include "kernels_pair_mma.cuh"
 
 namespace cafeq {
 
@@ -76,246 +77,38 @@ struct BdMulti {
 };
 
 constexpr int BD_THREADS = 64 + 2 * 256;
-constexpr int BD_STAGE_BYTES = 16384;  // one TMA box: 64 columns x 128 rows of bf16
-constexpr int BD_STAGES_PER_TILE = 4;
-constexpr uint64_t BD_WAIT_NS = 2000000000ull;
-
-// ------------------------------------------------------------------------------------------------
-// PTX wrappers
-// ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok;
-}
-__device__ __forceinline__ uint64_t global_timer_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait: false when the limit ran out here or in another role (abort flag).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
-                                          uint64_t limit_ns = BD_WAIT_NS) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
-  for (uint32_t spin = 0;; ++spin) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((spin & 63u) == 63u) {
-      if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > limit_ns) {
-        *abort_flag = 1;
-        raise_status(status, CAFEQ_ERR_TIMEOUT);
-        return false;
-      }
-      __nanosleep(32);
-    }
-  }
-}
-
-// Self-test of the bounded wait: one thread waits, with the given limit, on a barrier phase that nobody completes
-// (expected: the wait gives up, raises CAFEQ_ERR_TIMEOUT and sets the abort flag), then completes that phase itself
-// and waits again (expected: success).  result[0] = 1 when the first wait gave up, result[1] = 1 when the second
-// succeeded.  Nothing here can block: both waits are bounded and the only arrival is the thread's own.
-__global__ void wait_probe_kernel(uint64_t limit_ns, int32_t* status, int* result) {
-  pdl_enter();
-  __shared__ uint64_t bar;
-  __shared__ int abort_flag;
-  if (threadIdx.x == 0) {
-    abort_flag = 0;
-    mbar_init(smem_u32(&bar), 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    const bool first = mbar_wait(smem_u32(&bar), 0, &abort_flag, status, limit_ns);
-    result[0] = first ? 0 : 1;
-    abort_flag = 0;
-    mbar_arrive(smem_u32(&bar));
-    const bool second = mbar_wait(smem_u32(&bar), 0, &abort_flag, nullptr, 1000000000ull);
-    result[1] = second ? 1 : 0;
-  }
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(map), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// the same with an L2 policy: evict_first for data that is read once per step, so that it does not displace what is reused
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-  uint64_t pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-  return pol;
-}
-__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
-      "l"(map), "r"(x), "r"(y), "r"(bar), "l"(pol)
-      : "memory");
-}
-
-__device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// one converged warp releases the tensor memory that it allocated
-__device__ __forceinline__ void tmem_free(uint32_t base, uint32_t cols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
-}
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// The same product with the operand descriptors given by their low words (umma_desc_lo; the high word is the same for
-// every operand of this library): stepping through a tile is one 32-bit addition per operand.
-constexpr uint32_t UMMA_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);  // stride 1024 B, version, SWIZZLE_128B
-__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr, uint32_t lbo_bytes = 16) {
-  return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16);
-}
-__device__ __forceinline__ void tc_mma_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-      "mov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}" ::"r"(tmem_d),
-      "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(UMMA_DESC_HI)
-      : "memory");
-}
-// one lane of a converged warp (a warp-uniform branch: the operands of the products inside stay in uniform registers)
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// 16 columns
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// 32 bytes per lane: one whole sector (the lanes' rows are far apart in memory, so narrower stores are partial sectors).
-// Bases that are not 32-byte aligned take 16-byte pieces.
-__device__ __forceinline__ void store32(void* dst, const uint32_t* v, bool wide) {
-  if (wide) {
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
-                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                 : "memory");
-  } else {
-    uint4* d = reinterpret_cast<uint4*>(dst);
-    d[0] = make_uint4(v[0], v[1], v[2], v[3]);
-    d[1] = make_uint4(v[4], v[5], v[6], v[7]);
-  }
-}
-
-// max of m, |a| and |b|; a NaN stays
-__device__ __forceinline__ float max_abs2(float m, float a, float b) {
-  float r;
-  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(a), "f"(b));
-  return r;
-}
-
-// Shared-memory matrix descriptor, 128-byte swizzle, rows of 128 bytes, 8-row groups 1024 bytes apart.
-// K-major operands step along K by moving the start address inside the swizzled row; MN-major operands
-// step along K by whole 8-row groups.
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;              // leading byte offset (unused: one swizzle chunk along the leading dim)
-  d |= (uint64_t)(1024 >> 4) << 32;    // stride byte offset: next 8-row group
-  d |= (uint64_t)1 << 46;              // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;              // SWIZZLE_128B
-  return d;
-}
-
-// Same, for an MN-major operand that spans several 64-element swizzle atoms along MN: `lbo_bytes` is the distance
-// between consecutive atoms.
-__device__ __forceinline__ uint64_t umma_desc_sw128_lbo(uint32_t saddr, uint32_t lbo_bytes) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N, int a_mn_major, int b_mn_major) {
-  return (1u << 4) /* fp32 accumulate */ | (1u << 7) /* A bf16 */ | (1u << 10) /* B bf16 */ |
-         ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
-}
+constexpr int BD_BOX_BYTES = 16384;  // one TMA box: 64 columns x 128 rows of bf16
+// A stage is two boxes: every wait of the issuing warp costs it some 400 cycles, and the four products of one box last 512.
+constexpr int BD_STAGE_BYTES = 2 * BD_BOX_BYTES;
+constexpr int BD_STAGES_PER_TILE = 2;
 
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
 template <int FORM, int K, int G>
 struct BdCfg {
+  // K = 256: CTA pairs (cta_group::2).  A tile is 256 rows x 256 columns; each CTA holds half of the operator block (its 128 rows:
+  // on the input axis the N half, on the output axis its accumulator rows) and half of the tile (input axis: its 128 rows; output
+  // axis: its 128 columns), and its 128 rows of the accumulator.
+  static constexpr bool PAIR = K == 256;
+  static constexpr int ROWS = PAIR ? 256 : 128;                       // IN: rows per tile
   static constexpr int NBLK = (FORM == BD_IN) ? 256 / K : 1;          // operator blocks resident per CTA
-  static constexpr int T_BYTES = NBLK * K * K * 2;
-  static constexpr int KH = (K >= 128) ? K / 128 : 1;                 // OUT: 128-row halves of the block
-  static constexpr int NC = 256 / KH;                                 // OUT: d_in columns per tile
-  static constexpr int NCC = NC / 64;                                 // OUT: 64-column chunks per tile
-  // as many stages as fit (even: the output-axis form consumes stages in pairs)
-  static constexpr int NSTAGE = (T_BYTES > 65536) ? 6 : ((T_BYTES > 32768) ? 10 : 12);
+  static constexpr int T_BYTES = PAIR ? K * K : NBLK * K * K * 2;
+  static constexpr int NC = 256;                                      // OUT: d_in columns per tile
+  static constexpr int NSTAGE = (T_BYTES > 65536) ? 3 : ((T_BYTES > 32768) ? 5 : 6);  // as many as fit
   static constexpr int SMEM = 1024 + T_BYTES + NSTAGE * BD_STAGE_BYTES + 256;
 };
 
 // The body takes the CTA's index and the number of CTAs that share its tile list, so that one launch can run two
-// lists side by side (bd_pass_dual_kernel below).
+// lists side by side (bd_pass_dual_kernel below); at K = 256 these are pairs.
 template <int FORM, int K, int G, int MODE>
 __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& mp, const int cta, const int ncta) {
   using C = BdCfg<FORM, K, G>;
   static_assert(K == 64 || K == 128 || K == 256, "block size");
   static_assert(FORM == BD_IN || K >= 128, "output-axis form needs k >= 128");
   static_assert(G == 64 || G == 128, "group size");
+  constexpr bool PAIR = C::PAIR;
+  const uint32_t rank = PAIR ? cluster_rank() : 0u;
   int32_t* const status = mp.p[0].status;
   const bool raised = status_raised(status);  // (awaited at the end of the set-up)
 
@@ -357,22 +150,32 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
     mbar_init(bar_tfree, 1);
     mbar_init(bar_accf, 1);
     mbar_init(bar_accf + 8, 1);
-    mbar_init(bar_acce, 8);
-    mbar_init(bar_acce + 8, 8);
+    mbar_init(bar_acce, PAIR ? 16 : 8);
+    mbar_init(bar_acce + 8, PAIR ? 16 : 8);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      tmem_alloc_pair(smem_u32(tmem_slot), 512u);
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
-  const bool stopped = __syncthreads_or(raised) != 0;
+  bool stopped;
+  if constexpr (PAIR) stopped = pair_stopped(raised, tmem_slot + 2);
+  else stopped = __syncthreads_or(raised) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  auto free_tmem = [&]() {
+    if constexpr (PAIR) tmem_free_pair(tmem_base, 512u);
+    else tmem_free(tmem_base, 512u);
+  };
   if (stopped) {
-    if (warp == 1) tmem_free(tmem_base, 512u);
+    if (warp == 1) free_tmem();
     return;
   }
 
@@ -382,6 +185,23 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
       uint32_t it = 0, tloads = 0;
       bool ok = true;
       const uint64_t pol = l2_evict_first_policy();
+      // (the leader's barriers count the loads of both CTAs)
+      auto arm = [&](uint32_t bar, uint32_t bytes) {
+        if constexpr (PAIR) {
+          if (rank == 0) mbar_expect_tx(bar, 2 * bytes);
+        } else {
+          mbar_expect_tx(bar, bytes);
+        }
+      };
+      auto load = [&](uint32_t dst, const CUtensorMap* m, int x, int y, uint32_t bar, bool hint) {
+        if constexpr (PAIR) {
+          if (hint) tma_load_pair_hint(dst, m, x, y, cluster_addr(bar, 0), pol);
+          else tma_load_pair(dst, m, x, y, cluster_addr(bar, 0));
+        } else {
+          if (hint) tma_load_2d_hint(dst, m, x, y, bar, pol);
+          else tma_load_2d(dst, m, x, y, bar);
+        }
+      };
       for (int sub = s_first; sub < mp.n && ok; ++sub) {
         const int base = sub ? mp.tile_end[sub - 1] : 0;
         if (base >= t_end) break;
@@ -396,17 +216,18 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
           if (major != cur_major) {
             // the products of the previous operator block must have finished reading it
             if (tloads > 0 && !mbar_wait(bar_tfree, (tloads - 1) & 1u, abort_flag, status)) { ok = false; break; }
+            constexpr int TR = PAIR ? 128 : K;  // operator rows (columns, stored transposed) of this CTA
             for (int bi = 0; bi < C::NBLK; ++bi) {
               const int tb = (FORM == BD_IN) ? (major * C::NBLK + bi) / p.r : major / p.r;
               for (int ci = 0; ci < K / 64; ++ci) {
                 const uint32_t bq = bar_tfull + 8 * (bi * (K / 64) + ci);  // at most four chunks: NBLK * K = 256 or NBLK = 1
-                mbar_expect_tx(bq, K * 128);
-                const uint32_t dst = smem_u32(sT + bi * K * K * 2 + ci * K * 128);
+                arm(bq, TR * 128);
+                const uint32_t dst = smem_u32(sT + bi * TR * K * 2 + ci * TR * 128);
                 if (FORM == BD_OUT && p.t_mn) {
-                  // 64 contraction rows x K columns as boxes of 64 x 64 (one swizzle atom each)
-                  for (int j = 0; j < K / 64; ++j) tma_load_2d(dst + j * 8192, tmT, j * 64, tb * K + ci * 64, bq);
+                  // 64 contraction rows x TR columns as boxes of 64 x 64 (one swizzle atom each)
+                  for (int j = 0; j < TR / 64; ++j) load(dst + j * 8192, tmT, (int)rank * 128 + j * 64, tb * K + ci * 64, bq, false);
                 } else {
-                  tma_load_2d(dst, tmT, ci * 64, tb * K, bq);
+                  load(dst, tmT, ci * 64, tb * K + (int)rank * 128, bq, false);
                 }
               }
             }
@@ -416,18 +237,23 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
           for (int sidx = 0; sidx < BD_STAGES_PER_TILE; ++sidx, ++it) {
             const uint32_t s = it % C::NSTAGE, ph = (it / C::NSTAGE) & 1u;
             if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, status)) { ok = false; break; }
-            mbar_expect_tx(bar_full + 8 * s, BD_STAGE_BYTES);
-            int x, y;
-            if constexpr (FORM == BD_IN) {
-              x = major * 256 + sidx * 64;
-              y = t * 128;
-            } else {
-              const int kh = sidx / C::NCC, nc = sidx % C::NCC;  // the chunks of one row half are consecutive stages
-              x = t * C::NC + nc * 64;
-              y = major * K + kh * 128;
+            arm(bar_full + 8 * s, BD_STAGE_BYTES);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int bx = 2 * sidx + h;
+              int x, y;
+              if constexpr (FORM == BD_IN) {
+                x = major * 256 + bx * 64;
+                y = t * C::ROWS + (int)rank * 128;
+              } else if constexpr (PAIR) {  // stage = 128 contraction rows x this CTA's 128 columns
+                x = t * C::NC + (int)rank * 128 + h * 64;
+                y = major * K + sidx * 128;
+              } else {
+                x = t * C::NC + bx * 64;
+                y = major * K;
+              }
+              load(smem_u32(sStage + s * BD_STAGE_BYTES + h * BD_BOX_BYTES), tmX, x, y, bar_full + 8 * s, mp.stream != 0);
             }
-            if (mp.stream) tma_load_2d_hint(smem_u32(sStage + s * BD_STAGE_BYTES), tmX, x, y, bar_full + 8 * s, pol);
-            else tma_load_2d(smem_u32(sStage + s * BD_STAGE_BYTES), tmX, x, y, bar_full + 8 * s);
           }
         }
       }
@@ -437,10 +263,15 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
     // The whole warp runs the loop and one elected lane issues (operands in uniform registers, descriptors stepped by one
     // 32-bit addition): beside the epilogue warps a single lane that builds 64-bit descriptors took 240 cycles per
     // instruction against the 128 that a 128 x 256 x 16 product lasts.
-    {
+    if (rank == 0) {  // (of a pair, the leader)
       bool ok = true;
+      auto commit = [&](uint32_t bar) {
+        if constexpr (PAIR) tc_commit_pair(bar);
+        else tc_commit(bar);
+      };
       uint32_t tfulls = 0;
-      constexpr uint32_t idesc_in = umma_idesc_bf16(128, K, 0, 0);
+      constexpr int MR = PAIR ? 256 : 128;  // accumulator rows of a product
+      constexpr uint32_t idesc_in = umma_idesc_bf16(MR, K, 0, 0);
       const uint32_t sSt_u = smem_u32(sStage);
       const uint32_t tlo = umma_desc_lo(smem_u32(sT));
       uint32_t st = 0, sph = 0, tl = 0;  // stage, its phase, tile
@@ -452,7 +283,8 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
         const int n_minor = mp.p[sub].n_minor;
         const bool t_mn = FORM == BD_OUT && mp.p[sub].t_mn;
         const bool pairs = FORM == BD_IN && K == 64 && mp.p[sub].pairs;
-        const uint32_t idesc_out = t_mn ? umma_idesc_bf16(128, 128, 1, 1) : umma_idesc_bf16(128, 128, 0, 1);
+        constexpr int NO = PAIR ? 256 : 128;
+        const uint32_t idesc_out = t_mn ? umma_idesc_bf16(MR, NO, 1, 1) : umma_idesc_bf16(MR, NO, 0, 1);
         const int lo = (t_begin > base ? t_begin : base) - base;
         const int hi = (t_end < mp.tile_end[sub] ? t_end : mp.tile_end[sub]) - base;
         int left = 0;  // tiles of this sub-problem left on the current operator block
@@ -476,62 +308,66 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
 #pragma unroll
             for (int sidx = 0; sidx < BD_STAGES_PER_TILE; ++sidx) {
               ok = wait_all(bar_full + 8 * st, sph);
-              // stage sidx multiplies the operator's chunk sidx
-              if (ok && fresh) ok = wait_all(bar_tfull + 8 * sidx, tph);
+              // box bx multiplies the operator's chunk bx
+              if (ok && fresh) ok = wait_all(bar_tfull + 16 * sidx, tph) && wait_all(bar_tfull + 16 * sidx + 8, tph);
               if (!ok) break;
               tc_fence_after();
-              const int bi = (sidx * 64) / K, ci = ((sidx * 64) % K) / 64;
               if (elect_one()) {
-                const uint32_t alo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES);
-                const uint32_t blo = tlo + ((bi * K * K * 2 + ci * K * 128) >> 4);
-                if (K == 64 && pairs) {
-                  // Each 32 columns meet their own block only, the diagonal quarter of the operator tile (rows 32 half ..).  The
-                  // whole tile would add products with zeros: exact, but an infinity or NaN times zero is NaN.
 #pragma unroll
-                  for (int kk = 0; kk < 4; ++kk)
-                    tc_mma_lo(dbase + bi * K + (kk >> 1) * 32, alo + 2 * kk, blo + (kk >> 1) * 256 + 2 * kk, umma_idesc_bf16(128, 32, 0, 0), kk & 1);
-                } else {
+                for (int h = 0; h < 2; ++h) {
+                  const int bx = 2 * sidx + h, bi = (bx * 64) / K, ci = ((bx * 64) % K) / 64;
+                  const uint32_t alo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES + h * BD_BOX_BYTES);
+                  const uint32_t blo = tlo + (PAIR ? bx * 1024 : ((bi * K * K * 2 + ci * K * 128) >> 4));
+                  if constexpr (PAIR) {
 #pragma unroll
-                  for (int kk = 0; kk < 4; ++kk) tc_mma_lo(dbase + bi * K, alo + 2 * kk, blo + 2 * kk, idesc_in, (ci | kk) != 0 ? 1u : 0u);
+                    for (int kk = 0; kk < 4; ++kk) tc_mma_pair(dbase, alo + 2 * kk, blo + 2 * kk, idesc_in, (bx | kk) != 0 ? 1u : 0u);
+                  } else if (K == 64 && pairs) {
+                    // Each 32 columns meet their own block only, the diagonal quarter of the operator tile (rows 32 half ..).  The
+                    // whole tile would add products with zeros: exact, but an infinity or NaN times zero is NaN.
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                      tc_mma_lo(dbase + bi * K + (kk >> 1) * 32, alo + 2 * kk, blo + (kk >> 1) * 256 + 2 * kk, umma_idesc_bf16(128, 32, 0, 0), kk & 1);
+                  } else {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) tc_mma_lo(dbase + bi * K, alo + 2 * kk, blo + 2 * kk, idesc_in, (ci | kk) != 0 ? 1u : 0u);
+                  }
                 }
-                tc_commit(bar_empty + 8 * st);
-                if (sidx == BD_STAGES_PER_TILE - 1) tc_commit(bar_accf + 8 * buf);
+                commit(bar_empty + 8 * st);
+                if (sidx == BD_STAGES_PER_TILE - 1) commit(bar_accf + 8 * buf);
               }
               __syncwarp();
               next();
             }
           } else {
-            // two consecutive stages = two 64-column chunks of the same 128 weight rows: one N = 128 product, the
-            // second swizzle atom of the MN-major operand one stage further on
+            // a stage = two 64-column chunks of the same 128 weight rows: one product of N = 128 (of a pair, each CTA's half of
+            // N = 256), the second swizzle atom of the MN-major operand one box further on
 #pragma unroll
-            for (int sidx = 0; sidx < BD_STAGES_PER_TILE; sidx += 2) {
-              ok = wait_all(bar_full + 8 * st, sph) && wait_all(bar_full + 8 * (st + 1), sph);
+            for (int sidx = 0; sidx < BD_STAGES_PER_TILE; ++sidx) {
+              ok = wait_all(bar_full + 8 * st, sph);
               if (!ok) break;
               tc_fence_after();
-              const int kh = sidx / C::NCC, nc = sidx % C::NCC;
               if (elect_one()) {
-                const uint32_t blo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES, BD_STAGE_BYTES);
+                const uint32_t blo = umma_desc_lo(sSt_u + st * BD_STAGE_BYTES, BD_BOX_BYTES);
                 // K-major operator: steps of 32 bytes inside the swizzled rows; MN-major: steps of sixteen 128-byte rows
-                const uint32_t alo = (t_mn ? umma_desc_lo(smem_u32(sT), 8192) : tlo) + ((kh * 2 * K * 128) >> 4);
+                const uint32_t alo = t_mn ? umma_desc_lo(smem_u32(sT), 8192) : tlo;
                 const uint32_t astep = t_mn ? 128 : 2;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-#pragma unroll
-                  for (int mh = 0; mh < C::KH; ++mh)
-                    tc_mma_lo(dbase + mh * C::NC + nc * 64, alo + (((ks / 4) * K * 128 + mh * 128 * 128) >> 4) + (ks % 4) * astep,
-                              blo + ks * 128, idesc_out, (kh | ks) != 0 ? 1u : 0u);
-                tc_commit(bar_empty + 8 * st);
-                tc_commit(bar_empty + 8 * (st + 1));
-                if (sidx == BD_STAGES_PER_TILE - 2) tc_commit(bar_accf + 8 * buf);
+                for (int ks = 0; ks < 8; ++ks) {
+                  if constexpr (PAIR)
+                    tc_mma_pair(dbase, alo + (2 * sidx + ks / 4) * 1024 + (ks % 4) * astep, blo + ks * 128, idesc_out, (sidx | ks) != 0 ? 1u : 0u);
+                  else
+                    tc_mma_lo(dbase + sidx * 128, alo + (ks / 4) * 1024 + (ks % 4) * astep, blo + ks * 128, idesc_out, ks != 0 ? 1u : 0u);
+                }
+                commit(bar_empty + 8 * st);
+                if (sidx == BD_STAGES_PER_TILE - 1) commit(bar_accf + 8 * buf);
               }
               __syncwarp();
-              next();
               next();
             }
           }
           // last tile of this operator block with more to come: signal when its products are done with the block
           if (--left == 0 || tile + 1 == hi) {
-            if (ok && base + tile + 1 < t_end && elect_one()) tc_commit(bar_tfree);
+            if (ok && base + tile + 1 < t_end && elect_one()) commit(bar_tfree);
             __syncwarp();
           }
         }
@@ -545,8 +381,9 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
     // against 2100 for the products and 2800 for the bytes).  Measured, one set -> two: records of a 9B-shaped layer (both
     // forms, 198 M weights) 127 -> 111 us, 27B-shaped with groups of 64 (515 M) 325 -> 286; codes of 14336 x 3584 86 -> 50;
     // the transformed matrix of 8192 x 2304 29.5 -> 20.5 (with its stores widened to whole sectors).
-    // What bounds the records now is the products themselves: operands, 12 KB per 128 x 256 x 16 product, and the arriving
-    // weights share the 128 bytes per cycle of shared memory, so a product takes 187 cycles instead of 128.
+    // Since then, records of the same layer, back to back: 105 us; arg-max by chunks and loads in flight 95 (without an epilogue 86,
+    // without loads 94, with a quarter of the products 94), stages of two boxes 93, blocks of 256 on CTA pairs 89.  There the
+    // products (2048 cycles a tile at K = 256) take 84 % of a CTA's time, at the clock that the power limit leaves.
     const int q = warp & 3, hw = ((warp - 2) >> 2) & 1;
     const uint32_t buf = (uint32_t)((warp - 2) >> 3);
     const int L = q * 32 + lane;
@@ -591,14 +428,11 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
         if ((tl & 1u) != buf) continue;
         int row, col0;
         if constexpr (FORM == BD_IN) {
-          row = t * 128 + L;
+          row = t * C::ROWS + (int)rank * 128 + L;
           col0 = major * 256 + hw * 128;
-        } else if constexpr (K == 256) {
-          row = major * 256 + hw * 128 + L;
-          col0 = t * 128;
         } else {
-          row = major * 128 + L;
-          col0 = t * 256 + hw * 128;
+          row = major * K + (int)rank * 128 + L;
+          col0 = t * C::NC + hw * 128;
         }
         const bool valid = (row < p.d_out) && (col0 < p.d_in);
         // Eq. 4 weights of this thread's groups, requested before the wait for the accumulator so that the
@@ -619,38 +453,47 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
         auto release = [&]() {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_acce + 8 * buf);
+          if (lane == 0) {
+            if constexpr (PAIR) mbar_arrive_cluster(cluster_addr(bar_acce + 8 * buf, 0));
+            else mbar_arrive(bar_acce + 8 * buf);
+          }
+        };
+        // This thread's 128 columns, 16 at a time, the next 16 requested while these are worked on (unrolled: a copy of the registers
+        // in flight would read them too early).
+        auto walk = [&](auto&& f) {
+          uint32_t raw[2][16];
+          tc_ld16_async(taddr, raw[0]);
+#pragma unroll
+          for (int ch = 0; ch < 8; ++ch) {
+            tc_ld16_wait(raw[ch & 1]);
+            if (ch < 7) tc_ld16_async(taddr + (ch + 1) * 16, raw[(ch + 1) & 1]);
+            float v[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(raw[ch & 1][e]);
+            f(ch, v);
+          }
         };
         if constexpr (MODE == BD_STORE) {
           // the transformed matrix itself, rounded to bf16 (inference-side apply of a block-diagonal operator)
           uint16_t* dst = p.delta + (long long)row * p.d_in + col0;
           const bool wide = ((uintptr_t)p.delta & 31) == 0;
+          walk([&](int ch, const float* v) {
+            if (ch == 7) release();
+            uint32_t pk[8];
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            float v[32];
-            tc_ld32(taddr + ch * 32, v);
-            if (ch == 3) release();
-            uint32_t pk[16];
-#pragma unroll
-            for (int e = 0; e < 32; e += 2)
+            for (int e = 0; e < 16; e += 2)
               pk[e >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[e])) |
                            ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[e + 1])) << 16);
-            if (valid) {
-              store32(dst + ch * 32, pk, wide);
-              store32(dst + ch * 32 + 16, pk + 8, wide);
-            }
-          }
+            if (valid) store32(dst + ch * 16, pk, wide);
+          });
         } else if constexpr (MODE == BD_SQSUM) {
           // sum of squares only (second pass of the l2 proxy)
           float sq4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {
-            float v[16];
-            tc_ld16(taddr + ch * 16, v);
+          walk([&](int ch, const float* v) {
             if (ch == 7) release();
 #pragma unroll
             for (int e = 0; e < 16; ++e) sq4[e & 3] = fmaf(v[e], v[e], sq4[e & 3]);
-          }
+          });
           sq_local += valid ? (double)((sq4[0] + sq4[1]) + (sq4[2] + sq4[3])) : 0.0;
         } else {
           float best[NG], bval[NG];
@@ -662,14 +505,11 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
             float m4[NG][2];
 #pragma unroll
             for (int gi = 0; gi < NG; ++gi) m4[gi][0] = m4[gi][1] = 0.f;
+            walk([&](int ch, const float* v) {
+              const int gi = ch * 16 / G;
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) {
-              float v[32];
-              tc_ld32(taddr + ch * 32, v);
-              const int gi = (G == 128) ? 0 : (ch >> 1);
-#pragma unroll
-              for (int e = 0; e < 32; e += 2) m4[gi][(e >> 1) & 1] = max_abs2(m4[gi][(e >> 1) & 1], v[e], v[e + 1]);
-            }
+              for (int e = 0; e < 16; e += 2) m4[gi][(e >> 1) & 1] = max_abs2(m4[gi][(e >> 1) & 1], v[e], v[e + 1]);
+            });
             bool nan = false;
 #pragma unroll
             for (int gi = 0; gi < NG; ++gi) {
@@ -693,43 +533,61 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               }
             }
           } else {
-            // group absmax with arg-max: four independent running candidates per group (columns e mod 4), merged at the
-            // end with the lowest index winning ties; the NaN-propagating maximum beside them is the range check
-            float bv[NG][4], nm[2] = {0.f, 0.f};
-            int bi[NG][4];
+            // Group absmax with arg-max.  Per chunk of 16 columns the maximum (two columns per instruction), and where it beats the
+            // chunks before it the chunk itself is kept, one select per column; the position inside the kept chunk is looked up
+            // once per group.  1.7 instructions per column and no long chains (compare, two selects and the range check per
+            // column took 4, in four chains), the next chunk's loads in flight meanwhile.  A strict comparison keeps the lowest
+            // of equal chunks, the downward search the lowest column.
+            float kept[16], nm = 0.f;
+            int kc = 0;
+            float b = 0.f;
 #pragma unroll
-            for (int gi = 0; gi < NG; ++gi)
+            for (int e = 0; e < 16; ++e) kept[e] = 0.f;
+            walk([&](int ch, const float* r) {
+              constexpr int CPG = G / 16;  // chunks per group
+              const int gi = ch / CPG;
+              float m[2] = {0.f, 0.f};
 #pragma unroll
-              for (int c = 0; c < 4; ++c) { bv[gi][c] = 0.f; bi[gi][c] = 0; }
+              for (int e = 0; e < 16; e += 2) m[(e >> 1) & 1] = max_abs2(m[(e >> 1) & 1], r[e], r[e + 1]);
+              const float cm = max_abs2(m[0], m[1], 0.f);
+              nm = max_abs2(nm, cm, 0.f);
+              const bool up = cm > b;
+              b = up ? cm : b;
+              kc = up ? ch % CPG : kc;
 #pragma unroll
-            for (int ch = 0; ch < 8; ++ch) {
-              float v[16];
-              tc_ld16(taddr + ch * 16, v);
-              const int gi = (G == 128) ? 0 : (ch >> 2);
-              const int e0 = (G == 128) ? ch * 16 : (ch & 3) * 16;
+              for (int e = 0; e < 16; ++e) kept[e] = up ? r[e] : kept[e];
+              if (ch % CPG == CPG - 1) {
+                float v = 0.f;
+                int ix = 0;
 #pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                const int c = e & 3;
-                if (fabsf(v[e]) > fabsf(bv[gi][c])) { bv[gi][c] = v[e]; bi[gi][c] = e0 + e; }
-                if (e & 1) nm[(e >> 1) & 1] = max_abs2(nm[(e >> 1) & 1], v[e - 1], v[e]);
+                for (int e = 15; e >= 0; --e)
+                  if (fabsf(kept[e]) == b) { v = kept[e]; ix = e; }
+                best[gi] = b;
+                bval[gi] = v;
+                bidx[gi] = kc * 16 + ix;
+                b = 0.f;
+                kc = 0;
+#pragma unroll
+                for (int e = 0; e < 16; ++e) kept[e] = 0.f;
+              }
+            });
+            if (__any_sync(0xffffffffu, nm != nm)) {
+              // A NaN hides its chunk from the comparisons above: the groups' maxima over their numbers, by the whole warp.
+#pragma unroll
+              for (int gi = 0; gi < NG; ++gi) {
+                best[gi] = bval[gi] = 0.f;
+                bidx[gi] = 0;
+#pragma unroll 1
+                for (int ch = 0; ch < G / 16; ++ch) {
+                  float v[16];
+                  tc_ld16(taddr + gi * G + ch * 16, v);
+#pragma unroll
+                  for (int e = 0; e < 16; ++e)
+                    if (fabsf(v[e]) > best[gi]) { best[gi] = fabsf(v[e]); bval[gi] = v[e]; bidx[gi] = ch * 16 + e; }
+                }
               }
             }
-#pragma unroll
-            for (int gi = 0; gi < NG; ++gi) {
-              float b = bv[gi][0];
-              int ix = bi[gi][0];
-#pragma unroll
-              for (int c = 1; c < 4; ++c) {
-                const float x = bv[gi][c];
-                const int jx = bi[gi][c];
-                const bool take = (fabsf(x) > fabsf(b)) || (fabsf(x) == fabsf(b) && jx < ix);
-                if (take) { b = x; ix = jx; }
-              }
-              best[gi] = fabsf(b);
-              bval[gi] = b;
-              bidx[gi] = ix;
-            }
-            if (valid && !(max_abs2(nm[0], nm[1], 0.f) <= 3.0e38f)) bad = true;
+            if (valid && !(nm <= 3.0e38f)) bad = true;
           }
           // Without a second walk over the accumulator (codes / residual) everything still needed is in registers:
           // hand the buffer back to the tensor cores now.  The arrive has release semantics, so issuing it after the
@@ -791,56 +649,56 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
             const float win = 0.5f - (p.qmax + 1.f) * 1.0e-6f;
             int8_t* dst = p.codes + (long long)row * p.d_in + col0;
             const bool wide = ((uintptr_t)p.codes & 31) == 0;
-#pragma unroll 1
-            for (int ch = 0; ch < 4; ++ch) {
-              const int gi = (G == 128) ? 0 : (ch >> 1);
-              const float s = __fdiv_rn((NG == 1 || gi == 0) ? best[0] : best[NG - 1], p.qmax);
-              const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
-              if (valid && ch % (G / 32) == 0) p.scales[(long long)row * (p.d_in / G) + (col0 / G + gi)] = s;
-              uint32_t cpk[8];
-              float dm = 0.f;
+            float s[NG], rs[NG];
 #pragma unroll
-              for (int hf = 0; hf < 2; ++hf) {
-                float v[16];
-                tc_ld16(taddr + ch * 32 + hf * 16, v);
+            for (int gi = 0; gi < NG; ++gi) {
+              s[gi] = __fdiv_rn(best[gi], p.qmax);
+              rs[gi] = (s[gi] > 0.f) ? __frcp_rn(s[gi]) : 0.f;
+              if (valid) p.scales[(long long)row * (p.d_in / G) + (col0 / G + gi)] = s[gi];
+            }
+            uint32_t cpk[8];
+            float dm = 0.f;
+            walk([&](int hc, const float* v) {
+              const int ch = hc >> 1, hf = hc & 1, gi = hc * 16 / G;  // 32 columns a store
+              if (hf == 0) dm = 0.f;
 #pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                  uint32_t cb[4];
-                  float d[4];
+              for (int w = 0; w < 4; ++w) {
+                uint32_t cb[4];
+                float d[4];
 #pragma unroll
-                  for (int e = 0; e < 4; ++e) {
-                    const float x = v[4 * w + e];
-                    const float tt = fmaf(x, rs, MAGIC);
-                    cb[e] = __float_as_uint(tt);
-                    d[e] = fmaf(x, rs, -(tt - MAGIC));
-                  }
-                  dm = max_abs2(dm, d[0], d[1]);
-                  dm = max_abs2(dm, d[2], d[3]);
-                  cpk[4 * hf + w] = __byte_perm(__byte_perm(cb[0], cb[1], 0x0040), __byte_perm(cb[2], cb[3], 0x0040), 0x5410);
+                for (int e = 0; e < 4; ++e) {
+                  const float x = v[4 * w + e];
+                  const float tt = fmaf(x, rs[gi], MAGIC);
+                  cb[e] = __float_as_uint(tt);
+                  d[e] = fmaf(x, rs[gi], -(tt - MAGIC));
                 }
+                dm = max_abs2(dm, d[0], d[1]);
+                dm = max_abs2(dm, d[2], d[3]);
+                cpk[4 * hf + w] = __byte_perm(__byte_perm(cb[0], cb[1], 0x0040), __byte_perm(cb[2], cb[3], 0x0040), 0x5410);
               }
+              if (hf == 0) return;
               // (also: a scale so small that its reciprocal overflows); the accumulator is read again by the whole warp
-              if (__any_sync(0xffffffffu, !(dm <= win) || !(rs < 3.0e38f))) {
+              if (__any_sync(0xffffffffu, !(dm <= win) || !(rs[gi] < 3.0e38f))) {
 #pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                  float v[16];
-                  tc_ld16(taddr + ch * 32 + hf * 16, v);
+                for (int h2 = 0; h2 < 2; ++h2) {
+                  float u[16];
+                  tc_ld16(taddr + ch * 32 + h2 * 16, u);
 #pragma unroll
                   for (int w = 0; w < 4; ++w) {
                     uint32_t pk = 0;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                      float qd = (s > 0.f) ? rintf(__fdiv_rn(v[4 * w + e], s)) : 0.f;
+                      float qd = (s[gi] > 0.f) ? rintf(__fdiv_rn(u[4 * w + e], s[gi])) : 0.f;
                       qd = fminf(fmaxf(qd, -p.qmax), p.qmax);
                       pk |= ((uint32_t)((int)qd) & 0xFFu) << (8 * e);
                     }
-                    cpk[4 * hf + w] = pk;
+                    cpk[4 * h2 + w] = pk;
                   }
                 }
               }
               if (ch == 3) release();
               if (valid) store32(dst + ch * 32, cpk, wide);
-            }
+            });
           }
           if constexpr (MODE == BD_DELTA) {
             // residual s * code - u as one or two bf16 terms, 16 columns at a time (rounding as above)
@@ -849,14 +707,16 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
             uint16_t* dst = p.delta + (long long)row * p.d_in + col0;
             uint16_t* dst_lo = p.delta_lo ? p.delta_lo + (long long)row * p.d_in + col0 : nullptr;
             const bool wide = (((uintptr_t)p.delta | (uintptr_t)p.delta_lo) & 31) == 0;
-#pragma unroll 1
-            for (int ch = 0; ch < 8; ++ch) {
-              const int gi = (G == 128) ? 0 : (ch >> 2);
-              const float s = __fdiv_rn((NG == 1 || gi == 0) ? best[0] : best[NG - 1], p.qmax);
-              const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
-              float v[16];
+            float s2[NG], rs2[NG];
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) {
+              s2[gi] = __fdiv_rn(best[gi], p.qmax);
+              rs2[gi] = (s2[gi] > 0.f) ? __frcp_rn(s2[gi]) : 0.f;
+            }
+            walk([&](int ch, const float* v) {
+              const int gi = ch * 16 / G;
+              const float s = s2[gi], rs = rs2[gi];
               float dm = 0.f;
-              tc_ld16(taddr + ch * 16, v);
               if (ch == 7) release();
               float qv[16];
 #pragma unroll
@@ -885,7 +745,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
                 store32(dst + ch * 16, hpk, wide);
                 if (dst_lo) store32(dst_lo + ch * 16, lpk, wide);
               }
-            }
+            });
           }
         }
       }
@@ -910,12 +770,14 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
 
   // ---------------------------------------------------------------- teardown
   pdl_release();
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // (neither CTA leaves while the other's products may read its shared memory)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_free(tmem_base, 512u);
+    free_tmem();
   }
 }
 
@@ -923,7 +785,8 @@ template <int FORM, int K, int G, int MODE>
 __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_kernel(const __grid_constant__ BdMaps maps, const __grid_constant__ BdMulti mp) {
   pdl_wait();
-  bd_pass_body<FORM, K, G, MODE>(maps, mp, (int)blockIdx.x, (int)gridDim.x);
+  constexpr int W = BdCfg<FORM, K, G>::PAIR ? 2 : 1;
+  bd_pass_body<FORM, K, G, MODE>(maps, mp, (int)blockIdx.x / W, (int)gridDim.x / W);
 }
 
 // Both forms in one launch: the first n_in CTAs run the input-axis list, the others the output-axis list (a layer
@@ -934,8 +797,10 @@ __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_dual_kernel(const __grid_constant__ BdMaps maps_in, const __grid_constant__ BdMulti mp_in,
                     const __grid_constant__ BdMaps maps_out, const __grid_constant__ BdMulti mp_out, const int n_in) {
   pdl_wait();
-  if ((int)blockIdx.x < n_in) bd_pass_body<BD_IN, K, G, BD_REC>(maps_in, mp_in, (int)blockIdx.x, n_in);
-  else bd_pass_body<BD_OUT, K, G, BD_REC>(maps_out, mp_out, (int)blockIdx.x - n_in, (int)gridDim.x - n_in);
+  constexpr int W = BdCfg<BD_IN, K, G>::PAIR ? 2 : 1;
+  const int cta = (int)blockIdx.x / W, n = (int)gridDim.x / W;  // (pairs at K = 256)
+  if (cta < n_in) bd_pass_body<BD_IN, K, G, BD_REC>(maps_in, mp_in, cta, n_in);
+  else bd_pass_body<BD_OUT, K, G, BD_REC>(maps_out, mp_out, cta - n_in, n - n_in);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1014,7 +879,7 @@ static void bd_fill_tiles(BdParams& p) {
   using C = BdCfg<FORM, K, G>;
   if (FORM == BD_IN) {
     p.n_major = (p.d_in + 255) / 256;
-    p.n_minor = (p.d_out + 127) / 128;
+    p.n_minor = (p.d_out + C::ROWS - 1) / C::ROWS;
   } else {
     p.n_major = p.d_out / K;
     p.n_minor = (p.d_in + C::NC - 1) / C::NC;
@@ -1033,14 +898,16 @@ static int bd_launch_multi_t(cudaStream_t st, const BdMaps& maps, BdMulti mp, in
     mp.tile_end[s] = (int)total;
   }
   for (int s = mp.n; s < BD_MAX_SUB; ++s) mp.tile_end[s] = (int)total;
-  mp.stream = (MODE == BD_REC || MODE == BD_CODES) ? l2_stream(65536.0 * total) : 0;
+  mp.stream = (MODE == BD_REC || MODE == BD_CODES) ? l2_stream(512.0 * C::ROWS * total) : 0;
   // one persistent CTA per SM at most; when several problems overlap in streams, small matrices take fewer CTAs
   // (at least min_tiles tiles each): the fixed cost of a CTA is spread over more tiles and the SMs left over
   // run another problem's kernel
   long long want = total / (min_tiles > 0 ? min_tiles : 1);
   if (want < 1) want = 1;
-  const int grid = want < 148 ? (int)want : 148;
-  launch_pdl(bd_pass_kernel<FORM, K, G, MODE>, grid, BD_THREADS, C::SMEM, st, maps, mp);
+  constexpr int most = C::PAIR ? 74 : 148;
+  const int grid = want < most ? (int)want : most;
+  if (C::PAIR) launch_pairs_if(true, bd_pass_kernel<FORM, K, G, MODE>, grid, BD_THREADS, C::SMEM, st, maps, mp);
+  else launch_pdl(bd_pass_kernel<FORM, K, G, MODE>, grid, BD_THREADS, C::SMEM, st, maps, mp);
   return CAFEQ_OK;
 }
 
@@ -1087,7 +954,7 @@ static int bd_launch(cudaStream_t st, int form, int k, int g, const void* X, lon
   BdMulti mp;
   memset(&mp, 0, sizeof(mp));
   if (!make_map_bf16(&maps.x[0], X, p.d_in, p.d_out, ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-  if (!make_map_bf16(&maps.t[0], Tb, k, (long long)nbT * k, k, p.t_mn ? 64 : k)) return CAFEQ_ERR_UNSUPPORTED;
+  if (!make_map_bf16(&maps.t[0], Tb, k, (long long)nbT * k, k, p.t_mn ? 64 : (k == 256 ? 128 : k))) return CAFEQ_ERR_UNSUPPORTED;
   for (int s = 1; s < BD_MAX_SUB; ++s) { maps.x[s] = maps.x[0]; maps.t[s] = maps.t[0]; }
   mp.n = 1;
   mp.p[0] = p;
@@ -1112,7 +979,7 @@ static int bd_launch_many(cudaStream_t st, int form, int k, int g, const BdSub* 
   memset(&mp, 0, sizeof(mp));
   for (int s = 0; s < n; ++s) {
     if (!make_map_bf16(&maps.x[s], subs[s].X, subs[s].p.d_in, subs[s].p.d_out, subs[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&maps.t[s], subs[s].Tb, k, (long long)subs[s].nbT * k, k, subs[s].p.t_mn ? 64 : k)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&maps.t[s], subs[s].Tb, k, (long long)subs[s].nbT * k, k, subs[s].p.t_mn ? 64 : (k == 256 ? 128 : k))) return CAFEQ_ERR_UNSUPPORTED;
     mp.p[s] = subs[s].p;
   }
   for (int s = n; s < BD_MAX_SUB; ++s) { maps.x[s] = maps.x[0]; maps.t[s] = maps.t[0]; }
@@ -1124,11 +991,11 @@ static int bd_launch_many(cudaStream_t st, int form, int k, int g, const BdSub* 
 // the two forms): sets how the CTAs of a dual launch are divided
 static std::atomic<int> g_dual_pass_pct{110}, g_dual_bwd_pct{100};
 
-static int dual_split(long long tiles_in, long long tiles_out, int out_weight_pct) {
+static int dual_split(long long tiles_in, long long tiles_out, int out_weight_pct, int n = 148) {
   const double wi = (double)tiles_in, wo = (double)tiles_out * out_weight_pct / 100.0;
-  int n_in = (int)(148.0 * wi / (wi + wo) + 0.5);
+  int n_in = (int)(n * wi / (wi + wo) + 0.5);
   if (n_in < 1) n_in = 1;
-  if (n_in > 147) n_in = 147;
+  if (n_in > n - 1) n_in = n - 1;
   return n_in;
 }
 
@@ -1150,9 +1017,11 @@ static int bd_launch_dual_t(cudaStream_t st, const BdMaps& mi, BdMulti pi, const
     po.tile_end[s] = (int)to;
   }
   for (int s = po.n; s < BD_MAX_SUB; ++s) po.tile_end[s] = (int)to;
-  pi.stream = po.stream = l2_stream(65536.0 * (ti + to));
-  const int n_in = dual_split(ti, to, g_dual_pass_pct.load(std::memory_order_relaxed));
-  launch_pdl_if(overlap, bd_pass_dual_kernel<K, G>, 148, BD_THREADS, SMEM, st, mi, pi, mo, po, n_in);
+  constexpr bool PAIR = BdCfg<BD_IN, K, G>::PAIR;
+  pi.stream = po.stream = l2_stream((PAIR ? 131072.0 : 65536.0) * (ti + to));
+  const int n_in = dual_split(ti, to, g_dual_pass_pct.load(std::memory_order_relaxed), PAIR ? 74 : 148);
+  if (PAIR) launch_pairs_if(overlap, bd_pass_dual_kernel<K, G>, 74, BD_THREADS, SMEM, st, mi, pi, mo, po, n_in);
+  else launch_pdl_if(overlap, bd_pass_dual_kernel<K, G>, 148, BD_THREADS, SMEM, st, mi, pi, mo, po, n_in);
   return CAFEQ_OK;
 }
 
@@ -1167,13 +1036,13 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
   memset(&po, 0, sizeof(po));
   for (int s = 0; s < n_in; ++s) {
     if (!make_map_bf16(&mi.x[s], in[s].X, in[s].p.d_in, in[s].p.d_out, in[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&mi.t[s], in[s].Tb, k, (long long)in[s].nbT * k, k, k)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&mi.t[s], in[s].Tb, k, (long long)in[s].nbT * k, k, k == 256 ? 128 : k)) return CAFEQ_ERR_UNSUPPORTED;
     pi.p[s] = in[s].p;
   }
   for (int s = n_in; s < BD_MAX_SUB; ++s) { mi.x[s] = mi.x[0]; mi.t[s] = mi.t[0]; }
   for (int s = 0; s < n_out; ++s) {
     if (!make_map_bf16(&mo.x[s], out[s].X, out[s].p.d_in, out[s].p.d_out, out[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&mo.t[s], out[s].Tb, k, (long long)out[s].nbT * k, k, out[s].p.t_mn ? 64 : k)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&mo.t[s], out[s].Tb, k, (long long)out[s].nbT * k, k, out[s].p.t_mn ? 64 : (k == 256 ? 128 : k))) return CAFEQ_ERR_UNSUPPORTED;
     po.p[s] = out[s].p;
   }
   for (int s = n_out; s < BD_MAX_SUB; ++s) { mo.x[s] = mo.x[0]; mo.t[s] = mo.t[0]; }

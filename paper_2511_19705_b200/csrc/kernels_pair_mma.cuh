@@ -7,7 +7,7 @@
 //   * Nothing is read through multicast loads.
 #pragma once
 
-#include "kernels_fused.cuh"
+#include "sm100.cuh"
 
 namespace cafeq {
 
@@ -33,8 +33,10 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
+// Arrival at a barrier of either CTA, with CTA scope: what it orders are reads of tensor memory (tcgen05 fences).  With cluster scope
+// it waits until the thread's global stores have landed, 2100 cycles a tile in the transform pass.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
 // Whether either CTA of the pair saw a raised status word: one answer for both (a CTA that left alone would leave the other
