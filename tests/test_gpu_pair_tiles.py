@@ -1,0 +1,67 @@
+"""Blocks of 256 run on CTA pairs: tiles of 256 rows (output axis: columns) in the transform pass, of 128 contraction entries in the
+sparse backward.  Sizes at the edges of those tiles, groups narrower and wider than a CTA's half and straddling it, against the
+shape-agnostic kernels."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(d_out, d_in, nb, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    W = torch.randn((d_out, d_in), generator=g, device="cuda")
+    W[:, 5] *= 12.0
+    M = torch.linalg.qr(torch.randn((nb, 256, 256), generator=g, device="cuda", dtype=torch.float64))[0]
+    return (W / d_in ** 0.5).bfloat16(), M.float().contiguous()
+
+
+# rows: less than one CTA's half, one more than a half, one tile, one more; columns: one and several blocks, a half tile at the end
+@pytest.mark.parametrize("axis,d_out,d_in,group", [
+    ("in", 1, 256, 128), ("in", 127, 512, 64), ("in", 129, 256, 128), ("in", 256, 768, 256), ("in", 257, 512, 128), ("in", 700, 1024, 512),
+    ("out", 256, 128, 128), ("out", 256, 384, 64), ("out", 512, 640, 128), ("out", 256, 1152, 192), ("out", 512, 768, 384),
+    ("out", 768, 1280, 256)])
+def test_loss_and_gradient(axis, d_out, d_in, group):
+    import paper_2511_19705_b200 as cq
+    W, M = _case(d_out, d_in, (d_in if axis == "in" else d_out) // 256, d_out + d_in)
+    kw = dict(bits=3, group=group, taxis=cq.AXIS_IN if axis == "in" else cq.AXIS_OUT)
+    got = cq.cafeq_proxy_loss_fwd_bwd(W, M, flags=cq.FLAG_EXACT_LOSS, **kw)
+    want = cq.cafeq_proxy_loss_fwd_bwd(W, M, flags=cq.FLAG_EXACT_LOSS | cq.FLAG_GENERIC, **kw)
+    assert int(got["status"].item()) == 0 and int(want["status"].item()) == 0
+    # coefficients as two bf16 terms: 2^-17; the inverse on one side by iteration, on the other by elimination in fp32: 1e-5.  The
+    # residual of Eq. 3 is kept in bf16: 2^-9 per entry, independent, so a sum of n squares is off by a few times 2^-9 / sqrt(n).
+    assert torch.allclose(got["losses"][0], want["losses"][0], rtol=2e-4)
+    assert torch.allclose(got["losses"][1], want["losses"][1], rtol=1e-4 + 8 * 2.0 ** -9 / W.numel() ** 0.5)
+    g, w = got["gradM"].double(), want["gradM"].double()
+    for b in range(g.shape[0]):
+        assert ((g[b] - w[b]).norm() / w[b].norm()).item() <= 5e-4, b
+
+
+@pytest.mark.parametrize("tokens,d_in,transposed", [(65, 256, True), (128, 512, False), (257, 768, True), (500, 1024, True)])
+def test_apply(tokens, d_in, transposed):
+    import paper_2511_19705_b200 as cq
+    X, T = _case(tokens, d_in, d_in // 256, tokens)
+    y = cq.cafeq_apply_transform(X, T, trole=cq.APPLY_TT if transposed else cq.APPLY_T).double()
+    P = T.bfloat16().double()
+    P = P.transpose(1, 2) if transposed else P
+    ref = torch.einsum("tbj,bij->tbi", X.double().reshape(tokens, -1, 256), P).reshape(tokens, d_in)
+    assert ((y - ref).abs() <= ref.abs() * 2.0 ** -8 + 1e-5 * ref.abs().max()).all()
+
+
+@pytest.mark.parametrize("axis,d_out,d_in", [("in", 130, 512), ("in", 300, 256), ("out", 512, 384)])
+def test_codes(axis, d_out, d_in):
+    import paper_2511_19705_b200 as cq
+    W, T = _case(d_out, d_in, (d_in if axis == "in" else d_out) // 256, 3)
+    codes, scales = cq.cafeq_rtn(W, T, bits=4, group=128, tblock=256, taxis=cq.AXIS_IN if axis == "in" else cq.AXIS_OUT)
+    P = T.bfloat16().double()
+    if axis == "in":
+        U = torch.einsum("obj,bij->obi", W.double().reshape(d_out, -1, 256), P).reshape(d_out, d_in)
+    else:
+        U = torch.einsum("bjc,bij->bic", W.double().reshape(-1, 256, d_in), P).reshape(d_out, d_in)
+    x = U.reshape(d_out, -1, 128)
+    s = x.abs().amax(-1, keepdim=True) / 7
+    q = x / s
+    assert torch.allclose(scales.double().reshape(s.shape[:2]), s[..., 0], rtol=1e-5)
+    c = codes.double().reshape(x.shape)
+    # a code may differ from the rounded quotient only where that lies next to a half-integer: sums of 256 terms in fp32
+    assert ((c - q).abs() <= 0.5 + 7 * 2.0 ** -18 * 16).all()
