@@ -16,6 +16,7 @@
 #include "kernels_fused.cuh"
 #include "kernels_bwd.cuh"
 #include "kernels_gemm.cuh"
+#include "kernels_gemm2.cuh"
 #include "kernels_small.cuh"
 #include "kernels_kk.cuh"
 #include "kernels_dense.cuh"
@@ -1061,7 +1062,13 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     // apply), and the scale path needs sum_e gDelta_e Delta_e per group.  Every product runs on the tensor cores
     // with the residual as a two-term bf16 split (three-term products: fp32-grade).
     KkWS& w = s.kk;
-    {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the d_out rows of the residual as it is stored
+    if (k == 256) {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the d_out rows of the residual as it is stored
+      const TgOperand o[2] = {TgOperand{s.m.Dbf, G.d_out, G.d_in, G.d_in}, TgOperand{s.Dlo, G.d_out, G.d_in, G.d_in}};
+      CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, s.tmp, 0.f, kk);
+      g_launches.fetch_add(1, std::memory_order_relaxed);
+      if ((s.err = tg_launch_split(st, 2, o, 2, o, G.d_out, G.nbT, 1, 1, 1.f, s.tmp, status))) return;
+      launch_split(st, s.tmp, k, kk, w.Ph, w.Pl, nullptr, nullptr, status);
+    } else {
       TgOperand oa[3], ob[3];
       const uint16_t* at[3] = {s.m.Dbf, s.Dlo, s.m.Dbf};
       const uint16_t* bt[3] = {s.m.Dbf, s.m.Dbf, s.Dlo};
@@ -1105,7 +1112,12 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       if ((s.err = launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr,
                    status))) return;
     }
-    {  // gDelta[o, B k + j] = 2 sum_l N_B[j][l] Delta[o, B k + l]  -> s.m.D (fp32 [d_out, d_in])
+    // gDelta[o, B k + j] = 2 sum_l N_B[j][l] Delta[o, B k + l], and per group the sum of gDelta Delta
+    if (k == 256) {
+      const T2Ste ste{s.m.Dbf, s.Dlo, G.d_in, s.m.a, s.m.usel, s.m.coef, G.g};
+      g_launches.fetch_add(1, std::memory_order_relaxed);
+      if ((s.err = tg_launch_ste(st, w.Qh, w.Ql, G.d_out, G.nbT, 2.f, ste, status))) return;
+    } else {  // gDelta in s.m.D (fp32 [d_out, d_in])
       TgOperand oa[3], ob[3];
       const uint16_t* at[3] = {s.m.Dbf, s.Dlo, s.m.Dbf};
       const uint16_t* bt[3] = {w.Qh, w.Qh, w.Ql};
@@ -1123,10 +1135,10 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       p.status = status;
       g_launches.fetch_add(1, std::memory_order_relaxed);
       if ((s.err = tg_launch(st, oa, ob, p))) return;
+      const long long nrec = (long long)G.d_out * G.ng;
+      CQ_LAUNCH(ste_scale_coef_kernel, (unsigned)((nrec * 32 + 255) / 256), 256, 0, st, s.m.D, (long long)G.d_in, s.m.Dbf, s.Dlo,
+                (long long)G.d_in, G.d_out, G.ng, G.g, s.m.a, s.m.usel, 1, s.m.coef, status);
     }
-    const long long nrec = (long long)G.d_out * G.ng;
-    CQ_LAUNCH(ste_scale_coef_kernel, (unsigned)((nrec * 32 + 255) / 256), 256, 0, st, s.m.D, (long long)G.d_in, s.m.Dbf, s.Dlo,
-              (long long)G.d_in, G.d_out, G.ng, G.g, s.m.a, s.m.usel, 1, s.m.coef, status);
     launch_scatter(st, W, G, s.m.coef, s.m.idx, gradM, 0, status, 1);
     s.err = minv_path_tc(st, s.Minv, s.gMinv, gradM, G.nbT, k, s.kk, status);
     return;
@@ -1338,6 +1350,13 @@ struct PairWS {
 static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, const uint16_t* Bh, const uint16_t* Bl, int nb, int k, int K,
                          float* out, int32_t* status) {
   TgOperand oa[2], ob[2];
+  if (k == 256) {  // (out was cleared: parts of the contraction are added)
+    oa[0] = TgOperand{A, (long long)nb * k, K, lda};
+    ob[0] = TgOperand{Bh, (long long)nb * k, K, K};
+    ob[1] = TgOperand{Bl, (long long)nb * k, K, K};
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return tg_launch_split(st, 1, oa, 2, ob, K, nb, 1, 0, 1.f, out, status);
+  }
   oa[0] = oa[1] = TgOperand{A, (long long)nb * k, K, lda};
   ob[0] = TgOperand{Bl, (long long)nb * k, K, K};
   ob[1] = TgOperand{Bh, (long long)nb * k, K, K};
@@ -1357,6 +1376,12 @@ static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, cons
 // factors as they are stored (contraction down the rows: MN-major operands), B bf16 [R, nb r k] (pitch ldb), Ah / Al dense.
 static int opgrad_in_tc(cudaStream_t st, const uint16_t* Ah, const uint16_t* Al, const uint16_t* B, long long ldb, int nb, int r, int k,
                         int R, float* out, int32_t* status) {
+  if (k == 256) {  // (as above; the replicas' parts as well)
+    const long long all = (long long)nb * r * k;
+    const TgOperand a[2] = {TgOperand{Ah, R, all, all}, TgOperand{Al, R, all, all}}, b = TgOperand{B, R, all, ldb};
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return tg_launch_split(st, 2, a, 1, &b, R, nb, r, 1, 1.f, out, status);
+  }
   for (int rep = 0; rep < r; ++rep) {
     TgOperand oa[2], ob[2];
     const long long cols = (long long)nb * r * k, c0 = (long long)rep * k;

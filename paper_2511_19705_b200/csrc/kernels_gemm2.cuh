@@ -29,6 +29,7 @@ struct T2Shape {
   int na, nb, nterms;
   int nstage;     // T2_NSLOT / (na + nb)
   int two;        // terms with ac = 1 have the second accumulator
+  int split;      // the product is one part of a contraction: alpha times it is added to C, nothing else is done
   int8_t ta[T2_MAX_TERMS], tb[T2_MAX_TERMS], ac[T2_MAX_TERMS];
 };
 struct T2Maps {
@@ -78,17 +79,34 @@ __device__ __forceinline__ bool t2_enter(T2Cta& c, uint8_t* smem_raw, bool raise
   return !stopped;
 }
 
+// The scale path of the straight-through gradient as a product's epilogue: with v = d loss / d Uhat (the product times alpha) and the
+// residual Delta = hi + lo, coef = sign(usel) / a * sum over the group of v Delta.  The product itself is not stored.  Records are
+// group-major.
+struct T2Ste {
+  const uint16_t *hi, *lo;  // [M, ld]
+  long long ld;
+  const float *a, *usel;    // [groups, M]
+  float* coef;
+  int g;                    // 64 or 128
+};
+
+// Where a tile of a batched or split product lies: corner of its operands, first chunk and number of chunks of its contraction,
+// batch (of the output).
+struct T2At {
+  int ax, ay, bx, by, c0, nc, b;
+};
+
 // One tile of one product, by all threads of both CTAs.  sq_acc: where the sum of squares goes (p.sq only says that there is
 // one).  chunks / tiles: contraction chunks and tiles this pair has done before
 // in this launch (the barriers' phases).  On return both CTAs are done with each other's shared memory.
 __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma, const CUtensorMap* mb, const TgParams& p,
-                                        const T2Shape& sh, double* sq_acc, const int ti, const int tj, const uint32_t chunks,
-                                        const uint32_t tiles) {
+                                        const T2Shape& sh, double* sq_acc, const int ti, const int tj, const T2At at,
+                                        const uint32_t chunks, const uint32_t tiles, const T2Ste* ste = nullptr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cta.rank, base = smem_u32(cta.smem);
   const int bn = sh.bn, bh = bn >> 1, narr = sh.na + sh.nb;
   const int m0 = ti * 256 + (int)rank * 128, n0 = tj * bn;  // this CTA's accumulator rows; the tile's columns
-  const int kchunks = p.K / TG_BK, nstage = sh.nstage;
+  const int kchunks = at.nc, nstage = sh.nstage;
   uint32_t s = chunks % nstage, ph = (chunks / nstage) & 1u;
 
   if (warp == 0) {
@@ -96,23 +114,23 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
       const int a_mn = p.a_mn, b_mn = p.b_mn;
       const int nrow = n0 + (int)rank * bh;  // this CTA's half of the B rows
       for (int c = 0; c < kchunks; ++c) {
-        const int l0 = c * TG_BK;
+        const int l0 = (at.c0 + c) * TG_BK;
         if (!mbar_wait(cta.bar_empty + 8 * s, ph ^ 1u, cta.abort_flag, p.status)) break;
         if (rank == 0) mbar_expect_tx(cta.bar_full + 8 * s, 2 * (sh.na * T2_SLOT + sh.nb * bh * 128));
         const uint32_t bar = cluster_addr(cta.bar_full + 8 * s, 0);
         uint32_t dst = base + s * narr * T2_SLOT;
         for (int u = 0; u < sh.na; ++u, dst += T2_SLOT) {
           if (a_mn) {
-            for (int j = 0; j < 2; ++j) tma_load_pair(dst + j * 8192, ma + u, m0 + j * 64, l0, bar);
+            for (int j = 0; j < 2; ++j) tma_load_pair(dst + j * 8192, ma + u, at.ax + m0 + j * 64, at.ay + l0, bar);
           } else {
-            tma_load_pair(dst, ma + u, l0, m0, bar);
+            tma_load_pair(dst, ma + u, at.ax + l0, at.ay + m0, bar);
           }
         }
         for (int u = 0; u < sh.nb; ++u, dst += T2_SLOT) {
           if (b_mn) {
-            for (int j = 0; j < bh / 64; ++j) tma_load_pair(dst + j * 8192, mb + u, nrow + j * 64, l0, bar);
+            for (int j = 0; j < bh / 64; ++j) tma_load_pair(dst + j * 8192, mb + u, at.bx + nrow + j * 64, at.by + l0, bar);
           } else {
-            tma_load_pair(dst, mb + u, l0, nrow, bar);
+            tma_load_pair(dst, mb + u, at.bx + l0, at.by + nrow, bar);
           }
         }
         if (++s == (uint32_t)nstage) { s = 0; ph ^= 1u; }
@@ -161,8 +179,82 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
       double sq = 0.0;
       float* tile = reinterpret_cast<float*>(cta.smem + (warp - 2) * 4608);  // [32][36] per warp (the slots are free now)
 #pragma unroll 1
+      if (ste) {
+        // this warp's 64 of 256 columns: a group of 64, or with the next warp one of 128
+        const int row = m0 + q * 32 + lane, col = at.b * 256 + part * 64;
+        const bool rv = row < p.M;
+        const long long rec = (long long)(col / ste->g) * p.M + row;
+        const float av = rv ? ste->a[rec] : 0.f, us = rv ? ste->usel[rec] : 0.f;
+        float sum = 0.f;
+#pragma unroll 1
+        for (int c8 = 0; c8 < 4; ++c8) {  // 16 columns
+          const long long o = (long long)row * ste->ld + col + c8 * 16;
+          uint4 h[2], l[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            h[j] = l[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (rv) {
+              h[j] = ld_plain(reinterpret_cast<const uint4*>(ste->hi + o) + j);
+              l[j] = ld_plain(reinterpret_cast<const uint4*>(ste->lo + o) + j);
+            }
+          }
+          float v[16], u[16];
+          tc_ld16(taddr + part * 64 + c8 * 16, v);
+          tc_ld16(taddr + 256u + part * 64 + c8 * 16, u);
+          const uint32_t* hw = reinterpret_cast<const uint32_t*>(h);
+          const uint32_t* lw = reinterpret_cast<const uint32_t*>(l);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            sum = fmaf(v[2 * e] + u[2 * e], __uint_as_float(hw[e] << 16) + __uint_as_float(lw[e] << 16), sum);
+            sum = fmaf(v[2 * e + 1] + u[2 * e + 1], __uint_as_float(hw[e] & 0xFFFF0000u) + __uint_as_float(lw[e] & 0xFFFF0000u), sum);
+          }
+        }
+        sum *= p.alpha;
+        if (ste->g == 128) {
+          float* half = reinterpret_cast<float*>(cta.smem) + (part >> 1) * 128 + q * 32;
+          if (part & 1) half[lane] = sum;
+          asm volatile("bar.sync %0, 64;" ::"r"(1 + (part >> 1) * 4 + q) : "memory");
+          if (!(part & 1)) sum += half[lane];
+        }
+        if (rv && (ste->g == 64 || !(part & 1))) {
+          const float sgn = (us > 0.f) ? 1.f : ((us < 0.f) ? -1.f : 0.f);
+          ste->coef[rec] = (av > 0.f) ? sgn * sum / av : 0.f;
+        }
+      } else if (sh.split) {
+        // part of a contraction: added to C (M, N multiples of 32, ldc a multiple of 4)
+#pragma unroll 1
+        for (int ch = part; ch < bn / 32; ch += TG_EPI_PARTS) {
+          if (n0 + ch * 32 >= p.N || m0 + q * 32 >= p.M) break;
+          float v[32];
+          tc_ld32(taddr + ch * 32, v);
+          if (sh.two) {
+            float u[32];
+            tc_ld32(taddr + 256u + ch * 32, u);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] += u[e];
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            *reinterpret_cast<float4*>(tile + lane * 36 + 4 * j) =
+                make_float4(p.alpha * v[4 * j], p.alpha * v[4 * j + 1], p.alpha * v[4 * j + 2], p.alpha * v[4 * j + 3]);
+          __syncwarp();
+          float* out = p.C + (long long)at.b * p.sCb + (long long)(m0 + q * 32) * p.ldc + n0 + ch * 32;
+          if (((uintptr_t)p.C & 15) == 0) {
+            out += (long long)(lane >> 3) * p.ldc + (lane & 7) * 4;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              atomicAdd(reinterpret_cast<float4*>(out + (long long)(4 * i) * p.ldc),
+                        *reinterpret_cast<const float4*>(tile + (i * 4 + (lane >> 3)) * 36 + (lane & 7) * 4));
+          } else {  // (a caller's gradient at any float address)
+#pragma unroll 1
+            for (int i = 0; i < 32; ++i) atomicAdd(out + (long long)i * p.ldc + lane, tile[i * 36 + lane]);
+          }
+          __syncwarp();
+        }
+      } else
+#pragma unroll 1
       for (int ch = part; ch < bn / 32; ch += TG_EPI_PARTS)
-        tg_epilogue_chunk(p, 0, m0, n0, ch, taddr, sh.two ? taddr + 256u : 0u, th, tl, tile, q, lane, sq);
+        tg_epilogue_chunk(p, at.b, m0, n0, ch, taddr, sh.two ? taddr + 256u : 0u, th, tl, tile, q, lane, sq);
       if (p.sq) {
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         if (lane == 0 && sq != 0.0) atomicAdd(sq_acc, (sh.sym && ti != tj) ? 2.0 * sq : sq);
@@ -202,7 +294,7 @@ tc_pair_gemm_kernel(const __grid_constant__ T2Maps maps, const __grid_constant__
   if (threadIdx.x < sh.na + sh.nb) tma_prefetch_desc((int)threadIdx.x < sh.na ? &maps.a[prob][threadIdx.x] : &maps.b[threadIdx.x - sh.na]);
   T2Cta cta;
   if (!t2_enter(cta, smem_raw, raised)) return;
-  t2_tile(cta, maps.a[prob], maps.b, tp.p[prob], sh, tp.p[prob].sq, ti, tj, 0, 0);
+  t2_tile(cta, maps.a[prob], maps.b, tp.p[prob], sh, tp.p[prob].sq, ti, tj, T2At{0, 0, 0, 0, 0, tp.p[prob].K / TG_BK, 0}, 0, 0);
   if ((threadIdx.x >> 5) == 1) tmem_free_pair(cta.tmem, 512u);
 }
 
@@ -266,7 +358,8 @@ pinv_loop_kernel(const __grid_constant__ T2LoopMaps maps, const __grid_constant_
       const T2Shape& sh = lp.sh[pr];
       for (int t = pair; t < sh.tm * sh.tn; t += npairs) {
         const int tj = t / sh.tm;
-        t2_tile(cta, maps.a[pr], maps.b[pr ? 1 + cur : 0], p, sh, p.sq + it, t - tj * sh.tm, tj, chunks, tiles);
+        t2_tile(cta, maps.a[pr], maps.b[pr ? 1 + cur : 0], p, sh, p.sq + it, t - tj * sh.tm, tj,
+                T2At{0, 0, 0, 0, 0, p.K / TG_BK, 0}, chunks, tiles);
         // the epilogue's scratch lies in the ring that bulk copies write next
         asm volatile("fence.proxy.async;" ::: "memory");
         __syncthreads();
@@ -278,6 +371,43 @@ pinv_loop_kernel(const __grid_constant__ T2LoopMaps maps, const __grid_constant_
     if (!ok) break;
   }
   cluster_sync();
+  if ((threadIdx.x >> 5) == 1) tmem_free_pair(cta.tmem, 512u);
+}
+
+// Batched 256 x 256 products with a long contraction (Gram matrices and operator gradients of blocks of 256): every pair takes a
+// slice of one block's contraction (and one of `reps` column blocks that are summed) and adds its product to C, which the caller
+// has cleared.  As tiles of 64 columns with the whole contraction each, 14 blocks had 112 CTAs with 64 chunks of three terms in a
+// row, 66 us; 70 pairs with 13 chunks take 18.
+__global__ void __launch_bounds__(TG_THREADS, 1)
+tc_pair_split_kernel(const __grid_constant__ T2Maps maps, const __grid_constant__ TgParams p, const __grid_constant__ T2Shape sh,
+                     const int reps, const int slices) {
+  pdl_enter();
+  const bool raised = status_raised(p.status);  // (awaited at the end of the set-up)
+  extern __shared__ uint8_t smem_raw[];
+  const int unit = (int)(blockIdx.x >> 1), s = unit % slices, rep = (unit / slices) % reps, b = unit / (slices * reps);
+  const int all = (p.K + TG_BK - 1) / TG_BK, c0 = (int)((long long)s * all / slices), c1 = (int)((long long)(s + 1) * all / slices);
+  if (threadIdx.x < sh.na + sh.nb) tma_prefetch_desc((int)threadIdx.x < sh.na ? &maps.a[0][threadIdx.x] : &maps.b[threadIdx.x - sh.na]);
+  T2Cta cta;
+  if (!t2_enter(cta, smem_raw, raised)) return;
+  const int blk = b * reps + rep;
+  t2_tile(cta, maps.a[0], maps.b, p, sh, nullptr, 0, 0,
+          T2At{blk * p.colsA_per_batch, blk * p.rowsA_per_batch, blk * p.colsB_per_batch, blk * p.rowsB_per_batch, c0, c1 - c0, b}, 0, 0);
+  if ((threadIdx.x >> 5) == 1) tmem_free_pair(cta.tmem, 512u);
+}
+
+// Scale path of the straight-through gradient on blocks of 256: v = alpha * (hi + lo) N_b over the columns of block b, reduced to one
+// coefficient per group in the epilogue.  4096 x 3584: the product stored as fp32, read again and reduced took 47 + 28 us.
+__global__ void __launch_bounds__(TG_THREADS, 1)
+tc_pair_ste_kernel(const __grid_constant__ T2Maps maps, const __grid_constant__ TgParams p, const __grid_constant__ T2Shape sh,
+                   const __grid_constant__ T2Ste ste) {
+  pdl_enter();
+  const bool raised = status_raised(p.status);  // (awaited at the end of the set-up)
+  extern __shared__ uint8_t smem_raw[];
+  const int unit = (int)(blockIdx.x >> 1), b = unit / sh.tm, ti = unit - b * sh.tm;
+  if (threadIdx.x < sh.na + sh.nb) tma_prefetch_desc((int)threadIdx.x < sh.na ? &maps.a[0][threadIdx.x] : &maps.b[threadIdx.x - sh.na]);
+  T2Cta cta;
+  if (!t2_enter(cta, smem_raw, raised)) return;
+  t2_tile(cta, maps.a[0], maps.b, p, sh, nullptr, ti, 0, T2At{b * 256, 0, 0, b * 256, 0, 4, b}, 0, 0, &ste);
   if ((threadIdx.x >> 5) == 1) tmem_free_pair(cta.tmem, 512u);
 }
 
@@ -363,6 +493,61 @@ static bool t2_wanted(int M, int N, double cost) {
     if (c < tiled) tiled = c;
   }
   return cost < tiled;
+}
+
+static int t2_split_launch(cudaStream_t st, const T2Maps& maps, const TgParams& p, const T2Shape& sh, int reps) {
+  static std::atomic<unsigned long long> done{0};
+  if (!opt_in_smem(tc_pair_split_kernel, T2_SMEM, done)) return CAFEQ_ERR_CUDA;
+  const int units = p.batch * reps, all = (p.K + TG_BK - 1) / TG_BK;
+  int slices = units < 74 ? 74 / units : 1;
+  if (slices > all / 4) slices = all / 4 > 0 ? all / 4 : 1;  // (four chunks at least: a tile's fixed part is some 8 us)
+  launch_pairs_if(true, tc_pair_split_kernel, units * slices, TG_THREADS, T2_SMEM, st, maps, p, sh, reps, slices);
+  return CAFEQ_OK;
+}
+
+// Dh / Dl: [M, nb * 256] (pitch ste.ld); Nh / Nl: blocks [nb * 256, 256]
+static int tg_launch_ste(cudaStream_t st, const uint16_t* Nh, const uint16_t* Nl, int M, int nb, float alpha, const T2Ste& ste, int32_t* status) {
+  static std::atomic<unsigned long long> done{0};
+  if (!opt_in_smem(tc_pair_ste_kernel, T2_SMEM, done)) return CAFEQ_ERR_CUDA;
+  T2Maps maps;
+  memset(&maps, 0, sizeof(maps));
+  const uint16_t* d[2] = {ste.hi, ste.lo};
+  const uint16_t* n[2] = {Nh, Nl};
+  for (int i = 0; i < 2; ++i)
+    if (!make_map_bf16(&maps.a[0][i], d[i], nb * 256ll, M, ste.ld, 128) || !make_map_bf16(&maps.b[i], n[i], 256, nb * 256ll, 256, 128))
+      return CAFEQ_ERR_UNSUPPORTED;
+  TgParams p;
+  memset(&p, 0, sizeof(p));
+  p.M = M; p.N = 256; p.K = 256; p.batch = nb; p.divA = 1;
+  p.alpha = alpha;
+  p.status = status;
+  const T2Shape sh = t2_shape(M, 256, 256, 2, 2, 2);
+  launch_pairs_if(true, tc_pair_ste_kernel, nb * sh.tm, TG_THREADS, T2_SMEM, st, maps, p, sh, ste);
+  return CAFEQ_OK;
+}
+
+// A: na arrays, B: nb arrays, each [rows, cols] with its pitch, either both stored with the contraction as rows (mn: [K, blocks * 256])
+// or both with it as columns ([blocks * 256, K]); C += alpha * sum over the column (row) blocks b * reps .. of A_b B_b^T.
+static int tg_launch_split(cudaStream_t st, int na, const TgOperand* A, int nb, const TgOperand* B, int K, int batch, int reps, int mn,
+                           float alpha, float* C, int32_t* status) {
+  T2Maps maps;
+  memset(&maps, 0, sizeof(maps));
+  bool ok = true;
+  for (int i = 0; i < na; ++i) ok = ok && make_map_bf16(&maps.a[0][i], A[i].ptr, A[i].cols, A[i].rows, A[i].pitch, mn ? 64 : 128);
+  for (int i = 0; i < nb; ++i) ok = ok && make_map_bf16(&maps.b[i], B[i].ptr, B[i].cols, B[i].rows, B[i].pitch, mn ? 64 : 128);
+  if (!ok) return CAFEQ_ERR_UNSUPPORTED;
+  TgParams p;
+  memset(&p, 0, sizeof(p));
+  p.M = p.N = 256; p.K = K; p.batch = batch; p.divA = 1;
+  p.a_mn = p.b_mn = mn;
+  if (mn) p.colsA_per_batch = p.colsB_per_batch = 256;
+  else p.rowsA_per_batch = p.rowsB_per_batch = 256;
+  p.alpha = alpha;
+  p.C = C; p.ldc = 256; p.sCb = 65536;
+  p.status = status;
+  T2Shape sh = t2_shape(256, 256, 256, na, nb, na > nb ? na : nb);
+  sh.split = 1;
+  return t2_split_launch(st, maps, p, sh, reps);
 }
 
 }  // namespace cafeq
