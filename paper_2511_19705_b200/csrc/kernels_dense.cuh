@@ -6,7 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "kernels_generic.cuh"
+#include "kernels_gemm.cuh"
 
 namespace cafeq {
 
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, 
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
                                                          uint16_t* __restrict__ t3 = nullptr, const double* only_bad = nullptr) {
   pdl_enter();
-  if (only_bad && *only_bad <= 0.25) return;  // (a restart that is not needed)
+  if (only_bad && !tg_bad_start(only_bad)) return;  // (a restart that is not needed)
   if (cta_stopped(status)) return;
   __shared__ uint32_t tile[64][65];
   __shared__ uint16_t tile3[64][66];

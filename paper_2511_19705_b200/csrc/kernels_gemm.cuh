@@ -51,7 +51,7 @@ struct TgParams {
                           // batch * colsA_per_batch / colsB_per_batch (B: its contraction at row batch * rowsB_per_batch)
   const double* stop_sq;  // optional: squared residuals of an iteration; this launch belongs to iteration stop_it, and is
   int stop_it;            // skipped when the rule (tg_stopped) ended the iteration before
-  int stop_guard;         // 1: iteration 0 checks its start; 2: this is its update, skipped when the start is bad
+  int stop_guard;         // + 1: iteration 0 checks its start; + 2: this is its update; + 4: an update
   int32_t* status;
 };
 
@@ -69,19 +69,22 @@ struct TgCfg {
 // falling (a rank-deficient matrix stalls at its rank defect).  With every eigenvalue of A X in (0, 2) the residual falls
 // monotonically: one that is still large and grows means that the starting scale was too small, which is reported.
 // The residuals of iterations that were skipped stay zero, so the last two decide.
-// With stop_guard, iteration 0 checks a start that is only good when its squared residual is at most 1/4; otherwise the iteration
-// has been restarted, and what came before iteration 1 does not count.  Iteration 0 itself then updates nothing.
-__device__ __forceinline__ bool tg_bad_start(const volatile double* stop_sq) { return !(stop_sq[0] <= 0.25); }
+// With stop_guard, iteration 0 checks a start that is only good when its residual is at most 0.9 (so every eigenvalue of I - A X is);
+// otherwise the iteration has been restarted, and what came before iteration 1 does not count.  Iteration 0 itself then updates
+// nothing.  An update that would start below the limit is left out: the step that follows the iteration squares the residual too.
+constexpr double TG_GOOD_START2 = 0.81, TG_DONE2 = 1e-6;
+__device__ __forceinline__ bool tg_bad_start(const volatile double* stop_sq) { return !(stop_sq[0] <= TG_GOOD_START2); }
 __device__ __forceinline__ bool tg_stopped(const TgParams& p, int it) {
   const volatile double* sq = p.stop_sq;  // (one launch may run several iterations: never from a cached line)
   if (!sq) return false;
+  if ((p.stop_guard & 4) && sq[it] <= TG_DONE2) return true;
   if (p.stop_guard) {
-    if (it == 0) return p.stop_guard == 2 && tg_bad_start(sq);
+    if (it == 0) return (p.stop_guard & 2) && tg_bad_start(sq);
     if (tg_bad_start(sq)) { ++sq; --it; }
   }
   if (it < 1) return false;
   const double cur = sq[it - 1];
-  if (!(cur > 1e-6)) return true;
+  if (!(cur > TG_DONE2)) return true;
   if (it < 2) return false;
   const double prev = sq[it - 2];
   if (cur > 1.5 * prev && cur > 1e-2 * (double)p.M) {

@@ -352,8 +352,9 @@ pinv_loop_kernel(const __grid_constant__ T2LoopMaps maps, const __grid_constant_
   for (int it = lp.it0; it < lp.it1; ++it) {
     if (it > lp.it0 && tg_stopped(lp.p[0][0], it)) break;
     const int cur = it & 1;
-    bool ok = true;
+    bool ok = true, done = false;
     for (int pr = 0; pr < 2 && ok; ++pr) {
+      if (pr && (done = tg_stopped(lp.p[1][cur], it))) break;
       const TgParams& p = lp.p[pr][cur];
       const T2Shape& sh = lp.sh[pr];
       for (int t = pair; t < sh.tm * sh.tn; t += npairs) {
@@ -368,7 +369,7 @@ pinv_loop_kernel(const __grid_constant__ T2LoopMaps maps, const __grid_constant_
       }
       ok = grid_meet(lp.arrived, ++met * gridDim.x, cta.abort_flag, p.status);
     }
-    if (!ok) break;
+    if (!ok || done) break;
   }
   cluster_sync();
   if ((threadIdx.x >> 5) == 1) tmem_free_pair(cta.tmem, 512u);

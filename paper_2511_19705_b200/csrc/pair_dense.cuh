@@ -168,9 +168,10 @@ static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, 
 // Y <- 2 mu Y - mu^2 Y B and B <- 2 mu B - mu^2 B B from B = G / c (c a little above ||G||_F), Y = I / c: B = G Y c throughout, and
 // with mu = 2 / (1 + l) for the smallest eigenvalue l of B the eigenvalues of B go to 1, l growing fourfold a step at first.
 // Both are polynomials in G, so one launch does both products on their upper tiles: 36 + 36 pairs at m = 2048, one wave, 45 us; a
-// step of the rectangular iteration takes 160.  l starts at 2^-14: smaller eigenvalues grow as far as that and are finished by the
-// rectangular iteration.  (Nothing here need be accurate: whatever Y is, A^T Y lies in the row space of A, and its error is what the
-// rectangular iteration corrects.)
+// step of the rectangular iteration takes 160.  l starts at 2^-13: smaller eigenvalues grow as far as that and are finished by the
+// rectangular iteration (the products' errors grow with them, fourfold a step: from 2^-14 they left residuals twice as large).
+// Nothing here need be accurate: whatever Y is, A^T Y lies in the row space of A, and its error is what the rectangular iteration
+// corrects.
 constexpr int GRAM_STEPS = 9;
 static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2, int32_t* status) {
   T2Maps maps;
@@ -192,7 +193,7 @@ static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2,
   uint16_t* Bs[2][2] = {{w.Yh, w.Yl}, {w.YTh[0], w.YTl[0]}};
   uint16_t* Ys[2][2] = {{w.YTh[1], w.YTl[1]}, {w.CTh, w.CTl}};
   static_assert(GRAM_STEPS % 2 == 1, "the result is left in the second pair of buffers");
-  double l = 1.0 / 16384.0;
+  double l = 1.0 / 8192.0;
   for (int j = 0; j < GRAM_STEPS; ++j) {
     const float mu = (float)(2.0 / (1.0 + l));
     l = 4.0 * l / ((1.0 + l) * (1.0 + l));
@@ -225,11 +226,11 @@ static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2,
 // that every product has both operands contraction-major.
 //   1. X0 = A^T G^-1 with the approximate inverse of the Gram matrix (gram_inverse), as five terms over A split three ways: the
 //      iteration below never corrects what lies outside the row space of A, so X0 must not leave it.
-//   2. Newton-Schulz X <- X + X (I - A X), until ||I - A X||_F falls below 1e-3 (the next update squares it) or stalls, which every
-//      product works out from the residuals itself.  Two updates for the 9B-shaped v-o factors (kappa^2 some thousands) instead of
+//   2. Newton-Schulz X <- X + X (I - A X), until ||I - A X||_F falls below 1e-3 (step 3 squares it) or stalls, which every product
+//      works out from the residuals itself.  Two updates for the 9B-shaped v-o factors (kappa^2 some thousands) instead of
 //      the sixteen from X0 = A^T / c.
 //   3. One step with the residual over three-way splits.
-// When A X0 is not within 1/2 of I (rank-deficient or very badly conditioned A) the iteration restarts from X0 = A^T / c, c a
+// When A X0 is not within 0.9 of I (rank-deficient or very badly conditioned A) the iteration restarts from X0 = A^T / c, c a
 // little above ||A A^T||_F: the eigenvalues of A X0 then lie in [0, 1], and it converges to the Moore-Penrose inverse (stalling at
 // the rank defect).  From there on it is one launch.
 // Error against a float64 pseudo-inverse (512 x 768, kappa^2 4000, emulated products): 1.3e-7; from X0 = A^T / c 7e-6.
@@ -273,7 +274,7 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
   auto update = [&](DenseOut& o, int cur) {                                                      // Y += C^T Y
     o.C0 = w.Y; o.ldc0 = n; o.C = w.Y; o.ldc = n;
     o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[cur ^ 1]; o.Ctlo = w.YTl[cur ^ 1];
-    o.stop_sq = rs; o.stop_guard = 1;
+    o.stop_sq = rs; o.stop_guard = 5;
   };
   constexpr int LAUNCHED = 3;
   for (int it = 0; it < LAUNCHED; ++it) {
@@ -286,7 +287,7 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     DenseOut u;
     update(u, cur);
     u.stop_it = it;
-    if (it == 0) u.stop_guard = 2;
+    if (it == 0) u.stop_guard = 7;
     if ((rc = launch_dense_tc(st, 2, ct, 2, yt, m, n, m, 1.f, 1.f, 0.f, u, nullptr, status))) return rc;
     if (it == 0) {  // the restart: what update 0 would have written
       if (wide) launch_split_rect(st, S, R, C, C, 1.f, c, w.Y, nullptr, w.Yh, w.Yl, w.YTh[1], w.YTl[1], status, nullptr, nullptr, rs);
