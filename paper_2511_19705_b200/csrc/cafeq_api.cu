@@ -377,11 +377,13 @@ static bool launch_group_quant_vec(cudaStream_t st, const SRC* U, long long ld, 
 #define GQ(L, N)                                                                                                              \
   CQ_LAUNCH((group_quant_kernel<L, N, SRC>), (unsigned)((groups * L + 255) / 256), 256, 0, st, U, ld, rows, ng, g, qmax, offsets, off_kind, \
             a, usel, idx, Delta, Uhat, codes, scales, status)
-  // as many lanes as the group has vectors of four, up to a warp; above eight vectors a lane, the whole CTA
-  if (g <= 32) GQ(8, 1);
-  else if (g <= 64) GQ(16, 1);
-  else if (g <= 128) GQ(32, 1);
-  else if (g <= 256) GQ(32, 2);
+  // Four vectors of four a lane where the group has them (two in groups of 32): a lane's loads are in flight together, and the
+  // reduction over lanes, fifteen shuffles for four values at one vector a lane of 32, is nine for sixteen.  Above eight vectors a
+  // lane, the whole CTA.
+  if (g <= 32) GQ(4, 2);
+  else if (g <= 64) GQ(4, 4);
+  else if (g <= 128) GQ(8, 4);
+  else if (g <= 256) GQ(16, 4);
   else if (g <= 512) GQ(32, 4);
   else if (g <= 1024) GQ(32, 8);
   else if (g <= 2048) GQ(256, 2);
@@ -1415,10 +1417,10 @@ static void launch_ste_split(cudaStream_t st, const MatWS& m, const float* gX, l
 #define SGS(L, N)                                                                                                              \
   CQ_LAUNCH((ste_grad_split_kernel<L, N>), (unsigned)((groups * L + 255) / 256), 256, 0, st, m.U, gX, ldg, G.d_out, G.ng, G.g, k, r, \
             m.a, m.usel, m.idx, qmax, hi, lo, status)
-  if (G.g <= 32) SGS(8, 1);
-  else if (G.g <= 64) SGS(16, 1);
-  else if (G.g <= 128) SGS(32, 1);
-  else if (G.g <= 256) SGS(32, 2);
+  if (G.g <= 32) SGS(4, 2);
+  else if (G.g <= 64) SGS(4, 4);
+  else if (G.g <= 128) SGS(8, 4);
+  else if (G.g <= 256) SGS(16, 4);
   else if (G.g <= 512) SGS(32, 4);
   else SGS(32, 8);
 #undef SGS
