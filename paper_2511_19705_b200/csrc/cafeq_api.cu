@@ -987,13 +987,16 @@ static bool lean_single_ok(const Geo& G, const cafeq_opt_cfg* cfg, const void* W
   if (!cfg || cfg->loss_kind != CAFEQ_LOSS_SURROGATE || cfg->eval_every != 0) return false;
   return sized_for_pass(G, W);
 }
-// Enqueue one forward(+backward) for a single matrix; gradM may be null.  hist is an optional [2] slot.
+static bool single_tc(const Geo& G) { return G.k == 32 || kk_fast(G.k); }
+// Enqueue one forward(+backward) for a single matrix; gradM may be null.  hist is an optional [2] slot.  Inside a run of many steps
+// (in_run, single_tc) the losses are left in s.acc for single_next_kernel, which also sets up the steps after the first (prepared).
 static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& G, const void* W, const float* M,
                         float* Minv_out, const void* offsets, int off_kind, int loss_kind, float kappa, bool want_exact,
                         float* losses, float* hist, float* gradM, int32_t* status, SingleWS& s, bool force_generic,
-                        bool warm = false, float* step_counter = nullptr, float* grad_offsets = nullptr, bool splits_kept = false) {
+                        bool warm = false, float* step_counter = nullptr, float* grad_offsets = nullptr, bool splits_kept = false,
+                        bool in_run = false, bool prepared = false) {
   const int k = G.k;
-  const bool tc = (k == 32 || kk_fast(k)) && !force_generic;
+  const bool tc = single_tc(G) && !force_generic;
   const long long kk = (long long)G.nbT * k * k;
   const float qm = qmax_of(d->bits);
   const bool ste = (loss_kind == CAFEQ_LOSS_L2_STE);
@@ -1011,10 +1014,11 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     pa.zero_f[1] = s.m.agrp; pa.zero_fn[1] = G.ng;
     if (in_r1) { pa.zero_f[2] = s.m.cw; pa.zero_fn[2] = G.ng; }
     if (want_grad) { pa.zero_f[3] = gradM; pa.zero_fn[3] = kk; }
-    pa.zero_d = s.acc; pa.zero_dn = 8;
+    pa.zero_d = s.acc; pa.zero_dn = in_run ? 6 : 8;
     pa.step_counter = step_counter;
+    pa.step_slot = in_run ? s.acc + 6 : nullptr;
     pa.status = status;
-    CQ_LAUNCH(step_prep_kernel, grid_for(kk), 256, 0, st, pa);
+    if (!prepared) CQ_LAUNCH(step_prep_kernel, grid_for(kk), 256, 0, st, pa);
     NsParams eq4;
     memset(&eq4, 0, sizeof(eq4));
     eq4.c = s.c;
@@ -1106,7 +1110,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     }
     CQ_LAUNCH(dot_f32_kernel, grid_for(kk), 256, 0, st, s.Nf, s.tmp, kk, s.acc + 1);
     CQ_LAUNCH(sqsum_bf16_kernel, grid_for(G.n), 256, 0, st, (const uint16_t*)W, G.ld, G.d_out, G.d_in, s.acc + 2, status);
-    CQ_LAUNCH(finalize_single_kernel, 1, 1, 0, st, s.acc, losses, hist, 1);
+    if (!in_run) CQ_LAUNCH(finalize_single_kernel, 1, 1, 0, st, s.acc, losses, hist, 1);
     if (!want_grad) return;
     {  // dL/dMinv = 2 Minv Gram (Gram is symmetric: its rows serve as the contraction-major second operand)
       const uint16_t* a2[3] = {w.Xh, w.Xl, w.Xh};
@@ -1165,7 +1169,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
                                                                  s.m.agrp, s.A, s.acc + 0, status);
   if (G.axis == CAFEQ_AXIS_IN && !in_r1)
     CQ_LAUNCH(expand_agrp_kernel, (G.d_in + 127) / 128, 128, 0, st, s.m.agrp, G.d_in, G.g, k, G.r, s.A);
-  CQ_LAUNCH(finalize_single_kernel, 1, 1, 0, st, s.acc, losses, hist, need_l2 ? 1 : 0);
+  if (!in_run) CQ_LAUNCH(finalize_single_kernel, 1, 1, 0, st, s.acc, losses, hist, need_l2 ? 1 : 0);
   if (!want_grad) return;
   if (!ste) {
     launch_scatter(st, W, G, s.m.coef, s.m.idx, gradM, 0, status, fused ? 1 : 0);
@@ -1282,10 +1286,27 @@ extern "C" int cafeq_optimize_single(const cafeq_matrix_desc* d, const void* W, 
   s.Minv = stored.inv;
   for (int it = 0; it < cfg->steps; ++it) {
     bool eval = cfg->eval_every > 0 && (it % cfg->eval_every == 0);
+    const bool in_run = single_tc(G);
     single_step(st, d, G, W, M, nullptr, nullptr, CAFEQ_OFFSETS_NONE, cfg->loss_kind, kappa, eval, nullptr,
-                loss_history + 2 * (size_t)it, grad, status, s, false, resume || it > 0, opt_state, nullptr, it > 0);
+                loss_history + 2 * (size_t)it, grad, status, s, false, resume || it > 0, opt_state, nullptr, it > 0, in_run,
+                in_run && it > 0);
     if (s.err) return s.err;
-    if (cfg->optimizer == CAFEQ_OPT_GD) {
+    if (in_run) {
+      SingleNextArgs na;
+      memset(&na, 0, sizeof(na));
+      na.M = M; na.grad = grad; na.state = opt_state; na.kk = kk;
+      na.adam = cfg->optimizer == CAFEQ_OPT_ADAM;
+      na.lr = cfg->lr; na.b1 = cfg->beta1; na.b2 = cfg->beta2; na.eps = cfg->eps;
+      na.acc = s.acc; na.hist = loss_history + 2 * (size_t)it;
+      na.want_exact = eval || cfg->loss_kind == CAFEQ_LOSS_L2_STE;
+      na.next = it + 1 < cfg->steps; na.slot = 6 + (it & 1);
+      na.Mc = s.Mc; na.Ab = s.kk.Ab;
+      na.zero_f[0] = s.A; na.zero_fn[0] = (long long)G.nbT * G.k;
+      na.zero_f[1] = s.m.agrp; na.zero_fn[1] = G.ng;
+      if (G.axis == CAFEQ_AXIS_IN && G.r == 1) { na.zero_f[2] = s.m.cw; na.zero_fn[2] = G.ng; }
+      na.status = status;
+      CQ_LAUNCH(single_next_kernel, grid_for(kk), 256, 0, st, na);
+    } else if (cfg->optimizer == CAFEQ_OPT_GD) {
       CQ_LAUNCH(gd_update_kernel, grid_for(kk), 256, 0, st, M, grad, cfg->lr, kk, status);
     } else {
       CQ_LAUNCH(adam_update_kernel, grid_for(kk), 256, 0, st, M, grad, opt_state, cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, kk,
