@@ -10,7 +10,16 @@
 
 namespace cafeq {
 
-// X fp32 [R, C] (row pitch ld) times `scale` (or times 1 / *inv_scale when inv_scale is given) ->
+// 2^-e with 4^e <= n2 < 4^(e + 1): the power of two that brings a matrix of squared norm n2 to a norm in [1, 2).  Exact as a factor,
+// so nothing but the exponents of what is computed from the matrix changes.  (e within the exponents of normal fp32 numbers; a norm
+// of zero or one that is not finite takes an end of that range.)
+__device__ __forceinline__ double unit_scale(const double n2) {
+  const int e = n2 > 0.0 ? (n2 < 1e300 ? ilogb(n2) >> 1 : 126) : 0;
+  return ldexp(1.0, -min(max(e, -126), 126));
+}
+
+// X fp32 [R, C] (row pitch ld) times `scale` (or times 1 / *inv_scale when inv_scale is given, times unit_scale(*norm2) when norm2
+// is) ->
 // bf16 hi / lo splits, row-major [R, C] and / or transposed [C, R]; optional fp32 copy Y of the scaled values
 // (row-major) and YT (transposed, holding hi + lo: used only as a starting guess).  h3 / t3: optional third term
 // bf16(x - hi - lo) in row-major / transposed order (hi + lo + third carries 24 significand bits: products over the
@@ -23,7 +32,8 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, 
                                                          float* __restrict__ YT, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
                                                          uint16_t* __restrict__ thi, uint16_t* __restrict__ tlo,
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
-                                                         uint16_t* __restrict__ t3 = nullptr, const double* only_bad = nullptr) {
+                                                         uint16_t* __restrict__ t3 = nullptr, const double* norm2 = nullptr,
+                                                         const double* only_bad = nullptr) {
   pdl_enter();
   if (only_bad && !tg_bad_start(only_bad)) return;  // (a restart that is not needed)
   if (cta_stopped(status)) return;
@@ -32,7 +42,8 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, 
   const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   float sc = scale;
-  if (inv_scale) sc = (float)((double)scale / fmax(*inv_scale, 1e-300));
+  if (inv_scale || norm2)
+    sc = (float)((double)scale * (norm2 ? unit_scale(*norm2) : 1.0) / (inv_scale ? fmax(*inv_scale, 1e-300) : 1.0));
   const bool trans = thi || tlo || YT;
   float2 x2[8];
   if (((uintptr_t)X & 7) == 0 && (ld & 1) == 0) {

@@ -104,8 +104,9 @@ static int launch_dense_tc(cudaStream_t st, int na, const uint16_t* const* A, in
 
 static void launch_split_rect(cudaStream_t st, const float* X, int R, int C, long long ld, float scale, const double* inv_scale,
                               float* Y, float* YT, uint16_t* hi, uint16_t* lo, uint16_t* thi, uint16_t* tlo, const int32_t* status,
-                              uint16_t* h3 = nullptr, uint16_t* t3 = nullptr, const double* only_bad = nullptr) {
-  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3, only_bad);
+                              uint16_t* h3 = nullptr, uint16_t* t3 = nullptr, const double* norm2 = nullptr, const double* only_bad = nullptr) {
+  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3, norm2,
+            only_bad);
 }
 
 // Scratch of the dense pair algebra for a pair with stored shapes U [h, d1], V [d3, rh]
@@ -223,7 +224,9 @@ static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2,
 }
 
 // out (hi / lo, shape [R, C] of S) = pinv(S^T) = pinv(S)^T on the wide orientation A of S ([m, n], m <= n), carried as Y = X^T so
-// that every product has both operands contraction-major.
+// that every product has both operands contraction-major.  A is S times a power of two that brings its norm to [1, 2): the norm of
+// its Gram matrix is taken from sums of fourth powers, which leave the range of fp32 at row norms of 4e9 and 1e-11.  The same power
+// brings the result back.
 //   1. X0 = A^T G^-1 with the approximate inverse of the Gram matrix (gram_inverse), as five terms over A split three ways: the
 //      iteration below never corrects what lies outside the row space of A, so X0 must not leave it.
 //   2. Newton-Schulz X <- X + X (I - A X), until ||I - A X||_F falls below 1e-3 (step 3 squares it) or stalls, which every product
@@ -238,12 +241,14 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
   const bool wide = R <= C;
   const int m = wide ? R : C, n = wide ? C : R;
   double* fro2 = w.sq + 120;
+  double* norm2 = w.sq + 121;
   double* c = w.sq + 123;
   double* rs = w.sq + 32;  // residuals per iteration
   int rc;
   CQ_LAUNCH(zero_f64_kernel, 1, 128, 0, st, w.sq + 32, DENSE_SQ - 32);
-  if (wide) launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status, w.Aw3, nullptr);
-  else launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Awh, w.Awl, status, nullptr, w.Aw3);
+  CQ_LAUNCH(sqsum_f32_kernel, grid_for((long long)R * C), 256, 0, st, S, (long long)R * C, norm2);
+  if (wide) launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status, w.Aw3, nullptr, norm2);
+  else launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Awh, w.Awl, status, nullptr, w.Aw3, norm2);
   if ((rc = gram_inverse(st, m, n, w, fro2, status))) return rc;
   {  // Y = G^-1 A (the rows of A, the contraction, are read as they are stored)
     const uint16_t* g[2] = {w.CTh, w.CTl};
@@ -290,8 +295,8 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     if (it == 0) u.stop_guard = 7;
     if ((rc = launch_dense_tc(st, 2, ct, 2, yt, m, n, m, 1.f, 1.f, 0.f, u, nullptr, status))) return rc;
     if (it == 0) {  // the restart: what update 0 would have written
-      if (wide) launch_split_rect(st, S, R, C, C, 1.f, c, w.Y, nullptr, w.Yh, w.Yl, w.YTh[1], w.YTl[1], status, nullptr, nullptr, rs);
-      else launch_split_rect(st, S, R, C, C, 1.f, c, nullptr, w.Y, w.YTh[1], w.YTl[1], w.Yh, w.Yl, status, nullptr, nullptr, rs);
+      if (wide) launch_split_rect(st, S, R, C, C, 1.f, c, w.Y, nullptr, w.Yh, w.Yl, w.YTh[1], w.YTl[1], status, nullptr, nullptr, norm2, rs);
+      else launch_split_rect(st, S, R, C, C, 1.f, c, nullptr, w.Y, w.YTh[1], w.YTl[1], w.Yh, w.Yl, status, nullptr, nullptr, norm2, rs);
     }
   }
   {
@@ -338,8 +343,8 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     o2.C0 = w.Y; o2.ldc0 = n; o2.C = w.Y; o2.ldc = n;
     if ((rc = launch_dense_tc(st, 2, a2, 2, b2, m, n, m, 1.f, 1.f, 0.f, o2, nullptr, status))) return rc;
   }
-  if (wide) launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, w.Oh, w.Ol, nullptr, nullptr, status, w.O3, nullptr);
-  else launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Oh, w.Ol, status, nullptr, w.O3);
+  if (wide) launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, w.Oh, w.Ol, nullptr, nullptr, status, w.O3, nullptr, norm2);
+  else launch_split_rect(st, w.Y, m, n, n, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Oh, w.Ol, status, nullptr, w.O3, norm2);
   return CAFEQ_OK;
 }
 

@@ -65,6 +65,31 @@ def test_first_half_step_against_float64(h, d1, d3, k, case):
     assert (o["codes2"].double().reshape(q.shape) != q).double().mean().item() <= 1e-4
 
 
+# A power of two on either factor changes exponents only.  Its fourth power is far outside fp32 here.
+@pytest.mark.parametrize("e1,e2", [(40, 0), (-40, 0), (0, 40), (0, -40), (55, -55), (-55, 55)])
+@pytest.mark.parametrize("case", ["full", "zero"])
+def test_alternation_at_other_scales(e1, e2, case):
+    import paper_2511_19705_b200 as cq
+    h, d1, d3, k, g = 256, 512, 448, 64, 64
+    W1, W2 = _weights(h, d1, d3, 1, 7)
+    if case == "zero":
+        W1[7] = 0
+    M = torch.eye(k, device="cuda").repeat(h // k, 1, 1)
+
+    def call(A, B):
+        o = cq.cafeq_adaptive_round(A, B, M, iters=1, bits=4, group1=g, group2=g)
+        assert int(o["status"].item()) == 0
+        return o
+
+    want, got = call(W1, W2), call(W1 * 2.0 ** e1, W2 * 2.0 ** e2)
+    # (sums that are added atomically may round another way: bounds as against float64 above)
+    s, w = got["scales2"].double() * 2.0 ** -e2, want["scales2"].double()
+    assert ((s - w).norm() / w.norm()).item() <= 3e-5
+    assert (got["codes2"] != want["codes2"]).double().mean().item() <= 1e-4
+    p, q = got["pqe"].double() * 2.0 ** -(e1 + e2), want["pqe"].double()
+    assert ((p - q).abs() <= 1e-3 * q).all()
+
+
 def test_same_codes_under_capture():
     import paper_2511_19705_b200 as cq
     h, d1, d3, k = 256, 512, 448, 64
