@@ -65,6 +65,28 @@ def test_first_half_step_against_float64(h, d1, d3, k, case):
     assert (o["codes2"].double().reshape(q.shape) != q).double().mean().item() <= 1e-4
 
 
+# One row of an otherwise orthonormal factor is weak, so that what is left of the iteration's residual lies in one direction, and with
+# W2's first column dominant that direction alone decides scales2, whose exact values are known (the first factor is on its grid, so
+# the target is W2).  Over the strengths of the row the residual before the last step passes through all of its range.
+def test_residual_in_one_direction():
+    import paper_2511_19705_b200 as cq
+    H = torch.ones(1, 1)
+    while H.shape[0] < 256:
+        H = torch.cat([torch.cat([H, H], 1), torch.cat([H, -H], 1)], 0)
+    g = torch.Generator().manual_seed(1)
+    V = torch.randn(256, 64, generator=g) * 0.01
+    V[:, 0] = 1 + torch.rand(256, generator=g)
+    W2 = V.bfloat16().cuda()
+    want = W2.double()[:, 0] / 127
+    for i in range(60):
+        W1 = H[:64].clone()
+        W1[0] *= 2.0 ** (-3 - i / 12)
+        o = cq.cafeq_adaptive_round(W1.bfloat16().cuda(), W2, None, iters=1, bits=8, group1=64, group2=64, k=64)
+        assert int(o["status"].item()) == 0
+        # the product W1 W2, its two target products and the last step round at fp32: 5.7e-7 with all updates made
+        assert ((o["scales2"].double()[:, 0] - want).abs() / want).max().item() <= 11 * 2.0 ** -24, i
+
+
 # A power of two on either factor changes exponents only.  Its fourth power is far outside fp32 here.
 @pytest.mark.parametrize("e1,e2", [(40, 0), (-40, 0), (0, 40), (0, -40), (55, -55), (-55, 55)])
 @pytest.mark.parametrize("case", ["full", "zero"])
