@@ -170,6 +170,9 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
     const int q = warp & 3, part = (warp - 2) >> 2;
     bool ok = mbar_wait(cta.bar_acc, tiles & 1u, cta.abort_flag, p.status);
     ok = __all_sync(0xffffffffu, ok);
+    float sum = 0.f, av = 0.f, us = 0.f;  // scale path: over this warp's 64 columns; the group's record
+    const int row = m0 + q * 32 + lane;
+    float* half = reinterpret_cast<float*>(cta.smem) + (part >> 1) * 128 + q * 32;
     if (ok) {
       tc_fence_after();
       const uint32_t taddr = cta.tmem + ((uint32_t)(q * 32) << 16);
@@ -178,14 +181,14 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
       uint16_t* tl = sh.sym ? (ti != tj ? p.Clo : nullptr) : p.Ctlo;
       double sq = 0.0;
       float* tile = reinterpret_cast<float*>(cta.smem + (warp - 2) * 4608);  // [32][36] per warp (the slots are free now)
-#pragma unroll 1
       if (ste) {
         // this warp's 64 of 256 columns: a group of 64, or with the next warp one of 128
-        const int row = m0 + q * 32 + lane, col = at.b * 256 + part * 64;
+        const int col = at.b * 256 + part * 64;
         const bool rv = row < p.M;
-        const long long rec = (long long)(col / ste->g) * p.M + row;
-        const float av = rv ? ste->a[rec] : 0.f, us = rv ? ste->usel[rec] : 0.f;
-        float sum = 0.f;
+        if (rv) {
+          av = ste->a[(long long)(col / ste->g) * p.M + row];
+          us = ste->usel[(long long)(col / ste->g) * p.M + row];
+        }
 #pragma unroll 1
         for (int c8 = 0; c8 < 4; ++c8) {  // 16 columns
           const long long o = (long long)row * ste->ld + col + c8 * 16;
@@ -210,16 +213,7 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
           }
         }
         sum *= p.alpha;
-        if (ste->g == 128) {
-          float* half = reinterpret_cast<float*>(cta.smem) + (part >> 1) * 128 + q * 32;
-          if (part & 1) half[lane] = sum;
-          asm volatile("bar.sync %0, 64;" ::"r"(1 + (part >> 1) * 4 + q) : "memory");
-          if (!(part & 1)) sum += half[lane];
-        }
-        if (rv && (ste->g == 64 || !(part & 1))) {
-          const float sgn = (us > 0.f) ? 1.f : ((us < 0.f) ? -1.f : 0.f);
-          ste->coef[rec] = (av > 0.f) ? sgn * sum / av : 0.f;
-        }
+        if (ste->g == 128 && (part & 1)) half[lane] = sum;
       } else if (sh.split) {
         // part of a contraction: added to C (M, N multiples of 32, ldc a multiple of 4)
 #pragma unroll 1
@@ -258,6 +252,16 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
       if (p.sq) {
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         if (lane == 0 && sq != 0.0) atomicAdd(sq_acc, (sh.sym && ti != tj) ? 2.0 * sq : sq);
+      }
+    }
+    if (ste) {
+      // The warps of a group of 128 meet whether or not their waits succeeded: this barrier has no limit of its own.
+      __syncwarp();
+      if (ste->g == 128) asm volatile("bar.sync %0, 64;" ::"r"(1 + (part >> 1) * 4 + q) : "memory");
+      if (ok && row < p.M && (ste->g == 64 || !(part & 1))) {
+        if (ste->g == 128) sum += half[lane];
+        const float sgn = (us > 0.f) ? 1.f : ((us < 0.f) ? -1.f : 0.f);
+        ste->coef[(long long)((at.b * 256 + part * 64) / ste->g) * p.M + row] = (av > 0.f) ? sgn * sum / av : 0.f;
       }
     }
   }

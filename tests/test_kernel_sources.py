@@ -82,3 +82,25 @@ def test_no_launch_result_is_dropped(path):
     dropped = re.findall(r"[;{})]\s*((?:%s)\s*\([^;{}]*;)" % RETURNING, _strip(open(path).read()))
     assert not dropped, dropped
     assert not re.search(r"static void (%s)\(" % RETURNING, _strip(open(path).read()))
+
+
+def _enclosing(text, pos):
+    """Heads of the blocks that the position lies in, the innermost first."""
+    heads, depth = [], 0
+    for j in range(pos - 1, -1, -1):
+        if text[j] == "}":
+            depth += 1
+        elif text[j] == "{":
+            if depth == 0:
+                heads.append(re.split(r"[;{}]", text[:j])[-1].strip())
+            else:
+                depth -= 1
+    return heads
+
+
+@pytest.mark.parametrize("path", sorted(glob.glob(os.path.join(CSRC, "*.cu*"))), ids=os.path.basename)
+def test_named_barriers_do_not_depend_on_a_wait(path):
+    """A bounded wait may give up in one warp and succeed in another; a barrier that only the second reaches has no limit."""
+    text = _strip(open(path).read())
+    for m in re.finditer(r"bar\.sync|barrier\.sync", text):
+        assert not [h for h in _enclosing(text, m.start()) if re.match(r"(else )?if \(.*\b(ok|mbar_wait)\b", h)]
