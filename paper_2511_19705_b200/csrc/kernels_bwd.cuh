@@ -422,18 +422,21 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
 // layer.)  A tile holds eight products: every wait of the issuing warp costs it some 400 cycles.
 // Both forms of a 9B-shaped layer, back to back: 102 us, issued by one elected lane of a converged warp 91, pairs 79.
 // ------------------------------------------------------------------------------------------------
-constexpr int BP_THREADS = 64 + 256 + 128;  // warp 0: TMA, warp 1: MMA, warps 2-9: operand builders, warps 10-13: flush
+constexpr int BP_THREADS = 64 + 256 + 128 + 64;  // warp 0: TMA, warp 1: MMA, warps 2-9: operand builders, 10-13: flush, 14-15: relays
 
 template <int F16>
 struct BpCfg {
   static constexpr int TERMS = F16 ? 1 : 2;
-  static constexpr int NSTAGE = F16 ? 4 : 2;
+  // A third S buffer, for one stage of the weights, where there is room: the relays (below) add more than a tile's time to an S tile's
+  // way to the products.
+  static constexpr int NSTAGE = F16 ? 3 : 2;
+  static constexpr int NBUF = F16 ? 3 : 2;
   static constexpr int STAGE_BYTES = 32768;   // 128 contraction entries x 128 of K
   static constexpr int S_TERM_BYTES = 32768;  // 128 targets x 128 contraction entries, K-major, two swizzle atoms of 64 entries
   static constexpr int S_BUF_BYTES = TERMS * S_TERM_BYTES;
   static constexpr int RDEPTH = 4;
   static constexpr int REC_BYTES = RDEPTH * 256 * 8;
-  static constexpr int SMEM = 1024 + NSTAGE * STAGE_BYTES + 2 * S_BUF_BYTES + REC_BYTES + 256;
+  static constexpr int SMEM = 1024 + NSTAGE * STAGE_BYTES + NBUF * S_BUF_BYTES + REC_BYTES + 256;
 };
 
 template <int FORM, int SWAP, int F16>
@@ -454,17 +457,18 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sStage = smem;
   uint8_t* sS = smem + C::NSTAGE * C::STAGE_BYTES;
-  uint8_t* sRec = sS + 2 * C::S_BUF_BYTES;
+  uint8_t* sRec = sS + C::NBUF * C::S_BUF_BYTES;
   uint64_t* bars = (uint64_t*)(sRec + C::REC_BYTES);
-  // barrier slots: wfull[NSTAGE], wempty[NSTAGE], sfull[2], sempty[2], accf[2], acce[2]; wfull, sfull and acce are signalled by
-  // both CTAs and awaited in the leader, the others are signalled in both by the leader's commits
+  // barrier slots: wfull[NSTAGE], wempty[NSTAGE], sfull[NBUF], sempty[NBUF], accf[2], acce[2]; wfull and acce are signalled by both CTAs
+  // and awaited in the leader, sfull by the own builders (in the leader also by the other CTA's relay), the others are signalled in
+  // both by the leader's commits
   const uint32_t bar_wfull = smem_u32(bars);
   const uint32_t bar_wempty = bar_wfull + 8 * C::NSTAGE;
   const uint32_t bar_sfull = bar_wempty + 8 * C::NSTAGE;
-  const uint32_t bar_sempty = bar_sfull + 16;
-  const uint32_t bar_accf = bar_sempty + 16;
+  const uint32_t bar_sempty = bar_sfull + 8 * C::NBUF;
+  const uint32_t bar_accf = bar_sempty + 8 * C::NBUF;
   const uint32_t bar_acce = bar_accf + 16;
-  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * C::NSTAGE + 8);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * C::NSTAGE + 2 * C::NBUF + 4);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -474,9 +478,11 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
       mbar_init(bar_wfull + 8 * s, 1);
       mbar_init(bar_wempty + 8 * s, 1);
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(bar_sfull + 8 * b, 16);  // eight builder warps of each CTA
+    for (int b = 0; b < C::NBUF; ++b) {
+      mbar_init(bar_sfull + 8 * b, rank == 0 ? 9 : 8);  // eight builder warps, the relay
       mbar_init(bar_sempty + 8 * b, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
       mbar_init(bar_accf + 8 * b, 1);
       mbar_init(bar_acce + 8 * b, 8);    // four flush warps of each CTA
     }
@@ -486,7 +492,7 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
   // the S tiles start as zeros; afterwards the builders clear exactly what they wrote
   {
     uint4* z = reinterpret_cast<uint4*>(sS);
-    for (int e = threadIdx.x; e < 2 * C::S_BUF_BYTES / 16; e += BP_THREADS) z[e] = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = threadIdx.x; e < C::NBUF * C::S_BUF_BYTES / 16; e += BP_THREADS) z[e] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async_smem();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), 512u);
@@ -499,6 +505,20 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
     return;
   }
 
+  // Relay of S buffer b (in the CTA that does not issue): the products that the leader issues read this CTA's S tiles, so the builders'
+  // stores have to be released at the scope of the cluster.  That costs more than a tile's time (1 us), hence a warp for each buffer; from
+  // a builder the arrival would wait for its records in flight too.  Step of a 9B-shaped layer: arrivals at the scope of the CTA, which do
+  // not order those stores, 334 us; released by the builders 407, by one relay with two S buffers 352, with three 345, by a relay for each
+  // of three 342.
+  auto relay = [&](const uint32_t b) {
+    if (b >= (uint32_t)C::NBUF || lane != 0) return;
+    const uint32_t sfull0 = cluster_addr(bar_sfull, 0);
+    uint32_t bph = 0;
+    for (int gt = t_begin + (int)b; gt < t_end; gt += C::NBUF, bph ^= 1u) {
+      if (!mbar_wait(bar_sfull + 8 * b, bph, abort_flag, status)) break;
+      mbar_arrive_pair(sfull0 + 8 * b);
+    }
+  };
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer: this CTA's half of one weight tile per stage
     if (lane == 0) {
@@ -534,8 +554,8 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
       const uint32_t sSt_u = smem_u32(sStage), sS_u = smem_u32(sS);
       auto wait_all = [&](uint32_t bar, uint32_t ph) { return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_flag, status)) != 0; };
       int sub = s_first, left = 0;  // tiles of the current block left in its list
-      uint32_t run = 0, st = 0, sph = 0, it = 0;
-      for (int gt = t_begin; gt < t_end; ++gt, ++it) {
+      uint32_t run = 0, st = 0, sph = 0, b = 0, bph = 0;
+      for (int gt = t_begin; gt < t_end; ++gt) {
         while (gt >= mp.tile_end[sub]) ++sub;
         const bool first = left == 0;
         if (first) {
@@ -545,9 +565,8 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
           if (!wait_all(bar_acce + 8 * (run & 1u), ((run >> 1) & 1u) ^ 1u)) break;
           tc_fence_after();
         }
-        const uint32_t b = it & 1u, bph = (it >> 1) & 1u;
         if (!wait_all(bar_wfull + 8 * st, sph)) break;
-        if (!wait_all(bar_sfull + 8 * b, bph)) break;
+        if (!__all_sync(0xffffffffu, mbar_wait_pair(bar_sfull + 8 * b, bph, abort_flag, status))) break;
         tc_fence_after();
         // last tile of this block in this pair's run: hand the accumulator to the flush
         const bool last = --left == 0 || gt + 1 == t_end;
@@ -572,7 +591,10 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
         __syncwarp();
         if (last) ++run;
         if (++st == C::NSTAGE) { st = 0; sph ^= 1u; }
+        if (++b == C::NBUF) { b = 0; bph ^= 1u; }
       }
+    } else {
+      relay(0);
     }
   } else if (warp < 10) {
     // ---------------------------------------------------------------- operand builders: one record per thread and tile
@@ -617,10 +639,12 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
       cp_async_commit();
       ++pre;
     };
-    uint32_t prevA = BW_NONE, prevB = BW_NONE;  // offsets this thread wrote into S buffer 0 / 1
+    uint32_t before[C::NBUF];  // offsets this thread wrote into each S buffer
+#pragma unroll
+    for (int i = 0; i < C::NBUF; ++i) before[i] = BW_NONE;
+    uint32_t b = 0, bph = 1;
     int cur_sub = -1;
     float scale = 1.f;
-    const uint32_t sfull0 = cluster_addr(bar_sfull, 0);
     for (int i = 0; i < C::RDEPTH; ++i) request();
     for (uint32_t tl = 0; cur.gt < t_end; ++tl) {
       if constexpr (F16) {
@@ -640,12 +664,13 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
         const int tg = (FORM == BW_IN) ? col : rl, kk = (FORM == BW_IN) ? rl : col;
         now = bw_s_offset(tg, kk);
       }
-      const uint32_t b = tl & 1u, sph = (tl >> 1) & 1u;
-      bool ok = mbar_wait(bar_sempty + 8 * b, sph ^ 1u, abort_flag, status);
+      bool ok = mbar_wait(bar_sempty + 8 * b, bph, abort_flag, status);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       uint8_t* buf = sS + b * C::S_BUF_BYTES;
-      const uint32_t prev = b ? prevB : prevA;
+      uint32_t prev = before[0];
+#pragma unroll
+      for (int i = 1; i < C::NBUF; ++i) prev = b == i ? before[i] : prev;
       if (prev != BW_NONE) {
         *reinterpret_cast<uint16_t*>(buf + prev) = 0;
         if constexpr (!F16) *reinterpret_cast<uint16_t*>(buf + C::S_TERM_BYTES + prev) = 0;
@@ -661,12 +686,16 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
           *reinterpret_cast<uint16_t*>(buf + C::S_TERM_BYTES + now) = __bfloat16_as_ushort(lo);
         }
       }
-      if (b) prevB = now; else prevA = now;
+#pragma unroll
+      for (int i = 0; i < C::NBUF; ++i) before[i] = b == i ? now : before[i];
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(sfull0 + 8 * b);
+      if (lane == 0) mbar_arrive(bar_sfull + 8 * b);
+      if (++b == C::NBUF) { b = 0; bph ^= 1u; }
       request();
     }
+  } else if (warp >= 14) {
+    if (rank != 0) relay(warp - 13);
   } else {
     // ---------------------------------------------------------------- flush: accumulators -> global memory, coalesced atomic adds
     const int q = warp & 3;
@@ -695,7 +724,7 @@ __device__ __forceinline__ void bd_bwd_pair_body(const BwMaps& maps, const BwMul
         if (ch == 7) {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(acce0 + 8 * (run & 1u));
+          if (lane == 0) mbar_arrive_pair_tmem(acce0 + 8 * (run & 1u));
         }
 #pragma unroll
         for (int c = 0; c < 32; ++c)

@@ -454,7 +454,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
           tc_fence_before();
           __syncwarp();
           if (lane == 0) {
-            if constexpr (PAIR) mbar_arrive_cluster(cluster_addr(bar_acce + 8 * buf, 0));
+            if constexpr (PAIR) mbar_arrive_pair_tmem(cluster_addr(bar_acce + 8 * buf, 0));
             else mbar_arrive(bar_acce + 8 * buf);
           }
         };

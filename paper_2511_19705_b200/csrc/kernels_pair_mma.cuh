@@ -33,10 +33,32 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-// Arrival at a barrier of either CTA, with CTA scope: what it orders are reads of tensor memory (tcgen05 fences).  With cluster scope
-// it waits until the thread's global stores have landed, 2100 cycles a tile in the transform pass.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+// Arrival at a barrier of either CTA after stores to shared memory that the other CTA's products read: releases them at the scope of
+// the cluster, and the barrier is awaited with mbar_wait_pair.  It also waits until the thread's global stores have landed.
+__device__ __forceinline__ void mbar_arrive_pair(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// Arrival after reads of tensor memory only (ordered by the tcgen05 fences): CTA scope.  With the scope of the cluster it waits for
+// the thread's global stores, 2100 cycles a tile in the transform pass.
+__device__ __forceinline__ void mbar_arrive_pair_tmem(uint32_t addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+struct PairAcquire {
+  static __device__ __forceinline__ uint32_t try_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok;
+  }
+};
+// bounded wait for arrivals of both CTAs (mbar_arrive_pair)
+__device__ __forceinline__ bool mbar_wait_pair(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
+  return mbar_wait<PairAcquire>(bar, parity, abort_flag, status);
 }
 
 // Whether either CTA of the pair saw a raised status word: one answer for both (a CTA that left alone would leave the other

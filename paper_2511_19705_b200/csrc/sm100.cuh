@@ -40,13 +40,17 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
+struct CtaAcquire {
+  static __device__ __forceinline__ uint32_t try_wait(uint32_t bar, uint32_t parity) { return mbar_try_wait(bar, parity); }
+};
 // Bounded wait: false when the limit ran out here or in another role (abort flag).
+template <typename Acquire = CtaAcquire>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                           uint64_t limit_ns = BD_WAIT_NS) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (Acquire::try_wait(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
   for (uint32_t spin = 0;; ++spin) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (Acquire::try_wait(bar, parity)) return true;
     if ((spin & 63u) == 63u) {
       if (*abort_flag) return false;
       if (global_timer_ns() - t0 > limit_ns) {

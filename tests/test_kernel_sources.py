@@ -104,3 +104,14 @@ def test_named_barriers_do_not_depend_on_a_wait(path):
     text = _strip(open(path).read())
     for m in re.finditer(r"bar\.sync|barrier\.sync", text):
         assert not [h for h in _enclosing(text, m.start()) if re.match(r"(else )?if \(.*\b(ok|mbar_wait)\b", h)]
+
+
+def test_operands_for_the_other_cta_are_released_at_cluster_scope():
+    """The issuing CTA of a pair multiplies what the other CTA's builders stored: the builders' arrivals and the issuer's wait order
+    those stores for it only at the scope of the cluster."""
+    text = _strip(open(os.path.join(CSRC, "kernels_bwd.cuh")).read())
+    body = text[text.index("void bd_bwd_pair_body"):text.index("constexpr int bw_threads")]
+    assert re.findall(r"(mbar_\w+)\(sfull0", body) == ["mbar_arrive_pair"]
+    assert re.findall(r"(mbar_wait\w*|wait_all)\(bar_sfull", body) == ["mbar_wait_pair"]
+    pair = _strip(open(os.path.join(CSRC, "kernels_pair_mma.cuh")).read())
+    assert "mbarrier.arrive.release.cluster.shared::cluster" in pair and "try_wait.parity.acquire.cluster" in pair
