@@ -107,11 +107,12 @@ def test_named_barriers_do_not_depend_on_a_wait(path):
 
 
 def test_operands_for_the_other_cta_are_released_at_cluster_scope():
-    """The issuing CTA of a pair multiplies what the other CTA's builders stored: the builders' arrivals and the issuer's wait order
-    those stores for it only at the scope of the cluster."""
+    """The issuing CTA of a pair multiplies what the other CTA's builders stored: what arrives there on their behalf, and its wait, order
+    those stores for it only at the scope of the cluster.  The builders themselves arrive in their own CTA, where a relay waits."""
     text = _strip(open(os.path.join(CSRC, "kernels_bwd.cuh")).read())
     body = text[text.index("void bd_bwd_pair_body"):text.index("constexpr int bw_threads")]
     assert re.findall(r"(mbar_\w+)\(sfull0", body) == ["mbar_arrive_pair"]
-    assert re.findall(r"(mbar_wait\w*|wait_all)\(bar_sfull", body) == ["mbar_wait_pair"]
+    assert sorted(re.findall(r"(mbar_wait\w*|wait_all)\(bar_sfull", body)) == ["mbar_wait", "mbar_wait_pair"]
+    assert re.findall(r"(mbar_arrive\w*)\(bar_sfull", body) == ["mbar_arrive"]
     pair = _strip(open(os.path.join(CSRC, "kernels_pair_mma.cuh")).read())
     assert "mbarrier.arrive.release.cluster.shared::cluster" in pair and "try_wait.parity.acquire.cluster" in pair
