@@ -293,6 +293,19 @@ static void launch_split(cudaStream_t st, const float* X, int k, long long n, ui
   CQ_LAUNCH(split_bf16_kernel, grid, dim3(32, 8), 0, st, X, k, hi, lo, thi, tlo, status);
 }
 
+// Batched products of 256 x 256 with their contraction in parts (tg_launch_split; parts: scratch for K / 256 * reps * batch of them), summed
+// into out and, optionally, its splits.
+static bool split_wanted(int k, int K) { return k == 256 && K >= 256; }
+static int launch_split_product(cudaStream_t st, int na, const TgOperand* A, int nb, const TgOperand* B, int K, int batch, int reps, int mn,
+                                float* parts, float* out, uint16_t* hi, uint16_t* lo, int32_t* status) {
+  int n = 0;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  const int rc = tg_launch_split(st, na, A, nb, B, K, batch, reps, mn, 1.f, parts, &n, status);
+  if (rc) return rc;
+  CQ_LAUNCH(sum_parts_kernel, 64u * (unsigned)batch, 256, 0, st, parts, n, out, hi, lo, status);
+  return CAFEQ_OK;
+}
+
 // Minv = inv(bf16(M)).  k = 128, 256: Newton-Schulz iteration X <- X + X (I - A X) on the tensor cores, every round of a block
 // in one launch, from X0 = A^T (cold: right for the near-orthogonal transforms the method starts from) or from the caller's
 // previous inverse (warm); a warm start runs as many rounds as the step size calls for (a block whose residual ||I - A X||_F
@@ -1068,12 +1081,9 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     // apply), and the scale path needs sum_e gDelta_e Delta_e per group.  Every product runs on the tensor cores
     // with the residual as a two-term bf16 split (three-term products: fp32-grade).
     KkWS& w = s.kk;
-    if (k == 256) {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the d_out rows of the residual as it is stored
+    if (split_wanted(k, G.d_out)) {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the rows of the residual as it is stored
       const TgOperand o[2] = {TgOperand{s.m.Dbf, G.d_out, G.d_in, G.d_in}, TgOperand{s.Dlo, G.d_out, G.d_in, G.d_in}};
-      CQ_LAUNCH(fill_f32_kernel, grid_for(kk), 256, 0, st, s.tmp, 0.f, kk);
-      g_launches.fetch_add(1, std::memory_order_relaxed);
-      if ((s.err = tg_launch_split(st, 2, o, 2, o, G.d_out, G.nbT, 1, 1, 1.f, s.tmp, status))) return;
-      launch_split(st, s.tmp, k, kk, w.Ph, w.Pl, nullptr, nullptr, status);
+      if ((s.err = launch_split_product(st, 2, o, 2, o, G.d_out, G.nbT, 1, 1, s.m.D, s.tmp, w.Ph, w.Pl, status))) return;
     } else {
       TgOperand oa[3], ob[3];
       const uint16_t* at[3] = {s.m.Dbf, s.Dlo, s.m.Dbf};
@@ -1370,15 +1380,15 @@ struct PairWS {
 
 // Operator gradients of a block-diagonal apply as batched k x k tensor-core products with a two-term split of the fp32 factor.
 // Output axis: out[b][m][n] = sum_l A[b k + m][l] (Bh + Bl)[b k + n][l]; A bf16 [nb k, K] (pitch lda), Bh / Bl [nb k, K].
+// parts: scratch of nb k K floats.
 static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, const uint16_t* Bh, const uint16_t* Bl, int nb, int k, int K,
-                         float* out, int32_t* status) {
+                         float* parts, float* out, int32_t* status) {
   TgOperand oa[2], ob[2];
-  if (k == 256) {  // (out was cleared: parts of the contraction are added)
+  if (split_wanted(k, K)) {
     oa[0] = TgOperand{A, (long long)nb * k, K, lda};
     ob[0] = TgOperand{Bh, (long long)nb * k, K, K};
     ob[1] = TgOperand{Bl, (long long)nb * k, K, K};
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return tg_launch_split(st, 1, oa, 2, ob, K, nb, 1, 0, 1.f, out, status);
+    return launch_split_product(st, 1, oa, 2, ob, K, nb, 1, 0, parts, out, nullptr, nullptr, status);
   }
   oa[0] = oa[1] = TgOperand{A, (long long)nb * k, K, lda};
   ob[0] = TgOperand{Bl, (long long)nb * k, K, K};
@@ -1396,14 +1406,14 @@ static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, cons
   return tg_launch(st, oa, ob, p);
 }
 // Input axis: out[b][m][n] = sum over replicas and rows o of (Ah + Al)[o][(b r + rep) k + m] B[o][(b r + rep) k + n]; both
-// factors as they are stored (contraction down the rows: MN-major operands), B bf16 [R, nb r k] (pitch ldb), Ah / Al dense.
+// factors as they are stored (contraction down the rows: MN-major operands), B bf16 [R, nb r k] (pitch ldb), Ah / Al dense.  parts: scratch
+// of R nb r k floats.
 static int opgrad_in_tc(cudaStream_t st, const uint16_t* Ah, const uint16_t* Al, const uint16_t* B, long long ldb, int nb, int r, int k,
-                        int R, float* out, int32_t* status) {
-  if (k == 256) {  // (as above; the replicas' parts as well)
+                        int R, float* parts, float* out, int32_t* status) {
+  if (split_wanted(k, R)) {
     const long long all = (long long)nb * r * k;
     const TgOperand a[2] = {TgOperand{Ah, R, all, all}, TgOperand{Al, R, all, all}}, b = TgOperand{B, R, all, ldb};
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return tg_launch_split(st, 2, a, 1, &b, R, nb, r, 1, 1.f, out, status);
+    return launch_split_product(st, 2, a, 1, &b, R, nb, r, 1, parts, out, nullptr, nullptr, status);
   }
   for (int rep = 0; rep < r; ++rep) {
     TgOperand oa[2], ob[2];
@@ -1645,12 +1655,13 @@ static void pair_step(cudaStream_t st, const cafeq_matrix_desc* d1, const cafeq_
     const bool og_tc = tc && ((uintptr_t)W1 % 16 == 0) && (G1.ld % 8 == 0) && ((uintptr_t)W2 % 16 == 0) && (G2.ld % 8 == 0) && G1.r == 1 &&
                        ste_split_ok(G1.g) && ste_split_ok(G2.g);
     if (og_tc) {
+      // (the parts' scratch: w.U, when its splits have been taken, and w.V, which this path does not use)
       // U side (operator M^T): gradM[b][m][n] = sum_c W1[b k + m][c] gU[b k + n][c]
       launch_ste_split(st, p.m1, w.U, w.d1, G1, k, 1, qmax_of(d1->bits), w.Awh, w.Awl, status);
-      if ((p.err = opgrad_out_tc(st, (const uint16_t*)W1, G1.ld, w.Awh, w.Awl, G1.nbT, k, G1.d_in, gradM, status))) return;
+      if ((p.err = opgrad_out_tc(st, (const uint16_t*)W1, G1.ld, w.Awh, w.Awl, G1.nbT, k, G1.d_in, w.U, gradM, status))) return;
       // V side (operator Minv): gMinv[b][i][j] = sum over replicas and rows o of gV[o][.. + i] W2[o][.. + j]
       launch_ste_split(st, p.m2, w.X0T, w.h, G2, k, G2.r, qmax_of(d2->bits), p.gVh, p.gVl, status);
-      if ((p.err = opgrad_in_tc(st, p.gVh, p.gVl, (const uint16_t*)W2, G2.ld, G1.nbT, G2.r, k, G2.d_out, p.gMinv, status))) return;
+      if ((p.err = opgrad_in_tc(st, p.gVh, p.gVl, (const uint16_t*)W2, G2.ld, G1.nbT, G2.r, k, G2.d_out, w.V, p.gMinv, status))) return;
     } else {
       CQ_LAUNCH(expand_cols_kernel, dim3(w.d3, (w.h + 1023) / 1024), 256, 0, st, w.X0T, w.h, w.k, w.r, 1.f, w.V);
       const long long n1w = (long long)G1.d_out * G1.ng, n2w = (long long)G2.d_out * G2.ng;

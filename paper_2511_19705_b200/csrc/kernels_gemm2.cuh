@@ -29,7 +29,7 @@ struct T2Shape {
   int na, nb, nterms;
   int nstage;     // T2_NSLOT / (na + nb)
   int two;        // terms with ac = 1 have the second accumulator
-  int split;      // the product is one part of a contraction: alpha times it is added to C, nothing else is done
+  int split;      // the product is one part of a contraction: alpha times it is stored in C, nothing else is done
   int8_t ta[T2_MAX_TERMS], tb[T2_MAX_TERMS], ac[T2_MAX_TERMS];
 };
 struct T2Maps {
@@ -215,7 +215,7 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
         sum *= p.alpha;
         if (ste->g == 128 && (part & 1)) half[lane] = sum;
       } else if (sh.split) {
-        // part of a contraction: added to C (M, N multiples of 32, ldc a multiple of 4)
+        // part of a contraction (M, N multiples of 32; C and its pitch of 16 bytes)
 #pragma unroll 1
         for (int ch = part; ch < bn / 32; ch += TG_EPI_PARTS) {
           if (n0 + ch * 32 >= p.N || m0 + q * 32 >= p.M) break;
@@ -232,17 +232,11 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
             *reinterpret_cast<float4*>(tile + lane * 36 + 4 * j) =
                 make_float4(p.alpha * v[4 * j], p.alpha * v[4 * j + 1], p.alpha * v[4 * j + 2], p.alpha * v[4 * j + 3]);
           __syncwarp();
-          float* out = p.C + (long long)at.b * p.sCb + (long long)(m0 + q * 32) * p.ldc + n0 + ch * 32;
-          if (((uintptr_t)p.C & 15) == 0) {
-            out += (long long)(lane >> 3) * p.ldc + (lane & 7) * 4;
+          float* out = p.C + (long long)at.b * p.sCb + (long long)(m0 + q * 32 + (lane >> 3)) * p.ldc + n0 + ch * 32 + (lane & 7) * 4;
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              atomicAdd(reinterpret_cast<float4*>(out + (long long)(4 * i) * p.ldc),
-                        *reinterpret_cast<const float4*>(tile + (i * 4 + (lane >> 3)) * 36 + (lane & 7) * 4));
-          } else {  // (a caller's gradient at any float address)
-#pragma unroll 1
-            for (int i = 0; i < 32; ++i) atomicAdd(out + (long long)i * p.ldc + lane, tile[i * 36 + lane]);
-          }
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<float4*>(out + (long long)(4 * i) * p.ldc) =
+                *reinterpret_cast<const float4*>(tile + (i * 4 + (lane >> 3)) * 36 + (lane & 7) * 4);
           __syncwarp();
         }
       } else
@@ -380,9 +374,10 @@ pinv_loop_kernel(const __grid_constant__ T2LoopMaps maps, const __grid_constant_
 }
 
 // Batched 256 x 256 products with a long contraction (Gram matrices and operator gradients of blocks of 256): every pair takes a
-// slice of one block's contraction (and one of `reps` column blocks that are summed) and adds its product to C, which the caller
-// has cleared.  As tiles of 64 columns with the whole contraction each, 14 blocks had 112 CTAs with 64 chunks of three terms in a
-// row, 66 us; 70 pairs with 13 chunks take 18.
+// slice of one block's contraction (and one of `reps` column blocks that are summed) and stores its product as a part of its own;
+// sum_parts_kernel adds a block's parts in their order, so that a call repeats itself bit for bit.  As tiles of 64 columns with
+// the whole contraction each, 14 blocks had 112 CTAs with 64 chunks of three terms in a row, 66 us.  Straight-through gradient of the
+// 9B-shaped v-o pair 792 -> 729 us (its parts added atomically, in no fixed order: 721).
 __global__ void __launch_bounds__(TG_THREADS, 1)
 tc_pair_split_kernel(const __grid_constant__ T2Maps maps, const __grid_constant__ TgParams p, const __grid_constant__ T2Shape sh,
                      const int reps, const int slices) {
@@ -396,8 +391,43 @@ tc_pair_split_kernel(const __grid_constant__ T2Maps maps, const __grid_constant_
   if (!t2_enter(cta, smem_raw, raised)) return;
   const int blk = b * reps + rep;
   t2_tile(cta, maps.a[0], maps.b, p, sh, nullptr, 0, 0,
-          T2At{blk * p.colsA_per_batch, blk * p.rowsA_per_batch, blk * p.colsB_per_batch, blk * p.rowsB_per_batch, c0, c1 - c0, b}, 0, 0);
+          T2At{blk * p.colsA_per_batch, blk * p.rowsA_per_batch, blk * p.colsB_per_batch, blk * p.rowsB_per_batch, c0, c1 - c0, unit}, 0, 0);
   if ((threadIdx.x >> 5) == 1) tmem_free_pair(cta.tmem, 512u);
+}
+
+// out[b] = sum of its n parts, in their order (blocks of 256 x 256), and optionally its bf16 splits.  Four entries a thread (grid: 64 per
+// block), the parts' loads in flight together; bound by reading the parts from L2.
+__global__ void __launch_bounds__(256) sum_parts_kernel(const float* parts, int n, float* __restrict__ out, uint16_t* __restrict__ hi,
+                                                        uint16_t* __restrict__ lo, const int32_t* status) {
+  pdl_enter();
+  if (cta_stopped(status)) return;
+  const long long b = blockIdx.x >> 6;
+  const int e = ((blockIdx.x & 63) * 256 + threadIdx.x) * 4;
+  const float* p = parts + b * n * 65536 + e;
+  float4 s = ld_plain(reinterpret_cast<const float4*>(p));
+#pragma unroll 8
+  for (int i = 1; i < n; ++i) {
+    const float4 x = ld_plain(reinterpret_cast<const float4*>(p + (long long)i * 65536));
+    s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+  }
+  const long long o = b * 65536 + e;
+  if (((uintptr_t)out & 15) == 0) {
+    *reinterpret_cast<float4*>(out + o) = s;
+  } else {  // (a caller's gradient at any float address)
+    out[o] = s.x; out[o + 1] = s.y; out[o + 2] = s.z; out[o + 3] = s.w;
+  }
+  if (hi) {
+    const float x[4] = {s.x, s.y, s.z, s.w};
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const __nv_bfloat16 t = __float2bfloat16_rn(x[j]);
+      h[j] = __bfloat16_as_ushort(t);
+      l[j] = __bfloat16_as_ushort(__float2bfloat16_rn(x[j] - __bfloat162float(t)));
+    }
+    *reinterpret_cast<uint2*>(hi + o) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+    *reinterpret_cast<uint2*>(lo + o) = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+  }
 }
 
 // Scale path of the straight-through gradient on blocks of 256: v = alpha * (hi + lo) N_b over the columns of block b, reduced to one
@@ -500,14 +530,10 @@ static bool t2_wanted(int M, int N, double cost) {
   return cost < tiled;
 }
 
-static int t2_split_launch(cudaStream_t st, const T2Maps& maps, const TgParams& p, const T2Shape& sh, int reps) {
-  static std::atomic<unsigned long long> done{0};
-  if (!opt_in_smem(tc_pair_split_kernel, T2_SMEM, done)) return CAFEQ_ERR_CUDA;
-  const int units = p.batch * reps, all = (p.K + TG_BK - 1) / TG_BK;
-  int slices = units < 74 ? 74 / units : 1;
-  if (slices > all / 4) slices = all / 4 > 0 ? all / 4 : 1;  // (four chunks at least: a tile's fixed part is some 8 us)
-  launch_pairs_if(true, tc_pair_split_kernel, units * slices, TG_THREADS, T2_SMEM, st, maps, p, sh, reps, slices);
-  return CAFEQ_OK;
+// Slices of a contraction of length K in 74 / units parts, of 256 entries at least (a tile's fixed part is some 8 us).
+static int t2_slices(int units, int K) {
+  const int s = units < 74 ? 74 / units : 1, most = K / 256;
+  return s < most ? s : (most > 0 ? most : 1);
 }
 
 // Dh / Dl: [M, nb * 256] (pitch ste.ld); Nh / Nl: blocks [nb * 256, 256]
@@ -532,9 +558,12 @@ static int tg_launch_ste(cudaStream_t st, const uint16_t* Nh, const uint16_t* Nl
 }
 
 // A: na arrays, B: nb arrays, each [rows, cols] with its pitch, either both stored with the contraction as rows (mn: [K, blocks * 256])
-// or both with it as columns ([blocks * 256, K]); C += alpha * sum over the column (row) blocks b * reps .. of A_b B_b^T.
+// or both with it as columns ([blocks * 256, K]).  Parts of alpha * sum over the column (row) blocks b * reps .. of A_b B_b^T: `count` of
+// them for each of the `batch` blocks in a row, 65536 floats each (at most K / 256 * reps * batch of them; K >= 256).
 static int tg_launch_split(cudaStream_t st, int na, const TgOperand* A, int nb, const TgOperand* B, int K, int batch, int reps, int mn,
-                           float alpha, float* C, int32_t* status) {
+                           float alpha, float* parts, int* count, int32_t* status) {
+  static std::atomic<unsigned long long> done{0};
+  if (!opt_in_smem(tc_pair_split_kernel, T2_SMEM, done)) return CAFEQ_ERR_CUDA;
   T2Maps maps;
   memset(&maps, 0, sizeof(maps));
   bool ok = true;
@@ -548,11 +577,14 @@ static int tg_launch_split(cudaStream_t st, int na, const TgOperand* A, int nb, 
   if (mn) p.colsA_per_batch = p.colsB_per_batch = 256;
   else p.rowsA_per_batch = p.rowsB_per_batch = 256;
   p.alpha = alpha;
-  p.C = C; p.ldc = 256; p.sCb = 65536;
+  p.C = parts; p.ldc = 256; p.sCb = 65536;
   p.status = status;
   T2Shape sh = t2_shape(256, 256, 256, na, nb, na > nb ? na : nb);
   sh.split = 1;
-  return t2_split_launch(st, maps, p, sh, reps);
+  const int units = batch * reps, slices = t2_slices(units, K);
+  *count = reps * slices;
+  launch_pairs_if(true, tc_pair_split_kernel, units * slices, TG_THREADS, T2_SMEM, st, maps, p, sh, reps, slices);
+  return CAFEQ_OK;
 }
 
 }  // namespace cafeq
