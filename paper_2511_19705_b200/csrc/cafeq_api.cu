@@ -295,7 +295,13 @@ static void launch_split(cudaStream_t st, const float* X, int k, long long n, ui
 
 // Batched products of 256 x 256 with their contraction in parts (tg_launch_split; parts: scratch for K / 256 * reps * batch of them), summed
 // into out and, optionally, its splits.
-static bool split_wanted(int k, int K) { return k == 256 && K >= 256; }
+// Against tiles with the whole contraction each (8 CTAs a block, K / 64 chunks in a row, some 0.8 us a chunk) the parts cost a longer
+// first tile, a launch, and a trip of 256 KB each.  Measured, tiles -> parts, Eq. 3 straight-through: blocks x K 1 x 256 188.7 -> 193.0
+// us, 4 x 700 205 -> 205, 4 x 1024 214 -> 209, 14 x 1024 225 -> 230, 8 x 1500 221 -> 212, 74 x 512 301 -> 304, 14 x 4096 348 -> 312;
+// Eq. 5: 16 x 1024 359 -> 364, 8 x 2048 327 -> 313, 8 x 3584 with two replicas 792 -> 729.
+static bool split_wanted(int k, int K, int batch, int reps) {
+  return k == 256 && K >= 256 && K / 64 >= 12 + batch * reps * t2_slices(batch * reps, K) / 8;
+}
 static int launch_split_product(cudaStream_t st, int na, const TgOperand* A, int nb, const TgOperand* B, int K, int batch, int reps, int mn,
                                 float* parts, float* out, uint16_t* hi, uint16_t* lo, int32_t* status) {
   int n = 0;
@@ -1081,7 +1087,7 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
     // apply), and the scale path needs sum_e gDelta_e Delta_e per group.  Every product runs on the tensor cores
     // with the residual as a two-term bf16 split (three-term products: fp32-grade).
     KkWS& w = s.kk;
-    if (split_wanted(k, G.d_out)) {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the rows of the residual as it is stored
+    if (split_wanted(k, G.d_out, G.nbT, 1)) {  // Gram (fp32 in s.tmp, splits in w.Ph / w.Pl): contraction over the rows of the residual as it is stored
       const TgOperand o[2] = {TgOperand{s.m.Dbf, G.d_out, G.d_in, G.d_in}, TgOperand{s.Dlo, G.d_out, G.d_in, G.d_in}};
       if ((s.err = launch_split_product(st, 2, o, 2, o, G.d_out, G.nbT, 1, 1, s.m.D, s.tmp, w.Ph, w.Pl, status))) return;
     } else {
@@ -1128,8 +1134,10 @@ static void single_step(cudaStream_t st, const cafeq_matrix_desc* d, const Geo& 
       if ((s.err = launch_kk_tc(st, 3, a2, b2, G.nbT, k, 2.f, 0.f, 0.f, nullptr, s.gMinv, nullptr, nullptr, nullptr, nullptr, nullptr,
                    status))) return;
     }
-    // gDelta[o, B k + j] = 2 sum_l N_B[j][l] Delta[o, B k + l], and per group the sum of gDelta Delta
-    if (k == 256) {
+    // gDelta[o, B k + j] = 2 sum_l N_B[j][l] Delta[o, B k + l], and per group the sum of gDelta Delta.  Blocks of 256 from 2^21 entries
+    // on: as the product's epilogue (256 x 512 188.8 -> 193.0 us a call, 1024 x 1024 206.8 -> 209.0, 4096 x 512 206.6 -> 206.4,
+    // 1500 x 2048 219 -> 212, 4096 x 3584 328 -> 312).
+    if (k == 256 && G.n >= 1ll << 21) {
       const T2Ste ste{s.m.Dbf, s.Dlo, G.d_in, s.m.a, s.m.usel, s.m.coef, G.g};
       g_launches.fetch_add(1, std::memory_order_relaxed);
       if ((s.err = tg_launch_ste(st, w.Qh, w.Ql, G.d_out, G.nbT, 2.f, ste, status))) return;
@@ -1384,7 +1392,7 @@ struct PairWS {
 static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, const uint16_t* Bh, const uint16_t* Bl, int nb, int k, int K,
                          float* parts, float* out, int32_t* status) {
   TgOperand oa[2], ob[2];
-  if (split_wanted(k, K)) {
+  if (split_wanted(k, K, nb, 1)) {
     oa[0] = TgOperand{A, (long long)nb * k, K, lda};
     ob[0] = TgOperand{Bh, (long long)nb * k, K, K};
     ob[1] = TgOperand{Bl, (long long)nb * k, K, K};
@@ -1410,7 +1418,7 @@ static int opgrad_out_tc(cudaStream_t st, const uint16_t* A, long long lda, cons
 // of R nb r k floats.
 static int opgrad_in_tc(cudaStream_t st, const uint16_t* Ah, const uint16_t* Al, const uint16_t* B, long long ldb, int nb, int r, int k,
                         int R, float* parts, float* out, int32_t* status) {
-  if (split_wanted(k, R)) {
+  if (split_wanted(k, R, nb, r)) {
     const long long all = (long long)nb * r * k;
     const TgOperand a[2] = {TgOperand{Ah, R, all, all}, TgOperand{Al, R, all, all}}, b = TgOperand{B, R, all, ldb};
     return launch_split_product(st, 2, a, 1, &b, R, nb, r, 1, parts, out, nullptr, nullptr, status);

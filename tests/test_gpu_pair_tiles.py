@@ -65,3 +65,28 @@ def test_codes(axis, d_out, d_in):
     c = codes.double().reshape(x.shape)
     # a code may differ from the rounded quotient only where that lies next to a half-integer: sums of 256 terms in fp32
     assert ((c - q).abs() <= 0.5 + 7 * 2.0 ** -18 * 16).all()
+
+
+# Straight-through Eq. 3 with the Gram matrix in parts and the scale path in the product's epilogue: rows off the chunks of 64, off the
+# parts, and in the last row tile's first and second half; and sizes below the line of each.  The transforms are permutations in which
+# half of the rows also take another's entry: sums of two and an inverse of 0, 1 and -1 are exact, so both sides round the same values.
+@pytest.mark.parametrize("d_out,d_in,group", [(1100, 2048, 128), (4200, 512, 64), (4165, 512, 128), (833, 2560, 64), (1030, 1024, 128),
+                                              (2113, 256, 64), (250, 512, 128)])
+def test_straight_through_gradient(d_out, d_in, group):
+    import paper_2511_19705_b200 as cq
+    W, _ = _case(d_out, d_in, d_in // 256, d_out)
+    g = torch.Generator().manual_seed(4)
+    M = torch.zeros(d_in // 256, 256, 256)
+    for m in M:
+        p = torch.randperm(256, generator=g)
+        m[torch.arange(256), p] = 1
+        m[torch.arange(128), p[128:]] = torch.where(torch.rand(128, generator=g) < 0.5, 1.0, -1.0)
+    M = M.cuda()
+    got = cq.cafeq_proxy_loss_fwd_bwd(W, M, bits=3, group=group, loss_kind=cq.LOSS_L2_STE)
+    want = cq.cafeq_proxy_loss_fwd_bwd(W, M, bits=3, group=group, loss_kind=cq.LOSS_L2_STE, flags=cq.FLAG_GENERIC)
+    assert int(got["status"].item()) == 0 and int(want["status"].item()) == 0
+    # two bf16 terms an operand: 2^-16 per entry of a product, in a chain of four of them
+    assert torch.allclose(got["losses"][:3], want["losses"][:3], rtol=2.0 ** -14)
+    g, w = got["gradM"].double(), want["gradM"].double()
+    for b in range(g.shape[0]):
+        assert ((g[b] - w[b]).norm() / w[b].norm()).item() <= 2.0 ** -14, b
