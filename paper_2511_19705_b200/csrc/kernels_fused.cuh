@@ -15,6 +15,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 #include <string.h>
 
 #include <cuda.h>
@@ -85,16 +86,20 @@ constexpr int BD_STAGES_PER_TILE = 2;
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
-template <int FORM, int K, int G>
+// CTA pairs (cta_group::2)
+constexpr bool bd_pair(int k, int mode) { return k == 256; }
+
+template <int FORM, int K, int G, int MODE>
 struct BdCfg {
-  // K = 256: CTA pairs (cta_group::2).  A tile is 256 rows x 256 columns; each CTA holds half of the operator block (its 128 rows:
+  // PAIR: a tile is 256 rows x 256 columns; each CTA holds half of the operator block (its 128 rows:
   // on the input axis the N half, on the output axis its accumulator rows) and half of the tile (input axis: its 128 rows; output
   // axis: its 128 columns), and its 128 rows of the accumulator.
-  static constexpr bool PAIR = K == 256;
+  static constexpr bool PAIR = bd_pair(K, MODE);
   static constexpr int ROWS = PAIR ? 256 : 128;                       // IN: rows per tile
   static constexpr int NBLK = (FORM == BD_IN) ? 256 / K : 1;          // operator blocks resident per CTA
   static constexpr int T_BYTES = PAIR ? K * K : NBLK * K * K * 2;
-  static constexpr int NC = 256;                                      // OUT: d_in columns per tile
+  static constexpr int MH = (FORM == BD_OUT && !PAIR) ? K / 128 : 1;  // OUT: 128-row halves of the accumulator in this CTA
+  static constexpr int NC = 256 / MH;                                 // OUT: d_in columns per tile
   static constexpr int NSTAGE = (T_BYTES > 65536) ? 3 : ((T_BYTES > 32768) ? 5 : 6);  // as many as fit
   static constexpr int SMEM = 1024 + T_BYTES + NSTAGE * BD_STAGE_BYTES + 256;
 };
@@ -103,7 +108,7 @@ struct BdCfg {
 // lists side by side (bd_pass_dual_kernel below); at K = 256 these are pairs.
 template <int FORM, int K, int G, int MODE>
 __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& mp, const int cta, const int ncta) {
-  using C = BdCfg<FORM, K, G>;
+  using C = BdCfg<FORM, K, G, MODE>;
   static_assert(K == 64 || K == 128 || K == 256, "block size");
   static_assert(FORM == BD_IN || K >= 128, "output-axis form needs k >= 128");
   static_assert(G == 64 || G == 128, "group size");
@@ -245,7 +250,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               if constexpr (FORM == BD_IN) {
                 x = major * 256 + bx * 64;
                 y = t * C::ROWS + (int)rank * 128;
-              } else if constexpr (PAIR) {  // stage = 128 contraction rows x this CTA's 128 columns
+              } else if constexpr (K == 256) {  // stage = 128 contraction rows x this CTA's 128 columns
                 x = t * C::NC + (int)rank * 128 + h * 64;
                 y = major * K + sidx * 128;
               } else {
@@ -355,6 +360,11 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
                 for (int ks = 0; ks < 8; ++ks) {
                   if constexpr (PAIR)
                     tc_mma_pair(dbase, alo + (2 * sidx + ks / 4) * 1024 + (ks % 4) * astep, blo + ks * 128, idesc_out, (sidx | ks) != 0 ? 1u : 0u);
+                  else if constexpr (K == 256)  // both halves of the operator's rows against the same columns
+#pragma unroll
+                    for (int mh = 0; mh < 2; ++mh)
+                      tc_mma_lo(dbase + mh * 128, alo + (2 * sidx + ks / 4) * 2048 + mh * 1024 + (ks % 4) * astep, blo + ks * 128, idesc_out,
+                                (sidx | ks) != 0 ? 1u : 0u);
                   else
                     tc_mma_lo(dbase + sidx * 128, alo + (ks / 4) * 1024 + (ks % 4) * astep, blo + ks * 128, idesc_out, ks != 0 ? 1u : 0u);
                 }
@@ -431,8 +441,8 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
           row = t * C::ROWS + (int)rank * 128 + L;
           col0 = major * 256 + hw * 128;
         } else {
-          row = major * K + (int)rank * 128 + L;
-          col0 = t * C::NC + hw * 128;
+          row = major * K + ((int)rank + (C::MH == 2 ? hw : 0)) * 128 + L;
+          col0 = t * C::NC + (C::MH == 2 ? 0 : hw * 128);
         }
         const bool valid = (row < p.d_out) && (col0 < p.d_in);
         // Eq. 4 weights of this thread's groups, requested before the wait for the accumulator so that the
@@ -458,26 +468,29 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
             else mbar_arrive(bar_acce + 8 * buf);
           }
         };
-        // This thread's 128 columns, 16 at a time, the next 16 requested while these are worked on (unrolled: a copy of the registers
-        // in flight would read them too early).
-        auto walk = [&](auto&& f) {
+        // This thread's columns from `addr` on, N times 16, the next 16 requested while these are worked on (unrolled: a copy of the
+        // registers in flight would read them too early).
+        auto walk = [&](uint32_t addr, auto count, auto&& f) {
+          constexpr int N = decltype(count)::value;
           uint32_t raw[2][16];
-          tc_ld16_async(taddr, raw[0]);
+          tc_ld16_async(addr, raw[0]);
 #pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {
+          for (int ch = 0; ch < N; ++ch) {
             tc_ld16_wait(raw[ch & 1]);
-            if (ch < 7) tc_ld16_async(taddr + (ch + 1) * 16, raw[(ch + 1) & 1]);
+            if (ch < N - 1) tc_ld16_async(addr + (ch + 1) * 16, raw[(ch + 1) & 1]);
             float v[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(raw[ch & 1][e]);
             f(ch, v);
           }
         };
+        constexpr std::integral_constant<int, 8> all{};        // its 128 columns
+        constexpr std::integral_constant<int, G / 16> group{};  // those of a group
         if constexpr (MODE == BD_STORE) {
           // the transformed matrix itself, rounded to bf16 (inference-side apply of a block-diagonal operator)
           uint16_t* dst = p.delta + (long long)row * p.d_in + col0;
           const bool wide = ((uintptr_t)p.delta & 31) == 0;
-          walk([&](int ch, const float* v) {
+          walk(taddr, all, [&](int ch, const float* v) {
             if (ch == 7) release();
             uint32_t pk[8];
 #pragma unroll
@@ -489,177 +502,57 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
         } else if constexpr (MODE == BD_SQSUM) {
           // sum of squares only (second pass of the l2 proxy)
           float sq4[4] = {0.f, 0.f, 0.f, 0.f};
-          walk([&](int ch, const float* v) {
+          walk(taddr, all, [&](int ch, const float* v) {
             if (ch == 7) release();
 #pragma unroll
             for (int e = 0; e < 16; ++e) sq4[e & 3] = fmaf(v[e], v[e], sq4[e & 3]);
           });
           sq_local += valid ? (double)((sq4[0] + sq4[1]) + (sq4[2] + sq4[3])) : 0.0;
-        } else {
-          float best[NG], bval[NG];
-          int bidx[NG];
+        } else if constexpr (MODE == BD_CODES) {
+          // Group after group (both groups of 64 at once took more registers than there are: 14336 x 3584 at k = 128 40.5 -> 43 us).
+          //
+          // code = rne(fl32(u / s)).  The IEEE division is a long dependent sequence with a slow-path branch per
+          // element; u * (1 / s), rounded once together with its addend below, differs from fl32(u / s) by less than
+          // (qmax + 1) * 2.4e-7, so it rounds to the same integer unless the quotient lies within that distance of a
+          // half-integer: those (rare: the transformed values are not on a coarse grid) chunks are redone with the
+          // division.  The rounding uses no conversion instruction: t = u / s + 1.5 * 2^23 holds rne(u / s) in its low
+          // mantissa bits (an fp32 result rounds to nearest even, as rintf does) and, 0x4B400000 having a zero low
+          // byte, the low byte of t's pattern is the two's-complement code; |u / s| <= qmax (1 + 3 * 2^-23), so
+          // nothing is clamped.
+          constexpr float MAGIC = 12582912.f;
+          const float win = 0.5f - (p.qmax + 1.f) * 1.0e-6f;
+          const bool wide = ((uintptr_t)p.codes & 31) == 0;
+#pragma unroll 1
+          for (int gi = 0; gi < NG; ++gi) {
+            const uint32_t gaddr = taddr + gi * G;
+            // the absmax: two columns per instruction, NaN and infinity stay visible in the maximum
+            float m2[2] = {0.f, 0.f};
+            walk(gaddr, group, [&](int, const float* v) {
 #pragma unroll
-          for (int gi = 0; gi < NG; ++gi) { best[gi] = 0.f; bval[gi] = 0.f; bidx[gi] = 0; }
-          if constexpr (MODE == BD_CODES) {
-            // group absmax only (no arg-max): two columns per instruction, NaN and infinity stay visible in the maximum
-            float m4[NG][2];
-#pragma unroll
-            for (int gi = 0; gi < NG; ++gi) m4[gi][0] = m4[gi][1] = 0.f;
-            walk([&](int ch, const float* v) {
-              const int gi = ch * 16 / G;
-#pragma unroll
-              for (int e = 0; e < 16; e += 2) m4[gi][(e >> 1) & 1] = max_abs2(m4[gi][(e >> 1) & 1], v[e], v[e + 1]);
+              for (int e = 0; e < 16; e += 2) m2[(e >> 1) & 1] = max_abs2(m2[(e >> 1) & 1], v[e], v[e + 1]);
             });
-            bool nan = false;
-#pragma unroll
-            for (int gi = 0; gi < NG; ++gi) {
-              best[gi] = max_abs2(m4[gi][0], m4[gi][1], 0.f);
-              if (valid && !(best[gi] <= 3.0e38f)) bad = true;
-              nan = nan || best[gi] != best[gi];
-            }
+            float best = max_abs2(m2[0], m2[1], 0.f);
+            if (valid && !(best <= 3.0e38f)) bad = true;
             // A group with a NaN keeps the maximum of its numbers (a non-finite weight spoils its own block only; the NaN itself
             // is coded -qmax): one more walk, by the whole warp, where any lane has met one.
-            if (__any_sync(0xffffffffu, nan)) {
-#pragma unroll
-              for (int gi = 0; gi < NG; ++gi) {
-                best[gi] = 0.f;
+            if (__any_sync(0xffffffffu, best != best)) {
+              best = 0.f;
 #pragma unroll 1
-                for (int ch = 0; ch < G / 16; ++ch) {
-                  float v[16];
-                  tc_ld16(taddr + gi * G + ch * 16, v);
+              for (int ch = 0; ch < G / 16; ++ch) {
+                float v[16];
+                tc_ld16(gaddr + ch * 16, v);
 #pragma unroll
-                  for (int e = 0; e < 16; ++e) best[gi] = fmaxf(best[gi], fabsf(v[e]));
-                }
+                for (int e = 0; e < 16; ++e) best = fmaxf(best, fabsf(v[e]));
               }
             }
-          } else {
-            // Group absmax with arg-max.  Per chunk of 16 columns the maximum (two columns per instruction), and where it beats the
-            // chunks before it the chunk itself is kept, one select per column; the position inside the kept chunk is looked up
-            // once per group.  1.7 instructions per column and no long chains (compare, two selects and the range check per
-            // column took 4, in four chains), the next chunk's loads in flight meanwhile.  A strict comparison keeps the lowest
-            // of equal chunks, the downward search the lowest column.
-            float kept[16], nm = 0.f;
-            int kc = 0;
-            float b = 0.f;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) kept[e] = 0.f;
-            walk([&](int ch, const float* r) {
-              constexpr int CPG = G / 16;  // chunks per group
-              const int gi = ch / CPG;
-              float m[2] = {0.f, 0.f};
-#pragma unroll
-              for (int e = 0; e < 16; e += 2) m[(e >> 1) & 1] = max_abs2(m[(e >> 1) & 1], r[e], r[e + 1]);
-              const float cm = max_abs2(m[0], m[1], 0.f);
-              nm = max_abs2(nm, cm, 0.f);
-              const bool up = cm > b;
-              b = up ? cm : b;
-              kc = up ? ch % CPG : kc;
-#pragma unroll
-              for (int e = 0; e < 16; ++e) kept[e] = up ? r[e] : kept[e];
-              if (ch % CPG == CPG - 1) {
-                float v = 0.f;
-                int ix = 0;
-#pragma unroll
-                for (int e = 15; e >= 0; --e)
-                  if (fabsf(kept[e]) == b) { v = kept[e]; ix = e; }
-                best[gi] = b;
-                bval[gi] = v;
-                bidx[gi] = kc * 16 + ix;
-                b = 0.f;
-                kc = 0;
-#pragma unroll
-                for (int e = 0; e < 16; ++e) kept[e] = 0.f;
-              }
-            });
-            if (__any_sync(0xffffffffu, nm != nm)) {
-              // A NaN hides its chunk from the comparisons above: the groups' maxima over their numbers, by the whole warp.
-#pragma unroll
-              for (int gi = 0; gi < NG; ++gi) {
-                best[gi] = bval[gi] = 0.f;
-                bidx[gi] = 0;
-#pragma unroll 1
-                for (int ch = 0; ch < G / 16; ++ch) {
-                  float v[16];
-                  tc_ld16(taddr + gi * G + ch * 16, v);
-#pragma unroll
-                  for (int e = 0; e < 16; ++e)
-                    if (fabsf(v[e]) > best[gi]) { best[gi] = fabsf(v[e]); bval[gi] = v[e]; bidx[gi] = ch * 16 + e; }
-                }
-              }
-            }
-            if (valid && !(nm <= 3.0e38f)) bad = true;
-          }
-          // Without a second walk over the accumulator (codes / residual) everything still needed is in registers:
-          // hand the buffer back to the tensor cores now.  The arrive has release semantics, so issuing it after the
-          // global stores below would make every tile wait for those stores to land.
-          if constexpr (MODE == BD_REC) release();
-          if constexpr (MODE != BD_CODES) {
-            if (valid && p.vmax && !((p.epi & EPI_SURR) && p.coef)) {
-#pragma unroll
-              for (int gi = 0; gi < NG; ++gi) vm = fmaxf(vm, best[gi]);
-            }
-            if (valid) {
-              // with Eq. 4 evaluated right here nothing downstream reads the maxima or their signs: the backward only
-              // needs (arg-max index, coefficient).  Every scattered 4-byte store is a partial-sector write at L2.
-              const bool need_a = !(p.epi & EPI_SURR) || p.a_always;
-#pragma unroll
-              for (int gi = 0; gi < NG; ++gi) {
-                // group-major records: consecutive rows of one group are contiguous, so a warp's store is one line
-                const long long w = (long long)(col0 / G + gi) * p.d_out + row;
-                if (need_a) {
-                  p.a[w] = best[gi];
-                  p.usel[w] = bval[gi];
-                }
-                p.idx[w] = bidx[gi];
-              }
-            }
-            if (p.epi & EPI_SURR) {
-              const int key = (FORM == BD_IN) ? major : row;  // (uniform over the warp on the input axis)
-              if (asum_key != key) {
-                if (asum_key >= 0) flush_asum();
-                asum_key = key;
-              }
-              float surf = 0.f;
-#pragma unroll
-              for (int gi = 0; gi < NG; ++gi) {
-                const float av = valid ? best[gi] : 0.f;
-                surf = fmaf(wgt[gi] * av, av, surf);
-                if (valid && p.coef) {
-                  const float sg = (bval[gi] > 0.f) ? 1.f : ((bval[gi] < 0.f) ? -1.f : 0.f);
-                  const float cf = 2.f * p.kappa * wgt[gi] * av;
-                  p.coef[(long long)(col0 / G + gi) * p.d_out + row] = cf * sg;
-                  vm = fmaxf(vm, cf);
-                }
-                float& as = asum[(FORM == BD_IN) ? gi : 0];
-                as = fmaf(av, av, as);
-              }
-              sur_local += (double)surf;
-            }
-          }
-          if constexpr (MODE == BD_CODES) {
-            // code = rne(fl32(u / s)).  The IEEE division is a long dependent sequence with a slow-path branch per
-            // element; u * (1 / s), rounded once together with its addend below, differs from fl32(u / s) by less than
-            // (qmax + 1) * 2.4e-7, so it rounds to the same integer unless the quotient lies within that distance of a
-            // half-integer: those (rare: the transformed values are not on a coarse grid) chunks are redone with the
-            // division.  The rounding uses no conversion instruction: t = u / s + 1.5 * 2^23 holds rne(u / s) in its low
-            // mantissa bits (an fp32 result rounds to nearest even, as rintf does) and, 0x4B400000 having a zero low
-            // byte, the low byte of t's pattern is the two's-complement code; |u / s| <= qmax (1 + 3 * 2^-23), so
-            // nothing is clamped.
-            constexpr float MAGIC = 12582912.f;
-            const float win = 0.5f - (p.qmax + 1.f) * 1.0e-6f;
-            int8_t* dst = p.codes + (long long)row * p.d_in + col0;
-            const bool wide = ((uintptr_t)p.codes & 31) == 0;
-            float s[NG], rs[NG];
-#pragma unroll
-            for (int gi = 0; gi < NG; ++gi) {
-              s[gi] = __fdiv_rn(best[gi], p.qmax);
-              rs[gi] = (s[gi] > 0.f) ? __frcp_rn(s[gi]) : 0.f;
-              if (valid) p.scales[(long long)row * (p.d_in / G) + (col0 / G + gi)] = s[gi];
-            }
+            const float s = __fdiv_rn(best, p.qmax);
+            const float rs = (s > 0.f) ? __frcp_rn(s) : 0.f;
+            if (valid) p.scales[(long long)row * (p.d_in / G) + (col0 / G + gi)] = s;
+            int8_t* dst = p.codes + (long long)row * p.d_in + col0 + gi * G;
             uint32_t cpk[8];
             float dm = 0.f;
-            walk([&](int hc, const float* v) {
-              const int ch = hc >> 1, hf = hc & 1, gi = hc * 16 / G;  // 32 columns a store
+            walk(gaddr, group, [&](int hc, const float* v) {
+              const int ch = hc >> 1, hf = hc & 1;  // 32 columns a store
               if (hf == 0) dm = 0.f;
 #pragma unroll
               for (int w = 0; w < 4; ++w) {
@@ -668,9 +561,9 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                   const float x = v[4 * w + e];
-                  const float tt = fmaf(x, rs[gi], MAGIC);
+                  const float tt = fmaf(x, rs, MAGIC);
                   cb[e] = __float_as_uint(tt);
-                  d[e] = fmaf(x, rs[gi], -(tt - MAGIC));
+                  d[e] = fmaf(x, rs, -(tt - MAGIC));
                 }
                 dm = max_abs2(dm, d[0], d[1]);
                 dm = max_abs2(dm, d[2], d[3]);
@@ -678,17 +571,17 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
               }
               if (hf == 0) return;
               // (also: a scale so small that its reciprocal overflows); the accumulator is read again by the whole warp
-              if (__any_sync(0xffffffffu, !(dm <= win) || !(rs[gi] < 3.0e38f))) {
+              if (__any_sync(0xffffffffu, !(dm <= win) || !(rs < 3.0e38f))) {
 #pragma unroll
                 for (int h2 = 0; h2 < 2; ++h2) {
                   float u[16];
-                  tc_ld16(taddr + ch * 32 + h2 * 16, u);
+                  tc_ld16(gaddr + ch * 32 + h2 * 16, u);
 #pragma unroll
                   for (int w = 0; w < 4; ++w) {
                     uint32_t pk = 0;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                      float qd = (s[gi] > 0.f) ? rintf(__fdiv_rn(u[4 * w + e], s[gi])) : 0.f;
+                      float qd = (s > 0.f) ? rintf(__fdiv_rn(u[4 * w + e], s)) : 0.f;
                       qd = fminf(fmaxf(qd, -p.qmax), p.qmax);
                       pk |= ((uint32_t)((int)qd) & 0xFFu) << (8 * e);
                     }
@@ -696,9 +589,114 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
                   }
                 }
               }
-              if (ch == 3) release();
+              if (ch == G / 32 - 1 && gi == NG - 1) release();
               if (valid) store32(dst + ch * 32, cpk, wide);
             });
+          }
+        } else {
+          float best[NG], bval[NG];
+          int bidx[NG];
+#pragma unroll
+          for (int gi = 0; gi < NG; ++gi) { best[gi] = 0.f; bval[gi] = 0.f; bidx[gi] = 0; }
+          // Group absmax with arg-max.  Per chunk of 16 columns the maximum (two columns per instruction), and where it beats the
+          // chunks before it the chunk itself is kept, one select per column; the position inside the kept chunk is looked up
+          // once per group.  1.7 instructions per column and no long chains (compare, two selects and the range check per
+          // column took 4, in four chains), the next chunk's loads in flight meanwhile.  A strict comparison keeps the lowest
+          // of equal chunks, the downward search the lowest column.
+          float kept[16], nm = 0.f;
+          int kc = 0;
+          float b = 0.f;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) kept[e] = 0.f;
+          walk(taddr, all, [&](int ch, const float* r) {
+            constexpr int CPG = G / 16;  // chunks per group
+            const int gi = ch / CPG;
+            float m[2] = {0.f, 0.f};
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) m[(e >> 1) & 1] = max_abs2(m[(e >> 1) & 1], r[e], r[e + 1]);
+            const float cm = max_abs2(m[0], m[1], 0.f);
+            nm = max_abs2(nm, cm, 0.f);
+            const bool up = cm > b;
+            b = up ? cm : b;
+            kc = up ? ch % CPG : kc;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) kept[e] = up ? r[e] : kept[e];
+            if (ch % CPG == CPG - 1) {
+              float v = 0.f;
+              int ix = 0;
+#pragma unroll
+              for (int e = 15; e >= 0; --e)
+                if (fabsf(kept[e]) == b) { v = kept[e]; ix = e; }
+              best[gi] = b;
+              bval[gi] = v;
+              bidx[gi] = kc * 16 + ix;
+              b = 0.f;
+              kc = 0;
+#pragma unroll
+              for (int e = 0; e < 16; ++e) kept[e] = 0.f;
+            }
+          });
+          if (__any_sync(0xffffffffu, nm != nm)) {
+            // A NaN hides its chunk from the comparisons above: the groups' maxima over their numbers, by the whole warp.
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) {
+              best[gi] = bval[gi] = 0.f;
+              bidx[gi] = 0;
+#pragma unroll 1
+              for (int ch = 0; ch < G / 16; ++ch) {
+                float v[16];
+                tc_ld16(taddr + gi * G + ch * 16, v);
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                  if (fabsf(v[e]) > best[gi]) { best[gi] = fabsf(v[e]); bval[gi] = v[e]; bidx[gi] = ch * 16 + e; }
+              }
+            }
+          }
+          if (valid && !(nm <= 3.0e38f)) bad = true;
+          // Without a second walk over the accumulator (codes / residual) everything still needed is in registers:
+          // hand the buffer back to the tensor cores now.  The arrive has release semantics, so issuing it after the
+          // global stores below would make every tile wait for those stores to land.
+          if constexpr (MODE == BD_REC) release();
+          if (valid && p.vmax && !((p.epi & EPI_SURR) && p.coef)) {
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) vm = fmaxf(vm, best[gi]);
+          }
+          if (valid) {
+            // with Eq. 4 evaluated right here nothing downstream reads the maxima or their signs: the backward only
+            // needs (arg-max index, coefficient).  Every scattered 4-byte store is a partial-sector write at L2.
+            const bool need_a = !(p.epi & EPI_SURR) || p.a_always;
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) {
+              // group-major records: consecutive rows of one group are contiguous, so a warp's store is one line
+              const long long w = (long long)(col0 / G + gi) * p.d_out + row;
+              if (need_a) {
+                p.a[w] = best[gi];
+                p.usel[w] = bval[gi];
+              }
+              p.idx[w] = bidx[gi];
+            }
+          }
+          if (p.epi & EPI_SURR) {
+            const int key = (FORM == BD_IN) ? major : row;  // (uniform over the warp on the input axis)
+            if (asum_key != key) {
+              if (asum_key >= 0) flush_asum();
+              asum_key = key;
+            }
+            float surf = 0.f;
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) {
+              const float av = valid ? best[gi] : 0.f;
+              surf = fmaf(wgt[gi] * av, av, surf);
+              if (valid && p.coef) {
+                const float sg = (bval[gi] > 0.f) ? 1.f : ((bval[gi] < 0.f) ? -1.f : 0.f);
+                const float cf = 2.f * p.kappa * wgt[gi] * av;
+                p.coef[(long long)(col0 / G + gi) * p.d_out + row] = cf * sg;
+                vm = fmaxf(vm, cf);
+              }
+              float& as = asum[(FORM == BD_IN) ? gi : 0];
+              as = fmaf(av, av, as);
+            }
+            sur_local += (double)surf;
           }
           if constexpr (MODE == BD_DELTA) {
             // residual s * code - u as one or two bf16 terms, 16 columns at a time (rounding as above)
@@ -707,31 +705,7 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
             uint16_t* dst = p.delta + (long long)row * p.d_in + col0;
             uint16_t* dst_lo = p.delta_lo ? p.delta_lo + (long long)row * p.d_in + col0 : nullptr;
             const bool wide = (((uintptr_t)p.delta | (uintptr_t)p.delta_lo) & 31) == 0;
-            float s2[NG], rs2[NG];
-#pragma unroll
-            for (int gi = 0; gi < NG; ++gi) {
-              s2[gi] = __fdiv_rn(best[gi], p.qmax);
-              rs2[gi] = (s2[gi] > 0.f) ? __frcp_rn(s2[gi]) : 0.f;
-            }
-            walk([&](int ch, const float* v) {
-              const int gi = ch * 16 / G;
-              const float s = s2[gi], rs = rs2[gi];
-              float dm = 0.f;
-              if (ch == 7) release();
-              float qv[16];
-#pragma unroll
-              for (int e = 0; e < 16; e += 2) {
-                qv[e] = fmaf(v[e], rs, MAGIC) - MAGIC;
-                qv[e + 1] = fmaf(v[e + 1], rs, MAGIC) - MAGIC;
-                dm = max_abs2(dm, fmaf(v[e], rs, -qv[e]), fmaf(v[e + 1], rs, -qv[e + 1]));
-              }
-              if (!(dm <= win) || !(rs < 3.0e38f)) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                  const float qd = (s > 0.f) ? rintf(__fdiv_rn(v[e], s)) : 0.f;
-                  qv[e] = fminf(fmaxf(qd, -p.qmax), p.qmax);
-                }
-              }
+            auto put = [&](int ch, const float* v, const float* qv, float s) {
               uint32_t hpk[8], lpk[8];
 #pragma unroll
               for (int e = 0; e < 16; e += 2) {
@@ -745,7 +719,50 @@ __device__ __forceinline__ void bd_pass_body(const BdMaps& maps, const BdMulti& 
                 store32(dst + ch * 16, hpk, wide);
                 if (dst_lo) store32(dst_lo + ch * 16, lpk, wide);
               }
-            });
+            };
+            float s[NG], rs[NG];
+            uint32_t redo = 0;
+#pragma unroll
+            for (int gi = 0; gi < NG; ++gi) {
+              s[gi] = __fdiv_rn(best[gi], p.qmax);
+              rs[gi] = (s[gi] > 0.f) ? __frcp_rn(s[gi]) : 0.f;
+            }
+            auto put16 = [&](int ch, const float* v, float sg, float r) {
+              float dm = 0.f, qv[16];
+#pragma unroll
+              for (int e = 0; e < 16; e += 2) {
+                qv[e] = fmaf(v[e], r, MAGIC) - MAGIC;
+                qv[e + 1] = fmaf(v[e + 1], r, MAGIC) - MAGIC;
+                dm = max_abs2(dm, fmaf(v[e], r, -qv[e]), fmaf(v[e + 1], r, -qv[e + 1]));
+              }
+              if (__any_sync(0xffffffffu, !(dm <= win) || !(r < 3.0e38f))) redo |= 1u << ch;
+              if (ch == 7 && !redo) release();
+              put(ch, v, qv, sg);
+            };
+            // (rolled: unrolled, with the next columns in flight, the code is eight times as long; Eq. 3's loss of 4096 x 3584 at k = 256
+            // 162 us, after other work 174, so 156 and 164)
+#pragma unroll 1
+            for (int ch = 0; ch < 8; ++ch) {
+              float v[16];
+              tc_ld16(taddr + ch * 16, v);
+              put16(ch, v, (NG == 1 || ch < 4) ? s[0] : s[NG - 1], (NG == 1 || ch < 4) ? rs[0] : rs[NG - 1]);
+            }
+            if (redo) {
+#pragma unroll 1
+              for (int ch = 0; ch < 8; ++ch) {
+                if (!((redo >> ch) & 1u)) continue;
+                const float s1 = (NG == 1 || ch < 4) ? s[0] : s[NG - 1];
+                float u[16], qv[16];
+                tc_ld16(taddr + ch * 16, u);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                  const float qd = (s1 > 0.f) ? rintf(__fdiv_rn(u[e], s1)) : 0.f;
+                  qv[e] = fminf(fmaxf(qd, -p.qmax), p.qmax);
+                }
+                put(ch, u, qv, s1);
+              }
+              release();
+            }
           }
         }
       }
@@ -785,7 +802,7 @@ template <int FORM, int K, int G, int MODE>
 __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_kernel(const __grid_constant__ BdMaps maps, const __grid_constant__ BdMulti mp) {
   pdl_wait();
-  constexpr int W = BdCfg<FORM, K, G>::PAIR ? 2 : 1;
+  constexpr int W = BdCfg<FORM, K, G, MODE>::PAIR ? 2 : 1;
   bd_pass_body<FORM, K, G, MODE>(maps, mp, (int)blockIdx.x / W, (int)gridDim.x / W);
 }
 
@@ -797,7 +814,7 @@ __global__ void __launch_bounds__(BD_THREADS, 1)
 bd_pass_dual_kernel(const __grid_constant__ BdMaps maps_in, const __grid_constant__ BdMulti mp_in,
                     const __grid_constant__ BdMaps maps_out, const __grid_constant__ BdMulti mp_out, const int n_in) {
   pdl_wait();
-  constexpr int W = BdCfg<BD_IN, K, G>::PAIR ? 2 : 1;
+  constexpr int W = BdCfg<BD_IN, K, G, BD_REC>::PAIR ? 2 : 1;
   const int cta = (int)blockIdx.x / W, n = (int)gridDim.x / W;  // (pairs at K = 256)
   if (cta < n_in) bd_pass_body<BD_IN, K, G, BD_REC>(maps_in, mp_in, cta, n_in);
   else bd_pass_body<BD_OUT, K, G, BD_REC>(maps_out, mp_out, cta - n_in, n - n_in);
@@ -874,9 +891,9 @@ static bool opt_in_smem(KernelT kernel, int bytes, std::atomic<unsigned long lon
 }
 
 // tile geometry of one sub-problem
-template <int FORM, int K, int G>
+template <int FORM, int K, int G, int MODE>
 static void bd_fill_tiles(BdParams& p) {
-  using C = BdCfg<FORM, K, G>;
+  using C = BdCfg<FORM, K, G, MODE>;
   if (FORM == BD_IN) {
     p.n_major = (p.d_in + 255) / 256;
     p.n_minor = (p.d_out + C::ROWS - 1) / C::ROWS;
@@ -888,12 +905,12 @@ static void bd_fill_tiles(BdParams& p) {
 
 template <int FORM, int K, int G, int MODE>
 static int bd_launch_multi_t(cudaStream_t st, const BdMaps& maps, BdMulti mp, int min_tiles) {
-  using C = BdCfg<FORM, K, G>;
+  using C = BdCfg<FORM, K, G, MODE>;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(bd_pass_kernel<FORM, K, G, MODE>, C::SMEM, done)) return CAFEQ_ERR_CUDA;
   long long total = 0;
   for (int s = 0; s < mp.n; ++s) {
-    bd_fill_tiles<FORM, K, G>(mp.p[s]);
+    bd_fill_tiles<FORM, K, G, MODE>(mp.p[s]);
     total += (long long)mp.p[s].n_major * mp.p[s].n_minor;
     mp.tile_end[s] = (int)total;
   }
@@ -918,6 +935,9 @@ static int bd_mode(int epi) {
   if (epi & EPI_CODES) return BD_CODES;
   return (epi & EPI_DELTA) ? BD_DELTA : BD_REC;
 }
+
+// rows of the operator in one box: all of a block, of a pair's CTA its half; stored transposed, one swizzle atom
+static int bd_operator_rows(int k, const BdParams& p) { return p.t_mn ? 64 : (bd_pair(k, bd_mode(p.epi)) ? 128 : k); }
 
 template <int FORM, int K, int G>
 static int bd_dispatch_mode(cudaStream_t st, const BdMaps& maps, const BdMulti& mp, int min_tiles) {
@@ -954,7 +974,7 @@ static int bd_launch(cudaStream_t st, int form, int k, int g, const void* X, lon
   BdMulti mp;
   memset(&mp, 0, sizeof(mp));
   if (!make_map_bf16(&maps.x[0], X, p.d_in, p.d_out, ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-  if (!make_map_bf16(&maps.t[0], Tb, k, (long long)nbT * k, k, p.t_mn ? 64 : (k == 256 ? 128 : k))) return CAFEQ_ERR_UNSUPPORTED;
+  if (!make_map_bf16(&maps.t[0], Tb, k, (long long)nbT * k, k, bd_operator_rows(k, p))) return CAFEQ_ERR_UNSUPPORTED;
   for (int s = 1; s < BD_MAX_SUB; ++s) { maps.x[s] = maps.x[0]; maps.t[s] = maps.t[0]; }
   mp.n = 1;
   mp.p[0] = p;
@@ -979,7 +999,7 @@ static int bd_launch_many(cudaStream_t st, int form, int k, int g, const BdSub* 
   memset(&mp, 0, sizeof(mp));
   for (int s = 0; s < n; ++s) {
     if (!make_map_bf16(&maps.x[s], subs[s].X, subs[s].p.d_in, subs[s].p.d_out, subs[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&maps.t[s], subs[s].Tb, k, (long long)subs[s].nbT * k, k, subs[s].p.t_mn ? 64 : (k == 256 ? 128 : k))) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&maps.t[s], subs[s].Tb, k, (long long)subs[s].nbT * k, k, bd_operator_rows(k, subs[s].p))) return CAFEQ_ERR_UNSUPPORTED;
     mp.p[s] = subs[s].p;
   }
   for (int s = n; s < BD_MAX_SUB; ++s) { maps.x[s] = maps.x[0]; maps.t[s] = maps.t[0]; }
@@ -1001,23 +1021,23 @@ static int dual_split(long long tiles_in, long long tiles_out, int out_weight_pc
 
 template <int K, int G>
 static int bd_launch_dual_t(cudaStream_t st, const BdMaps& mi, BdMulti pi, const BdMaps& mo, BdMulti po, bool overlap) {
-  constexpr int SMEM = BdCfg<BD_IN, K, G>::SMEM > BdCfg<BD_OUT, K, G>::SMEM ? BdCfg<BD_IN, K, G>::SMEM : BdCfg<BD_OUT, K, G>::SMEM;
+  constexpr int SMEM = BdCfg<BD_IN, K, G, BD_REC>::SMEM > BdCfg<BD_OUT, K, G, BD_REC>::SMEM ? BdCfg<BD_IN, K, G, BD_REC>::SMEM : BdCfg<BD_OUT, K, G, BD_REC>::SMEM;
   static std::atomic<unsigned long long> done{0};
   if (!opt_in_smem(bd_pass_dual_kernel<K, G>, SMEM, done)) return CAFEQ_ERR_CUDA;
   long long ti = 0, to = 0;
   for (int s = 0; s < pi.n; ++s) {
-    bd_fill_tiles<BD_IN, K, G>(pi.p[s]);
+    bd_fill_tiles<BD_IN, K, G, BD_REC>(pi.p[s]);
     ti += (long long)pi.p[s].n_major * pi.p[s].n_minor;
     pi.tile_end[s] = (int)ti;
   }
   for (int s = pi.n; s < BD_MAX_SUB; ++s) pi.tile_end[s] = (int)ti;
   for (int s = 0; s < po.n; ++s) {
-    bd_fill_tiles<BD_OUT, K, G>(po.p[s]);
+    bd_fill_tiles<BD_OUT, K, G, BD_REC>(po.p[s]);
     to += (long long)po.p[s].n_major * po.p[s].n_minor;
     po.tile_end[s] = (int)to;
   }
   for (int s = po.n; s < BD_MAX_SUB; ++s) po.tile_end[s] = (int)to;
-  constexpr bool PAIR = BdCfg<BD_IN, K, G>::PAIR;
+  constexpr bool PAIR = BdCfg<BD_IN, K, G, BD_REC>::PAIR;
   pi.stream = po.stream = l2_stream((PAIR ? 131072.0 : 65536.0) * (ti + to));
   const int n_in = dual_split(ti, to, g_dual_pass_pct.load(std::memory_order_relaxed), PAIR ? 74 : 148);
   if (PAIR) launch_pairs_if(overlap, bd_pass_dual_kernel<K, G>, 74, BD_THREADS, SMEM, st, mi, pi, mo, po, n_in);
@@ -1036,13 +1056,13 @@ static int bd_launch_dual(cudaStream_t st, int k, int g, const BdSub* in, int n_
   memset(&po, 0, sizeof(po));
   for (int s = 0; s < n_in; ++s) {
     if (!make_map_bf16(&mi.x[s], in[s].X, in[s].p.d_in, in[s].p.d_out, in[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&mi.t[s], in[s].Tb, k, (long long)in[s].nbT * k, k, k == 256 ? 128 : k)) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&mi.t[s], in[s].Tb, k, (long long)in[s].nbT * k, k, bd_operator_rows(k, in[s].p))) return CAFEQ_ERR_UNSUPPORTED;
     pi.p[s] = in[s].p;
   }
   for (int s = n_in; s < BD_MAX_SUB; ++s) { mi.x[s] = mi.x[0]; mi.t[s] = mi.t[0]; }
   for (int s = 0; s < n_out; ++s) {
     if (!make_map_bf16(&mo.x[s], out[s].X, out[s].p.d_in, out[s].p.d_out, out[s].ld, 128)) return CAFEQ_ERR_UNSUPPORTED;
-    if (!make_map_bf16(&mo.t[s], out[s].Tb, k, (long long)out[s].nbT * k, k, out[s].p.t_mn ? 64 : (k == 256 ? 128 : k))) return CAFEQ_ERR_UNSUPPORTED;
+    if (!make_map_bf16(&mo.t[s], out[s].Tb, k, (long long)out[s].nbT * k, k, bd_operator_rows(k, out[s].p))) return CAFEQ_ERR_UNSUPPORTED;
     po.p[s] = out[s].p;
   }
   for (int s = n_out; s < BD_MAX_SUB; ++s) { mo.x[s] = mo.x[0]; mo.t[s] = mo.t[0]; }

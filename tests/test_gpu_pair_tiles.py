@@ -67,6 +67,31 @@ def test_codes(axis, d_out, d_in):
     assert ((c - q).abs() <= 0.5 + 7 * 2.0 ** -18 * 16).all()
 
 
+# Weights on a coarse grid under permutations: quotients fall on half-integers everywhere, and those are decided by the division of the
+# quantiser without a transform.  Groups of both widths, a half tile of columns and of rows.
+@pytest.mark.parametrize("axis,k,d_out,d_in", [("in", 64, 130, 640), ("in", 128, 257, 384), ("in", 256, 200, 768), ("out", 128, 384, 640),
+                                               ("out", 256, 512, 896)])
+@pytest.mark.parametrize("group", [64, 128])
+def test_codes_at_ties(axis, k, d_out, d_in, group):
+    import paper_2511_19705_b200 as cq
+    g = torch.Generator().manual_seed(6)
+    W = (torch.randint(-8, 9, (d_out, d_in), generator=g) / 64.0).bfloat16().cuda()
+    n = (d_in if axis == "in" else d_out) // k
+    p = torch.stack([torch.randperm(k, generator=g) + b * k for b in range(n)]).reshape(-1)
+    T = torch.zeros(n, k, k)
+    for b in range(n):
+        T[b, torch.arange(k), p[b * k:(b + 1) * k] - b * k] = 1
+    U = (W[:, p.cuda()] if axis == "in" else W[p.cuda()]).contiguous()
+    want, ws = cq.cafeq_rtn(U, None, bits=3, group=group)
+    got, gs = cq.cafeq_rtn(W, T.cuda(), bits=3, group=group, tblock=k, taxis=cq.AXIS_IN if axis == "in" else cq.AXIS_OUT)
+    assert torch.equal(got, want) and torch.equal(gs, ws)
+    if axis == "in":  # the residual takes the same decisions: straight-through gradient against the shape-agnostic kernels
+        kw = dict(bits=3, group=group, loss_kind=cq.LOSS_L2_STE)
+        a = cq.cafeq_proxy_loss_fwd_bwd(W, T.cuda(), **kw)["gradM"].double()
+        b = cq.cafeq_proxy_loss_fwd_bwd(W, T.cuda(), flags=cq.FLAG_GENERIC, **kw)["gradM"].double()
+        assert ((a - b).norm() / b.norm()).item() <= 2.0 ** -14
+
+
 # Straight-through Eq. 3 with the Gram matrix in parts and the scale path in the product's epilogue: rows off the chunks of 64, off the
 # parts, and in the last row tile's first and second half; and sizes below the line of each.  The transforms are permutations in which
 # half of the rows also take another's entry: sums of two and an inverse of 0, 1 and -1 are exact, so both sides round the same values.
