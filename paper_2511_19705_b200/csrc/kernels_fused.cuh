@@ -6,7 +6,7 @@
 // X through a TMA ring; accumulators are double-buffered in tensor memory so the epilogue of tile t overlaps
 // the products of tile t+1.
 //
-// Blocks of 256 run on pairs of CTAs (cta_group::2, BdCfg below): the leader issues products of 256 rows for both.
+// The records of blocks of 256 run on pairs of CTAs (cta_group::2, bd_pair below): the leader issues products of 256 rows for both.
 // Warp roles (576 threads): warp 0 = TMA producer, warp 1 = MMA issuer (and tensor-memory owner), warps 2..9 and 10..17 =
 // two epilogue sets, one per accumulator buffer (two warps per 32-lane quarter, each owning 128 accumulator columns).
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises CAFEQ_ERR_TIMEOUT in the status
@@ -86,8 +86,12 @@ constexpr int BD_STAGES_PER_TILE = 2;
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
-// CTA pairs (cta_group::2)
-constexpr bool bd_pair(int k, int mode) { return k == 256; }
+// CTA pairs (cta_group::2): records at K = 256, where the products set the pace and a pair reads a third less of operands.  The other
+// epilogues are longer than the products and lose more to a pair's larger tiles (half as many of them, of 512 KB: a last wave that is
+// emptier, longer first loads) than they gain.  One CTA against pairs: codes of 4096 x 3584 17.8 us, pairs 20.1, of 14336 x 3584
+// 38.9 and 40.6, of 2304 x 9216 25.1 and 29.3, residual and its square 4096 x 3584 156 and 166, apply of 2048 x 3584 13.3 and 14.0.
+// Records: a 9B-shaped layer's step 343 us on pairs, 350 without, 27B-shaped with groups of 64 900 either way.
+constexpr bool bd_pair(int k, int mode) { return k == 256 && mode == BD_REC; }
 
 template <int FORM, int K, int G, int MODE>
 struct BdCfg {
