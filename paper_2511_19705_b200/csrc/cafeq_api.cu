@@ -397,9 +397,15 @@ static bool launch_group_quant_vec(cudaStream_t st, const SRC* U, long long ld, 
   CQ_LAUNCH((group_quant_kernel<L, N, SRC>), (unsigned)((groups * L + 255) / 256), 256, 0, st, U, ld, rows, ng, g, qmax, offsets, off_kind, \
             a, usel, idx, Delta, Uhat, codes, scales, status)
   // Four vectors of four a lane where the group has them (two in groups of 32): a lane's loads are in flight together, and the
-  // reduction over lanes, fifteen shuffles for four values at one vector a lane of 32, is nine for sixteen.  Above eight vectors a
-  // lane, the whole CTA.
-  if (g <= 32) GQ(4, 2);
+  // reduction over lanes, fifteen shuffles for four values at one vector a lane of 32, is nine for sixteen.  Where that leaves less than
+  // 512 threads an SM (2^20 entries) a lane has one (Eq. 5's straight-through gradient of 512 x 1024 with blocks of 64: four vectors 166.5
+  // us a call, one 164.5; Eq. 3's of 1024 x 1024 192.5 and 194.5).  Above eight vectors a lane, the whole CTA.
+  const bool few = groups * g < 1ll << 20;
+  if (few && g <= 32) GQ(8, 1);
+  else if (few && g <= 64) GQ(16, 1);
+  else if (few && g <= 128) GQ(32, 1);
+  else if (few && g <= 256) GQ(32, 2);
+  else if (g <= 32) GQ(4, 2);
   else if (g <= 64) GQ(4, 4);
   else if (g <= 128) GQ(8, 4);
   else if (g <= 256) GQ(16, 4);
@@ -1456,7 +1462,12 @@ static void launch_ste_split(cudaStream_t st, const MatWS& m, const float* gX, l
 #define SGS(L, N)                                                                                                              \
   CQ_LAUNCH((ste_grad_split_kernel<L, N>), (unsigned)((groups * L + 255) / 256), 256, 0, st, m.U, gX, ldg, G.d_out, G.ng, G.g, k, r, \
             m.a, m.usel, m.idx, qmax, hi, lo, status)
-  if (G.g <= 32) SGS(4, 2);
+  const bool few = groups * G.g < 1ll << 20;  // (as in launch_group_quant_vec)
+  if (few && G.g <= 32) SGS(8, 1);
+  else if (few && G.g <= 64) SGS(16, 1);
+  else if (few && G.g <= 128) SGS(32, 1);
+  else if (few && G.g <= 256) SGS(32, 2);
+  else if (G.g <= 32) SGS(4, 2);
   else if (G.g <= 64) SGS(4, 4);
   else if (G.g <= 128) SGS(8, 4);
   else if (G.g <= 256) SGS(16, 4);

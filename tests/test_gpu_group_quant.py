@@ -32,3 +32,10 @@ def test_codes_and_scales_bit_exact(cq, d_out, d_in, group, bits):
     Q = orc.quant_sym(w64(Wb), bits, group)
     assert np.array_equal(codes.cpu().numpy().astype(np.int32), Q["q"])
     assert np.array_equal(scales.cpu().numpy(), Q["s"])
+
+
+# the same from 2^20 entries on, where a lane takes more of a group
+@pytest.mark.parametrize("d_out,d_in,group", [(1031, 1024, 32), (1000, 1080, 36), (1025, 1024, 64), (820, 1360, 68), (1024, 1024, 128),
+                                              (1000, 1056, 132), (1027, 1024, 256), (1010, 1040, 260)])
+def test_codes_and_scales_bit_exact_large(cq, d_out, d_in, group):
+    test_codes_and_scales_bit_exact(cq, d_out, d_in, group, 3)
