@@ -32,10 +32,8 @@ __global__ void __launch_bounds__(256) split_rect_kernel(const float* X, int R, 
                                                          float* __restrict__ YT, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
                                                          uint16_t* __restrict__ thi, uint16_t* __restrict__ tlo,
                                                          const int32_t* status, uint16_t* __restrict__ h3 = nullptr,
-                                                         uint16_t* __restrict__ t3 = nullptr, const double* norm2 = nullptr,
-                                                         const double* only_bad = nullptr) {
+                                                         uint16_t* __restrict__ t3 = nullptr, const double* norm2 = nullptr) {
   pdl_enter();
-  if (only_bad && !tg_bad_start(only_bad)) return;  // (a restart that is not needed)
   if (cta_stopped(status)) return;
   __shared__ uint32_t tile[64][65];
   __shared__ uint16_t tile3[64][66];
@@ -343,11 +341,13 @@ __global__ void __launch_bounds__(256) dot_f32_kernel(const float* x, const floa
 
 // Start of the Gram iteration: G = A A^T (fp32 [m, m], tiles of 256 on and above the diagonal) -> B0 = G / c with c = 1.0001 ||G||_F,
 // so that its eigenvalues lie in [0, 1], and Y1 = (2 mu I - mu^2 B0) / c, both as fp32 (same tiles; B in place of G) and as bf16
-// splits of the whole symmetric matrix.  *c_out = c.  One 64 x 64 tile per CTA (grid: m / 64, m / 64); memory-bound.
+// splits of the whole symmetric matrix.  A row of zeros in A sets *singular, and the first residual to one that a start is not used at.
+// One 64 x 64 tile per CTA (grid: m / 64, m / 64); memory-bound.
 __global__ void __launch_bounds__(256) gram_start_kernel(float* G, int m, const double* fro2, float mu, float* __restrict__ Y,
                                                          uint16_t* __restrict__ Bh, uint16_t* __restrict__ Bl,
                                                          uint16_t* __restrict__ Yh, uint16_t* __restrict__ Yl,
-                                                         double* __restrict__ c_out, const int32_t* status) {
+                                                         double* __restrict__ singular, double* __restrict__ first,
+                                                         const int32_t* status) {
   pdl_enter();
   if (cta_stopped(status)) return;
   if ((blockIdx.x >> 2) < (blockIdx.y >> 2)) return;
@@ -356,7 +356,6 @@ __global__ void __launch_bounds__(256) gram_start_kernel(float* G, int m, const 
   const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
   const double c = 1.0001 * sqrt(*fro2);
   const float inv = c > 0.0 ? (float)(1.0 / c) : 0.f;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *c_out = c;
   auto split = [](float x) -> uint32_t {
     const __nv_bfloat16 h = __float2bfloat16_rn(x);
     return (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(h))) << 16);
@@ -366,6 +365,7 @@ __global__ void __launch_bounds__(256) gram_start_kernel(float* G, int m, const 
     const int i = w + 8 * q, row = r0 + i, col = c0 + 2 * tx;
     const long long o = (long long)row * m + col;
     const float2 g = ld_plain(reinterpret_cast<const float2*>(G + o));
+    if ((row == col && g.x == 0.f) || (row == col + 1 && g.y == 0.f)) { *singular = 1.0; *first = 1e300; }  // (a row of zeros)
     const float2 b = make_float2(g.x * inv, g.y * inv);
     const float2 y = make_float2(((row == col ? 2.f * mu : 0.f) - mu * mu * b.x) * inv, ((row == col + 1 ? 2.f * mu : 0.f) - mu * mu * b.y) * inv);
     *reinterpret_cast<float2*>(G + o) = b;

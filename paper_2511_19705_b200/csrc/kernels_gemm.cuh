@@ -51,7 +51,8 @@ struct TgParams {
                           // batch * colsA_per_batch / colsB_per_batch (B: its contraction at row batch * rowsB_per_batch)
   const double* stop_sq;  // optional: squared residuals of an iteration; this launch belongs to iteration stop_it, and is
   int stop_it;            // skipped when the rule (tg_stopped) ended the iteration before
-  int stop_guard;         // + 1: iteration 0 checks its start; + 2: this is its update; + 4: an update
+  int stop_guard;         // + 1: iteration 0 checks its start; + 2: this is its update; + 4: an update; + 8: a restart;
+                          // 16: stop_sq is a flag, and the launch is skipped where it is set
   int32_t* status;
 };
 
@@ -74,25 +75,28 @@ struct TgCfg {
 // nothing.  An update that would start below 1e-4 is left out: the step that follows the iteration squares the residual too, and
 // leaves less than 2^-24 of it even where all of it is in one direction (from 1e-3 that direction ended at 1e-6).
 constexpr double TG_GOOD_START2 = 0.81, TG_DONE2 = 1e-6, TG_SKIP2 = 1e-8;
-__device__ __forceinline__ bool tg_bad_start(const volatile double* stop_sq) { return !(stop_sq[0] <= TG_GOOD_START2); }
 __device__ __forceinline__ bool tg_stopped(const TgParams& p, int it) {
   const volatile double* sq = p.stop_sq;  // (one launch may run several iterations: never from a cached line)
   if (!sq) return false;
-  if ((p.stop_guard & 4) && sq[it] <= TG_SKIP2) return true;
+  // (requested together: one after the other, as the rule asks for them, they took 1700 cycles)
+  const double first = sq[0], now = sq[it], s1 = sq[it > 0 ? it - 1 : 0], s2 = sq[it > 1 ? it - 2 : 0];
+  const bool bad = !(first <= TG_GOOD_START2);
+  if (p.stop_guard & 16) return first != 0.0;
+  if (p.stop_guard & 8) return !bad;
+  if ((p.stop_guard & 4) && now <= TG_SKIP2) return true;
+  int done = it;  // residuals that count
   if (p.stop_guard) {
-    if (it == 0) return (p.stop_guard & 2) && tg_bad_start(sq);
-    if (tg_bad_start(sq)) { ++sq; --it; }
+    if (it == 0) return (p.stop_guard & 2) && bad;
+    if (bad) --done;
   }
-  if (it < 1) return false;
-  const double cur = sq[it - 1];
-  if (!(cur > TG_DONE2)) return true;
-  if (it < 2) return false;
-  const double prev = sq[it - 2];
-  if (cur > 1.5 * prev && cur > 1e-2 * (double)p.M) {
+  if (done < 1) return false;
+  if (!(s1 > TG_DONE2)) return true;
+  if (done < 2) return false;
+  if (s1 > 1.5 * s2 && s1 > 1e-2 * (double)p.M) {
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) raise_status(p.status, CAFEQ_ERR_NONFINITE);
     return true;
   }
-  return it >= 5 && cur > prev * (1.0 - 1e-7) && cur < prev * (1.0 + 1e-7);
+  return done >= 5 && s1 > s2 * (1.0 - 1e-7) && s1 < s2 * (1.0 + 1e-7);
 }
 __device__ __forceinline__ bool tg_stopped(const TgParams& p) { return tg_stopped(p, p.stop_it); }
 
@@ -123,7 +127,7 @@ __device__ __forceinline__ void tg_epilogue_chunk(const TgParams& p, const int b
       for (int e = 0; e < 16; ++e) v[hf * 16 + e] += w[e];
     }
   }
-  const bool inner = (nb0 + 32 <= p.N) && (m0 + 128 <= p.M);  // no edge in this chunk
+  const bool inner = (nb0 + 32 <= p.N) && (rbase + 32 <= p.M);  // no edge in this chunk
   // Vector path (no edge, every pitch a multiple of 4 elements, aligned bases): a lane moves 16 bytes per
   // shared-memory access (pitch 36 floats: conflict-free by quarter warps) and a warp instruction covers
   // 4 rows x 128 bytes of global memory.  In the accumulator a lane owns a ROW; global traffic wants a

@@ -101,7 +101,7 @@ struct T2At {
 // in this launch (the barriers' phases).  On return both CTAs are done with each other's shared memory.
 __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma, const CUtensorMap* mb, const TgParams& p,
                                         const T2Shape& sh, double* sq_acc, const int ti, const int tj, const T2At at,
-                                        const uint32_t chunks, const uint32_t tiles, const T2Ste* ste = nullptr) {
+                                        const uint32_t chunks, const uint32_t tiles, const T2Ste* ste = nullptr, const bool meets = false) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cta.rank, base = smem_u32(cta.smem);
   const int bn = sh.bn, bh = bn >> 1, narr = sh.na + sh.nb;
@@ -259,9 +259,11 @@ __device__ __forceinline__ void t2_tile(const T2Cta& cta, const CUtensorMap* ma,
       }
     }
   }
-  // neither CTA goes on (or leaves) while the other's products may read its shared memory or signal its barriers
+  // neither CTA goes on (or leaves) while the other's products may read its shared memory or signal its barriers (meets: the grid meets
+  // next, which includes that)
   __syncwarp();
   tc_fence_before();
+  if (meets) return;
   __syncthreads();
   cluster_sync();
   tc_fence_after();
@@ -314,7 +316,7 @@ struct T2LoopParams {
 
 // All CTAs of the grid, bounded; false: some CTA did not come (status raised).
 __device__ __forceinline__ bool grid_meet(uint32_t* arrived, uint32_t target, volatile int* abort_flag, int32_t* status) {
-  asm volatile("fence.proxy.async;" ::: "memory");  // what was stored is read by bulk copies next
+  asm volatile("fence.proxy.async;" ::: "memory");  // what was stored (or lies in shared memory that is filled next) meets bulk copies
   __threadfence();
   __syncthreads();
   bool ok = true;
@@ -358,14 +360,16 @@ pinv_loop_kernel(const __grid_constant__ T2LoopMaps maps, const __grid_constant_
       for (int t = pair; t < sh.tm * sh.tn; t += npairs) {
         const int tj = t / sh.tm;
         t2_tile(cta, maps.a[pr], maps.b[pr ? 1 + cur : 0], p, sh, p.sq + it, t - tj * sh.tm, tj,
-                T2At{0, 0, 0, 0, 0, p.K / TG_BK, 0}, chunks, tiles);
-        // the epilogue's scratch lies in the ring that bulk copies write next
-        asm volatile("fence.proxy.async;" ::: "memory");
-        __syncthreads();
+                T2At{0, 0, 0, 0, 0, p.K / TG_BK, 0}, chunks, tiles, nullptr, t + npairs >= sh.tm * sh.tn);
+        if (t + npairs < sh.tm * sh.tn) {  // the epilogue's scratch lies in the ring that bulk copies write next
+          asm volatile("fence.proxy.async;" ::: "memory");
+          __syncthreads();
+        }
         chunks += p.K / TG_BK;
         ++tiles;
       }
       ok = grid_meet(lp.arrived, ++met * gridDim.x, cta.abort_flag, p.status);
+      tc_fence_after();
     }
     if (!ok || done) break;
   }
@@ -481,12 +485,12 @@ static int pinv_loop_launch(cudaStream_t st, const T2LoopMaps& maps, const T2Loo
   return cudaLaunchKernelEx(&cfg, pinv_loop_kernel, maps, lp) == cudaSuccess ? CAFEQ_OK : CAFEQ_ERR_CUDA;
 }
 
-// Tile width of a product of M rows: waves of 74 pairs times the width.
-static int t2_width(int M, int N, int b_mn, double* cost) {
+// Tile width of a product of M rows: waves of 74 pairs times the width; `least` at least.
+static int t2_width(int M, int N, int b_mn, double* cost, int least = 128) {
   const long long tm = (M + 255) / 256;
   int best = 0;
   double bc = 1e30;
-  for (int bn = 256; bn >= 128; bn -= b_mn ? 128 : 32) {
+  for (int bn = 256; bn >= least; bn -= b_mn ? 128 : 32) {
     const long long waves = (tm * ((N + bn - 1) / bn) + 73) / 74;
     const double c = (double)waves * (bn + 24);  // (+ the fixed part of a tile: first loads, epilogue)
     if (c < bc) { bc = c; best = bn; }

@@ -104,9 +104,8 @@ static int launch_dense_tc(cudaStream_t st, int na, const uint16_t* const* A, in
 
 static void launch_split_rect(cudaStream_t st, const float* X, int R, int C, long long ld, float scale, const double* inv_scale,
                               float* Y, float* YT, uint16_t* hi, uint16_t* lo, uint16_t* thi, uint16_t* tlo, const int32_t* status,
-                              uint16_t* h3 = nullptr, uint16_t* t3 = nullptr, const double* norm2 = nullptr, const double* only_bad = nullptr) {
-  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3, norm2,
-            only_bad);
+                              uint16_t* h3 = nullptr, uint16_t* t3 = nullptr, const double* norm2 = nullptr) {
+  CQ_LAUNCH(split_rect_kernel, dim3(C / 64, R / 64), 256, 0, st, X, R, C, ld, scale, inv_scale, Y, YT, hi, lo, thi, tlo, status, h3, t3, norm2);
 }
 
 // Scratch of the dense pair algebra for a pair with stored shapes U [h, d1], V [d3, rh]
@@ -165,7 +164,7 @@ static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, 
   return b.used + 4096;
 }
 
-// Approximate G^-1 = (A A^T)^-1 for the splits of A in w.Aw* ([m, n], m <= n), left as bf16 splits in w.CTh / w.CTl; w.sq + 123: c.
+// Approximate G^-1 = (A A^T)^-1 for the splits of A in w.Aw* ([m, n], m <= n), left as bf16 splits in w.CTh / w.CTl.
 // Y <- 2 mu Y - mu^2 Y B and B <- 2 mu B - mu^2 B B from B = G / c (c a little above ||G||_F), Y = I / c: B = G Y c throughout, and
 // with mu = 2 / (1 + l) for the smallest eigenvalue l of B the eigenvalues of B go to 1, l growing fourfold a step at first.
 // Both are polynomials in G, so one launch does both products on their upper tiles: 36 + 36 pairs at m = 2048, one wave, 45 us; a
@@ -173,8 +172,11 @@ static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, 
 // rectangular iteration (the products' errors grow with them, fourfold a step: from 2^-14 they left residuals twice as large).
 // Nothing here need be accurate: whatever Y is, A^T Y lies in the row space of A, and its error is what the rectangular iteration
 // corrects.
+// The Y of gram_restart(m) steps is kept in w.Oh / w.Ol for the restart (pinv_rows); the steps after it are skipped on a matrix with a
+// row of zeros.
 constexpr int GRAM_STEPS = 9;
-static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2, int32_t* status) {
+static int gram_restart(int m) { return m < 512 ? 1 : 2; }
+static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2, double* rs, double* singular, int32_t* status) {
   T2Maps maps;
   T2Params tp;
   int rc;
@@ -193,28 +195,31 @@ static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2,
   if ((rc = t2_launch(st, maps, tp))) return rc;
   uint16_t* Bs[2][2] = {{w.Yh, w.Yl}, {w.YTh[0], w.YTl[0]}};
   uint16_t* Ys[2][2] = {{w.YTh[1], w.YTl[1]}, {w.CTh, w.CTl}};
+  uint16_t* kept[2] = {w.Oh, w.Ol};
+  const int keep = gram_restart(m);
   static_assert(GRAM_STEPS % 2 == 1, "the result is left in the second pair of buffers");
   double l = 1.0 / 8192.0;
   for (int j = 0; j < GRAM_STEPS; ++j) {
     const float mu = (float)(2.0 / (1.0 + l));
     l = 4.0 * l / ((1.0 + l) * (1.0 + l));
     if (j == 0)
-      CQ_LAUNCH(gram_start_kernel, dim3(m / 64, m / 64), 256, 0, st, w.Y, m, fro2, mu, w.Cf, Bs[0][0], Bs[0][1], Ys[1][0], Ys[1][1],
-                w.sq + 123, status);
+      CQ_LAUNCH(gram_start_kernel, dim3(m / 64, m / 64), 256, 0, st, w.Y, m, fro2, mu, w.Cf, Bs[0][0], Bs[0][1],
+                keep == 1 ? kept[0] : Ys[1][0], keep == 1 ? kept[1] : Ys[1][1], singular, rs, status);
     const int b = j & 1;
     tp.nprob = 0;
-    auto add = [&](uint16_t* (*S)[2], float* X) {
+    auto add = [&](uint16_t* const* from, uint16_t* const* to, float* X) {
       DenseOut o;
       o.C0 = X; o.ldc0 = m; o.C = X; o.ldc = m;
-      o.Chi = S[b ^ 1][0]; o.Clo = S[b ^ 1][1];
+      o.Chi = to[0]; o.Clo = to[1];
+      if (j >= keep) { o.stop_sq = singular; o.stop_guard = 16; }
       tp.p[tp.nprob] = dense_params(m, m, m, -mu * mu, 2.f * mu, 0.f, o, status, 0);
       for (int i = 0; i < 2; ++i)
-        if (!make_map_bf16(&maps.a[tp.nprob][i], S[b][i], m, m, m, 128)) return false;
+        if (!make_map_bf16(&maps.a[tp.nprob][i], from[i], m, m, m, 128)) return false;
       ++tp.nprob;
       return true;
     };
-    if (j + 1 < GRAM_STEPS && !add(Bs, w.Y)) return CAFEQ_ERR_UNSUPPORTED;
-    if (j > 0 && !add(Ys, w.Cf)) return CAFEQ_ERR_UNSUPPORTED;
+    if (j + 1 < GRAM_STEPS && !add(Bs[b], Bs[b ^ 1], w.Y)) return CAFEQ_ERR_UNSUPPORTED;
+    if (j > 0 && !add(j == keep ? kept : Ys[b], j + 1 == keep ? kept : Ys[b ^ 1], w.Cf)) return CAFEQ_ERR_UNSUPPORTED;
     for (int i = 0; i < 2; ++i)
       if (!make_map_bf16(&maps.b[i], Bs[b][i], m, m, m, 128)) return CAFEQ_ERR_UNSUPPORTED;
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -233,25 +238,28 @@ static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2,
 //      (step 3 squares it), or until the residual stalls, which every product works out from the residuals itself.  Two updates for the 9B-shaped v-o factors (kappa^2 some thousands) instead of
 //      the sixteen from X0 = A^T / c.
 //   3. One step with the residual over three-way splits.
-// When A X0 is not within 0.9 of I (rank-deficient or very badly conditioned A) the iteration restarts from X0 = A^T / c, c a
-// little above ||A A^T||_F: the eigenvalues of A X0 then lie in [0, 1], and it converges to the Moore-Penrose inverse (stalling at
-// the rank defect).  From there on it is one launch.
+// When A X0 is not within 0.9 of I (rank-deficient or very badly conditioned A) the iteration restarts from X0 = A^T Y with the Y of
+// one or two Gram steps: the eigenvalues of A X0 lie in [0, 1], and it converges to the Moore-Penrose inverse (stalling at the rank
+// defect).  Each Gram step saves two iterations, and lets Y grow fourfold where A A^T is singular; there A^T Y cancels only to the
+// rounding of what cancels.  With 4^steps about the square root of m that stays below the rounding of the iteration itself: against
+// float64, 64 x 192 with one of its rows repeated, scales off by 1.4e-7 after one step (none 2.3e-7), 3.1e-6 after four.
 // Error against a float64 pseudo-inverse (512 x 768, kappa^2 4000, emulated products): 1.3e-7; from X0 = A^T / c 7e-6.
 static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, int32_t* status) {
   const bool wide = R <= C;
   const int m = wide ? R : C, n = wide ? C : R;
   double* fro2 = w.sq + 120;
   double* norm2 = w.sq + 121;
-  double* c = w.sq + 123;
+  double* singular = w.sq + 122;
   double* rs = w.sq + 32;  // residuals per iteration
   int rc;
   CQ_LAUNCH(zero_f64_kernel, 1, 128, 0, st, w.sq + 32, DENSE_SQ - 32);
   CQ_LAUNCH(sqsum_f32_kernel, grid_for((long long)R * C), 256, 0, st, S, (long long)R * C, norm2);
   if (wide) launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, w.Awh, w.Awl, nullptr, nullptr, status, w.Aw3, nullptr, norm2);
   else launch_split_rect(st, S, R, C, C, 1.f, nullptr, nullptr, nullptr, nullptr, nullptr, w.Awh, w.Awl, status, nullptr, w.Aw3, norm2);
-  if ((rc = gram_inverse(st, m, n, w, fro2, status))) return rc;
-  {  // Y = G^-1 A (the rows of A, the contraction, are read as they are stored)
-    const uint16_t* g[2] = {w.CTh, w.CTl};
+  if ((rc = gram_inverse(st, m, n, w, fro2, rs, singular, status))) return rc;
+  // Y = (g0 + g1) A (the rows of A, the contraction, are read as they are stored)
+  auto start = [&](const uint16_t* g0, const uint16_t* g1, int cur, const double* sq, int guard) -> int {
+    const uint16_t* g[2] = {g0, g1};
     const uint16_t* a[3] = {w.Awh, w.Awl, w.Aw3};
     const int bn = t2_width(m, n, 1, nullptr);
     T2Maps maps;
@@ -264,14 +272,16 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     if (!ok) return CAFEQ_ERR_UNSUPPORTED;
     DenseOut o;
     o.C = w.Y; o.ldc = n;
-    o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[0]; o.Ctlo = w.YTl[0];
+    o.Chi = w.Yh; o.Clo = w.Yl; o.Cthi = w.YTh[cur]; o.Ctlo = w.YTl[cur];
+    o.stop_sq = sq; o.stop_guard = guard;
     tp.p[0] = dense_params(m, n, m, 1.f, 0.f, 0.f, o, status, 0);
     tp.p[0].b_mn = 1;
     tp.nprob = 1;
     tp.sh = t2_shape(m, n, bn, 2, 3, 3);
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    if ((rc = t2_launch(st, maps, tp))) return rc;
-  }
+    return t2_launch(st, maps, tp);
+  };
+  if ((rc = start(w.CTh, w.CTl, 0, singular, 16))) return rc;
   const uint16_t* aw[2] = {w.Awh, w.Awl};
   const uint16_t* ct[2] = {w.CTh, w.CTl};
   const uint16_t* y[2] = {w.Yh, w.Yl};
@@ -294,17 +304,16 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     u.stop_it = it;
     if (it == 0) u.stop_guard = 7;
     if ((rc = launch_dense_tc(st, 2, ct, 2, yt, m, n, m, 1.f, 1.f, 0.f, u, nullptr, status))) return rc;
-    if (it == 0) {  // the restart: what update 0 would have written
-      if (wide) launch_split_rect(st, S, R, C, C, 1.f, c, w.Y, nullptr, w.Yh, w.Yl, w.YTh[1], w.YTl[1], status, nullptr, nullptr, norm2, rs);
-      else launch_split_rect(st, S, R, C, C, 1.f, c, nullptr, w.Y, w.YTh[1], w.YTl[1], w.Yh, w.Yl, status, nullptr, nullptr, norm2, rs);
-    }
+    if (it == 0 && (rc = start(w.Oh, w.Ol, 1, rs, 8))) return rc;  // the restart: what update 0 would have written
   }
   {
     T2LoopMaps maps;
     T2LoopParams lp;
     memset(&maps, 0, sizeof(maps));
     memset(&lp, 0, sizeof(lp));
-    const int bm = t2_width(m, m, 0, nullptr), bn = t2_width(m, n, 0, nullptr);
+    // (narrow tiles where there are few: with these and without the barriers that the grid's include an iteration of 256 x 512 takes 18
+    // us, of tiles of 128 columns and more 25)
+    const int bm = t2_width(m, m, 0, nullptr, 64), bn = t2_width(m, n, 0, nullptr, 64);
     bool ok = true;
     for (int i = 0; i < 2; ++i) {
       ok = ok && make_map_bf16(&maps.a[0][i], aw[i], n, m, n, 128) && make_map_bf16(&maps.b[0][i], y[i], n, m, n, bm / 2);

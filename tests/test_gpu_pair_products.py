@@ -65,6 +65,28 @@ def test_first_half_step_against_float64(h, d1, d3, k, case):
     assert (o["codes2"].double().reshape(q.shape) != q).double().mean().item() <= 1e-4
 
 
+# The restart from a start that is not usable: what it keeps of the Gram iteration must not leave the row space of the factor.
+@pytest.mark.parametrize("h,d1,d3", [(64, 192, 256), (256, 512, 448), (512, 768, 896)])
+@pytest.mark.parametrize("case", ["zero", "repeated"])
+def test_singular_factor_to_fp32(h, d1, d3, case):
+    import paper_2511_19705_b200 as cq
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    W1 = (torch.randn((h, d1), generator=g, device="cuda") / d1 ** 0.5).bfloat16()
+    W2 = (torch.randn((d3, h), generator=g, device="cuda") / h ** 0.5).bfloat16()
+    if case == "zero":
+        W1[5] = 0
+    else:
+        W1[0] = W1[40]
+    o = cq.cafeq_adaptive_round(W1, W2, None, iters=1, bits=4, group1=64, group2=64, k=64)
+    assert int(o["status"].item()) == 0
+    _, _, Uh = _quant(W1.double(), 64, 4)
+    T = (torch.linalg.pinv(Uh.t(), rtol=1e-10) @ (W1.double().t() @ W2.double().t())).t()
+    s = T.reshape(d3, -1, 64).abs().amax(-1) / 7
+    # sums of h terms at fp32; 1.2e-7 to 5.5e-7 measured, with four Gram steps kept 3.1e-6 at the repeated row of 64
+    assert ((o["scales2"].double() - s).norm() / s.norm()).item() <= 2.0 ** -24 * h ** 0.5
+
+
 # One row of an otherwise orthonormal factor is weak, so that what is left of the iteration's residual lies in one direction, and with
 # W2's first column dominant that direction alone decides scales2, whose exact values are known (the first factor is on its grid, so
 # the target is W2).  Over the strengths of the row the residual before the last step passes through all of its range.
