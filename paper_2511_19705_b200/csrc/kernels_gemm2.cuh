@@ -13,6 +13,7 @@
 
 #include "kernels_gemm.cuh"
 #include "kernels_pair_mma.cuh"
+#include "pair_rules.cuh"
 
 namespace cafeq {
 
@@ -485,20 +486,6 @@ static int pinv_loop_launch(cudaStream_t st, const T2LoopMaps& maps, const T2Loo
   return cudaLaunchKernelEx(&cfg, pinv_loop_kernel, maps, lp) == cudaSuccess ? CAFEQ_OK : CAFEQ_ERR_CUDA;
 }
 
-// Tile width of a product of M rows: waves of 74 pairs times the width; `least` at least.
-static int t2_width(int M, int N, int b_mn, double* cost, int least = 128) {
-  const long long tm = (M + 255) / 256;
-  int best = 0;
-  double bc = 1e30;
-  for (int bn = 256; bn >= least; bn -= b_mn ? 128 : 32) {
-    const long long waves = (tm * ((N + bn - 1) / bn) + 73) / 74;
-    const double c = (double)waves * (bn + 24);  // (+ the fixed part of a tile: first loads, epilogue)
-    if (c < bc) { bc = c; best = bn; }
-  }
-  if (cost) *cost = bc;
-  return best;
-}
-
 // Products of M x N in tiles of 256 x bn over na and nb arrays: the terms A_i B_j with i + j < order, all but the leading one on the
 // second accumulator.
 static T2Shape t2_shape(int M, int N, int bn, int na, int nb, int order) {
@@ -516,22 +503,6 @@ static T2Shape t2_shape(int M, int N, int bn, int na, int nb, int order) {
   s.two = s.nterms > 1;
   s.nstage = T2_NSLOT / (na + nb);
   return s;
-}
-
-// Whether CTA pairs are the better choice: waves x width of both kernels, the tiled one's (148 CTAs of 128 rows) weighted by what
-// it loses to its operand traffic.  Measured, tiled -> pairs: 2048 x 2048 x 3584, three terms 65 -> 60 us, six 131 -> 112;
-// 2048 x 3584 x 2048 with C, C0 and four splits 102 -> 95, six terms (two launches before) 203 -> 152; 3584 x 2048 x 3584 131 -> 119,
-// 258 -> 217; 1024 x 1024 x 2048 35 -> 27, 70 -> 47; 3584 x 3584 x 2048, three waves of pairs, three terms 130 -> 134.
-static bool t2_wanted(int M, int N, double cost) {
-  const long long mt = (M + 127) / 128;
-  double tiled = 1e30;
-  for (int bn : {256, 224, 128, 64}) {
-    const long long tiles = mt * ((N + bn - 1) / bn);
-    if (bn > 128 && tiles < 96) continue;
-    const double c = (double)((tiles + 147) / 148) * ((bn == 64 ? 1.6 : bn == 128 ? 1.4 : 1.25) * bn + 24);
-    if (c < tiled) tiled = c;
-  }
-  return cost < tiled;
 }
 
 // Slices of a contraction of length K in 74 / units parts, of 256 entries at least (a tile's fixed part is some 8 us).

@@ -56,14 +56,13 @@ static int tg_launch_dense(cudaStream_t st, int nterms, const uint16_t* const* A
 // are three terms (fp32-grade to about 2^-17 per entry), with three each six, down to 2^-24: what is left is the rounding of the
 // fp32 accumulators.  acc: fp32 [M, N] for the first half of more than three terms on the tiled kernel (it may be o.C).
 //
-// Large products run on CTA pairs.  The line lies where tiles of 256 rows fill the chip worse than the tiled kernel's 128-row
-// ones by more than the latter lose to their operand traffic.
+// Six terms, and three with a long contraction, run on CTA pairs (t2_wanted).
 static int launch_dense_tc(cudaStream_t st, int na, const uint16_t* const* A, int nb, const uint16_t* const* B, int M, int N, int K,
                         float alpha, float beta, float gamma, const DenseOut& o, float* acc, int32_t* status, int a_mn = 0) {
   const int order = na > nb ? na : nb;
   double cost;
   const int bn = t2_width(M, N, 0, &cost);
-  if (K % TG_BK == 0 && t2_wanted(M, N, cost)) {
+  if (K % TG_BK == 0 && t2_wanted(M, N, K, order, cost)) {
     T2Maps maps;
     T2Params tp;
     memset(&maps, 0, sizeof(maps));
