@@ -1,5 +1,5 @@
-"""Blocks of 256 run on CTA pairs: tiles of 256 rows (output axis: columns) in the transform pass, of 128 contraction entries in the
-sparse backward.  Sizes at the edges of those tiles, groups narrower and wider than a CTA's half and straddling it, against the
+"""Blocks of 256 run on CTA pairs where records are made (tiles of 256 rows, output axis: columns) and in the sparse backward (tiles of
+128 contraction entries), their codes, residuals and products with activations on one CTA a tile.  Sizes at the edges of those tiles, groups narrower and wider than a CTA's half and straddling it, against the
 shape-agnostic kernels."""
 import pytest
 import torch
@@ -35,6 +35,34 @@ def test_loss_and_gradient(axis, d_out, d_in, group):
     g, w = got["gradM"].double(), want["gradM"].double()
     for b in range(g.shape[0]):
         assert ((g[b] - w[b]).norm() / w[b].norm()).item() <= 5e-4, b
+
+
+# half a tile of contraction entries at the end of the paired backward on the output axis
+@pytest.mark.parametrize("d_out,d_in,group", [(256, 64, 64), (512, 192, 64), (256, 576, 192), (512, 704, 64)])
+def test_loss_and_gradient_half_tile(d_out, d_in, group):
+    test_loss_and_gradient("out", d_out, d_in, group)
+
+
+# rows apart by more than their width: the padding holds NaN and must not be met
+@pytest.mark.parametrize("axis,d_out,d_in,group,pad", [("in", 300, 512, 128, 8), ("in", 257, 768, 64, 256), ("out", 512, 384, 64, 24),
+                                                       ("out", 256, 640, 128, 128)])
+def test_padded_rows(axis, d_out, d_in, group, pad):
+    import paper_2511_19705_b200 as cq
+    W, M = _case(d_out, d_in, (d_in if axis == "in" else d_out) // 256, d_out + d_in)
+    wide = torch.full((d_out, d_in + pad), float("nan"), device="cuda", dtype=torch.bfloat16)
+    wide[:, :d_in] = W
+    kw = dict(bits=3, group=group, taxis=cq.AXIS_IN if axis == "in" else cq.AXIS_OUT)
+    for loss in (cq.LOSS_SURROGATE, cq.LOSS_L2_STE):
+        got = cq.cafeq_proxy_loss_fwd_bwd(wide[:, :d_in], M, loss_kind=loss, **kw)
+        want = cq.cafeq_proxy_loss_fwd_bwd(W, M, loss_kind=loss, **kw)
+        assert int(got["status"].item()) == 0
+        n = 1 if loss == cq.LOSS_SURROGATE else 3
+        assert torch.allclose(got["losses"][:n], want["losses"][:n], rtol=1e-5)
+        g, w = got["gradM"].double(), want["gradM"].double()
+        assert ((g - w).norm() / w.norm()).item() <= 1e-5  # (the same values, summed in another order)
+    c, s = cq.cafeq_rtn(wide[:, :d_in], M, bits=3, group=group, tblock=256, taxis=kw["taxis"])
+    cw, sw = cq.cafeq_rtn(W, M, bits=3, group=group, tblock=256, taxis=kw["taxis"])
+    assert torch.equal(c, cw) and torch.equal(s, sw)
 
 
 @pytest.mark.parametrize("tokens,d_in,transposed", [(65, 256, True), (128, 512, False), (257, 768, True), (500, 1024, True)])
