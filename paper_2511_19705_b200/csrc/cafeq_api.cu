@@ -578,9 +578,6 @@ __global__ void resid_sq_kernel(float* __restrict__ R, const float* P, long long
   if (threadIdx.x == 0) atomicAdd(acc, s);
 }
 
-__global__ void store_sqrt_kernel(const double* acc, float* out) {
-  pdl_enter(); *out = (float)sqrt(*acc); }
-
 // ------------------------------------------------------------------------------------------------
 // per-matrix scratch
 // ------------------------------------------------------------------------------------------------

@@ -631,17 +631,6 @@ __global__ void expand_agrp_kernel(const float* Agrp, int d_in, int g, int k, in
   atomicAdd(&A[(B / r) * k + (t - B * k)], Agrp[t / g]);
 }
 
-// gMinv[b][i][t] = scale * Minv[b][i][t] * A[b][t]
-__global__ void scale_cols_kernel(const float* Minv, const float* A, float scale, int k,
-                                  long long n, float* __restrict__ out) {
-  pdl_enter();
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    long long b = e / ((long long)k * k);
-    int t = (int)(e % k);
-    out[e] = scale * Minv[e] * A[b * k + t];
-  }
-}
-
 // ------------------------------------------------------------------------------------------------
 // straight-through scale path: coef[row, G] = sign(U[e*]) / qmax * sum_{e in G} gDelta_e (q_e - U_e / s_G)
 // (+ optionally, for the pair PQE loss, the direct term stays in gU and is handled by a dense product)
@@ -1324,47 +1313,8 @@ __global__ void sqsum_bf16_kernel(const uint16_t* W, long long ld, int rows, int
 // ------------------------------------------------------------------------------------------------
 // pair: LogSumExp over group maxima (two passes), orthonormality penalty
 // ------------------------------------------------------------------------------------------------
-__global__ void max_f32_kernel(const float* a, long long n, float* __restrict__ out_max,
-                               const int32_t* status) {
-  pdl_enter();
-  // a >= 0, so an integer atomicMax on the bit pattern orders correctly
-  if (warp_stopped(status)) return;
-  float m = 0.f;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    m = fmaxf(m, a[i]);
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax((int*)out_max, __float_as_int(m));
-}
 
-__global__ void sumexp_kernel(const float* a, long long n, const float* amax, float t,
-                              double* __restrict__ acc, const int32_t* status) {
-  pdl_enter();
-  if (cta_stopped(status)) return;
-  __shared__ double red[32];
-  const float mx = *amax;
-  double local = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    local += (double)expf(t * (a[i] - mx));
-  double s = block_sum_double(local, red);
-  if (threadIdx.x == 0) atomicAdd(acc, s);
-}
-
-// coef[w] = exp(t (a - max)) / Z * sign(U[arg-max])
-__global__ void lse_coef_kernel(const float* a, const float* usel, long long n,
-                                const float* amax, float t, const double* Z,
-                                float* __restrict__ coef, const int32_t* status) {
-  pdl_enter();
-  if (status && *status) return;
-  const float mx = *amax;
-  const float zinv = (float)(1.0 / *Z);
-  for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < n; w += (long long)gridDim.x * blockDim.x) {
-    float u = usel[w];
-    float sgn = (u > 0.f) ? 1.f : ((u < 0.f) ? -1.f : 0.f);
-    coef[w] = expf(t * (a[w] - mx)) * zinv * sgn;
-  }
-}
-
-// two-array forms of the three LogSumExp kernels (the group maxima of U and of V in one launch each)
+// LogSumExp over the group maxima of U and of V, both in each launch
 __global__ void max2_f32_kernel(const float* a1, long long n1, const float* a2, long long n2,
                                 float* __restrict__ out_max, const int32_t* status) {
   pdl_enter();

@@ -156,13 +156,6 @@ static bool carve_dense(Bump& b, int h, int d1, int d3, int r, int k, int ng1, i
   return !b.overflow;
 }
 
-static size_t dense_scratch_bytes(int h, int d1, int d3, int r, int k, int ng1, int ng2) {
-  Bump b(nullptr, (size_t)-1);
-  DenseWS w;
-  carve_dense(b, h, d1, d3, r, k, ng1, ng2, &w);
-  return b.used + 4096;
-}
-
 // Approximate G^-1 = (A A^T)^-1 for the splits of A in w.Aw* ([m, n], m <= n), left as bf16 splits in w.CTh / w.CTl.
 // Y <- 2 mu Y - mu^2 Y B and B <- 2 mu B - mu^2 B B from B = G / c (c a little above ||G||_F), Y = I / c: B = G Y c throughout, and
 // with mu = 2 / (1 + l) for the smallest eigenvalue l of B the eigenvalues of B go to 1, l growing fourfold a step at first.

@@ -53,7 +53,7 @@ def test_kernel_waits_for_its_predecessor_first(file, name, body):
 
 
 # functions that meet at a barrier or exchange values between lanes, directly or in what they call
-COLLECTIVE = re.compile(r"__syncthreads|__syncwarp|_sync\(|mbar_|block_sum_double|gauss_jordan|pw_norm2")
+COLLECTIVE = re.compile(r"__syncthreads|__syncwarp|_sync\(|mbar_|block_sum_double|gauss_jordan")
 
 
 @pytest.mark.parametrize("file,name,body", [f for f in KERNELS + _functions(r"__device__ __forceinline__ void(?= bd_)") if COLLECTIVE.search(f[2])],
@@ -72,7 +72,7 @@ def test_inputs_are_read_with_ordinary_loads(path):
     assert not re.search(r"\bconst\s+\w+\s*\*\s*__restrict__", text)
 
 
-RETURNING = (r"launch_dense_tc6?|launch_kk_tc|tg_launch|tb_launch|bd_launch\w*|bw_launch\w*|ns_block_launch|kk_chain_launch|ns_inverse|"
+RETURNING = (r"launch_dense_tc|launch_kk_tc|launch_split_product|tg_launch\w*|t2_launch|pinv_loop_launch|gram_inverse|tb_launch|bd_launch\w*|bw_launch\w*|ns_block_launch|kk_chain_launch|ns_inverse|"
              r"minv_path_tc|penalty_tc|opgrad_\w+_tc|pinv_rows|dense_product|dense_pqe|alg1_run")
 
 
