@@ -72,9 +72,9 @@ struct TgCfg {
 // The residuals of iterations that were skipped stay zero, so the last two decide.
 // With stop_guard, iteration 0 checks a start that is only good when its residual is at most 0.9 (so every eigenvalue of I - A X is);
 // otherwise the iteration has been restarted, and what came before iteration 1 does not count.  Iteration 0 itself then updates
-// nothing.  An update that would start below 1e-4 is left out: the step that follows the iteration squares the residual too, and
-// leaves less than 2^-24 of it even where all of it is in one direction (from 1e-3 that direction ended at 1e-6).
-constexpr double TG_GOOD_START2 = 0.81, TG_DONE2 = 1e-6, TG_SKIP2 = 1e-8;
+// nothing.  An update that would start below 2^-12 is left out: the step that follows the iteration squares the residual too, and
+// leaves 2^-24 at most even where all of it is in one direction (from 1e-3 that direction ended at 1e-6).
+constexpr double TG_GOOD_START2 = 0.81, TG_DONE2 = 1e-6, TG_SKIP2 = 1.0 / (1 << 24);
 __device__ __forceinline__ bool tg_stopped(const TgParams& p, int it) {
   const volatile double* sq = p.stop_sq;  // (one launch may run several iterations: never from a cached line)
   if (!sq) return false;

@@ -226,9 +226,9 @@ static int gram_inverse(cudaStream_t st, int m, int n, DenseWS& w, double* fro2,
 // brings the result back.
 //   1. X0 = A^T G^-1 with the approximate inverse of the Gram matrix (gram_inverse), as five terms over A split three ways: the
 //      iteration below never corrects what lies outside the row space of A, so X0 must not leave it.
-//   2. Newton-Schulz X <- X + X (I - A X), until an update that began below ||I - A X||_F = 1e-3 or until one would begin below 1e-4
-//      (step 3 squares it), or until the residual stalls, which every product works out from the residuals itself.  Two updates for the 9B-shaped v-o factors (kappa^2 some thousands) instead of
-//      the sixteen from X0 = A^T / c.
+//   2. Newton-Schulz X <- X + X (I - A X), until an update that began below ||I - A X||_F = 1e-3 or until one would begin below
+//      2^-12 (step 3 squares it), or until the residual stalls, which every product works out from the residuals itself.  One or two
+//      updates for the 9B-shaped v-o factors (kappa^2 some thousands) instead of the sixteen from X0 = A^T / c.
 //   3. One step with the residual over three-way splits.
 // When A X0 is not within 0.9 of I (rank-deficient or very badly conditioned A) the iteration restarts from X0 = A^T Y with the Y of
 // one or two Gram steps: the eigenvalues of A X0 lie in [0, 1], and it converges to the Moore-Penrose inverse (stalling at the rank
@@ -327,7 +327,7 @@ static int pinv_rows(cudaStream_t st, const float* S, int R, int C, DenseWS& w, 
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if ((rc = pinv_loop_launch(st, maps, lp))) return rc;
   }
-  // The loop above stops at a residual of 1e-4 at most (Frobenius), in the accuracy of its three-term products.  One more
+  // The loop above stops at a residual of 2^-12 at most (Frobenius), in the accuracy of its three-term products.  One more
   // step with the residual evaluated over three-way splits (fp32-grade) squares what is left: the quantised targets
   // of Algorithm 1 then agree with a float64 pseudo-inverse except at rounding ties.  The correction C^T Y is small,
   // three terms are enough for it.  (A rank-deficient matrix stalls where it stalled before: the step changes nothing.)
