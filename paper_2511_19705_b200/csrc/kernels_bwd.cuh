@@ -420,7 +420,8 @@ __device__ __forceinline__ void bd_bwd_body(const BwMaps& maps, const BwMulti& m
 // columns, so a block's sum is flushed by warps of its own while the next block is accumulated, and a pair flushes a block once where
 // two CTAs did.  (One CTA with the whole accumulator in its tensor memory stood still during each flush: 15 of 91 us of a 9B-shaped
 // layer.)  A tile holds eight products: every wait of the issuing warp costs it some 400 cycles.
-// Both forms of a 9B-shaped layer, back to back: 102 us, issued by one elected lane of a converged warp 91, pairs 79.
+// Both forms of a 9B-shaped layer, back to back: 102 us, issued by one elected lane of a converged warp 91, pairs 79, with the S tiles released
+// at the scope of the cluster (relays, below) some 87.
 // ------------------------------------------------------------------------------------------------
 constexpr int BP_THREADS = 64 + 256 + 128 + 64;  // warp 0: TMA, warp 1: MMA, warps 2-9: operand builders, 10-13: flush, 14-15: relays
 

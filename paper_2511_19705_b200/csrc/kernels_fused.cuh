@@ -87,7 +87,7 @@ constexpr int BD_STAGES_PER_TILE = 2;
 // the kernel
 // ------------------------------------------------------------------------------------------------
 // CTA pairs (cta_group::2): records at K = 256, where the products set the pace and a pair reads a third less of operands.  The other
-// epilogues are longer than the products and lose more to a pair's larger tiles (half as many of them, of 512 KB: a last wave that is
+// epilogues are longer than the products and lose more to a pair's larger tiles (half as many of them, of 128 KB: a last wave that is
 // emptier, longer first loads) than they gain.  One CTA against pairs: codes of 4096 x 3584 17.8 us, pairs 20.1, of 14336 x 3584
 // 38.9 and 40.6, of 2304 x 9216 25.1 and 29.3, residual and its square 4096 x 3584 156 and 166, apply of 2048 x 3584 13.3 and 14.0.
 // Records: a 9B-shaped layer's step 343 us on pairs, 350 without, 27B-shaped with groups of 64 900 either way.
