@@ -53,7 +53,7 @@ def test_kernel_waits_for_its_predecessor_first(file, name, body):
 
 
 # functions that meet at a barrier or exchange values between lanes, directly or in what they call
-COLLECTIVE = re.compile(r"__syncthreads|__syncwarp|_sync\(|mbar_|block_sum_double|gauss_jordan")
+COLLECTIVE = re.compile(r"__syncthreads|__syncwarp|_sync\(|mbar_|block_sum_double|gauss_jordan|pw_norm2")
 
 
 @pytest.mark.parametrize("file,name,body", [f for f in KERNELS + _functions(r"__device__ __forceinline__ void(?= bd_)") if COLLECTIVE.search(f[2])],
@@ -72,7 +72,7 @@ def test_inputs_are_read_with_ordinary_loads(path):
     assert not re.search(r"\bconst\s+\w+\s*\*\s*__restrict__", text)
 
 
-RETURNING = (r"launch_dense_tc|launch_kk_tc|launch_split_product|tg_launch\w*|t2_launch|pinv_loop_launch|gram_inverse|tb_launch|bd_launch\w*|bw_launch\w*|ns_block_launch|kk_chain_launch|ns_inverse|"
+RETURNING = (r"launch_dense_tc6?|launch_kk_tc|tg_launch|tb_launch|bd_launch\w*|bw_launch\w*|ns_block_launch|kk_chain_launch|ns_inverse|"
              r"minv_path_tc|penalty_tc|opgrad_\w+_tc|pinv_rows|dense_product|dense_pqe|alg1_run")
 
 
@@ -82,6 +82,14 @@ def test_no_launch_result_is_dropped(path):
     dropped = re.findall(r"[;{})]\s*((?:%s)\s*\([^;{}]*;)" % RETURNING, _strip(open(path).read()))
     assert not dropped, dropped
     assert not re.search(r"static void (%s)\(" % RETURNING, _strip(open(path).read()))
+
+
+@pytest.mark.parametrize("path", sorted(glob.glob(os.path.join(CSRC, "*.cu*"))), ids=os.path.basename)
+def test_no_launch_result_of_a_paired_product_is_dropped(path):
+    names = r"launch_split_product|tg_launch_\w+|t2_launch|pinv_loop_launch|gram_inverse"
+    text = _strip(open(path).read())
+    assert not re.findall(r"[;{})]\s*((?:%s)\s*\([^;{}]*;)" % names, text)
+    assert not re.search(r"static void (%s)\(" % names, text)
 
 
 def _enclosing(text, pos):
